@@ -202,7 +202,7 @@ WsPlan plan_workspace(const moe_shape& s) {
   p.st_dw = c.take(sizeof(float) * (size_t)s.T_max * s.k);
   p.st_logits = c.take(sizeof(float) * (size_t)s.T_max * s.E);
   p.ctr_count = ctr_ints((int)(cap / BLOCK_M) + 1);
-  p.ctr = c.take(sizeof(int) * (size_t)p.ctr_count);
+  p.ctr = c.take(sizeof(int) * (size_t)p.ctr_count * (train ? 2 : 1));   // forward, backward
   p.trace_cap = (s.flags & MOE_FLAG_TRACE) ? TRACE_RECORDS : 0;
   p.trace = c.take((size_t)p.trace_cap * 32);
   p.total = c.off;
@@ -224,6 +224,8 @@ struct moe_ctx {
   int saved_T = -1;  // T of the forward whose tensors are in the workspace (-1: none)
   const void *saved_x = nullptr, *saved_ids = nullptr, *saved_w = nullptr;  // that forward's inputs
   uint64_t budget_ns = 2000ull * 1000 * 1000;
+  int* last_ctr = nullptr;      // event counters of the last persistent launch
+  bool bwd_ctr_clear = false;   // the backward's event counters are zero (the forward's layout clears both sets)
   int dep_extra = 0;  // test hook: makes the activation dependencies of the persistent launch unreachable
   bool plain_launch = false;  // diagnostic: persistent launches without the cooperative attribute
   cudaStream_t last_stream = nullptr;
@@ -282,7 +284,7 @@ struct moe_ctx {
     lv.meta = at<int>(plan.meta);
     lv.blk_hist = at<int>(plan.blk_hist);
     lv.combine_order = at<int>(plan.combine_order);
-    lv.tok_last = (!(shape.flags & MOE_FLAG_SERIAL_LAUNCH) && shape.F % 16 == 0) ? at<int>(plan.tok_last) : nullptr;
+    lv.tok_last = at<int>(plan.tok_last);
     return lv;
   }
   Dims dims(int T) const { return Dims{T, shape.d, shape.E, shape.k, shape.n_shared, shape.F}; }
@@ -509,7 +511,8 @@ FusedArgs fused_base(moe_ctx* c, bool bwd, int T) {
   FusedArgs fa;
   memset(&fa, 0, sizeof fa);
   fa.lv = c->layout();
-  fa.ctr = c->at<int>(p.ctr);
+  fa.ctr = c->at<int>(p.ctr) + (bwd ? p.ctr_count : 0);
+  c->last_ctr = fa.ctr;
   fa.d = s.d;
   fa.kp = s.k + s.n_shared;
   fa.trace = p.trace_cap ? c->at<uint4>(p.trace) : nullptr;
@@ -590,9 +593,11 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
   c->saved_T = -1;
   {
     Phase ph(c, MOE_PHASE_LAYOUT, st);
-    MOE_CUDA(launch_layout(ids, dm, lv, c->status(), st, &c->launches));
-    // with shared experts every token's last row belongs to the last expert: token order is as good as any
-    if (!serial_mode(c)) MOE_CUDA(launch_layout_order(dm, lv, p.cap_rows / BLOCK_M, st, &c->launches));
+    // the event counters of this pass, and of the backward that may follow, start at zero
+    const bool persistent = !serial_mode(c);
+    MOE_CUDA(launch_layout(ids, dm, lv, persistent, p.cap_rows / BLOCK_M, persistent ? c->at<int>(p.ctr) : nullptr,
+                           persistent ? p.ctr_count * (c->train() ? 2 : 1) : 0, c->status(), st, &c->launches));
+    c->bwd_ctr_clear = persistent && c->train();
   }
   if (serial_mode(c)) {
     {
@@ -625,7 +630,6 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     fa.combine_rows = c->at<uint16_t>(p.Y);
     fa.combine_out = out;
     Phase ph(c, MOE_PHASE_FUSED_FWD, st);
-    MOE_CUDA(cudaMemsetAsync(fa.ctr, 0, sizeof(int) * (size_t)p.ctr_count, st));
     MOE_CUDA(launch_fused(false, fa, c->num_sms, !c->plain_launch, st, &c->launches));
     if (out_host && (rc = copy_out_to_host(c, out, out_host, 2 * (size_t)T * c->shape.d, st))) return rc;
   }
@@ -707,9 +711,9 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     fa.dw_nparts = p.ntn_act * DW_PARTS_PER_TILE;
     fa.d_topk_w = d_w;
     Phase ph(c, MOE_PHASE_FUSED_BWD, st);
-    MOE_CUDA(cudaMemsetAsync(fa.ctr, 0, sizeof(int) * (size_t)p.ctr_count, st));
-    // slots dropped for an invalid expert id have no row: their gradient is zero
-    if (d_w) MOE_CUDA(cudaMemsetAsync(d_w, 0, sizeof(float) * (size_t)T * s.k, st));
+    // the forward's layout cleared the counters; a second backward of one forward clears them itself
+    if (!c->bwd_ctr_clear) MOE_CUDA(cudaMemsetAsync(fa.ctr, 0, sizeof(int) * (size_t)p.ctr_count, st));
+    c->bwd_ctr_clear = false;
     // Host buffers: dx is complete when the last backward-combine task is, well before the last weight-gradient
     // strips; the kernel then sets a word the copy-out stream waits for, so the copy overlaps the rest of the launch.
     StreamValueFn wait_value = dx_host ? get_stream_value_fn(true) : nullptr;
@@ -718,7 +722,7 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     const CUdeviceptr ready_word = reinterpret_cast<CUdeviceptr>(fa.ctr + CTR_OUT_READY);
     fa.announce_out = early_out ? 1 : 0;
     if (early_out) {
-      MOE_CUDA(cudaEventRecord(c->ev_chunk[0], st));   // the word is cleared (the memset above) before anyone waits on it
+      MOE_CUDA(cudaEventRecord(c->ev_chunk[0], st));   // the word is cleared before anyone waits on it
       MOE_CUDA(cudaStreamWaitEvent(c->d2h_stream, c->ev_chunk[0], 0));
       if (wait_value(c->d2h_stream, ready_word, 1, CU_STREAM_WAIT_VALUE_GEQ) != CUDA_SUCCESS) return cuda_fail(cudaErrorUnknown, "cuStreamWaitValue32");
       MOE_CUDA(cudaMemcpyAsync(dx_host, dx, 2 * (size_t)T * s.d, cudaMemcpyDeviceToHost, c->d2h_stream));
@@ -919,7 +923,7 @@ int moe_layout(moe_ctx* c, const int32_t* topk_ids, int32_t T, int32_t* counts, 
   c->saved_T = -1;
   const Dims dm = c->dims(T);
   const LayoutView lv = c->layout();
-  MOE_CUDA(launch_layout(topk_ids, dm, lv, c->status(), st, &c->launches));
+  MOE_CUDA(launch_layout(topk_ids, dm, lv, false, 0, nullptr, 0, c->status(), st, &c->launches));
   const size_t n = (size_t)dm.slots(), Ep = dm.Ep();
   if (counts) MOE_CUDA(cudaMemcpyAsync(counts, lv.counts, sizeof(int) * Ep, cudaMemcpyDeviceToDevice, st));
   if (offsets) MOE_CUDA(cudaMemcpyAsync(offsets, lv.offsets, sizeof(int) * (Ep + 1), cudaMemcpyDeviceToDevice, st));
@@ -1110,7 +1114,7 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
     case MOE_BUF_DXP: off = p.Y; n = cap * s.d; break;
     case MOE_BUF_META: off = p.meta; n = 8; break;
     case MOE_BUF_TRACE: if (!p.trace_cap) return MOE_ERR_STATE; off = p.trace; n = (size_t)p.trace_cap * 8; break;
-    case MOE_BUF_EVENT_COUNTERS: off = p.ctr; n = p.ctr_count; break;
+    case MOE_BUF_EVENT_COUNTERS: off = c->last_ctr ? (size_t)(reinterpret_cast<uint8_t*>(c->last_ctr) - c->ws) : p.ctr; n = p.ctr_count; break;
     default: return MOE_ERR_INVALID_ARG;
   }
   *ptr = c->ws + off;
@@ -1259,7 +1263,7 @@ int moe_debug_trace(moe_ctx* c, moe_trace_record* records, size_t max_records, s
   if (!c->plan.trace_cap) return MOE_ERR_STATE;
   MOE_CUDA(cudaStreamSynchronize(c->last_stream));
   int produced = 0;
-  MOE_CUDA(cudaMemcpy(&produced, c->at<int>(c->plan.ctr) + CTR_TRACE_CURSOR, sizeof(int), cudaMemcpyDeviceToHost));
+  MOE_CUDA(cudaMemcpy(&produced, (c->last_ctr ? c->last_ctr : c->at<int>(c->plan.ctr)) + CTR_TRACE_CURSOR, sizeof(int), cudaMemcpyDeviceToHost));
   *n_written = (size_t)produced;
   size_t n = std::min<size_t>(std::min<size_t>((size_t)produced, (size_t)c->plan.trace_cap), max_records);
   if (n == 0) return MOE_OK;

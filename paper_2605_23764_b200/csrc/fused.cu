@@ -100,6 +100,9 @@ __device__ __forceinline__ bool vec_combine(const FusedArgs& fa, int task, int l
   for (int i = i0; i < i1; ++i) {
     const int t = fa.lv.combine_order ? fa.lv.combine_order[i] : i;   // tokens in the order in which their last row is produced
     const int* prow = fa.lv.prow_of + (size_t)t * kp;
+    if (fa.d_topk_w)   // a slot dropped for an invalid expert id has no row: its weight's gradient is zero
+      for (int j = lane; j < fa.cp.k; j += 32)
+        if (prow[j] < 0) fa.d_topk_w[(size_t)t * fa.cp.k + j] = 0.f;
     // dependent events: `done` of every M-block that holds one of the token's rows
     int ok = 1;
     for (int j = lane; j < kp; j += 32) {

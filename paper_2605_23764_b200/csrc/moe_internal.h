@@ -26,7 +26,7 @@ inline int padded_rows_max(int T_max, int kp, int Ep) {
   return (int)(((r + BLOCK_M - 1) / BLOCK_M) * BLOCK_M);
 }
 
-constexpr int LAYOUT_CHUNK = 2048;  // flat slots per block of the layout kernels (8 warps x 256)
+constexpr int LAYOUT_CHUNK = 2048;  // flat slots per block of the layout kernels
 
 // Device arrays describing one dispatch layout.
 struct LayoutView {
@@ -54,11 +54,12 @@ struct LayoutView {
 constexpr int GATE_RENORM = 1, GATE_SIGMOID = 2;
 cudaError_t launch_route(const float* logits, int T, int E, int k, int gate_mode, int* topk_ids, float* topk_w,
                          int* counts, cudaStream_t s, int* launches);
-cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView& lv, DevStatus* status,
-                          cudaStream_t s, int* launches);
+// want_order: also the combine order of the persistent launch (lv.tok_last, lv.combine_order; cap_mblocks bounds its
+// keys).  zero[0, nzero): ints cleared on the way (event counters, a status word).
+cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView& lv, bool want_order, int cap_mblocks,
+                          int* zero, int nzero, DevStatus* status, cudaStream_t s, int* launches);
 // process-wide switch of moe_sched_study's persistent launches (diagnostic; see moe_debug_set_plain_launch)
 std::atomic<bool>& study_plain_launch();
-cudaError_t launch_layout_order(const Dims& dm, const LayoutView& lv, int cap_mblocks, cudaStream_t s, int* launches);
 
 // ---- permute.cu
 // Xp[p] = src[token of padded row p] (zeros on padding rows); optionally prow_w[p] = routing weight

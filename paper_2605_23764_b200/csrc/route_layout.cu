@@ -4,6 +4,7 @@
 #include <limits.h>
 
 #include "moe_internal.h"
+#include "topk.cuh"
 
 namespace moe {
 
@@ -19,49 +20,41 @@ __global__ void __launch_bounds__(256) route_kernel(const float* __restrict__ lo
                                                      float* __restrict__ topk_w, int* __restrict__ counts) {
   const int lane = threadIdx.x & 31;
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  pdl_wait();
+  pdl_trigger();
   if (t >= T) return;
   const float* row = logits + (size_t)t * E;
   float v[NPL];
-  float mx = -INFINITY;
 #pragma unroll
   for (int i = 0; i < NPL; ++i) {
     int e = i * 32 + lane;
     v[i] = e < E ? row[e] : -INFINITY;
-    mx = fmaxf(mx, v[i]);
   }
+  uint32_t key[NPL];
 #pragma unroll
-  for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  float den = 0.f;
-#pragma unroll
-  for (int i = 0; i < NPL; ++i)
-    if (i * 32 + lane < E) den += expf(v[i] - mx);
-#pragma unroll
-  for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
-
-  uint32_t taken = 0;
+  for (int i = 0; i < NPL; ++i) key[i] = i * 32 + lane < E ? float_key(v[i]) : 0u;
   int my_id = 0;
-  float my_p = 0.f, wsum = 0.f;
-  for (int j = 0; j < k; ++j) {
-    float bv = 0.f;
-    int bi = INT_MAX;
+  float my_l = 0.f;
+  warp_topk<NPL>(key, k, lane, &my_id, &my_l);
+  float my_p;
+  if (renorm & GATE_SIGMOID) {
+    my_p = 1.0f / (1.0f + expf(-my_l));
+  } else {
+    const float mx = __shfl_sync(0xffffffffu, my_l, 0);
+    float den = 0.f;
 #pragma unroll
-    for (int i = 0; i < NPL; ++i) {
-      int e = i * 32 + lane;
-      if (e < E && !((taken >> i) & 1u) && (bi == INT_MAX || v[i] > bv)) { bv = v[i]; bi = e; }
-    }
+    for (int i = 0; i < NPL; ++i)
+      if (i * 32 + lane < E) den += expf(v[i] - mx);
 #pragma unroll
-    for (int off = 16; off; off >>= 1) {
-      float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      if (oi != INT_MAX && (bi == INT_MAX || ov > bv || (ov == bv && oi < bi))) { bv = ov; bi = oi; }
-    }
-    if ((bi & 31) == lane) taken |= 1u << (bi >> 5);
-    float p = (renorm & GATE_SIGMOID) ? 1.0f / (1.0f + expf(-bv)) : expf(bv - mx) / den;
-    if (lane == j) { my_id = bi; my_p = p; }
-    wsum += p;
+    for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+    my_p = expf(my_l - mx) / den;
+  }
+  if (renorm & GATE_RENORM) {
+    float wsum = 0.f;
+    for (int j = 0; j < k; ++j) wsum += __shfl_sync(0xffffffffu, my_p, j);
+    my_p /= wsum;
   }
   if (lane < k) {
-    if (renorm & GATE_RENORM) my_p /= wsum;
     topk_ids[(size_t)t * k + lane] = my_id;
     topk_w[(size_t)t * k + lane] = my_p;
     if (counts) atomicAdd(&counts[my_id], 1);
@@ -78,8 +71,9 @@ cudaError_t launch_route(const float* logits, int T, int E, int k, int gate_mode
   const int threads = 256, tokens_per_block = threads / 32;
   dim3 grid((T + tokens_per_block - 1) / tokens_per_block);
   const int npl = (E + 31) / 32;
+  cudaError_t e = cudaSuccess;
 #define MOE_ROUTE_CASE(N) \
-  route_kernel<N><<<grid, threads, 0, s>>>(logits, T, E, k, gate_mode, topk_ids, topk_w, counts)
+  e = launch_dependent(route_kernel<N>, grid, dim3(threads), 0, s, logits, T, E, k, gate_mode, topk_ids, topk_w, counts)
   if (npl <= 1) MOE_ROUTE_CASE(1);
   else if (npl <= 2) MOE_ROUTE_CASE(2);
   else if (npl <= 4) MOE_ROUTE_CASE(4);
@@ -88,239 +82,265 @@ cudaError_t launch_route(const float* logits, int T, int E, int k, int gate_mode
   else MOE_ROUTE_CASE(32);
 #undef MOE_ROUTE_CASE
   ++*launches;
-  return cudaGetLastError();
+  return e;
 }
 
 // ------------------------------------------------------------------------------------------
 // Dispatch layout.  Flat slot i = t*kp + j; block b owns slots [b*CHUNK, (b+1)*CHUNK), warp w of
-// the block owns 256 consecutive slots of it, processed 32 at a time in slot order.
+// the block owns CHUNK / warps consecutive slots of it, processed 32 at a time in slot order.
+//
+// Three kernels -- histograms, scans, ranks -- each bound by the latency of a few dependent accesses, not by bytes: many
+// warps with two or four groups of 32 slots each, every slot's id loaded before the first is used, and each kernel
+// started while the one before it runs (programmatic dependent launch).  Fewer than LAYOUT_ONE_SLOTS slots (token
+// generation) take one kernel of one block instead.
 // ------------------------------------------------------------------------------------------
-constexpr int LAYOUT_THREADS = 256;
-constexpr int LAYOUT_WARPS = LAYOUT_THREADS / 32;
-constexpr int SLOTS_PER_WARP = LAYOUT_CHUNK / LAYOUT_WARPS;
-
 __device__ __forceinline__ int slot_expert(const int* __restrict__ ids, int i, int k, int kp, int E) {
   int t = i / kp, j = i - t * kp;
   if (j >= k) return E + (j - k);
-  int e = ids[(size_t)t * k + j];
+  int e = __ldcg(ids + (size_t)t * k + j);
   return (e >= 0 && e < E) ? e : -1;
 }
 
-// Per-warp histograms of this block's chunk into shared memory whist[LAYOUT_WARPS][Ep].
-__device__ __forceinline__ void chunk_histogram(const int* __restrict__ ids, int n, int k, int kp, int E, int Ep,
-                                                int* whist) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int q = threadIdx.x; q < LAYOUT_WARPS * Ep; q += LAYOUT_THREADS) whist[q] = 0;
+constexpr int HIST_THREADS = 1024;
+__global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __restrict__ ids, int n, int k, int kp, int E,
+                                                                   int Ep, int* __restrict__ blk_hist, int* __restrict__ tok_last,
+                                                                   int* __restrict__ zero, int nzero) {
+  extern __shared__ int hist[];   // [Ep]
+  for (int e = threadIdx.x; e < Ep; e += HIST_THREADS) hist[e] = 0;
+  pdl_wait();      // the ids; and the previous launch on the stream may still use what is cleared here
+  pdl_trigger();   // behind the wait: whoever starts from here on finds the ids complete
   __syncthreads();
-  int* mine = whist + warp * Ep;
-  const int base = blockIdx.x * LAYOUT_CHUNK + warp * SLOTS_PER_WARP;
-  for (int g = 0; g < SLOTS_PER_WARP; g += 32) {
-    int i = base + g + lane;
-    int e = i < n ? slot_expert(ids, i, k, kp, E) : -1;
-    uint32_t peers = __match_any_sync(0xffffffffu, e);
-    if (e >= 0 && lane == __ffs(peers) - 1) mine[e] += __popc(peers);
+  const int base = blockIdx.x * LAYOUT_CHUNK + threadIdx.x;
+  int e[LAYOUT_CHUNK / HIST_THREADS];
+#pragma unroll
+  for (int g = 0; g < LAYOUT_CHUNK / HIST_THREADS; ++g) {
+    const int i = base + g * HIST_THREADS;
+    e[g] = i < n ? slot_expert(ids, i, k, kp, E) : -1;
+  }
+  if (tok_last)   // the tokens whose first slot lies in this block's chunk
+    for (int i = base; i < min(n, (int)(blockIdx.x + 1) * LAYOUT_CHUNK); i += HIST_THREADS)
+      if (i % kp == 0) tok_last[i / kp] = 0;
+  for (int i = blockIdx.x * HIST_THREADS + threadIdx.x; i < nzero; i += gridDim.x * HIST_THREADS) zero[i] = 0;
+#pragma unroll
+  for (int g = 0; g < LAYOUT_CHUNK / HIST_THREADS; ++g) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, e[g]);
+    if (e[g] >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&hist[e[g]], __popc(peers));
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < Ep; q += HIST_THREADS) blk_hist[(size_t)blockIdx.x * Ep + q] = hist[q];
+}
+
+// Exclusive scans over the experts of a block of 1024 threads: s_counts[Ep] -> offsets of rows, M-blocks, pairs of
+// M-blocks and work items, in shared memory (each Ep + 1 long) and in the layout's tables.
+struct ExpertScan { int *counts, *off, *mb, *pr, *wi; };   // shared memory
+__device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const ExpertScan& sc, int (*totals)[33]) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int carry[4] = {0, 0, 0, 0};
+  for (int e0 = 0; e0 < Ep; e0 += 1024) {
+    const int e = e0 + threadIdx.x;
+    const int c = e < Ep ? sc.counts[e] : 0;
+    const int m = (c + BLOCK_M - 1) / BLOCK_M;
+    const int pr = (m + 1) >> 1;  // pairs of M-blocks (the tensor-core tile of a CTA pair)
+    // work items of the token-column GEMM kernels that merge: the units of the expert, except that an expert
+    // that merges (schedule.h) has its last two units (one block; block + tail) share one k-loop
+    const int val[4] = {c, m, pr, pr - (expert_merges(c, m) ? 1 : 0)};
+    int inc[4] = {val[0], val[1], val[2], val[3]};
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int o = __shfl_up_sync(0xffffffffu, inc[q], off);
+        if (lane >= off) inc[q] += o;
+      }
+    }
+    if (lane == 31) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) totals[q][warp] = inc[q];
+    }
+    __syncthreads();
+    if (warp < 4) {   // warp q: exclusive scan of quantity q's warp totals, the block's total behind them
+      const int w = totals[warp][lane];
+      int wi = w;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, wi, off);
+        if (lane >= off) wi += o;
+      }
+      totals[warp][lane] = wi - w;
+      if (lane == 31) totals[warp][32] = wi;
+    }
+    __syncthreads();
+    int ex[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) ex[q] = carry[q] + totals[q][warp] + inc[q] - val[q];
+    if (e < Ep) {
+      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.pr[e] = ex[2]; sc.wi[e] = ex[3];
+      lv.counts[e] = c;
+      lv.offsets[e] = ex[0];
+      lv.mb_start[e] = ex[1];
+      lv.pad_off[e] = ex[1] * BLOCK_M;
+      lv.pair_start[e] = ex[2];
+      lv.work_start[e] = ex[3];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) carry[q] += totals[q][32];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.pr[Ep] = carry[2]; sc.wi[Ep] = carry[3];
+    lv.offsets[Ep] = carry[0];
+    lv.mb_start[Ep] = carry[1];
+    lv.pad_off[Ep] = carry[1] * BLOCK_M;
+    lv.pair_start[Ep] = carry[2];
+    lv.work_start[Ep] = carry[3];
+    lv.meta[0] = carry[1];
+    lv.meta[1] = carry[1] * BLOCK_M;
+    lv.meta[2] = carry[0];
+    lv.meta[3] = carry[2];
+    lv.meta[4] = carry[3];
+  }
+  __syncthreads();
+}
+// table[i] = the last expert whose start is <= i, for i < start[Ep]
+__device__ __forceinline__ void expert_table(int Ep, const int* start, int* table) {
+  const int num = start[Ep];
+  for (int i = threadIdx.x; i < num; i += blockDim.x) {
+    int lo = 0, hi = Ep - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (start[mid] <= i) lo = mid; else hi = mid - 1;
+    }
+    table[i] = lo;
+  }
+}
+__device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, const ExpertScan& sc) {
+  expert_table(Ep, sc.mb, lv.mblk_expert);
+  expert_table(Ep, sc.pr, lv.pblk_expert);
+  expert_table(Ep, sc.wi, lv.wblk_expert);
+}
+
+// One block.  (1) per expert, exclusive scan of the block histograms over blocks: a thread per expert and range of
+// blocks (as many ranges as the block has threads for), so that the reads of a row are coalesced and independent;
+// (2) scans over experts; (3) M-block, pair and work-item -> expert tables.
+__global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int Ep, LayoutView lv) {
+  extern __shared__ int sm[];
+  __shared__ int totals[4][33];
+  const ExpertScan sc{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3};
+  int* part = sm + 5 * Ep + 4;   // [ranges][Ep]
+  pdl_trigger();
+  pdl_wait();
+  const int ranges = Ep <= 1024 ? 1024 / Ep : 1;
+  const int len = (nblk + ranges - 1) / ranges;
+  for (int q = threadIdx.x; q < ranges * Ep; q += 1024) {
+    const int g = q / Ep, e = q - g * Ep;
+    const int b1 = min(nblk, (g + 1) * len);
+    int sum = 0;
+#pragma unroll 8
+    for (int b = g * len; b < b1; ++b) sum += __ldcg(lv.blk_hist + (size_t)b * Ep + e);
+    part[q] = sum;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < Ep; e += 1024) {
+    int run = 0;
+    for (int g = 0; g < ranges; ++g) { const int c = part[g * Ep + e]; part[g * Ep + e] = run; run += c; }
+    sc.counts[e] = run;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < ranges * Ep; q += 1024) {
+    const int g = q / Ep, e = q - g * Ep;
+    const int b0 = g * len, b1 = min(nblk, b0 + len);
+    int run = part[q];
+    for (int b = b0; b < b1; b += 8) {   // eight reads in flight, then the running sums
+      int c[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c[u] = b + u < b1 ? __ldcg(lv.blk_hist + (size_t)(b + u) * Ep + e) : 0;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (b + u < b1) { lv.blk_hist[(size_t)(b + u) * Ep + e] = run; run += c[u]; }
+    }
+  }
+  scan_experts(Ep, lv, sc, totals);
+  expert_tables(Ep, lv, sc);
+}
+
+// Ranks.  WARPS warps of LAYOUT_CHUNK / WARPS slots.  The part in front of pdl_wait() -- the ids, the slots' ranks
+// inside their warp and the warps' histograms -- needs nothing of the scan kernel and runs beside it (this kernel starts
+// once every block of the histogram kernel is past its own wait, so the ids are complete).
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32) layout_rank_kernel(const int* __restrict__ ids, int n, int k, int kp, int E,
+                                                                 int Ep, LayoutView lv, DevStatus* status) {
+  constexpr int G = LAYOUT_CHUNK / WARPS / 32;   // groups of 32 slots per warp
+  extern __shared__ int sm[];
+  int* base = sm;                                              // [Ep] first row of this block's rows of the expert
+  int* pad = sm + Ep;                                          // [Ep] padded row - row of the expert
+  int* last = sm + 2 * Ep;                                     // [LAYOUT_CHUNK / kp + 2] key of the chunk's tokens
+  const int nlast = LAYOUT_CHUNK / kp + 2;
+  uint16_t* whist = reinterpret_cast<uint16_t*>(last + nlast + (nlast & 1));   // [WARPS][Ep + (Ep & 1)]
+  const int ld = Ep + (Ep & 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_trigger();
+  const int i0 = blockIdx.x * LAYOUT_CHUNK + warp * (G * 32) + lane;
+  int e[G], r[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) e[g] = i0 + 32 * g < n ? slot_expert(ids, i0 + 32 * g, k, kp, E) : -1;
+  for (int q = threadIdx.x; q < WARPS * ld / 2; q += WARPS * 32) reinterpret_cast<uint32_t*>(whist)[q] = 0;
+  for (int q = threadIdx.x; q < nlast; q += WARPS * 32) last[q] = 0;
+  __syncthreads();
+  uint16_t* mine = whist + warp * ld;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, e[g]);
+    r[g] = e[g] >= 0 ? mine[e[g]] + __popc(peers & ((1u << lane) - 1u)) : 0;
+    __syncwarp();
+    if (e[g] >= 0 && lane == __ffs(peers) - 1) mine[e[g]] += (uint16_t)__popc(peers);
     __syncwarp();
   }
   __syncthreads();
-}
-
-__global__ void __launch_bounds__(LAYOUT_THREADS) layout_hist_kernel(const int* __restrict__ ids, int n, int k,
-                                                                      int kp, int E, int Ep,
-                                                                      int* __restrict__ blk_hist, int* __restrict__ tok_last) {
-  extern __shared__ int whist[];
-  if (tok_last)   // the tokens whose first slot lies in this block's chunk
-    for (int i = blockIdx.x * LAYOUT_CHUNK + threadIdx.x; i < min(n, (blockIdx.x + 1) * LAYOUT_CHUNK); i += LAYOUT_THREADS)
-      if (i % kp == 0) tok_last[i / kp] = 0;
-  chunk_histogram(ids, n, k, kp, E, Ep, whist);
-  for (int e = threadIdx.x; e < Ep; e += LAYOUT_THREADS) {
-    int tot = 0;
-#pragma unroll
-    for (int w = 0; w < LAYOUT_WARPS; ++w) tot += whist[w * Ep + e];
-    blk_hist[(size_t)blockIdx.x * Ep + e] = tot;
-  }
-}
-
-// One block.  (1) per expert, exclusive scan of the block histograms over blocks (warp per expert);
-// (2) exclusive scans over experts for row offsets and M-block starts; (3) M-block -> expert table.
-__global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int Ep, LayoutView lv) {
-  extern __shared__ int sm[];
-  int* s_counts = sm;            // [Ep]
-  int* s_mbstart = sm + Ep;      // [Ep+1]
-  int* s_pstart = sm + 2 * Ep + 1;  // [Ep+1]
-  int* s_wstart = sm + 3 * Ep + 2;  // [Ep+1]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int e = warp; e < Ep; e += 32) {
-    int carry = 0;
-    for (int b0 = 0; b0 < nblk; b0 += 32) {
-      int b = b0 + lane;
-      int v = b < nblk ? lv.blk_hist[(size_t)b * Ep + e] : 0;
-      int incl = v;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        int o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += o;
-      }
-      if (b < nblk) lv.blk_hist[(size_t)b * Ep + e] = carry + incl - v;
-      carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) s_counts[e] = carry;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    int carry_rows = 0, carry_mb = 0, carry_pr = 0, carry_wi = 0;
-    for (int e0 = 0; e0 < Ep; e0 += 32) {
-      int e = e0 + lane;
-      int c = e < Ep ? s_counts[e] : 0;
-      int m = (c + BLOCK_M - 1) / BLOCK_M;
-      int pr = (m + 1) >> 1;  // pairs of M-blocks (the tensor-core tile of a CTA pair)
-      // work items of the token-column GEMM kernels that merge: the units of the expert, except that an expert
-      // that merges (schedule.h) has its last two units (one block; block + tail) share one k-loop
-      int wi = pr - (expert_merges(c, m) ? 1 : 0);
-      int ic = c, im = m, ip = pr, iw = wi;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        int oc = __shfl_up_sync(0xffffffffu, ic, off);
-        int om = __shfl_up_sync(0xffffffffu, im, off);
-        int op = __shfl_up_sync(0xffffffffu, ip, off);
-        int ow = __shfl_up_sync(0xffffffffu, iw, off);
-        if (lane >= off) { ic += oc; im += om; ip += op; iw += ow; }
-      }
-      if (e < Ep) {
-        lv.counts[e] = c;
-        lv.offsets[e] = carry_rows + ic - c;
-        int ms = carry_mb + im - m;
-        s_mbstart[e] = ms;
-        lv.mb_start[e] = ms;
-        lv.pad_off[e] = ms * BLOCK_M;
-        const int ps = carry_pr + ip - pr;
-        s_pstart[e] = ps;
-        lv.pair_start[e] = ps;
-        const int ws = carry_wi + iw - wi;
-        s_wstart[e] = ws;
-        lv.work_start[e] = ws;
-      }
-      carry_rows += __shfl_sync(0xffffffffu, ic, 31);
-      carry_mb += __shfl_sync(0xffffffffu, im, 31);
-      carry_pr += __shfl_sync(0xffffffffu, ip, 31);
-      carry_wi += __shfl_sync(0xffffffffu, iw, 31);
-    }
-    if (lane == 0) {
-      lv.offsets[Ep] = carry_rows;
-      s_mbstart[Ep] = carry_mb;
-      lv.mb_start[Ep] = carry_mb;
-      lv.pad_off[Ep] = carry_mb * BLOCK_M;
-      lv.meta[0] = carry_mb;
-      lv.meta[1] = carry_mb * BLOCK_M;
-      lv.meta[2] = carry_rows;
-      s_pstart[Ep] = carry_pr;
-      lv.pair_start[Ep] = carry_pr;
-      lv.meta[3] = carry_pr;
-      s_wstart[Ep] = carry_wi;
-      lv.work_start[Ep] = carry_wi;
-      lv.meta[4] = carry_wi;
-    }
-  }
-  __syncthreads();
-  const int num_mb = s_mbstart[Ep];
-  for (int mb = threadIdx.x; mb < num_mb; mb += blockDim.x) {
-    int lo = 0, hi = Ep - 1;  // last expert whose mb_start <= mb
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (s_mbstart[mid] <= mb) lo = mid; else hi = mid - 1;
-    }
-    lv.mblk_expert[mb] = lo;
-  }
-  const int num_pr = s_pstart[Ep];
-  for (int pb = threadIdx.x; pb < num_pr; pb += blockDim.x) {
-    int lo = 0, hi = Ep - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (s_pstart[mid] <= pb) lo = mid; else hi = mid - 1;
-    }
-    lv.pblk_expert[pb] = lo;
-  }
-  const int num_wi = s_wstart[Ep];
-  for (int wb = threadIdx.x; wb < num_wi; wb += blockDim.x) {
-    int lo = 0, hi = Ep - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (s_wstart[mid] <= wb) lo = mid; else hi = mid - 1;
-    }
-    lv.wblk_expert[wb] = lo;
-  }
-}
-
-__global__ void __launch_bounds__(LAYOUT_THREADS) layout_rank_kernel(const int* __restrict__ ids, int n, int k,
-                                                                      int kp, int E, int Ep, LayoutView lv,
-                                                                      DevStatus* status) {
-  extern __shared__ int whist[];
-  chunk_histogram(ids, n, k, kp, E, Ep, whist);
-  // per expert: running base of each warp inside the block = block prefix + earlier warps
-  for (int e = threadIdx.x; e < Ep; e += LAYOUT_THREADS) {
-    int run = lv.blk_hist[(size_t)blockIdx.x * Ep + e];
-#pragma unroll
-    for (int w = 0; w < LAYOUT_WARPS; ++w) {
-      int c = whist[w * Ep + e];
-      whist[w * Ep + e] = run;
+  // per expert: the block's rows in front of each warp's
+  for (int q = threadIdx.x; q < Ep; q += WARPS * 32) {
+    int run = 0;
+#pragma unroll 8
+    for (int w = 0; w < WARPS; ++w) {
+      const int c = whist[w * ld + q];
+      whist[w * ld + q] = (uint16_t)run;
       run += c;
     }
   }
+  pdl_wait();
+  for (int q = threadIdx.x; q < Ep; q += WARPS * 32) {
+    const int off = __ldcg(lv.offsets + q);
+    base[q] = off + __ldcg(lv.blk_hist + (size_t)blockIdx.x * Ep + q);
+    pad[q] = __ldcg(lv.pad_off + q) - off;
+  }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int* mine = whist + warp * Ep;
-  const int base = blockIdx.x * LAYOUT_CHUNK + warp * SLOTS_PER_WARP;
-  for (int g = 0; g < SLOTS_PER_WARP; g += 32) {
-    int i = base + g + lane;
-    int e = i < n ? slot_expert(ids, i, k, kp, E) : -1;
-    uint32_t peers = __match_any_sync(0xffffffffu, e);
-    int r = 0;
-    if (e >= 0) r = mine[e] + __popc(peers & ((1u << lane) - 1u));
-    __syncwarp();
-    if (e >= 0 && lane == __ffs(peers) - 1) mine[e] += __popc(peers);
-    __syncwarp();
-    if (i < n) {
-      if (e >= 0) {
-        int row = lv.offsets[e] + r;
-        lv.row_of[i] = row;
-        lv.prow_of[i] = lv.pad_off[e] + r;
-        lv.src_of[row] = i;
-        // the combine order's key: the token's last ROUTED row (shared experts are taken first by the persistent launch)
-        if (lv.tok_last && i % kp < k) atomicMax(&lv.tok_last[i / kp], lv.pad_off[e] + r + 1);
-      } else {
-        lv.row_of[i] = -1;
-        lv.prow_of[i] = -1;
-        note(status, /*MOE_ERR_BAD_EXPERT_ID*/ 1, i);  // the slot is dropped, the layer carries on
-      }
+  const int t_first = blockIdx.x * LAYOUT_CHUNK / kp;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int i = i0 + 32 * g;
+    if (i >= n) continue;
+    if (e[g] >= 0) {
+      const int row = base[e[g]] + mine[e[g]] + r[g], prow = row + pad[e[g]];
+      lv.row_of[i] = row;
+      lv.prow_of[i] = prow;
+      lv.src_of[row] = i;
+      // the combine order's key: the token's last ROUTED row (shared experts are taken first by the persistent launch)
+      if (lv.tok_last && i % kp < k) atomicMax(&last[i / kp - t_first], prow + 1);
+    } else {
+      lv.row_of[i] = -1;
+      lv.prow_of[i] = -1;
+      note(status, /*MOE_ERR_BAD_EXPERT_ID*/ 1, i);  // the slot is dropped, the layer carries on
     }
   }
+  if (!lv.tok_last) return;
+  __syncthreads();
+  for (int q = threadIdx.x; q < nlast; q += WARPS * 32)   // a token whose slots straddle two chunks gets both chunks' keys
+    if (last[q]) atomicMax(&lv.tok_last[t_first + q], last[q]);
 }
 
-// Combine order of the persistent launch: tokens sorted by the M-block of their LAST row in the expert-ordered
-// row space (a counting sort; one block).  The operators walk the experts in order, so this is the order in
-// which tokens become complete: combine tasks taken in this order find their dependent events met one after
-// the other instead of all at the very end.  Tokens without any row come first.
-constexpr int ORDER_MAX_BINS = 12000;   // bins (M-blocks + 1) that fit the block's shared memory
-__global__ void __launch_bounds__(1024) layout_order_kernel(int T, int kp, LayoutView lv) {
-  extern __shared__ int bins[];
-  __shared__ int carry_s;
-  __shared__ int warp_sums[32];
-  const int nb = lv.meta[0] + 1;
-  if (nb > ORDER_MAX_BINS) {   // beyond the shared-memory histogram: token order
-    for (int t = threadIdx.x; t < T; t += blockDim.x) lv.combine_order[t] = t;
-    return;
-  }
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) bins[i] = 0;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  auto key_of = [&](int t) {   // tok_last[t] = 1 + the token's largest padded row (0: no row), from the rank kernel
-    const int last = lv.tok_last[t];
-    return last == 0 ? 0 : (last - 1) / BLOCK_M + 1;
-  };
-  for (int t = threadIdx.x; t < T; t += blockDim.x) atomicAdd(&bins[key_of(t)], 1);
-  __syncthreads();
-  // exclusive scan of the bins, 1024 at a time
+// Exclusive scan of bins[nb] in shared memory by a block of 1024 threads.
+__device__ __forceinline__ void scan_bins(int* bins, int nb, int* warp_sums, int* carry_s) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int base = 0; base < nb; base += blockDim.x) {
+  for (int base = 0; base < nb; base += 1024) {
     const int i = base + threadIdx.x;
     const int v = i < nb ? bins[i] : 0;
     int incl = v;
@@ -341,33 +361,174 @@ __global__ void __launch_bounds__(1024) layout_order_kernel(int T, int kp, Layou
       warp_sums[lane] = wi - w;
     }
     __syncthreads();
-    const int excl = carry_s + warp_sums[warp] + incl - v;
+    const int excl = *carry_s + warp_sums[warp] + incl - v;
     if (i < nb) bins[i] = excl;
     __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry_s = excl + v;
+    if (threadIdx.x == 1023) *carry_s = excl + v;
     __syncthreads();
   }
-  for (int t = threadIdx.x; t < T; t += blockDim.x) lv.combine_order[atomicAdd(&bins[key_of(t)], 1)] = t;
+}
+// Key of a token in the combine order from `last` = 1 + its largest padded routed row (0: no row).
+__device__ __forceinline__ int order_key(int last) { return last == 0 ? 0 : (last - 1) / BLOCK_M + 1; }
+
+// Combine order of the persistent launch: tokens sorted by the M-block of their LAST row in the expert-ordered
+// row space (a counting sort; one block).  The operators walk the experts in order, so this is the order in
+// which tokens become complete: combine tasks taken in this order find their dependent events met one after
+// the other instead of all at the very end.  Tokens without any row come first.
+constexpr int ORDER_MAX_BINS = 12000;   // bins (M-blocks + 1) that fit the block's shared memory
+__global__ void __launch_bounds__(1024) layout_order_kernel(int T, LayoutView lv) {
+  extern __shared__ int bins[];
+  __shared__ int carry_s;
+  __shared__ int warp_sums[32];
+  if (threadIdx.x == 0) carry_s = 0;
+  pdl_trigger();
+  pdl_wait();
+  const int nb = __ldcg(lv.meta) + 1;
+  if (nb > ORDER_MAX_BINS) {   // beyond the shared-memory histogram: token order
+    for (int t = threadIdx.x; t < T; t += 1024) lv.combine_order[t] = t;
+    return;
+  }
+  for (int i = threadIdx.x; i < nb; i += 1024) bins[i] = 0;
+  __syncthreads();
+  // sixteen tokens per thread at a time: their keys are read together and kept for the second pass
+  constexpr int U = 16;
+  int key[U];
+  for (int t0 = threadIdx.x; t0 < T; t0 += U * 1024) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) key[u] = t0 + u * 1024 < T ? __ldcg(lv.tok_last + t0 + u * 1024) : -1;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (key[u] >= 0) atomicAdd(&bins[key[u] = order_key(key[u])], 1);
+  }
+  __syncthreads();
+  scan_bins(bins, nb, warp_sums, &carry_s);
+  const bool kept = T <= U * 1024;
+  for (int t0 = threadIdx.x; t0 < T; t0 += U * 1024) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (t0 + u * 1024 < T)
+        lv.combine_order[atomicAdd(&bins[kept ? key[u] : order_key(__ldcg(lv.tok_last + t0 + u * 1024))], 1)] = t0 + u * 1024;
+  }
 }
 
-cudaError_t launch_layout_order(const Dims& dm, const LayoutView& lv, int cap_mblocks, cudaStream_t s, int* launches) {
-  int nb = cap_mblocks + 2;
-  if (nb > ORDER_MAX_BINS) nb = ORDER_MAX_BINS;
-  layout_order_kernel<<<1, 1024, sizeof(int) * (size_t)nb, s>>>(dm.T, dm.kp(), lv);
-  ++*launches;
-  return cudaGetLastError();
+// The whole layout of fewer than LAYOUT_ONE_SLOTS slots in one block: a thread per slot in the first 31 warps, tables
+// in shared memory, nothing read back.  Token generation (V3-shaped layer, 64 tokens) spends 8 us here against 45 us
+// in the four kernels and the clearing of the counters.  One chunk of the large form would hold 2048 slots, but its three short kernels overlap, and from a
+// thousand slots on they are as fast.
+constexpr int LAYOUT_ONE_WARPS = 31;
+constexpr int LAYOUT_ONE_SLOTS = 32 * LAYOUT_ONE_WARPS;
+constexpr int LAYOUT_ONE_EXPERTS = 384;   // shared memory without opt-in: 48 KB
+__global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict__ ids, int n, int T, int k, int kp, int E,
+                                                          int Ep, LayoutView lv, int want_order, DevStatus* status,
+                                                          int* __restrict__ zero, int nzero) {
+  extern __shared__ int sm[];
+  __shared__ int totals[4][33];
+  __shared__ int carry_s;
+  const ExpertScan sc{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3};
+  int* s_last = sm + 5 * Ep + 4;                       // [LAYOUT_ONE_SLOTS] 1 + padded row of the slot
+  int* bins = s_last + LAYOUT_ONE_SLOTS;               // [LAYOUT_ONE_SLOTS + 1]
+  uint16_t* whist = reinterpret_cast<uint16_t*>(bins + LAYOUT_ONE_SLOTS + 2 + (Ep & 1));   // [warps in use][ld]
+  const int ld = Ep + (Ep & 1);
+  const int warps = (n + 31) >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = threadIdx.x;
+  for (int q = threadIdx.x; q < warps * ld / 2; q += 1024) reinterpret_cast<uint32_t*>(whist)[q] = 0;
+  if (i <= LAYOUT_ONE_SLOTS) bins[i] = 0;
+  if (i == 0) carry_s = 0;
+  pdl_trigger();
+  pdl_wait();
+  const int e = i < n ? slot_expert(ids, i, k, kp, E) : -1;
+  for (int q = threadIdx.x; q < nzero; q += 1024) zero[q] = 0;
+  __syncthreads();
+  int r = 0;
+  if (warp < warps) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, e);
+    r = __popc(peers & ((1u << lane) - 1u));
+    if (e >= 0 && r == 0) whist[warp * ld + e] = (uint16_t)__popc(peers);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < Ep; q += 1024) {
+    int run = 0;
+#pragma unroll 8
+    for (int w = 0; w < warps; ++w) {
+      const int c = whist[w * ld + q];
+      whist[w * ld + q] = (uint16_t)run;
+      run += c;
+    }
+    sc.counts[q] = run;
+  }
+  __syncthreads();
+  scan_experts(Ep, lv, sc, totals);
+  if (i < n) {
+    int prow = -1;
+    if (e >= 0) {
+      const int in_expert = whist[warp * ld + e] + r, row = sc.off[e] + in_expert;
+      prow = sc.mb[e] * BLOCK_M + in_expert;
+      lv.row_of[i] = row;
+      lv.src_of[row] = i;
+    } else {
+      lv.row_of[i] = -1;
+      note(status, /*MOE_ERR_BAD_EXPERT_ID*/ 1, i);
+    }
+    lv.prow_of[i] = prow;
+    s_last[i] = prow + 1;
+  }
+  expert_tables(Ep, lv, sc);
+  if (!want_order) return;
+  __syncthreads();
+  int key = 0, at = 0;
+  if (i < T) {
+    int last = 0;
+    for (int j = 0; j < k; ++j) last = max(last, s_last[i * kp + j]);
+    key = order_key(last);   // at most the number of M-blocks, which is at most n
+    at = atomicAdd(&bins[key], 1);
+  }
+  __syncthreads();
+  scan_bins(bins, sc.mb[Ep] + 1, totals[0], &carry_s);
+  if (i < T) lv.combine_order[bins[key] + at] = i;
 }
 
-cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView& lv, DevStatus* status,
-                          cudaStream_t s, int* launches) {
-  const int n = dm.slots(), Ep = dm.Ep();
+cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView& lv, bool want_order, int cap_mblocks,
+                          int* zero, int nzero, DevStatus* status, cudaStream_t s, int* launches) {
+  const int n = dm.slots(), Ep = dm.Ep(), kp = dm.kp();
+  cudaError_t e;
+  if (n < LAYOUT_ONE_SLOTS && Ep <= LAYOUT_ONE_EXPERTS) {
+    const size_t smem = sizeof(int) * (size_t)(5 * Ep + 8 + 2 * LAYOUT_ONE_SLOTS) +
+                        sizeof(uint16_t) * (size_t)((n + 31) / 32) * (Ep + (Ep & 1));
+    ++*launches;
+    return launch_dependent(layout_one_kernel, dim3(1), dim3(1024), smem, s, topk_ids, n, dm.T, dm.k, kp, dm.E, Ep, lv,
+                            want_order ? 1 : 0, status, zero, nzero);
+  }
   const int nblk = n > 0 ? (n + LAYOUT_CHUNK - 1) / LAYOUT_CHUNK : 1;
-  const size_t sm_hist = sizeof(int) * (size_t)LAYOUT_WARPS * Ep;
-  layout_hist_kernel<<<nblk, LAYOUT_THREADS, sm_hist, s>>>(topk_ids, n, dm.k, dm.kp(), dm.E, Ep, lv.blk_hist, lv.tok_last);
-  layout_scan_kernel<<<1, 1024, sizeof(int) * (size_t)(4 * Ep + 3), s>>>(nblk, Ep, lv);
-  layout_rank_kernel<<<nblk, LAYOUT_THREADS, sm_hist, s>>>(topk_ids, n, dm.k, dm.kp(), dm.E, Ep, lv, status);
+  int* const tok_last = want_order ? lv.tok_last : nullptr;
+  LayoutView lr = lv;
+  lr.tok_last = tok_last;
+  if ((e = launch_dependent(layout_hist_kernel, dim3(nblk), dim3(HIST_THREADS), sizeof(int) * (size_t)Ep, s, topk_ids, n, dm.k,
+                            kp, dm.E, Ep, lv.blk_hist, tok_last, zero, nzero)))
+    return e;
+  const int ranges = Ep <= 1024 ? 1024 / Ep : 1;
+  if ((e = launch_dependent(layout_scan_kernel, dim3(1), dim3(1024), sizeof(int) * ((size_t)(5 + ranges) * Ep + 4), s, nblk, Ep, lv)))
+    return e;
+  const size_t nlast = LAYOUT_CHUNK / kp + 2;
+  auto rank_smem = [&](int warps) {
+    return sizeof(int) * (2 * (size_t)Ep + nlast + (nlast & 1)) + sizeof(uint16_t) * (size_t)warps * (Ep + (Ep & 1));
+  };
+  // as many warps as have room for their histograms in 48 KB of shared memory (32 up to about 500 experts)
+  constexpr size_t ROOM = 48 * 1024;
+  if (rank_smem(32) <= ROOM)
+    e = launch_dependent(layout_rank_kernel<32>, dim3(nblk), dim3(1024), rank_smem(32), s, topk_ids, n, dm.k, kp, dm.E, Ep, lr, status);
+  else if (rank_smem(16) <= ROOM)
+    e = launch_dependent(layout_rank_kernel<16>, dim3(nblk), dim3(512), rank_smem(16), s, topk_ids, n, dm.k, kp, dm.E, Ep, lr, status);
+  else
+    e = launch_dependent(layout_rank_kernel<8>, dim3(nblk), dim3(256), rank_smem(8), s, topk_ids, n, dm.k, kp, dm.E, Ep, lr, status);
+  if (e) return e;
   *launches += 3;
-  return cudaGetLastError();
+  if (want_order) {
+    int nb = cap_mblocks + 2;
+    if (nb > ORDER_MAX_BINS) nb = ORDER_MAX_BINS;
+    if ((e = launch_dependent(layout_order_kernel, dim3(1), dim3(1024), sizeof(int) * (size_t)nb, s, dm.T, lv))) return e;
+    ++*launches;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace moe
@@ -445,8 +606,6 @@ extern "C" int moe_layout_noalloc(const int32_t* topk_ids, int32_t T, int32_t E,
     sc = g_na_ptr[dev];
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the array keeps the previous call's contents: the status word must start at zero
-  if (cudaMemsetAsync(&sc->status, 0, sizeof(moe::DevStatus), st) != cudaSuccess) return MOE_ERR_CUDA;
   moe::Dims dm{T, 8, E, k, n_shared, 8};
   moe::LayoutView lv{};   // (fields not set below stay NULL: no combine order here)
   lv.counts = counts;
@@ -464,7 +623,10 @@ extern "C" int moe_layout_noalloc(const int32_t* topk_ids, int32_t T, int32_t E,
   lv.meta = sc->meta;
   lv.blk_hist = sc->blk_hist;
   int launches = 0;
-  if (moe::launch_layout(topk_ids, dm, lv, &sc->status, st, &launches) != cudaSuccess) return MOE_ERR_CUDA;
+  // the array keeps the previous call's contents: the first kernel clears the status word
+  if (moe::launch_layout(topk_ids, dm, lv, false, 0, reinterpret_cast<int*>(&sc->status), sizeof(moe::DevStatus) / sizeof(int),
+                         &sc->status, st, &launches) != cudaSuccess)
+    return MOE_ERR_CUDA;
   if (status2 &&
       cudaMemcpyAsync(status2, &sc->status, 2 * sizeof(int), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return MOE_ERR_CUDA;
