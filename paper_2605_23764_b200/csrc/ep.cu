@@ -8,7 +8,9 @@
 #include <vector>
 
 #include "../../include/moe_b200.h"
+#include "launch_pairs.cuh"
 #include "moe_internal.h"
+#include "topk.cuh"
 
 namespace moe {
 
@@ -95,6 +97,19 @@ __device__ __forceinline__ bool ep_wait(const int* counter, int threshold, const
 
 struct EpPeers { moe_ep_peer p[MOE_EP_MAX_RANKS]; };
 
+// Counters, tickets and status a call starts from: up to two arrays per rank and the status words, cleared by one
+// kernel (a memset each was 17 launches of 4 us in front of each half of an eight-rank exchange).
+struct EpClearArgs {
+  int* ptr[2 * MOE_EP_MAX_RANKS + 1];
+  int count[2 * MOE_EP_MAX_RANKS + 1];
+  int n;
+  void add(int* p, int c) { ptr[n] = p; count[n] = c; ++n; }
+};
+__global__ void __launch_bounds__(256) ep_clear_kernel(const __grid_constant__ EpClearArgs a) {
+  pdl_wait();
+  for (int i = threadIdx.x; i < a.count[blockIdx.x]; i += 256) a.ptr[blockIdx.x][i] = 0;
+}
+
 struct EpDispatchArgs {
   EpPeers peers;
   moe_ep_local locals[MOE_EP_MAX_RANKS];
@@ -105,20 +120,24 @@ struct EpDispatchArgs {
 };
 
 // Dispatch.  Producer block: one communication task at a time (rows of one expert bound for one rank), a warp per row.
+// Where one launch plays several ranks, their task lists are worked off one rank after the other by all producers: a
+// token's row is read once per routed copy, and the rows of the ranks in flight then fit L2 (all eight ranks side by side
+// read 600 MB from DRAM for 117 MB of tokens).
 // Consumer block: the receive buffer of its rank, one 128-row block at a time, as soon as the block's rows have arrived.
 __global__ void __launch_bounds__(EP_THREADS, 4) ep_dispatch_kernel(const __grid_constant__ EpDispatchArgs a) {
   const WaitCtl wc{a.status, a.budget_ns};
-  const int li = blockIdx.x / a.blocks_per_rank, role = blockIdx.x % a.blocks_per_rank;
-  const moe_ep_local& me = a.locals[li];
+  const int own = blockIdx.x / a.blocks_per_rank, role = blockIdx.x % a.blocks_per_rank;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nvec = a.d >> 3;
   __shared__ int task_s, ok_s;
-  if (role < a.producers_per_rank || !me.consumed) {   // without a consumer buffer every block of the rank produces
-    while (true) {
+  if (role < a.producers_per_rank || !a.locals[own].consumed) {   // without a consumer buffer every block of the rank produces
+    for (int li = 0; li < a.n_local;) {
+      const moe_ep_local& me = a.locals[li];
       if (threadIdx.x == 0) task_s = atomicAdd(me.ticket, 1);
       __syncthreads();
       const int ti = task_s;
-      if (ti >= me.n_tasks) break;
+      __syncthreads();
+      if (ti >= me.n_tasks) { ++li; continue; }
       const moe_ep_task tk = me.tasks[ti];
       // a task list that is not this rank's plan must not steer stores: what can be checked here is
       if ((unsigned)tk.dst_rank >= (unsigned)a.R || tk.nrows < 0 || tk.nrows > MOE_EP_TILE_ROWS || tk.src_row0 < 0 ||
@@ -150,6 +169,7 @@ __global__ void __launch_bounds__(EP_THREADS, 4) ep_dispatch_kernel(const __grid
       }
     }
   } else {
+    const moe_ep_local& me = a.locals[own];
     const int ci = role - a.producers_per_rank, nc = a.blocks_per_rank - a.producers_per_rank;
     const moe_ep_peer& mine = a.peers.p[me.rank];
     const int nblk = (me.recv_rows + MOE_EP_BLOCK_ROWS - 1) / MOE_EP_BLOCK_ROWS;
@@ -186,8 +206,13 @@ struct EpCombineArgs {
 // Combine.  Producer block: tiles of 32 rows of the rank's expert outputs, each row returned to ret[slot] of its
 // source rank (a warp per row); when the tile's rows are stored, one thread per row signals (the fences of a tile run
 // side by side instead of one after the other); the tile list starts at a rank-dependent position so that the
-// ranks do not all return to the same source at once.  Consumer block: token blocks of its rank; once every row of a
-// block has come back, out[t] = sum over the token's k rows in slot order (fp32).
+// ranks do not all return to the same source at once.
+// Consumer block: groups of EP_SUM_TOKENS tokens of its rank by ticket; once every row of the group's token block has come
+// back, out[t] = sum over the token's k rows in slot order (fp32), a warp per token.  A token block is complete only
+// when the last expert's rows are back, so nearly all sums run after the producers: every producer joins the
+// consumers when its tiles are gone (a quarter of the blocks doing all sums was a tail of 300 us on 65536 rows of 14 KB).
+constexpr int EP_SUM_TOKENS = EP_WARPS;
+static_assert(MOE_EP_TOKEN_BLOCK % EP_SUM_TOKENS == 0, "a group lies in one token block");
 __global__ void __launch_bounds__(EP_THREADS, 4) ep_combine_kernel(const __grid_constant__ EpCombineArgs a) {
   const WaitCtl wc{a.status, a.budget_ns};
   const int li = blockIdx.x / a.blocks_per_rank, role = blockIdx.x % a.blocks_per_rank;
@@ -223,58 +248,82 @@ __global__ void __launch_bounds__(EP_THREADS, 4) ep_combine_kernel(const __grid_
       __syncthreads();   // every row of the tile is stored: one thread per row makes them visible and signals
       if ((int)threadIdx.x < n && sig_s[threadIdx.x]) ep_signal(sig_s[threadIdx.x], 1);
     }
-  } else {
-    const int ci = role - a.producers_per_rank, nc = a.blocks_per_rank - a.producers_per_rank;
-    const int nblk = (me.T + MOE_EP_TOKEN_BLOCK - 1) / MOE_EP_TOKEN_BLOCK;
-    for (int b = ci; b < nblk; b += nc) {
-      const int t0 = b * MOE_EP_TOKEN_BLOCK, nt = min(MOE_EP_TOKEN_BLOCK, me.T - t0);
-      if (threadIdx.x == 0) ok_s = ep_wait(mine.ret_counters + b, nt * a.k, wc, b) ? 1 : 0;
-      __syncthreads();
-      if (!ok_s) break;
-      for (int t = t0 + warp; t < t0 + nt; t += EP_WARPS) {
-        for (int v = lane; v < nvec; v += 32) {
-          float acc[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) acc[q] = 0.f;
-          for (int j0 = 0; j0 < a.k; j0 += 8) {   // eight of the token's rows in flight; summed in slot order
-            uint4 rr[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              if (j0 + u < a.k) rr[u] = ep_ld_cg(reinterpret_cast<const uint4*>(mine.ret + ((size_t)t * a.k + j0 + u) * a.d) + v);
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              if (j0 + u < a.k) {
-                const uint4 r = rr[u];
-                acc[0] += bf16lo(r.x); acc[1] += bf16hi(r.x);
-                acc[2] += bf16lo(r.y); acc[3] += bf16hi(r.y);
-                acc[4] += bf16lo(r.z); acc[5] += bf16hi(r.z);
-                acc[6] += bf16lo(r.w); acc[7] += bf16hi(r.w);
-              }
-          }
-          uint4 o;
-          o.x = pack_bf16x2(acc[0], acc[1]); o.y = pack_bf16x2(acc[2], acc[3]);
-          o.z = pack_bf16x2(acc[4], acc[5]); o.w = pack_bf16x2(acc[6], acc[7]);
-          reinterpret_cast<uint4*>(me.out + (size_t)t * a.d)[v] = o;
-        }
+  }
+  const int ngroups = (me.T + EP_SUM_TOKENS - 1) / EP_SUM_TOKENS;
+  while (true) {
+    if (threadIdx.x == 0) {
+      const int g = atomicAdd(me.ticket + 1, 1);
+      task_s = g;
+      ok_s = 1;
+      if (g < ngroups) {
+        const int b = g * EP_SUM_TOKENS / MOE_EP_TOKEN_BLOCK, t0 = b * MOE_EP_TOKEN_BLOCK;
+        ok_s = ep_wait(mine.ret_counters + b, min(MOE_EP_TOKEN_BLOCK, me.T - t0) * a.k, wc, b) ? 1 : 0;
       }
-      __syncthreads();
     }
+    __syncthreads();
+    const int g = task_s;
+    if (g >= ngroups || !ok_s) break;
+    const int t = g * EP_SUM_TOKENS + warp;
+    if (t < me.T) {
+      for (int v = lane; v < nvec; v += 32) {
+        float acc[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+        for (int j0 = 0; j0 < a.k; j0 += 8) {   // eight of the token's rows in flight; summed in slot order
+          uint4 rr[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (j0 + u < a.k) rr[u] = ep_ld_cg(reinterpret_cast<const uint4*>(mine.ret + ((size_t)t * a.k + j0 + u) * a.d) + v);
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            if (j0 + u < a.k) {
+              const uint4 r = rr[u];
+              acc[0] += bf16lo(r.x); acc[1] += bf16hi(r.x);
+              acc[2] += bf16lo(r.y); acc[3] += bf16hi(r.y);
+              acc[4] += bf16lo(r.z); acc[5] += bf16hi(r.z);
+              acc[6] += bf16lo(r.w); acc[7] += bf16hi(r.w);
+            }
+        }
+        uint4 o;
+        o.x = pack_bf16x2(acc[0], acc[1]); o.y = pack_bf16x2(acc[2], acc[3]);
+        o.z = pack_bf16x2(acc[4], acc[5]); o.w = pack_bf16x2(acc[6], acc[7]);
+        reinterpret_cast<uint4*>(me.out + (size_t)t * a.d)[v] = o;
+      }
+    }
+    __syncthreads();
   }
 }
 
-// resident blocks a cooperative launch may use, split among the local ranks; three of four blocks produce
-static int ep_grid(const void* kernel, int n_local, int* blocks_per_rank, int* producers_per_rank) {
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return MOE_ERR_NO_DEVICE;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, EP_THREADS, 0) != cudaSuccess || per_sm < 1)
-    return MOE_ERR_CUDA;
-  int total = sms * (per_sm < 4 ? per_sm : 4);
+// Resident blocks a cooperative launch may use (a property of kernel and device, looked up once per device), split among
+// the local ranks; three of four blocks produce.
+struct EpGrid {
+  std::mutex mu;
+  int blocks[MAX_DEVICES] = {};
+};
+static int ep_grid(EpGrid& g, const void* kernel, int dev, int n_local, int* blocks_per_rank, int* producers_per_rank) {
+  int total = 0;
+  {
+    std::lock_guard<std::mutex> lock(g.mu);
+    if (!g.blocks[dev]) {
+      int sms = 0, per_sm = 0;
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, EP_THREADS, 0) != cudaSuccess || per_sm < 1)
+        return MOE_ERR_CUDA;
+      g.blocks[dev] = sms * (per_sm < 4 ? per_sm : 4);
+    }
+    total = g.blocks[dev];
+  }
   int bpr = total / n_local;
   if (bpr < 2) return MOE_ERR_TOO_LARGE;
   *blocks_per_rank = bpr;
   *producers_per_rank = bpr - (bpr + 3) / 4;
   return MOE_OK;
+}
+static int ep_device(int* dev) {
+  int major = 0;
+  if (cudaGetDevice(dev) != cudaSuccess || *dev < 0 || *dev >= MAX_DEVICES) return MOE_ERR_NO_DEVICE;
+  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, *dev);
+  return major == 10 ? MOE_OK : MOE_ERR_NO_DEVICE;
 }
 
 }  // namespace moe
@@ -338,10 +387,10 @@ int moe_ep_dispatch(const moe_ep_peer* peers, const moe_ep_local* locals, int32_
     return MOE_ERR_INVALID_ARG;
   if (ep_check_peers(peers, R)) return MOE_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int major = 0, dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return MOE_ERR_NO_DEVICE;
-  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-  if (major != 10) return MOE_ERR_NO_DEVICE;
+  int dev = 0;
+  if (ep_device(&dev)) return MOE_ERR_NO_DEVICE;
+  EpClearArgs clear;
+  clear.n = 0;
   EpDispatchArgs a;
   memset(&a, 0, sizeof a);
   for (int q = 0; q < R; ++q) a.peers.p[q] = peers[q];
@@ -350,18 +399,20 @@ int moe_ep_dispatch(const moe_ep_peer* peers, const moe_ep_local* locals, int32_
     if (l.rank < 0 || l.rank >= R || l.T < 0 || l.n_tasks < 0 || l.recv_rows < 0 || !l.ticket || (l.n_tasks && !l.tasks) ||
         (l.T && (!l.x || !l.topk_w || !l.src_of)) || (l.recv_rows && (!peers[l.rank].recv || !peers[l.rank].recv_meta)))
       return MOE_ERR_INVALID_ARG;
-    if (cudaMemsetAsync(l.ticket, 0, 2 * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
+    clear.add(l.ticket, 2);
     const int nblk = (l.recv_rows + MOE_EP_BLOCK_ROWS - 1) / MOE_EP_BLOCK_ROWS;
-    if (nblk && cudaMemsetAsync(peers[l.rank].recv_counters, 0, sizeof(int) * (size_t)nblk, st) != cudaSuccess) return MOE_ERR_CUDA;
+    if (nblk) clear.add(peers[l.rank].recv_counters, nblk);
   }
-  if (cudaMemsetAsync(status, 0, 4 * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
+  clear.add(status, 4);
   for (int i = 0; i < n_local; ++i) a.locals[i] = locals[i];
   a.n_local = n_local; a.R = R; a.k = k; a.d = d;
   a.status = reinterpret_cast<DevStatus*>(status);
   a.budget_ns = 2000ull * 1000 * 1000;
   const void* fn = reinterpret_cast<const void*>(ep_dispatch_kernel);
-  int rc = ep_grid(fn, n_local, &a.blocks_per_rank, &a.producers_per_rank);
+  static EpGrid grid;
+  int rc = ep_grid(grid, fn, dev, n_local, &a.blocks_per_rank, &a.producers_per_rank);
   if (rc) return rc;
+  if (launch_dependent(ep_clear_kernel, dim3(clear.n), dim3(256), 0, st, clear) != cudaSuccess) return MOE_ERR_CUDA;
   void* params[] = {&a};
   // cooperative: consumer blocks wait for producer blocks of the same launch
   cudaError_t e = study_plain_launch().load()   // profiling aid, see moe_debug_set_plain_launch(NULL, ..)
@@ -376,10 +427,10 @@ int moe_ep_combine(const moe_ep_peer* peers, const moe_ep_local_combine* locals,
     return MOE_ERR_INVALID_ARG;
   if (ep_check_peers(peers, R)) return MOE_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int major = 0, dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return MOE_ERR_NO_DEVICE;
-  cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
-  if (major != 10) return MOE_ERR_NO_DEVICE;
+  int dev = 0;
+  if (ep_device(&dev)) return MOE_ERR_NO_DEVICE;
+  EpClearArgs clear;
+  clear.n = 0;
   EpCombineArgs a;
   memset(&a, 0, sizeof a);
   for (int q = 0; q < R; ++q) a.peers.p[q] = peers[q];
@@ -388,18 +439,20 @@ int moe_ep_combine(const moe_ep_peer* peers, const moe_ep_local_combine* locals,
     if (l.rank < 0 || l.rank >= R || l.T < 0 || l.recv_rows < 0 || !l.ticket || (l.recv_rows && (!l.y || !peers[l.rank].recv_meta)) ||
         (l.T && (!l.out || !peers[l.rank].ret)))
       return MOE_ERR_INVALID_ARG;
-    if (cudaMemsetAsync(l.ticket, 0, 2 * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
+    clear.add(l.ticket, 2);
     const int nblk = (l.T + MOE_EP_TOKEN_BLOCK - 1) / MOE_EP_TOKEN_BLOCK;
-    if (nblk && cudaMemsetAsync(peers[l.rank].ret_counters, 0, sizeof(int) * (size_t)nblk, st) != cudaSuccess) return MOE_ERR_CUDA;
+    if (nblk) clear.add(peers[l.rank].ret_counters, nblk);
   }
-  if (cudaMemsetAsync(status, 0, 4 * sizeof(int), st) != cudaSuccess) return MOE_ERR_CUDA;
+  clear.add(status, 4);
   for (int i = 0; i < n_local; ++i) a.locals[i] = locals[i];
   a.n_local = n_local; a.R = R; a.k = k; a.d = d;
   a.status = reinterpret_cast<DevStatus*>(status);
   a.budget_ns = 2000ull * 1000 * 1000;
   const void* fn = reinterpret_cast<const void*>(ep_combine_kernel);
-  int rc = ep_grid(fn, n_local, &a.blocks_per_rank, &a.producers_per_rank);
+  static EpGrid grid;
+  int rc = ep_grid(grid, fn, dev, n_local, &a.blocks_per_rank, &a.producers_per_rank);
   if (rc) return rc;
+  if (launch_dependent(ep_clear_kernel, dim3(clear.n), dim3(256), 0, st, clear) != cudaSuccess) return MOE_ERR_CUDA;
   void* params[] = {&a};
   cudaError_t e = study_plain_launch().load()
                       ? cudaLaunchKernel(fn, dim3(a.blocks_per_rank * n_local), dim3(EP_THREADS), params, 0, st)
