@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 
 import torch
 
@@ -155,27 +156,34 @@ def load_library() -> ctypes.CDLL:
 
 
 def _check(rc: int, what: str):
-    if rc != 0:
+    if rc:
         lib = load_library()
         msg = lib.moe_strerror(rc).decode()
         extra = lib.moe_last_cuda_error().decode()
         raise MoeError(f"{what}: {msg} ({rc})" + (f" [{extra}]" if extra and rc == -3 else ""))
 
 
-def _dev(t, dtype, name):
+# Argument checks sit on the path of calls that take 20 us on the GPU: each tensor is looked at once (type, place, layout,
+# size) and pointers travel as plain integers, which ctypes converts by the functions' argtypes.
+def _dev(t, dtype, name, n=0):
+    """Device pointer of a tensor of at least n elements (an undersized tensor would make a kernel leave its bounds)."""
     if t is None:
         return None
-    if not (t.is_cuda and t.dtype == dtype and t.is_contiguous()):
+    if not (t.is_cuda and t.dtype is dtype and t.is_contiguous()):
         raise MoeError(f"{name}: expected a contiguous CUDA tensor of {dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    if t.numel() < n:
+        raise MoeError(f"{name}: {t.numel()} elements, the call needs {n}")
+    return t.data_ptr()
 
 
-def _host(t, dtype, name):
+def _host(t, dtype, name, n=0):
     if t is None:
         return None
-    if t.is_cuda or t.dtype != dtype or not t.is_contiguous():
+    if t.is_cuda or t.dtype is not dtype or not t.is_contiguous():
         raise MoeError(f"{name}: expected a contiguous CPU tensor of {dtype}")
-    return ctypes.c_void_p(t.data_ptr())
+    if t.numel() < n:
+        raise MoeError(f"{name}: {t.numel()} elements, the call needs {n}")
+    return t.data_ptr()
 
 
 _CTX_SHAPE = {}   # context handle -> (T_max, d, E, k, n_shared, F, flags): what the size checks need
@@ -194,8 +202,17 @@ def _need(t, n, name):
         raise MoeError(f"{name}: {t.numel()} elements, the call needs {n}")
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+try:   # torch.cuda.current_stream() builds a Stream object (3.4 us); the calls only need the handle
+    _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+    def _stream():
+        return _raw_stream(_current_device())
+except AttributeError:
+    def _stream():
+        return torch.cuda.current_stream().cuda_stream
+
+
+_BF, _I32, _F32 = torch.bfloat16, torch.int32, torch.float32
 
 
 def _shape(T_max, d, E, k, n_shared, F, flags):
@@ -229,93 +246,71 @@ def moe_destroy(ctx):
 
 def moe_route(ctx, logits, T, topk_ids, topk_w, counts=None):
     _, _, E, k, _, _, _ = _shape_of(ctx)
-    _need(logits, T * E, "logits"); _need(topk_ids, T * k, "topk_ids"); _need(topk_w, T * k, "topk_w")
-    _need(counts, E, "counts")
-    _check(load_library().moe_route(ctx, _dev(logits, torch.float32, "logits"), T,
-                                    _dev(topk_ids, torch.int32, "topk_ids"), _dev(topk_w, torch.float32, "topk_w"),
-                                    _dev(counts, torch.int32, "counts"), _stream()), "moe_route")
+    _check(load_library().moe_route(ctx, _dev(logits, _F32, "logits", T * E), T, _dev(topk_ids, _I32, "topk_ids", T * k),
+                                    _dev(topk_w, _F32, "topk_w", T * k), _dev(counts, _I32, "counts", E), _stream()),
+           "moe_route")
 
 
 def moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits=None, counts=None):
     _, d, E, k, _, _, _ = _shape_of(ctx)
-    _need(x, T * d, "x"); _need(W_r, E * d, "W_r"); _need(topk_ids, T * k, "topk_ids"); _need(topk_w, T * k, "topk_w")
-    _need(logits, T * E, "logits"); _need(counts, E, "counts")
-    _check(load_library().moe_router_fwd(ctx, _dev(x, torch.bfloat16, "x"), _dev(W_r, torch.bfloat16, "W_r"), T,
-                                         _dev(topk_ids, torch.int32, "topk_ids"), _dev(topk_w, torch.float32, "topk_w"),
-                                         _dev(logits, torch.float32, "logits"), _dev(counts, torch.int32, "counts"),
-                                         _stream()), "moe_router_fwd")
+    _check(load_library().moe_router_fwd(ctx, _dev(x, _BF, "x", T * d), _dev(W_r, _BF, "W_r", E * d), T,
+                                         _dev(topk_ids, _I32, "topk_ids", T * k), _dev(topk_w, _F32, "topk_w", T * k),
+                                         _dev(logits, _F32, "logits", T * E), _dev(counts, _I32, "counts", E), _stream()),
+           "moe_router_fwd")
 
 
 def moe_router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits):
     _, _, E, k, _, _, _ = _shape_of(ctx)
-    _need(logits, T * E, "logits"); _need(topk_ids, T * k, "topk_ids"); _need(d_topk_w, T * k, "d_topk_w")
-    _need(d_logits, T * E, "d_logits")
-    _check(load_library().moe_router_bwd(ctx, _dev(logits, torch.float32, "logits"), _dev(topk_ids, torch.int32, "topk_ids"),
-                                         _dev(d_topk_w, torch.float32, "d_topk_w"), T,
-                                         _dev(d_logits, torch.float32, "d_logits"), _stream()), "moe_router_bwd")
+    _check(load_library().moe_router_bwd(ctx, _dev(logits, _F32, "logits", T * E), _dev(topk_ids, _I32, "topk_ids", T * k),
+                                         _dev(d_topk_w, _F32, "d_topk_w", T * k), T, _dev(d_logits, _F32, "d_logits", T * E),
+                                         _stream()), "moe_router_bwd")
 
 
 def moe_layout(ctx, topk_ids, T, counts=None, offsets=None, row_of=None, src_of=None):
     _, _, E, k, S, _, _ = _shape_of(ctx)
-    _need(topk_ids, T * k, "topk_ids"); _need(counts, E + S, "counts"); _need(offsets, E + S + 1, "offsets")
-    _need(row_of, T * (k + S), "row_of"); _need(src_of, T * (k + S), "src_of")
-    _check(load_library().moe_layout(ctx, _dev(topk_ids, torch.int32, "topk_ids"), T,
-                                     _dev(counts, torch.int32, "counts"), _dev(offsets, torch.int32, "offsets"),
-                                     _dev(row_of, torch.int32, "row_of"), _dev(src_of, torch.int32, "src_of"),
-                                     _stream()), "moe_layout")
-
-
-def _need_layer_tensors(ctx, T, acts, ids_w, W_gate_up, W_down):
-    _, d, E, k, S, F, _ = _shape_of(ctx)
-    for name, t in acts.items():
-        _need(t, T * d, name)
-    for name, t in ids_w.items():
-        _need(t, T * k, name)
-    _need(W_gate_up, (E + S) * 2 * F * d, "W_gate_up")
-    _need(W_down, (E + S) * d * F, "W_down")
+    n = T * (k + S)
+    _check(load_library().moe_layout(ctx, _dev(topk_ids, _I32, "topk_ids", T * k), T, _dev(counts, _I32, "counts", E + S),
+                                     _dev(offsets, _I32, "offsets", E + S + 1), _dev(row_of, _I32, "row_of", n),
+                                     _dev(src_of, _I32, "src_of", n), _stream()), "moe_layout")
 
 
 def moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T):
-    bf = torch.bfloat16
-    _need_layer_tensors(ctx, T, {"x": x, "out": out}, {"topk_ids": topk_ids, "topk_w": topk_w}, W_gate_up, W_down)
-    _check(load_library().moe_ffn_fwd(ctx, _dev(x, bf, "x"), _dev(topk_ids, torch.int32, "topk_ids"),
-                                      _dev(topk_w, torch.float32, "topk_w"), _dev(W_gate_up, bf, "W_gate_up"),
-                                      _dev(W_down, bf, "W_down"), _dev(out, bf, "out"), T, _stream()), "moe_ffn_fwd")
+    _, d, E, k, S, F, _ = _shape_of(ctx)
+    td, tk, nw = T * d, T * k, (E + S) * d * F
+    _check(load_library().moe_ffn_fwd(ctx, _dev(x, _BF, "x", td), _dev(topk_ids, _I32, "topk_ids", tk),
+                                      _dev(topk_w, _F32, "topk_w", tk), _dev(W_gate_up, _BF, "W_gate_up", 2 * nw),
+                                      _dev(W_down, _BF, "W_down", nw), _dev(out, _BF, "out", td), T, _stream()), "moe_ffn_fwd")
 
 
 def moe_ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T):
-    bf = torch.bfloat16
-    _need_layer_tensors(ctx, T, {"dout": dout, "x": x, "dx": dx},
-                        {"topk_ids": topk_ids, "topk_w": topk_w, "d_topk_w": d_topk_w}, W_gate_up, W_down)
-    _need(dW_gate_up, W_gate_up.numel(), "dW_gate_up"); _need(dW_down, W_down.numel(), "dW_down")
-    _check(load_library().moe_ffn_bwd(ctx, _dev(dout, bf, "dout"), _dev(x, bf, "x"),
-                                      _dev(topk_ids, torch.int32, "topk_ids"), _dev(topk_w, torch.float32, "topk_w"),
-                                      _dev(W_gate_up, bf, "W_gate_up"), _dev(W_down, bf, "W_down"),
-                                      _dev(dx, bf, "dx"), _dev(dW_gate_up, bf, "dW_gate_up"),
-                                      _dev(dW_down, bf, "dW_down"), _dev(d_topk_w, torch.float32, "d_topk_w"),
+    _, d, E, k, S, F, _ = _shape_of(ctx)
+    td, tk, nw = T * d, T * k, (E + S) * d * F
+    _check(load_library().moe_ffn_bwd(ctx, _dev(dout, _BF, "dout", td), _dev(x, _BF, "x", td),
+                                      _dev(topk_ids, _I32, "topk_ids", tk), _dev(topk_w, _F32, "topk_w", tk),
+                                      _dev(W_gate_up, _BF, "W_gate_up", 2 * nw), _dev(W_down, _BF, "W_down", nw),
+                                      _dev(dx, _BF, "dx", td), _dev(dW_gate_up, _BF, "dW_gate_up", 2 * nw),
+                                      _dev(dW_down, _BF, "dW_down", nw), _dev(d_topk_w, _F32, "d_topk_w", tk),
                                       T, _stream()), "moe_ffn_bwd")
 
 
 def moe_ffn_fwd_host(ctx, x_host, topk_ids_host, topk_w_host, W_gate_up, W_down, out_host, T):
-    bf = torch.bfloat16
-    _need_layer_tensors(ctx, T, {"x_host": x_host, "out_host": out_host},
-                        {"topk_ids_host": topk_ids_host, "topk_w_host": topk_w_host}, W_gate_up, W_down)
-    _check(load_library().moe_ffn_fwd_host(ctx, _host(x_host, bf, "x_host"),
-                                           _host(topk_ids_host, torch.int32, "topk_ids_host"),
-                                           _host(topk_w_host, torch.float32, "topk_w_host"),
-                                           _dev(W_gate_up, bf, "W_gate_up"), _dev(W_down, bf, "W_down"),
-                                           _host(out_host, bf, "out_host"), T, _stream()), "moe_ffn_fwd_host")
+    _, d, E, k, S, F, _ = _shape_of(ctx)
+    td, tk, nw = T * d, T * k, (E + S) * d * F
+    _check(load_library().moe_ffn_fwd_host(ctx, _host(x_host, _BF, "x_host", td),
+                                           _host(topk_ids_host, _I32, "topk_ids_host", tk),
+                                           _host(topk_w_host, _F32, "topk_w_host", tk),
+                                           _dev(W_gate_up, _BF, "W_gate_up", 2 * nw), _dev(W_down, _BF, "W_down", nw),
+                                           _host(out_host, _BF, "out_host", td), T, _stream()), "moe_ffn_fwd_host")
 
 
 def moe_ffn_bwd_host(ctx, dout_host, W_gate_up, W_down, dx_host, dW_gate_up, dW_down, d_topk_w_host, T):
-    bf = torch.bfloat16
-    _need_layer_tensors(ctx, T, {"dout_host": dout_host, "dx_host": dx_host}, {"d_topk_w_host": d_topk_w_host},
-                        W_gate_up, W_down)
-    _need(dW_gate_up, W_gate_up.numel(), "dW_gate_up"); _need(dW_down, W_down.numel(), "dW_down")
-    _check(load_library().moe_ffn_bwd_host(ctx, _host(dout_host, bf, "dout_host"), _dev(W_gate_up, bf, "W_gate_up"),
-                                           _dev(W_down, bf, "W_down"), _host(dx_host, bf, "dx_host"),
-                                           _dev(dW_gate_up, bf, "dW_gate_up"), _dev(dW_down, bf, "dW_down"),
-                                           _host(d_topk_w_host, torch.float32, "d_topk_w_host"), T, _stream()),
+    _, d, E, k, S, F, _ = _shape_of(ctx)
+    td, tk, nw = T * d, T * k, (E + S) * d * F
+    _check(load_library().moe_ffn_bwd_host(ctx, _host(dout_host, _BF, "dout_host", td),
+                                           _dev(W_gate_up, _BF, "W_gate_up", 2 * nw), _dev(W_down, _BF, "W_down", nw),
+                                           _host(dx_host, _BF, "dx_host", td), _dev(dW_gate_up, _BF, "dW_gate_up", 2 * nw),
+                                           _dev(dW_down, _BF, "dW_down", nw),
+                                           _host(d_topk_w_host, _F32, "d_topk_w_host", tk), T, _stream()),
            "moe_ffn_bwd_host")
 
 
@@ -346,27 +341,22 @@ def moe_get_phase_ms(ctx) -> dict:
 
 def moe_route_host(ctx, logits_host, T, topk_ids_host, topk_w_host):
     _, _, E, k, _, _, _ = _shape_of(ctx)
-    _need(logits_host, T * E, "logits_host"); _need(topk_ids_host, T * k, "topk_ids_host")
-    _need(topk_w_host, T * k, "topk_w_host")
-    _check(load_library().moe_route_host(ctx, _host(logits_host, torch.float32, "logits_host"), T,
-                                         _host(topk_ids_host, torch.int32, "topk_ids_host"),
-                                         _host(topk_w_host, torch.float32, "topk_w_host"), _stream()),
-           "moe_route_host")
+    _check(load_library().moe_route_host(ctx, _host(logits_host, _F32, "logits_host", T * E), T,
+                                         _host(topk_ids_host, _I32, "topk_ids_host", T * k),
+                                         _host(topk_w_host, _F32, "topk_w_host", T * k), _stream()), "moe_route_host")
 
 
 def moe_layout_noalloc(topk_ids, T, E, k, n_shared, counts, offsets, row_of, src_of, status2=None):
     """Dispatch layout through the entry point that allocates nothing and needs no context (for
     callers that may not cudaMalloc).  All tensors are caller-owned CUDA int32 tensors."""
-    i32 = torch.int32
     n, Ep = T * (k + n_shared), E + n_shared
     # a problem beyond the entry point's fixed limits is refused by the library itself before it touches memory
-    if 0 <= n <= 262144 and Ep <= 1088 and -(-n // 2048) * Ep <= 131072:
-        _need(topk_ids, T * k, "topk_ids"); _need(counts, Ep, "counts"); _need(offsets, Ep + 1, "offsets")
-        _need(row_of, n, "row_of"); _need(src_of, n, "src_of"); _need(status2, 2, "status2")
-    _check(load_library().moe_layout_noalloc(_dev(topk_ids, i32, "topk_ids"), T, E, k, n_shared,
-                                             _dev(counts, i32, "counts"), _dev(offsets, i32, "offsets"),
-                                             _dev(row_of, i32, "row_of"), _dev(src_of, i32, "src_of"),
-                                             _dev(status2, i32, "status2"), _stream()), "moe_layout_noalloc")
+    fits = 0 <= n <= 262144 and Ep <= 1088 and -(-n // 2048) * Ep <= 131072
+    need = (T * k, Ep, Ep + 1, n, n, 2) if fits else (0,) * 6
+    _check(load_library().moe_layout_noalloc(_dev(topk_ids, _I32, "topk_ids", need[0]), T, E, k, n_shared,
+                                             _dev(counts, _I32, "counts", need[1]), _dev(offsets, _I32, "offsets", need[2]),
+                                             _dev(row_of, _I32, "row_of", need[3]), _dev(src_of, _I32, "src_of", need[4]),
+                                             _dev(status2, _I32, "status2", need[5]), _stream()), "moe_layout_noalloc")
 
 
 MOE_STUDY_SERIAL, MOE_STUDY_STATIC, MOE_STUDY_DYNAMIC = 0, 1, 2
@@ -379,13 +369,11 @@ def moe_sched_study_workspace_bytes(M, tile_rows) -> int:
 def moe_sched_study(mode, x, r, s, z, M, C, tile_rows, workspace):
     """SwiGLU + Add operator pair under one of the three schedules; all tensors are CUDA tensors
     (bf16 x[M][2C], r/s/z[M][C]; workspace: any dtype, at least moe_sched_study_workspace_bytes)."""
-    bf = torch.bfloat16
-    _need(x, M * 2 * C, "x"); _need(r, M * C, "r"); _need(s, M * C, "s"); _need(z, M * C, "z")
     if workspace is None or not workspace.is_cuda or not workspace.is_contiguous():
         raise MoeError("workspace: expected a contiguous CUDA tensor")
     nbytes = workspace.numel() * workspace.element_size()
-    _check(load_library().moe_sched_study(int(mode), _dev(x, bf, "x"), _dev(r, bf, "r"), _dev(s, bf, "s"),
-                                          _dev(z, bf, "z"), int(M), int(C), int(tile_rows),
+    _check(load_library().moe_sched_study(int(mode), _dev(x, _BF, "x", M * 2 * C), _dev(r, _BF, "r", M * C),
+                                          _dev(s, _BF, "s", M * C), _dev(z, _BF, "z", M * C), int(M), int(C), int(tile_rows),
                                           ctypes.c_void_p(workspace.data_ptr()), nbytes, _stream()), "moe_sched_study")
 
 
@@ -477,44 +465,47 @@ def moe_ep_plan(counts, rank):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return 0 if t is None else t.data_ptr()
 
 
 def moe_ep_peer(recv, recv_meta, recv_counters, ret, ret_counters):
     """What one rank exposes: CUDA tensors (bf16 recv/ret, int32 meta/counters) living on, or peer-mapped into, the
     calling device."""
-    return MoeEpPeer(_ptr(recv).value if recv is not None else None, _ptr(recv_meta).value if recv_meta is not None else None,
-                     _ptr(recv_counters).value, _ptr(ret).value if ret is not None else None, _ptr(ret_counters).value)
+    return MoeEpPeer(_ptr(recv), _ptr(recv_meta), _ptr(recv_counters), _ptr(ret), _ptr(ret_counters))
+
+
+# one rank's part of a call as the bytes of its struct (filling a ctypes array field by field costs several times as much)
+_EP_LOCAL, _EP_LOCAL_COMBINE = struct.Struct("=4i6Q"), struct.Struct("=4i3Q")
+assert _EP_LOCAL.size == ctypes.sizeof(MoeEpLocal) and _EP_LOCAL_COMBINE.size == ctypes.sizeof(MoeEpLocalCombine)
 
 
 def moe_ep_dispatch(peers, locals_, k, d, status):
     """peers: [MoeEpPeer] for every rank; locals_: [dict(rank, T, x, topk_w, src_of, tasks (CUDA int32 [n,5]), recv_rows,
     consumed|None, ticket)] for the ranks this call acts for; status: CUDA int32[4]."""
     R = len(peers)
-    ps = (MoeEpPeer * R)(*peers)
-    ls = (MoeEpLocal * len(locals_))()
-    for i, l in enumerate(locals_):
-        _need(l["x"], l["T"] * d, "x"); _need(l["topk_w"], l["T"] * k, "topk_w"); _need(l["src_of"], l["T"] * k, "src_of")
-        _need(l.get("consumed"), l["recv_rows"] * d, "consumed"); _need(l["ticket"], 2, "ticket")
-        n_tasks = 0 if l["tasks"] is None else l["tasks"].shape[0]
-        ls[i] = MoeEpLocal(l["rank"], l["T"], n_tasks, l["recv_rows"], _ptr(l["x"]), _ptr(l["topk_w"]), _ptr(l["src_of"]),
-                           _ptr(l["tasks"]), _ptr(l.get("consumed")), _ptr(l["ticket"]))
-    _need(status, 4, "status")
-    _check(load_library().moe_ep_dispatch(ps, ls, len(locals_), R, k, d, _dev(status, torch.int32, "status"), _stream()),
-           "moe_ep_dispatch")
+    parts = []
+    for l in locals_:
+        T, rows, tasks, consumed = l["T"], l["recv_rows"], l["tasks"], l.get("consumed")
+        _need(l["x"], T * d, "x"); _need(l["topk_w"], T * k, "topk_w"); _need(l["src_of"], T * k, "src_of")
+        _need(consumed, rows * d, "consumed"); _need(l["ticket"], 2, "ticket")
+        parts.append(_EP_LOCAL.pack(l["rank"], T, 0 if tasks is None else tasks.shape[0], rows, _ptr(l["x"]), _ptr(l["topk_w"]),
+                                    _ptr(l["src_of"]), _ptr(tasks), _ptr(consumed), _ptr(l["ticket"])))
+    ls = (MoeEpLocal * len(parts)).from_buffer_copy(b"".join(parts))
+    _check(load_library().moe_ep_dispatch((MoeEpPeer * R)(*peers), ls, len(parts), R, k, d, _dev(status, _I32, "status", 4),
+                                          _stream()), "moe_ep_dispatch")
 
 
 def moe_ep_combine(peers, locals_, k, d, status):
     """locals_: [dict(rank, T, recv_rows, y, out, ticket)]."""
     R = len(peers)
-    ps = (MoeEpPeer * R)(*peers)
-    ls = (MoeEpLocalCombine * len(locals_))()
-    for i, l in enumerate(locals_):
-        _need(l["y"], l["recv_rows"] * d, "y"); _need(l["out"], l["T"] * d, "out"); _need(l["ticket"], 2, "ticket")
-        ls[i] = MoeEpLocalCombine(l["rank"], l["T"], l["recv_rows"], 0, _ptr(l["y"]), _ptr(l["out"]), _ptr(l["ticket"]))
-    _need(status, 4, "status")
-    _check(load_library().moe_ep_combine(ps, ls, len(locals_), R, k, d, _dev(status, torch.int32, "status"), _stream()),
-           "moe_ep_combine")
+    parts = []
+    for l in locals_:
+        T, rows = l["T"], l["recv_rows"]
+        _need(l["y"], rows * d, "y"); _need(l["out"], T * d, "out"); _need(l["ticket"], 2, "ticket")
+        parts.append(_EP_LOCAL_COMBINE.pack(l["rank"], T, rows, 0, _ptr(l["y"]), _ptr(l["out"]), _ptr(l["ticket"])))
+    ls = (MoeEpLocalCombine * len(parts)).from_buffer_copy(b"".join(parts))
+    _check(load_library().moe_ep_combine((MoeEpPeer * R)(*peers), ls, len(parts), R, k, d, _dev(status, _I32, "status", 4),
+                                         _stream()), "moe_ep_combine")
 
 
 def moe_debug_simulate_schedule(counts, T, k, n_shared, d, F, is_bwd, pairs, vec_workers):
@@ -599,9 +590,10 @@ class MoeLayer:
 
     def route(self, logits, with_counts=False):
         T = logits.shape[0]
-        ids = torch.empty(T, self.k, dtype=torch.int32, device="cuda")
-        w = torch.empty(T, self.k, dtype=torch.float32, device="cuda")
-        counts = torch.empty(self.E, dtype=torch.int32, device="cuda") if with_counts else None
+        dev = logits.device
+        ids = torch.empty(T, self.k, dtype=_I32, device=dev)
+        w = torch.empty(T, self.k, dtype=_F32, device=dev)
+        counts = torch.empty(self.E, dtype=_I32, device=dev) if with_counts else None
         moe_route(self.ctx, logits, T, ids, w, counts)
         return (ids, w, counts) if with_counts else (ids, w)
 
@@ -617,7 +609,7 @@ class MoeLayer:
     def ffn_fwd(self, x, topk_ids, topk_w, W_gate_up, W_down, out=None):
         T = x.shape[0]
         if out is None:
-            out = torch.empty(T, self.d, dtype=torch.bfloat16, device="cuda")
+            out = torch.empty(T, self.d, dtype=_BF, device=x.device)
         moe_ffn_fwd(self.ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T)
         return out
 
@@ -628,7 +620,7 @@ class MoeLayer:
         dW_gate_up = torch.empty_like(W_gate_up) if dW_gate_up is None else dW_gate_up
         dW_down = torch.empty_like(W_down) if dW_down is None else dW_down
         if d_topk_w is None and want_d_topk_w:
-            d_topk_w = torch.empty(T, self.k, dtype=torch.float32, device="cuda")
+            d_topk_w = torch.empty(T, self.k, dtype=_F32, device=x.device)
         moe_ffn_bwd(self.ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T)
         return dx, dW_gate_up, dW_down, d_topk_w
 
