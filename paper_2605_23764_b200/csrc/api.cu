@@ -867,15 +867,14 @@ int moe_router_fwd(moe_ctx* c, const uint16_t* x, const uint16_t* W_r, int32_t T
   RouterArgs a;
   memset(&a, 0, sizeof a);
   a.T = T; a.E = s.E; a.k = s.k; a.d = s.d;
-  a.N = ((s.E + 15) / 16) * 16;
-  if (a.N < 32) a.N = 32;
   a.renorm = gate_mode(c);
   a.topk_ids = topk_ids; a.topk_w = topk_w; a.logits = logits; a.counts = counts;
   a.status = c->status();
   a.budget_ns = c->budget_ns;
-  int rc = encode_2d(&a.tmX, x, (uint64_t)T, (uint64_t)s.d, 128, 64);   // 128 token rows x one 64-wide k-block
+  MOE_CUDA(plan_router_fwd(a, c->num_sms));
+  int rc = encode_2d(&a.tmX, x, (uint64_t)T, (uint64_t)s.d, (uint32_t)a.ntok, 64);   // a tile's tokens x one 64-wide k-block
   if (rc) return rc;
-  if ((rc = encode_2d(&a.tmW, W_r, (uint64_t)s.E, (uint64_t)s.d, (uint32_t)(a.N / 2), 64))) return rc;
+  if ((rc = encode_2d(&a.tmW, W_r, (uint64_t)s.E, (uint64_t)s.d, 128, 64))) return rc;
   Phase ph(c, MOE_PHASE_ROUTE, c->last_stream);
   MOE_CUDA(launch_router_fwd(a, c->num_sms, c->last_stream, &c->launches));
   return MOE_OK;

@@ -161,10 +161,12 @@ struct FusedArgs {
 
 // Router in the path (router.cu)
 struct RouterArgs {
-  CUtensorMap tmX;          // x [T][d] bf16, box 128 rows x 64 columns
-  CUtensorMap tmW;          // W_r [E][d] bf16, box N/2 rows x 64 columns (rows beyond E read as zeros)
+  CUtensorMap tmX;          // x [T][d] bf16, box `ntok` rows x 64 columns
+  CUtensorMap tmW;          // W_r [E][d] bf16, box 128 rows x 64 columns (rows beyond E read as zeros)
   int T, E, k, d;
-  int N;                    // accumulator columns: E rounded up to a multiple of 16, at least 32, at most 256
+  int ntok;                 // tokens per tile, a multiple of 16 up to 256
+  int csize;                // CTAs of a cluster: each takes 1/csize of the reduction
+  int stages, smem_bytes;
   int renorm;               // gate mode bits (GATE_RENORM | GATE_SIGMOID)
   int* topk_ids;
   float* topk_w;
@@ -173,6 +175,8 @@ struct RouterArgs {
   DevStatus* status;
   uint64_t budget_ns;
 };
+// fills ntok, csize, stages and smem_bytes from T, E, d
+cudaError_t plan_router_fwd(RouterArgs& a, int num_sms);
 cudaError_t launch_router_fwd(const RouterArgs& a, int num_sms, cudaStream_t s, int* launches);
 cudaError_t launch_router_bwd(const float* logits, const int* ids, const float* g, int T, int E, int k, int gate_mode,
                               float* dlogits, cudaStream_t s, int* launches);

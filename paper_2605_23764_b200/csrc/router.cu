@@ -2,213 +2,297 @@
 // top k): logits = x W_r^T on the tensor cores with the softmax top-k of route_layout.cu's router fused into the
 // epilogue, and the gradient of the k scores with respect to the logits.
 //
-// Forward: CTA pairs (tcgen05 cta_group::2) over tiles of 256 tokens.  A = 128 token rows of x per CTA, B = W_r
-// (all E experts, each CTA stages half of the rows), K = d in 64-wide blocks through a 6-stage TMA ring; the
-// accumulator of a CTA is [128 tokens][E] fp32 in TMEM, two of them so that the epilogue of one tile overlaps the
-// MMAs of the next.  Epilogue: TMEM lane = token, so one thread owns one token's E logits and reads them 16 columns
-// at a time, twice: once to select (insertion into a sorted list of k, raw logits compared, strict '>' while
-// scanning expert ids upward, so ties go to the lower id and slots come out in descending order), once to sum
-// exp(l - max) and, if asked, to store the logits.
+// Forward: the router weights are the A operand (128 experts per accumulator, two accumulators above 128 experts), a
+// tile of up to 256 tokens the B operand, and a cluster of 1, 2, 4 or 8 CTAs shares a tile by splitting the reduction
+// over d.  Each CTA streams its k-blocks through a TMA ring into TMEM; then the CTAs exchange partial sums through
+// distributed shared memory -- every CTA ends up with all experts' partials for its share of the tile's tokens, adds them in
+// CTA order, so the result does not depend on timing -- and its sixteen warps select, one token per warp
+// (warp_topk: raw logits compared, ties to the lower id, slots in descending order).
+//
+// What bounds it: few tokens, latency -- W_r is 3.7 MB at 256 x 7168 and one CTA pair needed 65 us to stream it; many tokens,
+// the reads of x, if all SMs have a share of them.  Tiles of 256 tokens without a split occupied 64 of 148 SMs on 8192
+// tokens, with the selection exposed behind them: 70 us.  See plan_router_fwd for the choice of tile and split.
 #include <limits.h>
 
 #include "gemm_pair.cuh"
 #include "launch_pairs.cuh"
 #include "moe_internal.h"
+#include "topk.cuh"
 
 namespace moe {
 
-constexpr int ROUTER_STAGES = 6;
-constexpr int ROUTER_THREADS = 192;   // warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
-constexpr int ROUTER_TILE_TOKENS = 256;
-constexpr int ROUTER_KMAX = 8;
-constexpr int ROUTER_ACC_COLS = 256;
+constexpr int ROUTER_WARPS = 16;      // warp 0 TMA producer, warp 1 MMA issuer and TMEM owner; all of them the epilogue
+constexpr int ROUTER_THREADS = 32 * ROUTER_WARPS;
+constexpr int ROUTER_MAX_STAGES = 8;
+constexpr int ROUTER_W_BYTES = 128 * BK * 2;   // 128 experts of one k-block
+constexpr int ROUTER_SMEM_MAX = 222 * 1024;    // operand ring, later the exchanged partial sums
+constexpr int ROUTER_MAX_CLUSTER = 8;
 
 struct RouterBarriers {
-  uint64_t full[ROUTER_STAGES], empty[ROUTER_STAGES];
-  uint64_t tmem_full[2], tmem_empty[2];
-  uint64_t drain;
+  uint64_t full[ROUTER_MAX_STAGES], empty[ROUTER_MAX_STAGES];
+  uint64_t acc_full;
   uint32_t tmem_base;
 };
-constexpr size_t ROUTER_SMEM_BYTES = 1024 + (size_t)ROUTER_STAGES * STAGE2_BYTES + sizeof(RouterBarriers) + 64;
 
-// One token's logits -> its k experts and scores.  `acc` = TMEM address of the thread's lane, column 0.
-__device__ __forceinline__ void router_epilogue_row(const RouterArgs& a, uint32_t acc, int token, bool valid) {
-  float val[ROUTER_KMAX];
-  int idx[ROUTER_KMAX];
+template <int NACC>
+__device__ __forceinline__ void router_select(const RouterArgs& a, const float* row, int token, int lane) {
+  constexpr int NPL = 4 * NACC;
+  float v[NPL];
+  uint32_t key[NPL];
+  float* lrow = a.logits ? a.logits + (size_t)token * a.E : nullptr;
 #pragma unroll
-  for (int j = 0; j < ROUTER_KMAX; ++j) { val[j] = -INFINITY; idx[j] = INT_MAX; }
-  // pass 1: selection (every thread of the warp takes part in the TMEM loads)
-  for (int c0 = 0; c0 < a.E; c0 += 16) {
-    float v[16];
-    tmem_ld16(acc + c0, v);
-    tmem_ld_wait();
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int e = c0 + i;
-      const float x = v[i];
-      if (e < a.E && x > val[ROUTER_KMAX - 1]) {
-#pragma unroll
-        for (int j = ROUTER_KMAX - 1; j > 0; --j) {
-          if (x > val[j - 1]) { val[j] = val[j - 1]; idx[j] = idx[j - 1]; }
-          else if (x > val[j]) { val[j] = x; idx[j] = e; }
-        }
-        if (x > val[0]) { val[0] = x; idx[0] = e; }
-      }
-    }
+  for (int i = 0; i < NPL; ++i) {
+    const int e = i * 32 + lane;
+    v[i] = row[e];
+    key[i] = e < a.E ? float_key(v[i]) : 0u;
+    if (lrow && e < a.E) lrow[e] = v[i];
   }
-  // pass 2: softmax denominator over all E (and the logits, if wanted)
-  const float mx = val[0];
-  float den = 0.f;
-  float* lrow = (a.logits && valid) ? a.logits + (size_t)token * a.E : nullptr;
-  for (int c0 = 0; c0 < a.E; c0 += 16) {
-    float v[16];
-    tmem_ld16(acc + c0, v);
-    tmem_ld_wait();
+  int my_id = 0;
+  float my_l = 0.f, my_p;
+  warp_topk<NPL>(key, a.k, lane, &my_id, &my_l);
+  if (a.renorm & GATE_SIGMOID) {
+    my_p = 1.0f / (1.0f + expf(-my_l));
+  } else {
+    const float mx = __shfl_sync(0xffffffffu, my_l, 0);
+    float den = 0.f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (c0 + i < a.E) den += expf(v[i] - mx);
-    if (lrow) {
-      if (c0 + 16 <= a.E && (a.E & 3) == 0) {
+    for (int i = 0; i < NPL; ++i)
+      if (i * 32 + lane < a.E) den += expf(v[i] - mx);
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          reinterpret_cast<float4*>(lrow + c0)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (c0 + i < a.E) lrow[c0 + i] = v[i];
-      }
-    }
+    for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+    my_p = expf(my_l - mx) / den;
   }
-  if (!valid) return;
-  float p[ROUTER_KMAX], wsum = 0.f;
-#pragma unroll
-  for (int j = 0; j < ROUTER_KMAX; ++j) {
-    p[j] = j >= a.k ? 0.f : (a.renorm & GATE_SIGMOID) ? 1.0f / (1.0f + expf(-val[j])) : expf(val[j] - mx) / den;
-    wsum += p[j];
+  if (a.renorm & GATE_RENORM) {
+    float wsum = 0.f;
+    for (int j = 0; j < a.k; ++j) wsum += __shfl_sync(0xffffffffu, my_p, j);
+    my_p /= wsum;
   }
-#pragma unroll
-  for (int j = 0; j < ROUTER_KMAX; ++j)
-    if (j < a.k) {
-      a.topk_ids[(size_t)token * a.k + j] = idx[j];
-      a.topk_w[(size_t)token * a.k + j] = (a.renorm & GATE_RENORM) ? p[j] / wsum : p[j];
-      if (a.counts) atomicAdd(&a.counts[idx[j]], 1);
-    }
+  if (lane < a.k) {
+    a.topk_ids[(size_t)token * a.k + lane] = my_id;
+    a.topk_w[(size_t)token * a.k + lane] = my_p;
+    if (a.counts) atomicAdd(&a.counts[my_id], 1);
+  }
 }
 
+template <int NACC>
 __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __grid_constant__ RouterArgs a) {
+  constexpr int EPAD = NACC * 128;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sA = smem;                                      // [ROUTER_STAGES][16 KB]: this CTA's 128 token rows
-  uint8_t* sB = smem + ROUTER_STAGES * A_STAGE_BYTES;      // [ROUTER_STAGES][16 KB]: this CTA's half of W_r's rows
-  RouterBarriers* bars = reinterpret_cast<RouterBarriers*>(smem + ROUTER_STAGES * STAGE2_BYTES);
+  __shared__ RouterBarriers bars;
+  float* part = reinterpret_cast<float*>(smem);   // after the k-loop: [csize - 1 sources][tokens of this CTA][EPAD]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rank = (int)cluster_ctarank();
-  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int C = a.csize, rank = (int)cluster_ctarank();
+  const int cluster = blockIdx.x / C, nclusters = gridDim.x / C;
   const WaitCtl wc{a.status, a.budget_ns};
-  const int ntiles = (a.T + ROUTER_TILE_TOKENS - 1) / ROUTER_TILE_TOKENS;
-  const int nkb = (a.d + BK - 1) / BK;
-  const uint32_t half_b_bytes = (uint32_t)(a.N / 2) * 128u;
+  const int ntok = a.ntok, npc = ntok / C;        // tokens of a tile; tokens this CTA finishes
+  const int ntiles = (a.T + ntok - 1) / ntok;
+  const int nkb_all = (a.d + BK - 1) / BK;
+  const int kb0 = (int)((long)nkb_all * rank / C), kb1 = (int)((long)nkb_all * (rank + 1) / C);
+  const int stage_bytes = NACC * ROUTER_W_BYTES + ntok * BK * 2;
+  int acc_cols = 32;
+  while (acc_cols < ntok) acc_cols <<= 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < ROUTER_STAGES; ++s) {
-      mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->empty[s], 1);
+    for (int s = 0; s < a.stages; ++s) {
+      mbar_init(&bars.full[s], 1);
+      mbar_init(&bars.empty[s], 1);
     }
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&bars->tmem_full[s], 1);
-      mbar_init(&bars->tmem_empty[s], 8);   // four epilogue warps in each CTA of the pair
-    }
-    mbar_init(&bars->drain, 1);
+    mbar_init(&bars.acc_full, 1);
     mbar_fence_init();
     fence_proxy_async();
     tma_prefetch_desc(&a.tmX);
     tma_prefetch_desc(&a.tmW);
   }
   if (warp == 1) {
-    tmem_alloc_pair(&bars->tmem_base, 2 * ROUTER_ACC_COLS);
-    tmem_relinquish_pair();
+    tmem_alloc_cta(&bars.tmem_base, NACC * acc_cols);
+    tmem_relinquish_cta();
   }
   tc_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();   // both CTAs' barriers exist before anyone signals across the pair
   tc_fence_after_sync();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = bars.tmem_base;
+  pdl_trigger();
+  pdl_wait();
 
-  if (warp == 0) {
-    // ------------------------------------------------ TMA producer (lane 0 of both CTAs)
-    if (lane == 0) {
-      uint32_t s = 0, ph = 1;
-      bool ok = true;
-      for (int t = pair; t < ntiles && ok; t += npairs) {
-        const int row0 = t * ROUTER_TILE_TOKENS + rank * BLOCK_M;
-        for (int kb = 0; kb < nkb; ++kb) {
-          if (!mbar_wait(&bars->empty[s], ph, wc, SITE_EMPTY, t, 50)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(&bars->full[s], 2 * (A_STAGE_BYTES + half_b_bytes));
-          tma_load_2d_pair(sA + s * A_STAGE_BYTES, &a.tmX, kb * BK, row0, &bars->full[s]);
-          tma_load_2d_pair(sB + s * HALF_B_BYTES, &a.tmW, kb * BK, rank * (a.N / 2), &bars->full[s]);
-          if (++s == ROUTER_STAGES) { s = 0; ph ^= 1; }
-        }
+  uint32_t s_ld = 0, ph_ld = 1, s_mma = 0, ph_mma = 0, n_tile = 0;
+  bool ok = true;   // a failed wait: this warp skips the work but still meets the barriers
+  for (int t = cluster; t < ntiles; t += nclusters, ++n_tile) {
+    const int t0 = t * ntok;
+    if (warp == 0 && lane == 0) {
+      for (int kb = kb0; kb < kb1 && ok; ++kb) {
+        if (!mbar_wait(&bars.empty[s_ld], ph_ld, wc, SITE_EMPTY, t, 20)) { ok = false; break; }
+        uint8_t* st = smem + s_ld * stage_bytes;
+        mbar_expect_tx(&bars.full[s_ld], stage_bytes);
+        tma_load_2d(st, &a.tmW, kb * BK, 0, &bars.full[s_ld]);
+        if (NACC == 2) tma_load_2d(st + ROUTER_W_BYTES, &a.tmW, kb * BK, 128, &bars.full[s_ld]);
+        tma_load_2d(st + NACC * ROUTER_W_BYTES, &a.tmX, kb * BK, t0, &bars.full[s_ld]);
+        if (++s_ld == (uint32_t)a.stages) { s_ld = 0; ph_ld ^= 1; }
       }
-    }
-  } else if (warp == 1) {
-    // ------------------------------------------------ MMA issuer (even CTA only)
-    if (lane == 0 && rank == 0) {
-      const uint32_t idesc = make_idesc_bf16(2 * BLOCK_M, a.N, 0, 0);
-      uint32_t it = 0, acc_it = 0;
-      bool ok = true;
-      for (int t = pair; t < ntiles && ok; t += npairs) {
-        const int as = acc_it & 1;
-        if (!mbar_wait(&bars->tmem_empty[as], ((acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) { ok = false; break; }
+    } else if (warp == 1 && lane == 0) {
+      const uint32_t idesc = make_idesc_bf16(BLOCK_M, ntok, 0, 0);
+      for (int kb = kb0; kb < kb1 && ok; ++kb) {
+        if (!mbar_wait(&bars.full[s_mma], ph_mma, wc, SITE_FULL, t)) { ok = false; break; }
         tc_fence_after_sync();
-        const uint32_t d_tmem = tmem_base + as * ROUTER_ACC_COLS;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % ROUTER_STAGES;
-          if (!mbar_wait(&bars->full[s], (it / ROUTER_STAGES) & 1, wc, SITE_FULL, t)) { ok = false; break; }
-          tc_fence_after_sync();
-          const uint32_t a_addr = smem_u32(sA + s * A_STAGE_BYTES), b_addr = smem_u32(sB + s * HALF_B_BYTES);
+        const uint32_t w_addr = smem_u32(smem + s_mma * stage_bytes), x_addr = w_addr + NACC * ROUTER_W_BYTES;
 #pragma unroll
-          for (int k16 = 0; k16 < BK / 16; ++k16)
-            tc_mma_bf16_pair(d_tmem, make_smem_desc(a_addr + k16 * 32, 16, 1024), make_smem_desc(b_addr + k16 * 32, 16, 1024),
-                             idesc, !(kb == 0 && k16 == 0));
-          tc_commit_pair(&bars->empty[s]);   // frees the stage in both CTAs
+        for (int k16 = 0; k16 < BK / 16; ++k16)
+#pragma unroll
+          for (int h = 0; h < NACC; ++h)
+            tc_mma_bf16_cta(tmem_base + h * acc_cols, make_smem_desc(w_addr + h * ROUTER_W_BYTES + k16 * 32, 16, 1024),
+                            make_smem_desc(x_addr + k16 * 32, 16, 1024), idesc, !(kb == kb0 && k16 == 0));
+        tc_commit_cta(&bars.empty[s_mma]);
+        if (++s_mma == (uint32_t)a.stages) { s_mma = 0; ph_mma ^= 1; }
+      }
+      tc_commit_cta(&bars.acc_full);   // also after a failed wait: what was issued has completed once this arrives
+    }
+    __syncwarp();
+    int up = 1;
+    if (lane == 0) up = mbar_wait(&bars.acc_full, n_tile & 1, wc, SITE_TMEM_FULL, t, 100) ? 1 : 0;
+    if (!__shfl_sync(0xffffffffu, up, 0)) ok = false;
+    tc_fence_after_sync();
+    cluster_sync_all();   // every CTA's MMAs are complete: the operand rings may be overwritten
+    // ---- warp w reads TMEM lanes 32 (w % 4) ..: 32 experts; chunks of 16 tokens are dealt to the four warps of a quad
+    const int quad = warp & 3, sub = warp >> 2;
+    const uint32_t trow = tmem_base + ((uint32_t)(quad * 32) << 16);
+    const int nchunks = ntok / 16;
+    const uint32_t part_addr = smem_u32(part);
+    for (int q = sub; q < nchunks * NACC && C > 1; q += 4) {
+      const int h = q / nchunks, c0 = (q - h * nchunks) * 16, e = h * 128 + quad * 32 + lane;
+      if (c0 >= rank * npc && c0 + 16 <= (rank + 1) * npc) continue;   // all of them this CTA's own
+      float v[16];
+      tmem_ld16(trow + h * acc_cols + c0, v);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int dst = (c0 + i) / npc;
+        if (dst == rank) continue;
+        const int slot = rank < dst ? rank : rank - 1;
+        st_cluster_f32(map_to_rank(part_addr + (((slot * npc) + (c0 + i - dst * npc)) * EPAD + e) * 4, dst), v[i]);
+      }
+    }
+    if (C > 1) cluster_sync_all();   // the partial sums of all CTAs have arrived
+    const int own0 = rank * npc, own1 = own0 + npc;
+    for (int q = sub; q < nchunks * NACC; q += 4) {
+      const int h = q / nchunks, c0 = (q - h * nchunks) * 16, e = h * 128 + quad * 32 + lane;
+      if (c0 >= own1 || c0 + 16 <= own0) continue;
+      float v[16];
+      tmem_ld16(trow + h * acc_cols + c0, v);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int j = c0 + i - own0;
+        if (j < 0 || j >= npc) continue;
+        float* p = part + j * EPAD + e;
+        float sum = 0.f;
+        for (int r = 0; r < C; ++r) {   // in CTA order
+          const float w = r == rank ? v[i] : p[(size_t)(r < rank ? r : r - 1) * npc * EPAD];
+          sum = r == 0 ? w : sum + w;
         }
-        if (!ok) break;
-        tc_commit_pair(&bars->tmem_full[as]);
-        ++acc_it;
-      }
-      if (!ok || *reinterpret_cast<volatile int*>(&a.status->abort)) {
-        tc_commit_pair(&bars->drain);
-        const WaitCtl shortwc{a.status, 20ull * 1000 * 1000};
-        mbar_wait(&bars->drain, 0, shortwc, SITE_DRAIN, 0);
+        *p = sum;
       }
     }
-  } else {
-    // ------------------------------------------------ epilogue warps (both CTAs): one thread per token
-    const int quad = warp & 3;
-    uint32_t acc_it = 0;
-    for (int t = pair; t < ntiles; t += npairs) {
-      const int as = acc_it & 1;
-      if (!mbar_wait(&bars->tmem_full[as], (acc_it >> 1) & 1, wc, SITE_TMEM_FULL, t, 200)) break;
-      tc_fence_after_sync();
-      const int token = t * ROUTER_TILE_TOKENS + rank * BLOCK_M + quad * 32 + lane;
-      router_epilogue_row(a, tmem_base + as * ROUTER_ACC_COLS + ((uint32_t)(quad * 32) << 16), token, token < a.T);
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_leader(&bars->tmem_empty[as]);
-      ++acc_it;
-    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (ok)
+      for (int j = warp; j < npc; j += ROUTER_WARPS) {
+        const int token = t0 + own0 + j;
+        if (token < a.T) router_select<NACC>(a, part + (size_t)j * EPAD, token, lane);
+      }
+    fence_proxy_async_smem();   // this tile's accesses to the ring's memory before the next tile's loads
+    if (t + nclusters < ntiles) cluster_sync_all();
   }
 
   // ---------------------------------------------------------------- teardown
-  if (*reinterpret_cast<volatile int*>(&a.status->abort)) __nanosleep(200000);
   tc_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();   // neither CTA leaves while its partner may still read its shared memory or signal it
+  cluster_sync_all();
   if (warp == 1) {
     tc_fence_after_sync();
-    tmem_dealloc_pair(tmem_base, 2 * ROUTER_ACC_COLS);
+    tmem_dealloc_cta(tmem_base, NACC * acc_cols);
   }
+}
+
+// Co-resident clusters of each size (SMs pair up inside a GPC, so fewer than SMs / size): a property of kernel and device.
+struct RouterDevice {
+  std::mutex mu;
+  bool ready[MAX_DEVICES] = {};
+  int clusters[MAX_DEVICES][2][4];   // [accumulators - 1][log2 of the cluster size]
+};
+static RouterDevice& router_device() { static RouterDevice r; return r; }
+
+static void router_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, int csize, int ctas, size_t smem, cudaStream_t s) {
+  memset(cfg, 0, sizeof *cfg);
+  cfg->gridDim = dim3(ctas);
+  cfg->blockDim = dim3(ROUTER_THREADS);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 2;
+}
+
+// Tile and split.  A CTA's time is the operand bytes it takes in: k-blocks x (expert rows + token rows of a tile), plus, per
+// tile, the exchange and selection (charged as ROUTER_TILE_COST rows).  With Q clusters of C CTAs co-resident, the tokens
+// are spread evenly over them in as few rounds as 256-token tiles allow.  8192 tokens x 256 experts, d = 7168: C = 4, tiles of
+// 240 tokens; 64 tokens: C = 8, tiles of 16.
+constexpr int ROUTER_TILE_COST = 1024;
+cudaError_t plan_router_fwd(RouterArgs& a, int num_sms) {
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
+  RouterDevice& rd = router_device();
+  {
+    std::lock_guard<std::mutex> lock(rd.mu);
+    if (!rd.ready[dev]) {
+      const int smem = ROUTER_SMEM_MAX + 1024;
+      if ((err = cudaFuncSetAttribute(router_fwd_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return err;
+      if ((err = cudaFuncSetAttribute(router_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return err;
+      for (int h = 0; h < 2; ++h)
+        for (int q = 0; q < 4; ++q) {
+          cudaLaunchConfig_t cfg;
+          cudaLaunchAttribute attr[2];
+          router_config(&cfg, attr, 1 << q, (num_sms >> q) << q, smem, nullptr);
+          cfg.numAttrs = 1;
+          int n = 0;
+          err = h ? cudaOccupancyMaxActiveClusters(&n, router_fwd_kernel<2>, &cfg) : cudaOccupancyMaxActiveClusters(&n, router_fwd_kernel<1>, &cfg);
+          if (err != cudaSuccess) return err;
+          rd.clusters[dev][h][q] = n > 0 ? n : 1;
+        }
+      rd.ready[dev] = true;
+    }
+  }
+  const int nacc = a.E > 128 ? 2 : 1, nkb = (a.d + BK - 1) / BK;
+  long best = -1;
+  for (int q = 0; q < 4; ++q) {
+    const int C = 1 << q, Q = rd.clusters[dev][nacc - 1][q];
+    if (C > nkb) break;   // every CTA needs a k-block
+    // tile: at most 256 tokens, and the partial sums a CTA receives (its own tokens' if it is alone) fit the ring's memory
+    int most = 256;
+    while ((long)(C > 1 ? C - 1 : 1) * (most / C) * nacc * 512 > ROUTER_SMEM_MAX) most -= 16;
+    const int rounds = (int)(((long)a.T + (long)Q * most - 1) / ((long)Q * most));
+    int ntok = (int)(((long)a.T + (long)Q * rounds - 1) / ((long)Q * rounds));
+    ntok = (ntok + 15) / 16 * 16;
+    const int tiles = (a.T + ntok - 1) / ntok;
+    const long cost = (long)((tiles + Q - 1) / Q) * ((long)((nkb + C - 1) / C) * (nacc * 128 + ntok) + ROUTER_TILE_COST);
+    if (best < 0 || cost < best) { best = cost; a.csize = C; a.ntok = ntok; }
+  }
+  const int stage = nacc * ROUTER_W_BYTES + a.ntok * BK * 2;
+  const int per_cta = (nkb + a.csize - 1) / a.csize;
+  a.stages = ROUTER_SMEM_MAX / stage;
+  if (a.stages > ROUTER_MAX_STAGES) a.stages = ROUTER_MAX_STAGES;
+  if (a.stages > per_cta) a.stages = per_cta;
+  int need = a.stages * stage;
+  const int sums = (a.csize > 1 ? a.csize - 1 : 1) * (a.ntok / a.csize) * nacc * 512;
+  if (sums > need) need = sums;
+  a.smem_bytes = need + 1024;
+  return cudaSuccess;
 }
 
 cudaError_t launch_router_fwd(const RouterArgs& a, int num_sms, cudaStream_t s, int* launches) {
@@ -218,8 +302,17 @@ cudaError_t launch_router_fwd(const RouterArgs& a, int num_sms, cudaStream_t s, 
     if (e != cudaSuccess) return e;
   }
   ++*launches;
-  static PairLaunchState st;
-  return launch_on_pairs(st, router_fwd_kernel, a, ROUTER_THREADS, ROUTER_SMEM_BYTES, num_sms, false, s);
+  const int tiles = (a.T + a.ntok - 1) / a.ntok;
+  int q = 0;
+  while ((1 << q) < a.csize) ++q;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const int Q = router_device().clusters[dev][a.E > 128 ? 1 : 0][q];
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  router_config(&cfg, attr, a.csize, (tiles < Q ? tiles : Q) * a.csize, a.smem_bytes, s);
+  return a.E > 128 ? cudaLaunchKernelEx(&cfg, router_fwd_kernel<2>, a) : cudaLaunchKernelEx(&cfg, router_fwd_kernel<1>, a);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -228,43 +321,56 @@ cudaError_t launch_router_fwd(const RouterArgs& a, int num_sms, cudaStream_t s, 
 //   renormalisation   : w = softmax over the selected experts; dl[e_j] = w_j (g_j - sum_i g_i w_i), 0 elsewhere
 // The selection passes no gradient.
 // ------------------------------------------------------------------------------------------
+// NPL logits per lane stay in registers (E <= 32 NPL): one read of the logits, one write of the gradient.
+template <int NPL>
 __global__ void __launch_bounds__(256) router_bwd_kernel(const float* __restrict__ logits, const int* __restrict__ ids,
                                                           const float* __restrict__ g, int T, int E, int k, int mode,
                                                           float* __restrict__ dlogits) {
   const int lane = threadIdx.x & 31;
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  pdl_wait();
+  pdl_trigger();
   if (t >= T) return;
   const float* l = logits + (size_t)t * E;
   float* dl = dlogits + (size_t)t * E;
-  float mx = -INFINITY;
-  for (int e = lane; e < E; e += 32) mx = fmaxf(mx, l[e]);
+  float v[NPL];
 #pragma unroll
-  for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  for (int i = 0; i < NPL; ++i) v[i] = i * 32 + lane < E ? l[i * 32 + lane] : -INFINITY;
   // the k selected experts, one per lane (k <= 32)
   const int my_id = lane < k ? ids[(size_t)t * k + lane] : -1;
   const bool have = my_id >= 0 && my_id < E;
   const float my_g = have ? g[(size_t)t * k + lane] : 0.f;
+  const float my_l = have ? l[my_id] : 0.f;
   const bool renorm = (mode & GATE_RENORM) != 0;
   if (mode & GATE_SIGMOID) {
     // per-expert scores s = sigmoid(l): only the selected experts get a gradient
-    const float s = have ? 1.0f / (1.0f + expf(-l[my_id])) : 0.f;
+    const float s = have ? 1.0f / (1.0f + expf(-my_l)) : 0.f;
     float Z = s;
 #pragma unroll
     for (int off = 16; off; off >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, off);
     float dot = renorm ? my_g * (s / Z) : 0.f;
 #pragma unroll
     for (int off = 16; off; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    for (int e = lane; e < E; e += 32) dl[e] = 0.f;
+#pragma unroll
+    for (int i = 0; i < NPL; ++i)
+      if (i * 32 + lane < E) dl[i * 32 + lane] = 0.f;
     __syncwarp();
     if (have) dl[my_id] = renorm ? s * (1.0f - s) / Z * (my_g - dot) : my_g * s * (1.0f - s);
     return;
   }
-  const float my_ex = have ? expf(l[my_id] - mx) : 0.f;
+  float mx = -INFINITY;
+#pragma unroll
+  for (int i = 0; i < NPL; ++i) mx = fmaxf(mx, v[i]);
+#pragma unroll
+  for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  const float my_ex = have ? expf(my_l - mx) : 0.f;
   float den = 0.f;
   if (renorm) {
     den = my_ex;
   } else {
-    for (int e = lane; e < E; e += 32) den += expf(l[e] - mx);
+#pragma unroll
+    for (int i = 0; i < NPL; ++i)
+      if (i * 32 + lane < E) { v[i] = expf(v[i] - mx); den += v[i]; }
   }
 #pragma unroll
   for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
@@ -273,7 +379,9 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(const float* __restrict
 #pragma unroll
   for (int off = 16; off; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
   // dense part
-  for (int e = lane; e < E; e += 32) dl[e] = renorm ? 0.f : -(expf(l[e] - mx) / den) * dot;
+#pragma unroll
+  for (int i = 0; i < NPL; ++i)
+    if (i * 32 + lane < E) dl[i * 32 + lane] = renorm ? 0.f : -(v[i] / den) * dot;
   __syncwarp();
   // the selected experts are distinct, so each lane corrects its own entry
   if (have) dl[my_id] = renorm ? my_w * (my_g - dot) : my_w * my_g - my_w * dot;
@@ -282,11 +390,19 @@ __global__ void __launch_bounds__(256) router_bwd_kernel(const float* __restrict
 cudaError_t launch_router_bwd(const float* logits, const int* ids, const float* g, int T, int E, int k, int gate_mode,
                               float* dlogits, cudaStream_t s, int* launches) {
   if (T == 0) return cudaSuccess;
-  const int threads = 256, tokens_per_block = threads / 32;
-  router_bwd_kernel<<<(T + tokens_per_block - 1) / tokens_per_block, threads, 0, s>>>(logits, ids, g, T, E, k,
-                                                                                      gate_mode, dlogits);
+  const dim3 threads(256), grid((T + 7) / 8);
+  const int npl = (E + 31) / 32;
+  cudaError_t e;
+#define MOE_ROUTER_BWD_CASE(N) e = launch_dependent(router_bwd_kernel<N>, grid, threads, 0, s, logits, ids, g, T, E, k, gate_mode, dlogits)
+  if (npl <= 1) MOE_ROUTER_BWD_CASE(1);
+  else if (npl <= 2) MOE_ROUTER_BWD_CASE(2);
+  else if (npl <= 4) MOE_ROUTER_BWD_CASE(4);
+  else if (npl <= 8) MOE_ROUTER_BWD_CASE(8);
+  else if (npl <= 16) MOE_ROUTER_BWD_CASE(16);
+  else MOE_ROUTER_BWD_CASE(32);
+#undef MOE_ROUTER_BWD_CASE
   ++*launches;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace moe
