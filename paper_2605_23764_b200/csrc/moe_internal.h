@@ -166,7 +166,7 @@ struct RouterArgs {
   int T, E, k, d;
   int ntok;                 // tokens per tile, a multiple of 16 up to 256
   int csize;                // CTAs of a cluster: each takes 1/csize of the reduction
-  int stages, smem_bytes;
+  int stages, smem_bytes, part_over_ring;
   int renorm;               // gate mode bits (GATE_RENORM | GATE_SIGMOID)
   int* topk_ids;
   float* topk_w;
@@ -175,7 +175,7 @@ struct RouterArgs {
   DevStatus* status;
   uint64_t budget_ns;
 };
-// fills ntok, csize, stages and smem_bytes from T, E, d
+// fills ntok, csize, stages, smem_bytes and part_over_ring from T, E, d
 cudaError_t plan_router_fwd(RouterArgs& a, int num_sms);
 cudaError_t launch_router_fwd(const RouterArgs& a, int num_sms, cudaStream_t s, int* launches);
 cudaError_t launch_router_bwd(const float* logits, const int* ids, const float* g, int T, int E, int k, int gate_mode,

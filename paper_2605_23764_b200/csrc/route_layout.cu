@@ -30,12 +30,14 @@ __global__ void __launch_bounds__(256) route_kernel(const float* __restrict__ lo
     int e = i * 32 + lane;
     v[i] = e < E ? row[e] : -INFINITY;
   }
-  uint32_t key[NPL];
+  uint32_t key[1][NPL];
 #pragma unroll
-  for (int i = 0; i < NPL; ++i) key[i] = i * 32 + lane < E ? float_key(v[i]) : 0u;
-  int my_id = 0;
-  float my_l = 0.f;
-  warp_topk<NPL>(key, k, lane, &my_id, &my_l);
+  for (int i = 0; i < NPL; ++i) key[0][i] = i * 32 + lane < E ? float_key(v[i]) : 0u;
+  int ids[1] = {0};
+  float ls[1] = {0.f};
+  warp_topk<NPL, 1>(key, k, lane, ids, ls);
+  const int my_id = ids[0];
+  const float my_l = ls[0];
   float my_p;
   if (renorm & GATE_SIGMOID) {
     my_p = 1.0f / (1.0f + expf(-my_l));

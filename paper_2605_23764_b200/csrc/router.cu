@@ -34,44 +34,78 @@ struct RouterBarriers {
   uint32_t tmem_base;
 };
 
+// Four tokens of one warp: `row` = their logits' partial sums [nslots][..][EPAD experts][4 tokens], added here.
 template <int NACC>
-__device__ __forceinline__ void router_select(const RouterArgs& a, const float* row, int token, int lane) {
+__device__ __forceinline__ void router_select(const RouterArgs& a, const float4* row, int nslots, size_t slot_stride, int token0,
+                                              int lane) {
   constexpr int NPL = 4 * NACC;
-  float v[NPL];
-  uint32_t key[NPL];
-  float* lrow = a.logits ? a.logits + (size_t)token * a.E : nullptr;
+  float v[4][NPL];
+  {
+    float4 acc[NPL];
 #pragma unroll
-  for (int i = 0; i < NPL; ++i) {
-    const int e = i * 32 + lane;
-    v[i] = row[e];
-    key[i] = e < a.E ? float_key(v[i]) : 0u;
-    if (lrow && e < a.E) lrow[e] = v[i];
+    for (int i = 0; i < NPL; ++i) acc[i] = row[i * 32 + lane];
+#pragma unroll 1
+    for (int r = 1; r < nslots; ++r) {
+      row += slot_stride;
+      float4 w[NPL];
+#pragma unroll
+      for (int i = 0; i < NPL; ++i) w[i] = row[i * 32 + lane];
+#pragma unroll
+      for (int i = 0; i < NPL; ++i) { acc[i].x += w[i].x; acc[i].y += w[i].y; acc[i].z += w[i].z; acc[i].w += w[i].w; }
+    }
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) { v[0][i] = acc[i].x; v[1][i] = acc[i].y; v[2][i] = acc[i].z; v[3][i] = acc[i].w; }
   }
-  int my_id = 0;
-  float my_l = 0.f, my_p;
-  warp_topk<NPL>(key, a.k, lane, &my_id, &my_l);
-  if (a.renorm & GATE_SIGMOID) {
-    my_p = 1.0f / (1.0f + expf(-my_l));
-  } else {
-    const float mx = __shfl_sync(0xffffffffu, my_l, 0);
-    float den = 0.f;
+  if (a.logits)
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int i = 0; i < NPL; ++i)
+        if (token0 + t < a.T && i * 32 + lane < a.E) a.logits[(size_t)(token0 + t) * a.E + i * 32 + lane] = v[t][i];
+  uint32_t key[4][NPL];
+  float mx[4], den[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) {
+      key[t][i] = i * 32 + lane < a.E ? float_key(v[t][i]) : 0u;
+      m = max(m, key[t][i]);
+    }
+    mx[t] = key_float(__reduce_max_sync(0xffffffffu, m));
+    den[t] = 0.f;
+  }
+  if (!(a.renorm & GATE_SIGMOID)) {
 #pragma unroll
     for (int i = 0; i < NPL; ++i)
-      if (i * 32 + lane < a.E) den += expf(v[i] - mx);
 #pragma unroll
-    for (int off = 16; off; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
-    my_p = expf(my_l - mx) / den;
+      for (int t = 0; t < 4; ++t)
+        if (i * 32 + lane < a.E) den[t] += expf(v[t][i] - mx[t]);
+#pragma unroll
+    for (int off = 16; off; off >>= 1)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) den[t] += __shfl_xor_sync(0xffffffffu, den[t], off);
   }
+  int id[4] = {0, 0, 0, 0};
+  float l[4] = {0.f, 0.f, 0.f, 0.f}, p[4], wsum[4] = {0.f, 0.f, 0.f, 0.f};
+  warp_topk<NPL, 4>(key, a.k, lane, id, l);
+#pragma unroll
+  for (int t = 0; t < 4; ++t) p[t] = (a.renorm & GATE_SIGMOID) ? 1.0f / (1.0f + expf(-l[t])) : expf(l[t] - mx[t]) / den[t];
   if (a.renorm & GATE_RENORM) {
-    float wsum = 0.f;
-    for (int j = 0; j < a.k; ++j) wsum += __shfl_sync(0xffffffffu, my_p, j);
-    my_p /= wsum;
+    for (int j = 0; j < a.k; ++j)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) wsum[t] += __shfl_sync(0xffffffffu, p[t], j);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) p[t] /= wsum[t];
   }
-  if (lane < a.k) {
-    a.topk_ids[(size_t)token * a.k + lane] = my_id;
-    a.topk_w[(size_t)token * a.k + lane] = my_p;
-    if (a.counts) atomicAdd(&a.counts[my_id], 1);
-  }
+  if (lane < a.k)
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (token0 + t < a.T) {
+        a.topk_ids[(size_t)(token0 + t) * a.k + lane] = id[t];
+        a.topk_w[(size_t)(token0 + t) * a.k + lane] = p[t];
+        if (a.counts) atomicAdd(&a.counts[id[t]], 1);
+      }
 }
 
 template <int NACC>
@@ -80,7 +114,9 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ RouterBarriers bars;
-  float* part = reinterpret_cast<float*>(smem);   // after the k-loop: [csize - 1 sources][tokens of this CTA][EPAD]
+  // partial sums of this CTA's tokens, four tokens side by side: [sources but itself (at least one)][token / 4][EPAD][4];
+  // behind the operand ring where both fit, in its place (after the k-loop) where they do not
+  float4* part = reinterpret_cast<float4*>(smem + (a.part_over_ring ? 0 : a.stages * (NACC * ROUTER_W_BYTES + a.ntok * BK * 2)));
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int C = a.csize, rank = (int)cluster_ctarank();
@@ -112,6 +148,7 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  if (C > 1) cluster_arrive();   // waited for before the first access to another CTA's shared memory
   const uint32_t tmem_base = bars.tmem_base;
   pdl_trigger();
   pdl_wait();
@@ -152,62 +189,66 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
     if (lane == 0) up = mbar_wait(&bars.acc_full, n_tile & 1, wc, SITE_TMEM_FULL, t, 100) ? 1 : 0;
     if (!__shfl_sync(0xffffffffu, up, 0)) ok = false;
     tc_fence_after_sync();
-    cluster_sync_all();   // every CTA's MMAs are complete: the operand rings may be overwritten
-    // ---- warp w reads TMEM lanes 32 (w % 4) ..: 32 experts; chunks of 16 tokens are dealt to the four warps of a quad
+    if (C > 1) {
+      if (n_tile == 0) cluster_wait();            // every CTA of the cluster runs
+      if (a.part_over_ring) cluster_sync_all();   // every CTA's MMAs are complete: the operand rings may be overwritten
+    } else if (a.part_over_ring) {
+      __syncthreads();
+    }
+    // ---- warp w reads TMEM lanes 32 (w % 4) ..: 32 experts; chunks of 16 tokens are dealt to the four warps of a quad.
+    // A lane writes four tokens of its expert at a time: 512 contiguous bytes per warp and store.
     const int quad = warp & 3, sub = warp >> 2;
     const uint32_t trow = tmem_base + ((uint32_t)(quad * 32) << 16);
-    const int nchunks = ntok / 16;
+    const int nchunks = ntok / 16, ngroups = npc / 4;
+    const size_t slot_stride = (size_t)ngroups * EPAD;
+    const int own0 = rank * npc, own1 = own0 + npc;
     const uint32_t part_addr = smem_u32(part);
     for (int q = sub; q < nchunks * NACC && C > 1; q += 4) {
       const int h = q / nchunks, c0 = (q - h * nchunks) * 16, e = h * 128 + quad * 32 + lane;
-      if (c0 >= rank * npc && c0 + 16 <= (rank + 1) * npc) continue;   // all of them this CTA's own
+      if (c0 >= own0 && c0 + 16 <= own1) continue;   // all of them this CTA's own
       float v[16];
       tmem_ld16(trow + h * acc_cols + c0, v);
       tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
+      for (int i = 0; i < 16; i += 4) {
         const int dst = (c0 + i) / npc;
         if (dst == rank) continue;
-        const int slot = rank < dst ? rank : rank - 1;
-        st_cluster_f32(map_to_rank(part_addr + (((slot * npc) + (c0 + i - dst * npc)) * EPAD + e) * 4, dst), v[i]);
+        const size_t slot = rank < dst ? rank : rank - 1;
+        const uint32_t at = (uint32_t)((slot * slot_stride + (size_t)((c0 + i - dst * npc) / 4) * EPAD + e) * 16);
+        st_cluster_v4(map_to_rank(part_addr + at, dst), make_uint4(__float_as_uint(v[i]), __float_as_uint(v[i + 1]),
+                                                                   __float_as_uint(v[i + 2]), __float_as_uint(v[i + 3])));
       }
     }
     if (C > 1) cluster_sync_all();   // the partial sums of all CTAs have arrived
-    const int own0 = rank * npc, own1 = own0 + npc;
-    for (int q = sub; q < nchunks * NACC; q += 4) {
+    for (int q = sub; q < nchunks * NACC; q += 4) {   // this CTA's own, added to the first source's
       const int h = q / nchunks, c0 = (q - h * nchunks) * 16, e = h * 128 + quad * 32 + lane;
       if (c0 >= own1 || c0 + 16 <= own0) continue;
       float v[16];
       tmem_ld16(trow + h * acc_cols + c0, v);
       tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
+      for (int i = 0; i < 16; i += 4) {
         const int j = c0 + i - own0;
         if (j < 0 || j >= npc) continue;
-        float* p = part + j * EPAD + e;
-        float sum = 0.f;
-        for (int r = 0; r < C; ++r) {   // in CTA order
-          const float w = r == rank ? v[i] : p[(size_t)(r < rank ? r : r - 1) * npc * EPAD];
-          sum = r == 0 ? w : sum + w;
-        }
-        *p = sum;
+        float4* p = part + (size_t)(j / 4) * EPAD + e;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (C > 1) s = *p;
+        *p = make_float4(s.x + v[i], s.y + v[i + 1], s.z + v[i + 2], s.w + v[i + 3]);
       }
     }
     tc_fence_before_sync();
     __syncthreads();
     if (ok)
-      for (int j = warp; j < npc; j += ROUTER_WARPS) {
-        const int token = t0 + own0 + j;
-        if (token < a.T) router_select<NACC>(a, part + (size_t)j * EPAD, token, lane);
-      }
+      for (int g = warp; g < ngroups; g += ROUTER_WARPS)
+        if (t0 + own0 + 4 * g < a.T)
+          router_select<NACC>(a, part + (size_t)g * EPAD, C > 1 ? C - 1 : 1, slot_stride, t0 + own0 + 4 * g, lane);
     fence_proxy_async_smem();   // this tile's accesses to the ring's memory before the next tile's loads
     if (t + nclusters < ntiles) cluster_sync_all();
   }
 
-  // ---------------------------------------------------------------- teardown
+  // ---------------------------------------------------------------- teardown (nobody touches another CTA's memory any more)
   tc_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc_cta(tmem_base, NACC * acc_cols);
@@ -275,10 +316,11 @@ cudaError_t plan_router_fwd(RouterArgs& a, int num_sms) {
     if (C > nkb) break;   // every CTA needs a k-block
     // tile: at most 256 tokens, and the partial sums a CTA receives (its own tokens' if it is alone) fit the ring's memory
     int most = 256;
-    while ((long)(C > 1 ? C - 1 : 1) * (most / C) * nacc * 512 > ROUTER_SMEM_MAX) most -= 16;
+    while ((long)(C > 1 ? C - 1 : 1) * (most / C) * nacc * 512 > ROUTER_SMEM_MAX) most -= 32;
     const int rounds = (int)(((long)a.T + (long)Q * most - 1) / ((long)Q * most));
     int ntok = (int)(((long)a.T + (long)Q * rounds - 1) / ((long)Q * rounds));
-    ntok = (ntok + 15) / 16 * 16;
+    const int grain = C == 8 ? 32 : 16;   // the MMA's granularity, and four tokens per CTA
+    ntok = (ntok + grain - 1) / grain * grain;
     const int tiles = (a.T + ntok - 1) / ntok;
     const long cost = (long)((tiles + Q - 1) / Q) * ((long)((nkb + C - 1) / C) * (nacc * 128 + ntok) + ROUTER_TILE_COST);
     if (best < 0 || cost < best) { best = cost; a.csize = C; a.ntok = ntok; }
@@ -288,10 +330,9 @@ cudaError_t plan_router_fwd(RouterArgs& a, int num_sms) {
   a.stages = ROUTER_SMEM_MAX / stage;
   if (a.stages > ROUTER_MAX_STAGES) a.stages = ROUTER_MAX_STAGES;
   if (a.stages > per_cta) a.stages = per_cta;
-  int need = a.stages * stage;
   const int sums = (a.csize > 1 ? a.csize - 1 : 1) * (a.ntok / a.csize) * nacc * 512;
-  if (sums > need) need = sums;
-  a.smem_bytes = need + 1024;
+  a.part_over_ring = a.stages * stage + sums > ROUTER_SMEM_MAX;
+  a.smem_bytes = 1024 + (a.part_over_ring ? (sums > a.stages * stage ? sums : a.stages * stage) : a.stages * stage + sums);
   return cudaSuccess;
 }
 

@@ -19,26 +19,46 @@ __device__ __forceinline__ float key_float(uint32_t key) {
   return __uint_as_float((key & 0x80000000u) ? (key & 0x7FFFFFFFu) : ~key);
 }
 
-// The k largest of the warp's keys: expert e = 32 i + lane in key[i] (0: no expert).  Lane j < k ends up with the j-th
-// expert's id and logit; equal logits go to the lower id.  One round is a local argmax and two warp reductions
-// (redux), against ten shuffles for a butterfly over {value, id}: the router over 16384 x 128 logits took 34 us with
-// the butterfly, its rounds being a serial chain.
-template <int NPL>
-__device__ __forceinline__ void warp_topk(uint32_t (&key)[NPL], int k, int lane, int* my_id, float* my_logit) {
+// The k largest of each of NT tokens' keys: expert e = 32 i + lane in key[t][i] (0: no expert).  Lane j < k ends up with the
+// j-th expert's id and logit of every token; equal logits go to the lower id.  One round is a local argmax -- a tree of
+// depth log2 NPL -- and two warp reductions (redux), against ten shuffles for a butterfly over {value, id}; the rounds
+// are a serial chain, so NT tokens side by side hide each other's latency.  16384 x 128 logits: 34 us with the
+// butterfly.
+template <int NPL, int NT>
+__device__ __forceinline__ void warp_topk(uint32_t (&key)[NT][NPL], int k, int lane, int (&my_id)[NT], float (&my_logit)[NT]) {
+#pragma unroll 1
   for (int j = 0; j < k; ++j) {
-    uint32_t bk = key[0];
-    int bi = 0;
+    uint32_t m[NT];
+    int id[NT];
 #pragma unroll
-    for (int i = 1; i < NPL; ++i)
-      if (key[i] > bk) { bk = key[i]; bi = i; }
-    const uint32_t m = __reduce_max_sync(0xffffffffu, bk);
-    const int id = __reduce_min_sync(0xffffffffu, bk == m ? bi * 32 + lane : INT_MAX);
-    if ((id & 31) == lane) {
+    for (int t = 0; t < NT; ++t) {
+      uint32_t b[NPL];
 #pragma unroll
-      for (int i = 0; i < NPL; ++i)
-        if (i == (id >> 5)) key[i] = 0;
+      for (int i = 0; i < NPL; ++i) b[i] = key[t][i];
+#pragma unroll
+      for (int w = 1; w < NPL; w <<= 1)
+#pragma unroll
+        for (int i = 0; i + w < NPL; i += 2 * w) b[i] = max(b[i], b[i + w]);
+      m[t] = b[0];
     }
-    if (lane == j) { *my_id = id; *my_logit = key_float(m); }
+#pragma unroll
+    for (int t = 0; t < NT; ++t) m[t] = __reduce_max_sync(0xffffffffu, m[t]);
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      int c = INT_MAX;
+#pragma unroll
+      for (int i = NPL - 1; i >= 0; --i) c = key[t][i] == m[t] ? i * 32 + lane : c;   // the lowest id of this lane
+      id[t] = c;
+    }
+#pragma unroll
+    for (int t = 0; t < NT; ++t) id[t] = __reduce_min_sync(0xffffffffu, id[t]);
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+#pragma unroll
+      for (int i = 0; i < NPL; ++i) key[t][i] = id[t] == i * 32 + lane ? 0u : key[t][i];
+      my_id[t] = lane == j ? id[t] : my_id[t];
+      my_logit[t] = lane == j ? key_float(m[t]) : my_logit[t];
+    }
   }
 }
 
