@@ -29,8 +29,7 @@
  *     their own contexts, may call concurrently.
  *   - Launch modes: by default a pass is ONE persistent launch (after the index-only layout
  *     kernels) in which gather, GEMM and combine tiles are ordered by event counters;
- *     MOE_FLAG_SERIAL_LAUNCH runs one launch per operator.  Shapes with F % 16 != 0 always take
- *     the one-launch-per-operator path.
+ *     MOE_FLAG_SERIAL_LAUNCH runs one launch per operator.
  *   - Test and diagnostic entry points (workspace views, schedule simulation, failure injection,
  *     trace read-out) are declared in moe_b200_debug.h.
  */

@@ -1,7 +1,6 @@
 // C ABI of libmoe_b200: context, workspace carving, tensor-map encoding and the launch
 // sequences of the forward and backward layer.  Argument marshalling and planning only; every
-// step of the layer runs in the kernels of route_layout.cu, permute.cu, gemm_tc3.cu, gemm_wgrad.cu,
-// gemm_tc2.cu and fused.cu.
+// step of the layer runs in the kernels of route_layout.cu, permute.cu, gemm_tc3.cu, gemm_wgrad.cu and fused.cu.
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -98,31 +97,25 @@ int encode_2d(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, u
   return encode_tiled(tm, base, 2, dims, strides, box);
 }
 
-// Store map of a [rows][2][F] view of a [rows][2F] matrix (gate half, up half): box 32 rows x 64 columns
-// of one half, so a column tile that ends past F is clipped instead of spilling into the other half.
-int encode_halves(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t F) {
-  const uint64_t dims[3] = {F, 2, rows}, strides[2] = {F * 2, 2 * F * 2};
-  const uint32_t box[3] = {64, 1, 32};
-  return encode_tiled(tm, base, 3, dims, strides, box);
-}
-
 // Store maps of the token-column tiles: un-swizzled boxes of 32 rows x `box_cols` columns.
 int encode_2d_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols) {
   const uint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
   const uint32_t box[2] = {box_cols, 32};
   return encode_tiled(tm, base, 2, dims, strides, box, false);
 }
+// [rows][2][F] view of a [rows][2F] matrix (gate half, up half): a column tile that ends past F is clipped instead of
+// spilling into the other half.
 int encode_halves_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t F, uint32_t box_cols) {
   const uint64_t dims[3] = {F, 2, rows}, strides[2] = {F * 2, 2 * F * 2};
   const uint32_t box[3] = {box_cols, 1, 32};
   return encode_tiled(tm, base, 3, dims, strides, box, false);
 }
-// Load map of W_gate_up viewed as [Ep][F/16 groups][gate | up][16 rows][d]: one box brings, for four
-// groups of 16 features, the 16 gate rows followed by the 16 up rows (needs F % 16 == 0).
+// Load map of W_gate_up viewed as [Ep][F/8 groups][gate | up][8 rows][d]: one box brings, for eight groups of 8
+// features, the 8 gate rows followed by the 8 up rows (8 divides every F).
 int encode_gate_up_rows(CUtensorMap* tm, const void* base, uint64_t Ep, uint64_t F, uint64_t d) {
-  const uint64_t dims[5] = {d, 16, 2, F / 16, Ep};
-  const uint64_t strides[4] = {d * 2, F * d * 2, 16 * d * 2, 2 * F * d * 2};
-  const uint32_t box[5] = {64, 16, 2, 4, 1};
+  const uint64_t dims[5] = {d, 8, 2, F / 8, Ep};
+  const uint64_t strides[4] = {d * 2, F * d * 2, 8 * d * 2, 2 * F * d * 2};
+  const uint32_t box[5] = {64, 8, 2, 8, 1};
   return encode_tiled(tm, base, 5, dims, strides, box);
 }
 
@@ -248,16 +241,13 @@ struct moe_ctx {
     for (bool& u : phase_used) u = false;
   }
   // tensor maps of workspace tensors (fixed for the context's lifetime)
-  CUtensorMap tm_Xp_k, tm_A_k, tm_dOutp_k, tm_dH_k;      // K-major A operands, box 128 x 64
   CUtensorMap tm_dOutp_mn, tm_A_mn, tm_dH_mn, tm_Xp_mn;  // MN-major operands of the weight gradients, box 64 x 64
   // tensor maps of the caller's weights, re-encoded when the pointers change
   const void* w1_ptr = nullptr;
   const void* w2_ptr = nullptr;
-  CUtensorMap tm_W1_k, tm_W2_k128, tm_W1_mn, tm_W2_mn;
-  CUtensorMap tm_W1_gu;  // token-column tiles: 16 gate rows + 16 up rows per box
+  CUtensorMap tm_W1_gu, tm_W2_k128, tm_W1_mn, tm_W2_mn;
   // store maps: workspace tensors (fixed) and the caller's weight gradients (re-encoded on change)
-  CUtensorMap ts_A, ts_H, ts_Y, ts_dH;
-  // token-column tiles: token operands with 64-row and 16-row boxes, un-swizzled store maps
+  // token operands with boxes of 16 .. 128 rows, un-swizzled store maps
   CUtensorMap tk_Xp[8], tk_A[8], tk_dOutp[8], tk_dH[8];
   CUtensorMap tp_A, tp_H, tp_Y, tp_dH;
   const void* dw1_ptr = nullptr;
@@ -316,9 +306,8 @@ int encode_weight_maps(moe_ctx* c, const uint16_t* W1, const uint16_t* W2) {
   const uint64_t Ep = s.E + s.n_shared;
   int rc;
   if (W1 != c->w1_ptr) {
-    if ((rc = encode_2d(&c->tm_W1_k, W1, Ep * 2 * s.F, s.d, 128, 64))) return rc;
     if ((rc = encode_2d(&c->tm_W1_mn, W1, Ep * 2 * s.F, s.d, 64, 64))) return rc;
-    if (s.F % 16 == 0 && (rc = encode_gate_up_rows(&c->tm_W1_gu, W1, Ep, s.F, s.d))) return rc;
+    if ((rc = encode_gate_up_rows(&c->tm_W1_gu, W1, Ep, s.F, s.d))) return rc;
     c->w1_ptr = W1;
   }
   if (W2 != c->w2_ptr) {
@@ -353,14 +342,14 @@ GemmArgs base_args(const moe_ctx* c) {
 GemmArgs args_gate_up(const moe_ctx* c) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
-  g.tmA = c->tm_Xp_k;
-  g.tmB = c->tm_W1_k;
+  memcpy(g.tmTok, c->tk_Xp, sizeof g.tmTok);
+  g.tmB = c->tm_W1_gu;
   g.n_tiles_n = (s.F + 127) / 128;
   g.K = s.d;
   g.N = s.F;
   g.b_rows_per_expert = 2 * s.F;
-  g.tmOut0 = c->ts_A;
-  g.tmOut1 = c->ts_H;
+  g.tmOut0 = c->tp_A;
+  g.tmOut1 = c->tp_H;
   g.save_h = c->train() ? 1 : 0;
   g.prow_w = c->at<float>(c->plan.prow_w);
   return g;
@@ -369,13 +358,13 @@ GemmArgs args_gate_up(const moe_ctx* c) {
 GemmArgs args_down(const moe_ctx* c) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
-  g.tmA = c->tm_A_k;
+  memcpy(g.tmTok, c->tk_A, sizeof g.tmTok);
   g.tmB = c->tm_W2_k128;  // each CTA of a pair loads 128 of the tile's 256 rows
   g.n_tiles_n = (s.d + 255) / 256;
   g.K = s.F;
   g.N = s.d;
   g.b_rows_per_expert = s.d;
-  g.tmOut0 = c->ts_Y;
+  g.tmOut0 = c->tp_Y;
   return g;
 }
 // act_grad + SwiGLU_grad (+ routing-weight gradient partials)
@@ -383,13 +372,13 @@ GemmArgs args_act_grad(const moe_ctx* c, bool want_dw) {
   const moe_shape& s = c->shape;
   const WsPlan& p = c->plan;
   GemmArgs g = base_args(c);
-  g.tmA = c->tm_dOutp_k;
+  memcpy(g.tmTok, c->tk_dOutp, sizeof g.tmTok);
   g.tmB = c->tm_W2_mn;
   g.n_tiles_n = p.ntn_act;
   g.K = s.d;
   g.N = s.F;
   g.b_rows_per_expert = s.d;
-  g.tmOut0 = c->ts_dH;
+  g.tmOut0 = c->tp_dH;
   g.in0 = c->at<uint16_t>(p.H);
   g.ld_in0 = 2 * s.F;
   g.prow_w = c->at<float>(p.prow_w);
@@ -413,13 +402,13 @@ GemmArgs args_wgrad_down(const moe_ctx* c) {
 GemmArgs args_gate_grad(const moe_ctx* c) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
-  g.tmA = c->tm_dH_k;
+  memcpy(g.tmTok, c->tk_dH, sizeof g.tmTok);
   g.tmB = c->tm_W1_mn;
   g.n_tiles_n = (s.d + 255) / 256;
   g.K = 2 * s.F;
   g.N = s.d;
   g.b_rows_per_expert = 2 * s.F;
-  g.tmOut0 = c->ts_Y;
+  g.tmOut0 = c->tp_Y;
   return g;
 }
 // w1_grad: dW_gate_up[e][n][c] = sum_rows dH[r][n] * Xp[r][c]   (shares dH with gate_grad)
@@ -436,45 +425,16 @@ GemmArgs args_wgrad_gate_up(const moe_ctx* c) {
   return g;
 }
 
-// Token-column tiles (gemm_tc3.cu, and the persistent launch) need the 16-feature gate/up groups of W_gate_up.
-bool token_col_tiles(const moe_ctx* c) { return c->shape.F % 16 == 0; }
-// Rewrites the arguments of a row-space operator for the token-column tiles: tmA/tmTok16 = tokens,
-// tmB = weights, un-swizzled store maps.
-GemmArgs to_token_cols(const moe_ctx* c, GemmMode mode, GemmArgs g) {
-  switch (mode) {
-    case GEMM_GATE_UP:
-      g.tmA = c->tm_Xp_k; memcpy(g.tmTok, c->tk_Xp, sizeof g.tmTok); g.tmB = c->tm_W1_gu;
-      g.tmOut0 = c->tp_A; g.tmOut1 = c->tp_H;
-      break;
-    case GEMM_DOWN:
-      g.tmA = c->tm_A_k; memcpy(g.tmTok, c->tk_A, sizeof g.tmTok); g.tmB = c->tm_W2_k128;
-      g.tmOut0 = c->tp_Y;
-      break;
-    case GEMM_ACT_GRAD:
-      g.tmA = c->tm_dOutp_k; memcpy(g.tmTok, c->tk_dOutp, sizeof g.tmTok);
-      g.tmOut0 = c->tp_dH;
-      break;
-    case GEMM_GATE_GRAD:
-      g.tmA = c->tm_dH_k; memcpy(g.tmTok, c->tk_dH, sizeof g.tmTok);
-      g.tmOut0 = c->tp_Y;
-      break;
-    default: break;
-  }
-  return g;
-}
 cudaError_t launch_gemm_serial(const moe_ctx* c, GemmMode mode, const GemmArgs& args, cudaStream_t st, int* launches) {
   if (mode == GEMM_WGRAD) return launch_wgrad_strips(args, c->num_sms, st, launches);
-  if (token_col_tiles(c)) return launch_gemm3(mode, to_token_cols(c, mode, args), c->num_sms, st, launches);
-  return launch_gemm2(mode, args, c->num_sms, st, launches);
+  return launch_gemm3(mode, args, c->num_sms, st, launches);
 }
 #define LAUNCH_GEMM_SERIAL(mode, args, sms, st, launches) launch_gemm_serial(c, mode, args, st, launches)
 
-// One launch per operator: on request, and for shapes the persistent launch does not cover (it runs the
-// token-column tiles only).
 int gate_mode(const moe_ctx* c) {
   return ((c->shape.flags & MOE_FLAG_RENORM_TOPK) ? GATE_RENORM : 0) | ((c->shape.flags & MOE_FLAG_SIGMOID_GATE) ? GATE_SIGMOID : 0);
 }
-bool serial_mode(const moe_ctx* c) { return (c->shape.flags & MOE_FLAG_SERIAL_LAUNCH) != 0 || !token_col_tiles(c); }
+bool serial_mode(const moe_ctx* c) { return (c->shape.flags & MOE_FLAG_SERIAL_LAUNCH) != 0; }
 
 ChainParams chain_params(const moe_ctx* c, bool bwd, int T, bool want_dw) {
   const moe_shape& s = c->shape;
@@ -621,8 +581,8 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     // one persistent launch: gather, GMM1+SwiGLU, GMM2 and combine tiles ordered by event counters
     FusedArgs fa = fused_base(c, false, T);
     fa.cp = chain_params(c, false, T, false);
-    fa.op[0] = to_token_cols(c, GEMM_GATE_UP, args_gate_up(c));
-    fa.op[1] = to_token_cols(c, GEMM_DOWN, args_down(c));
+    fa.op[0] = args_gate_up(c);
+    fa.op[1] = args_down(c);
     fa.gather_src = x;
     fa.gather_dst = c->at<uint16_t>(p.Xp);
     fa.topk_w = w;
@@ -669,7 +629,7 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     }
     if (d_w) {
       Phase ph(c, MOE_PHASE_DW_REDUCE, st);
-      MOE_CUDA(launch_dw_reduce(c->at<float>(p.dw_partial), token_col_tiles(c) ? p.ntn_act * DW_PARTS_PER_TILE : p.ntn_act,
+      MOE_CUDA(launch_dw_reduce(c->at<float>(p.dw_partial), p.ntn_act * DW_PARTS_PER_TILE,
                                 dm, lv, d_w, st, &c->launches));
     }
     {
@@ -699,9 +659,9 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
   } else {
     FusedArgs fa = fused_base(c, true, T);
     fa.cp = chain_params(c, true, T, d_w != nullptr);
-    fa.op[0] = to_token_cols(c, GEMM_ACT_GRAD, args_act_grad(c, d_w != nullptr));
+    fa.op[0] = args_act_grad(c, d_w != nullptr);
     fa.op[1] = args_wgrad_down(c);
-    fa.op[2] = to_token_cols(c, GEMM_GATE_GRAD, args_gate_grad(c));
+    fa.op[2] = args_gate_grad(c);
     fa.op[3] = args_wgrad_gate_up(c);
     fa.gather_src = dout;
     fa.gather_dst = c->at<uint16_t>(p.dOutp);
@@ -790,14 +750,6 @@ int moe_create(moe_ctx** out, const moe_shape* shape, void* workspace, size_t wo
   int rc = MOE_OK;
   cudaError_t e = cudaMemset(c->ws, 0, p.Xp);  // status, tables and small arrays start at zero
   if (e != cudaSuccess) rc = cuda_fail(e, "cudaMemset(workspace)");
-  if (!rc) rc = encode_2d(&c->tm_Xp_k, c->ws + p.Xp, cap, s.d, 128, 64);
-  if (!rc) rc = encode_2d(&c->tm_A_k, c->ws + p.A, cap, s.F, 128, 64);
-  if (!rc) rc = encode_2d(&c->ts_A, c->ws + p.A, cap, s.F, 32, 64);
-  if (!rc) rc = encode_2d(&c->ts_Y, c->ws + p.Y, cap, s.d, 32, 64);
-  if (!rc && train) rc = encode_halves(&c->ts_H, c->ws + p.H, cap, s.F);
-  if (!rc && train) rc = encode_halves(&c->ts_dH, c->ws + p.dH, cap, s.F);
-  if (!rc && train) rc = encode_2d(&c->tm_dOutp_k, c->ws + p.dOutp, cap, s.d, 128, 64);
-  if (!rc && train) rc = encode_2d(&c->tm_dH_k, c->ws + p.dH, cap, 2 * s.F, 128, 64);
   if (!rc && train) rc = encode_2d(&c->tm_dOutp_mn, c->ws + p.dOutp, cap, s.d, 64, 64);
   if (!rc && train) rc = encode_2d(&c->tm_A_mn, c->ws + p.A, cap, s.F, 64, 64);
   if (!rc && train) rc = encode_2d(&c->tm_dH_mn, c->ws + p.dH, cap, 2 * s.F, 64, 64);

@@ -402,7 +402,7 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
       tc_fence_after_sync();
       const int slot = st.resident ? kb : (int)is.a_s;
       if (issue) {
-        mma_kblock_pair<GEMM_WGRAD>(d_tmem, smem_u32(sA + slot * A_STAGE_BYTES), smem_u32(sB + is.s * HALF_B_BYTES),
+        mma_kblock_wgrad(d_tmem, smem_u32(sA + slot * A_STAGE_BYTES), smem_u32(sB + is.s * HALF_B_BYTES),
                                     kb == 0, k16_steps_of(st.rows, kb));
         tc_commit_pair(&bars->empty[is.s]);
         if (last_use) tc_commit_pair(&bars->a_empty[slot]);

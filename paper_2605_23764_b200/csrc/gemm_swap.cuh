@@ -111,9 +111,9 @@ __device__ __forceinline__ void load_weights_swap(const GemmArgs& a, const SwapT
   __syncwarp();
   const int brow = st.e * a.b_rows_per_expert;
   if (MODE == GEMM_GATE_UP) {
-    // one box [4 groups][gate | up][16 rows][64 k]: per epilogue warp 16 gate rows, then the 16 up rows
-    // of the same features (W_gate_up viewed as [Ep][F/16][2][16][d])
-    if (lane == 0) tma_load_5d_pair(sW, &a.tmB, k0, 0, 0, (st.n0 + rank * 64) >> 4, st.e, bar);
+    // one box [8 groups][gate | up][8 rows][64 k]: per group of 8 features the 8 gate rows, then the 8 up rows
+    // (W_gate_up viewed as [Ep][F/8][2][8][d]); groups beyond F read as zeros
+    if (lane == 0) tma_load_5d_pair(sW, &a.tmB, k0, 0, 0, (st.n0 + rank * 64) >> 3, st.e, bar);
   } else if (MODE == GEMM_DOWN) {
     if (lane == 0) tma_load_2d_pair(sW, &a.tmB, k0, brow + st.n0 + rank * 128, bar);
   } else {
@@ -209,11 +209,11 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
       }
     }
   } else if (MODE == GEMM_GATE_UP) {
-    // lanes 0..15: gate pre-activations of 16 features, lanes 16..31: up pre-activations of the same
-    // features.  For a token pair (j, j+1) the halves swap one value: the low half finishes token j,
-    // the high half token j+1.
-    const int fl = lane & 15;
-    const bool hi = lane >= 16;
+    // lanes 0..7 and 16..23: gate pre-activations of features 0..7 and 8..15 of the warp, lanes 8..15 and 24..31: up
+    // pre-activations of the same features.  For a token pair (j, j+1) gate and up lane of a feature swap one value: the
+    // gate lane finishes token j, the up lane token j+1.
+    const int fl = (lane & 7) + ((lane >> 4) << 3);
+    const bool hi = (lane & 8) != 0;
     const int fw0 = st.n0 + rank * 64 + quad * 16;   // first feature of this warp
     if (fw0 >= a.F) return;
 #pragma unroll 1
@@ -229,7 +229,7 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
 #pragma unroll
       for (int j = 0; j < 32; j += 2) {
         const float send = hi ? v[j] : v[j + 1];
-        const float recv = __shfl_xor_sync(0xffffffffu, send, 16);
+        const float recv = __shfl_xor_sync(0xffffffffu, send, 8);
         const float g = hi ? recv : v[j];
         const float u = hi ? v[j + 1] : recv;
         const int tj = j + (hi ? 1 : 0);

@@ -85,8 +85,8 @@ enum GemmMode : int {
 };
 
 struct GemmArgs {
-  CUtensorMap tmA;     // A operand
-  CUtensorMap tmB;     // B operand
+  CUtensorMap tmA;     // weight gradients: A operand
+  CUtensorMap tmB;     // row-space operators: the weights; weight gradients: B operand
   CUtensorMap tmOut0;  // store map of out0: [rows][N] (2-D), [rows][2][F] (dH), or [Ep][M][N] (WGRAD)
   CUtensorMap tmOut1;  // GATE_UP: store map of H as [rows][2][F]
   CUtensorMap tmTok[8]; // token-column tiles: the token operand with boxes of 16, 32, .., 128 rows (one TMA instruction
@@ -118,10 +118,6 @@ struct GemmArgs {
   DevStatus* status;
   uint64_t budget_ns;
 };
-
-// ---- gemm_tc2.cu: token-row tiles on CTA pairs (tcgen05 cta_group::2, 256 x 256): the row-space operators
-// of shapes the token-column tiles do not cover (F % 16 != 0)
-cudaError_t launch_gemm2(GemmMode mode, const GemmArgs& a, int num_sms, cudaStream_t s, int* launches);
 
 // ---- gemm_tc3.cu: the row-space operators with the tokens as accumulator COLUMNS (weights take the
 // 256 accumulator rows of a CTA pair), so a tile's MMA time follows the expert's real token count
