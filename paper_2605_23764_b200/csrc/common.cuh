@@ -100,6 +100,31 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   }
 }
 
+// The same for a converged warp that goes on with warp-uniform control flow: every lane polls, all lanes get one answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, const WaitCtl& wc, int site, int tile,
+                                               uint32_t sleep_ns = 0) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  uint64_t t0 = 0;
+  const uint32_t check = sleep_ns ? 63u : 1023u;
+  for (uint32_t spin = 1;; ++spin) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (sleep_ns) __nanosleep(sleep_ns);
+    if ((spin & check) == 0) {
+      int stop = 0;
+      if ((threadIdx.x & 31) == 0) {
+        stop = *reinterpret_cast<volatile int*>(&wc.status->abort);
+        const uint64_t now = globaltimer_ns();
+        if (t0 == 0) t0 = now;
+        else if (!stop && now - t0 > wc.budget_ns) {
+          report(wc.status, /*MOE_ERR_TIMEOUT*/ 2, (site << 24) | (tile & 0xFFFFFF));
+          stop = 1;
+        }
+      }
+      if (__shfl_sync(0xffffffffu, stop, 0)) return false;
+    }
+  }
+}
+
 // Bounded acquire-poll of a dependency counter in global memory until it reaches `threshold`
 // (the paper's "dependent event", Section 4.3).
 __device__ __forceinline__ bool counter_wait(const int* ctr, int threshold, const WaitCtl& wc, int tile,
@@ -238,19 +263,38 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// Warp-uniform issue.  tcgen05.mma, tcgen05.commit and TMA take their operands from uniform registers.  The compiler keeps
+// values there only where it can prove that the whole warp agrees: a warp index from __shfl_sync instead of
+// threadIdx.x >> 5, loop counters under uniform control flow, values read from memory passed through uniform(); and a
+// single issuing thread only where it is chosen by elect.sync next to the instruction.  A loop that issued under
+// `if (lane == 0)` from ordinary registers took 740 clocks per 64-deep k-block whatever the tile's size, more than the 512
+// clocks of a 256 x 256 tile's MMAs; this form takes 240, and the 256 x 256 main loop runs at the tensor cores' rate.
+// All lanes of a converged warp call these functions; elect.sync picks the same lane every time.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+__device__ __forceinline__ void mbar_expect_tx_elect(uint64_t* bar, uint32_t bytes) {
+  asm volatile(
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(smem_u32(bar)), "r"(bytes)
+      : "memory");
+}
 // TMA load whose completion bytes are counted on the EVEN CTA's barrier at the same offset.
 __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorMap* m, int x, int y, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];"
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];\n}"
       ::"r"(smem_u32(smem_dst)), "l"(m), "r"(x), "r"(y), "r"(smem_u32(bar) & PEER_BIT_MASK)
       : "memory");
 }
 __device__ __forceinline__ void tma_load_5d_pair(void* smem_dst, const CUtensorMap* m, int c0, int c1, int c2, int c3,
                                                  int c4, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n}"
       ::"r"(smem_u32(smem_dst)), "l"(m), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4),
         "r"(smem_u32(bar) & PEER_BIT_MASK)
       : "memory");
@@ -273,29 +317,36 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 // Arrive on `bar` in BOTH CTAs of the pair once the MMAs issued so far have completed.
 __device__ __forceinline__ void tc_commit_pair(uint64_t* bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}"
       ::"r"(smem_u32(bar)), "h"(static_cast<uint16_t>(3))
       : "memory");
 }
-__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                 uint32_t accumulate) {
+// STEPS 16-deep MMAs of a k-block: D (+)= A . B, descriptors given as low words (address and leading offset; the high word
+// is common to all operands here), advanced by ASTEP / BSTEP 16-byte units per step.
+template <int ASTEP, int BSTEP>
+__device__ __forceinline__ void tc_mma4_bf16_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                  uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred e, p;\n .reg .b64 da, db;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %5, 0;\n"
+      " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n"
+      " add.u64 da, da, %6;\n add.u64 db, db, %7;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, 1;\n"
+      " add.u64 da, da, %6;\n add.u64 db, db, %7;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, 1;\n"
+      " add.u64 da, da, %6;\n add.u64 db, db, %7;\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, 1;\n}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate), "n"(ASTEP), "n"(BSTEP)
       : "memory");
 }
-
-// The same with the descriptors given as 32-bit halves: the single issuing thread's instruction stream
-// is what bounds short MMAs, so its loop keeps the constant high words in registers and only adds
-// the k-step to the low words (address field, bits 0..13, in 16-byte units).
-__device__ __forceinline__ void tc_mma_bf16_pair_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                                      uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma1_bf16_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                  uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n .reg .b64 da, db;\n mov.b64 da, {%1, %2};\n mov.b64 db, {%3, %4};\n"
-      " setp.ne.b32 p, %6, 0;\n"
-      " tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %5, p;\n}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred e, p;\n .reg .b64 da, db;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %5, 0;\n"
+      " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Halves of make_smem_desc(addr, lbo, sbo)
@@ -359,12 +410,13 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 
 }  // namespace moe
 
-// ---------------------------------------------------------------- single-CTA forms (tcgen05 cta_group::1)
+// ---------------------------------------------------------------- single-CTA forms (tcgen05 cta_group::1), issued like the pair's
 namespace moe {
 
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* m, int x, int y, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n}"
       ::"r"(smem_u32(smem_dst)), "l"(m), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
@@ -379,14 +431,24 @@ __device__ __forceinline__ void tmem_dealloc_cta(uint32_t taddr, uint32_t ncols)
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 __device__ __forceinline__ void tc_commit_cta(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void tc_mma_bf16_cta(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                                uint32_t accumulate) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+      " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar)) : "memory");
+}
+// Four 16-deep MMAs of a k-block, both operands K-major.
+__device__ __forceinline__ void tc_mma4_bf16_cta(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc,
+                                                 uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred e, p;\n .reg .b64 da, db;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %5, 0;\n"
+      " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n"
+      " add.u64 da, da, 2;\n add.u64 db, db, 2;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, 1;\n"
+      " add.u64 da, da, 2;\n add.u64 db, db, 2;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, 1;\n"
+      " add.u64 da, da, 2;\n add.u64 db, db, 2;\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, 1;\n}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }

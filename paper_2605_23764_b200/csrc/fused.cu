@@ -411,18 +411,18 @@ __device__ __forceinline__ bool load_item(const FusedArgs& fa, const WorkDesc& w
 }
 template <bool BWD>
 __device__ __forceinline__ bool issue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
-                                           uint32_t tmem_base, IssuerState& is, bool issue, const WaitCtl& wc,
+                                           uint32_t tmem_base, IssuerState& is, const WaitCtl& wc,
                                            const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
   if (BWD && (phase == 1 || phase == 3))
-    return wgrad_issue_strip(fa.op[phase], smem, bars, tmem_base, is, issue, desc_strip(wd), t, wc, dep);
+    return wgrad_issue_strip(fa.op[phase], smem, bars, tmem_base, is, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
-    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], smem, bars, tmem_base, is, issue, wk, t, wc, dep);
-    return swap_issue_item<GEMM_DOWN>(fa.op[1], smem, bars, tmem_base, is, issue, wk, t, wc, dep);
+    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], smem, bars, tmem_base, is, wk, t, wc, dep);
+    return swap_issue_item<GEMM_DOWN>(fa.op[1], smem, bars, tmem_base, is, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, tmem_base, is, issue, wk, t, wc, dep);
-  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, tmem_base, is, issue, wk, t, wc, dep);
+  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, tmem_base, is, wk, t, wc, dep);
+  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, tmem_base, is, wk, t, wc, dep);
 }
 template <bool BWD>
 __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   static_assert(sizeof(PipeBarriers) <= 256 && sizeof(TicketRing) <= 384, "shared-memory bookkeeping");
   TicketRing* ring = reinterpret_cast<TicketRing*>(reinterpret_cast<uint8_t*>(bars) + 256);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const WaitCtl wc{fa.status, fa.budget_ns};
   const TraceCtl tr{fa.trace, fa.trace_cap, fa.ctr + CTR_TRACE_CURSOR};
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers exist before anyone signals across the pair
   tc_fence_after_sync();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = uniform(bars->tmem_base);
 
   if (warp == SCHED_WARP && rank == 0) {
     // ------------------------------------------------ scheduler of the pair (even CTA)
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (warp == 0 || warp == 6)
         ok = load_item<BWD>(fa, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
       else if (warp == 1)
-        ok = issue_item<BWD>(fa, wd, smem, bars, tmem_base, is, lane == 0, wc, dep);
+        ok = issue_item<BWD>(fa, wd, smem, bars, tmem_base, is, wc, dep);
       else
         ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, warp & 3, lane, wc, dep);
     }
@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       tma_store_wait_all();
       epi_enter_phase(bars, warp & 3, SCHED_MAX_SEG);   // nothing of this warp is left in shared memory
     }
-    if (warp == 1 && lane == 0 && (!ok || *reinterpret_cast<volatile int*>(&fa.status->abort))) issuer_drain(bars, fa.status);
+    if (warp == 1 && uniform(!ok || *reinterpret_cast<volatile int*>(&fa.status->abort) ? 1 : 0)) issuer_drain(bars, fa.status);
   }
 
   // ------------------------------------------------ vector workers: the dedicated warps from the start, the

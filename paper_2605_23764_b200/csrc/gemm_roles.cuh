@@ -80,10 +80,10 @@ __device__ __forceinline__ bool phase_wait(PipeBarriers* bars, int phase, const 
 }
 
 // After a failed or aborted launch: let the tensor core finish what was issued before TMEM is freed.
-__device__ __forceinline__ void issuer_drain(PipeBarriers* bars, DevStatus* status) {   // one lane
+__device__ __forceinline__ void issuer_drain(PipeBarriers* bars, DevStatus* status) {   // the issuing warp
   tc_commit_pair(&bars->drain);
   const WaitCtl shortwc{status, 20ull * 1000 * 1000};
-  mbar_wait(&bars->drain, 0, shortwc, SITE_DRAIN, 0);
+  mbar_wait_warp(&bars->drain, 0, shortwc, SITE_DRAIN, 0);
 }
 
 // ---------------------------------------------------------------- per-tile trace (optional)
@@ -163,68 +163,65 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem,
   // with events: the item was published only after its dependent events were met (acquired by the scheduler,
   // handed on through the ticket ring); what the producers wrote must be seen by the TMA loads
   if (DEP::kOn && tok_warp) fence_proxy_async();
-  for (int kb = 0; kb < wk.a.nkb; ++kb) {
-    int go = 1;
-    if (lane == 0) go = mbar_wait(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, t, 50) ? 1 : 0;
-    go = __shfl_sync(0xffffffffu, go, 0);
-    if (!go) return false;
+  const int nkb = uniform(wk.a.nkb), e = uniform(wk.a.e), n0 = uniform(wk.a.n0);
+  const int row_a = uniform(wk.a.row0), half_a = uniform(wk.a.ntok) >> 1;
+  const int row_b = uniform(wk.b.row0), half_b = wk.merged ? uniform(wk.b.ntok) >> 1 : 0;
+  for (int kb = 0; kb < nkb; ++kb) {
+    if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, t, 50)) return false;
     ls.empty_par ^= 1u << ls.s;
     if (!tok_warp) {
-      load_weights_swap<MODE>(a, wk.a, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], lane, wk.a.ntok + wk.b.ntok);
+      load_weights_swap<MODE>(a, e, n0, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], 2 * (half_a + half_b));
     } else {
-      load_tokens_swap(a, wk.a, kb, rank, sT + ls.s * TOKB, &bars->full[ls.s], lane);
-      if (wk.merged)   // lane 1: the second token tile, behind the first in the stage
-        load_tokens_swap(a, wk.b, kb, rank, sT + ls.s * TOKB + (wk.a.ntok >> 1) * (BK * 2), &bars->full[ls.s], lane - 1);
+      load_tokens_swap(a, row_a, half_a, kb, rank, sT + ls.s * TOKB, &bars->full[ls.s]);
+      if (half_b)   // the second token tile, behind the first in the stage
+        load_tokens_swap(a, row_b, half_b, kb, rank, sT + ls.s * TOKB + half_a * (BK * 2), &bars->full[ls.s]);
     }
     if (++ls.s == PIPE_STAGES) ls.s = 0;
   }
   return true;
 }
 
-// MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop (uniform control flow: lanes parked at a
-// warp barrier while one lane loops would share that lane's issue slots) and lane 0 (`issue`) alone issues
-// the MMAs and commits.  The loop bounds the tensor pipe when a k-block's MMAs are short: stage index, phase
-// and descriptor words are carried in registers.
+// MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop with uniform control flow and operands; one elected
+// lane issues (common.cuh).
 template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
-                                                IssuerState& is, bool issue, const SwapWork& wk, int t,
-                                                const WaitCtl& wc, const DEP& dep) {
+                                                IssuerState& is, const SwapWork& wk, int t, const WaitCtl& wc,
+                                                const DEP& dep) {
   constexpr int TOKB = tok_stage_bytes<MODE>();
   const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
   const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + PIPE_STAGES * W_STAGE_BYTES), 16);
   uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * (TOKB >> 4);
   const int as = is.acc_it & 1;
-  if (!mbar_wait(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
-  if (wk.merged &&   // the second token tile accumulates in the other buffer
-      !mbar_wait(&bars->tmem_empty[as ^ 1], (((is.acc_it + 1) >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
+  const int nkb = uniform(wk.a.nkb), ntok = uniform(wk.a.ntok), ntok_b = uniform(wk.merged ? wk.b.ntok : 0);
+  if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
+  if (ntok_b &&   // the second token tile accumulates in the other buffer
+      !mbar_wait_warp(&bars->tmem_empty[as ^ 1], (((is.acc_it + 1) >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
   tc_fence_after_sync();
   const uint32_t d_tmem = tmem_base + as * BN, d_tmem_b = tmem_base + (as ^ 1) * BN;
-  const uint32_t idesc = swap_idesc<MODE>(wk.a.ntok), idesc_b = swap_idesc<MODE>(wk.merged ? wk.b.ntok : TOK_GRAIN);
-  const uint32_t t_off_b = (uint32_t)((wk.a.ntok >> 1) * (BK * 2)) >> 4;
+  const uint32_t idesc = swap_idesc<MODE>(ntok), idesc_b = swap_idesc<MODE>(ntok_b ? ntok_b : TOK_GRAIN);
+  const uint32_t t_off_b = (uint32_t)((ntok >> 1) * (BK * 2)) >> 4;
   uint64_t t0 = 0;
-  for (int kb = 0; kb < wk.a.nkb; ++kb) {
-    if (!mbar_wait(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, t)) return false;
+  for (int kb = 0; kb < nkb; ++kb) {
+    if (!mbar_wait_warp(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, t)) return false;
     is.full_par ^= 1u << is.s;
-    if (DEP::kOn && kb == 0 && issue && dep.tracing()) t0 = globaltimer_ns();
+    if (DEP::kOn && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
     tc_fence_after_sync();
-    if (issue) {
-      mma_kblock_swap<MODE>(d_tmem, w_lo, t_lo, idesc, kb == 0);
-      if (wk.merged) mma_kblock_swap<MODE>(d_tmem_b, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
-      tc_commit_pair(&bars->empty[is.s]);   // frees the stage in both CTAs
-    }
+    mma_kblock_swap<MODE>(d_tmem, w_lo, t_lo, idesc, kb == 0);
+    if (ntok_b) mma_kblock_swap<MODE>(d_tmem_b, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
+    tc_commit_pair(&bars->empty[is.s]);   // frees the stage in both CTAs
     if (++is.s == PIPE_STAGES) {
       is.s = 0; w_lo = w_lo0; t_lo = t_lo0;
     } else {
       w_lo += W_STAGE_BYTES >> 4; t_lo += TOKB >> 4;
     }
   }
-  if (issue) tc_commit_pair(&bars->tmem_full[as]);  // accumulator slices ready in both CTAs
+  tc_commit_pair(&bars->tmem_full[as]);  // accumulator slices ready in both CTAs
   ++is.acc_it;
-  if (wk.merged) {
-    if (issue) tc_commit_pair(&bars->tmem_full[as ^ 1]);
+  if (ntok_b) {
+    tc_commit_pair(&bars->tmem_full[as ^ 1]);
     ++is.acc_it;
   }
-  if (DEP::kOn && issue && dep.tracing()) dep.trace(TR_MMA, t, t0, t0, globaltimer_ns());
+  if (DEP::kOn && dep.tracing() && (threadIdx.x & 31) == 0) dep.trace(TR_MMA, t, t0, t0, globaltimer_ns());
   return true;
 }
 
@@ -346,35 +343,29 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
                                                  const WaitCtl& wc, const DEP& dep) {
   uint8_t* sA = smem;                                   // [PIPE_STAGES][16 KB] A slots
   uint8_t* sB = smem + PIPE_STAGES * A_STAGE_BYTES;     // [WG_B_STAGES][16 KB] B stages
-  const int m0 = st.m0(rank);
+  const int m0 = uniform(st.m0(rank)), row0 = uniform(st.row0), nkb = uniform(st.nkb);
+  const bool resident = nkb <= A_RES_KB;
   if (DEP::kOn) fence_proxy_async();   // as in swap_load_item
   for (int nb = 0; nb < a.n_tiles_n; ++nb) {
-    const bool load_a = !st.resident || nb == 0;
-    for (int kb = 0; kb < st.nkb; ++kb) {
-      const int slot = st.resident ? kb : (int)ls.a_s;
-      int go = 1;
-      if (lane == 0) {
-        go = mbar_wait(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, sp, 50) ? 1 : 0;
-        if (go && !b_warp && load_a)
-          go = mbar_wait(&bars->a_empty[slot], (ls.a_ph >> slot) & 1, wc, SITE_EMPTY, sp, 50) ? 1 : 0;
-      }
-      go = __shfl_sync(0xffffffffu, go, 0);
-      if (!go) return false;
-      const int k0 = kb * BK;
+    const bool load_a = !resident || nb == 0;
+    for (int kb = 0; kb < nkb; ++kb) {
+      const int slot = resident ? kb : (int)ls.a_s;
+      if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, sp, 50)) return false;
+      if (!b_warp && load_a && !mbar_wait_warp(&bars->a_empty[slot], (ls.a_ph >> slot) & 1, wc, SITE_EMPTY, sp, 50)) return false;
+      const int k0 = row0 + kb * BK;
       if (!b_warp) {
-        if (lane == 0 && rank == 0)
-          mbar_expect_tx(&bars->full[ls.s], 2 * (HALF_B_BYTES + (load_a ? A_STAGE_BYTES : 0)));
-        __syncwarp();
-        if (load_a && lane < 2)
-          tma_load_2d_pair(sA + slot * A_STAGE_BYTES + lane * MN_BOX_BYTES, &a.tmA, m0 + lane * 64, st.row0 + k0,
-                           &bars->full[ls.s]);
-      } else if (lane < 2) {
-        tma_load_2d_pair(sB + ls.s * HALF_B_BYTES + lane * MN_BOX_BYTES, &a.tmB, nb * BN + (2 * rank + lane) * 64,
-                         st.row0 + k0, &bars->full[ls.s]);
+        if (rank == 0) mbar_expect_tx_elect(&bars->full[ls.s], 2 * (HALF_B_BYTES + (load_a ? A_STAGE_BYTES : 0)));
+        if (load_a) {
+          tma_load_2d_pair(sA + slot * A_STAGE_BYTES, &a.tmA, m0, k0, &bars->full[ls.s]);
+          tma_load_2d_pair(sA + slot * A_STAGE_BYTES + MN_BOX_BYTES, &a.tmA, m0 + 64, k0, &bars->full[ls.s]);
+        }
+      } else {
+        tma_load_2d_pair(sB + ls.s * HALF_B_BYTES, &a.tmB, nb * BN + 2 * rank * 64, k0, &bars->full[ls.s]);
+        tma_load_2d_pair(sB + ls.s * HALF_B_BYTES + MN_BOX_BYTES, &a.tmB, nb * BN + (2 * rank + 1) * 64, k0, &bars->full[ls.s]);
       }
       ls.empty_par ^= 1u << ls.s;
       if (load_a) ls.a_ph ^= 1u << slot;
-      if (!st.resident && ++ls.a_s == PIPE_STAGES) ls.a_s = 0;
+      if (!resident && ++ls.a_s == PIPE_STAGES) ls.a_s = 0;
       if (++ls.s == WG_B_STAGES) ls.s = 0;
     }
   }
@@ -383,37 +374,47 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
 
 template <class DEP>
 __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
-                                                  IssuerState& is, bool issue, const Strip& st, int sp,
-                                                  const WaitCtl& wc, const DEP& dep) {
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + PIPE_STAGES * A_STAGE_BYTES;
-  if (st.nkb == 0) return true;
+                                                  IssuerState& is, const Strip& st, int sp, const WaitCtl& wc,
+                                                  const DEP& dep) {
+  const uint32_t a_lo0 = smem_desc_lo(smem_u32(smem), MN_BOX_BYTES);
+  const uint32_t b_lo0 = smem_desc_lo(smem_u32(smem + PIPE_STAGES * A_STAGE_BYTES), MN_BOX_BYTES);
+  constexpr uint32_t idesc = make_idesc_bf16(2 * BLOCK_M, BN, 1, 1), hi = smem_desc_hi(1024);
+  constexpr int KSTEP = 2048 >> 4;   // 16 k-rows of an MN-major box
+  const int nkb = uniform(st.nkb), rows = uniform(st.rows);
+  const bool resident = nkb <= A_RES_KB;
+  if (nkb == 0) return true;
   uint64_t t0 = 0;
   for (int nb = 0; nb < a.n_tiles_n; ++nb) {
     const int as = is.acc_it & 1;
-    if (!mbar_wait(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, sp)) return false;
+    if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, sp)) return false;
     tc_fence_after_sync();
     const uint32_t d_tmem = tmem_base + as * BN;
-    const bool last_use = !st.resident || nb == a.n_tiles_n - 1;
-    for (int kb = 0; kb < st.nkb; ++kb) {
-      if (!mbar_wait(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, sp)) return false;
+    const bool last_use = !resident || nb == a.n_tiles_n - 1;
+    for (int kb = 0; kb < nkb; ++kb) {
+      if (!mbar_wait_warp(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, sp)) return false;
       is.full_par ^= 1u << is.s;
-      if (DEP::kOn && nb == 0 && kb == 0 && issue && dep.tracing()) t0 = globaltimer_ns();
+      if (DEP::kOn && nb == 0 && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
       tc_fence_after_sync();
-      const int slot = st.resident ? kb : (int)is.a_s;
-      if (issue) {
-        mma_kblock_wgrad(d_tmem, smem_u32(sA + slot * A_STAGE_BYTES), smem_u32(sB + is.s * HALF_B_BYTES),
-                                    kb == 0, k16_steps_of(st.rows, kb));
-        tc_commit_pair(&bars->empty[is.s]);
-        if (last_use) tc_commit_pair(&bars->a_empty[slot]);
+      const int slot = resident ? kb : (int)is.a_s;
+      const uint32_t a_lo = a_lo0 + slot * (A_STAGE_BYTES >> 4), b_lo = b_lo0 + is.s * (HALF_B_BYTES >> 4);
+      // the last k-block may hold fewer than 64 rows of the expert: the 16-row steps that would only multiply
+      // zero padding are not issued
+      const int steps = k16_steps_of(rows, kb);
+      if (steps == BK / 16) {
+        tc_mma4_bf16_pair<KSTEP, KSTEP>(d_tmem, a_lo, b_lo, hi, idesc, kb != 0);
+      } else {
+        for (int k16 = 0; k16 < steps; ++k16)
+          tc_mma1_bf16_pair(d_tmem, a_lo + k16 * KSTEP, b_lo + k16 * KSTEP, hi, idesc, kb != 0 || k16 != 0);
       }
-      if (!st.resident && ++is.a_s == PIPE_STAGES) is.a_s = 0;
+      tc_commit_pair(&bars->empty[is.s]);
+      if (last_use) tc_commit_pair(&bars->a_empty[slot]);
+      if (!resident && ++is.a_s == PIPE_STAGES) is.a_s = 0;
       if (++is.s == WG_B_STAGES) is.s = 0;
     }
-    if (issue) tc_commit_pair(&bars->tmem_full[as]);
+    tc_commit_pair(&bars->tmem_full[as]);
     ++is.acc_it;
   }
-  if (DEP::kOn && issue && dep.tracing()) dep.trace(TR_MMA, sp, t0, t0, globaltimer_ns());
+  if (DEP::kOn && dep.tracing() && (threadIdx.x & 31) == 0) dep.trace(TR_MMA, sp, t0, t0, globaltimer_ns());
   return true;
 }
 

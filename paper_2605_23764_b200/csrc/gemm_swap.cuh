@@ -94,45 +94,40 @@ __device__ __forceinline__ uint32_t swap_stage_tx_bytes(int ntok) {
   return 2u * (uint32_t)(W_STAGE_BYTES + (ntok >> 1) * BK * 2);   // both CTAs: weights + half of the tokens
 }
 
-// This CTA's loads of one k-block are split over two producer warps, one box per lane (issuing a TMA
-// box costs its thread on the order of a hundred cycles, and a k-block of a short tile only lasts a
-// few hundred).  Tokens: rows [row0 + rank * ntok/2, + ntok/2) as ONE box (a tensor map per box height).  The even CTA's weight producer arms the barrier for both CTAs' bytes.
-__device__ __forceinline__ void load_tokens_swap(const GemmArgs& a, const SwapTile& st, int kb, int rank, uint8_t* sT,
-                                                 uint64_t* bar, int lane) {
-  if (lane != 0) return;
-  const int half = st.ntok >> 1;   // a multiple of 16, at most 128: one box of exactly that many rows
-  tma_load_2d_pair(sT, &a.tmTok[(half >> 4) - 1], kb * BK, st.row0 + rank * half, bar);
+// This CTA's loads of one k-block are split over two producer warps.  Tokens: rows [row0 + rank * ntok/2, + ntok/2) as ONE
+// box (a tensor map per box height).  The even CTA's weight producer arms the barrier for both CTAs' bytes.
+__device__ __forceinline__ void load_tokens_swap(const GemmArgs& a, int row0, int half, int kb, int rank, uint8_t* sT,
+                                                 uint64_t* bar) {
+  // half: a multiple of 16, at most 128: one box of exactly that many rows
+  tma_load_2d_pair(sT, &a.tmTok[(half >> 4) - 1], kb * BK, row0 + rank * half, bar);
 }
 template <int MODE>
-__device__ __forceinline__ void load_weights_swap(const GemmArgs& a, const SwapTile& st, int kb, int rank, uint8_t* sW,
-                                                  uint64_t* bar, int lane, int ntok_total = -1) {
+__device__ __forceinline__ void load_weights_swap(const GemmArgs& a, int e, int n0, int kb, int rank, uint8_t* sW,
+                                                  uint64_t* bar, int ntok_total) {
   const int k0 = kb * BK;
-  if (lane == 0 && rank == 0) mbar_expect_tx(bar, swap_stage_tx_bytes(ntok_total < 0 ? st.ntok : ntok_total));
-  __syncwarp();
-  const int brow = st.e * a.b_rows_per_expert;
+  if (rank == 0) mbar_expect_tx_elect(bar, swap_stage_tx_bytes(ntok_total));
+  const int brow = e * a.b_rows_per_expert;
   if (MODE == GEMM_GATE_UP) {
     // one box [8 groups][gate | up][8 rows][64 k]: per group of 8 features the 8 gate rows, then the 8 up rows
     // (W_gate_up viewed as [Ep][F/8][2][8][d]); groups beyond F read as zeros
-    if (lane == 0) tma_load_5d_pair(sW, &a.tmB, k0, 0, 0, (st.n0 + rank * 64) >> 3, st.e, bar);
+    tma_load_5d_pair(sW, &a.tmB, k0, 0, 0, (n0 + rank * 64) >> 3, e, bar);
   } else if (MODE == GEMM_DOWN) {
-    if (lane == 0) tma_load_2d_pair(sW, &a.tmB, k0, brow + st.n0 + rank * 128, bar);
+    tma_load_2d_pair(sW, &a.tmB, k0, brow + n0 + rank * 128, bar);
   } else {
     // ACT_GRAD / GATE_GRAD: the forward weight read along its rows -> two MN-major [64 k][64 features] boxes
-    if (lane < 2) tma_load_2d_pair(sW + lane * MN_BOX_BYTES, &a.tmB, st.n0 + (2 * rank + lane) * 64, brow + k0, bar);
+    tma_load_2d_pair(sW, &a.tmB, n0 + 2 * rank * 64, brow + k0, bar);
+    tma_load_2d_pair(sW + MN_BOX_BYTES, &a.tmB, n0 + (2 * rank + 1) * 64, brow + k0, bar);
   }
 }
 
 // One 64-deep k-block: D[256 features x ntok tokens] (+)= W . X^T.  w_lo / t_lo: low descriptor words of
-// the stage's weight and token tiles (smem_desc_lo); the issuing thread only adds the k-step.
+// the stage's weight and token tiles (smem_desc_lo).
 template <int MODE>
 __device__ __forceinline__ void mma_kblock_swap(uint32_t d_tmem, uint32_t w_lo, uint32_t t_lo, uint32_t idesc,
                                                 bool first_kblock) {
   constexpr bool W_MN = (MODE == GEMM_ACT_GRAD || MODE == GEMM_GATE_GRAD);
-  constexpr uint32_t hi = smem_desc_hi(1024);
-  constexpr uint32_t wstep = W_MN ? (2048 >> 4) : (32 >> 4);   // 16 k-rows of an MN-major box / 32 bytes of a K-major row
-#pragma unroll
-  for (int k16 = 0; k16 < BK / 16; ++k16)
-    tc_mma_bf16_pair_lohi(d_tmem, w_lo + k16 * wstep, hi, t_lo + k16 * 2, hi, idesc, !(first_kblock && k16 == 0));
+  // 16 k-rows of an MN-major box / 32 bytes of a K-major row
+  tc_mma4_bf16_pair<W_MN ? (2048 >> 4) : (32 >> 4), (32 >> 4)>(d_tmem, w_lo, t_lo, smem_desc_hi(1024), idesc, !first_kblock);
 }
 template <int MODE>
 __device__ __forceinline__ uint32_t swap_w_desc_lo(uint32_t w_addr) {

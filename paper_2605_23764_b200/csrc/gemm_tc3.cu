@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + swap_layout_bytes<MODE>());
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const WaitCtl wc{a.status, a.budget_ns};
@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers exist before anyone signals across the pair
   tc_fence_after_sync();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = uniform(bars->tmem_base);
 
   // Items pair, pair + npairs, ..; each role decodes item i + 1 before it works on item i (the decode's chain of
   // global loads then completes behind the item's work).
@@ -65,9 +65,9 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       bool ok = true;
       for (int t = pair; t < total && ok; t += npairs, cur = next) {
         if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-        ok = swap_issue_item<MODE>(a, smem, bars, tmem_base, is, lane == 0, cur, t, wc, dep);
+        ok = swap_issue_item<MODE>(a, smem, bars, tmem_base, is, cur, t, wc, dep);
       }
-      if (lane == 0 && (!ok || *reinterpret_cast<volatile int*>(&a.status->abort))) issuer_drain(bars, a.status);
+      if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
   } else {
     EpiState es;

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) grouped_wgrad_pair_kernel(const
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + WGRAD_LAYOUT_BYTES);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   const WaitCtl wc{a.status, a.budget_ns};
@@ -38,7 +38,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) grouped_wgrad_pair_kernel(const
   __syncthreads();
   cluster_sync_all();
   tc_fence_after_sync();
-  const uint32_t tmem_base = bars->tmem_base;
+  const uint32_t tmem_base = uniform(bars->tmem_base);
 
   // Strips pair, pair + npairs, ..; each role decodes strip i + 1 before it works on strip i.
   const int total = wgrad_strips(a);
@@ -56,9 +56,9 @@ __global__ void __launch_bounds__(WG_THREADS, 1) grouped_wgrad_pair_kernel(const
       bool ok = true;
       for (int sp = pair; sp < total && ok; sp += npairs, cur = next) {
         if (sp + npairs < total) next = decode_strip(a, sp + npairs);
-        ok = wgrad_issue_strip(a, smem, bars, tmem_base, is, lane == 0, cur, sp, wc, dep);
+        ok = wgrad_issue_strip(a, smem, bars, tmem_base, is, cur, sp, wc, dep);
       }
-      if (lane == 0 && (!ok || *reinterpret_cast<volatile int*>(&a.status->abort))) issuer_drain(bars, a.status);
+      if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
   } else {
     EpiState es;

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
   // behind the operand ring where both fit, in its place (after the k-loop) where they do not
   float4* part = reinterpret_cast<float4*>(smem + (a.part_over_ring ? 0 : a.stages * (NACC * ROUTER_W_BYTES + a.ntok * BK * 2)));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int C = a.csize, rank = (int)cluster_ctarank();
   const int cluster = blockIdx.x / C, nclusters = gridDim.x / C;
   const WaitCtl wc{a.status, a.budget_ns};
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
   __syncthreads();
   tc_fence_after_sync();
   if (C > 1) cluster_arrive();   // waited for before the first access to another CTA's shared memory
-  const uint32_t tmem_base = bars.tmem_base;
+  const uint32_t tmem_base = uniform(bars.tmem_base);
   pdl_trigger();
   pdl_wait();
 
@@ -157,28 +157,26 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
   bool ok = true;   // a failed wait: this warp skips the work but still meets the barriers
   for (int t = cluster; t < ntiles; t += nclusters, ++n_tile) {
     const int t0 = t * ntok;
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
       for (int kb = kb0; kb < kb1 && ok; ++kb) {
-        if (!mbar_wait(&bars.empty[s_ld], ph_ld, wc, SITE_EMPTY, t, 20)) { ok = false; break; }
+        if (!mbar_wait_warp(&bars.empty[s_ld], ph_ld, wc, SITE_EMPTY, t, 20)) { ok = false; break; }
         uint8_t* st = smem + s_ld * stage_bytes;
-        mbar_expect_tx(&bars.full[s_ld], stage_bytes);
+        mbar_expect_tx_elect(&bars.full[s_ld], stage_bytes);
         tma_load_2d(st, &a.tmW, kb * BK, 0, &bars.full[s_ld]);
         if (NACC == 2) tma_load_2d(st + ROUTER_W_BYTES, &a.tmW, kb * BK, 128, &bars.full[s_ld]);
         tma_load_2d(st + NACC * ROUTER_W_BYTES, &a.tmX, kb * BK, t0, &bars.full[s_ld]);
         if (++s_ld == (uint32_t)a.stages) { s_ld = 0; ph_ld ^= 1; }
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       const uint32_t idesc = make_idesc_bf16(BLOCK_M, ntok, 0, 0);
+      const uint32_t ring_lo = smem_desc_lo(smem_u32(smem), 16);
       for (int kb = kb0; kb < kb1 && ok; ++kb) {
-        if (!mbar_wait(&bars.full[s_mma], ph_mma, wc, SITE_FULL, t)) { ok = false; break; }
+        if (!mbar_wait_warp(&bars.full[s_mma], ph_mma, wc, SITE_FULL, t)) { ok = false; break; }
         tc_fence_after_sync();
-        const uint32_t w_addr = smem_u32(smem + s_mma * stage_bytes), x_addr = w_addr + NACC * ROUTER_W_BYTES;
+        const uint32_t w_lo = ring_lo + s_mma * (stage_bytes >> 4), x_lo = w_lo + NACC * (ROUTER_W_BYTES >> 4);
 #pragma unroll
-        for (int k16 = 0; k16 < BK / 16; ++k16)
-#pragma unroll
-          for (int h = 0; h < NACC; ++h)
-            tc_mma_bf16_cta(tmem_base + h * acc_cols, make_smem_desc(w_addr + h * ROUTER_W_BYTES + k16 * 32, 16, 1024),
-                            make_smem_desc(x_addr + k16 * 32, 16, 1024), idesc, !(kb == kb0 && k16 == 0));
+        for (int h = 0; h < NACC; ++h)
+          tc_mma4_bf16_cta(tmem_base + h * acc_cols, w_lo + h * (ROUTER_W_BYTES >> 4), x_lo, smem_desc_hi(1024), idesc, kb != kb0);
         tc_commit_cta(&bars.empty[s_mma]);
         if (++s_mma == (uint32_t)a.stages) { s_mma = 0; ph_mma ^= 1; }
       }
