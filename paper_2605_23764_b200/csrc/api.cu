@@ -97,17 +97,17 @@ int encode_2d(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, u
   return encode_tiled(tm, base, 2, dims, strides, box);
 }
 
-// Store maps of the token-column tiles: un-swizzled boxes of 32 rows x `box_cols` columns.
-int encode_2d_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols) {
+// Store maps of the token-column tiles: un-swizzled boxes of box_rows x box_cols.
+int encode_2d_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
   const uint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
-  const uint32_t box[2] = {box_cols, 32};
+  const uint32_t box[2] = {box_cols, box_rows};
   return encode_tiled(tm, base, 2, dims, strides, box, false);
 }
 // [rows][2][F] view of a [rows][2F] matrix (gate half, up half): a column tile that ends past F is clipped instead of
 // spilling into the other half.
-int encode_halves_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t F, uint32_t box_cols) {
+int encode_halves_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t F, uint32_t box_cols, uint32_t box_rows) {
   const uint64_t dims[3] = {F, 2, rows}, strides[2] = {F * 2, 2 * F * 2};
-  const uint32_t box[3] = {box_cols, 1, 32};
+  const uint32_t box[3] = {box_cols, 1, box_rows};
   return encode_tiled(tm, base, 3, dims, strides, box, false);
 }
 // Load map of W_gate_up viewed as [Ep][F/8 groups][gate | up][8 rows][d]: one box brings, for eight groups of 8
@@ -761,10 +761,10 @@ int moe_create(moe_ctx** out, const moe_shape* shape, void* workspace, size_t wo
     if (!rc && train) rc = encode_2d(&c->tk_dOutp[i], c->ws + p.dOutp, cap, s.d, br, 64);
     if (!rc && train) rc = encode_2d(&c->tk_dH[i], c->ws + p.dH, cap, 2 * s.F, br, 64);
   }
-  if (!rc) rc = encode_2d_plain(&c->tp_A, c->ws + p.A, cap, s.F, 16);
-  if (!rc) rc = encode_2d_plain(&c->tp_Y, c->ws + p.Y, cap, s.d, 32);
-  if (!rc && train) rc = encode_halves_plain(&c->tp_H, c->ws + p.H, cap, s.F, 16);
-  if (!rc && train) rc = encode_halves_plain(&c->tp_dH, c->ws + p.dH, cap, s.F, 32);
+  if (!rc) rc = encode_2d_plain(&c->tp_A, c->ws + p.A, cap, s.F, 16, 32);
+  if (!rc) rc = encode_2d_plain(&c->tp_Y, c->ws + p.Y, cap, s.d, 32, 16);
+  if (!rc && train) rc = encode_halves_plain(&c->tp_H, c->ws + p.H, cap, s.F, 16, 32);
+  if (!rc && train) rc = encode_halves_plain(&c->tp_dH, c->ws + p.dH, cap, s.F, 32, 16);
   if (rc) {
     if (c->owns_ws) cudaFree(c->ws);
     delete c;

@@ -3,11 +3,11 @@
 // One cooperative grid of one CTA per SM in clusters of two runs the whole operator chain.  Per CTA:
 //   warp 0      TMA producer of the weights (weight gradients: of the A operand)
 //   warp 1      tcgen05.mma issuer (even CTA) and TMEM owner
-//   warps 2-5   epilogue: TMEM -> fused element-wise math -> TMA store, then the tile's trigger event
+//   warps 2-5, 8-11  epilogue: TMEM -> fused element-wise math -> TMA store, then the tile's trigger event
 //   warp 6      TMA producer of the tokens (weight gradients: of the B operand)
 //   warp 7      even CTA: scheduler of the pair -- takes the next ticket of the matrix queue, waits for
 //               the item's dependent events, publishes it to the other roles; odd CTA: vector worker
-//   warps 8-14  vector workers: tickets of the vector queue (permute-gather, routing-weight
+//   warps 12-15 vector workers: tickets of the vector queue (permute-gather, routing-weight
 //               gradient, combine); the matrix-role warps join them once the matrix queue is empty.
 // The matrix roles are the ones of the one-launch-per-operator kernels (gemm_roles.cuh); here they
 // take the items of all operators of the pass from one ticket queue (schedule.h) with the pipeline
@@ -21,10 +21,9 @@
 
 namespace moe {
 
-constexpr int ROLE_WARPS = 7;
 constexpr int SCHED_WARP = 7;   // even CTA: scheduler of the pair; odd CTA: a vector worker
-constexpr int VEC_WARPS = 8;
-constexpr int FUSED_THREADS = 32 * (ROLE_WARPS + VEC_WARPS);
+constexpr int VEC_WARPS = 4;
+constexpr int FUSED_THREADS = 32 * (GEMM_ROLE_WARPS + VEC_WARPS);
 
 constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
 constexpr size_t FUSED_LAYOUT_BYTES =
@@ -268,7 +267,7 @@ struct __align__(16) TicketRing {
   uint64_t full[TK_RING];    // in each CTA: the slot holds an item
   uint64_t empty[TK_RING];   // used in the even CTA: every consumer of both CTAs has read the slot
 };
-// consumers: in each CTA both loaders and the 4 epilogue warps, plus the MMA issuer of the even CTA
+// consumers: in each CTA both loaders and the epilogue warps, plus the MMA issuer of the even CTA
 constexpr int TK_CONSUMERS = 2 * (2 + EPI_WARPS) + 1;
 
 __device__ __forceinline__ void ring_publish(TicketRing* r, uint32_t n, const WorkDesc& wd) {   // one lane; the slot is free
@@ -426,20 +425,20 @@ __device__ __forceinline__ bool issue_item(const FusedArgs& fa, const WorkDesc& 
 }
 template <bool BWD>
 __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
-                                              uint32_t tmem_base, EpiState& es, int rank, int quad, int lane,
+                                              uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                               const WaitCtl& wc, const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
   if (BWD && (phase == 1 || phase == 3))
-    return wgrad_epilogue_strip(fa.op[phase], smem, bars, tmem_base, es, rank, quad, lane, desc_strip(wd), t, wc, dep);
+    return wgrad_epilogue_strip(fa.op[phase], smem, bars, tmem_base, es, rank, ew, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
     if (phase == 0)
-      return swap_epilogue_item<GEMM_GATE_UP>(fa.op[0], smem, bars, tmem_base, es, rank, quad, lane, wk, t, wc, dep);
-    return swap_epilogue_item<GEMM_DOWN>(fa.op[1], smem, bars, tmem_base, es, rank, quad, lane, wk, t, wc, dep);
+      return swap_epilogue_item<GEMM_GATE_UP>(fa.op[0], smem, bars, tmem_base, es, rank, ew, lane, wk, t, wc, dep);
+    return swap_epilogue_item<GEMM_DOWN>(fa.op[1], smem, bars, tmem_base, es, rank, ew, lane, wk, t, wc, dep);
   }
   if (phase == 0)
-    return swap_epilogue_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, tmem_base, es, rank, quad, lane, wk, t, wc, dep);
-  return swap_epilogue_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, tmem_base, es, rank, quad, lane, wk, t, wc, dep);
+    return swap_epilogue_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, tmem_base, es, rank, ew, lane, wk, t, wc, dep);
+  return swap_epilogue_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, tmem_base, es, rank, ew, lane, wk, t, wc, dep);
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -513,7 +512,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         if (tr.buf) dep.trace(TR_SCHED, wd.item, t0, td, globaltimer_ns());
       }
     }
-  } else if (warp < ROLE_WARPS && !(warp == 1 && rank != 0)) {
+  } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
     LoaderState ls;
     IssuerState is;
@@ -534,9 +533,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         if (warp != 1) {
           int go = 1;
           if (lane == 0) {
-            if (warp >= 2 && warp < 2 + EPI_WARPS) {
+            if (is_epilogue_warp(warp)) {
               tma_store_wait_all();
-              epi_enter_phase(bars, warp & 3, phase);
+              epi_enter_phase(bars, epilogue_index(warp), phase);
             }
             go = phase_wait(bars, phase, wc) ? 1 : 0;
           }
@@ -549,11 +548,11 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       else if (warp == 1)
         ok = issue_item<BWD>(fa, wd, smem, bars, tmem_base, is, wc, dep);
       else
-        ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, warp & 3, lane, wc, dep);
+        ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, wc, dep);
     }
-    if (warp >= 2 && warp < 2 + EPI_WARPS && lane == 0) {
+    if (is_epilogue_warp(warp) && lane == 0) {
       tma_store_wait_all();
-      epi_enter_phase(bars, warp & 3, SCHED_MAX_SEG);   // nothing of this warp is left in shared memory
+      epi_enter_phase(bars, epilogue_index(warp), SCHED_MAX_SEG);   // nothing of this warp is left in shared memory
     }
     if (warp == 1 && uniform(!ok || *reinterpret_cast<volatile int*>(&fa.status->abort) ? 1 : 0)) issuer_drain(bars, fa.status);
   }
@@ -562,7 +561,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   // matrix-role warps once the matrix queue is empty (the tail of the vector queue -- combine -- runs on the
   // whole SM)
   __syncwarp();
-  vector_worker_loop(fa, wc, tr, M, lane, warp > SCHED_WARP && warp <= SCHED_WARP + BACKGROUND_GATHERERS);
+  vector_worker_loop(fa, wc, tr, M, lane, warp >= GEMM_ROLE_WARPS && warp < GEMM_ROLE_WARPS + BACKGROUND_GATHERERS);
 
   // ---------------------------------------------------------------- teardown
   if (*reinterpret_cast<volatile int*>(&fa.status->abort)) __nanosleep(200000);

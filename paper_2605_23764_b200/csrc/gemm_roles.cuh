@@ -20,12 +20,18 @@ constexpr int PIPE_STAGES = 5;   // row-space operators: operand stages of 16 KB
 constexpr int WG_B_STAGES = 7;   // weight gradients: 16 KB stages of the streamed B operand
 constexpr int MAX_STAGES = 8;
 
+// Warps of a GEMM CTA: 0 weight loader, 1 MMA issuer, 2-5 and 8-11 epilogue, 6 token loader, 7 left to the kernel (scheduler).
+// TMEM lanes 32 (w % 4) .. are what warp w can read.
+constexpr int GEMM_ROLE_WARPS = 12;
+__device__ __forceinline__ bool is_epilogue_warp(int warp) { return (warp >= 2 && warp < 6) || (warp >= 8 && warp < 12); }
+__device__ __forceinline__ int epilogue_index(int warp) { return (warp & 3) + (warp >= 8 ? 4 : 0); }
+
 struct __align__(8) PipeBarriers {
   uint64_t full[MAX_STAGES];      // used in the even CTA: bytes of both CTAs' loads of the stage
   uint64_t empty[MAX_STAGES];     // in each CTA: the stage's MMAs are complete
   uint64_t a_empty[PIPE_STAGES];  // weight gradients, in each CTA: every MMA that reads the A slot's content is complete
   uint64_t tmem_full[2];          // in each CTA: accumulator ready
-  uint64_t tmem_empty[2];         // used in the even CTA: the 8 epilogue warps of the pair have drained it
+  uint64_t tmem_empty[2];         // used in the even CTA: the epilogue warps of the pair have drained it
   uint64_t drain;
   uint32_t tmem_base;
   int epi_phase[EPI_WARPS];       // in each CTA: the phase each epilogue warp is in (its stores of earlier phases have read shared memory)
@@ -56,14 +62,20 @@ __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
 // per operator, so the roles that write it -- loaders, and epilogue warps (staging) -- enter phase p only when
 // every epilogue warp of their CTA has: all MMAs of earlier phases are then complete and every store has read
 // its staging slot.  A word per warp rather than an mbarrier: a pair may pass several phases at once.
-__device__ __forceinline__ void epi_enter_phase(PipeBarriers* bars, int quad, int phase) {   // one lane
+__device__ __forceinline__ void epi_enter_phase(PipeBarriers* bars, int ew, int phase) {   // one lane
   __threadfence_block();
-  *reinterpret_cast<volatile int*>(&bars->epi_phase[quad]) = phase;
+  *reinterpret_cast<volatile int*>(&bars->epi_phase[ew]) = phase;
 }
 __device__ __forceinline__ bool phase_wait(PipeBarriers* bars, int phase, const WaitCtl& wc) {   // one lane
   volatile int* c = bars->epi_phase;
   uint64_t t0 = 0;
-  for (uint32_t spin = 1; c[0] < phase || c[1] < phase || c[2] < phase || c[3] < phase; ++spin) {
+  auto behind = [&]() {
+    int least = phase;
+#pragma unroll
+    for (int w = 0; w < EPI_WARPS; ++w) least = min(least, c[w]);
+    return least < phase;
+  };
+  for (uint32_t spin = 1; behind(); ++spin) {
     __nanosleep(100);
     if ((spin & 63u) == 0) {
       if (*reinterpret_cast<volatile int*>(&wc.status->abort)) return false;
@@ -142,13 +154,11 @@ struct ChainDeps {
 // =====================================================================================================
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
-template <int MODE>
-__host__ __device__ constexpr int swap_staging_slot_bytes() { return swap_merges<MODE>() ? SW_SLOT_BYTES / 2 : SW_SLOT_BYTES; }
 // shared memory of a phase, from the 1024-byte aligned base: weights | tokens | staging | act_grad scratch
 template <int MODE>
 __host__ __device__ constexpr size_t swap_layout_bytes() {
-  return (size_t)PIPE_STAGES * (W_STAGE_BYTES + tok_stage_bytes<MODE>()) + 4 * SW_SLOTS * swap_staging_slot_bytes<MODE>() +
-         (MODE == GEMM_ACT_GRAD ? 4 * SW_SCRATCH_BYTES : 0);
+  return (size_t)PIPE_STAGES * (W_STAGE_BYTES + tok_stage_bytes<MODE>()) + EPI_WARPS * sw_slots<MODE>() * sw_slot_bytes<MODE>() +
+         (MODE == GEMM_ACT_GRAD ? EPI_WARPS * SW_SCRATCH_BYTES : 0);
 }
 
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
@@ -230,21 +240,20 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem
 // through TMA (fence.proxy.async) and released at GPU scope.
 template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
-                                                   uint32_t tmem_base, EpiState& es, int rank, int quad, int lane,
+                                                   uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                    const SwapWork& wk, int t, const WaitCtl& wc, const DEP& dep) {
-  constexpr int SLOTB = swap_staging_slot_bytes<MODE>();
+  constexpr int WARPB = sw_slots<MODE>() * sw_slot_bytes<MODE>();
   uint8_t* sOut = smem + PIPE_STAGES * (W_STAGE_BYTES + tok_stage_bytes<MODE>());
-  uint8_t* sScr = sOut + 4 * SW_SLOTS * SLOTB;   // act_grad: per epilogue warp 4 KB for the saved pre-activations
-  SwStaging sg{sOut + quad * SW_SLOTS * SLOTB, es.round, sScr + quad * SW_SCRATCH_BYTES, SW_SLOTS, (uint32_t)SLOTB};
+  SwStaging sg{sOut + ew * WARPB, es.round, sOut + EPI_WARPS * WARPB + ew * SW_SCRATCH_BYTES};
   bool ok = true;
   for (int part = 0; part < (wk.merged ? 2 : 1); ++part) {   // a merged item is two consecutive tiles here
     const SwapTile& st = part ? wk.b : wk.a;
     const int as = es.acc_it & 1;
     if (!mbar_wait(&bars->tmem_full[as], (es.acc_it >> 1) & 1, wc, SITE_TMEM_FULL, t, 200)) { ok = false; break; }
     uint64_t t0 = 0;
-    if (DEP::kOn && quad == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
+    if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
     tc_fence_after_sync();
-    epilogue_swap<MODE>(a, st, tmem_base + as * BN, rank, quad, lane, sg);
+    epilogue_swap<MODE>(a, st, tmem_base + as * BN, rank, ew, lane, sg);
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) mbar_arrive_leader(&bars->tmem_empty[as]);
@@ -254,7 +263,7 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
         tma_store_wait_all();
         fence_proxy_async();
         dep.signal(st.mb_first, st.mb_count);
-        if (quad == 0 && dep.tracing()) dep.trace(TR_EPI, t, t0, t0, globaltimer_ns());
+        if (ew == 0 && dep.tracing()) dep.trace(TR_EPI, t, t0, t0, globaltimer_ns());
       }
       __syncwarp();
     }
@@ -276,21 +285,21 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
 //
 // With K of only four or five k-blocks a column tile lasts about as long as the latency of its B loads, so the
 // B ring is deeper than one tile (WG_B_STAGES): the loads of tile i + 1 are in flight while tile i multiplies.
-// The staging of the epilogue is what pays for it: one 4 KB box of 32 rows x 64 columns at a time, two per warp.
+// The staging of the epilogue is what pays for it: one 4 KB box of 32 rows x 64 columns per warp.
 constexpr int A_RES_KB = PIPE_STAGES;        // k-blocks of A that can stay resident
-constexpr int WG_OUT_SLOTS = 2;              // staging boxes per epilogue warp
 constexpr size_t WGRAD_LAYOUT_BYTES =
-    (size_t)PIPE_STAGES * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES + 4 * WG_OUT_SLOTS * OUT_BOX_BYTES;
+    (size_t)PIPE_STAGES * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES + EPI_WARPS * OUT_BOX_BYTES;
 
-// Epilogue of one 128 x 256 accumulator slice of a weight gradient (or zeros for an expert without rows): warp
-// `quad` stores its 32 rows, 64 columns per staging box.
-__device__ __forceinline__ void epilogue_wgrad_tile(const GemmArgs& a, const Tile& tl, uint32_t tmem_acc, int quad, int lane,
-                                                    uint8_t* slots, uint32_t& round) {
+// Epilogue of one 128 x 256 accumulator slice of a weight gradient (or zeros for an expert without rows): warps `quad`
+// and `quad + 4` store 32 rows, 64 columns at a time in turn, each through a staging box of its own.
+__device__ __forceinline__ void epilogue_wgrad_tile(const GemmArgs& a, const Tile& tl, uint32_t tmem_acc, int ew, int lane,
+                                                    uint8_t* box) {
+  const int quad = ew & 3;
   const uint32_t trow = tmem_acc + (static_cast<uint32_t>(quad * 32) << 16);
   const int y0 = tl.m0 + quad * 32;
   if (y0 >= a.M) return;
 #pragma unroll 1
-  for (int c0 = 0; c0 < BN; c0 += 64) {
+  for (int c0 = (ew >> 2) * 64; c0 < BN; c0 += 128) {
     if (tl.n0 + c0 >= a.N) break;
     float v[64];
     if (tl.nkb == 0) {
@@ -302,10 +311,8 @@ __device__ __forceinline__ void epilogue_wgrad_tile(const GemmArgs& a, const Til
       for (int q = 0; q < 4; ++q) tmem_ld16(trow + c0 + 16 * q, v + 16 * q);
       tmem_ld_wait();
     }
-    if (lane == 0) tma_store_wait_read_n<WG_OUT_SLOTS - 1>();   // the box's previous store has read it
+    if (lane == 0) tma_store_wait_read();   // the box's previous store has read it
     __syncwarp();
-    uint8_t* box = slots + (round % WG_OUT_SLOTS) * OUT_BOX_BYTES;
-    ++round;
 #pragma unroll
     for (int h = 0; h < 64; h += 8) stage8(box, lane, h >> 3, v + h);
     staging_release();
@@ -420,31 +427,31 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
 
 template <class DEP>
 __device__ __forceinline__ bool wgrad_epilogue_strip(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
-                                                     uint32_t tmem_base, EpiState& es, int rank, int quad, int lane,
+                                                     uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                      const Strip& st, int sp, const WaitCtl& wc, const DEP& dep) {
-  uint8_t* slots = smem + PIPE_STAGES * A_STAGE_BYTES + WG_B_STAGES * HALF_B_BYTES + quad * WG_OUT_SLOTS * OUT_BOX_BYTES;
+  uint8_t* box = smem + PIPE_STAGES * A_STAGE_BYTES + WG_B_STAGES * HALF_B_BYTES + ew * OUT_BOX_BYTES;
   Tile tl;
   tl.e = st.e; tl.row0 = st.row0; tl.m0 = st.m0(rank); tl.nkb = st.nkb;
   const bool idle = tl.m0 >= a.M;   // the strip's second half lies outside dW: nothing to store
   bool ok = true;
   uint64_t t0 = 0;
-  if (DEP::kOn && quad == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
+  if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
   for (int nb = 0; nb < a.n_tiles_n; ++nb) {
     tl.nb = nb; tl.n0 = nb * BN;
     if (st.nkb == 0) {
-      if (!idle) epilogue_wgrad_tile(a, tl, 0, quad, lane, slots, es.round);  // an expert without rows: zeros
+      if (!idle) epilogue_wgrad_tile(a, tl, 0, ew, lane, box);  // an expert without rows: zeros
       continue;
     }
     const int as = es.acc_it & 1;
     if (!mbar_wait(&bars->tmem_full[as], (es.acc_it >> 1) & 1, wc, SITE_TMEM_FULL, sp, 200)) { ok = false; break; }
     tc_fence_after_sync();
-    if (!idle) epilogue_wgrad_tile(a, tl, tmem_base + as * BN, quad, lane, slots, es.round);
+    if (!idle) epilogue_wgrad_tile(a, tl, tmem_base + as * BN, ew, lane, box);
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) mbar_arrive_leader(&bars->tmem_empty[as]);
     ++es.acc_it;
   }
-  if (DEP::kOn && quad == 0 && lane == 0 && dep.tracing()) dep.trace(TR_EPI, sp, t0, t0, globaltimer_ns());
+  if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) dep.trace(TR_EPI, sp, t0, t0, globaltimer_ns());
   return ok;
 }
 

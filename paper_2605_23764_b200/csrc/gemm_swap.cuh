@@ -16,11 +16,6 @@ namespace moe {
 
 constexpr int TOK_GRAIN = 32;                    // tokens per tile: a multiple of 32 (16 rows of B per CTA)
 constexpr int W_STAGE_BYTES = A_STAGE_BYTES;     // 128 weight rows (or 2 MN-major boxes) x 64 k: 16 KB
-constexpr int SW_SLOT_BYTES = 4096;              // one staging slot of an epilogue warp
-#ifndef MOE_SW_SLOTS
-#define MOE_SW_SLOTS 2
-#endif
-constexpr int SW_SLOTS = MOE_SW_SLOTS;           // ring of slots per warp
 
 struct SwapTile {
   int e;      // expert
@@ -141,22 +136,26 @@ __device__ __forceinline__ uint32_t swap_idesc(int ntok) {
 }
 
 // ---------------------------------------------------------------- staging ring of an epilogue warp
+// Tokens per staging slot, bytes of a slot, slots per warp.  gate+up: A, H gate, H up of 16 features each; act_grad: d(gate) and
+// d(up) of 32 features; down, gate_grad: 32 features.  What is left of the 227 KB beside the operand ring decides.
+template <int MODE>
+__host__ __device__ constexpr int sw_chunk() { return MODE == GEMM_GATE_UP ? 32 : 16; }
+template <int MODE>
+__host__ __device__ constexpr int sw_slot_bytes() { return MODE == GEMM_GATE_UP ? 3072 : MODE == GEMM_ACT_GRAD ? 2048 : 1024; }
+template <int MODE>
+__host__ __device__ constexpr int sw_slots() { return MODE == GEMM_DOWN || MODE == GEMM_GATE_GRAD ? 3 : 2; }
+constexpr int SW_SCRATCH_BYTES = 4096;   // act_grad, per warp: saved pre-activations, two halves of [gate | up][16 tokens][32 features]
 struct SwStaging {
-  uint8_t* base;     // SW_SLOTS slots of SW_SLOT_BYTES
+  uint8_t* base;     // this warp's slots
   uint32_t round;
-  uint8_t* scratch;  // act_grad: 4 KB of this warp (two halves of [gate | up][16 tokens][32 features])
-  uint32_t slots;       // staging slots of this warp (1 or 2)
-  uint32_t slot_bytes;  // SW_SLOT_BYTES, or 2 KB in the plain-store operators that give room to the operand stages
+  uint8_t* scratch;  // act_grad
 };
-constexpr int SW_SCRATCH_BYTES = 4096;
+template <int MODE>
 __device__ __forceinline__ uint8_t* sw_acquire(SwStaging& sg, int lane) {
-  if (lane == 0) {   // the slot's previous stores have read it
-    if (sg.slots == 1) tma_store_wait_read();
-    else tma_store_wait_read_n<SW_SLOTS - 1>();
-  }
+  if (lane == 0) tma_store_wait_read_n<sw_slots<MODE>() - 1>();   // the slot's previous stores have read it
   __syncwarp();
-  uint8_t* slot = sg.base + (sg.round % sg.slots) * sg.slot_bytes;
-  ++sg.round;
+  uint8_t* slot = sg.base + sg.round * sw_slot_bytes<MODE>();
+  if (++sg.round == sw_slots<MODE>()) sg.round = 0;
   return slot;
 }
 __device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
@@ -169,30 +168,33 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint16_t* p) {
 
 
 // ---------------------------------------------------------------- epilogues (transposed accumulator)
-// Warp `quad` of CTA `rank` owns TMEM lanes 32*quad .. 32*quad+31 (32 output features) and walks the
-// tile's tokens 32 columns at a time.  A thread (= one feature) writes one bf16 per token into a
-// staging box laid out [token][feature]; lane 0 stores the box with TMA (clipped at the tensor edge).
+// Warps `quad` and `quad + 4` of CTA `rank` own TMEM lanes 32*quad .. 32*quad+31 (32 output features) and walk the tile's
+// tokens in alternating chunks.  A thread (= one feature) writes one bf16 per token into a staging box laid out
+// [token][feature]; lane 0 stores the box with TMA (clipped at the tensor edge).  With one warp per quarter the epilogue of
+// a 256-token tile took 11-16 us, as long as the MMAs of 32-64 k-blocks: latency, two warps hide each other's.
 template <int MODE>
 __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile& st, uint32_t tmem_acc, int rank,
-                                              int quad, int lane, SwStaging& sg) {
+                                              int ew, int lane, SwStaging& sg) {
+  const int quad = ew & 3;
+  constexpr int CH = sw_chunk<MODE>();
+  const int first = (ew >> 2) * CH;
   const uint32_t trow = tmem_acc + (static_cast<uint32_t>(quad * 32) << 16);
   if (MODE == GEMM_DOWN || MODE == GEMM_GATE_GRAD) {
     const int f0 = st.n0 + rank * 128 + quad * 32;   // first output column of this warp
     if (f0 >= a.N) return;
 #pragma unroll 1
-    for (int c0 = 0; c0 < st.ntok; c0 += 32) {
-      float v[32];
+    for (int c0 = first; c0 < st.ntok; c0 += 2 * CH) {
+      float v[16];
       tmem_ld16(trow + c0, v);
-      tmem_ld16(trow + c0 + 16, v + 16);
       tmem_ld_wait();
-      uint8_t* box = sw_acquire(sg, lane);
-      // [32 tokens][32 features].  Neighbouring lanes (features 2i, 2i+1) swap one value per token pair, so that
+      uint8_t* box = sw_acquire<MODE>(sg, lane);
+      // [16 tokens][32 features].  Neighbouring lanes (features 2i, 2i+1) swap one value per token pair, so that
       // every lane stores 4 bytes: the even lane the feature pair of token j, the odd lane that of token j+1 -- 128
       // contiguous bytes per warp store instead of 64.
       uint32_t* box32 = reinterpret_cast<uint32_t*>(box) + (lane >> 1);
       const bool odd = lane & 1;
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
+      for (int j = 0; j < CH; j += 2) {
         const float send = odd ? v[j] : v[j + 1];
         const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
         box32[(j + (odd ? 1 : 0)) * 16] = odd ? pack_bf16x2(recv, v[j + 1]) : pack_bf16x2(v[j], recv);
@@ -211,18 +213,20 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
     const bool hi = (lane & 8) != 0;
     const int fw0 = st.n0 + rank * 64 + quad * 16;   // first feature of this warp
     if (fw0 >= a.F) return;
+    float w_next = first < st.ntok ? a.prow_w[st.row0 + first + lane] : 0.f;
 #pragma unroll 1
-    for (int c0 = 0; c0 < st.ntok; c0 += 32) {
+    for (int c0 = first; c0 < st.ntok; c0 += 2 * CH) {
       float v[32];
       tmem_ld16(trow + c0, v);
       tmem_ld16(trow + c0 + 16, v + 16);
-      const float wl = a.prow_w[st.row0 + c0 + lane];   // routing weight of token c0 + lane
+      const float wl = w_next;   // routing weight of token c0 + lane; the next chunk's is on its way
+      if (c0 + 2 * CH < st.ntok) w_next = a.prow_w[st.row0 + c0 + 2 * CH + lane];
       tmem_ld_wait();
-      uint8_t* box = sw_acquire(sg, lane);
+      uint8_t* box = sw_acquire<MODE>(sg, lane);
       uint16_t* abox = reinterpret_cast<uint16_t*>(box);           // A: [32 tokens][16 features]
       uint16_t* hbox = reinterpret_cast<uint16_t*>(box + 1024 + (hi ? 1024 : 0));   // H gate / H up
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
+      for (int j = 0; j < CH; j += 2) {
         const float send = hi ? v[j] : v[j + 1];
         const float recv = __shfl_xor_sync(0xffffffffu, send, 8);
         const float g = hi ? recv : v[j];
@@ -233,7 +237,7 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
       }
       if (a.save_h) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) hbox[j * 16 + fl] = bf16_bits(v[j]);
+        for (int j = 0; j < CH; ++j) hbox[j * 16 + fl] = bf16_bits(v[j]);
       }
       staging_release();
       if (lane == 0) {
@@ -252,7 +256,7 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
     if (f0 >= a.F) {
       // no features here: the partial slots of this warp still take part in the reduction
       if (a.dw_partial)
-        for (int j = lane; j < st.ntok; j += 32) a.dw_partial[(size_t)(st.row0 + j) * nparts + slot] = 0.f;
+        for (int j = lane + 32 * (ew >> 2); j < st.ntok; j += 64) a.dw_partial[(size_t)(st.row0 + j) * nparts + slot] = 0.f;
       return;
     }
     // The saved pre-activations of 16 tokens x 32 features (gate and up: 1 KB each) come in as four
@@ -272,30 +276,32 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
         pre[2 * i + 1] = cvalid ? ld_nc_v4(p + a.F) : make_uint4(0, 0, 0, 0);
       }
     };
-    fetch(0);
-    uint8_t* box = nullptr;
-    float wl = 0.f;
+    if (first >= st.ntok) return;
+    fetch(first);
+    float w_next = a.prow_w[st.row0 + first + (lane & 15)];
+    int half = 0;
 #pragma unroll 1
-    for (int h0 = 0; h0 < st.ntok; h0 += 16) {
-      const int hh = h0 & 16;   // which half of the 32-token staging box
-      if (hh == 0) {
-        box = sw_acquire(sg, lane);
-        wl = a.prow_w[st.row0 + h0 + lane];
-      }
-      uint8_t* scr = sg.scratch + (((h0 >> 4) & 1) ? 2048 : 0);
+    for (int h0 = first; h0 < st.ntok; h0 += 2 * CH) {
+      uint8_t* box = sw_acquire<MODE>(sg, lane);
+      const float wl = w_next;
+      uint8_t* scr = sg.scratch + half;
+      half ^= 2048;
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int t = (lane + 32 * i) >> 2;
         *reinterpret_cast<uint4*>(scr + t * 64 + part * 16) = pre[2 * i];
         *reinterpret_cast<uint4*>(scr + 1024 + t * 64 + part * 16) = pre[2 * i + 1];
       }
-      if (h0 + 16 < st.ntok) fetch(h0 + 16);
+      if (h0 + 2 * CH < st.ntok) {
+        fetch(h0 + 2 * CH);
+        w_next = a.prow_w[st.row0 + h0 + 2 * CH + (lane & 15)];
+      }
       float da[16], pr[16];
       tmem_ld16(trow + h0, da);
       __syncwarp();
       tmem_ld_wait();
-      uint16_t* gbox = reinterpret_cast<uint16_t*>(box) + lane;          // d(gate): [32 tokens][32 features]
-      uint16_t* ubox = reinterpret_cast<uint16_t*>(box + 2048) + lane;   // d(up)
+      uint16_t* gbox = reinterpret_cast<uint16_t*>(box) + lane;          // d(gate): [16 tokens][32 features]
+      uint16_t* ubox = reinterpret_cast<uint16_t*>(box + 1024) + lane;   // d(up)
       const uint16_t* gs16 = reinterpret_cast<const uint16_t*>(scr) + lane;
       const uint16_t* us16 = reinterpret_cast<const uint16_t*>(scr + 1024) + lane;
 #pragma unroll
@@ -304,10 +310,10 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
         const float s = sigmoidf_fast(g);
         const float gs = g * s;
         pr[j] = da[j] * (gs * u);                   // <dA_unweighted, a>: gradient of the routing weight
-        const float w = __shfl_sync(0xffffffffu, wl, hh + j);
+        const float w = __shfl_sync(0xffffffffu, wl, j);
         const float dav = w * da[j];                // backward Dispatch's weight, applied here
-        gbox[(hh + j) * 32] = bf16_bits(dav * u * (s * (1.0f + g * (1.0f - s))));
-        ubox[(hh + j) * 32] = bf16_bits(dav * gs);
+        gbox[j * 32] = bf16_bits(dav * u * (s * (1.0f + g * (1.0f - s))));
+        ubox[j * 32] = bf16_bits(dav * gs);
       }
       if (a.dw_partial) {
         // sum over the warp's 32 features: a transposing butterfly leaves token (lane >> 1) in each lane
@@ -324,15 +330,11 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
         pr[0] += __shfl_xor_sync(0xffffffffu, pr[0], 1);
         if ((lane & 1) == 0) a.dw_partial[(size_t)(st.row0 + h0 + (lane >> 1)) * nparts + slot] = pr[0];
       }
-      if (hh == 16) {
-        staging_release();
-        if (lane == 0) {
-          tma_store_3d(&a.tmOut0, f0, 0, st.row0 + h0 - 16, box);
-          tma_store_3d(&a.tmOut0, f0, 1, st.row0 + h0 - 16, box + 2048);
-          tma_store_commit();
-        }
-      } else {
-        __syncwarp();   // the scratch half written two rounds from now is the one just read
+      staging_release();   // (also: the scratch half written two rounds from now is the one just read)
+      if (lane == 0) {
+        tma_store_3d(&a.tmOut0, f0, 0, st.row0 + h0, box);
+        tma_store_3d(&a.tmOut0, f0, 1, st.row0 + h0, box + 1024);
+        tma_store_commit();
       }
     }
   }

@@ -4,7 +4,7 @@
 // Section 5.2).
 //
 // Roles per CTA: warp 0 TMA producer of the weights, warp 1 MMA issuer (even CTA) and TMEM owner,
-// warps 2..5 epilogue, warp 6 TMA producer of the tokens.
+// warps 2-5 and 8-11 epilogue, warp 6 TMA producer of the tokens.
 #include "gemm_roles.cuh"
 #include "launch_pairs.cuh"
 
@@ -16,7 +16,7 @@ static_assert(gemm3_smem_bytes<GEMM_GATE_UP>() <= 227 * 1024 && gemm3_smem_bytes
                   gemm3_smem_bytes<GEMM_ACT_GRAD>() <= 227 * 1024 && gemm3_smem_bytes<GEMM_GATE_GRAD>() <= 227 * 1024,
               "shared memory budget");
 
-constexpr int GEMM3_THREADS = 224;
+constexpr int GEMM3_THREADS = 32 * GEMM_ROLE_WARPS;
 
 template <int MODE>
 __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(const __grid_constant__ GemmArgs a) {
@@ -69,11 +69,11 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       }
       if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
-  } else {
+  } else if (is_epilogue_warp(warp)) {
     EpiState es;
     for (int t = pair; t < total; t += npairs, cur = next) {
       if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-      if (!swap_epilogue_item<MODE>(a, smem, bars, tmem_base, es, rank, warp & 3, lane, cur, t, wc, dep)) break;
+      if (!swap_epilogue_item<MODE>(a, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, cur, t, wc, dep)) break;
     }
     if (lane == 0) tma_store_wait_all();
   }

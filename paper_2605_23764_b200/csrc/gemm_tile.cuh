@@ -15,7 +15,6 @@ constexpr int BK = 64;                        // reduction elements per stage (o
 constexpr int A_STAGE_BYTES = BLOCK_M * BK * 2;  // 16 KB
 constexpr int B_STAGE_BYTES = BN * BK * 2;       // 32 KB
 constexpr int MN_BOX_BYTES = 64 * BK * 2;        // one [64 k][64 mn] box of an MN-major operand
-constexpr int GEMM_THREADS = 192;
 constexpr int TMEM_COLS = 512;
 constexpr int OUT_BOX_BYTES = 32 * 64 * 2;       // epilogue staging box: 32 rows x 64 bf16 columns
 

@@ -1,13 +1,13 @@
 // Weight gradients on CTA pairs, strip by strip (gemm_roles.cuh), one launch per operator.
 //
 // Roles per CTA: warp 0 TMA producer of A (and the stage's byte count), warp 6 TMA producer of B,
-// warp 1 MMA issuer (even CTA) and TMEM owner, warps 2..5 epilogue.
+// warp 1 MMA issuer (even CTA) and TMEM owner, warps 2-5 and 8-11 epilogue.
 #include "gemm_roles.cuh"
 #include "launch_pairs.cuh"
 
 namespace moe {
 
-constexpr int WG_THREADS = GEMM_THREADS + 32;
+constexpr int WG_THREADS = 32 * GEMM_ROLE_WARPS;
 constexpr size_t WGRAD_SMEM_BYTES = 1024 + WGRAD_LAYOUT_BYTES + sizeof(PipeBarriers);
 static_assert(WGRAD_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
@@ -60,11 +60,11 @@ __global__ void __launch_bounds__(WG_THREADS, 1) grouped_wgrad_pair_kernel(const
       }
       if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
-  } else {
+  } else if (is_epilogue_warp(warp)) {
     EpiState es;
     for (int sp = pair; sp < total; sp += npairs, cur = next) {
       if (sp + npairs < total) next = decode_strip(a, sp + npairs);
-      if (!wgrad_epilogue_strip(a, smem, bars, tmem_base, es, rank, warp & 3, lane, cur, sp, wc, dep)) break;
+      if (!wgrad_epilogue_strip(a, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, cur, sp, wc, dep)) break;
     }
     if (lane == 0) tma_store_wait_all();
   }

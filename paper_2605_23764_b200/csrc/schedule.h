@@ -43,7 +43,7 @@ namespace moe {
 constexpr int SCHED_MAX_SEG = 4;       // phases of a pass
 constexpr int GATHER_SUB = 32;         // vector sub-tasks per M-block gather (4 rows each: the first M-blocks of a
                                        // launch, which every CTA pair waits for, are complete after a few microseconds)
-constexpr int EPI_WARPS = 4;           // epilogue warps per CTA
+constexpr int EPI_WARPS = 8;           // epilogue warps per CTA: two per quarter of the accumulator rows
 constexpr int SIG = 2 * EPI_WARPS;     // signals per (M-block, column tile): every epilogue warp of the pair
 constexpr int COMBINE_TOKENS = 1;      // tokens per combine task
 
