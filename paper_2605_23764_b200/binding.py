@@ -7,8 +7,10 @@ CPU tensors for the *_host calls).  The current torch stream is passed as the st
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import struct
+import threading
 
 import torch
 
@@ -163,27 +165,55 @@ def _check(rc: int, what: str):
         raise MoeError(f"{what}: {msg} ({rc})" + (f" [{extra}]" if extra and rc == -3 else ""))
 
 
-# Argument checks sit on the path of calls that take 20 us on the GPU: each tensor is looked at once (type, place, layout,
-# size) and pointers travel as plain integers, which ctypes converts by the functions' argtypes.
+# Argument checks sit on the path of calls that take 20 us on the GPU: each tensor is looked at once (size, type, place, layout)
+# and pointers travel as plain integers, which ctypes converts by the functions' argtypes.  A call reports a wrong size in
+# preference to a wrong type or place of another tensor: the first such fault makes _sizes_first look at the sizes alone.
+class _TypeFault(MoeError):
+    pass
+
+
+_sizes_only = threading.local()
+
+
+def _fault(name, kind, dtype):
+    if not getattr(_sizes_only, "on", False):
+        raise _TypeFault(f"{name}: expected a contiguous {kind} tensor of {dtype}")
+
+
 def _dev(t, dtype, name, n=0):
     """Device pointer of a tensor of at least n elements (an undersized tensor would make a kernel leave its bounds)."""
     if t is None:
         return None
-    if not (t.is_cuda and t.dtype is dtype and t.is_contiguous()):
-        raise MoeError(f"{name}: expected a contiguous CUDA tensor of {dtype}")
     if t.numel() < n:
         raise MoeError(f"{name}: {t.numel()} elements, the call needs {n}")
+    if not (t.is_cuda and t.dtype is dtype and t.is_contiguous()):
+        _fault(name, "CUDA", dtype)
     return t.data_ptr()
 
 
 def _host(t, dtype, name, n=0):
     if t is None:
         return None
-    if t.is_cuda or t.dtype is not dtype or not t.is_contiguous():
-        raise MoeError(f"{name}: expected a contiguous CPU tensor of {dtype}")
     if t.numel() < n:
         raise MoeError(f"{name}: {t.numel()} elements, the call needs {n}")
+    if t.is_cuda or t.dtype is not dtype or not t.is_contiguous():
+        _fault(name, "CPU", dtype)
     return t.data_ptr()
+
+
+def _sizes_first(fn):
+    @functools.wraps(fn)
+    def call(*args, **kwargs):
+        try:
+            return fn(*args, **kwargs)
+        except _TypeFault as fault:
+            _sizes_only.on, _sizes_only.fault = True, fault
+            try:
+                fn(*args, **kwargs)   # ends in _stream(), the last argument of every call
+            finally:
+                _sizes_only.on, _sizes_only.fault = False, None
+            raise
+    return call
 
 
 _CTX_SHAPE = {}   # context handle -> (T_max, d, E, k, n_shared, F, flags): what the size checks need
@@ -206,9 +236,13 @@ try:   # torch.cuda.current_stream() builds a Stream object (3.4 us); the calls 
     _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
     def _stream():
+        if getattr(_sizes_only, "on", False):
+            raise _sizes_only.fault
         return _raw_stream(_current_device())
 except AttributeError:
     def _stream():
+        if getattr(_sizes_only, "on", False):
+            raise _sizes_only.fault
         return torch.cuda.current_stream().cuda_stream
 
 
@@ -244,6 +278,7 @@ def moe_destroy(ctx):
     _CTX_SHAPE.pop(getattr(ctx, "value", None), None)
 
 
+@_sizes_first
 def moe_route(ctx, logits, T, topk_ids, topk_w, counts=None):
     _, _, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_route(ctx, _dev(logits, _F32, "logits", T * E), T, _dev(topk_ids, _I32, "topk_ids", T * k),
@@ -251,6 +286,7 @@ def moe_route(ctx, logits, T, topk_ids, topk_w, counts=None):
            "moe_route")
 
 
+@_sizes_first
 def moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits=None, counts=None):
     _, d, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_router_fwd(ctx, _dev(x, _BF, "x", T * d), _dev(W_r, _BF, "W_r", E * d), T,
@@ -259,6 +295,7 @@ def moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits=None, counts=None):
            "moe_router_fwd")
 
 
+@_sizes_first
 def moe_router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits):
     _, _, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_router_bwd(ctx, _dev(logits, _F32, "logits", T * E), _dev(topk_ids, _I32, "topk_ids", T * k),
@@ -266,6 +303,7 @@ def moe_router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits):
                                          _stream()), "moe_router_bwd")
 
 
+@_sizes_first
 def moe_layout(ctx, topk_ids, T, counts=None, offsets=None, row_of=None, src_of=None):
     _, _, E, k, S, _, _ = _shape_of(ctx)
     n = T * (k + S)
@@ -274,6 +312,7 @@ def moe_layout(ctx, topk_ids, T, counts=None, offsets=None, row_of=None, src_of=
                                      _dev(src_of, _I32, "src_of", n), _stream()), "moe_layout")
 
 
+@_sizes_first
 def moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T):
     _, d, E, k, S, F, _ = _shape_of(ctx)
     td, tk, nw = T * d, T * k, (E + S) * d * F
@@ -282,6 +321,7 @@ def moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T):
                                       _dev(W_down, _BF, "W_down", nw), _dev(out, _BF, "out", td), T, _stream()), "moe_ffn_fwd")
 
 
+@_sizes_first
 def moe_ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T):
     _, d, E, k, S, F, _ = _shape_of(ctx)
     td, tk, nw = T * d, T * k, (E + S) * d * F
@@ -293,6 +333,7 @@ def moe_ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_u
                                       T, _stream()), "moe_ffn_bwd")
 
 
+@_sizes_first
 def moe_ffn_fwd_host(ctx, x_host, topk_ids_host, topk_w_host, W_gate_up, W_down, out_host, T):
     _, d, E, k, S, F, _ = _shape_of(ctx)
     td, tk, nw = T * d, T * k, (E + S) * d * F
@@ -303,6 +344,7 @@ def moe_ffn_fwd_host(ctx, x_host, topk_ids_host, topk_w_host, W_gate_up, W_down,
                                            _host(out_host, _BF, "out_host", td), T, _stream()), "moe_ffn_fwd_host")
 
 
+@_sizes_first
 def moe_ffn_bwd_host(ctx, dout_host, W_gate_up, W_down, dx_host, dW_gate_up, dW_down, d_topk_w_host, T):
     _, d, E, k, S, F, _ = _shape_of(ctx)
     td, tk, nw = T * d, T * k, (E + S) * d * F
@@ -339,6 +381,7 @@ def moe_get_phase_ms(ctx) -> dict:
     return {name: float(buf[i]) for i, name in enumerate(PHASES) if buf[i] > 0.0}
 
 
+@_sizes_first
 def moe_route_host(ctx, logits_host, T, topk_ids_host, topk_w_host):
     _, _, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_route_host(ctx, _host(logits_host, _F32, "logits_host", T * E), T,
@@ -346,6 +389,7 @@ def moe_route_host(ctx, logits_host, T, topk_ids_host, topk_w_host):
                                          _host(topk_w_host, _F32, "topk_w_host", T * k), _stream()), "moe_route_host")
 
 
+@_sizes_first
 def moe_layout_noalloc(topk_ids, T, E, k, n_shared, counts, offsets, row_of, src_of, status2=None):
     """Dispatch layout through the entry point that allocates nothing and needs no context (for
     callers that may not cudaMalloc).  All tensors are caller-owned CUDA int32 tensors."""
@@ -366,6 +410,7 @@ def moe_sched_study_workspace_bytes(M, tile_rows) -> int:
     return int(load_library().moe_sched_study_workspace_bytes(int(M), int(tile_rows)))
 
 
+@_sizes_first
 def moe_sched_study(mode, x, r, s, z, M, C, tile_rows, workspace):
     """SwiGLU + Add operator pair under one of the three schedules; all tensors are CUDA tensors
     (bf16 x[M][2C], r/s/z[M][C]; workspace: any dtype, at least moe_sched_study_workspace_bytes)."""

@@ -145,7 +145,7 @@ struct Carve {
 
 // Byte offsets of every workspace tensor.
 struct WsPlan {
-  size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, pair_start, pblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, prow_w,
+  size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, pair_start, pblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, group_start, group_row, group_slot, prow_w,
       dw_partial, Xp, H, A, Y, dOutp, dH, st_x, st_dout, st_ids, st_w, st_out, st_dx, st_dw, st_logits, ctr, trace, total;
   int cap_rows, nblk_max, ntn_act, ctr_count, trace_cap;
 };
@@ -178,6 +178,9 @@ WsPlan plan_workspace(const moe_shape& s) {
   p.prow_of = c.take(sizeof(int) * (slots + 1));
   p.combine_order = c.take(sizeof(int) * ((size_t)s.T_max + 1));
   p.tok_last = c.take(sizeof(int) * ((size_t)s.T_max + 1));
+  p.group_start = c.take(sizeof(int) * (Ep + 1));
+  p.group_row = c.take(sizeof(int) * (cap / GROUP_ROWS + 1));
+  p.group_slot = c.take(sizeof(int) * cap);
   p.prow_w = c.take(sizeof(float) * cap);
   p.dw_partial = c.take(train ? sizeof(float) * cap * p.ntn_act * DW_PARTS_PER_TILE : 0);
   p.Xp = c.take(2 * cap * s.d);
@@ -275,6 +278,9 @@ struct moe_ctx {
     lv.blk_hist = at<int>(plan.blk_hist);
     lv.combine_order = at<int>(plan.combine_order);
     lv.tok_last = at<int>(plan.tok_last);
+    lv.group_start = at<int>(plan.group_start);
+    lv.group_row = at<int>(plan.group_row);
+    lv.group_slot = at<int>(plan.group_slot);
     return lv;
   }
   Dims dims(int T) const { return Dims{T, shape.d, shape.E, shape.k, shape.n_shared, shape.F}; }
@@ -447,6 +453,7 @@ ChainParams chain_params(const moe_ctx* c, bool bwd, int T, bool want_dw) {
   cp.kp = s.k + s.n_shared;
   cp.dep_extra = c->dep_extra;
   cp.want_dw = want_dw ? 1 : 0;
+  cp.combine_split = combine_split_of(T, s.d);
   if (!bwd) {
     cp.n_phases = 2;
     cp.ntn[0] = (s.F + 127) / 128;                 // gate+up: 128 features (gate and up) per pair tile
@@ -1097,6 +1104,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   ChainParams cp;
   memset(&cp, 0, sizeof cp);
   cp.is_bwd = is_bwd; cp.Ep = Ep; cp.T = T; cp.k = k; cp.kp = k + n_shared; cp.want_dw = 1;
+  cp.combine_split = combine_split_of(T, d);
   if (!is_bwd) {
     cp.n_phases = 2; cp.ntn[0] = (F + 127) / 128; cp.ntn[1] = (d + 255) / 256; cp.merges[1] = 1;
   } else {
@@ -1104,7 +1112,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     cp.ntn[2] = (d + 255) / 256; cp.merges[2] = 1; cp.ntn[3] = (d + 255) / 256; cp.strips[3] = (2 * F + 255) / 256;
   }
   // items of every phase: {first M-block, M-blocks of unit a, M-blocks of unit b} (strips: the expert's M-blocks)
-  struct Item { int phase, mb_first, mb_a, mb_b; };
+  struct Item { int phase, mb_first, mb_a, mb_b, e; };
   std::vector<std::vector<Item>> queue(pairs);
   long n_items = 0;
   std::vector<std::vector<int>> cover(cp.n_phases, std::vector<int>(M + 1, 0));
@@ -1113,7 +1121,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
       const int total = Ep * cp.strips[ph];
       for (int sidx = 0; sidx < total; ++sidx) {
         const int e = sidx / cp.strips[ph];
-        queue[sidx % pairs].push_back(Item{ph, mb_start[e], mb_start[e + 1] - mb_start[e], 0});
+        queue[sidx % pairs].push_back(Item{ph, mb_start[e], mb_start[e + 1] - mb_start[e], 0, e});
         ++n_items;
       }
     } else {
@@ -1129,7 +1137,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
             it.mb_count > 3 || it.mb_count_a < 1)
           return 10;
         for (int q = 0; q < it.mb_count; ++q) cover[ph][it.mb_first + q]++;
-        queue[tq % pairs].push_back(Item{ph, it.mb_first, it.mb_count_a, it.mb_count - it.mb_count_a});
+        queue[tq % pairs].push_back(Item{ph, it.mb_first, it.mb_count_a, it.mb_count - it.mb_count_a, it.e});
         ++n_items;
       }
     }
@@ -1142,7 +1150,14 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   // 2. execution with a bounded number of workers
   std::vector<long> ctr(ctr_ints(M + 1), 0);
   std::vector<size_t> cursor(pairs, 0);
-  const int ngather = gather_total(M), npost = post_total(cp, M);
+  // 32-row groups: first of each expert, M-block of each
+  std::vector<int> group_start(Ep + 1, 0), group_mb;
+  for (int e = 0; e < Ep; ++e) {
+    const int g = (counts[e] + GROUP_ROWS - 1) / GROUP_ROWS;
+    group_start[e + 1] = group_start[e] + g;
+    for (int i = 0; i < g; ++i) group_mb.push_back(mb_start[e] + i * GROUP_ROWS / BLOCK_M);
+  }
+  const int ngather = gather_total(group_start[Ep]), npost = post_total(cp, M);
   struct VecWorker { bool holding = false; VecTask v; };
   std::vector<VecWorker> vw(vec_workers);
   // rows of each token (slot order is irrelevant here): token t's k+S rows live in M-blocks drawn round-robin
@@ -1161,10 +1176,11 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     for (int q = 0; q < pairs; ++q) {
       if (cursor[q] >= queue[q].size()) continue;
       const Item& it = queue[q][cursor[q]];
-      const int wk = phase_wait_kind(cp, it.phase), thr = phase_wait_thr(cp, it.phase);
+      const int wk = phase_wait_kind(cp, it.phase);
       bool ready = true;
       for (int m = 0; m < it.mb_a + it.mb_b; ++m)
-        if (ctr[ctr_index(it.mb_first + m, wk)] < thr) ready = false;
+        if (ctr[ctr_index(it.mb_first + m, wk)] < phase_wait_thr(cp, it.phase, counts[it.e], it.mb_first - mb_start[it.e] + m))
+          ready = false;
       if (!ready) { ++stalls; continue; }
       const int tk = phase_trigger_kind(cp, it.phase);
       if (tk >= 0)
@@ -1173,8 +1189,8 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     }
     for (size_t wi = 0; wi < vw.size(); ++wi) {
       auto& w = vw[wi];
-      // worker 0 is a background gatherer; the others leave the gather queue after the first M-blocks
-      const bool may_gather = next_gather < ngather && (wi == 0 || next_gather < GATHER_SUB * GATHER_FAST_MBLOCKS);
+      // worker 0 is a background gatherer; the others leave the gather queue after the first tasks
+      const bool may_gather = next_gather < ngather && (wi == 0 || next_gather < GATHER_FAST_TASKS);
       if (!w.holding && may_gather) {
         w.v.op = VEC_GATHER; w.v.idx = next_gather++;
         w.holding = true;
@@ -1189,10 +1205,11 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
       if (w.v.op == VEC_DW)
         ready = ctr[ctr_index(rotate_index(w.v.idx, n_shared > 0 ? mb_start[Ep - n_shared] : 0, M), CTR_ACTIVATED)] >= thr_activated(cp);
       if (w.v.op == VEC_COMBINE)
-        ready = token_mblocks_done(w.v.idx * COMBINE_TOKENS, std::min(T, (w.v.idx + 1) * COMBINE_TOKENS));
+        ready = token_mblocks_done(w.v.idx / cp.combine_split, w.v.idx / cp.combine_split + 1);
       if (!ready) { ++stalls; continue; }
       if (w.v.op == VEC_GATHER)
-        ctr[ctr_index(rotate_index(w.v.idx, n_shared > 0 ? mb_start[Ep - n_shared] * GATHER_SUB : 0, ngather) / GATHER_SUB, CTR_GATHERED)] += 1;
+        ctr[ctr_index(group_mb[rotate_index(w.v.idx, n_shared > 0 ? group_start[Ep - n_shared] * GATHER_SUB : 0, ngather) / GATHER_SUB],
+                      CTR_GATHERED)] += 1;
       w.holding = false;
       ++done_vec;
       progress = true;
@@ -1201,10 +1218,11 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     if (!progress) return 20;  // deadlock
   }
   // 3. every counter ends exactly at its threshold
-  for (int mb = 0; mb < M; ++mb)
-    if (ctr[ctr_index(mb, CTR_GATHERED)] != thr_gathered() || ctr[ctr_index(mb, CTR_ACTIVATED)] != thr_activated(cp) ||
-        ctr[ctr_index(mb, CTR_DONE)] != thr_done(cp))
-      return 30;
+  for (int e = 0; e < Ep; ++e)
+    for (int mb = mb_start[e]; mb < mb_start[e + 1]; ++mb)
+      if (ctr[ctr_index(mb, CTR_GATHERED)] != thr_gathered(counts[e], mb - mb_start[e]) ||
+          ctr[ctr_index(mb, CTR_ACTIVATED)] != thr_activated(cp) || ctr[ctr_index(mb, CTR_DONE)] != thr_done(cp))
+        return 30;
   if (stats) { stats[0] = n_items; stats[1] = vtotal; stats[2] = rounds; stats[3] = stalls; }
   return MOE_OK;
 }

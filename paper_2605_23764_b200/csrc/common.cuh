@@ -144,15 +144,16 @@ __device__ __forceinline__ bool counter_wait(const int* ctr, int threshold, cons
         return false;
       }
     }
-    __nanosleep(sleep_ns);  // back off: pollers must not crowd the L2 slice that holds the counter
-    if (sleep_ns < max_sleep_ns) sleep_ns <<= 1;
+    // back off: pollers must not crowd the L2 slice that holds the counter.  The sleep grows with the time waited, so that
+    // a wait is overshot by a few per cent of its length
+    __nanosleep(sleep_ns);
+    if (sleep_ns < max_sleep_ns) sleep_ns += 16;
   }
 }
 
 // Release-increment of a trigger counter (the paper's "trigger event"): call after the tile's
-// global stores, from one thread, behind a barrier that orders the other threads' stores.
+// global stores, from one thread, behind a barrier that orders the other threads' stores (the release is cumulative).
 __device__ __forceinline__ void counter_signal(int* ctr, int inc) {
-  __threadfence();
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(ctr), "r"(inc) : "memory");
 }
 

@@ -47,27 +47,24 @@ __device__ __forceinline__ uint4 ldg_cg_v4(const void* p) {
   return v;
 }
 
-// Dispatch / backward Dispatch: GATHER_ROWS rows of one M-block of the padded expert-ordered row space.  The
-// index chains of the rows are resolved first, then the rows are copied together: 16 independent 16-byte
-// loads in flight per lane.
-constexpr int GATHER_ROWS = BLOCK_M / GATHER_SUB;
-__device__ __forceinline__ void vec_gather(const FusedArgs& fa, int task, int lane) {
-  const int mb = task / GATHER_SUB, sub = task - mb * GATHER_SUB;
+// Dispatch / backward Dispatch: GATHER_ROWS rows of one 32-row group of an expert.  The rows' slots and place are two
+// independent loads by group; then the rows are copied together: 16 independent 16-byte loads in flight per lane.
+// Returns the rows' M-block.
+__device__ __forceinline__ int vec_gather(const FusedArgs& fa, int task, int lane) {
+  const int g = task / GATHER_SUB, sub = (task - g * GATHER_SUB) * GATHER_ROWS;
   const LayoutView& lv = fa.lv;
-  const int e = lv.mblk_expert[mb];
-  const int cnt = lv.counts[e], pad0 = lv.pad_off[e], off0 = lv.offsets[e];
+  const int4 sl = *reinterpret_cast<const int4*>(lv.group_slot + (size_t)g * GROUP_ROWS + sub);
+  const int p0 = lv.group_row[g] + sub;
+  const int slots[GATHER_ROWS] = {sl.x, sl.y, sl.z, sl.w};
   const int nvec = fa.d >> 3;
   const int k = fa.cp.k;
-  const int p0 = mb * BLOCK_M + sub * GATHER_ROWS;
   const uint4* in[GATHER_ROWS];
 #pragma unroll
   for (int r = 0; r < GATHER_ROWS; ++r) {
-    const int local = p0 + r - pad0;
     in[r] = nullptr;
     float w = 0.0f;
-    if (local < cnt) {
-      const int slot = lv.src_of[off0 + local];
-      const int t = slot / fa.kp, j = slot - t * fa.kp;
+    if (slots[r] >= 0) {
+      const int t = slots[r] / fa.kp, j = slots[r] - t * fa.kp;
       in[r] = reinterpret_cast<const uint4*>(fa.gather_src + (size_t)t * fa.d);
       if (fa.prow_w) w = j < k ? fa.topk_w[(size_t)t * k + j] : 1.0f;
     }
@@ -88,18 +85,21 @@ __device__ __forceinline__ void vec_gather(const FusedArgs& fa, int task, int la
       for (int u = 0; u < U; ++u)
         if (v + 32 * u < nvec) out[(size_t)r * nvec + v + 32 * u] = q[r][u];   // padding rows are zero-filled
   }
+  return p0 / BLOCK_M;
 }
 
-// Combine / backward Combine of COMBINE_TOKENS tokens.  Dependent events: `done` of every M-block that
-// holds one of a token's rows (many-to-many, Section 4.3): each lane polls the counter of one row.
+// Combine / backward Combine of one token, or of one of its column chunks.  Dependent events: `done` of every M-block that
+// holds one of the token's rows (many-to-many, Section 4.3): each lane polls the counter of one row.
 __device__ __forceinline__ bool vec_combine(const FusedArgs& fa, int task, int lane, const WaitCtl& wc) {
-  const int nvec = fa.d >> 3, kp = fa.kp, T = fa.cp.T;
-  const int i0 = task * COMBINE_TOKENS, i1 = min(T, i0 + COMBINE_TOKENS);
+  const int kp = fa.kp, split = fa.cp.combine_split;
   const int thr = thr_done(fa.cp);
-  for (int i = i0; i < i1; ++i) {
+  const int i = task / split, chunk = task - i * split;
+  const int per = (((fa.d >> 3) + split - 1) / split + 31) & ~31;   // vectors of a chunk
+  const int v0 = chunk * per, nvec = min(fa.d >> 3, v0 + per);
+  {
     const int t = fa.lv.combine_order ? fa.lv.combine_order[i] : i;   // tokens in the order in which their last row is produced
     const int* prow = fa.lv.prow_of + (size_t)t * kp;
-    if (fa.d_topk_w)   // a slot dropped for an invalid expert id has no row: its weight's gradient is zero
+    if (fa.d_topk_w && chunk == 0)   // a slot dropped for an invalid expert id has no row: its weight's gradient is zero
       for (int j = lane; j < fa.cp.k; j += 32)
         if (prow[j] < 0) fa.d_topk_w[(size_t)t * fa.cp.k + j] = 0.f;
     // dependent events: `done` of every M-block that holds one of the token's rows
@@ -110,7 +110,7 @@ __device__ __forceinline__ bool vec_combine(const FusedArgs& fa, int task, int l
     }
     if (!__all_sync(0xffffffffu, ok)) return false;
     // two vector positions per lane and step: sixteen independent row loads in flight (a warp alone is latency-bound)
-    for (int v = lane; v < nvec; v += 64) {
+    for (int v = v0 + lane; v < nvec; v += 64) {
       const bool two = v + 32 < nvec;
       float acc[16];
 #pragma unroll
@@ -179,7 +179,7 @@ __device__ __forceinline__ bool vec_dw(const FusedArgs& fa, int mb, int lane, co
   return true;
 }
 
-// Vector workers.  The gather of the first GATHER_FAST_MBLOCKS M-blocks -- what the first matrix items of every
+// Vector workers.  The first GATHER_FAST_TASKS gather tasks -- what the first matrix items of every
 // pair wait for -- is taken by every worker; after that only BACKGROUND_GATHERERS warps per CTA keep gathering,
 // a few M-blocks' worth of traffic at a time, well ahead of the matrix queue but far below the bandwidth the
 // GEMMs need: a gather at full speed takes its bytes from the loads of the matrix tiles and slows them by more
@@ -188,10 +188,10 @@ constexpr int BACKGROUND_GATHERERS = 2;
 __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const WaitCtl& wc, const TraceCtl& tr, int M,
                                                    int lane, bool background_gatherer) {
   if (*reinterpret_cast<volatile int*>(&fa.status->abort)) return;
-  const int ngather = gather_total(M), fast = GATHER_SUB * GATHER_FAST_MBLOCKS;
-  // with shared experts the gather starts at their first M-block, like the matrix queue (schedule.h, rotate_index)
+  const int ngather = gather_total(fa.lv.meta[5]), fast = GATHER_FAST_TASKS;
+  // with shared experts the gather starts at their first row, like the matrix queue (schedule.h, rotate_index)
   const int S = fa.cp.kp - fa.cp.k;
-  const int gather_first = S > 0 ? fa.lv.mb_start[fa.cp.Ep - S] * GATHER_SUB : 0;
+  const int gather_first = S > 0 ? fa.lv.group_start[fa.cp.Ep - S] * GATHER_SUB : 0;
   while (true) {
     int t = ngather;
     if (lane == 0) {
@@ -203,21 +203,21 @@ __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const Wa
     t = rotate_index(t, gather_first, ngather);
     uint64_t t0 = 0;
     if (tr.buf && lane == 0) t0 = globaltimer_ns();
-    vec_gather(fa, t, lane);
+    const int mb = vec_gather(fa, t, lane);
     __syncwarp();
     if (lane == 0) {
-      counter_signal(fa.ctr + ctr_index(t / GATHER_SUB, CTR_GATHERED), 1);
+      counter_signal(fa.ctr + ctr_index(mb, CTR_GATHERED), 1);
       if (tr.buf) trace_put(tr, TR_VEC, VEC_GATHER, t, t0, t0, globaltimer_ns());
     }
   }
-  const int npost = post_total(fa.cp, M);
+  const int npost = post_total(fa.cp, M), dw_first = S > 0 ? fa.lv.mb_start[fa.cp.Ep - S] : 0;
   while (true) {
     int t = 0;
     if (lane == 0) t = atomicAdd(&fa.ctr[CTR_POST_TICKET], 1);
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= npost) break;
     VecTask v = decode_post_ticket(fa.cp, t, M);
-    if (v.op == VEC_DW) v.idx = rotate_index(v.idx, gather_first / GATHER_SUB, M);   // in the order act_grad produces them
+    if (v.op == VEC_DW) v.idx = rotate_index(v.idx, dw_first, M);   // in the order act_grad produces them
     uint64_t t0 = 0;
     if (tr.buf && lane == 0) t0 = globaltimer_ns();
     const bool ok = v.op == VEC_COMBINE ? vec_combine(fa, v.idx, lane, wc) : vec_dw(fa, v.idx, lane, wc);
@@ -230,8 +230,7 @@ __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const Wa
       __syncwarp();
       if (lane == 0) {
         __threadfence();
-        const int ncombine = (fa.cp.T + COMBINE_TOKENS - 1) / COMBINE_TOKENS;
-        if (atomicAdd(&fa.ctr[CTR_COMBINE_DONE], 1) + 1 == ncombine) {
+        if (atomicAdd(&fa.ctr[CTR_COMBINE_DONE], 1) + 1 == combine_total(fa.cp)) {
           __threadfence_system();
           *reinterpret_cast<volatile int*>(&fa.ctr[CTR_OUT_READY]) = 1;
         }
@@ -384,7 +383,7 @@ __device__ __forceinline__ ChainDeps phase_deps(const FusedArgs& fa, int phase, 
   ChainDeps d;
   d.ctr = fa.ctr;
   d.wait_kind = phase_wait_kind(fa.cp, phase);
-  d.wait_thr = phase_wait_thr(fa.cp, phase);
+  d.cp = &fa.cp;
   d.trig_kind = phase_trigger_kind(fa.cp, phase);
   d.phase = phase;
   d.wc = wc;
@@ -505,7 +504,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (tr.buf && lane == 0) t0 = globaltimer_ns();
       int first, count;
       decode_item<BWD>(fa, wd.phase, wd.item, wd, &first, &count);
-      if (!dep.wait(first, count, lane, t)) break;   // the item's dependent events (Section 4.3)
+      if (!dep.wait(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane, t)) break;   // the item's dependent events (Section 4.3)
       if (lane == 0) {
         const uint64_t td = tr.buf ? globaltimer_ns() : 0;
         ring_publish(ring, n, wd);

@@ -119,7 +119,6 @@ __device__ __forceinline__ void trace_put(const TraceCtl& tr, int role, int phas
 // No events: the one-launch-per-operator kernels (the kernel boundary orders the operators).
 struct NoDeps {
   static constexpr bool kOn = false;
-  __device__ __forceinline__ bool wait(int, int, int, int) const { return true; }
   __device__ __forceinline__ void signal(int, int) const {}
   __device__ __forceinline__ bool tracing() const { return false; }
   __device__ __forceinline__ void trace(int, int, uint64_t, uint64_t, uint64_t) const {}
@@ -128,16 +127,18 @@ struct NoDeps {
 struct ChainDeps {
   static constexpr bool kOn = true;
   int* ctr;
-  int wait_kind, wait_thr;   // dependent event of the phase's items
+  int wait_kind;             // dependent event of the phase's items
+  const ChainParams* cp;     // (its thresholds)
   int trig_kind;             // trigger event (CTR_NONE: nothing consumes the phase's output inside the launch)
   int phase;
   WaitCtl wc;
   TraceCtl tr;
-  // All lanes of a warp: wait until the counters of M-blocks [first, first + count) reach the threshold.
-  __device__ __forceinline__ bool wait(int first, int count, int lane, int item) const {
+  // All lanes of a warp: wait until the counters of M-blocks [first, first + count), the first of them M-block `rel` of its
+  // expert with `rows` rows, reach their thresholds.
+  __device__ __forceinline__ bool wait(int first, int count, int rows, int rel, int lane, int item) const {
     int ok = 1;
     for (int q = lane; q < count; q += 32)
-      if (!counter_wait(ctr + ctr_index(first + q, wait_kind), wait_thr, wc, item)) ok = 0;
+      if (!counter_wait(ctr + ctr_index(first + q, wait_kind), phase_wait_thr(*cp, phase, rows, rel + q), wc, item)) ok = 0;
     return __all_sync(0xffffffffu, ok) != 0;
   }
   // One lane, after its warp's stores of the tile are complete and ordered (see the epilogue roles).

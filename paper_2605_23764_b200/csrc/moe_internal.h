@@ -43,7 +43,10 @@ struct LayoutView {
   int* work_start;   // [Ep+1]  first work item of each expert (token-column GEMMs that merge: its units, the last
                      //         two of an odd M-block count >= 3 merged into one item)
   int* wblk_expert;  // [items] expert of each work item
-  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, 0...}
+  int* group_start;  // [Ep+1]  first 32-row group of each expert (an expert's rows up to a multiple of 32); NULL: not wanted
+  int* group_row;    // [groups] first padded row of each group
+  int* group_slot;   // [groups * 32] slot of each of the groups' rows, -1 for padding
+  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, num_groups, 0...}
   int* blk_hist;     // [nblk][Ep] per-block histograms, then per-block exclusive prefixes
   int* combine_order; // [T] persistent launch: tokens in the order in which their last row is produced (NULL: token order)
   int* tok_last;      // [T] 1 + largest padded row of each token (0: none); NULL when the combine order is not wanted
@@ -62,8 +65,8 @@ cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView&
 std::atomic<bool>& study_plain_launch();
 
 // ---- permute.cu
-// Xp[p] = src[token of padded row p] (zeros on padding rows); optionally prow_w[p] = routing weight
-// of the row (1 for shared experts, 0 on padding rows).
+// Xp[p] = src[token of padded row p] (zeros on padding rows), up to each expert's last 32-row group (nothing reads the
+// rows behind it); optionally prow_w[p] = routing weight of the row (1 for shared experts, 0 on padding rows).
 cudaError_t launch_gather(const uint16_t* src, const float* topk_w, const Dims& dm, const LayoutView& lv,
                           uint16_t* dst, float* prow_w, int rows_cap, cudaStream_t s, int* launches,
                           DevStatus* status = nullptr, uint64_t budget_ns = 0);

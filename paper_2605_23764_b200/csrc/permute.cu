@@ -18,30 +18,37 @@ __device__ __forceinline__ uint4 ld_nc_v4(const void* p) {
   return v;
 }
 
-// dst[p][:] = src[token(p)][:] for every padded row p < R_pad; padding rows are zero-filled so
-// that reductions over an expert's rows (weight gradients) may run over whole M-blocks.
+// A row of the gather: its place in the padded row space, its token (-1: padding) and routing weight.
+struct GatherRow { int p, t; float w; };
+__device__ __forceinline__ GatherRow gather_row(const LayoutView& lv, int i, const float* topk_w, int k, int kp) {
+  GatherRow r;
+  r.p = lv.group_row[i / GROUP_ROWS] + (i & (GROUP_ROWS - 1));
+  const int slot = lv.group_slot[i];
+  r.t = -1;
+  r.w = 0.0f;
+  if (slot >= 0) {
+    r.t = slot / kp;
+    const int j = slot - r.t * kp;
+    r.w = j < k ? (topk_w ? topk_w[(size_t)r.t * k + j] : 0.0f) : 1.0f;
+  }
+  return r;
+}
+
+// dst[p][:] = src[token(p)][:] for every row p of the experts' 32-row groups; padding rows are zero-filled so
+// that reductions over an expert's rows (weight gradients) may run over whole groups.
 __global__ void __launch_bounds__(PERM_THREADS) gather_rows_kernel(const uint16_t* __restrict__ src,
                                                                     const float* __restrict__ topk_w, int d, int k,
                                                                     int kp, LayoutView lv,
                                                                     uint16_t* __restrict__ dst,
                                                                     float* __restrict__ prow_w) {
-  const int r_pad = lv.meta[1];
+  const int n = lv.meta[5] * GROUP_ROWS;
   const int nvec = d >> 3;
-  for (int p = blockIdx.x; p < r_pad; p += gridDim.x) {
-    const int e = lv.mblk_expert[p / BLOCK_M];
-    const int local = p - lv.pad_off[e];
-    const bool valid = local < lv.counts[e];
-    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)p * d);
-    if (valid) {
-      const int slot = lv.src_of[lv.offsets[e] + local];
-      const int t = slot / kp, j = slot - t * kp;
-      const uint4* in = reinterpret_cast<const uint4*>(src + (size_t)t * d);
-      for (int v = threadIdx.x; v < nvec; v += PERM_THREADS) out[v] = ld_nc_v4(in + v);
-      if (prow_w && threadIdx.x == 0) prow_w[p] = j < k ? topk_w[(size_t)t * k + j] : 1.0f;
-    } else {
-      for (int v = threadIdx.x; v < nvec; v += PERM_THREADS) out[v] = make_uint4(0, 0, 0, 0);
-      if (prow_w && threadIdx.x == 0) prow_w[p] = 0.0f;
-    }
+  for (int i = blockIdx.x; i < n; i += gridDim.x) {
+    const GatherRow r = gather_row(lv, i, topk_w, k, kp);
+    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)r.p * d);
+    const uint4* in = reinterpret_cast<const uint4*>(src + (size_t)(r.t < 0 ? 0 : r.t) * d);
+    for (int v = threadIdx.x; v < nvec; v += PERM_THREADS) out[v] = r.t < 0 ? make_uint4(0, 0, 0, 0) : ld_nc_v4(in + v);
+    if (prow_w && threadIdx.x == 0) prow_w[r.p] = r.w;
   }
 }
 
@@ -51,25 +58,16 @@ __global__ void __launch_bounds__(PERM_THREADS) gather_rows_warp_kernel(const ui
                                                                          int kp, LayoutView lv,
                                                                          uint16_t* __restrict__ dst,
                                                                          float* __restrict__ prow_w) {
-  const int r_pad = lv.meta[1];
+  const int n = lv.meta[5] * GROUP_ROWS;
   const int nvec = d >> 3;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int WPB = PERM_THREADS / 32;
-  for (int p = blockIdx.x * WPB + warp; p < r_pad; p += gridDim.x * WPB) {
-    const int e = lv.mblk_expert[p / BLOCK_M];
-    const int local = p - lv.pad_off[e];
-    const bool valid = local < lv.counts[e];
-    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)p * d);
-    if (valid) {
-      const int slot = lv.src_of[lv.offsets[e] + local];
-      const int t = slot / kp, j = slot - t * kp;
-      const uint4* in = reinterpret_cast<const uint4*>(src + (size_t)t * d);
-      for (int v = lane; v < nvec; v += 32) out[v] = ld_nc_v4(in + v);
-      if (prow_w && lane == 0) prow_w[p] = j < k ? topk_w[(size_t)t * k + j] : 1.0f;
-    } else {
-      for (int v = lane; v < nvec; v += 32) out[v] = make_uint4(0, 0, 0, 0);
-      if (prow_w && lane == 0) prow_w[p] = 0.0f;
-    }
+  for (int i = blockIdx.x * WPB + warp; i < n; i += gridDim.x * WPB) {
+    const GatherRow r = gather_row(lv, i, topk_w, k, kp);
+    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)r.p * d);
+    const uint4* in = reinterpret_cast<const uint4*>(src + (size_t)(r.t < 0 ? 0 : r.t) * d);
+    for (int v = lane; v < nvec; v += 32) out[v] = r.t < 0 ? make_uint4(0, 0, 0, 0) : ld_nc_v4(in + v);
+    if (prow_w && lane == 0) prow_w[r.p] = r.w;
   }
 }
 
@@ -98,51 +96,44 @@ __global__ void __launch_bounds__(32) gather_rows_bulk_kernel(const uint16_t* __
   __syncwarp();
   if (lane >= lanes) return;
   const WaitCtl wc{status, budget_ns};
-  const int r_pad = lv.meta[1];
+  const int total = lv.meta[5] * GROUP_ROWS;
   const int stride = gridDim.x * lanes;
   uint8_t* my = slots + (size_t)lane * 2 * row_bytes;
-  // row -> source row (or -1 for a padding row); also writes the row's routing weight
-  auto source_of = [&](int p) -> long {
-    const int e = lv.mblk_expert[p / BLOCK_M];
-    const int local = p - lv.pad_off[e];
-    if (local >= lv.counts[e]) {
-      if (prow_w) prow_w[p] = 0.0f;
-      return -1;
-    }
-    const int slot = lv.src_of[lv.offsets[e] + local];
-    const int t = slot / kp, j = slot - t * kp;
-    if (prow_w) prow_w[p] = j < k ? topk_w[(size_t)t * k + j] : 1.0f;
-    return t;
+  auto row_at = [&](int i) {   // also writes the row's routing weight
+    const GatherRow r = gather_row(lv, i, topk_w, k, kp);
+    if (prow_w) prow_w[r.p] = r.w;
+    return r;
   };
-  auto load = [&](long t, int b) {
+  auto load = [&](int t, int b) {
     mbar_expect_tx(&full[2 * lane + b], row_bytes);
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_u32(my + (size_t)b * row_bytes)), "l"(src + (size_t)t * d), "r"(row_bytes),
                    "r"(smem_u32(&full[2 * lane + b]))
                  : "memory");
   };
-  int p = blockIdx.x * lanes + lane;
+  int i = blockIdx.x * lanes + lane;
   uint32_t n = 0, ph[2] = {0, 0};
-  long t_cur = p < r_pad ? source_of(p) : -1;
-  if (p < r_pad && t_cur >= 0) load(t_cur, 0);
-  for (; p < r_pad; p += stride, ++n) {
+  GatherRow cur{0, -1, 0.f}, next{0, -1, 0.f};
+  if (i < total) cur = row_at(i);
+  if (cur.t >= 0) load(cur.t, 0);
+  for (; i < total; i += stride, ++n) {
     const int b = n & 1;
-    const int pn = p + stride;
-    const long t_next = pn < r_pad ? source_of(pn) : -1;
+    next.t = -1;
+    if (i + stride < total) next = row_at(i + stride);
     // the other slot is free once the previous row's store has read it
     tma_store_wait_read();
-    if (pn < r_pad && t_next >= 0) load(t_next, b ^ 1);
+    if (next.t >= 0) load(next.t, b ^ 1);
     const uint8_t* from = zero_row;
-    if (t_cur >= 0) {
-      if (!mbar_wait(&full[2 * lane + b], ph[b], wc, SITE_FULL, p)) break;
+    if (cur.t >= 0) {
+      if (!mbar_wait(&full[2 * lane + b], ph[b], wc, SITE_FULL, i)) break;
       ph[b] ^= 1;
       from = my + (size_t)b * row_bytes;
     }
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 ::"l"(dst + (size_t)p * d), "r"(smem_u32(from)), "r"(row_bytes)
+                 ::"l"(dst + (size_t)cur.p * d), "r"(smem_u32(from)), "r"(row_bytes)
                  : "memory");
     tma_store_commit();
-    t_cur = t_next;
+    cur = next;
   }
   tma_store_wait_all();
 }

@@ -133,11 +133,16 @@ __global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __
 }
 
 // Exclusive scans over the experts of a block of 1024 threads: s_counts[Ep] -> offsets of rows, M-blocks, pairs of
-// M-blocks and work items, in shared memory (each Ep + 1 long) and in the layout's tables.
-struct ExpertScan { int *counts, *off, *mb, *pr, *wi; };   // shared memory
+// M-blocks, work items and 32-row groups, in shared memory (each Ep + 1 long) and in the layout's tables.
+struct ExpertScan { int *counts, *off, *mb, *pr, *wi, *gr; };   // shared memory
+__host__ __device__ constexpr int expert_scan_ints(int Ep) { return 6 * Ep + 5; }
+__device__ __forceinline__ ExpertScan expert_scan_at(int* sm, int Ep) {
+  return ExpertScan{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3, sm + 5 * Ep + 4};
+}
 __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const ExpertScan& sc, int (*totals)[33]) {
+  constexpr int NQ = 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int carry[4] = {0, 0, 0, 0};
+  int carry[NQ] = {0, 0, 0, 0, 0};
   for (int e0 = 0; e0 < Ep; e0 += 1024) {
     const int e = e0 + threadIdx.x;
     const int c = e < Ep ? sc.counts[e] : 0;
@@ -145,22 +150,22 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
     const int pr = (m + 1) >> 1;  // pairs of M-blocks (the tensor-core tile of a CTA pair)
     // work items of the token-column GEMM kernels that merge: the units of the expert, except that an expert
     // that merges (schedule.h) has its last two units (one block; block + tail) share one k-loop
-    const int val[4] = {c, m, pr, pr - (expert_merges(c, m) ? 1 : 0)};
-    int inc[4] = {val[0], val[1], val[2], val[3]};
+    const int val[NQ] = {c, m, pr, pr - (expert_merges(c, m) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS};
+    int inc[NQ] = {val[0], val[1], val[2], val[3], val[4]};
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < NQ; ++q) {
         const int o = __shfl_up_sync(0xffffffffu, inc[q], off);
         if (lane >= off) inc[q] += o;
       }
     }
     if (lane == 31) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) totals[q][warp] = inc[q];
+      for (int q = 0; q < NQ; ++q) totals[q][warp] = inc[q];
     }
     __syncthreads();
-    if (warp < 4) {   // warp q: exclusive scan of quantity q's warp totals, the block's total behind them
+    if (warp < NQ) {   // warp q: exclusive scan of quantity q's warp totals, the block's total behind them
       const int w = totals[warp][lane];
       int wi = w;
 #pragma unroll
@@ -172,24 +177,28 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
       if (lane == 31) totals[warp][32] = wi;
     }
     __syncthreads();
-    int ex[4];
+    int ex[NQ];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) ex[q] = carry[q] + totals[q][warp] + inc[q] - val[q];
+    for (int q = 0; q < NQ; ++q) ex[q] = carry[q] + totals[q][warp] + inc[q] - val[q];
     if (e < Ep) {
-      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.pr[e] = ex[2]; sc.wi[e] = ex[3];
+      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.pr[e] = ex[2]; sc.wi[e] = ex[3]; sc.gr[e] = ex[4];
       lv.counts[e] = c;
       lv.offsets[e] = ex[0];
       lv.mb_start[e] = ex[1];
       lv.pad_off[e] = ex[1] * BLOCK_M;
       lv.pair_start[e] = ex[2];
       lv.work_start[e] = ex[3];
+      if (lv.group_start) {
+        lv.group_start[e] = ex[4];
+        for (int r = c; r < val[4] * GROUP_ROWS; ++r) lv.group_slot[ex[4] * GROUP_ROWS + r] = -1;   // padding rows of the last group
+      }
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) carry[q] += totals[q][32];
+    for (int q = 0; q < NQ; ++q) carry[q] += totals[q][32];
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.pr[Ep] = carry[2]; sc.wi[Ep] = carry[3];
+    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.pr[Ep] = carry[2]; sc.wi[Ep] = carry[3]; sc.gr[Ep] = carry[4];
     lv.offsets[Ep] = carry[0];
     lv.mb_start[Ep] = carry[1];
     lv.pad_off[Ep] = carry[1] * BLOCK_M;
@@ -200,25 +209,29 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
     lv.meta[2] = carry[0];
     lv.meta[3] = carry[2];
     lv.meta[4] = carry[3];
+    lv.meta[5] = carry[4];
+    if (lv.group_start) lv.group_start[Ep] = carry[4];
   }
   __syncthreads();
 }
-// table[i] = the last expert whose start is <= i, for i < start[Ep]
-__device__ __forceinline__ void expert_table(int Ep, const int* start, int* table) {
-  const int num = start[Ep];
-  for (int i = threadIdx.x; i < num; i += blockDim.x) {
-    int lo = 0, hi = Ep - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (start[mid] <= i) lo = mid; else hi = mid - 1;
-    }
-    table[i] = lo;
+// the last expert whose start is <= i
+__device__ __forceinline__ int expert_at(int Ep, const int* start, int i) {
+  int lo = 0, hi = Ep - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (start[mid] <= i) lo = mid; else hi = mid - 1;
   }
+  return lo;
 }
 __device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, const ExpertScan& sc) {
-  expert_table(Ep, sc.mb, lv.mblk_expert);
-  expert_table(Ep, sc.pr, lv.pblk_expert);
-  expert_table(Ep, sc.wi, lv.wblk_expert);
+  for (int i = threadIdx.x; i < sc.mb[Ep]; i += blockDim.x) lv.mblk_expert[i] = expert_at(Ep, sc.mb, i);
+  for (int i = threadIdx.x; i < sc.pr[Ep]; i += blockDim.x) lv.pblk_expert[i] = expert_at(Ep, sc.pr, i);
+  for (int i = threadIdx.x; i < sc.wi[Ep]; i += blockDim.x) lv.wblk_expert[i] = expert_at(Ep, sc.wi, i);
+  if (lv.group_start)
+    for (int i = threadIdx.x; i < sc.gr[Ep]; i += blockDim.x) {
+      const int e = expert_at(Ep, sc.gr, i);
+      lv.group_row[i] = sc.mb[e] * BLOCK_M + (i - sc.gr[e]) * GROUP_ROWS;
+    }
 }
 
 // One block.  (1) per expert, exclusive scan of the block histograms over blocks: a thread per expert and range of
@@ -226,9 +239,9 @@ __device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, cons
 // (2) scans over experts; (3) M-block, pair and work-item -> expert tables.
 __global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int Ep, LayoutView lv) {
   extern __shared__ int sm[];
-  __shared__ int totals[4][33];
-  const ExpertScan sc{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3};
-  int* part = sm + 5 * Ep + 4;   // [ranges][Ep]
+  __shared__ int totals[5][33];
+  const ExpertScan sc = expert_scan_at(sm, Ep);
+  int* part = sm + expert_scan_ints(Ep);   // [ranges][Ep]
   pdl_trigger();
   pdl_wait();
   const int ranges = Ep <= 1024 ? 1024 / Ep : 1;
@@ -275,9 +288,10 @@ __global__ void __launch_bounds__(WARPS * 32) layout_rank_kernel(const int* __re
   extern __shared__ int sm[];
   int* base = sm;                                              // [Ep] first row of this block's rows of the expert
   int* pad = sm + Ep;                                          // [Ep] padded row - row of the expert
-  int* last = sm + 2 * Ep;                                     // [LAYOUT_CHUNK / kp + 2] key of the chunk's tokens
+  int* grp = sm + 2 * Ep;                                      // [Ep] place among the groups' rows - row of the expert
+  int* last = sm + 3 * Ep;                                     // [LAYOUT_CHUNK / kp + 2] key of the chunk's tokens
   const int nlast = LAYOUT_CHUNK / kp + 2;
-  uint16_t* whist = reinterpret_cast<uint16_t*>(last + nlast + (nlast & 1));   // [WARPS][Ep + (Ep & 1)]
+  uint16_t* whist = reinterpret_cast<uint16_t*>(last + nlast + ((nlast + Ep) & 1));   // [WARPS][Ep + (Ep & 1)]
   const int ld = Ep + (Ep & 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_trigger();
@@ -313,6 +327,7 @@ __global__ void __launch_bounds__(WARPS * 32) layout_rank_kernel(const int* __re
     const int off = __ldcg(lv.offsets + q);
     base[q] = off + __ldcg(lv.blk_hist + (size_t)blockIdx.x * Ep + q);
     pad[q] = __ldcg(lv.pad_off + q) - off;
+    if (lv.group_start) grp[q] = __ldcg(lv.group_start + q) * GROUP_ROWS - off;
   }
   __syncthreads();
   const int t_first = blockIdx.x * LAYOUT_CHUNK / kp;
@@ -325,6 +340,7 @@ __global__ void __launch_bounds__(WARPS * 32) layout_rank_kernel(const int* __re
       lv.row_of[i] = row;
       lv.prow_of[i] = prow;
       lv.src_of[row] = i;
+      if (lv.group_start) lv.group_slot[row + grp[e[g]]] = i;
       // the combine order's key: the token's last ROUTED row (shared experts are taken first by the persistent launch)
       if (lv.tok_last && i % kp < k) atomicMax(&last[i / kp - t_first], prow + 1);
     } else {
@@ -424,10 +440,10 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
                                                           int Ep, LayoutView lv, int want_order, DevStatus* status,
                                                           int* __restrict__ zero, int nzero) {
   extern __shared__ int sm[];
-  __shared__ int totals[4][33];
+  __shared__ int totals[5][33];
   __shared__ int carry_s;
-  const ExpertScan sc{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3};
-  int* s_last = sm + 5 * Ep + 4;                       // [LAYOUT_ONE_SLOTS] 1 + padded row of the slot
+  const ExpertScan sc = expert_scan_at(sm, Ep);
+  int* s_last = sm + expert_scan_ints(Ep);                       // [LAYOUT_ONE_SLOTS] 1 + padded row of the slot
   int* bins = s_last + LAYOUT_ONE_SLOTS;               // [LAYOUT_ONE_SLOTS + 1]
   uint16_t* whist = reinterpret_cast<uint16_t*>(bins + LAYOUT_ONE_SLOTS + 2 + (Ep & 1));   // [warps in use][ld]
   const int ld = Ep + (Ep & 1);
@@ -467,6 +483,7 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
       prow = sc.mb[e] * BLOCK_M + in_expert;
       lv.row_of[i] = row;
       lv.src_of[row] = i;
+      if (lv.group_start) lv.group_slot[sc.gr[e] * GROUP_ROWS + in_expert] = i;
     } else {
       lv.row_of[i] = -1;
       note(status, /*MOE_ERR_BAD_EXPERT_ID*/ 1, i);
@@ -494,7 +511,7 @@ cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView&
   const int n = dm.slots(), Ep = dm.Ep(), kp = dm.kp();
   cudaError_t e;
   if (n < LAYOUT_ONE_SLOTS && Ep <= LAYOUT_ONE_EXPERTS) {
-    const size_t smem = sizeof(int) * (size_t)(5 * Ep + 8 + 2 * LAYOUT_ONE_SLOTS) +
+    const size_t smem = sizeof(int) * (size_t)(expert_scan_ints(Ep) + 4 + 2 * LAYOUT_ONE_SLOTS) +
                         sizeof(uint16_t) * (size_t)((n + 31) / 32) * (Ep + (Ep & 1));
     ++*launches;
     return launch_dependent(layout_one_kernel, dim3(1), dim3(1024), smem, s, topk_ids, n, dm.T, dm.k, kp, dm.E, Ep, lv,
@@ -508,11 +525,11 @@ cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView&
                             kp, dm.E, Ep, lv.blk_hist, tok_last, zero, nzero)))
     return e;
   const int ranges = Ep <= 1024 ? 1024 / Ep : 1;
-  if ((e = launch_dependent(layout_scan_kernel, dim3(1), dim3(1024), sizeof(int) * ((size_t)(5 + ranges) * Ep + 4), s, nblk, Ep, lv)))
+  if ((e = launch_dependent(layout_scan_kernel, dim3(1), dim3(1024), sizeof(int) * (expert_scan_ints(Ep) + (size_t)ranges * Ep), s, nblk, Ep, lv)))
     return e;
   const size_t nlast = LAYOUT_CHUNK / kp + 2;
   auto rank_smem = [&](int warps) {
-    return sizeof(int) * (2 * (size_t)Ep + nlast + (nlast & 1)) + sizeof(uint16_t) * (size_t)warps * (Ep + (Ep & 1));
+    return sizeof(int) * (3 * (size_t)Ep + nlast + 1) + sizeof(uint16_t) * (size_t)warps * (Ep + (Ep & 1));
   };
   // as many warps as have room for their histograms in 48 KB of shared memory (32 up to about 500 experts)
   constexpr size_t ROOM = 48 * 1024;

@@ -16,7 +16,7 @@
 //
 // Events (Section 4.3).  Per M-block (128 rows of the padded expert-ordered row space) three
 // counters with static thresholds:
-//   gathered   += 1 per gather sub-task (4 rows)                  threshold GATHER_SUB
+//   gathered   += 1 per gather task (4 rows)                      threshold: its rows up to the expert's last 32-row group / 4
 //   activated  += 1 per epilogue warp and column tile of phase 0  threshold SIG * column tiles
 //   done       += 1 per epilogue warp and column tile of the last row-space phase (down / gate_grad)
 // A phase-0 item depends on `gathered` of its M-blocks, a down / gate_grad item and a w1_grad
@@ -41,11 +41,12 @@
 namespace moe {
 
 constexpr int SCHED_MAX_SEG = 4;       // phases of a pass
-constexpr int GATHER_SUB = 32;         // vector sub-tasks per M-block gather (4 rows each: the first M-blocks of a
-                                       // launch, which every CTA pair waits for, are complete after a few microseconds)
+constexpr int GROUP_ROWS = 32;         // an expert's rows are gathered (and multiplied) up to a multiple of this
+constexpr int GATHER_ROWS = 4;         // rows of a gather task: the first M-blocks of a launch, which every CTA pair
+                                       // waits for, are complete after a few microseconds
+constexpr int GATHER_SUB = GROUP_ROWS / GATHER_ROWS;   // gather tasks per row group
 constexpr int EPI_WARPS = 8;           // epilogue warps per CTA: two per quarter of the accumulator rows
 constexpr int SIG = 2 * EPI_WARPS;     // signals per (M-block, column tile): every epilogue warp of the pair
-constexpr int COMBINE_TOKENS = 1;      // tokens per combine task
 
 enum VecOp : int { VEC_GATHER = 0, VEC_DW = 2, VEC_COMBINE = 3 };
 
@@ -123,8 +124,13 @@ struct ChainParams {
   int merges[SCHED_MAX_SEG];    // row-space phases: 1 if the phase merges the last two units of odd experts
   int dep_extra;                // test hook: added to the `activated` threshold (> 0 = never reached)
   int want_dw;                  // backward: routing-weight-gradient tasks are part of the vector queue
+  int combine_split;            // combine tasks per token (column chunks)
 };
-MOE_HD int thr_gathered() { return GATHER_SUB; }
+// Gather tasks of M-block `rel` (relative to its expert's first) of an expert with `rows` rows.
+MOE_HD int thr_gathered(int rows, int rel) {
+  const int left = ((rows + GROUP_ROWS - 1) & ~(GROUP_ROWS - 1)) - rel * 128;
+  return (left < 128 ? left : 128) / GATHER_ROWS;
+}
 MOE_HD int thr_activated(const ChainParams& cp) { return SIG * cp.ntn[0] + cp.dep_extra; }
 MOE_HD int thr_done(const ChainParams& cp) { return SIG * cp.ntn[cp.is_bwd ? 2 : 1]; }
 
@@ -152,8 +158,9 @@ MOE_HD int phase_wait_kind(const ChainParams& cp, int phase) {
   if (!cp.is_bwd) return phase == 0 ? CTR_GATHERED : CTR_ACTIVATED;
   return (phase == 0 || phase == 1) ? CTR_GATHERED : CTR_ACTIVATED;
 }
-MOE_HD int phase_wait_thr(const ChainParams& cp, int phase) {
-  return phase_wait_kind(cp, phase) == CTR_GATHERED ? thr_gathered() : thr_activated(cp);
+// threshold of M-block `rel` of an expert with `rows` rows
+MOE_HD int phase_wait_thr(const ChainParams& cp, int phase, int rows, int rel) {
+  return phase_wait_kind(cp, phase) == CTR_GATHERED ? thr_gathered(rows, rel) : thr_activated(cp);
 }
 MOE_HD int phase_trigger_kind(const ChainParams& cp, int phase) {
   if (!cp.is_bwd) return phase == 0 ? CTR_ACTIVATED : CTR_DONE;
@@ -161,20 +168,29 @@ MOE_HD int phase_trigger_kind(const ChainParams& cp, int phase) {
 }
 
 // ---------------------------------------------------------------- vector queues (ticket order)
-// Two queues: the gather sub-tasks in M-block order, and behind them the tasks that consume matrix tiles
+// Two queues: the gather tasks in row order, and behind them the tasks that consume matrix tiles
 // (backward: the routing-weight gradient per M-block; then the combine tasks).  A worker leaves the first
 // queue for the second only when the first is empty -- or earlier, when it is not one of the few workers
 // that keep gathering in the background (see fused.cu).
-constexpr int GATHER_FAST_MBLOCKS = 32;   // M-blocks every vector worker helps to gather at the start of a launch
+constexpr int GATHER_FAST_TASKS = 1024;   // gather tasks every vector worker helps with at the start of a launch
 struct VecTask {
   int op;       // VecOp
-  int idx;      // gather: M-block * GATHER_SUB + sub-task; dw: M-block; combine: task (COMBINE_TOKENS tokens)
+  int idx;      // gather: row group * GATHER_SUB + sub-task; dw: M-block; combine: token position * combine_split + column chunk
 };
-MOE_HD int gather_total(int M) { return GATHER_SUB * M; }
+MOE_HD int gather_total(int groups) { return GATHER_SUB * groups; }
+MOE_HD int combine_total(const ChainParams& cp) { return cp.T * cp.combine_split; }
 MOE_HD int post_total(const ChainParams& cp, int M) {
-  int n = (cp.T + COMBINE_TOKENS - 1) / COMBINE_TOKENS;
+  int n = combine_total(cp);
   if (cp.is_bwd && cp.want_dw) n += M;
   return n;
+}
+// Column chunks of a combine task: one warp sums a token's rows of 14 KB in 15-20 us, most of it latency.  With many tokens
+// the warps hide each other's; with few, a token is cut into chunks of 64 16-byte vectors as long as no more than about two
+// tasks fall on each of the launch's vector warps.
+MOE_HD int combine_split_of(int T, int d) {
+  const int chunks = (d / 8 + 63) / 64, room = T > 0 ? 1024 / T : 1;
+  const int s = chunks < room ? chunks : room;
+  return s > 1 ? s : 1;
 }
 MOE_HD VecTask decode_post_ticket(const ChainParams& cp, int t, int M) {
   VecTask v;
