@@ -18,6 +18,7 @@
 #include "gemm_roles.cuh"
 #include "launch_pairs.cuh"
 #include "schedule.h"
+#include "topk.cuh"
 
 namespace moe {
 
@@ -25,12 +26,8 @@ constexpr int SCHED_WARP = 7;   // even CTA: scheduler of the pair; odd CTA: a v
 constexpr int VEC_WARPS = 4;
 constexpr int FUSED_THREADS = 32 * (GEMM_ROLE_WARPS + VEC_WARPS);
 
-constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
-constexpr size_t FUSED_LAYOUT_BYTES =
-    cmax(cmax(swap_layout_bytes<GEMM_GATE_UP>(), swap_layout_bytes<GEMM_DOWN>()),
-         cmax(cmax(swap_layout_bytes<GEMM_ACT_GRAD>(), swap_layout_bytes<GEMM_GATE_GRAD>()), WGRAD_LAYOUT_BYTES));
-constexpr size_t FUSED_SMEM_BYTES = 1024 + FUSED_LAYOUT_BYTES + 256 /* PipeBarriers */ + 384 /* TicketRing */;
-static_assert(FUSED_SMEM_BYTES <= 227 * 1024, "shared memory budget");
+constexpr size_t FUSED_SMEM_BYTES = 1024 + LAYOUT_BYTES + PIPE_BARRIER_BYTES + 384 /* TicketRing */;
+static_assert(WGRAD_LAYOUT_BYTES <= LAYOUT_BYTES && FUSED_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
 // ---------------------------------------------------------------- vector work (one warp per task)
 __device__ __forceinline__ uint4 ldg_nc_v4(const void* p) {
@@ -247,19 +244,21 @@ __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const Wa
 // microseconds of each other and meet in L2, however the pairs' speeds differ -- a static deal of
 // items to pairs loses that as soon as gather or combine traffic makes the pairs drift apart.
 // The scheduler warp of the even CTA takes the pair's tickets -- as soon as a ring slot is free, so up to
-// TK_RING items ahead of the epilogue -- polls the item's dependent events (one M-block per lane) and
-// only then publishes the ticket to every role of both CTAs through a small ring in shared memory:
-// ticket, decode and polls hide behind the loads of the items before it.
+// TK_RING items ahead of the epilogue -- looks at the item's dependent events (one M-block per lane) and
+// publishes the ticket to every role of both CTAs through a small ring in shared memory: ticket, decode and look
+// hide behind the loads of the items before it.  If the events are not met yet, whoever loads what they stand for waits for
+// them (the token loader; both loaders of a weight gradient): the weights, which depend on nothing, are under way meanwhile.
 constexpr int TK_RING = 4;
 // A published item: the ticket and the decoded work (decoding takes a chain of dependent global loads; the
 // scheduler does it once, ahead of time, for every role of both CTAs).
 struct __align__(16) WorkDesc {
   int ticket;                                  // -1: the queue is empty
-  int phase, item, merged;
+  int phase, item, flags;                      // WD_MERGED, WD_READY
   int e, n0, nb, nkb;                          // strips: nb = 256-row block of dW
   int a_row0, a_ntok, a_mb_first, a_mb_count;  // strips: a_row0 = first padded row, a_ntok = rows of the expert
   int b_row0, b_ntok, b_mb_first, b_mb_count;
 };
+constexpr int WD_MERGED = 1, WD_READY = 2;   // READY: the dependent events were met when the item was published
 static_assert(sizeof(WorkDesc) == 64, "published as four 16-byte stores");
 struct __align__(16) TicketRing {
   WorkDesc work[TK_RING];
@@ -293,7 +292,7 @@ __device__ __forceinline__ bool ring_take(TicketRing* r, uint32_t n, WorkDesc* w
 }
 __device__ __forceinline__ SwapWork desc_swap_work(const WorkDesc& wd) {
   SwapWork w;
-  w.merged = wd.merged != 0;
+  w.merged = (wd.flags & WD_MERGED) != 0;
   w.a.e = w.b.e = wd.e; w.a.n0 = w.b.n0 = wd.n0; w.a.nb = w.b.nb = wd.nb; w.a.nkb = w.b.nkb = wd.nkb;
   w.a.row0 = wd.a_row0; w.a.ntok = wd.a_ntok; w.a.mb_first = wd.a_mb_first; w.a.mb_count = wd.a_mb_count;
   w.b.row0 = wd.b_row0; w.b.ntok = wd.b_ntok; w.b.mb_first = wd.b_mb_first; w.b.mb_count = wd.b_mb_count;
@@ -306,7 +305,7 @@ __device__ __forceinline__ Strip desc_strip(const WorkDesc& wd) {
   return st;
 }
 __device__ __forceinline__ void pack_swap_work(WorkDesc& wd, const SwapWork& w) {
-  wd.merged = w.merged ? 1 : 0;
+  wd.flags = w.merged ? WD_MERGED : 0;
   wd.e = w.a.e; wd.n0 = w.a.n0; wd.nb = w.a.nb; wd.nkb = w.a.nkb;
   wd.a_row0 = w.a.row0; wd.a_ntok = w.a.ntok; wd.a_mb_first = w.a.mb_first; wd.a_mb_count = w.a.mb_count;
   wd.b_row0 = w.b.row0; wd.b_ntok = w.b.ntok; wd.b_mb_first = w.b.mb_first; wd.b_mb_count = w.b.mb_count;
@@ -318,7 +317,7 @@ __device__ __forceinline__ void decode_item(const FusedArgs& fa, int phase, int 
   if (strip) {
     const GemmArgs& a = fa.op[phase];
     const Strip st = decode_strip(a, item);
-    wd.merged = 0; wd.e = st.e; wd.n0 = 0; wd.nb = st.mp; wd.nkb = st.nkb;
+    wd.flags = 0; wd.e = st.e; wd.n0 = 0; wd.nb = st.mp; wd.nkb = st.nkb;
     wd.a_row0 = st.row0; wd.a_ntok = st.rows; wd.a_mb_first = a.mb_start[st.e];
     wd.a_mb_count = a.mb_start[st.e + 1] - a.mb_start[st.e];
     wd.b_row0 = wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
@@ -397,7 +396,12 @@ __device__ __forceinline__ bool load_item(const FusedArgs& fa, const WorkDesc& w
                                           LoaderState& ls, bool second_warp, int rank, int lane, const WaitCtl& wc,
                                           const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
-  if (BWD && (phase == 1 || phase == 3))
+  const bool strip = BWD && (phase == 1 || phase == 3);
+  if (!(wd.flags & WD_READY) && (second_warp || strip)) {   // the item's dependent events (Section 4.3)
+    const int first = wd.a_mb_first, count = strip && wd.nkb == 0 ? 0 : wd.a_mb_count + wd.b_mb_count;
+    if (!dep.wait(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane, t)) return false;
+  }
+  if (strip)
     return wgrad_load_strip(fa.op[phase], smem, bars, ls, second_warp, rank, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
@@ -445,15 +449,14 @@ template <bool BWD>
 __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __grid_constant__ FusedArgs fa) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + FUSED_LAYOUT_BYTES);
-  static_assert(sizeof(PipeBarriers) <= 256 && sizeof(TicketRing) <= 384, "shared-memory bookkeeping");
-  TicketRing* ring = reinterpret_cast<TicketRing*>(reinterpret_cast<uint8_t*>(bars) + 256);
+  PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + LAYOUT_BYTES);
+  static_assert(sizeof(PipeBarriers) <= PIPE_BARRIER_BYTES && sizeof(TicketRing) <= 384, "shared-memory bookkeeping");
+  TicketRing* ring = reinterpret_cast<TicketRing*>(reinterpret_cast<uint8_t*>(bars) + PIPE_BARRIER_BYTES);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   const WaitCtl wc{fa.status, fa.budget_ns};
   const TraceCtl tr{fa.trace, fa.trace_cap, fa.ctr + CTR_TRACE_CURSOR};
-  const int M = fa.lv.meta[0];
 
   if (threadIdx.x == 0) {
     pipe_init(bars);
@@ -473,6 +476,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   cluster_sync_all();  // both CTAs' barriers exist before anyone signals across the pair
   tc_fence_after_sync();
   const uint32_t tmem_base = uniform(bars->tmem_base);
+  pdl_wait();   // the layout's tables, and everything else in front of this launch
+  const int M = fa.lv.meta[0];
 
   if (warp == SCHED_WARP && rank == 0) {
     // ------------------------------------------------ scheduler of the pair (even CTA)
@@ -491,7 +496,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       wd.ticket = t;
       if (t >= total) {
         wd.ticket = -1;
-        wd.phase = wd.item = wd.merged = wd.e = wd.n0 = wd.nb = wd.nkb = 0;
+        wd.phase = wd.item = wd.flags = wd.e = wd.n0 = wd.nb = wd.nkb = 0;
         wd.a_row0 = wd.a_ntok = wd.a_mb_first = wd.a_mb_count = wd.b_row0 = wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
         if (lane == 0) ring_publish(ring, n, wd);
         break;
@@ -504,7 +509,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (tr.buf && lane == 0) t0 = globaltimer_ns();
       int first, count;
       decode_item<BWD>(fa, wd.phase, wd.item, wd, &first, &count);
-      if (!dep.wait(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane, t)) break;   // the item's dependent events (Section 4.3)
+      if (dep.met(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane)) wd.flags |= WD_READY;
       if (lane == 0) {
         const uint64_t td = tr.buf ? globaltimer_ns() : 0;
         ring_publish(ring, n, wd);
@@ -524,8 +529,15 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (!ok || wd.ticket < 0) break;
       const int phase = wd.phase;
       const ChainDeps dep = phase_deps(fa, phase, wc, tr);
-      // ---- phase boundary (see phase_wait): staging and operand ring of the new phase overlap the old ones
-      if (phase != cur_phase) {
+      if (!BWD && phase != cur_phase) {
+        // the forward's two operators have one layout: the ring runs on, only the staging slots change their size
+        cur_phase = phase;
+        es.round = 0;
+        if (is_epilogue_warp(warp) && lane == 0) tma_store_wait_read();
+        __syncwarp();
+      }
+      // ---- phase boundary of the backward (see phase_wait): staging and operand ring of the new phase overlap the old ones
+      if (BWD && phase != cur_phase) {
         cur_phase = phase;
         ls.s = ls.a_s = 0;   // every stage has been consumed: the new phase's ring (of its own depth) starts at 0
         is.s = is.a_s = 0;
@@ -577,8 +589,8 @@ cudaError_t launch_fused(bool bwd, const FusedArgs& fa, int num_sms, bool cooper
   ++*launches;
   static PairLaunchState st_fwd, st_bwd;
   if (bwd)
-    return launch_on_pairs(st_bwd, fused_chain_kernel<true>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, cooperative, s);
-  return launch_on_pairs(st_fwd, fused_chain_kernel<false>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, cooperative, s);
+    return launch_on_pairs(st_bwd, fused_chain_kernel<true>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, cooperative, s, true);
+  return launch_on_pairs(st_fwd, fused_chain_kernel<false>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, cooperative, s, true);
 }
 
 }  // namespace moe

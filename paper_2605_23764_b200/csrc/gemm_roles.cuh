@@ -15,10 +15,9 @@
 
 namespace moe {
 
-constexpr int PIPE_STAGES = 5;   // row-space operators: operand stages of 16 KB of weights + 16..24 KB of tokens;
-                                 // weight gradients: 16 KB slots of the strip's A operand
+constexpr int WG_A_SLOTS = 5;    // weight gradients: 16 KB slots of the strip's A operand
 constexpr int WG_B_STAGES = 7;   // weight gradients: 16 KB stages of the streamed B operand
-constexpr int MAX_STAGES = 8;
+constexpr int MAX_STAGES = 12;   // row-space operators: see plan_ring
 
 // Warps of a GEMM CTA: 0 weight loader, 1 MMA issuer, 2-5 and 8-11 epilogue, 6 token loader, 7 left to the kernel (scheduler).
 // TMEM lanes 32 (w % 4) .. are what warp w can read.
@@ -29,7 +28,7 @@ __device__ __forceinline__ int epilogue_index(int warp) { return (warp & 3) + (w
 struct __align__(8) PipeBarriers {
   uint64_t full[MAX_STAGES];      // used in the even CTA: bytes of both CTAs' loads of the stage
   uint64_t empty[MAX_STAGES];     // in each CTA: the stage's MMAs are complete
-  uint64_t a_empty[PIPE_STAGES];  // weight gradients, in each CTA: every MMA that reads the A slot's content is complete
+  uint64_t a_empty[WG_A_SLOTS];  // weight gradients, in each CTA: every MMA that reads the A slot's content is complete
   uint64_t tmem_full[2];          // in each CTA: accumulator ready
   uint64_t tmem_empty[2];         // used in the even CTA: the epilogue warps of the pair have drained it
   uint64_t drain;
@@ -41,7 +40,7 @@ struct __align__(8) PipeBarriers {
 // Pipeline state of a role, carried from item to item (the barriers persist).  The parity to wait for is kept per
 // stage, so operators with rings of different depth can follow one another in one launch (the ring position
 // restarts at 0 at such a boundary, where every stage has been consumed).
-struct LoaderState { uint32_t s = 0, empty_par = (1u << MAX_STAGES) - 1, a_s = 0, a_ph = (1u << PIPE_STAGES) - 1; };
+struct LoaderState { uint32_t s = 0, empty_par = (1u << MAX_STAGES) - 1, a_s = 0, a_ph = (1u << WG_A_SLOTS) - 1; };
 struct IssuerState { uint32_t s = 0, full_par = 0, a_s = 0, acc_it = 0; };
 struct EpiState { uint32_t acc_it = 0, round = 0; };   // round: position in the warp's ring of staging slots
 
@@ -50,7 +49,7 @@ __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
     mbar_init(&bars->full[s], 1);
     mbar_init(&bars->empty[s], 1);
   }
-  for (int s = 0; s < PIPE_STAGES; ++s) mbar_init(&bars->a_empty[s], 1);
+  for (int s = 0; s < WG_A_SLOTS; ++s) mbar_init(&bars->a_empty[s], 1);
   for (int s = 0; s < 2; ++s) {
     mbar_init(&bars->tmem_full[s], 1);
     mbar_init(&bars->tmem_empty[s], 2 * EPI_WARPS);
@@ -141,6 +140,16 @@ struct ChainDeps {
       if (!counter_wait(ctr + ctr_index(first + q, wait_kind), phase_wait_thr(*cp, phase, rows, rel + q), wc, item)) ok = 0;
     return __all_sync(0xffffffffu, ok) != 0;
   }
+  // The same without waiting: are they there now?
+  __device__ __forceinline__ bool met(int first, int count, int rows, int rel, int lane) const {
+    int ok = 1;
+    for (int q = lane; q < count; q += 32) {
+      int v;
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr + ctr_index(first + q, wait_kind)) : "memory");
+      if (v < phase_wait_thr(*cp, phase, rows, rel + q)) ok = 0;
+    }
+    return __all_sync(0xffffffffu, ok) != 0;
+  }
   // One lane, after its warp's stores of the tile are complete and ordered (see the epilogue roles).
   __device__ __forceinline__ void signal(int first, int count) const {
     if (trig_kind < 0) return;
@@ -155,24 +164,27 @@ struct ChainDeps {
 // =====================================================================================================
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
-// shared memory of a phase, from the 1024-byte aligned base: weights | tokens | staging | act_grad scratch
-template <int MODE>
-__host__ __device__ constexpr size_t swap_layout_bytes() {
-  return (size_t)PIPE_STAGES * (W_STAGE_BYTES + tok_stage_bytes<MODE>()) + EPI_WARPS * sw_slots<MODE>() * sw_slot_bytes<MODE>() +
-         (MODE == GEMM_ACT_GRAD ? EPI_WARPS * SW_SCRATCH_BYTES : 0);
+// Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes] |
+// staging | act_grad scratch, all of it within LAYOUT_BYTES.  An expert holds at most T rows, so a tile of T <= 256 tokens needs
+// n32(T) / 2 rows per CTA and nothing merges; beyond, a merged item (128 + 256) / 2.  What the token stages do not need
+// goes into more stages: with 32 tokens eleven, 198 KB of weights in flight instead of 80 -- a pass over few tokens is a
+// stream of weights from HBM.
+constexpr size_t PIPE_BARRIER_BYTES = 384;
+constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - 384 /* TicketRing of the persistent launch */;
+__host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) {
+  return EPI_WARPS * ((size_t)sw_staging_bytes(mode) + (mode == GEMM_ACT_GRAD ? SW_SCRATCH_BYTES : 0));
 }
-
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
 // tokens.
 template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
                                                bool tok_warp, int rank, int lane, const SwapWork& wk, int t,
                                                const WaitCtl& wc, const DEP& dep) {
-  constexpr int TOKB = tok_stage_bytes<MODE>();
-  uint8_t* sW = smem;                                    // [PIPE_STAGES][16 KB] weights
-  uint8_t* sT = smem + PIPE_STAGES * W_STAGE_BYTES;      // [PIPE_STAGES][TOKB] tokens (this CTA's half)
-  // with events: the item was published only after its dependent events were met (acquired by the scheduler,
-  // handed on through the ticket ring); what the producers wrote must be seen by the TMA loads
+  const int stages = a.stages, tokb = a.tok_bytes;
+  uint8_t* sW = smem;                              // [stages][16 KB] weights
+  uint8_t* sT = smem + stages * W_STAGE_BYTES;     // [stages][tokb] tokens (this CTA's half)
+  // with events: the tokens are there (acquired by the scheduler and handed on through the ticket ring, or by the caller);
+  // what the producers wrote must be seen by the TMA loads
   if (DEP::kOn && tok_warp) fence_proxy_async();
   const int nkb = uniform(wk.a.nkb), e = uniform(wk.a.e), n0 = uniform(wk.a.n0);
   const int row_a = uniform(wk.a.row0), half_a = uniform(wk.a.ntok) >> 1;
@@ -183,11 +195,11 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem,
     if (!tok_warp) {
       load_weights_swap<MODE>(a, e, n0, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], 2 * (half_a + half_b));
     } else {
-      load_tokens_swap(a, row_a, half_a, kb, rank, sT + ls.s * TOKB, &bars->full[ls.s]);
+      load_tokens_swap(a, row_a, half_a, kb, rank, sT + ls.s * tokb, &bars->full[ls.s]);
       if (half_b)   // the second token tile, behind the first in the stage
-        load_tokens_swap(a, row_b, half_b, kb, rank, sT + ls.s * TOKB + half_a * (BK * 2), &bars->full[ls.s]);
+        load_tokens_swap(a, row_b, half_b, kb, rank, sT + ls.s * tokb + half_a * (BK * 2), &bars->full[ls.s]);
     }
-    if (++ls.s == PIPE_STAGES) ls.s = 0;
+    if (++ls.s == (uint32_t)stages) ls.s = 0;
   }
   return true;
 }
@@ -198,10 +210,10 @@ template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
                                                 IssuerState& is, const SwapWork& wk, int t, const WaitCtl& wc,
                                                 const DEP& dep) {
-  constexpr int TOKB = tok_stage_bytes<MODE>();
+  const uint32_t stages = a.stages, t_step = a.tok_bytes >> 4;
   const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
-  const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + PIPE_STAGES * W_STAGE_BYTES), 16);
-  uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * (TOKB >> 4);
+  const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + stages * W_STAGE_BYTES), 16);
+  uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * t_step;
   const int as = is.acc_it & 1;
   const int nkb = uniform(wk.a.nkb), ntok = uniform(wk.a.ntok), ntok_b = uniform(wk.merged ? wk.b.ntok : 0);
   if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
@@ -220,10 +232,10 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem
     mma_kblock_swap<MODE>(d_tmem, w_lo, t_lo, idesc, kb == 0);
     if (ntok_b) mma_kblock_swap<MODE>(d_tmem_b, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
     tc_commit_pair(&bars->empty[is.s]);   // frees the stage in both CTAs
-    if (++is.s == PIPE_STAGES) {
+    if (++is.s == stages) {
       is.s = 0; w_lo = w_lo0; t_lo = t_lo0;
     } else {
-      w_lo += W_STAGE_BYTES >> 4; t_lo += TOKB >> 4;
+      w_lo += W_STAGE_BYTES >> 4; t_lo += t_step;
     }
   }
   tc_commit_pair(&bars->tmem_full[as]);  // accumulator slices ready in both CTAs
@@ -243,8 +255,8 @@ template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
                                                    uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                    const SwapWork& wk, int t, const WaitCtl& wc, const DEP& dep) {
-  constexpr int WARPB = sw_slots<MODE>() * sw_slot_bytes<MODE>();
-  uint8_t* sOut = smem + PIPE_STAGES * (W_STAGE_BYTES + tok_stage_bytes<MODE>());
+  constexpr int WARPB = sw_staging_bytes((GemmMode)MODE);
+  uint8_t* sOut = smem + a.stages * (W_STAGE_BYTES + a.tok_bytes);
   SwStaging sg{sOut + ew * WARPB, es.round, sOut + EPI_WARPS * WARPB + ew * SW_SCRATCH_BYTES};
   bool ok = true;
   for (int part = 0; part < (wk.merged ? 2 : 1); ++part) {   // a merged item is two consecutive tiles here
@@ -287,9 +299,9 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
 // With K of only four or five k-blocks a column tile lasts about as long as the latency of its B loads, so the
 // B ring is deeper than one tile (WG_B_STAGES): the loads of tile i + 1 are in flight while tile i multiplies.
 // The staging of the epilogue is what pays for it: one 4 KB box of 32 rows x 64 columns per warp.
-constexpr int A_RES_KB = PIPE_STAGES;        // k-blocks of A that can stay resident
+constexpr int A_RES_KB = WG_A_SLOTS;         // k-blocks of A that can stay resident
 constexpr size_t WGRAD_LAYOUT_BYTES =
-    (size_t)PIPE_STAGES * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES + EPI_WARPS * OUT_BOX_BYTES;
+    (size_t)WG_A_SLOTS * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES + EPI_WARPS * OUT_BOX_BYTES;
 
 // Epilogue of one 128 x 256 accumulator slice of a weight gradient (or zeros for an expert without rows): warps `quad`
 // and `quad + 4` store 32 rows, 64 columns at a time in turn, each through a staging box of its own.
@@ -349,8 +361,8 @@ template <class DEP>
 __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
                                                  bool b_warp, int rank, int lane, const Strip& st, int sp,
                                                  const WaitCtl& wc, const DEP& dep) {
-  uint8_t* sA = smem;                                   // [PIPE_STAGES][16 KB] A slots
-  uint8_t* sB = smem + PIPE_STAGES * A_STAGE_BYTES;     // [WG_B_STAGES][16 KB] B stages
+  uint8_t* sA = smem;                                   // [WG_A_SLOTS][16 KB] A slots
+  uint8_t* sB = smem + WG_A_SLOTS * A_STAGE_BYTES;     // [WG_B_STAGES][16 KB] B stages
   const int m0 = uniform(st.m0(rank)), row0 = uniform(st.row0), nkb = uniform(st.nkb);
   const bool resident = nkb <= A_RES_KB;
   if (DEP::kOn) fence_proxy_async();   // as in swap_load_item
@@ -373,7 +385,7 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
       }
       ls.empty_par ^= 1u << ls.s;
       if (load_a) ls.a_ph ^= 1u << slot;
-      if (!resident && ++ls.a_s == PIPE_STAGES) ls.a_s = 0;
+      if (!resident && ++ls.a_s == WG_A_SLOTS) ls.a_s = 0;
       if (++ls.s == WG_B_STAGES) ls.s = 0;
     }
   }
@@ -385,7 +397,7 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
                                                   IssuerState& is, const Strip& st, int sp, const WaitCtl& wc,
                                                   const DEP& dep) {
   const uint32_t a_lo0 = smem_desc_lo(smem_u32(smem), MN_BOX_BYTES);
-  const uint32_t b_lo0 = smem_desc_lo(smem_u32(smem + PIPE_STAGES * A_STAGE_BYTES), MN_BOX_BYTES);
+  const uint32_t b_lo0 = smem_desc_lo(smem_u32(smem + WG_A_SLOTS * A_STAGE_BYTES), MN_BOX_BYTES);
   constexpr uint32_t idesc = make_idesc_bf16(2 * BLOCK_M, BN, 1, 1), hi = smem_desc_hi(1024);
   constexpr int KSTEP = 2048 >> 4;   // 16 k-rows of an MN-major box
   const int nkb = uniform(st.nkb), rows = uniform(st.rows);
@@ -416,7 +428,7 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
       }
       tc_commit_pair(&bars->empty[is.s]);
       if (last_use) tc_commit_pair(&bars->a_empty[slot]);
-      if (!resident && ++is.a_s == PIPE_STAGES) is.a_s = 0;
+      if (!resident && ++is.a_s == WG_A_SLOTS) is.a_s = 0;
       if (++is.s == WG_B_STAGES) is.s = 0;
     }
     tc_commit_pair(&bars->tmem_full[as]);
@@ -430,7 +442,7 @@ template <class DEP>
 __device__ __forceinline__ bool wgrad_epilogue_strip(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
                                                      uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                      const Strip& st, int sp, const WaitCtl& wc, const DEP& dep) {
-  uint8_t* box = smem + PIPE_STAGES * A_STAGE_BYTES + WG_B_STAGES * HALF_B_BYTES + ew * OUT_BOX_BYTES;
+  uint8_t* box = smem + WG_A_SLOTS * A_STAGE_BYTES + WG_B_STAGES * HALF_B_BYTES + ew * OUT_BOX_BYTES;
   Tile tl;
   tl.e = st.e; tl.row0 = st.row0; tl.m0 = st.m0(rank); tl.nkb = st.nkb;
   const bool idle = tl.m0 >= a.M;   // the strip's second half lies outside dW: nothing to store

@@ -54,10 +54,6 @@ struct SwapWork {
 };
 template <int MODE>
 __host__ __device__ constexpr bool swap_merges() { return MODE == GEMM_DOWN || MODE == GEMM_GATE_GRAD; }
-// token bytes of a stage per CTA: up to 128 rows, or (128 + 256) / 2 rows of a merged item
-template <int MODE>
-__host__ __device__ constexpr int tok_stage_bytes() { return (swap_merges<MODE>() ? 3 : 2) * 64 * BK * 2; }
-
 template <int MODE>
 __device__ __forceinline__ int total_swap_work(const GemmArgs& a) {
   return (swap_merges<MODE>() ? a.meta[4] : a.meta[3]) * a.n_tiles_n;
@@ -136,14 +132,20 @@ __device__ __forceinline__ uint32_t swap_idesc(int ntok) {
 }
 
 // ---------------------------------------------------------------- staging ring of an epilogue warp
-// Tokens per staging slot, bytes of a slot, slots per warp.  gate+up: A, H gate, H up of 16 features each; act_grad: d(gate) and
-// d(up) of 32 features; down, gate_grad: 32 features.  What is left of the 227 KB beside the operand ring decides.
+// Tokens per staging slot, bytes of a slot, slots per warp.  gate+up: A and, if they are kept, H gate and H up of 16 features
+// each; act_grad: d(gate) and d(up) of 32 features; down, gate_grad: 32 features.
 template <int MODE>
 __host__ __device__ constexpr int sw_chunk() { return MODE == GEMM_GATE_UP ? 32 : 16; }
 template <int MODE>
-__host__ __device__ constexpr int sw_slot_bytes() { return MODE == GEMM_GATE_UP ? 3072 : MODE == GEMM_ACT_GRAD ? 2048 : 1024; }
+__device__ __forceinline__ int sw_slot_bytes(const GemmArgs& a) {
+  return MODE == GEMM_GATE_UP ? (a.save_h ? 3072 : 1024) : MODE == GEMM_ACT_GRAD ? 2048 : 1024;
+}
 template <int MODE>
-__host__ __device__ constexpr int sw_slots() { return MODE == GEMM_DOWN || MODE == GEMM_GATE_GRAD ? 3 : 2; }
+__device__ __forceinline__ uint32_t sw_slots(const GemmArgs& a) {
+  return MODE == GEMM_GATE_UP ? (a.save_h ? 1 : 3) : MODE == GEMM_ACT_GRAD ? 2 : 3;
+}
+// staging bytes of a warp: the same for gate+up and down, which share one layout in the persistent forward launch
+__host__ __device__ constexpr int sw_staging_bytes(GemmMode mode) { return mode == GEMM_ACT_GRAD ? 4096 : 3072; }
 constexpr int SW_SCRATCH_BYTES = 4096;   // act_grad, per warp: saved pre-activations, two halves of [gate | up][16 tokens][32 features]
 struct SwStaging {
   uint8_t* base;     // this warp's slots
@@ -151,11 +153,16 @@ struct SwStaging {
   uint8_t* scratch;  // act_grad
 };
 template <int MODE>
-__device__ __forceinline__ uint8_t* sw_acquire(SwStaging& sg, int lane) {
-  if (lane == 0) tma_store_wait_read_n<sw_slots<MODE>() - 1>();   // the slot's previous stores have read it
+__device__ __forceinline__ uint8_t* sw_acquire(const GemmArgs& a, SwStaging& sg, int lane) {
+  const uint32_t slots = sw_slots<MODE>(a);
+  if (lane == 0) {   // the slot's previous stores have read it
+    if (slots == 1) tma_store_wait_read();
+    else if (slots == 2) tma_store_wait_read_n<1>();
+    else tma_store_wait_read_n<2>();
+  }
   __syncwarp();
-  uint8_t* slot = sg.base + sg.round * sw_slot_bytes<MODE>();
-  if (++sg.round == sw_slots<MODE>()) sg.round = 0;
+  uint8_t* slot = sg.base + sg.round * sw_slot_bytes<MODE>(a);
+  if (++sg.round == slots) sg.round = 0;
   return slot;
 }
 __device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
@@ -187,7 +194,7 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
       float v[16];
       tmem_ld16(trow + c0, v);
       tmem_ld_wait();
-      uint8_t* box = sw_acquire<MODE>(sg, lane);
+      uint8_t* box = sw_acquire<MODE>(a, sg, lane);
       // [16 tokens][32 features].  Neighbouring lanes (features 2i, 2i+1) swap one value per token pair, so that
       // every lane stores 4 bytes: the even lane the feature pair of token j, the odd lane that of token j+1 -- 128
       // contiguous bytes per warp store instead of 64.
@@ -222,7 +229,7 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
       const float wl = w_next;   // routing weight of token c0 + lane; the next chunk's is on its way
       if (c0 + 2 * CH < st.ntok) w_next = a.prow_w[st.row0 + c0 + 2 * CH + lane];
       tmem_ld_wait();
-      uint8_t* box = sw_acquire<MODE>(sg, lane);
+      uint8_t* box = sw_acquire<MODE>(a, sg, lane);
       uint16_t* abox = reinterpret_cast<uint16_t*>(box);           // A: [32 tokens][16 features]
       uint16_t* hbox = reinterpret_cast<uint16_t*>(box + 1024 + (hi ? 1024 : 0));   // H gate / H up
 #pragma unroll
@@ -282,7 +289,7 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
     int half = 0;
 #pragma unroll 1
     for (int h0 = first; h0 < st.ntok; h0 += 2 * CH) {
-      uint8_t* box = sw_acquire<MODE>(sg, lane);
+      uint8_t* box = sw_acquire<MODE>(a, sg, lane);
       const float wl = w_next;
       uint8_t* scr = sg.scratch + half;
       half ^= 2048;

@@ -10,11 +10,8 @@
 
 namespace moe {
 
-template <int MODE>
-__host__ __device__ constexpr size_t gemm3_smem_bytes() { return 1024 + swap_layout_bytes<MODE>() + sizeof(PipeBarriers); }
-static_assert(gemm3_smem_bytes<GEMM_GATE_UP>() <= 227 * 1024 && gemm3_smem_bytes<GEMM_DOWN>() <= 227 * 1024 &&
-                  gemm3_smem_bytes<GEMM_ACT_GRAD>() <= 227 * 1024 && gemm3_smem_bytes<GEMM_GATE_GRAD>() <= 227 * 1024,
-              "shared memory budget");
+constexpr size_t GEMM3_SMEM_BYTES = 1024 + LAYOUT_BYTES + PIPE_BARRIER_BYTES;
+static_assert(sizeof(PipeBarriers) <= PIPE_BARRIER_BYTES && GEMM3_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
 constexpr int GEMM3_THREADS = 32 * GEMM_ROLE_WARPS;
 
@@ -22,7 +19,7 @@ template <int MODE>
 __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(const __grid_constant__ GemmArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + swap_layout_bytes<MODE>());
+  PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + LAYOUT_BYTES);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
@@ -89,10 +86,18 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   }
 }
 
+void plan_ring(GemmMode mode, int T, GemmArgs& a) {
+  const bool merges = mode == GEMM_DOWN || mode == GEMM_GATE_GRAD || mode == GEMM_GATE_UP;   // gate+up: laid out like down
+  const int n32 = (T + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN;
+  a.tok_bytes = T <= 256 ? n32 / 2 * BK * 2 : (merges ? 3 : 2) * 64 * BK * 2;
+  a.stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + a.tok_bytes));
+  if (a.stages > MAX_STAGES) a.stages = MAX_STAGES;
+}
+
 template <int MODE>
 static cudaError_t launch_swap_mode(const GemmArgs& a, int num_sms, cudaStream_t s) {
   static PairLaunchState st;
-  return launch_on_pairs(st, grouped_gemm_swap_kernel<MODE>, a, GEMM3_THREADS, gemm3_smem_bytes<MODE>(), num_sms,
+  return launch_on_pairs(st, grouped_gemm_swap_kernel<MODE>, a, GEMM3_THREADS, GEMM3_SMEM_BYTES, num_sms,
                          false, s);
 }
 

@@ -112,6 +112,9 @@ struct GemmArgs {
   int M;               // WGRAD: rows of dW per expert
   int b_rows_per_expert;  // rows of the B tensor map per expert slab
   int F;               // intermediate size (GATE_UP / ACT_GRAD epilogues)
+  // row-space modes: shared memory of the operator (gemm_roles.cuh, plan_ring)
+  int stages;          // operand stages
+  int tok_bytes;       // token bytes of a stage per CTA
   // epilogue tensors
   int save_h;          // GATE_UP: also store the pre-activations H
   const uint16_t* in0; // ACT_GRAD: H
@@ -122,6 +125,8 @@ struct GemmArgs {
   uint64_t budget_ns;
 };
 
+// Shared-memory plan of a row-space operator for calls of T tokens: fills stages and tok_bytes.
+void plan_ring(GemmMode mode, int T, GemmArgs& a);
 // ---- gemm_tc3.cu: the row-space operators with the tokens as accumulator COLUMNS (weights take the
 // 256 accumulator rows of a CTA pair), so a tile's MMA time follows the expert's real token count
 cudaError_t launch_gemm3(GemmMode mode, const GemmArgs& a, int num_sms, cudaStream_t s, int* launches);
