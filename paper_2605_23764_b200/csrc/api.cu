@@ -146,7 +146,7 @@ struct Carve {
 // Byte offsets of every workspace tensor.
 struct WsPlan {
   size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, pair_start, pblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, group_start, group_row, group_slot, prow_w,
-      dw_partial, Xp, H, A, Y, dOutp, dH, st_x, st_dout, st_ids, st_w, st_out, st_dx, st_dw, st_logits, ctr, trace, total;
+      dw_partial, Xp, H, A, Y, dOutp, dH, st_x[2], st_dout, st_ids, st_w, st_out, st_dx, st_dw, st_logits, ctr, trace, total;
   int cap_rows, nblk_max, ntn_act, ctr_count, trace_cap;
 };
 
@@ -189,7 +189,7 @@ WsPlan plan_workspace(const moe_shape& s) {
   p.Y = c.take(2 * cap * s.d);
   p.dOutp = c.take(train ? 2 * cap * s.d : 0);
   p.dH = c.take(train ? 2 * cap * 2 * s.F : 0);
-  p.st_x = c.take(2 * (size_t)s.T_max * s.d);
+  for (int i = 0; i < 2; ++i) p.st_x[i] = c.take(2 * (size_t)s.T_max * s.d);   // the next call's arrives while this call reads its own
   p.st_dout = c.take(train ? 2 * (size_t)s.T_max * s.d : 0);
   p.st_ids = c.take(sizeof(int) * (size_t)s.T_max * s.k);
   p.st_w = c.take(sizeof(float) * (size_t)s.T_max * s.k);
@@ -229,10 +229,12 @@ struct moe_ctx {
   // call still computes) and a copy-out stream (the result leaves in token chunks behind the combine)
   bool copy_ready = false;
   cudaStream_t h2d_stream = nullptr, d2h_stream = nullptr;
-  cudaEvent_t ev_x_free = nullptr, ev_dout_free = nullptr, ev_h2d_done = nullptr, ev_d2h_done = nullptr, ev_out_done = nullptr;
+  cudaEvent_t ev_x_free[2] = {}, ev_dout_free = nullptr, ev_fwd_start = nullptr, ev_h2d_done = nullptr, ev_d2h_done = nullptr, ev_out_done = nullptr;
   bool out_pending = false;   // MOE_FLAG_DEFER_OUT_COPY: the copy of the last forward's result may still be running
   cudaEvent_t ev_chunk[HOST_CHUNKS] = {};
-  bool x_used = false, dout_used = false;
+  bool host_fwd = false;      // the last forward was a host-buffer call: ev_fwd_start is its
+  int x_turn = 0;             // x staging buffer of the next call
+  bool x_used[2] = {}, dout_used = false;   // its event says when the buffer may be overwritten
   // optional per-operator timing
   bool profiling = false;
   bool events_made = false;
@@ -497,11 +499,25 @@ int ensure_copy_streams(moe_ctx* c) {
   if (c->copy_ready) return MOE_OK;
   MOE_CUDA(cudaStreamCreateWithFlags(&c->h2d_stream, cudaStreamNonBlocking));
   MOE_CUDA(cudaStreamCreateWithFlags(&c->d2h_stream, cudaStreamNonBlocking));
-  cudaEvent_t* evs[] = {&c->ev_x_free, &c->ev_dout_free, &c->ev_h2d_done, &c->ev_d2h_done, &c->ev_out_done};
+  cudaEvent_t* evs[] = {&c->ev_x_free[0], &c->ev_x_free[1], &c->ev_dout_free, &c->ev_fwd_start, &c->ev_h2d_done, &c->ev_d2h_done, &c->ev_out_done};
   for (cudaEvent_t* e : evs) MOE_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   for (int i = 0; i < HOST_CHUNKS; ++i) MOE_CUDA(cudaEventCreateWithFlags(&c->ev_chunk[i], cudaEventDisableTiming));
   c->copy_ready = true;
   return MOE_OK;
+}
+
+// Device address of `n` elements of pinned (mapped) host memory; NULL for any other memory.  Both ends are looked up: a
+// buffer may reach beyond the range that was registered.
+template <class T>
+T* mapped_host(T* p, size_t n) {
+  cudaPointerAttributes a, b;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, p + n - 1) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
+  T* const first = static_cast<T*>(a.devicePointer);
+  return static_cast<T*>(b.devicePointer) == first + (n - 1) ? first : nullptr;
 }
 
 // The forward result leaves for the host: on `st`, or -- MOE_FLAG_DEFER_OUT_COPY -- on the copy-out stream behind an
@@ -555,7 +571,7 @@ int combine_and_maybe_copy_out(moe_ctx* c, const Dims& dm, const LayoutView& lv,
 }
 
 int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, const uint16_t* W1,
-            const uint16_t* W2, uint16_t* out, int T, cudaStream_t st, uint16_t* out_host = nullptr) {
+            const uint16_t* W2, uint16_t* out, int T, cudaStream_t st, uint16_t* out_host = nullptr, cudaEvent_t x_free = nullptr) {
   const WsPlan& p = c->plan;
   const Dims dm = c->dims(T);
   const LayoutView lv = c->layout();
@@ -570,11 +586,14 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
                            persistent ? p.ctr_count * (c->train() ? 2 : 1) : 0, c->status(), st, &c->launches));
     c->bwd_ctr_clear = persistent && c->train();
   }
+  if (out_host) MOE_CUDA(cudaEventRecord(c->ev_fwd_start, st));
+  c->host_fwd = out_host != nullptr;
   if (serial_mode(c)) {
     {
       Phase ph(c, MOE_PHASE_GATHER, st);
       MOE_CUDA(launch_gather(x, w, dm, lv, c->at<uint16_t>(p.Xp), c->at<float>(p.prow_w), p.cap_rows, st,
                              &c->launches, c->status(), c->budget_ns));
+      if (x_free) MOE_CUDA(cudaEventRecord(x_free, st));
     }
     {
       Phase ph(c, MOE_PHASE_GEMM_GATE_UP, st);
@@ -602,6 +621,7 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     fa.combine_out = out;
     Phase ph(c, MOE_PHASE_FUSED_FWD, st);
     MOE_CUDA(launch_fused(false, fa, c->num_sms, !c->plain_launch, st, &c->launches));
+    if (x_free) MOE_CUDA(cudaEventRecord(x_free, st));
     if (out_host && (rc = copy_out_to_host(c, out, out_host, 2 * (size_t)T * c->shape.d, st))) return rc;
   }
   if (c->train()) {
@@ -612,7 +632,7 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
 }
 
 int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t* W2, uint16_t* dx, uint16_t* dW1,
-            uint16_t* dW2, float* d_w, int T, cudaStream_t st, uint16_t* dx_host = nullptr) {
+            uint16_t* dW2, float* d_w, int T, cudaStream_t st, uint16_t* dx_host = nullptr, cudaEvent_t dout_free = nullptr) {
   const moe_shape& s = c->shape;
   const WsPlan& p = c->plan;
   const Dims dm = c->dims(T);
@@ -633,6 +653,7 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
       Phase ph(c, MOE_PHASE_BWD_GATHER, st);
       MOE_CUDA(launch_gather(dout, nullptr, dm, lv, c->at<uint16_t>(p.dOutp), nullptr, p.cap_rows, st,
                              &c->launches, c->status(), c->budget_ns));
+      if (dout_free) MOE_CUDA(cudaEventRecord(dout_free, st));
     }
     {
       Phase ph(c, MOE_PHASE_ACT_GRAD, st);
@@ -666,7 +687,6 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
       Phase ph(c, MOE_PHASE_WGRAD_GATE_UP, st);
       MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_WGRAD, args_wgrad_gate_up(c), c->num_sms, st, &c->launches));
     }
-    if (dx_host) MOE_CUDA(cudaStreamWaitEvent(st, c->ev_d2h_done, 0));  // dx_host is complete once `st` is
   } else {
     FusedArgs fa = fused_base(c, true, T);
     fa.cp = chain_params(c, true, T, d_w != nullptr);
@@ -692,21 +712,19 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     const bool early_out = wait_value && write_value;
     const CUdeviceptr ready_word = reinterpret_cast<CUdeviceptr>(fa.ctr + CTR_OUT_READY);
     fa.announce_out = early_out ? 1 : 0;
+    if (early_out) MOE_CUDA(cudaEventRecord(c->ev_chunk[0], st));   // the word is cleared before anyone waits on it
+    MOE_CUDA(launch_fused(true, fa, c->num_sms, !c->plain_launch, st, &c->launches));
+    if (dout_free) MOE_CUDA(cudaEventRecord(dout_free, st));
     if (early_out) {
-      MOE_CUDA(cudaEventRecord(c->ev_chunk[0], st));   // the word is cleared before anyone waits on it
+      // The launch and everything that sets the word are submitted before the wait for it: streams share hardware queues, and
+      // the first launch of a kernel may have to load it, so a wait in front of what ends it could hold that up for good.  A
+      // launch that gave up on an expired wait never sets the word: it is set behind the launch in every case.
+      if (write_value(st, ready_word, 1, CU_STREAM_WRITE_VALUE_DEFAULT) != CUDA_SUCCESS) return cuda_fail(cudaErrorUnknown, "cuStreamWriteValue32");
       MOE_CUDA(cudaStreamWaitEvent(c->d2h_stream, c->ev_chunk[0], 0));
       if (wait_value(c->d2h_stream, ready_word, 1, CU_STREAM_WAIT_VALUE_GEQ) != CUDA_SUCCESS) return cuda_fail(cudaErrorUnknown, "cuStreamWaitValue32");
       MOE_CUDA(cudaMemcpyAsync(dx_host, dx, 2 * (size_t)T * s.d, cudaMemcpyDeviceToHost, c->d2h_stream));
       MOE_CUDA(cudaEventRecord(c->ev_d2h_done, c->d2h_stream));
     }
-    const cudaError_t launched = launch_fused(true, fa, c->num_sms, !c->plain_launch, st, &c->launches);
-    if (early_out) {
-      // a launch that failed, or gave up on an expired wait, never sets the word: set it behind the launch so that
-      // the copy-out stream is released in every case, then make `st` cover the copy
-      if (write_value(st, ready_word, 1, CU_STREAM_WRITE_VALUE_DEFAULT) != CUDA_SUCCESS) return cuda_fail(cudaErrorUnknown, "cuStreamWriteValue32");
-      MOE_CUDA(cudaStreamWaitEvent(st, c->ev_d2h_done, 0));
-    }
-    MOE_CUDA(launched);
     if (!early_out && dx_host) {
       MOE_CUDA(cudaMemcpyAsync(dx_host, dx, 2 * (size_t)T * s.d, cudaMemcpyDeviceToHost, st));
     }
@@ -797,8 +815,10 @@ int moe_destroy(moe_ctx* c) {
     cudaStreamSynchronize(c->d2h_stream);
     cudaStreamDestroy(c->h2d_stream);
     cudaStreamDestroy(c->d2h_stream);
-    cudaEventDestroy(c->ev_x_free);
+    for (cudaEvent_t e : c->ev_x_free) cudaEventDestroy(e);
     cudaEventDestroy(c->ev_dout_free);
+    cudaEventDestroy(c->ev_fwd_start);
+    cudaEventDestroy(c->ev_out_done);
     cudaEventDestroy(c->ev_h2d_done);
     cudaEventDestroy(c->ev_d2h_done);
     for (int i = 0; i < HOST_CHUNKS; ++i) cudaEventDestroy(c->ev_chunk[i]);
@@ -863,17 +883,25 @@ int moe_route_host(moe_ctx* c, const float* logits_host, int32_t T, int32_t* top
   if (T == 0) return MOE_OK;
   const moe_shape& s = c->shape;
   const WsPlan& p = c->plan;
-  MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_logits, logits_host, sizeof(float) * (size_t)T * s.E,
-                           cudaMemcpyHostToDevice, st));
+  // Pinned buffers: the kernel reads the logits from the host and writes the result there.  4096 x 64 logits take 30 us,
+  // a copy in, the kernel and two copies out 50 us -- and a copy engine serves one copy at a time, so those waited
+  // hundreds of microseconds behind the next call's x or dout.
+  const float* logits = mapped_host(logits_host, (size_t)T * s.E);
+  int32_t* ids_out = mapped_host(topk_ids_host, (size_t)T * s.k);
+  float* w_out = mapped_host(topk_w_host, (size_t)T * s.k);
+  if (!logits) {
+    MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_logits, logits_host, sizeof(float) * (size_t)T * s.E, cudaMemcpyHostToDevice, st));
+    logits = c->at<float>(p.st_logits);
+  }
   {
     Phase ph(c, MOE_PHASE_ROUTE, st);
-    MOE_CUDA(launch_route(c->at<float>(p.st_logits), T, s.E, s.k, gate_mode(c),
-                          c->at<int32_t>(p.st_ids), c->at<float>(p.st_w), nullptr, st, &c->launches));
+    MOE_CUDA(launch_route(logits, T, s.E, s.k, gate_mode(c), ids_out ? ids_out : c->at<int32_t>(p.st_ids),
+                          w_out ? w_out : c->at<float>(p.st_w), nullptr, st, &c->launches));
   }
-  MOE_CUDA(cudaMemcpyAsync(topk_ids_host, c->ws + p.st_ids, sizeof(int) * (size_t)T * s.k, cudaMemcpyDeviceToHost,
-                           st));
-  MOE_CUDA(cudaMemcpyAsync(topk_w_host, c->ws + p.st_w, sizeof(float) * (size_t)T * s.k, cudaMemcpyDeviceToHost,
-                           st));
+  if (!ids_out)
+    MOE_CUDA(cudaMemcpyAsync(topk_ids_host, c->ws + p.st_ids, sizeof(int) * (size_t)T * s.k, cudaMemcpyDeviceToHost, st));
+  if (!w_out)
+    MOE_CUDA(cudaMemcpyAsync(topk_w_host, c->ws + p.st_w, sizeof(float) * (size_t)T * s.k, cudaMemcpyDeviceToHost, st));
   return MOE_OK;
 }
 
@@ -942,21 +970,28 @@ int moe_ffn_fwd_host(moe_ctx* c, const uint16_t* x_host, const int32_t* topk_ids
   int rc = ensure_copy_streams(c);
   if (rc) return rc;
   if ((rc = join_out_copy(c, st))) return rc;   // a deferred copy of the previous result still reads the staging buffer
-  // x goes in on the copy-in stream as soon as the previous forward has read its staging buffer:
-  // it overlaps whatever this context's earlier calls still have running on `st`
-  if (c->x_used) MOE_CUDA(cudaStreamWaitEvent(c->h2d_stream, c->ev_x_free, 0));
-  MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_x, x_host, 2 * (size_t)T * s.d, cudaMemcpyHostToDevice, c->h2d_stream));
+  // x goes in on the copy-in stream, into the staging buffer that the call before the previous one has read: it
+  // overlaps whatever this context's earlier calls still have running on `st`
+  const int turn = c->x_turn;
+  uint16_t* const x = c->at<uint16_t>(p.st_x[turn]);
+  if (c->x_used[turn]) MOE_CUDA(cudaStreamWaitEvent(c->h2d_stream, c->ev_x_free[turn], 0));
+  MOE_CUDA(cudaMemcpyAsync(x, x_host, 2 * (size_t)T * s.d, cudaMemcpyHostToDevice, c->h2d_stream));
   MOE_CUDA(cudaEventRecord(c->ev_h2d_done, c->h2d_stream));
-  MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_ids, topk_ids_host, sizeof(int) * (size_t)T * s.k, cudaMemcpyHostToDevice,
-                           st));
-  MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_w, topk_w_host, sizeof(float) * (size_t)T * s.k, cudaMemcpyHostToDevice,
-                           st));
+  const size_t n = (size_t)T * s.k;
+  const int32_t* ids_in = mapped_host(topk_ids_host, n);
+  const float* w_in = mapped_host(topk_w_host, n);
+  if (ids_in && w_in) {   // by a kernel, not behind whatever the copy engine is at (see moe_route_host)
+    MOE_CUDA(launch_pull_routing(c->at<int32_t>(p.st_ids), ids_in, c->at<float>(p.st_w), w_in, n, st, &c->launches));
+  } else {
+    MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_ids, topk_ids_host, sizeof(int) * n, cudaMemcpyHostToDevice, st));
+    MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_w, topk_w_host, sizeof(float) * n, cudaMemcpyHostToDevice, st));
+  }
   MOE_CUDA(cudaStreamWaitEvent(st, c->ev_h2d_done, 0));
-  rc = run_fwd(c, c->at<uint16_t>(p.st_x), c->at<int32_t>(p.st_ids), c->at<float>(p.st_w), W_gate_up, W_down,
-               c->at<uint16_t>(p.st_out), T, st, out_host);
+  rc = run_fwd(c, x, c->at<int32_t>(p.st_ids), c->at<float>(p.st_w), W_gate_up, W_down, c->at<uint16_t>(p.st_out), T, st,
+               out_host, c->ev_x_free[turn]);
   if (rc) return rc;
-  MOE_CUDA(cudaEventRecord(c->ev_x_free, st));
-  c->x_used = true;
+  c->x_used[turn] = true;
+  c->x_turn = turn ^ 1;
   return MOE_OK;
 }
 
@@ -973,20 +1008,22 @@ int moe_ffn_bwd_host(moe_ctx* c, const uint16_t* dout_host, const uint16_t* W_ga
   const WsPlan& p = c->plan;
   int rc = ensure_copy_streams(c);
   if (rc) return rc;
-  // dout has a staging buffer of its own and goes in on the copy-in stream: it arrives while the
-  // forward that was enqueued before this call is still computing
+  // dout has a staging buffer of its own and goes in on the copy-in stream: it arrives while the forward that was
+  // enqueued before this call computes.  Not earlier: routing and layout in front of that forward read the host's memory
+  // and their launches travel over the same link, 0.1 ms of latencies that a large copy beside them made 0.6 ms.
   if (c->dout_used) MOE_CUDA(cudaStreamWaitEvent(c->h2d_stream, c->ev_dout_free, 0));
+  if (c->host_fwd) MOE_CUDA(cudaStreamWaitEvent(c->h2d_stream, c->ev_fwd_start, 0));
   MOE_CUDA(cudaMemcpyAsync(c->ws + p.st_dout, dout_host, 2 * (size_t)T * s.d, cudaMemcpyHostToDevice, c->h2d_stream));
   MOE_CUDA(cudaEventRecord(c->ev_h2d_done, c->h2d_stream));
   MOE_CUDA(cudaStreamWaitEvent(st, c->ev_h2d_done, 0));
   rc = run_bwd(c, c->at<uint16_t>(p.st_dout), W_gate_up, W_down, c->at<uint16_t>(p.st_dx), dW_gate_up, dW_down,
-               d_topk_w_host ? c->at<float>(p.st_dw) : nullptr, T, st, dx_host);
+               d_topk_w_host ? c->at<float>(p.st_dw) : nullptr, T, st, dx_host, c->ev_dout_free);
   if (rc) return rc;
-  MOE_CUDA(cudaEventRecord(c->ev_dout_free, st));
   c->dout_used = true;
   if (d_topk_w_host)
     MOE_CUDA(cudaMemcpyAsync(d_topk_w_host, c->ws + p.st_dw, sizeof(float) * (size_t)T * s.k,
                              cudaMemcpyDeviceToHost, st));
+  MOE_CUDA(cudaStreamWaitEvent(st, c->ev_d2h_done, 0));   // dx_host is complete once `st` is
   return join_out_copy(c, st);   // the forward's deferred result is complete once this call's work on `st` is
 }
 

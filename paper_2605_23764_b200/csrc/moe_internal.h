@@ -78,6 +78,9 @@ cudaError_t launch_combine(const uint16_t* rows, const Dims& dm, const LayoutVie
 cudaError_t launch_dw_reduce(const float* partial, int nparts, const Dims& dm, const LayoutView& lv,
                              float* d_topk_w, cudaStream_t s, int* launches);
 
+// ids[n], w[n] from device addresses of pinned host memory
+cudaError_t launch_pull_routing(int* ids, const int* ids_host, float* w, const float* w_host, size_t n, cudaStream_t s, int* launches);
+
 // ---- grouped GEMMs (tcgen05 on CTA pairs)
 enum GemmMode : int {
   GEMM_GATE_UP = 0,    // H = Xp . W_gate_up[e]^T, epilogue A = w * silu(g) * u     (fwd GMM1 + SwiGLU)

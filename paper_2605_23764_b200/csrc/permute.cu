@@ -239,4 +239,22 @@ cudaError_t launch_dw_reduce(const float* partial, int nparts, const Dims& dm, c
   return cudaGetLastError();
 }
 
+// Routing results from pinned host memory.  A few hundred KB: bound by the link's latency, every word is in flight at once.
+__global__ void pull_routing_kernel(int* __restrict__ ids, const int* __restrict__ ids_host, float* __restrict__ w,
+                                    const float* __restrict__ w_host, size_t n) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int id = ids_host[i];
+  const float v = w_host[i];
+  ids[i] = id;
+  w[i] = v;
+}
+
+cudaError_t launch_pull_routing(int* ids, const int* ids_host, float* w, const float* w_host, size_t n, cudaStream_t s,
+                                int* launches) {
+  ++*launches;
+  pull_routing_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(ids, ids_host, w, w_host, n);
+  return cudaGetLastError();
+}
+
 }  // namespace moe
