@@ -65,7 +65,7 @@ EncodeTiledFn get_encode_fn() {
 // bf16 tensor of `rank` dimensions (dims[0] innermost, strides in bytes for dims 1..), 128-byte
 // swizzle, zero fill outside the tensor on loads, clipping on stores.
 int encode_tiled(CUtensorMap* tm, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-                 const uint32_t* box, bool swizzle = true) {
+                 const uint32_t* box) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) {
     g_cuda_error = "cuTensorMapEncodeTiled entry point not available";
@@ -76,7 +76,7 @@ int encode_tiled(CUtensorMap* tm, const void* base, int rank, const uint64_t* di
   for (int i = 0; i < rank; ++i) { gdim[i] = dims[i]; bx[i] = box[i]; }
   for (int i = 0; i + 1 < rank; ++i) gstr[i] = strides[i];
   CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), gdim, gstr, bx, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
@@ -97,19 +97,6 @@ int encode_2d(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, u
   return encode_tiled(tm, base, 2, dims, strides, box);
 }
 
-// Store maps of the token-column tiles: un-swizzled boxes of box_rows x box_cols.
-int encode_2d_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
-  const uint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
-  const uint32_t box[2] = {box_cols, box_rows};
-  return encode_tiled(tm, base, 2, dims, strides, box, false);
-}
-// [rows][2][F] view of a [rows][2F] matrix (gate half, up half): a column tile that ends past F is clipped instead of
-// spilling into the other half.
-int encode_halves_plain(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t F, uint32_t box_cols, uint32_t box_rows) {
-  const uint64_t dims[3] = {F, 2, rows}, strides[2] = {F * 2, 2 * F * 2};
-  const uint32_t box[3] = {box_cols, 1, box_rows};
-  return encode_tiled(tm, base, 3, dims, strides, box, false);
-}
 // Load map of W_gate_up viewed as [Ep][F/8 groups][gate | up][8 rows][d]: one box brings, for eight groups of 8
 // features, the 8 gate rows followed by the 8 up rows (8 divides every F).
 int encode_gate_up_rows(CUtensorMap* tm, const void* base, uint64_t Ep, uint64_t F, uint64_t d) {
@@ -252,9 +239,8 @@ struct moe_ctx {
   const void* w2_ptr = nullptr;
   CUtensorMap tm_W1_gu, tm_W2_k128, tm_W1_mn, tm_W2_mn;
   // store maps: workspace tensors (fixed) and the caller's weight gradients (re-encoded on change)
-  // token operands with boxes of 16 .. 128 rows, un-swizzled store maps
+  // token operands with boxes of 16 .. 128 rows
   CUtensorMap tk_Xp[8], tk_A[8], tk_dOutp[8], tk_dH[8];
-  CUtensorMap tp_A, tp_H, tp_Y, tp_dH;
   const void* dw1_ptr = nullptr;
   const void* dw2_ptr = nullptr;
   CUtensorMap ts_dW1, ts_dW2;
@@ -357,9 +343,8 @@ GemmArgs args_gate_up(const moe_ctx* c, int T) {
   g.K = s.d;
   g.N = s.F;
   g.b_rows_per_expert = 2 * s.F;
-  g.tmOut0 = c->tp_A;
-  g.tmOut1 = c->tp_H;
-  g.save_h = c->train() ? 1 : 0;
+  g.out0 = c->at<uint16_t>(c->plan.A);
+  g.out1 = c->train() ? c->at<uint16_t>(c->plan.H) : nullptr;
   g.prow_w = c->at<float>(c->plan.prow_w);
   return g;
 }
@@ -374,7 +359,7 @@ GemmArgs args_down(const moe_ctx* c, int T) {
   g.K = s.F;
   g.N = s.d;
   g.b_rows_per_expert = s.d;
-  g.tmOut0 = c->tp_Y;
+  g.out0 = c->at<uint16_t>(c->plan.Y);
   return g;
 }
 // act_grad + SwiGLU_grad (+ routing-weight gradient partials)
@@ -389,7 +374,7 @@ GemmArgs args_act_grad(const moe_ctx* c, int T, bool want_dw) {
   g.K = s.d;
   g.N = s.F;
   g.b_rows_per_expert = s.d;
-  g.tmOut0 = c->tp_dH;
+  g.out0 = c->at<uint16_t>(p.dH);
   g.in0 = c->at<uint16_t>(p.H);
   g.ld_in0 = 2 * s.F;
   g.prow_w = c->at<float>(p.prow_w);
@@ -420,7 +405,7 @@ GemmArgs args_gate_grad(const moe_ctx* c, int T) {
   g.K = 2 * s.F;
   g.N = s.d;
   g.b_rows_per_expert = 2 * s.F;
-  g.tmOut0 = c->tp_Y;
+  g.out0 = c->at<uint16_t>(c->plan.Y);
   return g;
 }
 // w1_grad: dW_gate_up[e][n][c] = sum_rows dH[r][n] * Xp[r][c]   (shares dH with gate_grad)
@@ -790,10 +775,6 @@ int moe_create(moe_ctx** out, const moe_shape* shape, void* workspace, size_t wo
     if (!rc && train) rc = encode_2d(&c->tk_dOutp[i], c->ws + p.dOutp, cap, s.d, br, 64);
     if (!rc && train) rc = encode_2d(&c->tk_dH[i], c->ws + p.dH, cap, 2 * s.F, br, 64);
   }
-  if (!rc) rc = encode_2d_plain(&c->tp_A, c->ws + p.A, cap, s.F, 16, 32);
-  if (!rc) rc = encode_2d_plain(&c->tp_Y, c->ws + p.Y, cap, s.d, 32, 16);
-  if (!rc && train) rc = encode_halves_plain(&c->tp_H, c->ws + p.H, cap, s.F, 16, 32);
-  if (!rc && train) rc = encode_halves_plain(&c->tp_dH, c->ws + p.dH, cap, s.F, 32, 16);
   if (rc) {
     if (c->owns_ws) cudaFree(c->ws);
     delete c;
@@ -1231,7 +1212,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     for (size_t wi = 0; wi < vw.size(); ++wi) {
       auto& w = vw[wi];
       // worker 0 is a background gatherer; the others leave the gather queue after the first tasks
-      const bool may_gather = next_gather < ngather && (wi == 0 || next_gather < GATHER_FAST_TASKS);
+      const bool may_gather = next_gather < ngather && (wi == 0 || next_gather < gather_fast_tasks(d));
       if (!w.holding && may_gather) {
         w.v.op = VEC_GATHER; w.v.idx = next_gather++;
         w.holding = true;

@@ -3,7 +3,7 @@
 // One cooperative grid of one CTA per SM in clusters of two runs the whole operator chain.  Per CTA:
 //   warp 0      TMA producer of the weights (weight gradients: of the A operand)
 //   warp 1      tcgen05.mma issuer (even CTA) and TMEM owner
-//   warps 2-5, 8-11  epilogue: TMEM -> fused element-wise math -> TMA store, then the tile's trigger event
+//   warps 2-5, 8-11  epilogue: TMEM -> fused element-wise math -> global memory, then the tile's trigger event
 //   warp 6      TMA producer of the tokens (weight gradients: of the B operand)
 //   warp 7      even CTA: scheduler of the pair -- takes the next ticket of the matrix queue, waits for
 //               the item's dependent events, publishes it to the other roles; odd CTA: vector worker
@@ -26,6 +26,7 @@ constexpr int SCHED_WARP = 7;   // even CTA: scheduler of the pair; odd CTA: a v
 constexpr int VEC_WARPS = 4;
 constexpr int FUSED_THREADS = 32 * (GEMM_ROLE_WARPS + VEC_WARPS);
 
+static_assert(GATHER_ROWS == 4, "vec_gather");
 constexpr size_t FUSED_SMEM_BYTES = 1024 + LAYOUT_BYTES + PIPE_BARRIER_BYTES + 384 /* TicketRing */;
 static_assert(WGRAD_LAYOUT_BYTES <= LAYOUT_BYTES && FUSED_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
@@ -59,13 +60,15 @@ __device__ __forceinline__ int vec_gather(const FusedArgs& fa, int task, int lan
 #pragma unroll
   for (int r = 0; r < GATHER_ROWS; ++r) {
     in[r] = nullptr;
-    float w = 0.0f;
-    if (slots[r] >= 0) {
-      const int t = slots[r] / fa.kp, j = slots[r] - t * fa.kp;
-      in[r] = reinterpret_cast<const uint4*>(fa.gather_src + (size_t)t * fa.d);
-      if (fa.prow_w) w = j < k ? fa.topk_w[(size_t)t * k + j] : 1.0f;
+    if (slots[r] >= 0) in[r] = reinterpret_cast<const uint4*>(fa.gather_src + (size_t)(slots[r] / fa.kp) * fa.d);
+  }
+  float w = 0.0f;   // routing weight, a lane per row (padding rows: 0); stored behind the rows, nothing waits for the load
+  if (fa.prow_w && lane < GATHER_ROWS) {
+    const int slot = lane == 0 ? slots[0] : lane == 1 ? slots[1] : lane == 2 ? slots[2] : slots[3];
+    if (slot >= 0) {
+      const int t = slot / fa.kp, j = slot - t * fa.kp;
+      w = j < k ? fa.topk_w[(size_t)t * k + j] : 1.0f;
     }
-    if (fa.prow_w && lane == 0) fa.prow_w[p0 + r] = w;   // padding rows: weight 0
   }
   uint4* out = reinterpret_cast<uint4*>(fa.gather_dst + (size_t)p0 * fa.d);
   constexpr int U = 16 / GATHER_ROWS;
@@ -82,6 +85,7 @@ __device__ __forceinline__ int vec_gather(const FusedArgs& fa, int task, int lan
       for (int u = 0; u < U; ++u)
         if (v + 32 * u < nvec) out[(size_t)r * nvec + v + 32 * u] = q[r][u];   // padding rows are zero-filled
   }
+  if (fa.prow_w && lane < GATHER_ROWS) fa.prow_w[p0 + lane] = w;
   return p0 / BLOCK_M;
 }
 
@@ -176,8 +180,8 @@ __device__ __forceinline__ bool vec_dw(const FusedArgs& fa, int mb, int lane, co
   return true;
 }
 
-// Vector workers.  The first GATHER_FAST_TASKS gather tasks -- what the first matrix items of every
-// pair wait for -- is taken by every worker; after that only BACKGROUND_GATHERERS warps per CTA keep gathering,
+// Vector workers.  The first gather_fast_tasks() gather tasks -- what the first matrix items of every
+// pair wait for -- are taken by every worker; after that only BACKGROUND_GATHERERS warps per CTA keep gathering,
 // a few M-blocks' worth of traffic at a time, well ahead of the matrix queue but far below the bandwidth the
 // GEMMs need: a gather at full speed takes its bytes from the loads of the matrix tiles and slows them by more
 // than it saves.  The other workers go on to the second queue and sleep on its dependent events.
@@ -185,7 +189,7 @@ constexpr int BACKGROUND_GATHERERS = 2;
 __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const WaitCtl& wc, const TraceCtl& tr, int M,
                                                    int lane, bool background_gatherer) {
   if (*reinterpret_cast<volatile int*>(&fa.status->abort)) return;
-  const int ngather = gather_total(fa.lv.meta[5]), fast = GATHER_FAST_TASKS;
+  const int ngather = gather_total(fa.lv.meta[5]), fast = gather_fast_tasks(fa.d);
   // with shared experts the gather starts at their first row, like the matrix queue (schedule.h, rotate_index)
   const int S = fa.cp.kp - fa.cp.k;
   const int gather_first = S > 0 ? fa.lv.group_start[fa.cp.Ep - S] * GATHER_SUB : 0;
@@ -529,28 +533,21 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (!ok || wd.ticket < 0) break;
       const int phase = wd.phase;
       const ChainDeps dep = phase_deps(fa, phase, wc, tr);
-      if (!BWD && phase != cur_phase) {
-        // the forward's two operators have one layout: the ring runs on, only the staging slots change their size
-        cur_phase = phase;
-        es.round = 0;
-        if (is_epilogue_warp(warp) && lane == 0) tma_store_wait_read();
-        __syncwarp();
-      }
-      // ---- phase boundary of the backward (see phase_wait): staging and operand ring of the new phase overlap the old ones
+      // the forward's two operators have one layout: the ring and the staging run on
+      // ---- phase boundary of the backward (gemm_roles.cuh): the new phase's ring, of its own depth, starts at stage 0
       if (BWD && phase != cur_phase) {
         cur_phase = phase;
-        ls.s = ls.a_s = 0;   // every stage has been consumed: the new phase's ring (of its own depth) starts at 0
-        is.s = is.a_s = 0;
-        if (warp != 1) {
+        if (warp == 0 || warp == 6) {
+          if (!loader_enter_phase(bars, ls, phase, wc)) break;
+        } else if (warp == 1) {
+          is.s = is.a_s = 0;
+        } else {
           int go = 1;
           if (lane == 0) {
-            if (is_epilogue_warp(warp)) {
-              tma_store_wait_all();
-              epi_enter_phase(bars, epilogue_index(warp), phase);
-            }
+            tma_store_wait_read();
+            epi_enter_phase(bars, epilogue_index(warp), phase);
             go = phase_wait(bars, phase, wc) ? 1 : 0;
           }
-          es.round = 0;
           if (!__shfl_sync(0xffffffffu, go, 0)) break;
         }
       }

@@ -18,6 +18,7 @@ namespace moe {
 constexpr int WG_A_SLOTS = 5;    // weight gradients: 16 KB slots of the strip's A operand
 constexpr int WG_B_STAGES = 7;   // weight gradients: 16 KB stages of the streamed B operand
 constexpr int MAX_STAGES = 12;   // row-space operators: see plan_ring
+constexpr size_t WGRAD_STAGING_AT = (size_t)WG_A_SLOTS * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES;   // behind both
 
 // Warps of a GEMM CTA: 0 weight loader, 1 MMA issuer, 2-5 and 8-11 epilogue, 6 token loader, 7 left to the kernel (scheduler).
 // TMEM lanes 32 (w % 4) .. are what warp w can read.
@@ -40,9 +41,12 @@ struct __align__(8) PipeBarriers {
 // Pipeline state of a role, carried from item to item (the barriers persist).  The parity to wait for is kept per
 // stage, so operators with rings of different depth can follow one another in one launch (the ring position
 // restarts at 0 at such a boundary, where every stage has been consumed).
-struct LoaderState { uint32_t s = 0, empty_par = (1u << MAX_STAGES) - 1, a_s = 0, a_ph = (1u << WG_A_SLOTS) - 1; };
+struct LoaderState {
+  uint32_t s = 0, empty_par = (1u << MAX_STAGES) - 1, a_s = 0, a_ph = (1u << WG_A_SLOTS) - 1;
+  int guard = 0;   // != 0: the phase whose epilogue warps must all have arrived before a stage above WGRAD_STAGING_AT is loaded
+};
 struct IssuerState { uint32_t s = 0, full_par = 0, a_s = 0, acc_it = 0; };
-struct EpiState { uint32_t acc_it = 0, round = 0; };   // round: position in the warp's ring of staging slots
+struct EpiState { uint32_t acc_it = 0; };
 
 __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
   for (int s = 0; s < MAX_STAGES; ++s) {
@@ -57,10 +61,12 @@ __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
   mbar_init(&bars->drain, 1);
   for (int w = 0; w < EPI_WARPS; ++w) bars->epi_phase[w] = 0;
 }
-// Phase boundaries of the persistent launch.  The shared memory of a phase (operand ring, staging) is carved
-// per operator, so the roles that write it -- loaders, and epilogue warps (staging) -- enter phase p only when
-// every epilogue warp of their CTA has: all MMAs of earlier phases are then complete and every store has read
-// its staging slot.  A word per warp rather than an mbarrier: a pair may pass several phases at once.
+// Phase boundaries of the persistent launch.  The shared memory of a phase (operand ring, staging) is carved per operator.
+// Operand rings start at the bottom, staging lies at the top (staging_at), so the loads of a phase start as soon as the
+// MMAs of the phase before are complete (loader_enter_phase) while its epilogue is still at work.  Who writes what another
+// warp's staging of an earlier phase may occupy -- epilogue warps, and loaders above WGRAD_STAGING_AT -- first waits until
+// every epilogue warp of the CTA has entered the phase.  A word per warp rather than an mbarrier: a pair may pass several
+// phases at once.
 __device__ __forceinline__ void epi_enter_phase(PipeBarriers* bars, int ew, int phase) {   // one lane
   __threadfence_block();
   *reinterpret_cast<volatile int*>(&bars->epi_phase[ew]) = phase;
@@ -87,6 +93,17 @@ __device__ __forceinline__ bool phase_wait(PipeBarriers* bars, int phase, const 
     }
   }
   __threadfence_block();
+  return true;
+}
+
+// A loader warp enters a phase with another ring: every stage of the old one has been multiplied (the commit that frees a
+// stage also covers the A slots of a weight gradient).  Stages the old ring did not use pass at once.
+__device__ __forceinline__ bool loader_enter_phase(PipeBarriers* bars, LoaderState& ls, int phase, const WaitCtl& wc) {
+#pragma unroll 1
+  for (int s = 0; s < MAX_STAGES; ++s)
+    if (!mbar_wait_warp(&bars->empty[s], (ls.empty_par >> s) & 1, wc, SITE_EMPTY, phase, 50)) return false;
+  ls.s = ls.a_s = 0;
+  ls.guard = phase;
   return true;
 }
 
@@ -164,15 +181,19 @@ struct ChainDeps {
 // =====================================================================================================
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
-// Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes] |
-// staging | act_grad scratch, all of it within LAYOUT_BYTES.  An expert holds at most T rows, so a tile of T <= 256 tokens needs
+// Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes], and at
+// the end of LAYOUT_BYTES the staging.  An expert holds at most T rows, so a tile of T <= 256 tokens needs
 // n32(T) / 2 rows per CTA and nothing merges; beyond, a merged item (128 + 256) / 2.  What the token stages do not need
 // goes into more stages: with 32 tokens eleven, 198 KB of weights in flight instead of 80 -- a pass over few tokens is a
 // stream of weights from HBM.
 constexpr size_t PIPE_BARRIER_BYTES = 384;
 constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - 384 /* TicketRing of the persistent launch */;
-__host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) {
-  return EPI_WARPS * ((size_t)sw_staging_bytes(mode) + (mode == GEMM_ACT_GRAD ? SW_SCRATCH_BYTES : 0));
+__host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return EPI_WARPS * (size_t)sw_staging_bytes(mode); }
+__host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
+// does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
+__device__ __forceinline__ bool above_guard(const GemmArgs& a, uint32_t s) {
+  return (size_t)a.stages * W_STAGE_BYTES + (size_t)(s + 1) * a.tok_bytes > WGRAD_STAGING_AT ||
+         (size_t)(s + 1) * W_STAGE_BYTES > WGRAD_STAGING_AT;
 }
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
 // tokens.
@@ -192,6 +213,10 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem,
   for (int kb = 0; kb < nkb; ++kb) {
     if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, t, 50)) return false;
     ls.empty_par ^= 1u << ls.s;
+    if (DEP::kOn && ls.guard && above_guard(a, ls.s)) {   // a weight gradient's staging may still be in use there
+      if (!uniform(lane == 0 ? (int)phase_wait(bars, ls.guard, wc) : 1)) return false;
+      ls.guard = 0;
+    }
     if (!tok_warp) {
       load_weights_swap<MODE>(a, e, n0, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], 2 * (half_a + half_b));
     } else {
@@ -248,41 +273,38 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem
   return true;
 }
 
-// Epilogue warps (both CTAs, own features).  With events: a warp signals the M-blocks of a tile once its
-// TMA stores of that tile are complete (cp.async.bulk.wait_group 0), ordered for consumers that read
-// through TMA (fence.proxy.async) and released at GPU scope.
+// Epilogue warps (both CTAs, own features).  With events: a warp signals the M-blocks of a tile behind its stores of that
+// tile: the release at GPU scope orders them, the consumer's fence.proxy.async makes them visible to its TMA loads.
 template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
                                                    uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                    const SwapWork& wk, int t, const WaitCtl& wc, const DEP& dep) {
-  constexpr int WARPB = sw_staging_bytes((GemmMode)MODE);
-  uint8_t* sOut = smem + a.stages * (W_STAGE_BYTES + a.tok_bytes);
-  SwStaging sg{sOut + ew * WARPB, es.round, sOut + EPI_WARPS * WARPB + ew * SW_SCRATCH_BYTES};
-  bool ok = true;
+  uint8_t* staging = smem + staging_at((GemmMode)MODE) + ew * sw_staging_bytes((GemmMode)MODE);
   for (int part = 0; part < (wk.merged ? 2 : 1); ++part) {   // a merged item is two consecutive tiles here
     const SwapTile& st = part ? wk.b : wk.a;
     const int as = es.acc_it & 1;
-    if (!mbar_wait(&bars->tmem_full[as], (es.acc_it >> 1) & 1, wc, SITE_TMEM_FULL, t, 200)) { ok = false; break; }
     uint64_t t0 = 0;
-    if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
-    tc_fence_after_sync();
-    epilogue_swap<MODE>(a, st, tmem_base + as * BN, rank, ew, lane, sg);
+    auto ready = [&]() {
+      if (!mbar_wait_warp(&bars->tmem_full[as], (es.acc_it >> 1) & 1, wc, SITE_TMEM_FULL, t, 200)) return false;
+      if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
+      __syncwarp();
+      tc_fence_after_sync();
+      return true;
+    };
+    if (!epilogue_swap<MODE>(a, st, tmem_base + as * BN, rank, ew, lane, staging, ready)) return false;
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) mbar_arrive_leader(&bars->tmem_empty[as]);
     ++es.acc_it;
     if (DEP::kOn) {
       if (lane == 0) {
-        tma_store_wait_all();
-        fence_proxy_async();
         dep.signal(st.mb_first, st.mb_count);
         if (ew == 0 && dep.tracing()) dep.trace(TR_EPI, t, t0, t0, globaltimer_ns());
       }
       __syncwarp();
     }
   }
-  es.round = sg.round;
-  return ok;
+  return true;
 }
 
 // =====================================================================================================
@@ -300,8 +322,9 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
 // B ring is deeper than one tile (WG_B_STAGES): the loads of tile i + 1 are in flight while tile i multiplies.
 // The staging of the epilogue is what pays for it: one 4 KB box of 32 rows x 64 columns per warp.
 constexpr int A_RES_KB = WG_A_SLOTS;         // k-blocks of A that can stay resident
-constexpr size_t WGRAD_LAYOUT_BYTES =
-    (size_t)WG_A_SLOTS * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES + EPI_WARPS * OUT_BOX_BYTES;
+constexpr size_t WGRAD_LAYOUT_BYTES = WGRAD_STAGING_AT + EPI_WARPS * OUT_BOX_BYTES;
+// the weight gradients' operands never touch the staging of a row-space operator in front of them
+static_assert(WGRAD_STAGING_AT <= staging_at(GEMM_ACT_GRAD) && WGRAD_STAGING_AT <= staging_at(GEMM_GATE_GRAD), "phase overlap");
 
 // Epilogue of one 128 x 256 accumulator slice of a weight gradient (or zeros for an expert without rows): warps `quad`
 // and `quad + 4` store 32 rows, 64 columns at a time in turn, each through a staging box of its own.
@@ -442,7 +465,7 @@ template <class DEP>
 __device__ __forceinline__ bool wgrad_epilogue_strip(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
                                                      uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                      const Strip& st, int sp, const WaitCtl& wc, const DEP& dep) {
-  uint8_t* box = smem + WG_A_SLOTS * A_STAGE_BYTES + WG_B_STAGES * HALF_B_BYTES + ew * OUT_BOX_BYTES;
+  uint8_t* box = smem + WGRAD_STAGING_AT + ew * OUT_BOX_BYTES;
   Tile tl;
   tl.e = st.e; tl.row0 = st.row0; tl.m0 = st.m0(rank); tl.nkb = st.nkb;
   const bool idle = tl.m0 >= a.M;   // the strip's second half lies outside dW: nothing to store

@@ -131,42 +131,20 @@ __device__ __forceinline__ uint32_t swap_idesc(int ntok) {
   return make_idesc_bf16(2 * BLOCK_M, ntok, W_MN ? 1 : 0, 0);
 }
 
-// ---------------------------------------------------------------- staging ring of an epilogue warp
-// Tokens per staging slot, bytes of a slot, slots per warp.  gate+up: A and, if they are kept, H gate and H up of 16 features
-// each; act_grad: d(gate) and d(up) of 32 features; down, gate_grad: 32 features.
+// ---------------------------------------------------------------- staging of an epilogue warp
+// A warp takes a chunk of tokens from TMEM as matrix fragments (pairs of tokens of one feature per register pair), writes
+// the bf16 results to its staging with transposing stmatrix -- rows of tokens there -- reads them back by row and stores
+// 16-byte vectors.  Nothing but the warp itself waits for the staging.  Rows of 32 or 64 bytes; their 16-byte
+// pieces are permuted so that the eight rows of a matrix fall into different banks.
 template <int MODE>
-__host__ __device__ constexpr int sw_chunk() { return MODE == GEMM_GATE_UP ? 32 : 16; }
-template <int MODE>
-__device__ __forceinline__ int sw_slot_bytes(const GemmArgs& a) {
-  return MODE == GEMM_GATE_UP ? (a.save_h ? 3072 : 1024) : MODE == GEMM_ACT_GRAD ? 2048 : 1024;
-}
-template <int MODE>
-__device__ __forceinline__ uint32_t sw_slots(const GemmArgs& a) {
-  return MODE == GEMM_GATE_UP ? (a.save_h ? 1 : 3) : MODE == GEMM_ACT_GRAD ? 2 : 3;
-}
-// staging bytes of a warp: the same for gate+up and down, which share one layout in the persistent forward launch
-__host__ __device__ constexpr int sw_staging_bytes(GemmMode mode) { return mode == GEMM_ACT_GRAD ? 4096 : 3072; }
-constexpr int SW_SCRATCH_BYTES = 4096;   // act_grad, per warp: saved pre-activations, two halves of [gate | up][16 tokens][32 features]
-struct SwStaging {
-  uint8_t* base;     // this warp's slots
-  uint32_t round;
-  uint8_t* scratch;  // act_grad
-};
-template <int MODE>
-__device__ __forceinline__ uint8_t* sw_acquire(const GemmArgs& a, SwStaging& sg, int lane) {
-  const uint32_t slots = sw_slots<MODE>(a);
-  if (lane == 0) {   // the slot's previous stores have read it
-    if (slots == 1) tma_store_wait_read();
-    else if (slots == 2) tma_store_wait_read_n<1>();
-    else tma_store_wait_read_n<2>();
-  }
-  __syncwarp();
-  uint8_t* slot = sg.base + sg.round * sw_slot_bytes<MODE>(a);
-  if (++sg.round == slots) sg.round = 0;
-  return slot;
-}
-__device__ __forceinline__ uint16_t bf16_bits(float x) { return __bfloat16_as_ushort(__float2bfloat16_rn(x)); }
-__device__ __forceinline__ float bf16_to_f32(uint16_t h) { return __uint_as_float(static_cast<uint32_t>(h) << 16); }
+__host__ __device__ constexpr int sw_chunk() { return MODE == GEMM_ACT_GRAD ? 16 : 32; }   // tokens of a chunk
+// Staging bytes of a warp.  gate+up: [32 tokens][16 features] of A, H gate, H up (down: the same, one layout in the persistent
+// forward launch); act_grad: [gate | up][16 tokens][32 features], the pre-activations in, their gradients out; gate_grad, down:
+// [32 tokens][32 features].
+__host__ __device__ constexpr int sw_staging_bytes(GemmMode mode) { return mode == GEMM_ACT_GRAD || mode == GEMM_GATE_GRAD ? 2048 : 3072; }
+// byte offset of 16-byte piece c of token t in rows of 64 and of 32 bytes
+__device__ __forceinline__ uint32_t piece64(int t, int c) { return t * 64 + ((c ^ ((t >> 1) & 3)) << 4); }
+__device__ __forceinline__ uint32_t piece32(int t, int c) { return t * 32 + ((c ^ ((t >> 2) & 1)) << 4); }
 __device__ __forceinline__ uint4 ld_nc_v4(const uint16_t* p) {
   uint4 r;
   asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
@@ -174,86 +152,122 @@ __device__ __forceinline__ uint4 ld_nc_v4(const uint16_t* p) {
 }
 
 
+// 1 / (1 + e^-g) of two values
+__device__ __forceinline__ float2x sigmoid2(float2x g) {
+  float lo, hi;
+  unpack2(mul2(g, pack2(-1.4426950408889634f, -1.4426950408889634f)), lo, hi);
+  asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(lo));
+  asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(hi));
+  unpack2(add2(pack2(lo, hi), pack2(1.0f, 1.0f)), lo, hi);
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(lo));
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(hi));
+  return pack2(lo, hi);
+}
+
 // ---------------------------------------------------------------- epilogues (transposed accumulator)
 // Warps `quad` and `quad + 4` of CTA `rank` own TMEM lanes 32*quad .. 32*quad+31 (32 output features) and walk the tile's
-// tokens in alternating chunks.  A thread (= one feature) writes one bf16 per token into a staging box laid out
-// [token][feature]; lane 0 stores the box with TMA (clipped at the tensor edge).  With one warp per quarter the epilogue of
-// a 256-token tile took 11-16 us, as long as the MMAs of 32-64 k-blocks: latency, two warps hide each other's.
-template <int MODE>
-__device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile& st, uint32_t tmem_acc, int rank,
-                                              int ew, int lane, SwStaging& sg) {
+// tokens in alternating chunks: latency, two warps hide each other's.  `ready` waits for the accumulator; what a chunk needs
+// besides it is fetched before.
+//
+// What bounds it is instructions: with a feature per lane, 2-byte staging accesses and shuffles between gate and up lanes
+// act_grad took 675 instructions per 16 tokens and warp, 19 us for a 256-token tile (gate+up with H kept 12 us, down 6 us) -- on
+// passes with a few tiles per SM longer than their MMAs, and exposed.
+template <int MODE, class READY>
+__device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile& st, uint32_t tmem_acc, int rank,
+                                              int ew, int lane, uint8_t* staging, READY ready) {
   const int quad = ew & 3;
   constexpr int CH = sw_chunk<MODE>();
   const int first = (ew >> 2) * CH;
   const uint32_t trow = tmem_acc + (static_cast<uint32_t>(quad * 32) << 16);
+  constexpr uint32_t HALF = 16u << 16;   // TMEM lanes 16.. of the warp
+  const uint32_t stg = smem_u32(staging);
+  const int mrow = lane & 7, mat = lane >> 3;   // this lane gives the address of row mrow of matrix mat
   if (MODE == GEMM_DOWN || MODE == GEMM_GATE_GRAD) {
+    if (!ready()) return false;
     const int f0 = st.n0 + rank * 128 + quad * 32;   // first output column of this warp
-    if (f0 >= a.N) return;
+    if (f0 >= a.N) return true;
+    const int part = lane & 3;
+    const bool inside = f0 + part * 8 < a.N;     // N % 8 == 0: a 16-byte piece is inside or outside as a whole
+    uint16_t* const out = a.out0 + (size_t)st.row0 * a.N + f0 + part * 8;
 #pragma unroll 1
     for (int c0 = first; c0 < st.ntok; c0 += 2 * CH) {
-      float v[16];
-      tmem_ld16(trow + c0, v);
+      float v[32];   // [features 0.. | 16..][token group of 8][feature, feature + 8][token pair]
+      tmem_ld_frag4(trow + c0, v);
+      tmem_ld_frag4(trow + HALF + c0, v + 16);
       tmem_ld_wait();
-      uint8_t* box = sw_acquire<MODE>(a, sg, lane);
-      // [16 tokens][32 features].  Neighbouring lanes (features 2i, 2i+1) swap one value per token pair, so that
-      // every lane stores 4 bytes: the even lane the feature pair of token j, the odd lane that of token j+1 -- 128
-      // contiguous bytes per warp store instead of 64.
-      uint32_t* box32 = reinterpret_cast<uint32_t*>(box) + (lane >> 1);
-      const bool odd = lane & 1;
+      __syncwarp();   // the chunk before has been read back
 #pragma unroll
-      for (int j = 0; j < CH; j += 2) {
-        const float send = odd ? v[j] : v[j + 1];
-        const float recv = __shfl_xor_sync(0xffffffffu, send, 1);
-        box32[(j + (odd ? 1 : 0)) * 16] = odd ? pack_bf16x2(recv, v[j + 1]) : pack_bf16x2(v[j], recv);
+      for (int f = 0; f < 4; ++f) {   // 8 features: matrices of the four token groups
+        const float* p = v + 16 * (f >> 1) + 2 * (f & 1);
+        stmatrix4_trans(stg + piece64(8 * mat + mrow, f), pack_bf16x2(p[0], p[1]), pack_bf16x2(p[4], p[5]),
+                        pack_bf16x2(p[8], p[9]), pack_bf16x2(p[12], p[13]));
       }
-      staging_release();
-      if (lane == 0) {
-        tma_store_2d(&a.tmOut0, f0, st.row0 + c0, box);
-        tma_store_commit();
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int t = (lane + 32 * i) >> 2;
+        const uint4 q = *reinterpret_cast<const uint4*>(staging + piece64(t, part));
+        if (inside) *reinterpret_cast<uint4*>(out + (size_t)(c0 + t) * a.N) = q;
       }
     }
   } else if (MODE == GEMM_GATE_UP) {
-    // lanes 0..7 and 16..23: gate pre-activations of features 0..7 and 8..15 of the warp, lanes 8..15 and 24..31: up
-    // pre-activations of the same features.  For a token pair (j, j+1) gate and up lane of a feature swap one value: the
-    // gate lane finishes token j, the up lane token j+1.
-    const int fl = (lane & 7) + ((lane >> 4) << 3);
-    const bool hi = (lane & 8) != 0;
+    // TMEM lanes 0..7 and 16..23: gate pre-activations of features 0..7 and 8..15 of the warp, lanes 8..15 and 24..31: up
+    // pre-activations of the same features: a fragment holds both of a feature in one thread.
     const int fw0 = st.n0 + rank * 64 + quad * 16;   // first feature of this warp
-    if (fw0 >= a.F) return;
-    float w_next = first < st.ntok ? a.prow_w[st.row0 + first + lane] : 0.f;
+    const float* wsrc = a.prow_w + st.row0 + 2 * (lane & 3);   // routing weights of the thread's token pairs
+    float2 w_next[4];
+    auto fetch = [&](int c0) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) w_next[b] = *reinterpret_cast<const float2*>(wsrc + c0 + 8 * b);
+    };
+    if (!ready()) return false;   // (the weights are complete with the tokens, which the MMAs have read)
+    if (fw0 >= a.F) return true;
+    if (first < st.ntok) fetch(first);
+    const int part = lane & 1;
+    const bool inside = fw0 + 8 * part < a.F;     // F % 8 == 0
+    const size_t col = fw0 + 8 * part;
 #pragma unroll 1
     for (int c0 = first; c0 < st.ntok; c0 += 2 * CH) {
-      float v[32];
-      tmem_ld16(trow + c0, v);
-      tmem_ld16(trow + c0 + 16, v + 16);
-      const float wl = w_next;   // routing weight of token c0 + lane; the next chunk's is on its way
-      if (c0 + 2 * CH < st.ntok) w_next = a.prow_w[st.row0 + c0 + 2 * CH + lane];
+      float v[32];   // [features 0..7 | 8..15][token group of 8][gate, up][token pair]
+      tmem_ld_frag4(trow + c0, v);
+      tmem_ld_frag4(trow + HALF + c0, v + 16);
+      float2x w[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) w[b] = pack2(w_next[b].x, w_next[b].y);
+      if (c0 + 2 * CH < st.ntok) fetch(c0 + 2 * CH);
       tmem_ld_wait();
-      uint8_t* box = sw_acquire<MODE>(a, sg, lane);
-      uint16_t* abox = reinterpret_cast<uint16_t*>(box);           // A: [32 tokens][16 features]
-      uint16_t* hbox = reinterpret_cast<uint16_t*>(box + 1024 + (hi ? 1024 : 0));   // H gate / H up
+      __syncwarp();   // the chunk before has been read back
 #pragma unroll
-      for (int j = 0; j < CH; j += 2) {
-        const float send = hi ? v[j] : v[j + 1];
-        const float recv = __shfl_xor_sync(0xffffffffu, send, 8);
-        const float g = hi ? recv : v[j];
-        const float u = hi ? v[j + 1] : recv;
-        const int tj = j + (hi ? 1 : 0);
-        const float w = __shfl_sync(0xffffffffu, wl, tj);
-        abox[tj * 16 + fl] = bf16_bits(w * (g * sigmoidf_fast(g) * u));
-      }
-      if (a.save_h) {
+      for (int h = 0; h < 2; ++h) {
+        uint32_t act[4], hg[4], hu[4];
 #pragma unroll
-        for (int j = 0; j < CH; ++j) hbox[j * 16 + fl] = bf16_bits(v[j]);
-      }
-      staging_release();
-      if (lane == 0) {
-        tma_store_2d(&a.tmOut0, fw0, st.row0 + c0, box);
-        if (a.save_h) {
-          tma_store_3d(&a.tmOut1, fw0, 0, st.row0 + c0, box + 1024);
-          tma_store_3d(&a.tmOut1, fw0, 1, st.row0 + c0, box + 2048);
+        for (int b = 0; b < 4; ++b) {
+          const float* p = v + 16 * h + 4 * b;
+          const float2x g = pack2(p[0], p[1]), u = pack2(p[2], p[3]);
+          act[b] = pack_bf16x2(mul2(w[b], mul2(mul2(g, sigmoid2(g)), u)));
+          hg[b] = pack_bf16x2(p[0], p[1]);
+          hu[b] = pack_bf16x2(p[2], p[3]);
         }
-        tma_store_commit();
+        const uint32_t at = stg + piece32(8 * mat + mrow, h);
+        stmatrix4_trans(at, act[0], act[1], act[2], act[3]);
+        if (a.out1) {
+          stmatrix4_trans(at + 1024, hg[0], hg[1], hg[2], hg[3]);
+          stmatrix4_trans(at + 2048, hu[0], hu[1], hu[2], hu[3]);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int t = (lane + 32 * i) >> 1;
+        const uint8_t* piece = staging + piece32(t, part);
+        const size_t row = st.row0 + c0 + t;
+        if (inside) {
+          *reinterpret_cast<uint4*>(a.out0 + row * a.F + col) = *reinterpret_cast<const uint4*>(piece);
+          if (a.out1) {
+            *reinterpret_cast<uint4*>(a.out1 + row * (2 * (size_t)a.F) + col) = *reinterpret_cast<const uint4*>(piece + 1024);
+            *reinterpret_cast<uint4*>(a.out1 + row * (2 * (size_t)a.F) + a.F + col) = *reinterpret_cast<const uint4*>(piece + 2048);
+          }
+        }
       }
     }
   } else if (MODE == GEMM_ACT_GRAD) {
@@ -262,89 +276,101 @@ __device__ __forceinline__ void epilogue_swap(const GemmArgs& a, const SwapTile&
     const int slot = (st.nb * 2 + rank) * 4 + quad;
     if (f0 >= a.F) {
       // no features here: the partial slots of this warp still take part in the reduction
+      if (!ready()) return false;
       if (a.dw_partial)
         for (int j = lane + 32 * (ew >> 2); j < st.ntok; j += 64) a.dw_partial[(size_t)(st.row0 + j) * nparts + slot] = 0.f;
-      return;
+      return true;
     }
     // The saved pre-activations of 16 tokens x 32 features (gate and up: 1 KB each) come in as four
     // 16-byte loads per lane (lane -> token (lane + 32 i) / 4, features 8 (lane % 4) ..), are parked in
-    // this warp's scratch [gate | up][16 tokens][32 features] and read back one feature column per lane.
-    // The loads of the next 16 tokens are in flight while the current ones are worked on.
+    // this warp's staging, read as fragments, replaced there by their gradients and read back by rows.
+    // The loads of the next 16 tokens are in flight while the current ones are worked on; pre-activations and routing weights
+    // are the forward launch's, so the first ones are on their way before the accumulator is ready.
     const int part = lane & 3;
-    const bool cvalid = f0 + part * 8 < a.F;     // F % 8 == 0: a 16-byte chunk is inside or outside as a whole
+    const bool inside = f0 + part * 8 < a.F;     // F % 8 == 0
     const uint16_t* hbase = a.in0 + (size_t)st.row0 * a.ld_in0 + f0 + part * 8;
+    uint16_t* const out = a.out0 + (size_t)st.row0 * a.ld_in0 + f0 + part * 8;   // dH has H's layout
+    const float* wsrc = a.prow_w + st.row0 + 2 * (lane & 3);
     uint4 pre[4];
+    float2 w_next[2];
     auto fetch = [&](int tok0) {
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const int t = (lane + 32 * i) >> 2;
-        const uint16_t* p = hbase + (size_t)(tok0 + t) * a.ld_in0;
-        pre[2 * i] = cvalid ? ld_nc_v4(p) : make_uint4(0, 0, 0, 0);
-        pre[2 * i + 1] = cvalid ? ld_nc_v4(p + a.F) : make_uint4(0, 0, 0, 0);
+        const uint16_t* p = hbase + (size_t)(tok0 + ((lane + 32 * i) >> 2)) * a.ld_in0;
+        pre[2 * i] = inside ? ld_nc_v4(p) : make_uint4(0, 0, 0, 0);
+        pre[2 * i + 1] = inside ? ld_nc_v4(p + a.F) : make_uint4(0, 0, 0, 0);
+        w_next[i] = *reinterpret_cast<const float2*>(wsrc + tok0 + 8 * i);
       }
     };
-    if (first >= st.ntok) return;
-    fetch(first);
-    float w_next = a.prow_w[st.row0 + first + (lane & 15)];
-    int half = 0;
+    if (first < st.ntok) fetch(first);
+    if (!ready()) return false;
+    const float2x one = pack2(1.0f, 1.0f), minus = pack2(-1.0f, -1.0f);
 #pragma unroll 1
     for (int h0 = first; h0 < st.ntok; h0 += 2 * CH) {
-      uint8_t* box = sw_acquire<MODE>(a, sg, lane);
-      const float wl = w_next;
-      uint8_t* scr = sg.scratch + half;
-      half ^= 2048;
+      float da[16];   // [features 0.. | 16..][token group of 8][feature, feature + 8][token pair]
+      tmem_ld_frag2(trow + h0, da);
+      tmem_ld_frag2(trow + HALF + h0, da + 8);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        uint8_t* piece = staging + piece64((lane + 32 * i) >> 2, part);
+        *reinterpret_cast<uint4*>(piece) = pre[2 * i];
+        *reinterpret_cast<uint4*>(piece + 1024) = pre[2 * i + 1];
+      }
+      float2x w[2] = {pack2(w_next[0].x, w_next[0].y), pack2(w_next[1].x, w_next[1].y)};
+      if (h0 + 2 * CH < st.ntok) fetch(h0 + 2 * CH);
+      __syncwarp();
+      tmem_ld_wait();
+      float2x pr[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};   // <dA_unweighted, a> over the thread's features, by token group
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        // matrices of (token group b, 8 features): q = 2 b + feature group
+        const uint32_t at = stg + piece64(8 * (mat >> 1) + mrow, 2 * h + (mat & 1));
+        uint32_t gr[4], ur[4];
+        ldmatrix4_trans(at, gr);
+        ldmatrix4_trans(at + 1024, ur);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int b = q >> 1;
+          const float* p = da + 8 * h + 4 * b + 2 * (q & 1);
+          const float2x g = pack2(bf16lo(gr[q]), bf16hi(gr[q])), u = pack2(bf16lo(ur[q]), bf16hi(ur[q])), d = pack2(p[0], p[1]);
+          const float2x s = sigmoid2(g), gs = mul2(g, s);
+          pr[b] = add2(pr[b], mul2(d, mul2(gs, u)));
+          const float2x dav = mul2(w[b], d);          // backward Dispatch's weight, applied here
+          const float2x ds = mul2(s, fma2(g, fma2(s, minus, one), one));   // derivative of g sigmoid(g)
+          gr[q] = pack_bf16x2(mul2(mul2(dav, u), ds));
+          ur[q] = pack_bf16x2(mul2(dav, gs));
+        }
+        stmatrix4_trans(at, gr[0], gr[1], gr[2], gr[3]);   // the pieces that this half's ldmatrix has read
+        stmatrix4_trans(at + 1024, ur[0], ur[1], ur[2], ur[3]);
+      }
+      __syncwarp();
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int t = (lane + 32 * i) >> 2;
-        *reinterpret_cast<uint4*>(scr + t * 64 + part * 16) = pre[2 * i];
-        *reinterpret_cast<uint4*>(scr + 1024 + t * 64 + part * 16) = pre[2 * i + 1];
-      }
-      if (h0 + 2 * CH < st.ntok) {
-        fetch(h0 + 2 * CH);
-        w_next = a.prow_w[st.row0 + h0 + 2 * CH + (lane & 15)];
-      }
-      float da[16], pr[16];
-      tmem_ld16(trow + h0, da);
-      __syncwarp();
-      tmem_ld_wait();
-      uint16_t* gbox = reinterpret_cast<uint16_t*>(box) + lane;          // d(gate): [16 tokens][32 features]
-      uint16_t* ubox = reinterpret_cast<uint16_t*>(box + 1024) + lane;   // d(up)
-      const uint16_t* gs16 = reinterpret_cast<const uint16_t*>(scr) + lane;
-      const uint16_t* us16 = reinterpret_cast<const uint16_t*>(scr + 1024) + lane;
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float g = bf16_to_f32(gs16[j * 32]), u = bf16_to_f32(us16[j * 32]);
-        const float s = sigmoidf_fast(g);
-        const float gs = g * s;
-        pr[j] = da[j] * (gs * u);                   // <dA_unweighted, a>: gradient of the routing weight
-        const float w = __shfl_sync(0xffffffffu, wl, j);
-        const float dav = w * da[j];                // backward Dispatch's weight, applied here
-        gbox[j * 32] = bf16_bits(dav * u * (s * (1.0f + g * (1.0f - s))));
-        ubox[j * 32] = bf16_bits(dav * gs);
+        const uint4 dg = *reinterpret_cast<const uint4*>(staging + piece64(t, part));
+        const uint4 du = *reinterpret_cast<const uint4*>(staging + 1024 + piece64(t, part));
+        if (inside) {
+          *reinterpret_cast<uint4*>(out + (size_t)(h0 + t) * a.ld_in0) = dg;
+          *reinterpret_cast<uint4*>(out + (size_t)(h0 + t) * a.ld_in0 + a.F) = du;
+        }
       }
       if (a.dw_partial) {
-        // sum over the warp's 32 features: a transposing butterfly leaves token (lane >> 1) in each lane
-#pragma unroll
-        for (int off = 16, n = 8; off >= 2; off >>= 1, n >>= 1) {
-          const bool up = (lane & off) != 0;
-#pragma unroll
-          for (int i = 0; i < n; ++i) {
-            const float keep = up ? pr[i + n] : pr[i];
-            const float send = up ? pr[i] : pr[i + n];
-            pr[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-          }
-        }
-        pr[0] += __shfl_xor_sync(0xffffffffu, pr[0], 1);
-        if ((lane & 1) == 0) a.dw_partial[(size_t)(st.row0 + h0 + (lane >> 1)) * nparts + slot] = pr[0];
+        // sum over the warp's 32 features: eight threads hold the same token pairs; each step halves what a thread keeps
+        float k0, k1, s0, s1;
+        const bool up = (lane & 16) != 0, odd = (lane & 8) != 0;
+        unpack2(up ? pr[1] : pr[0], k0, k1);
+        unpack2(up ? pr[0] : pr[1], s0, s1);
+        k0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+        k1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+        float v = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        const int t = (up ? 8 : 0) + 2 * (lane & 3) + (odd ? 1 : 0);
+        if ((lane & 4) == 0) a.dw_partial[(size_t)(st.row0 + h0 + t) * nparts + slot] = v;
       }
-      staging_release();   // (also: the scratch half written two rounds from now is the one just read)
-      if (lane == 0) {
-        tma_store_3d(&a.tmOut0, f0, 0, st.row0 + h0, box);
-        tma_store_3d(&a.tmOut0, f0, 1, st.row0 + h0, box + 1024);
-        tma_store_commit();
-      }
+      __syncwarp();   // the staging has been read back
     }
   }
+  return true;
 }
 
 }  // namespace moe

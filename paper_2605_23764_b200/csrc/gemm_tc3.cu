@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
     fence_proxy_async();
     for (int i = 0; i < 8; ++i) tma_prefetch_desc(&a.tmTok[i]);
     tma_prefetch_desc(&a.tmB);
-    tma_prefetch_desc(&a.tmOut0);
   }
   if (warp == 1) {
     tmem_alloc_pair(&bars->tmem_base, TMEM_COLS);
@@ -72,7 +71,6 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
       if (!swap_epilogue_item<MODE>(a, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, cur, t, wc, dep)) break;
     }
-    if (lane == 0) tma_store_wait_all();
   }
 
   // ---------------------------------------------------------------- teardown

@@ -36,7 +36,6 @@ __device__ __forceinline__ void stage8(uint8_t* box, int lane, int j, const floa
                        pack_bf16x2(v[6], v[7]));
   *reinterpret_cast<uint4*>(box + lane * 128 + ((j ^ (lane & 7)) << 4)) = q;
 }
-__device__ __forceinline__ float sigmoidf_fast(float g) { return __fdividef(1.0f, 1.0f + __expf(-g)); }
 
 // After filling: publish the writes to the async proxy; lane 0 then issues the stores.
 __device__ __forceinline__ void staging_release() {

@@ -93,8 +93,7 @@ enum GemmMode : int {
 struct GemmArgs {
   CUtensorMap tmA;     // weight gradients: A operand
   CUtensorMap tmB;     // row-space operators: the weights; weight gradients: B operand
-  CUtensorMap tmOut0;  // store map of out0: [rows][N] (2-D), [rows][2][F] (dH), or [Ep][M][N] (WGRAD)
-  CUtensorMap tmOut1;  // GATE_UP: store map of H as [rows][2][F]
+  CUtensorMap tmOut0;  // WGRAD: store map of the output [Ep][M][N]
   CUtensorMap tmTok[8]; // token-column tiles: the token operand with boxes of 16, 32, .., 128 rows (one TMA instruction
                         // per k-block whatever the tile's token count)
   // tile table
@@ -119,7 +118,8 @@ struct GemmArgs {
   int stages;          // operand stages
   int tok_bytes;       // token bytes of a stage per CTA
   // epilogue tensors
-  int save_h;          // GATE_UP: also store the pre-activations H
+  uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]
+  uint16_t* out1;      // GATE_UP: H [rows][2F], NULL: the pre-activations are not kept
   const uint16_t* in0; // ACT_GRAD: H
   const float* prow_w; // GATE_UP, ACT_GRAD: routing weight per padded row
   float* dw_partial;   // ACT_GRAD: [R_pad][n_tiles_n] partial <dA_unweighted, a> (may be NULL)

@@ -172,7 +172,15 @@ MOE_HD int phase_trigger_kind(const ChainParams& cp, int phase) {
 // (backward: the routing-weight gradient per M-block; then the combine tasks).  A worker leaves the first
 // queue for the second only when the first is empty -- or earlier, when it is not one of the few workers
 // that keep gathering in the background (see fused.cu).
-constexpr int GATHER_FAST_TASKS = 1024;   // gather tasks every vector worker helps with at the start of a launch
+// Gather tasks every vector worker helps with at the start of a launch: the first M-blocks, which every CTA pair waits for,
+// and at least GATHER_FAST_BYTES of rows.  A pass with no more rows than that is bound by the latency of its tasks, not by the
+// bytes they take from the matrix tiles' loads: 1777 tokens x 4 rows of 2320 bytes took 48 us when 1024 tasks were
+// everybody's (now 24), and every second matrix item waited.
+constexpr int GATHER_FAST_TASKS = 1024, GATHER_FAST_BYTES = 24 << 20;
+MOE_HD int gather_fast_tasks(int d) {
+  const int n = GATHER_FAST_BYTES / (GATHER_ROWS * 2 * d);
+  return n > GATHER_FAST_TASKS ? n : GATHER_FAST_TASKS;
+}
 struct VecTask {
   int op;       // VecOp
   int idx;      // gather: row group * GATHER_SUB + sub-task; dw: M-block; combine: token position * combine_split + column chunk
