@@ -132,7 +132,7 @@ struct Carve {
 
 // Byte offsets of every workspace tensor.
 struct WsPlan {
-  size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, pair_start, pblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, group_start, group_row, group_slot, prow_w,
+  size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, pair_start, pblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, wg_order, group_start, group_row, group_slot, prow_w,
       dw_partial, Xp, H, A, Y, dOutp, dH, st_x[2], st_dout, st_ids, st_w, st_out, st_dx, st_dw, st_logits, ctr, trace, total;
   int cap_rows, nblk_max, ntn_act, ctr_count, trace_cap;
 };
@@ -165,6 +165,7 @@ WsPlan plan_workspace(const moe_shape& s) {
   p.prow_of = c.take(sizeof(int) * (slots + 1));
   p.combine_order = c.take(sizeof(int) * ((size_t)s.T_max + 1));
   p.tok_last = c.take(sizeof(int) * ((size_t)s.T_max + 1));
+  p.wg_order = c.take(sizeof(int) * Ep);
   p.group_start = c.take(sizeof(int) * (Ep + 1));
   p.group_row = c.take(sizeof(int) * (cap / GROUP_ROWS + 1));
   p.group_slot = c.take(sizeof(int) * cap);
@@ -266,6 +267,7 @@ struct moe_ctx {
     lv.blk_hist = at<int>(plan.blk_hist);
     lv.combine_order = at<int>(plan.combine_order);
     lv.tok_last = at<int>(plan.tok_last);
+    lv.wg_order = at<int>(plan.wg_order);
     lv.group_start = at<int>(plan.group_start);
     lv.group_row = at<int>(plan.group_row);
     lv.group_slot = at<int>(plan.group_slot);
@@ -324,6 +326,7 @@ GemmArgs base_args(const moe_ctx* c) {
   g.pblk_expert = lv.pblk_expert;
   g.work_start = lv.work_start;
   g.wblk_expert = lv.wblk_expert;
+  g.wg_order = lv.wg_order;
   g.cap_rows = c->plan.cap_rows;
   g.Ep = c->shape.E + c->shape.n_shared;
   g.F = c->shape.F;
@@ -1117,6 +1120,10 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     pair_start[e + 1] = pair_start[e] + pr;
     work_start[e + 1] = work_start[e] + pr - (expert_merges(counts[e], m) ? 1 : 0);
   }
+  std::vector<int> long_before(Ep + 1, 0), order(Ep, -1);
+  for (int e = 0; e < Ep; ++e) long_before[e + 1] = long_before[e] + strip_long(counts[e]);
+  const int n_long = long_before[Ep], E = Ep - n_shared;
+  for (int e = 0; e < Ep; ++e) order[strip_order(e, counts[e], E, Ep, long_before[e], long_before[E], n_long)] = e;
   const int M = mb_start[Ep];
   std::vector<int> pblk(pair_start[Ep] + 1, 0), wblk(work_start[Ep] + 1, 0);
   for (int e = 0; e < Ep; ++e) {
@@ -1136,16 +1143,22 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   // items of every phase: {first M-block, M-blocks of unit a, M-blocks of unit b} (strips: the expert's M-blocks)
   struct Item { int phase, mb_first, mb_a, mb_b, e; };
   std::vector<std::vector<Item>> queue(pairs);
-  long n_items = 0;
+  long n_items = 0, n_queued = 0;
   std::vector<std::vector<int>> cover(cp.n_phases, std::vector<int>(M + 1, 0));
   for (int ph = 0; ph < cp.n_phases; ++ph) {
     if (cp.strips[ph]) {
-      const int total = Ep * cp.strips[ph];
-      for (int sidx = 0; sidx < total; ++sidx) {
-        const int e = sidx / cp.strips[ph];
-        queue[sidx % pairs].push_back(Item{ph, mb_start[e], mb_start[e + 1] - mb_start[e], 0, e});
-        ++n_items;
+      const int total = strip_items(Ep, cp.strips[ph], cp.ntn[ph], n_long);
+      std::vector<int> tiles((size_t)Ep * cp.strips[ph], 0);
+      for (int t = 0; t < total; ++t) {
+        const StripItem it = decode_strip_item(t, cp.strips[ph], cp.ntn[ph], n_long, order.data());
+        if (it.e < 0 || it.e >= Ep || it.strip < 0 || it.strip >= cp.strips[ph] || it.nb0 < 0 || it.nb1 > cp.ntn[ph]) return 11;
+        tiles[(size_t)it.e * cp.strips[ph] + it.strip] += it.nb1 - it.nb0;
+        queue[t % pairs].push_back(Item{ph, mb_start[it.e], mb_start[it.e + 1] - mb_start[it.e], 0, it.e});
+        ++n_queued;
+        n_items += it.nb0 == 0;   // the column tiles of a long expert's strip count once
       }
+      for (int n : tiles)
+        if (n != cp.ntn[ph]) return 14;
     } else {
       const bool mg = cp.merges[ph] != 0;
       const int total = (mg ? work_start[Ep] : pair_start[Ep]) * cp.ntn[ph];
@@ -1160,7 +1173,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
           return 10;
         for (int q = 0; q < it.mb_count; ++q) cover[ph][it.mb_first + q]++;
         queue[tq % pairs].push_back(Item{ph, it.mb_first, it.mb_count_a, it.mb_count - it.mb_count_a, it.e});
-        ++n_items;
+        ++n_items, ++n_queued;
       }
     }
   }
@@ -1193,7 +1206,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   long done_mat = 0, done_vec = 0, rounds = 0, stalls = 0;
   int next_gather = 0, next_post = 0;
   const int vtotal = ngather + npost;
-  while (done_mat < n_items || done_vec < vtotal) {
+  while (done_mat < n_queued || done_vec < vtotal) {
     bool progress = false;
     for (int q = 0; q < pairs; ++q) {
       if (cursor[q] >= queue[q].size()) continue;

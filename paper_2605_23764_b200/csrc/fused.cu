@@ -258,9 +258,9 @@ constexpr int TK_RING = 4;
 struct __align__(16) WorkDesc {
   int ticket;                                  // -1: the queue is empty
   int phase, item, flags;                      // WD_MERGED, WD_READY
-  int e, n0, nb, nkb;                          // strips: nb = 256-row block of dW
+  int e, n0, nb, nkb;                          // strips: nb = 256-row block of dW, n0 = first column tile
   int a_row0, a_ntok, a_mb_first, a_mb_count;  // strips: a_row0 = first padded row, a_ntok = rows of the expert
-  int b_row0, b_ntok, b_mb_first, b_mb_count;
+  int b_row0, b_ntok, b_mb_first, b_mb_count;  // strips: b_row0 = end of the column tiles
 };
 constexpr int WD_MERGED = 1, WD_READY = 2;   // READY: the dependent events were met when the item was published
 static_assert(sizeof(WorkDesc) == 64, "published as four 16-byte stores");
@@ -305,7 +305,7 @@ __device__ __forceinline__ SwapWork desc_swap_work(const WorkDesc& wd) {
 __device__ __forceinline__ Strip desc_strip(const WorkDesc& wd) {
   Strip st;
   st.e = wd.e; st.mp = wd.nb; st.row0 = wd.a_row0; st.rows = wd.a_ntok; st.nkb = wd.nkb;
-  st.resident = st.nkb <= A_RES_KB;
+  st.nb0 = wd.n0; st.nb1 = wd.b_row0;
   return st;
 }
 __device__ __forceinline__ void pack_swap_work(WorkDesc& wd, const SwapWork& w) {
@@ -321,10 +321,11 @@ __device__ __forceinline__ void decode_item(const FusedArgs& fa, int phase, int 
   if (strip) {
     const GemmArgs& a = fa.op[phase];
     const Strip st = decode_strip(a, item);
-    wd.flags = 0; wd.e = st.e; wd.n0 = 0; wd.nb = st.mp; wd.nkb = st.nkb;
+    wd.flags = 0; wd.e = st.e; wd.n0 = st.nb0; wd.nb = st.mp; wd.nkb = st.nkb;
     wd.a_row0 = st.row0; wd.a_ntok = st.rows; wd.a_mb_first = a.mb_start[st.e];
     wd.a_mb_count = a.mb_start[st.e + 1] - a.mb_start[st.e];
-    wd.b_row0 = wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
+    wd.b_row0 = st.nb1;
+    wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
     *first = wd.a_mb_first; *count = st.nkb > 0 ? wd.a_mb_count : 0;   // all rows of the expert
     return;
   }

@@ -35,6 +35,7 @@ struct __align__(8) PipeBarriers {
   uint64_t drain;
   uint32_t tmem_base;
   int epi_phase[EPI_WARPS];       // in each CTA: the phase each epilogue warp is in (its stores of earlier phases have read shared memory)
+  int epi_done[2];                // in each CTA, per accumulator: epilogue warps whose stores of the tile are under way
   int pad;
 };
 
@@ -60,6 +61,7 @@ __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
   }
   mbar_init(&bars->drain, 1);
   for (int w = 0; w < EPI_WARPS; ++w) bars->epi_phase[w] = 0;
+  bars->epi_done[0] = bars->epi_done[1] = 0;
 }
 // Phase boundaries of the persistent launch.  The shared memory of a phase (operand ring, staging) is carved per operator.
 // Operand rings start at the bottom, staging lies at the top (staging_at), so the loads of a phase start as soon as the
@@ -170,7 +172,9 @@ struct ChainDeps {
   // One lane, after its warp's stores of the tile are complete and ordered (see the epilogue roles).
   __device__ __forceinline__ void signal(int first, int count) const {
     if (trig_kind < 0) return;
-    for (int q = 0; q < count; ++q) counter_signal(ctr + ctr_index(first + q, trig_kind), 1);
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");   // one for all of them
+    for (int q = 0; q < count; ++q)
+      asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(ctr + ctr_index(first + q, trig_kind)) : "memory");
   }
   __device__ __forceinline__ bool tracing() const { return tr.buf != nullptr; }
   __device__ __forceinline__ void trace(int role, int item, uint64_t t0, uint64_t t_dep, uint64_t t1) const {
@@ -273,8 +277,10 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem
   return true;
 }
 
-// Epilogue warps (both CTAs, own features).  With events: a warp signals the M-blocks of a tile behind its stores of that
-// tile: the release at GPU scope orders them, the consumer's fence.proxy.async makes them visible to its TMA loads.
+// Epilogue warps (both CTAs, own features).  With events: the CTA's last warp to finish a tile signals its M-blocks.  Its
+// release at GPU scope covers what the other warps stored before they counted themselves; the consumer's fence.proxy.async
+// makes it visible to its TMA loads.  When every warp released its own stores, each waited 4-6 us for all of the SM's to
+// drain, longer than the work on the tile (1777 tokens: 10 us a gate+up tile, 3 of them work).
 template <int MODE, class DEP>
 __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars,
                                                    uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
@@ -294,15 +300,23 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
     if (!epilogue_swap<MODE>(a, st, tmem_base + as * BN, rank, ew, lane, staging, ready)) return false;
     tc_fence_before_sync();
     __syncwarp();
-    if (lane == 0) mbar_arrive_leader(&bars->tmem_empty[as]);
-    ++es.acc_it;
-    if (DEP::kOn) {
-      if (lane == 0) {
-        dep.signal(st.mb_first, st.mb_count);
+    if (lane == 0) {
+      bool last = false;
+      if (DEP::kOn) {
+        // counted before the accumulator is given back: the tile after the next, which uses this counter again, follows
+        int before;
+        asm volatile("atom.acq_rel.cta.shared::cta.add.s32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(&bars->epi_done[as])) : "memory");
+        last = before == EPI_WARPS - 1;
+        if (last) *reinterpret_cast<volatile int*>(&bars->epi_done[as]) = 0;
+      }
+      mbar_arrive_leader(&bars->tmem_empty[as]);
+      if (DEP::kOn) {
+        if (last) dep.signal(st.mb_first, st.mb_count);
         if (ew == 0 && dep.tracing()) dep.trace(TR_EPI, t, t0, t0, globaltimer_ns());
       }
-      __syncwarp();
     }
+    ++es.acc_it;
+    __syncwarp();
   }
   return true;
 }
@@ -361,21 +375,24 @@ __device__ __forceinline__ void epilogue_wgrad_tile(const GemmArgs& a, const Til
 
 struct Strip {
   int e, mp, row0, nkb, rows;   // expert, 256-row block of dW, first padded row, k-blocks, rows of the expert
-  bool resident;
+  int nb0, nb1;                 // column tiles
   __device__ __forceinline__ int m0(int rank) const { return (2 * mp + rank) * BLOCK_M; }   // this CTA's 128 rows
 };
-__device__ __forceinline__ int wgrad_strips(const GemmArgs& a) { return a.Ep * ((a.n_tiles_m + 1) / 2); }
-// Strip s of the operator: expert-major, so the pairs working at the same time share the expert's B operand
-// in L2.
+__device__ __forceinline__ int wgrad_strips(const GemmArgs& a) {
+  return strip_items(a.Ep, (a.n_tiles_m + 1) / 2, a.n_tiles_n, a.meta[6]);
+}
+// Item s of the operator (schedule.h).  Strips are expert-major, so the pairs working at the same time share the expert's
+// B operand in L2.
 __device__ __forceinline__ Strip decode_strip(const GemmArgs& a, int s) {
+  const StripItem it = decode_strip_item(s, (a.n_tiles_m + 1) / 2, a.n_tiles_n, a.meta[6], a.wg_order);
   Strip st;
-  const int tm2 = (a.n_tiles_m + 1) / 2;
-  st.e = s / tm2;
-  st.mp = s - st.e * tm2;
+  st.e = it.e;
+  st.mp = it.strip;
+  st.nb0 = it.nb0;
+  st.nb1 = it.nb1;
   st.row0 = a.mb_start[st.e] * BLOCK_M;
   st.rows = a.counts[st.e];
   st.nkb = (st.rows + BK - 1) / BK;
-  st.resident = st.nkb <= A_RES_KB;
   return st;
 }
 
@@ -389,8 +406,9 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
   const int m0 = uniform(st.m0(rank)), row0 = uniform(st.row0), nkb = uniform(st.nkb);
   const bool resident = nkb <= A_RES_KB;
   if (DEP::kOn) fence_proxy_async();   // as in swap_load_item
-  for (int nb = 0; nb < a.n_tiles_n; ++nb) {
-    const bool load_a = !resident || nb == 0;
+  const int nb0 = uniform(st.nb0), nb1 = uniform(st.nb1);
+  for (int nb = nb0; nb < nb1; ++nb) {
+    const bool load_a = !resident || nb == nb0;
     for (int kb = 0; kb < nkb; ++kb) {
       const int slot = resident ? kb : (int)ls.a_s;
       if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, sp, 50)) return false;
@@ -427,16 +445,17 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
   const bool resident = nkb <= A_RES_KB;
   if (nkb == 0) return true;
   uint64_t t0 = 0;
-  for (int nb = 0; nb < a.n_tiles_n; ++nb) {
+  const int nb0 = uniform(st.nb0), nb1 = uniform(st.nb1);
+  for (int nb = nb0; nb < nb1; ++nb) {
     const int as = is.acc_it & 1;
     if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, sp)) return false;
     tc_fence_after_sync();
     const uint32_t d_tmem = tmem_base + as * BN;
-    const bool last_use = !resident || nb == a.n_tiles_n - 1;
+    const bool last_use = !resident || nb == nb1 - 1;
     for (int kb = 0; kb < nkb; ++kb) {
       if (!mbar_wait_warp(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, sp)) return false;
       is.full_par ^= 1u << is.s;
-      if (DEP::kOn && nb == 0 && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
+      if (DEP::kOn && nb == nb0 && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
       tc_fence_after_sync();
       const int slot = resident ? kb : (int)is.a_s;
       const uint32_t a_lo = a_lo0 + slot * (A_STAGE_BYTES >> 4), b_lo = b_lo0 + is.s * (HALF_B_BYTES >> 4);
@@ -472,7 +491,7 @@ __device__ __forceinline__ bool wgrad_epilogue_strip(const GemmArgs& a, uint8_t*
   bool ok = true;
   uint64_t t0 = 0;
   if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
-  for (int nb = 0; nb < a.n_tiles_n; ++nb) {
+  for (int nb = st.nb0; nb < st.nb1; ++nb) {
     tl.nb = nb; tl.n0 = nb * BN;
     if (st.nkb == 0) {
       if (!idle) epilogue_wgrad_tile(a, tl, 0, ew, lane, box);  // an expert without rows: zeros

@@ -43,10 +43,11 @@ struct LayoutView {
   int* work_start;   // [Ep+1]  first work item of each expert (token-column GEMMs that merge: its units, the last
                      //         two of an odd M-block count >= 3 merged into one item)
   int* wblk_expert;  // [items] expert of each work item
+  int* wg_order;     // [Ep]    experts in the order of the weight-gradient phases (schedule.h); NULL: not wanted
   int* group_start;  // [Ep+1]  first 32-row group of each expert (an expert's rows up to a multiple of 32); NULL: not wanted
   int* group_row;    // [groups] first padded row of each group
   int* group_slot;   // [groups * 32] slot of each of the groups' rows, -1 for padding
-  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, num_groups, 0...}
+  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, num_groups, long experts, 0}
   int* blk_hist;     // [nblk][Ep] per-block histograms, then per-block exclusive prefixes
   int* combine_order; // [T] persistent launch: tokens in the order in which their last row is produced (NULL: token order)
   int* tok_last;      // [T] 1 + largest padded row of each token (0: none); NULL when the combine order is not wanted
@@ -105,6 +106,7 @@ struct GemmArgs {
   const int* pblk_expert;  // CTA-pair kernels: expert of each M-block pair
   const int* work_start;   // token-column kernel: first work item of each expert
   const int* wblk_expert;  // token-column kernel: expert of each work item
+  const int* wg_order;     // WGRAD: order of the experts
   int cap_rows;            // rows of the padded row space (a row coordinate >= cap_rows reads zeros)
   int Ep;
   int n_tiles_n;       // tiles along N per M-block (row-space modes) / per expert (WGRAD)

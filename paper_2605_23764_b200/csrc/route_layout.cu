@@ -133,16 +133,17 @@ __global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __
 }
 
 // Exclusive scans over the experts of a block of 1024 threads: s_counts[Ep] -> offsets of rows, M-blocks, pairs of
-// M-blocks, work items and 32-row groups, in shared memory (each Ep + 1 long) and in the layout's tables.
-struct ExpertScan { int *counts, *off, *mb, *pr, *wi, *gr; };   // shared memory
-__host__ __device__ constexpr int expert_scan_ints(int Ep) { return 6 * Ep + 5; }
+// M-blocks, work items, 32-row groups and long experts, in shared memory (each Ep + 1 long) and in the layout's tables.
+constexpr int SCAN_Q = 6;
+struct ExpertScan { int *counts, *off, *mb, *pr, *wi, *gr, *lg; };   // shared memory
+__host__ __device__ constexpr int expert_scan_ints(int Ep) { return 7 * Ep + 6; }
 __device__ __forceinline__ ExpertScan expert_scan_at(int* sm, int Ep) {
-  return ExpertScan{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3, sm + 5 * Ep + 4};
+  return ExpertScan{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3, sm + 5 * Ep + 4, sm + 6 * Ep + 5};
 }
-__device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const ExpertScan& sc, int (*totals)[33]) {
-  constexpr int NQ = 5;
+__device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv, const ExpertScan& sc, int (*totals)[33]) {
+  constexpr int NQ = SCAN_Q;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int carry[NQ] = {0, 0, 0, 0, 0};
+  int carry[NQ] = {0, 0, 0, 0, 0, 0};
   for (int e0 = 0; e0 < Ep; e0 += 1024) {
     const int e = e0 + threadIdx.x;
     const int c = e < Ep ? sc.counts[e] : 0;
@@ -150,8 +151,9 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
     const int pr = (m + 1) >> 1;  // pairs of M-blocks (the tensor-core tile of a CTA pair)
     // work items of the token-column GEMM kernels that merge: the units of the expert, except that an expert
     // that merges (schedule.h) has its last two units (one block; block + tail) share one k-loop
-    const int val[NQ] = {c, m, pr, pr - (expert_merges(c, m) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS};
-    int inc[NQ] = {val[0], val[1], val[2], val[3], val[4]};
+    const int val[NQ] = {c, m, pr, pr - (expert_merges(c, m) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS,
+                         strip_long(c)};
+    int inc[NQ] = {val[0], val[1], val[2], val[3], val[4], val[5]};
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
 #pragma unroll
@@ -181,7 +183,7 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
 #pragma unroll
     for (int q = 0; q < NQ; ++q) ex[q] = carry[q] + totals[q][warp] + inc[q] - val[q];
     if (e < Ep) {
-      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.pr[e] = ex[2]; sc.wi[e] = ex[3]; sc.gr[e] = ex[4];
+      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.pr[e] = ex[2]; sc.wi[e] = ex[3]; sc.gr[e] = ex[4]; sc.lg[e] = ex[5];
       lv.counts[e] = c;
       lv.offsets[e] = ex[0];
       lv.mb_start[e] = ex[1];
@@ -198,7 +200,7 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.pr[Ep] = carry[2]; sc.wi[Ep] = carry[3]; sc.gr[Ep] = carry[4];
+    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.pr[Ep] = carry[2]; sc.wi[Ep] = carry[3]; sc.gr[Ep] = carry[4]; sc.lg[Ep] = carry[5];
     lv.offsets[Ep] = carry[0];
     lv.mb_start[Ep] = carry[1];
     lv.pad_off[Ep] = carry[1] * BLOCK_M;
@@ -210,9 +212,13 @@ __device__ __forceinline__ void scan_experts(int Ep, const LayoutView& lv, const
     lv.meta[3] = carry[2];
     lv.meta[4] = carry[3];
     lv.meta[5] = carry[4];
+    lv.meta[6] = carry[5];
     if (lv.group_start) lv.group_start[Ep] = carry[4];
   }
   __syncthreads();
+  if (lv.wg_order)
+    for (int e = threadIdx.x; e < Ep; e += 1024)
+      lv.wg_order[strip_order(e, sc.counts[e], E, Ep, sc.lg[e], sc.lg[E], sc.lg[Ep])] = e;
 }
 // the last expert whose start is <= i
 __device__ __forceinline__ int expert_at(int Ep, const int* start, int i) {
@@ -237,9 +243,9 @@ __device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, cons
 // One block.  (1) per expert, exclusive scan of the block histograms over blocks: a thread per expert and range of
 // blocks (as many ranges as the block has threads for), so that the reads of a row are coalesced and independent;
 // (2) scans over experts; (3) M-block, pair and work-item -> expert tables.
-__global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int Ep, LayoutView lv) {
+__global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int E, int Ep, LayoutView lv) {
   extern __shared__ int sm[];
-  __shared__ int totals[5][33];
+  __shared__ int totals[SCAN_Q][33];
   const ExpertScan sc = expert_scan_at(sm, Ep);
   int* part = sm + expert_scan_ints(Ep);   // [ranges][Ep]
   pdl_trigger();
@@ -274,7 +280,7 @@ __global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int Ep, Lay
         if (b + u < b1) { lv.blk_hist[(size_t)(b + u) * Ep + e] = run; run += c[u]; }
     }
   }
-  scan_experts(Ep, lv, sc, totals);
+  scan_experts(E, Ep, lv, sc, totals);
   expert_tables(Ep, lv, sc);
 }
 
@@ -440,7 +446,7 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
                                                           int Ep, LayoutView lv, int want_order, DevStatus* status,
                                                           int* __restrict__ zero, int nzero) {
   extern __shared__ int sm[];
-  __shared__ int totals[5][33];
+  __shared__ int totals[SCAN_Q][33];
   __shared__ int carry_s;
   const ExpertScan sc = expert_scan_at(sm, Ep);
   int* s_last = sm + expert_scan_ints(Ep);                       // [LAYOUT_ONE_SLOTS] 1 + padded row of the slot
@@ -475,7 +481,7 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
     sc.counts[q] = run;
   }
   __syncthreads();
-  scan_experts(Ep, lv, sc, totals);
+  scan_experts(E, Ep, lv, sc, totals);
   if (i < n) {
     int prow = -1;
     if (e >= 0) {
@@ -525,7 +531,7 @@ cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView&
                             kp, dm.E, Ep, lv.blk_hist, tok_last, zero, nzero)))
     return e;
   const int ranges = Ep <= 1024 ? 1024 / Ep : 1;
-  if ((e = launch_dependent(layout_scan_kernel, dim3(1), dim3(1024), sizeof(int) * (expert_scan_ints(Ep) + (size_t)ranges * Ep), s, nblk, Ep, lv)))
+  if ((e = launch_dependent(layout_scan_kernel, dim3(1), dim3(1024), sizeof(int) * (expert_scan_ints(Ep) + (size_t)ranges * Ep), s, nblk, dm.E, Ep, lv)))
     return e;
   const size_t nlast = LAYOUT_CHUNK / kp + 2;
   auto rank_smem = [&](int warps) {

@@ -17,8 +17,8 @@
 // Events (Section 4.3).  Per M-block (128 rows of the padded expert-ordered row space) three
 // counters with static thresholds:
 //   gathered   += 1 per gather task (4 rows)                      threshold: its rows up to the expert's last 32-row group / 4
-//   activated  += 1 per epilogue warp and column tile of phase 0  threshold SIG * column tiles
-//   done       += 1 per epilogue warp and column tile of the last row-space phase (down / gate_grad)
+//   activated  += 1 per CTA and column tile of phase 0            threshold SIG * column tiles
+//   done       += 1 per CTA and column tile of the last row-space phase (down / gate_grad)
 // A phase-0 item depends on `gathered` of its M-blocks, a down / gate_grad item and a w1_grad
 // strip on `activated`, a w2_grad strip on `gathered`; a combine task depends on `done` of the
 // M-blocks that hold its token's rows (many-to-many: up to k+S counters per token), the
@@ -46,7 +46,7 @@ constexpr int GATHER_ROWS = 4;         // rows of a gather task: the first M-blo
                                        // waits for, are complete after a few microseconds
 constexpr int GATHER_SUB = GROUP_ROWS / GATHER_ROWS;   // gather tasks per row group
 constexpr int EPI_WARPS = 8;           // epilogue warps per CTA: two per quarter of the accumulator rows
-constexpr int SIG = 2 * EPI_WARPS;     // signals per (M-block, column tile): every epilogue warp of the pair
+constexpr int SIG = 2;                 // signals per (M-block, column tile): the last epilogue warp of each CTA of the pair
 
 enum VecOp : int { VEC_GATHER = 0, VEC_DW = 2, VEC_COMBINE = 3 };
 
@@ -112,6 +112,42 @@ MOE_HD SwapItem decode_swap_item(int t, int n_tiles_n, bool merges, const int* s
     it.mb_count += c2;
   }
   return it;
+}
+
+// Items of a weight-gradient phase.  A strip is 256 rows of dW[e] across all column tiles, its A operand resident in shared
+// memory -- for an expert of up to 320 rows.  Longer experts stream A anyway; from WG_LONG_KB k-blocks (961 rows) on, a
+// column tile is long enough (5 us) to be an item of its own, and these items come first: a shared expert of 1777 rows, last
+// in expert order with three or five tiles to a strip, kept single pairs busy for 50 us after everyone else had finished.
+// Behind them the other experts' strips, shared experts first as in the row-space phases.  order[]: the experts in that
+// order, the n_long long ones in front.
+constexpr int WG_LONG_KB = 16;
+MOE_HD int strip_long(int rows) { return (rows + 63) / 64 >= WG_LONG_KB ? 1 : 0; }
+struct StripItem { int e, strip, nb0, nb1; };   // expert, 256-row block of dW, column tiles [nb0, nb1)
+MOE_HD int strip_items(int Ep, int strips, int ntn, int n_long) { return strips * (Ep - n_long + n_long * ntn); }
+MOE_HD StripItem decode_strip_item(int t, int strips, int ntn, int n_long, const int* order) {
+  StripItem it;
+  const int per = strips * ntn;
+  if (t < n_long * per) {
+    it.e = order[t / per];
+    const int r = t % per;
+    it.strip = r / ntn;
+    it.nb0 = r - it.strip * ntn;
+    it.nb1 = it.nb0 + 1;
+  } else {
+    t -= n_long * per;
+    it.e = order[n_long + t / strips];
+    it.strip = t % strips;
+    it.nb0 = 0;
+    it.nb1 = ntn;
+  }
+  return it;
+}
+// Place of expert e in order[] given the number of long experts before it (long_before), before the first shared expert E
+// (long_before_E) and in all.
+MOE_HD int strip_order(int e, int rows, int E, int Ep, int long_before, int long_before_E, int n_long) {
+  if (strip_long(rows)) return long_before;
+  const int nl = e - long_before, nl_E = E - long_before_E, total = Ep - n_long;
+  return n_long + (e >= E ? nl - nl_E : nl + total - nl_E);
 }
 
 // What a pass consists of (filled on the host from the layer's shape).
