@@ -80,3 +80,29 @@ def test_invalid_expert_id_is_reported_and_dropped():
     assert c.sum().item() == T * k - 2 and o[-1].item() == T * k - 2
     assert layer.status() == (0, 0)  # reading clears the record
     layer.close()
+
+
+@pytest.mark.parametrize("T,E,k,S", [(2048, 24, 1, 0), (2049, 24, 1, 0), (1025, 16, 2, 0), (683, 30, 2, 1),   # one chunk, a slot more
+                                     (8 * 128, 32, 8, 0), (8 * 128 + 1, 32, 8, 0),         # eight blocks' last slot, a token more
+                                     (16 * 512, 32, 8, 0), (16 * 512 + 1, 32, 8, 0),       # sixteen blocks' last slot, a token more
+                                     (2333, 382, 7, 2), (2333, 383, 7, 2),                 # the last expert, one more
+                                     (8 * 341 + 1, 40, 3, 0)])                             # a last block that is nearly empty
+def test_layout_path_edges(T, E, k, S):
+    g = torch.Generator().manual_seed(T)
+    logits = torch.randn(T, E, generator=g)
+    logits[:, 3] += 2.0                      # an expert with most of the tokens, and an empty one
+    logits[:, 1] = -50.0
+    _check_route_layout(logits.cuda(), E, k, S, True)
+    # the order in which the persistent launch combines: every token once
+    d, F = 64, 32
+    layer = MoeLayer(T, d, E, k, S, F)
+    ids, w = layer.route(logits.cuda())
+    x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
+    W1 = (torch.randn(E + S, 2 * F, d, generator=g) / 8).to(torch.bfloat16).cuda()
+    W2 = (torch.randn(E + S, d, F, generator=g) / 6).to(torch.bfloat16).cuda()
+    out = layer.ffn_fwd(x, ids, w, W1, W2, out=torch.full((T, d), float("nan"), dtype=torch.bfloat16, device="cuda"))
+    serial = MoeLayer(T, d, E, k, S, F, serial=True)
+    assert torch.equal(out, serial.ffn_fwd(x, ids, w, W1, W2))   # token by token the same sums in both launch modes
+    assert layer.status() == (0, 0) and serial.status() == (0, 0)
+    layer.close()
+    serial.close()
