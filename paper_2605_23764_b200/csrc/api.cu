@@ -394,6 +394,7 @@ GemmArgs args_wgrad_down(const moe_ctx* c) {
   g.N = s.F;
   g.n_tiles_m = (s.d + 127) / 128;
   g.n_tiles_n = (s.F + 255) / 256;
+  g.split = strip_split(s.E + s.n_shared, (s.d + 255) / 256, g.n_tiles_n, c->num_sms / 2);
   g.tmOut0 = c->ts_dW2;
   return g;
 }
@@ -421,6 +422,7 @@ GemmArgs args_wgrad_gate_up(const moe_ctx* c) {
   g.N = s.d;
   g.n_tiles_m = (2 * s.F + 127) / 128;
   g.n_tiles_n = (s.d + 255) / 256;
+  g.split = strip_split(s.E + s.n_shared, (2 * s.F + 255) / 256, g.n_tiles_n, c->num_sms / 2);
   g.tmOut0 = c->ts_dW1;
   return g;
 }
@@ -463,6 +465,16 @@ ChainParams chain_params(const moe_ctx* c, bool bwd, int T, bool want_dw) {
     cp.ntn[3] = (s.d + 255) / 256;                 // w1_grad
     cp.strips[3] = (2 * s.F + 255) / 256;
   }
+  // k-blocks of an item: the reduction, or a strip's column tiles times those of an average expert
+  const int kb_d = (s.d + 63) / 64, kb_F = (s.F + 63) / 64, kb_rows = (int)(((long)T * cp.kp / cp.Ep + 63) / 64);
+  for (int ph = 0; ph < cp.n_phases; ++ph) {
+    int kb = ph == 0 ? kb_d : bwd ? 2 * kb_F : kb_F;
+    if (cp.strips[ph]) {
+      cp.split[ph] = strip_split(cp.Ep, cp.strips[ph], cp.ntn[ph], c->num_sms / 2);
+      kb = (cp.ntn[ph] + cp.split[ph] - 1) / cp.split[ph] * (kb_rows > 4 ? kb_rows : 4);   // a tile's stores are worth four
+    }
+    cp.batch[ph] = sched_batch(kb);
+  }
   return cp;
 }
 
@@ -476,6 +488,7 @@ FusedArgs fused_base(moe_ctx* c, bool bwd, int T) {
   c->last_ctr = fa.ctr;
   fa.d = s.d;
   fa.kp = s.k + s.n_shared;
+  fa.gatherers = background_gatherers(bwd ? 1 : 0, s.F, vector_warps());
   fa.trace = p.trace_cap ? c->at<uint4>(p.trace) : nullptr;
   fa.trace_cap = p.trace_cap;
   fa.status = c->status();
@@ -1147,15 +1160,16 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   std::vector<std::vector<int>> cover(cp.n_phases, std::vector<int>(M + 1, 0));
   for (int ph = 0; ph < cp.n_phases; ++ph) {
     if (cp.strips[ph]) {
-      const int total = strip_items(Ep, cp.strips[ph], cp.ntn[ph], n_long);
+      const int split = strip_split(Ep, cp.strips[ph], cp.ntn[ph], pairs);
+      const int total = strip_items(Ep, cp.strips[ph], cp.ntn[ph], split, n_long);
       std::vector<int> tiles((size_t)Ep * cp.strips[ph], 0);
       for (int t = 0; t < total; ++t) {
-        const StripItem it = decode_strip_item(t, cp.strips[ph], cp.ntn[ph], n_long, order.data());
+        const StripItem it = decode_strip_item(t, cp.strips[ph], cp.ntn[ph], split, n_long, order.data());
         if (it.e < 0 || it.e >= Ep || it.strip < 0 || it.strip >= cp.strips[ph] || it.nb0 < 0 || it.nb1 > cp.ntn[ph]) return 11;
         tiles[(size_t)it.e * cp.strips[ph] + it.strip] += it.nb1 - it.nb0;
         queue[t % pairs].push_back(Item{ph, mb_start[it.e], mb_start[it.e + 1] - mb_start[it.e], 0, it.e});
         ++n_queued;
-        n_items += it.nb0 == 0;   // the column tiles of a long expert's strip count once
+        n_items += it.nb0 == 0;   // the pieces of a strip count once
       }
       for (int n : tiles)
         if (n != cp.ntn[ph]) return 14;

@@ -27,7 +27,7 @@ constexpr int VEC_WARPS = 4;
 constexpr int FUSED_THREADS = 32 * (GEMM_ROLE_WARPS + VEC_WARPS);
 
 static_assert(GATHER_ROWS == 4, "vec_gather");
-constexpr size_t FUSED_SMEM_BYTES = 1024 + LAYOUT_BYTES + PIPE_BARRIER_BYTES + 384 /* TicketRing */;
+constexpr size_t FUSED_SMEM_BYTES = 1024 + LAYOUT_BYTES + PIPE_BARRIER_BYTES + TICKET_RING_BYTES;
 static_assert(WGRAD_LAYOUT_BYTES <= LAYOUT_BYTES && FUSED_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 
 // ---------------------------------------------------------------- vector work (one warp per task)
@@ -181,11 +181,10 @@ __device__ __forceinline__ bool vec_dw(const FusedArgs& fa, int mb, int lane, co
 }
 
 // Vector workers.  The first gather_fast_tasks() gather tasks -- what the first matrix items of every
-// pair wait for -- are taken by every worker; after that only BACKGROUND_GATHERERS warps per CTA keep gathering,
+// pair wait for -- are taken by every worker; after that fa.gatherers warps per CTA keep gathering,
 // a few M-blocks' worth of traffic at a time, well ahead of the matrix queue but far below the bandwidth the
 // GEMMs need: a gather at full speed takes its bytes from the loads of the matrix tiles and slows them by more
 // than it saves.  The other workers go on to the second queue and sleep on its dependent events.
-constexpr int BACKGROUND_GATHERERS = 2;
 __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const WaitCtl& wc, const TraceCtl& tr, int M,
                                                    int lane, bool background_gatherer) {
   if (*reinterpret_cast<volatile int*>(&fa.status->abort)) return;
@@ -247,12 +246,11 @@ __device__ __forceinline__ void vector_worker_loop(const FusedArgs& fa, const Wa
 // column tile share its weight slab, the strips of one expert share its rows) start within
 // microseconds of each other and meet in L2, however the pairs' speeds differ -- a static deal of
 // items to pairs loses that as soon as gather or combine traffic makes the pairs drift apart.
-// The scheduler warp of the even CTA takes the pair's tickets -- as soon as a ring slot is free, so up to
-// TK_RING items ahead of the epilogue -- looks at the item's dependent events (one M-block per lane) and
-// publishes the ticket to every role of both CTAs through a small ring in shared memory: ticket, decode and look
-// hide behind the loads of the items before it.  If the events are not met yet, whoever loads what they stand for waits for
+// The scheduler warp of the even CTA takes the pair's tickets -- a few items ahead of the epilogue (sched_hold) --
+// looks at the items' dependent events and publishes the items to every role of both CTAs through a small ring in shared
+// memory: ticket, decode and look hide behind the loads of the items before.  If the events are not met yet, whoever loads what they stand for waits for
 // them (the token loader; both loaders of a weight gradient): the weights, which depend on nothing, are under way meanwhile.
-constexpr int TK_RING = 4;
+constexpr int TK_RING = 8;
 // A published item: the ticket and the decoded work (decoding takes a chain of dependent global loads; the
 // scheduler does it once, ahead of time, for every role of both CTAs).
 struct __align__(16) WorkDesc {
@@ -272,15 +270,36 @@ struct __align__(16) TicketRing {
 // consumers: in each CTA both loaders and the epilogue warps, plus the MMA issuer of the even CTA
 constexpr int TK_CONSUMERS = 2 * (2 + EPI_WARPS) + 1;
 
-__device__ __forceinline__ void ring_publish(TicketRing* r, uint32_t n, const WorkDesc& wd) {   // one lane; the slot is free
-  const int slot = n % TK_RING;
+// The scheduler's `batch` groups of lanes (32 / batch lanes each) publish an item each, item n + group, as their slots come
+// free; `mine`: this group has an item.  Eight lanes store to both CTAs, one releases.
+__device__ __forceinline__ bool ring_publish(TicketRing* r, uint32_t n, const WorkDesc& wd, bool mine, int group, int sub,
+                                             uint32_t own /* the group's lanes */, const WaitCtl& wc) {
+  const uint32_t it = n + group, slot = it % TK_RING;
   const uint4* src = reinterpret_cast<const uint4*>(&wd);
-#pragma unroll
-  for (uint32_t rank = 0; rank < 2; ++rank) {
-    const uint32_t dst = map_to_rank(smem_u32(&r->work[slot]), rank);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) st_cluster_v4(dst + 16 * q, src[q]);
-    mbar_arrive_cluster_addr(map_to_rank(smem_u32(&r->full[slot]), rank));   // release: the item is visible
+  const uint4 piece = (sub & 3) == 0 ? src[0] : (sub & 3) == 1 ? src[1] : (sub & 3) == 2 ? src[2] : src[3];
+  uint64_t t0 = 0;
+  for (uint32_t spin = 1;; ++spin) {
+    const uint32_t free = __ballot_sync(0xffffffffu, mine && mbar_try_wait_cluster(&r->empty[slot], ((it / TK_RING) & 1) ^ 1));
+    const bool go = (free & own) == own;   // every lane of the group has seen it
+    if (go && sub < 8) st_cluster_v4(map_to_rank(smem_u32(&r->work[slot]), sub >> 2) + 16 * (sub & 3), piece);
+    __syncwarp();
+    if (go && sub == 0) {
+      mbar_arrive_cluster_addr(map_to_rank(smem_u32(&r->full[slot]), 0));
+      mbar_arrive_cluster_addr(map_to_rank(smem_u32(&r->full[slot]), 1));
+    }
+    if (go) mine = false;
+    if (!__any_sync(0xffffffffu, mine)) return true;
+    __nanosleep(50);
+    if ((spin & 63u) == 0) {
+      int gone = *reinterpret_cast<volatile int*>(&wc.status->abort);
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > wc.budget_ns) {
+        report(wc.status, /*MOE_ERR_TIMEOUT*/ 2, (SITE_EMPTY << 24) | 0xFFFFF9);
+        gone = 1;
+      }
+      if (__any_sync(0xffffffffu, gone)) return false;
+    }
   }
 }
 // All lanes of a consumer warp; returns false on a failed wait.
@@ -455,7 +474,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   PipeBarriers* bars = reinterpret_cast<PipeBarriers*>(smem + LAYOUT_BYTES);
-  static_assert(sizeof(PipeBarriers) <= PIPE_BARRIER_BYTES && sizeof(TicketRing) <= 384, "shared-memory bookkeeping");
+  static_assert(sizeof(PipeBarriers) <= PIPE_BARRIER_BYTES && sizeof(TicketRing) <= TICKET_RING_BYTES, "shared-memory bookkeeping");
   TicketRing* ring = reinterpret_cast<TicketRing*>(reinterpret_cast<uint8_t*>(bars) + PIPE_BARRIER_BYTES);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
@@ -489,37 +508,53 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
     const PhaseTable pt = make_phase_table<BWD>(fa);
     const PhaseTable rot = make_rotation_table<BWD>(fa);   // first item of the first shared expert in each row-space phase
     const int total = pt.start[SCHED_MAX_SEG];
-    for (uint32_t n = 0;; ++n) {
-      // a free ring slot first, then the ticket: a pair never holds more unstarted items than the ring has slots
+    // batches pay with many items to a pair; with few, the last ones would lie with some of the pairs
+    int batches = 0;   // two bits a phase: log2
+#pragma unroll
+    for (int p = 0; p < SCHED_MAX_SEG; ++p) {
+      const int items = pt.start[p + 1] - pt.start[p], most = fa.cp.batch[p];   // 16 and 8 for each pair
+      batches |= (items >= 8 * (int)gridDim.x && most == 4 ? 2 : items >= 4 * (int)gridDim.x && most >= 2 ? 1 : 0) << (2 * p);
+    }
+    int batch = 1 << (batches & 3);   // of the phase the last ticket belonged to
+    bool more = true;
+    for (uint32_t n = 0; more;) {
+      // the item sched_hold() before the batch's last has been taken first, then the tickets
       int ok = 1;
-      if (lane == 0) ok = mbar_wait_cluster(&ring->empty[n % TK_RING], ((n / TK_RING) & 1) ^ 1, wc, SITE_EMPTY, -7, 100) ? 1 : 0;
+      const uint32_t hold = sched_hold(batch), next = n + batch;
+      if (lane == 0 && next > hold)
+        ok = mbar_wait_cluster(&ring->empty[(next - 1 - hold) % TK_RING], ((next - 1 - hold) / TK_RING) & 1, wc, SITE_EMPTY, -7, 100) ? 1 : 0;
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
       int t = 0;
-      if (lane == 0) t = atomicAdd(&fa.ctr[CTR_MAT_TICKET], 1);
+      if (lane == 0) t = atomicAdd(&fa.ctr[CTR_MAT_TICKET], batch);
       t = __shfl_sync(0xffffffffu, t, 0);
+      // `batch` groups of lanes decode a ticket each; a group's lanes share the look at its item's events
+      const int lanes = 32 / batch, group = lane / lanes, sub = lane - group * lanes;
+      t += group;
+      uint64_t t0 = 0;
+      if (tr.buf) t0 = globaltimer_ns();
       WorkDesc wd;
-      wd.ticket = t;
-      if (t >= total) {
-        wd.ticket = -1;
+      wd.ticket = t < total ? t : -1;
+      bool met = true;
+      if (t < total) {
+        wd.phase = phase_of(pt, t);
+        wd.item = t - pt.start[wd.phase];
+        if (rot.start[wd.phase]) wd.item = rotate_index(wd.item, rot.start[wd.phase], pt.start[wd.phase + 1] - pt.start[wd.phase]);
+        int first, count;
+        decode_item<BWD>(fa, wd.phase, wd.item, wd, &first, &count);
+        met = phase_deps(fa, wd.phase, wc, tr).met(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], sub, lanes);
+      } else {
         wd.phase = wd.item = wd.flags = wd.e = wd.n0 = wd.nb = wd.nkb = 0;
         wd.a_row0 = wd.a_ntok = wd.a_mb_first = wd.a_mb_count = wd.b_row0 = wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
-        if (lane == 0) ring_publish(ring, n, wd);
-        break;
       }
-      wd.phase = phase_of(pt, t);
-      wd.item = t - pt.start[wd.phase];
-      if (rot.start[wd.phase]) wd.item = rotate_index(wd.item, rot.start[wd.phase], pt.start[wd.phase + 1] - pt.start[wd.phase]);
-      const ChainDeps dep = phase_deps(fa, wd.phase, wc, tr);
-      uint64_t t0 = 0;
-      if (tr.buf && lane == 0) t0 = globaltimer_ns();
-      int first, count;
-      decode_item<BWD>(fa, wd.phase, wd.item, wd, &first, &count);
-      if (dep.met(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane)) wd.flags |= WD_READY;
-      if (lane == 0) {
-        const uint64_t td = tr.buf ? globaltimer_ns() : 0;
-        ring_publish(ring, n, wd);
-        if (tr.buf) dep.trace(TR_SCHED, wd.item, t0, td, globaltimer_ns());
-      }
+      const uint32_t unmet = __ballot_sync(0xffffffffu, !met), own = (lanes == 32 ? ~0u : (1u << lanes) - 1u) << (group * lanes);
+      if (wd.ticket >= 0 && (unmet & own) == 0) wd.flags |= WD_READY;
+      const uint64_t td = tr.buf ? globaltimer_ns() : 0;
+      const bool mine = t < total || group == 0 || t - 1 < total;   // the end of the queue is published once
+      if (!ring_publish(ring, n, wd, mine, group, sub, own, wc)) break;
+      if (tr.buf && sub == 0 && wd.ticket >= 0) phase_deps(fa, wd.phase, wc, tr).trace(TR_SCHED, wd.item, t0, td, globaltimer_ns());
+      more = !__any_sync(0xffffffffu, wd.ticket < 0);
+      n += batch;
+      batch = 1 << ((batches >> (2 * __shfl_sync(0xffffffffu, wd.phase, 31))) & 3);
     }
   } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
@@ -570,7 +605,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   // matrix-role warps once the matrix queue is empty (the tail of the vector queue -- combine -- runs on the
   // whole SM)
   __syncwarp();
-  vector_worker_loop(fa, wc, tr, M, lane, warp >= GEMM_ROLE_WARPS && warp < GEMM_ROLE_WARPS + BACKGROUND_GATHERERS);
+  vector_worker_loop(fa, wc, tr, M, lane, warp >= GEMM_ROLE_WARPS && warp < GEMM_ROLE_WARPS + fa.gatherers);
 
   // ---------------------------------------------------------------- teardown
   if (*reinterpret_cast<volatile int*>(&fa.status->abort)) __nanosleep(200000);
@@ -582,6 +617,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
     tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
 }
+
+int vector_warps() { return VEC_WARPS; }
 
 cudaError_t launch_fused(bool bwd, const FusedArgs& fa, int num_sms, bool cooperative, cudaStream_t s, int* launches) {
   ++*launches;

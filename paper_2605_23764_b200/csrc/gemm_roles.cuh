@@ -159,15 +159,15 @@ struct ChainDeps {
       if (!counter_wait(ctr + ctr_index(first + q, wait_kind), phase_wait_thr(*cp, phase, rows, rel + q), wc, item)) ok = 0;
     return __all_sync(0xffffffffu, ok) != 0;
   }
-  // The same without waiting: are they there now?
-  __device__ __forceinline__ bool met(int first, int count, int rows, int rel, int lane) const {
-    int ok = 1;
-    for (int q = lane; q < count; q += 32) {
+  // The same without waiting, by a group of `lanes` lanes of which this is lane `sub`: has this lane found its counters there?
+  __device__ __forceinline__ bool met(int first, int count, int rows, int rel, int sub, int lanes) const {
+    bool ok = true;
+    for (int q = sub; q < count; q += lanes) {
       int v;
       asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(ctr + ctr_index(first + q, wait_kind)) : "memory");
-      if (v < phase_wait_thr(*cp, phase, rows, rel + q)) ok = 0;
+      if (v < phase_wait_thr(*cp, phase, rows, rel + q)) ok = false;
     }
-    return __all_sync(0xffffffffu, ok) != 0;
+    return ok;
   }
   // One lane, after its warp's stores of the tile are complete and ordered (see the epilogue roles).
   __device__ __forceinline__ void signal(int first, int count) const {
@@ -191,7 +191,8 @@ struct ChainDeps {
 // goes into more stages: with 32 tokens eleven, 198 KB of weights in flight instead of 80 -- a pass over few tokens is a
 // stream of weights from HBM.
 constexpr size_t PIPE_BARRIER_BYTES = 384;
-constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - 384 /* TicketRing of the persistent launch */;
+constexpr size_t TICKET_RING_BYTES = 640;   // of the persistent launch
+constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_RING_BYTES;
 __host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return EPI_WARPS * (size_t)sw_staging_bytes(mode); }
 __host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
 // does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
@@ -379,12 +380,12 @@ struct Strip {
   __device__ __forceinline__ int m0(int rank) const { return (2 * mp + rank) * BLOCK_M; }   // this CTA's 128 rows
 };
 __device__ __forceinline__ int wgrad_strips(const GemmArgs& a) {
-  return strip_items(a.Ep, (a.n_tiles_m + 1) / 2, a.n_tiles_n, a.meta[6]);
+  return strip_items(a.Ep, (a.n_tiles_m + 1) / 2, a.n_tiles_n, a.split, a.meta[6]);
 }
 // Item s of the operator (schedule.h).  Strips are expert-major, so the pairs working at the same time share the expert's
 // B operand in L2.
 __device__ __forceinline__ Strip decode_strip(const GemmArgs& a, int s) {
-  const StripItem it = decode_strip_item(s, (a.n_tiles_m + 1) / 2, a.n_tiles_n, a.meta[6], a.wg_order);
+  const StripItem it = decode_strip_item(s, (a.n_tiles_m + 1) / 2, a.n_tiles_n, a.split, a.meta[6], a.wg_order);
   Strip st;
   st.e = it.e;
   st.mp = it.strip;

@@ -111,6 +111,7 @@ struct GemmArgs {
   int Ep;
   int n_tiles_n;       // tiles along N per M-block (row-space modes) / per expert (WGRAD)
   int n_tiles_m;       // WGRAD only: tiles along M per expert
+  int split;           // WGRAD only: ranges of column tiles per strip (schedule.h)
   int K;               // reduction length (row-space modes)
   int N;               // output columns (for masking); WGRAD: columns of dW
   int M;               // WGRAD: rows of dW per expert
@@ -149,6 +150,7 @@ struct FusedArgs {
   int* ctr;                 // event counters (zeroed before the launch), schedule.h
   int d, kp;
   // gather (Dispatch / backward Dispatch)
+  int gatherers;            // vector warps per CTA that keep gathering after the first tasks
   const uint16_t* gather_src;
   uint16_t* gather_dst;
   const float* topk_w;
@@ -190,6 +192,7 @@ cudaError_t launch_router_fwd(const RouterArgs& a, int num_sms, cudaStream_t s, 
 cudaError_t launch_router_bwd(const float* logits, const int* ids, const float* g, int T, int E, int k, int gate_mode,
                               float* dlogits, cudaStream_t s, int* launches);
 
+int vector_warps();   // vector warps per CTA of the persistent launch
 // cooperative = false drops the co-residency guarantee of the launch (profilers that reject cooperative cluster
 // launches); the grid is sized to the resident capacity either way and every wait is bounded
 cudaError_t launch_fused(bool bwd, const FusedArgs& fa, int num_sms, bool cooperative, cudaStream_t s, int* launches);

@@ -119,12 +119,24 @@ MOE_HD SwapItem decode_swap_item(int t, int n_tiles_n, bool merges, const int* s
 // column tile is long enough (5 us) to be an item of its own, and these items come first: a shared expert of 1777 rows, last
 // in expert order with three or five tiles to a strip, kept single pairs busy for 50 us after everyone else had finished.
 // Behind them the other experts' strips, shared experts first as in the row-space phases.  order[]: the experts in that
-// order, the n_long long ones in front.
+// order, the n_long long ones in front.  With few strips to a CTA pair (strip_split) a strip is cut into `split` ranges of
+// column tiles, whose A operand is loaded again: 8 experts of 192 x 6328 left 58 of 74 pairs without a strip.
 constexpr int WG_LONG_KB = 16;
 MOE_HD int strip_long(int rows) { return (rows + 63) / 64 >= WG_LONG_KB ? 1 : 0; }
 struct StripItem { int e, strip, nb0, nb1; };   // expert, 256-row block of dW, column tiles [nb0, nb1)
-MOE_HD int strip_items(int Ep, int strips, int ntn, int n_long) { return strips * (Ep - n_long + n_long * ntn); }
-MOE_HD StripItem decode_strip_item(int t, int strips, int ntn, int n_long, const int* order) {
+MOE_HD int strip_split(int Ep, int strips, int ntn, int pairs) {
+  const int n = Ep * strips;
+  int split = (8 * pairs + n - 1) / n;          // about eight items for each pair, of at least four tiles
+  if (split > ntn / 4) split = ntn / 4;
+  if (split < 1) split = 1;
+  if (n * split < pairs) {                      // fewer than one: of any size
+    split = (pairs + n - 1) / n;
+    if (split > ntn) split = ntn;
+  }
+  return split;
+}
+MOE_HD int strip_items(int Ep, int strips, int ntn, int split, int n_long) { return strips * ((Ep - n_long) * split + n_long * ntn); }
+MOE_HD StripItem decode_strip_item(int t, int strips, int ntn, int split, int n_long, const int* order) {
   StripItem it;
   const int per = strips * ntn;
   if (t < n_long * per) {
@@ -135,10 +147,11 @@ MOE_HD StripItem decode_strip_item(int t, int strips, int ntn, int n_long, const
     it.nb1 = it.nb0 + 1;
   } else {
     t -= n_long * per;
-    it.e = order[n_long + t / strips];
-    it.strip = t % strips;
-    it.nb0 = 0;
-    it.nb1 = ntn;
+    const int piece = t % split, st = t / split;
+    it.e = order[n_long + st / strips];
+    it.strip = st % strips;
+    it.nb0 = piece * ntn / split;
+    it.nb1 = (piece + 1) * ntn / split;
   }
   return it;
 }
@@ -161,7 +174,20 @@ struct ChainParams {
   int dep_extra;                // test hook: added to the `activated` threshold (> 0 = never reached)
   int want_dw;                  // backward: routing-weight-gradient tasks are part of the vector queue
   int combine_split;            // combine tasks per token (column chunks)
+  int split[SCHED_MAX_SEG];     // weight-gradient phases: ranges of column tiles per strip
+  int batch[SCHED_MAX_SEG];     // items a pair's scheduler takes and decodes together (1, 2 or 4)
 };
+// Ticket, decode and the look at the dependent events are a chain of four or five accesses to L2, 3 us; one at a time that is
+// the pace of a pair whose items are shorter (down with F = 192: 0.7 us of MMAs, 4 us an item).  Items of a few k-blocks are
+// therefore taken two or four at a time.  Not longer ones: the last items of a launch would lie with few pairs.
+MOE_HD int sched_batch(int kblocks) { return kblocks <= 8 ? 4 : kblocks <= 16 ? 2 : 1; }
+// Items a pair holds at most that its epilogue has not begun.
+MOE_HD int sched_hold(int batch) { return batch == 4 ? 8 : 4; }
+// Vector warps per CTA that keep gathering after the first tasks.  Two gather 1.4 TB/s in and out, the pace of gate+up at
+// F = 800 and of act_grad at twice that; below, the matrix items waited for the rows (9678 tokens x 10 rows, F = 536: 250 us of
+// MMAs in 420).  Where the products are longer than the gather, more only take from the bandwidth of their loads.
+MOE_HD int background_gatherers(int is_bwd, int F, int all) { return F <= (is_bwd ? 1536 : 1024) ? all : 2; }
+
 // Gather tasks of M-block `rel` (relative to its expert's first) of an expert with `rows` rows.
 MOE_HD int thr_gathered(int rows, int rel) {
   const int left = ((rows + GROUP_ROWS - 1) & ~(GROUP_ROWS - 1)) - rel * 128;
