@@ -95,6 +95,14 @@ class MoeTfTd(ctypes.Structure):
 
 _lib = None
 
+# The calls of a step go through csrc/fastcall.cpp; it answers None for arguments it does not take as they are, and the
+# functions below then look at them one by one and say what is wrong.  Without it (torch's C++ interface has changed since it
+# was built) everything goes that way.
+try:
+    from . import _fastcall as _fast
+except ImportError:
+    _fast = None
+
 
 def lib_path() -> str:
     return os.path.join(os.path.dirname(os.path.abspath(__file__)), "libmoe_b200.so")
@@ -153,6 +161,9 @@ def load_library() -> ctypes.CDLL:
     lib.moe_strerror.restype = ctypes.c_char_p
     lib.moe_strerror.argtypes = [ctypes.c_int]
     lib.moe_last_cuda_error.restype = ctypes.c_char_p
+    if _fast is not None:
+        _fast.setup(*(ctypes.cast(getattr(lib, f), vp).value for f in (
+            "moe_route", "moe_router_fwd", "moe_router_bwd", "moe_layout_noalloc", "moe_ffn_fwd", "moe_ffn_bwd")))
     _lib = lib
     return lib
 
@@ -270,24 +281,44 @@ def moe_create(T_max, d, E, k, n_shared, F, flags=0, workspace: torch.Tensor | N
     ws_bytes = workspace.numel() if workspace is not None else 0
     _check(load_library().moe_create(ctypes.byref(h), ctypes.byref(s), ws_ptr, ws_bytes), "moe_create")
     _CTX_SHAPE[h.value] = (int(T_max), int(d), int(E), int(k), int(n_shared), int(F), int(flags))
+    if _fast is not None:
+        _fast.add(h, int(T_max), int(d), int(E), int(k), int(n_shared), int(F))
     return h
 
 
 def moe_destroy(ctx):
     _check(load_library().moe_destroy(ctx), "moe_destroy")
+    if _fast is not None:
+        _fast.drop(ctx)
     _CTX_SHAPE.pop(getattr(ctx, "value", None), None)
 
 
-@_sizes_first
 def moe_route(ctx, logits, T, topk_ids, topk_w, counts=None):
+    rc = _fast.route(ctx, logits, T, topk_ids, topk_w, counts) if _fast is not None else None
+    if rc is None:
+        _moe_route(ctx, logits, T, topk_ids, topk_w, counts)
+    elif rc:
+        _check(rc, "moe_route")
+
+
+@_sizes_first
+def _moe_route(ctx, logits, T, topk_ids, topk_w, counts=None):
     _, _, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_route(ctx, _dev(logits, _F32, "logits", T * E), T, _dev(topk_ids, _I32, "topk_ids", T * k),
                                     _dev(topk_w, _F32, "topk_w", T * k), _dev(counts, _I32, "counts", E), _stream()),
            "moe_route")
 
 
-@_sizes_first
 def moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits=None, counts=None):
+    rc = _fast.router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits, counts) if _fast is not None else None
+    if rc is None:
+        _moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits, counts)
+    elif rc:
+        _check(rc, "moe_router_fwd")
+
+
+@_sizes_first
+def _moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits=None, counts=None):
     _, d, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_router_fwd(ctx, _dev(x, _BF, "x", T * d), _dev(W_r, _BF, "W_r", E * d), T,
                                          _dev(topk_ids, _I32, "topk_ids", T * k), _dev(topk_w, _F32, "topk_w", T * k),
@@ -295,8 +326,16 @@ def moe_router_fwd(ctx, x, W_r, T, topk_ids, topk_w, logits=None, counts=None):
            "moe_router_fwd")
 
 
-@_sizes_first
 def moe_router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits):
+    rc = _fast.router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits) if _fast is not None else None
+    if rc is None:
+        _moe_router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits)
+    elif rc:
+        _check(rc, "moe_router_bwd")
+
+
+@_sizes_first
+def _moe_router_bwd(ctx, logits, topk_ids, d_topk_w, T, d_logits):
     _, _, E, k, _, _, _ = _shape_of(ctx)
     _check(load_library().moe_router_bwd(ctx, _dev(logits, _F32, "logits", T * E), _dev(topk_ids, _I32, "topk_ids", T * k),
                                          _dev(d_topk_w, _F32, "d_topk_w", T * k), T, _dev(d_logits, _F32, "d_logits", T * E),
@@ -312,8 +351,16 @@ def moe_layout(ctx, topk_ids, T, counts=None, offsets=None, row_of=None, src_of=
                                      _dev(src_of, _I32, "src_of", n), _stream()), "moe_layout")
 
 
-@_sizes_first
 def moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T):
+    rc = _fast.ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T) if _fast is not None else None
+    if rc is None:
+        _moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T)
+    elif rc:
+        _check(rc, "moe_ffn_fwd")
+
+
+@_sizes_first
+def _moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T):
     _, d, E, k, S, F, _ = _shape_of(ctx)
     td, tk, nw = T * d, T * k, (E + S) * d * F
     _check(load_library().moe_ffn_fwd(ctx, _dev(x, _BF, "x", td), _dev(topk_ids, _I32, "topk_ids", tk),
@@ -321,8 +368,16 @@ def moe_ffn_fwd(ctx, x, topk_ids, topk_w, W_gate_up, W_down, out, T):
                                       _dev(W_down, _BF, "W_down", nw), _dev(out, _BF, "out", td), T, _stream()), "moe_ffn_fwd")
 
 
-@_sizes_first
 def moe_ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T):
+    rc = _fast.ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T) if _fast is not None else None
+    if rc is None:
+        _moe_ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T)
+    elif rc:
+        _check(rc, "moe_ffn_bwd")
+
+
+@_sizes_first
+def _moe_ffn_bwd(ctx, dout, x, topk_ids, topk_w, W_gate_up, W_down, dx, dW_gate_up, dW_down, d_topk_w, T):
     _, d, E, k, S, F, _ = _shape_of(ctx)
     td, tk, nw = T * d, T * k, (E + S) * d * F
     _check(load_library().moe_ffn_bwd(ctx, _dev(dout, _BF, "dout", td), _dev(x, _BF, "x", td),
@@ -389,10 +444,18 @@ def moe_route_host(ctx, logits_host, T, topk_ids_host, topk_w_host):
                                          _host(topk_w_host, _F32, "topk_w_host", T * k), _stream()), "moe_route_host")
 
 
-@_sizes_first
 def moe_layout_noalloc(topk_ids, T, E, k, n_shared, counts, offsets, row_of, src_of, status2=None):
     """Dispatch layout through the entry point that allocates nothing and needs no context (for
     callers that may not cudaMalloc).  All tensors are caller-owned CUDA int32 tensors."""
+    rc = _fast.layout_noalloc(topk_ids, T, E, k, n_shared, counts, offsets, row_of, src_of, status2) if _fast is not None else None
+    if rc is None:
+        _moe_layout_noalloc(topk_ids, T, E, k, n_shared, counts, offsets, row_of, src_of, status2)
+    elif rc:
+        _check(rc, "moe_layout_noalloc")
+
+
+@_sizes_first
+def _moe_layout_noalloc(topk_ids, T, E, k, n_shared, counts, offsets, row_of, src_of, status2=None):
     n, Ep = T * (k + n_shared), E + n_shared
     # a problem beyond the entry point's fixed limits is refused by the library itself before it touches memory
     fits = 0 <= n <= 262144 and Ep <= 1088 and -(-n // 2048) * Ep <= 131072
@@ -634,6 +697,12 @@ class MoeLayer:
             pass
 
     def route(self, logits, with_counts=False):
+        if not with_counts and _fast is not None:
+            r = _fast.route_new(self.ctx, logits)
+            if r is not None:
+                if r[0]:
+                    _check(r[0], "moe_route")
+                return r[1], r[2]
         T = logits.shape[0]
         dev = logits.device
         ids = torch.empty(T, self.k, dtype=_I32, device=dev)
@@ -652,6 +721,12 @@ class MoeLayer:
         return counts, offsets, row_of, src_of
 
     def ffn_fwd(self, x, topk_ids, topk_w, W_gate_up, W_down, out=None):
+        if out is None and _fast is not None:
+            r = _fast.ffn_fwd_new(self.ctx, x, topk_ids, topk_w, W_gate_up, W_down)
+            if r is not None:
+                if r[0]:
+                    _check(r[0], "moe_ffn_fwd")
+                return r[1]
         T = x.shape[0]
         if out is None:
             out = torch.empty(T, self.d, dtype=_BF, device=x.device)

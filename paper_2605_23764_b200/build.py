@@ -1,14 +1,16 @@
-"""Builds libmoe_b200.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds libmoe_b200.so in-tree with nvcc for sm_100a (no JIT cache), and _fastcall.so, the step calls' way in from Python."""
 from __future__ import annotations
 
 import concurrent.futures
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 OUT = os.path.join(PKG, "libmoe_b200.so")
+FAST = os.path.join(PKG, "_fastcall.so")
 OBJ = os.path.join(PKG, "_build")
 SOURCES = ["api.cu", "route_layout.cu", "permute.cu", "gemm_tc3.cu", "gemm_wgrad.cu", "fused.cu", "study.cu", "router.cu", "taskflow.cu", "ep.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -23,9 +25,9 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(OUT):
+    if not (os.path.exists(OUT) and os.path.exists(FAST)):
         return True
-    t = os.path.getmtime(OUT)
+    t = min(os.path.getmtime(OUT), os.path.getmtime(FAST))
     inc = os.path.join(PKG, "..", "include")
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(inc, f) for f in os.listdir(inc)]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -42,13 +44,30 @@ def _compile(src: str) -> str:
     return obj
 
 
+def _build_fastcall() -> None:
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = FAST + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"),
+           os.path.join(CSRC, "fastcall.cpp"), "-o", tmp, "-L" + os.path.join(root, "lib"),
+           "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on fastcall.cpp:\n{r.stdout}{r.stderr}")
+    os.replace(tmp, FAST)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source for sm_100a and link the C-ABI shared library.  Returns its path."""
     if not force and not _stale():
         return OUT
     os.makedirs(OBJ, exist_ok=True)
-    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        fast = ex.submit(_build_fastcall)
         objs = list(ex.map(_compile, SOURCES))
+        fast.result()
     tmp = OUT + f".tmp{os.getpid()}"
     cmd = [_nvcc(), "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
     subprocess.check_call(cmd)
