@@ -211,7 +211,6 @@ struct moe_ctx {
   int* last_ctr = nullptr;      // event counters of the last persistent launch
   bool bwd_ctr_clear = false;   // the backward's event counters are zero (the forward's layout clears both sets)
   int dep_extra = 0;  // test hook: makes the activation dependencies of the persistent launch unreachable
-  bool plain_launch = false;  // diagnostic: persistent launches without the cooperative attribute
   cudaStream_t last_stream = nullptr;
   // host-buffer entry points: a copy-in stream (the next call's large input arrives while the previous
   // call still computes) and a copy-out stream (the result leaves in token chunks behind the combine)
@@ -621,7 +620,7 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     fa.combine_rows = c->at<uint16_t>(p.Y);
     fa.combine_out = out;
     Phase ph(c, MOE_PHASE_FUSED_FWD, st);
-    MOE_CUDA(launch_fused(false, fa, c->num_sms, !c->plain_launch, st, &c->launches));
+    MOE_CUDA(launch_fused(false, fa, c->num_sms, st, &c->launches));
     if (x_free) MOE_CUDA(cudaEventRecord(x_free, st));
     if (out_host && (rc = copy_out_to_host(c, out, out_host, 2 * (size_t)T * c->shape.d, st))) return rc;
   }
@@ -714,7 +713,7 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     const CUdeviceptr ready_word = reinterpret_cast<CUdeviceptr>(fa.ctr + CTR_OUT_READY);
     fa.announce_out = early_out ? 1 : 0;
     if (early_out) MOE_CUDA(cudaEventRecord(c->ev_chunk[0], st));   // the word is cleared before anyone waits on it
-    MOE_CUDA(launch_fused(true, fa, c->num_sms, !c->plain_launch, st, &c->launches));
+    MOE_CUDA(launch_fused(true, fa, c->num_sms, st, &c->launches));
     if (dout_free) MOE_CUDA(cudaEventRecord(dout_free, st));
     if (early_out) {
       // The launch and everything that sets the word are submitted before the wait for it: streams share hardware queues, and
@@ -1083,8 +1082,7 @@ int moe_debug_set_plain_launch(moe_ctx* c, int32_t on) {
     study_plain_launch().store(on != 0);
     return MOE_OK;
   }
-  c->plain_launch = on != 0;
-  return MOE_OK;
+  return MOE_OK;   // a context's launches are made without the attribute anyway
 }
 
 int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {

@@ -1,6 +1,6 @@
 // The single persistent, dependency-driven launch of the forward (and of the backward) layer.
 //
-// One cooperative grid of one CTA per SM in clusters of two runs the whole operator chain.  Per CTA:
+// One grid of one CTA per SM in clusters of two runs the whole operator chain.  Per CTA:
 //   warp 0      TMA producer of the weights (weight gradients: of the A operand)
 //   warp 1      tcgen05.mma issuer (even CTA) and TMEM owner
 //   warps 2-5, 8-11  epilogue: TMEM -> fused element-wise math -> global memory, then the tile's trigger event
@@ -500,11 +500,15 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   cluster_sync_all();  // both CTAs' barriers exist before anyone signals across the pair
   tc_fence_after_sync();
   const uint32_t tmem_base = uniform(bars->tmem_base);
+  // (No trigger for the next launch: a router that takes the SMs as this launch's CTAs leave them is 2-3 % slower.)
   pdl_wait();   // the layout's tables, and everything else in front of this launch
   const int M = fa.lv.meta[0];
 
   if (warp == SCHED_WARP && rank == 0) {
     // ------------------------------------------------ scheduler of the pair (even CTA)
+    // the first ticket is on its way while the tables are read
+    int first_ticket = 0;
+    if (lane == 0) first_ticket = atomicAdd(&fa.ctr[CTR_MAT_TICKET], 1);
     const PhaseTable pt = make_phase_table<BWD>(fa);
     const PhaseTable rot = make_rotation_table<BWD>(fa);   // first item of the first shared expert in each row-space phase
     const int total = pt.start[SCHED_MAX_SEG];
@@ -515,7 +519,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       const int items = pt.start[p + 1] - pt.start[p], most = fa.cp.batch[p];   // 16 and 8 for each pair
       batches |= (items >= 8 * (int)gridDim.x && most == 4 ? 2 : items >= 4 * (int)gridDim.x && most >= 2 ? 1 : 0) << (2 * p);
     }
-    int batch = 1 << (batches & 3);   // of the phase the last ticket belonged to
+    int batch = 1;   // of the phase the last ticket belonged to
     bool more = true;
     for (uint32_t n = 0; more;) {
       // the item sched_hold() before the batch's last has been taken first, then the tickets
@@ -524,8 +528,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (lane == 0 && next > hold)
         ok = mbar_wait_cluster(&ring->empty[(next - 1 - hold) % TK_RING], ((next - 1 - hold) / TK_RING) & 1, wc, SITE_EMPTY, -7, 100) ? 1 : 0;
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-      int t = 0;
-      if (lane == 0) t = atomicAdd(&fa.ctr[CTR_MAT_TICKET], batch);
+      int t = first_ticket;
+      if (lane == 0 && n > 0) t = atomicAdd(&fa.ctr[CTR_MAT_TICKET], batch);
       t = __shfl_sync(0xffffffffu, t, 0);
       // `batch` groups of lanes decode a ticket each; a group's lanes share the look at its item's events
       const int lanes = 32 / batch, group = lane / lanes, sub = lane - group * lanes;
@@ -620,12 +624,12 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
 
 int vector_warps() { return VEC_WARPS; }
 
-cudaError_t launch_fused(bool bwd, const FusedArgs& fa, int num_sms, bool cooperative, cudaStream_t s, int* launches) {
+cudaError_t launch_fused(bool bwd, const FusedArgs& fa, int num_sms, cudaStream_t s, int* launches) {
   ++*launches;
   static PairLaunchState st_fwd, st_bwd;
   if (bwd)
-    return launch_on_pairs(st_bwd, fused_chain_kernel<true>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, cooperative, s, true);
-  return launch_on_pairs(st_fwd, fused_chain_kernel<false>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, cooperative, s, true);
+    return launch_on_pairs(st_bwd, fused_chain_kernel<true>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, s, true);
+  return launch_on_pairs(st_fwd, fused_chain_kernel<false>, fa, FUSED_THREADS, FUSED_SMEM_BYTES, num_sms, s, true);
 }
 
 }  // namespace moe

@@ -95,8 +95,7 @@ void plan_ring(GemmMode mode, int T, GemmArgs& a) {
 template <int MODE>
 static cudaError_t launch_swap_mode(const GemmArgs& a, int num_sms, cudaStream_t s) {
   static PairLaunchState st;
-  return launch_on_pairs(st, grouped_gemm_swap_kernel<MODE>, a, GEMM3_THREADS, GEMM3_SMEM_BYTES, num_sms,
-                         false, s);
+  return launch_on_pairs(st, grouped_gemm_swap_kernel<MODE>, a, GEMM3_THREADS, GEMM3_SMEM_BYTES, num_sms, s);
 }
 
 cudaError_t launch_gemm3(GemmMode mode, const GemmArgs& a, int num_sms, cudaStream_t s, int* launches) {

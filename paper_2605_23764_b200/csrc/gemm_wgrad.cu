@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) grouped_wgrad_pair_kernel(const
 cudaError_t launch_wgrad_strips(const GemmArgs& a, int num_sms, cudaStream_t s, int* launches) {
   ++*launches;
   static PairLaunchState st;
-  return launch_on_pairs(st, grouped_wgrad_pair_kernel, a, WG_THREADS, WGRAD_SMEM_BYTES, num_sms, false, s);
+  return launch_on_pairs(st, grouped_wgrad_pair_kernel, a, WG_THREADS, WGRAD_SMEM_BYTES, num_sms, s);
 }
 
 }  // namespace moe

@@ -21,7 +21,7 @@ struct PairLaunchState {
 
 template <class Kernel, class Args>
 cudaError_t launch_on_pairs(PairLaunchState& st, Kernel kernel, const Args& args, int threads, size_t smem_bytes,
-                            int num_sms, bool cooperative, cudaStream_t s, bool dependent = false) {
+                            int num_sms, cudaStream_t s, bool dependent = false) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -32,17 +32,13 @@ cudaError_t launch_on_pairs(PairLaunchState& st, Kernel kernel, const Args& args
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = s;
-  cudaLaunchAttribute attr[3];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cooperative) {   // the launch fails rather than run with CTAs that are not all resident
-    attr[cfg.numAttrs].id = cudaLaunchAttributeCooperative;
-    attr[cfg.numAttrs++].val.cooperative = 1;
-  }
   int pairs = 0;
   {
     std::lock_guard<std::mutex> lock(st.mu);

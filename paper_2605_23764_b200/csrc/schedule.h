@@ -26,8 +26,10 @@
 //
 // Deadlock freedom: every item's producers have smaller tickets (an earlier phase) or are vector
 // tasks that never wait for matrix items of the same or a later phase; tickets are taken in order
-// by pairs that are all resident (cooperative launch), so the holder of the smallest unfinished
-// ticket always finds its dependent events met in finite time.
+// and only by CTAs that are running, so the holder of the smallest unfinished ticket always finds its dependent events
+// met in finite time -- with any number of CTAs resident, as when another stream's launch holds some of the SMs: a CTA
+// that has not started holds nothing.  Vector tasks alike: a worker that waits in the second queue is not one of the
+// background gatherers, which empty the first.
 #pragma once
 
 #include <stdint.h>
