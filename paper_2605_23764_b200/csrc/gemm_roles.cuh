@@ -211,7 +211,7 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem,
   uint8_t* sT = smem + stages * W_STAGE_BYTES;     // [stages][tokb] tokens (this CTA's half)
   // with events: the tokens are there (acquired by the scheduler and handed on through the ticket ring, or by the caller);
   // what the producers wrote must be seen by the TMA loads
-  if (DEP::kOn && tok_warp) fence_proxy_async();
+  if (DEP::kOn && tok_warp) fence_proxy_async_global();
   const int nkb = uniform(wk.a.nkb), e = uniform(wk.a.e), n0 = uniform(wk.a.n0);
   const int row_a = uniform(wk.a.row0), half_a = uniform(wk.a.ntok) >> 1;
   const int row_b = uniform(wk.b.row0), half_b = wk.merged ? uniform(wk.b.ntok) >> 1 : 0;
@@ -406,7 +406,7 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
   uint8_t* sB = smem + WG_A_SLOTS * A_STAGE_BYTES;     // [WG_B_STAGES][16 KB] B stages
   const int m0 = uniform(st.m0(rank)), row0 = uniform(st.row0), nkb = uniform(st.nkb);
   const bool resident = nkb <= A_RES_KB;
-  if (DEP::kOn) fence_proxy_async();   // as in swap_load_item
+  if (DEP::kOn) fence_proxy_async_global();   // as in swap_load_item
   const int nb0 = uniform(st.nb0), nb1 = uniform(st.nb1);
   for (int nb = nb0; nb < nb1; ++nb) {
     const bool load_a = !resident || nb == nb0;
