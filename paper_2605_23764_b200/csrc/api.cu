@@ -91,8 +91,8 @@ int encode_tiled(CUtensorMap* tm, const void* base, int rank, const uint64_t* di
 
 // Row-major [rows][cols] matrix, box [box_rows][box_cols].
 int encode_2d(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows,
-              uint32_t box_cols) {
-  const uint64_t dims[2] = {cols, rows}, strides[1] = {cols * 2};
+              uint32_t box_cols, uint64_t ld = 0 /* elements from row to row; 0: cols */) {
+  const uint64_t dims[2] = {cols, rows}, strides[1] = {(ld ? ld : cols) * 2};
   const uint32_t box[2] = {box_cols, box_rows};
   return encode_tiled(tm, base, 2, dims, strides, box);
 }
@@ -171,12 +171,12 @@ WsPlan plan_workspace(const moe_shape& s) {
   p.group_slot = c.take(sizeof(int) * cap);
   p.prow_w = c.take(sizeof(float) * cap);
   p.dw_partial = c.take(train ? sizeof(float) * cap * p.ntn_act * DW_PARTS_PER_TILE : 0);
-  p.Xp = c.take(2 * cap * s.d);
-  p.H = c.take(train ? 2 * cap * 2 * s.F : 0);
-  p.A = c.take(2 * cap * s.F);
-  p.Y = c.take(2 * cap * s.d);
-  p.dOutp = c.take(train ? 2 * cap * s.d : 0);
-  p.dH = c.take(train ? 2 * cap * 2 * s.F : 0);
+  p.Xp = c.take(2 * cap * row_ld(s.d));
+  p.H = c.take(train ? 2 * cap * row_ld(2 * s.F) : 0);
+  p.A = c.take(2 * cap * row_ld(s.F));
+  p.Y = c.take(2 * cap * row_ld(s.d));
+  p.dOutp = c.take(train ? 2 * cap * row_ld(s.d) : 0);
+  p.dH = c.take(train ? 2 * cap * row_ld(2 * s.F) : 0);
   for (int i = 0; i < 2; ++i) p.st_x[i] = c.take(2 * (size_t)s.T_max * s.d);   // the next call's arrives while this call reads its own
   p.st_dout = c.take(train ? 2 * (size_t)s.T_max * s.d : 0);
   p.st_ids = c.take(sizeof(int) * (size_t)s.T_max * s.k);
@@ -212,6 +212,8 @@ struct moe_ctx {
   bool bwd_ctr_clear = false;   // the backward's event counters are zero (the forward's layout clears both sets)
   int dep_extra = 0;  // test hook: makes the activation dependencies of the persistent launch unreachable
   cudaStream_t last_stream = nullptr;
+  void* debug_copy = nullptr;   // moe_debug_buffer: the last row-space tensor asked for, compact
+  size_t debug_bytes = 0;
   // host-buffer entry points: a copy-in stream (the next call's large input arrives while the previous
   // call still computes) and a copy-out stream (the result leaves in token chunks behind the combine)
   bool copy_ready = false;
@@ -378,7 +380,6 @@ GemmArgs args_act_grad(const moe_ctx* c, int T, bool want_dw) {
   g.b_rows_per_expert = s.d;
   g.out0 = c->at<uint16_t>(p.dH);
   g.in0 = c->at<uint16_t>(p.H);
-  g.ld_in0 = 2 * s.F;
   g.prow_w = c->at<float>(p.prow_w);
   g.dw_partial = want_dw ? c->at<float>(p.dw_partial) : nullptr;
   return g;
@@ -776,19 +777,20 @@ int moe_create(moe_ctx** out, const moe_shape* shape, void* workspace, size_t wo
   const WsPlan& p = c->plan;
   const uint64_t cap = p.cap_rows;
   const bool train = c->train();
+  const uint64_t ld_d = row_ld(s.d), ld_F = row_ld(s.F), ld_2F = row_ld(2 * s.F);
   int rc = MOE_OK;
   cudaError_t e = cudaMemset(c->ws, 0, p.Xp);  // status, tables and small arrays start at zero
   if (e != cudaSuccess) rc = cuda_fail(e, "cudaMemset(workspace)");
-  if (!rc && train) rc = encode_2d(&c->tm_dOutp_mn, c->ws + p.dOutp, cap, s.d, 64, 64);
-  if (!rc && train) rc = encode_2d(&c->tm_A_mn, c->ws + p.A, cap, s.F, 64, 64);
-  if (!rc && train) rc = encode_2d(&c->tm_dH_mn, c->ws + p.dH, cap, 2 * s.F, 64, 64);
-  if (!rc && train) rc = encode_2d(&c->tm_Xp_mn, c->ws + p.Xp, cap, s.d, 64, 64);
+  if (!rc && train) rc = encode_2d(&c->tm_dOutp_mn, c->ws + p.dOutp, cap, s.d, 64, 64, ld_d);
+  if (!rc && train) rc = encode_2d(&c->tm_A_mn, c->ws + p.A, cap, s.F, 64, 64, ld_F);
+  if (!rc && train) rc = encode_2d(&c->tm_dH_mn, c->ws + p.dH, cap, 2 * s.F, 64, 64, ld_2F);
+  if (!rc && train) rc = encode_2d(&c->tm_Xp_mn, c->ws + p.Xp, cap, s.d, 64, 64, ld_d);
   for (int i = 0; i < 8 && !rc; ++i) {
     const uint32_t br = 16u * (i + 1);
-    rc = encode_2d(&c->tk_Xp[i], c->ws + p.Xp, cap, s.d, br, 64);
-    if (!rc) rc = encode_2d(&c->tk_A[i], c->ws + p.A, cap, s.F, br, 64);
-    if (!rc && train) rc = encode_2d(&c->tk_dOutp[i], c->ws + p.dOutp, cap, s.d, br, 64);
-    if (!rc && train) rc = encode_2d(&c->tk_dH[i], c->ws + p.dH, cap, 2 * s.F, br, 64);
+    rc = encode_2d(&c->tk_Xp[i], c->ws + p.Xp, cap, s.d, br, 64, ld_d);
+    if (!rc) rc = encode_2d(&c->tk_A[i], c->ws + p.A, cap, s.F, br, 64, ld_F);
+    if (!rc && train) rc = encode_2d(&c->tk_dOutp[i], c->ws + p.dOutp, cap, s.d, br, 64, ld_d);
+    if (!rc && train) rc = encode_2d(&c->tk_dH[i], c->ws + p.dH, cap, 2 * s.F, br, 64, ld_2F);
   }
   if (rc) {
     if (c->owns_ws) cudaFree(c->ws);
@@ -819,6 +821,7 @@ int moe_destroy(moe_ctx* c) {
     cudaEventDestroy(c->ev_d2h_done);
     for (int i = 0; i < HOST_CHUNKS; ++i) cudaEventDestroy(c->ev_chunk[i]);
   }
+  if (c->debug_copy) cudaFree(c->debug_copy);
   if (c->owns_ws) cudaFree(c->ws);
   delete c;
   return MOE_OK;
@@ -1091,7 +1094,7 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
   const WsPlan& p = c->plan;
   const size_t Ep = s.E + s.n_shared, slots = (size_t)s.T_max * (s.k + s.n_shared), cap = p.cap_rows;
   const bool train = c->train();
-  size_t off = 0, n = 0;
+  size_t off = 0, n = 0, cols = 0;   // cols: columns of a row-space tensor
   switch (which) {
     case MOE_BUF_COUNTS: off = p.counts; n = Ep; break;
     case MOE_BUF_OFFSETS: off = p.offsets; n = Ep + 1; break;
@@ -1099,20 +1102,34 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
     case MOE_BUF_SRC_OF: off = p.src_of; n = slots; break;
     case MOE_BUF_PROW_OF: off = p.prow_of; n = slots; break;
     case MOE_BUF_PAD_OFF: off = p.pad_off; n = Ep + 1; break;
-    case MOE_BUF_XP: off = p.Xp; n = cap * s.d; break;
-    case MOE_BUF_H: if (!train) return MOE_ERR_STATE; off = p.H; n = cap * 2 * s.F; break;
-    case MOE_BUF_A: off = p.A; n = cap * s.F; break;
-    case MOE_BUF_Y: off = p.Y; n = cap * s.d; break;
-    case MOE_BUF_DOUTP: if (!train) return MOE_ERR_STATE; off = p.dOutp; n = cap * s.d; break;
-    case MOE_BUF_DH: if (!train) return MOE_ERR_STATE; off = p.dH; n = cap * 2 * s.F; break;
-    case MOE_BUF_DXP: off = p.Y; n = cap * s.d; break;
+    case MOE_BUF_XP: off = p.Xp; cols = s.d; break;
+    case MOE_BUF_H: if (!train) return MOE_ERR_STATE; off = p.H; cols = 2 * s.F; break;
+    case MOE_BUF_A: off = p.A; cols = s.F; break;
+    case MOE_BUF_Y: off = p.Y; cols = s.d; break;
+    case MOE_BUF_DOUTP: if (!train) return MOE_ERR_STATE; off = p.dOutp; cols = s.d; break;
+    case MOE_BUF_DH: if (!train) return MOE_ERR_STATE; off = p.dH; cols = 2 * s.F; break;
+    case MOE_BUF_DXP: off = p.Y; cols = s.d; break;
     case MOE_BUF_META: off = p.meta; n = 8; break;
     case MOE_BUF_TRACE: if (!p.trace_cap) return MOE_ERR_STATE; off = p.trace; n = (size_t)p.trace_cap * 8; break;
     case MOE_BUF_EVENT_COUNTERS: off = c->last_ctr ? (size_t)(reinterpret_cast<uint8_t*>(c->last_ctr) - c->ws) : p.ctr; n = p.ctr_count; break;
     default: return MOE_ERR_INVALID_ARG;
   }
   *ptr = c->ws + off;
-  *elems = n;
+  *elems = cols ? cap * cols : n;
+  if (cols && cols != (size_t)row_ld((int)cols)) {   // rows are farther apart in the workspace: a compact copy
+    const size_t ld = row_ld((int)cols), bytes = 2 * cap * cols;
+    if (bytes > c->debug_bytes) {
+      MOE_CUDA(cudaStreamSynchronize(c->last_stream));
+      if (c->debug_copy) MOE_CUDA(cudaFree(c->debug_copy));
+      c->debug_copy = nullptr;
+      c->debug_bytes = 0;
+      MOE_CUDA(cudaMalloc(&c->debug_copy, bytes));
+      c->debug_bytes = bytes;
+    }
+    MOE_CUDA(cudaMemcpy2DAsync(c->debug_copy, 2 * cols, c->ws + off, 2 * ld, 2 * cols, cap, cudaMemcpyDeviceToDevice, c->last_stream));
+    MOE_CUDA(cudaStreamSynchronize(c->last_stream));
+    *ptr = c->debug_copy;
+  }
   return MOE_OK;
 }
 

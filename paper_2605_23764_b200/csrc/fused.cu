@@ -70,7 +70,8 @@ __device__ __forceinline__ int vec_gather(const FusedArgs& fa, int task, int lan
       w = j < k ? fa.topk_w[(size_t)t * k + j] : 1.0f;
     }
   }
-  uint4* out = reinterpret_cast<uint4*>(fa.gather_dst + (size_t)p0 * fa.d);
+  const int ldv = row_ld(fa.d) >> 3;
+  uint4* out = reinterpret_cast<uint4*>(fa.gather_dst) + (size_t)p0 * ldv;
   constexpr int U = 16 / GATHER_ROWS;
   for (int v = lane; v < nvec; v += 32 * U) {
     uint4 q[GATHER_ROWS][U];
@@ -83,7 +84,7 @@ __device__ __forceinline__ int vec_gather(const FusedArgs& fa, int task, int lan
     for (int r = 0; r < GATHER_ROWS; ++r)
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (v + 32 * u < nvec) out[(size_t)r * nvec + v + 32 * u] = q[r][u];   // padding rows are zero-filled
+        if (v + 32 * u < nvec) out[(size_t)r * ldv + v + 32 * u] = q[r][u];   // padding rows are zero-filled
   }
   if (fa.prow_w && lane < GATHER_ROWS) fa.prow_w[p0 + lane] = w;
   return p0 / BLOCK_M;
@@ -122,7 +123,7 @@ __device__ __forceinline__ bool vec_combine(const FusedArgs& fa, int task, int l
         for (int u = 0; u < 8; ++u) {
           const int j = j0 + u;
           const int p = j < kp ? prow[j] : -1;
-          const uint4* row = reinterpret_cast<const uint4*>(fa.combine_rows + (size_t)(p >= 0 ? p : 0) * fa.d);
+          const uint4* row = reinterpret_cast<const uint4*>(fa.combine_rows + (size_t)(p >= 0 ? p : 0) * row_ld(fa.d));
           r[u] = p >= 0 ? ldg_cg_v4(row + v) : make_uint4(0, 0, 0, 0);
           r2[u] = (p >= 0 && two) ? ldg_cg_v4(row + v + 32) : make_uint4(0, 0, 0, 0);
         }

@@ -188,7 +188,8 @@ __device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile&
     if (f0 >= a.N) return true;
     const int part = lane & 3;
     const bool inside = f0 + part * 8 < a.N;     // N % 8 == 0: a 16-byte piece is inside or outside as a whole
-    uint16_t* const out = a.out0 + (size_t)st.row0 * a.N + f0 + part * 8;
+    const size_t ld = row_ld(a.N);
+    uint16_t* const out = a.out0 + st.row0 * ld + f0 + part * 8;
 #pragma unroll 1
     for (int c0 = first; c0 < st.ntok; c0 += 2 * CH) {
       float v[32];   // [features 0.. | 16..][token group of 8][feature, feature + 8][token pair]
@@ -207,7 +208,7 @@ __device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile&
       for (int i = 0; i < 4; ++i) {
         const int t = (lane + 32 * i) >> 2;
         const uint4 q = *reinterpret_cast<const uint4*>(staging + piece64(t, part));
-        if (inside) *reinterpret_cast<uint4*>(out + (size_t)(c0 + t) * a.N) = q;
+        if (inside) *reinterpret_cast<uint4*>(out + (c0 + t) * ld) = q;
       }
     }
   } else if (MODE == GEMM_GATE_UP) {
@@ -225,7 +226,7 @@ __device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile&
     if (first < st.ntok) fetch(first);
     const int part = lane & 1;
     const bool inside = fw0 + 8 * part < a.F;     // F % 8 == 0
-    const size_t col = fw0 + 8 * part;
+    const size_t col = fw0 + 8 * part, ld_a = row_ld(a.F), ld_h = row_ld(2 * a.F);
 #pragma unroll 1
     for (int c0 = first; c0 < st.ntok; c0 += 2 * CH) {
       float v[32];   // [features 0..7 | 8..15][token group of 8][gate, up][token pair]
@@ -262,10 +263,10 @@ __device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile&
         const uint8_t* piece = staging + piece32(t, part);
         const size_t row = st.row0 + c0 + t;
         if (inside) {
-          *reinterpret_cast<uint4*>(a.out0 + row * a.F + col) = *reinterpret_cast<const uint4*>(piece);
+          *reinterpret_cast<uint4*>(a.out0 + row * ld_a + col) = *reinterpret_cast<const uint4*>(piece);
           if (a.out1) {
-            *reinterpret_cast<uint4*>(a.out1 + row * (2 * (size_t)a.F) + col) = *reinterpret_cast<const uint4*>(piece + 1024);
-            *reinterpret_cast<uint4*>(a.out1 + row * (2 * (size_t)a.F) + a.F + col) = *reinterpret_cast<const uint4*>(piece + 2048);
+            *reinterpret_cast<uint4*>(a.out1 + row * ld_h + col) = *reinterpret_cast<const uint4*>(piece + 1024);
+            *reinterpret_cast<uint4*>(a.out1 + row * ld_h + a.F + col) = *reinterpret_cast<const uint4*>(piece + 2048);
           }
         }
       }
@@ -288,15 +289,16 @@ __device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile&
     // are the forward launch's, so the first ones are on their way before the accumulator is ready.
     const int part = lane & 3;
     const bool inside = f0 + part * 8 < a.F;     // F % 8 == 0
-    const uint16_t* hbase = a.in0 + (size_t)st.row0 * a.ld_in0 + f0 + part * 8;
-    uint16_t* const out = a.out0 + (size_t)st.row0 * a.ld_in0 + f0 + part * 8;   // dH has H's layout
+    const size_t ld = row_ld(2 * a.F);           // H and dH
+    const uint16_t* hbase = a.in0 + st.row0 * ld + f0 + part * 8;
+    uint16_t* const out = a.out0 + st.row0 * ld + f0 + part * 8;
     const float* wsrc = a.prow_w + st.row0 + 2 * (lane & 3);
     uint4 pre[4];
     float2 w_next[2];
     auto fetch = [&](int tok0) {
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const uint16_t* p = hbase + (size_t)(tok0 + ((lane + 32 * i) >> 2)) * a.ld_in0;
+        const uint16_t* p = hbase + (tok0 + ((lane + 32 * i) >> 2)) * ld;
         pre[2 * i] = inside ? ld_nc_v4(p) : make_uint4(0, 0, 0, 0);
         pre[2 * i + 1] = inside ? ld_nc_v4(p + a.F) : make_uint4(0, 0, 0, 0);
         w_next[i] = *reinterpret_cast<const float2*>(wsrc + tok0 + 8 * i);
@@ -350,8 +352,8 @@ __device__ __forceinline__ bool epilogue_swap(const GemmArgs& a, const SwapTile&
         const uint4 dg = *reinterpret_cast<const uint4*>(staging + piece64(t, part));
         const uint4 du = *reinterpret_cast<const uint4*>(staging + 1024 + piece64(t, part));
         if (inside) {
-          *reinterpret_cast<uint4*>(out + (size_t)(h0 + t) * a.ld_in0) = dg;
-          *reinterpret_cast<uint4*>(out + (size_t)(h0 + t) * a.ld_in0 + a.F) = du;
+          *reinterpret_cast<uint4*>(out + (h0 + t) * ld) = dg;
+          *reinterpret_cast<uint4*>(out + (h0 + t) * ld + a.F) = du;
         }
       }
       if (a.dw_partial) {

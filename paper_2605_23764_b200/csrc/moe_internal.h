@@ -26,6 +26,11 @@ inline int padded_rows_max(int T_max, int kp, int Ep) {
   return (int)(((r + BLOCK_M - 1) / BLOCK_M) * BLOCK_M);
 }
 
+// Elements from row to row of the row-space tensors (Xp, H, A, Y, dOutp, dH): whole 128-byte lines.  A row of 64 columns that
+// starts inside a line is two lines to a TMA box and partial sectors to a store: with 2056 instead of 2048 columns a pass
+// took 17-20 % longer, half of it for these tensors (the caller's weights have the caller's rows).
+constexpr __host__ __device__ int row_ld(int cols) { return (cols + 63) & ~63; }
+
 constexpr int LAYOUT_CHUNK = 2048;  // flat slots per block of the layout kernels
 
 // Device arrays describing one dispatch layout.
@@ -121,12 +126,11 @@ struct GemmArgs {
   int stages;          // operand stages
   int tok_bytes;       // token bytes of a stage per CTA
   // epilogue tensors
-  uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]
+  uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]; rows row_ld(..) apart
   uint16_t* out1;      // GATE_UP: H [rows][2F], NULL: the pre-activations are not kept
   const uint16_t* in0; // ACT_GRAD: H
   const float* prow_w; // GATE_UP, ACT_GRAD: routing weight per padded row
   float* dw_partial;   // ACT_GRAD: [R_pad][n_tiles_n] partial <dA_unweighted, a> (may be NULL)
-  long ld_in0;
   DevStatus* status;
   uint64_t budget_ns;
 };

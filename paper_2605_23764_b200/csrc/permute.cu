@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(PERM_THREADS) gather_rows_kernel(const uint16_
   const int nvec = d >> 3;
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     const GatherRow r = gather_row(lv, i, topk_w, k, kp);
-    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)r.p * d);
+    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)r.p * row_ld(d));
     const uint4* in = reinterpret_cast<const uint4*>(src + (size_t)(r.t < 0 ? 0 : r.t) * d);
     for (int v = threadIdx.x; v < nvec; v += PERM_THREADS) out[v] = r.t < 0 ? make_uint4(0, 0, 0, 0) : ld_nc_v4(in + v);
     if (prow_w && threadIdx.x == 0) prow_w[r.p] = r.w;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(PERM_THREADS) gather_rows_warp_kernel(const ui
   constexpr int WPB = PERM_THREADS / 32;
   for (int i = blockIdx.x * WPB + warp; i < n; i += gridDim.x * WPB) {
     const GatherRow r = gather_row(lv, i, topk_w, k, kp);
-    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)r.p * d);
+    uint4* out = reinterpret_cast<uint4*>(dst + (size_t)r.p * row_ld(d));
     const uint4* in = reinterpret_cast<const uint4*>(src + (size_t)(r.t < 0 ? 0 : r.t) * d);
     for (int v = lane; v < nvec; v += 32) out[v] = r.t < 0 ? make_uint4(0, 0, 0, 0) : ld_nc_v4(in + v);
     if (prow_w && lane == 0) prow_w[r.p] = r.w;
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(32) gather_rows_bulk_kernel(const uint16_t* __
       from = my + (size_t)b * row_bytes;
     }
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                 ::"l"(dst + (size_t)cur.p * d), "r"(smem_u32(from)), "r"(row_bytes)
+                 ::"l"(dst + (size_t)cur.p * row_ld(d)), "r"(smem_u32(from)), "r"(row_bytes)
                  : "memory");
     tma_store_commit();
     cur = next;
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(PERM_THREADS) combine_rows_kernel(const uint16
       for (int j = 0; j < kp; ++j) {
         int p = prow_of[(size_t)t * kp + j];
         if (p < 0) continue;
-        uint4 r = ld_nc_v4(reinterpret_cast<const uint4*>(rows + (size_t)p * d) + v);
+        uint4 r = ld_nc_v4(reinterpret_cast<const uint4*>(rows + (size_t)p * row_ld(d)) + v);
         acc[0] += bf16lo(r.x); acc[1] += bf16hi(r.x);
         acc[2] += bf16lo(r.y); acc[3] += bf16hi(r.y);
         acc[4] += bf16lo(r.z); acc[5] += bf16hi(r.z);
