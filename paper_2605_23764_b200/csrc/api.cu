@@ -484,6 +484,7 @@ FusedArgs fused_base(moe_ctx* c, bool bwd, int T) {
   FusedArgs fa;
   memset(&fa, 0, sizeof fa);
   fa.lv = c->layout();
+  if (T < COMBINE_ORDER_TOKENS) fa.lv.combine_order = nullptr;
   fa.ctr = c->at<int>(p.ctr) + (bwd ? p.ctr_count : 0);
   c->last_ctr = fa.ctr;
   fa.d = s.d;
@@ -583,7 +584,7 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     Phase ph(c, MOE_PHASE_LAYOUT, st);
     // the event counters of this pass, and of the backward that may follow, start at zero
     const bool persistent = !serial_mode(c);
-    MOE_CUDA(launch_layout(ids, dm, lv, persistent, p.cap_rows / BLOCK_M, persistent ? c->at<int>(p.ctr) : nullptr,
+    MOE_CUDA(launch_layout(ids, dm, lv, persistent && T >= COMBINE_ORDER_TOKENS, p.cap_rows / BLOCK_M, persistent ? c->at<int>(p.ctr) : nullptr,
                            persistent ? p.ctr_count * (c->train() ? 2 : 1) : 0, c->status(), st, &c->launches));
     c->bwd_ctr_clear = persistent && c->train();
   }

@@ -264,6 +264,9 @@ MOE_HD int combine_split_of(int T, int d) {
   const int s = chunks < room ? chunks : room;
   return s > 1 ? s : 1;
 }
+// From this many tokens on combine tasks are taken in the order in which the tokens are completed.  With fewer about every
+// task has a warp of its own that waits for it, and the sort only makes the layout longer (1-2 us of 7-10).
+constexpr int COMBINE_ORDER_TOKENS = 512;
 MOE_HD VecTask decode_post_ticket(const ChainParams& cp, int t, int M) {
   VecTask v;
   if (cp.is_bwd && cp.want_dw) {
