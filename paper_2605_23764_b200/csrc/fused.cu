@@ -520,12 +520,12 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       const int items = pt.start[p + 1] - pt.start[p], most = fa.cp.batch[p];   // 16 and 8 for each pair
       batches |= (items >= 8 * (int)gridDim.x && most == 4 ? 2 : items >= 4 * (int)gridDim.x && most >= 2 ? 1 : 0) << (2 * p);
     }
-    int batch = 1;   // of the phase the last ticket belonged to
+    int batch = 1, phase = 0;   // of the last ticket
     bool more = true;
     for (uint32_t n = 0; more;) {
       // the item sched_hold() before the batch's last has been taken first, then the tickets
       int ok = 1;
-      const uint32_t hold = sched_hold(batch), next = n + batch;
+      const uint32_t hold = sched_hold(batch, fa.cp.strips[phase] != 0), next = n + batch;
       if (lane == 0 && next > hold)
         ok = mbar_wait_cluster(&ring->empty[(next - 1 - hold) % TK_RING], ((next - 1 - hold) / TK_RING) & 1, wc, SITE_EMPTY, -7, 100) ? 1 : 0;
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
@@ -559,7 +559,8 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       if (tr.buf && sub == 0 && wd.ticket >= 0) phase_deps(fa, wd.phase, wc, tr).trace(TR_SCHED, wd.item, t0, td, globaltimer_ns());
       more = !__any_sync(0xffffffffu, wd.ticket < 0);
       n += batch;
-      batch = 1 << ((batches >> (2 * __shfl_sync(0xffffffffu, wd.phase, 31))) & 3);
+      phase = __shfl_sync(0xffffffffu, wd.phase, 31);
+      batch = 1 << ((batches >> (2 * phase)) & 3);
     }
   } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order

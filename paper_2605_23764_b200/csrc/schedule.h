@@ -183,8 +183,10 @@ struct ChainParams {
 // the pace of a pair whose items are shorter (down with F = 192: 0.7 us of MMAs, 4 us an item).  Items of a few k-blocks are
 // therefore taken two or four at a time.  Not longer ones: the last items of a launch would lie with few pairs.
 MOE_HD int sched_batch(int kblocks) { return kblocks <= 8 ? 4 : kblocks <= 16 ? 2 : 1; }
-// Items a pair holds at most that its epilogue has not begun.
-MOE_HD int sched_hold(int batch) { return batch == 4 ? 8 : 4; }
+// Items a pair holds at most that its epilogue has not begun: enough to hide the 3 us (with one fewer than four row-space
+// items the passes over few tokens were 2-6 % slower).  Strips of a weight gradient are tens of microseconds long and of
+// unequal length, four and a half to a pair in a step of 3400 tokens: what a pair holds beyond the next two nobody else can take.
+MOE_HD int sched_hold(int batch, bool strips) { return batch == 4 ? 8 : batch == 1 && strips ? 2 : 4; }
 // Vector warps per CTA that keep gathering after the first tasks.  Two gather 1.4 TB/s in and out, the pace of gate+up at
 // F = 800 and of act_grad at twice that; below, the matrix items waited for the rows (9678 tokens x 10 rows, F = 536: 250 us of
 // MMAs in 420).  Where the products are longer than the gather, more only take from the bandwidth of their loads.
