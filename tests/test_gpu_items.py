@@ -1,0 +1,96 @@
+"""The matrix queue's items where its rules change: column tiles of long experts, strips cut into pieces, items taken in
+batches, the combine order's token limit; and host buffers that are not pinned."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2605_23764_b200 import MoeLayer, binding as B
+from tests.gpu_util import assert_close_bf16, small_problem
+
+pytestmark = pytest.mark.gpu
+
+
+def _against_oracle(ids, w, x, W1, W2, dout, serial):
+    T, d = x.shape
+    E, F = W2.shape[0], W2.shape[2]
+    layer = MoeLayer(T, d, E, ids.shape[1], 0, F, save_for_bwd=True, serial=serial)
+    out = layer.ffn_fwd(x, ids, w, W1, W2)
+    dx, dW1, dW2, dw = layer.ffn_bwd(dout, x, ids, w, W1, W2)
+    torch.cuda.synchronize()
+    assert layer.status() == (0, 0)
+    assert_close_bf16(out, oracle.fwd(x, ids.cpu(), w.cpu(), W1, W2), "out")
+    rdx, rdW1, rdW2, rdw = oracle.bwd(dout, x, ids.cpu(), w.cpu(), W1, W2)
+    assert_close_bf16(dx, rdx, "dx")
+    assert_close_bf16(dw, rdw, "d_topk_w")
+    for e in range(E):   # expert by expert: a tile left out would hide in the whole tensors' norms
+        if (ids == e).any():
+            assert_close_bf16(dW1[e], rdW1[e], f"dW_gate_up[{e}]")
+            assert_close_bf16(dW2[e], rdW2[e], f"dW_down[{e}]")
+        else:
+            assert torch.count_nonzero(dW1[e]).item() == 0 and torch.count_nonzero(dW2[e]).item() == 0
+    layer.close()
+
+
+@pytest.mark.parametrize("counts,d,F", [
+    ([960, 961, 0, 40], 1320, 72),       # the last resident-strip expert and the first long one; fewer strips than pairs
+    ([1025, 320, 321, 7], 520, 392),     # a long expert beside strips that stay resident and that do not
+])
+@pytest.mark.parametrize("serial", [False, True])
+def test_weight_gradient_items(counts, d, F, serial):
+    E, T = len(counts), sum(counts)
+    g = torch.Generator().manual_seed(T)
+    ids = torch.from_numpy(np.repeat(np.arange(E), counts).astype(np.int32))[torch.randperm(T, generator=g)].reshape(T, 1)
+    w = torch.rand(T, 1, generator=g) + 0.25
+    x, W1, W2, _, dout = small_problem(T, d, E, 1, 0, F, T)
+    _against_oracle(ids.contiguous().cuda(), w.cuda(), x, W1, W2, dout, serial)
+
+
+@pytest.mark.parametrize("d", [4096, 2048])   # 20 and 10 items of one k-block to a CTA pair: batches of four and of two
+def test_short_items_in_batches(d):
+    T, E, k, F = 640, 96, 3, 64
+    x, W1, W2, logits, dout = small_problem(T, d, E, k, 0, F, d)
+    layer = MoeLayer(T, d, E, k, 0, F)
+    ids, w = layer.route(logits)
+    torch.cuda.synchronize()
+    layer.close()
+    _against_oracle(ids, w, x, W1, W2, dout, False)
+
+
+@pytest.mark.parametrize("T", [511, 512, 513])
+def test_combine_with_and_without_an_order(T):
+    d, E, k, S, F = 136, 12, 3, 1, 72
+    x, W1, W2, logits, _ = small_problem(T, d, E, k, S, F, T)
+    outs = []
+    for serial in (False, True):
+        layer = MoeLayer(T, d, E, k, S, F, serial=serial)
+        ids, w = layer.route(logits)
+        outs.append(layer.ffn_fwd(x, ids, w, W1, W2).clone())
+        assert layer.status() == (0, 0)
+        layer.close()
+    assert torch.equal(*outs)   # the same sums in slot order
+
+
+def test_host_buffers_that_are_not_pinned():
+    T, d, E, k, S, F = 300, 136, 12, 3, 1, 72
+    x, W1, W2, logits, dout = small_problem(T, d, E, k, S, F, 3)
+    res = []
+    for pin in (True, False):
+        def host(t):
+            return t.cpu().pin_memory() if pin else t.cpu()
+        def empty(*shape, dtype):
+            return torch.empty(*shape, dtype=dtype, pin_memory=pin)
+        layer = MoeLayer(T, d, E, k, S, F, save_for_bwd=True)
+        ids, w, dw = empty(T, k, dtype=torch.int32), empty(T, k, dtype=torch.float32), empty(T, k, dtype=torch.float32)
+        out, dx = empty(T, d, dtype=torch.bfloat16), empty(T, d, dtype=torch.bfloat16)
+        dW1, dW2 = torch.empty_like(W1), torch.empty_like(W2)
+        B.moe_route_host(layer.ctx, host(logits), T, ids, w)
+        torch.cuda.synchronize()
+        B.moe_ffn_fwd_host(layer.ctx, host(x), ids, w, W1, W2, out, T)
+        torch.cuda.synchronize()
+        B.moe_ffn_bwd_host(layer.ctx, host(dout), W1, W2, dx, dW1, dW2, dw, T)
+        torch.cuda.synchronize()
+        assert layer.status() == (0, 0)
+        res.append((ids, w, out, dx, dw, dW1, dW2))
+        layer.close()
+    assert all(torch.equal(a, b) for a, b in zip(*res))
