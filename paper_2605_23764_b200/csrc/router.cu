@@ -201,8 +201,11 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
     const size_t slot_stride = (size_t)ngroups * EPAD;
     const int own0 = rank * npc, own1 = own0 + npc;
     const uint32_t part_addr = smem_u32(part);
+    // each CTA begins with the next CTA's tokens: in one order they would all write to the same CTA at a time
+    const int first = (rank + 1 < C ? own1 : 0) / 16;
     for (int q = sub; q < nchunks * NACC && C > 1; q += 4) {
-      const int h = q / nchunks, c0 = (q - h * nchunks) * 16, e = h * 128 + quad * 32 + lane;
+      const int h = q / nchunks, cq = q - h * nchunks + first;
+      const int c0 = (cq < nchunks ? cq : cq - nchunks) * 16, e = h * 128 + quad * 32 + lane;
       if (c0 >= own0 && c0 + 16 <= own1) continue;   // all of them this CTA's own
       float v[16];
       tmem_ld16(trow + h * acc_cols + c0, v);
