@@ -21,6 +21,7 @@ template <int NPL>
 __global__ void __launch_bounds__(256) route_kernel(const float* __restrict__ logits, int T, int E, int k,
                                                      int renorm, int* __restrict__ topk_ids,
                                                      float* __restrict__ topk_w, int* __restrict__ counts) {
+  __shared__ uint64_t pool[8][TOPK_POOL];
   const int lane = threadIdx.x & 31;
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   pdl_wait();
@@ -38,7 +39,7 @@ __global__ void __launch_bounds__(256) route_kernel(const float* __restrict__ lo
   for (int i = 0; i < NPL; ++i) key[0][i] = i * 32 + lane < E ? float_key(v[i]) : 0u;
   int ids[1] = {0};
   float ls[1] = {0.f};
-  warp_topk<NPL, 1>(key, k, lane, ids, ls);
+  warp_topk<NPL, 1>(key, k, lane, pool[threadIdx.x >> 5], ids, ls);
   const int my_id = ids[0];
   const float my_l = ls[0];
   float my_p;

@@ -36,10 +36,11 @@ struct RouterBarriers {
 
 // Four tokens of one warp: `row` = their logits' partial sums [nslots][..][EPAD experts][4 tokens], added here.
 template <int NACC>
-__device__ __forceinline__ void router_select(const RouterArgs& a, const float4* row, int nslots, size_t slot_stride, int token0,
+__device__ __forceinline__ void router_select(const RouterArgs& a, float4* row, int nslots, size_t slot_stride, int token0,
                                               int lane) {
   constexpr int NPL = 4 * NACC;
   float v[4][NPL];
+  uint64_t* pool = reinterpret_cast<uint64_t*>(row);   // the first source's sums, once they are read: 2 or 4 KB
   {
     float4 acc[NPL];
 #pragma unroll
@@ -66,13 +67,9 @@ __device__ __forceinline__ void router_select(const RouterArgs& a, const float4*
   float mx[4], den[4];
 #pragma unroll
   for (int t = 0; t < 4; ++t) {
-    uint32_t m = 0;
 #pragma unroll
-    for (int i = 0; i < NPL; ++i) {
-      key[t][i] = i * 32 + lane < a.E ? float_key(v[t][i]) : 0u;
-      m = max(m, key[t][i]);
-    }
-    mx[t] = key_float(__reduce_max_sync(0xffffffffu, m));
+    for (int i = 0; i < NPL; ++i) key[t][i] = i * 32 + lane < a.E ? float_key(v[t][i]) : 0u;
+    mx[t] = key_float(__reduce_max_sync(0xffffffffu, lane_max<NPL>(key[t])));
     den[t] = 0.f;
   }
   if (!(a.renorm & GATE_SIGMOID)) {
@@ -88,7 +85,7 @@ __device__ __forceinline__ void router_select(const RouterArgs& a, const float4*
   }
   int id[4] = {0, 0, 0, 0};
   float l[4] = {0.f, 0.f, 0.f, 0.f}, p[4], wsum[4] = {0.f, 0.f, 0.f, 0.f};
-  warp_topk<NPL, 4>(key, a.k, lane, id, l);
+  warp_topk<NPL, 4>(key, a.k, lane, pool, id, l);
 #pragma unroll
   for (int t = 0; t < 4; ++t) p[t] = (a.renorm & GATE_SIGMOID) ? 1.0f / (1.0f + expf(-l[t])) : expf(l[t] - mx[t]) / den[t];
   if (a.renorm & GATE_RENORM) {

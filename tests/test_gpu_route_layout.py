@@ -46,6 +46,20 @@ def test_route_ties_and_extremes():
     _check_route_layout(l.cuda(), 16, 16, 0, False)
 
 
+@pytest.mark.parametrize("E,k", [(128, 8), (129, 1), (256, 8), (256, 16), (256, 17), (500, 16), (1024, 32)])
+def test_selection_edges(E, k):
+    """Four logits a lane and more, sixteen slots and more; distinct logits, some equal, more equal than a warp has lanes, all equal."""
+    g = torch.Generator().manual_seed(E + k)
+    l = torch.randn(96, E, generator=g)
+    l[24:48] = torch.round(l[24:48] * 8) / 8
+    l[48:72] = torch.round(l[48:72])
+    l[72:80] = 0.25
+    l[80:88] = torch.where(torch.arange(E) < E // 2, 1.0, l[80:88])
+    l[88:, :] = -1e30
+    l[88:, 5::32] = torch.randn(8, len(range(5, E, 32)), generator=g)   # the largest of a token in one lane
+    _check_route_layout(l.cuda(), E, k, 0, False)
+
+
 def test_all_tokens_to_one_expert_and_empty_experts():
     T, E = 700, 12
     l = torch.full((T, E), -5.0)

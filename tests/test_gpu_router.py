@@ -84,6 +84,20 @@ def test_equal_logits_go_to_the_lower_expert_id():
     layer.close()
 
 
+@pytest.mark.parametrize("T,E,k", [(130, 128, 8), (300, 256, 8), (300, 130, 1), (70, 200, 6)])
+def test_many_equal_logits(T, E, k):
+    """Tokens with all logits equal beside tokens with pairs of equal ones: four of them share a warp."""
+    import oracle
+    d = 128
+    x, W = _inputs(T, d, E, 7, dup=[(e, e + 50) for e in range(0, 50, 3)])
+    x[1::5] = 0
+    layer, ids, w, logits, _ = _run_fwd(T, d, E, k, False, x, W)
+    ids_ref, w_ref = oracle.route(logits, k, False)
+    assert np.array_equal(ids, ids_ref)
+    np.testing.assert_allclose(w, w_ref, rtol=2e-6, atol=1e-30)
+    layer.close()
+
+
 def test_logits_are_optional():
     T, d, E, k = 130, 192, 24, 2
     x, W = _inputs(T, d, E, 5)
