@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(ROUTER_THREADS, 1) router_fwd_kernel(const __g
     const size_t slot_stride = (size_t)ngroups * EPAD;
     const int own0 = rank * npc, own1 = own0 + npc;
     const uint32_t part_addr = smem_u32(part);
-    // each CTA begins with the next CTA's tokens: in one order they would all write to the same CTA at a time
+    // each CTA begins with the next CTA's tokens: in one order they all wrote to the same CTA at a time, and 8192 tokens x
+    // 256 experts, d = 7168, with the score gradient took 56.9 us instead of 54.0
     const int first = (rank + 1 < C ? own1 : 0) / 16;
     for (int q = sub; q < nchunks * NACC && C > 1; q += 4) {
       const int h = q / nchunks, cq = q - h * nchunks + first;
