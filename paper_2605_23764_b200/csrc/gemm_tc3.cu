@@ -47,13 +47,14 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   // Items pair, pair + npairs, ..; each role decodes item i + 1 before it works on item i (the decode's chain of
   // global loads then completes behind the item's work).
   const int total = total_swap_work<MODE>(a);
+  const Ring ring = ring_of((GemmMode)MODE, a.meta[7]);
   SwapWork cur, next;
   if (pair < total) cur = decode_swap_work<MODE>(a, pair);
   if (warp == 0 || warp == 6) {
     LoaderState ls;
     for (int t = pair; t < total; t += npairs, cur = next) {
       if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-      if (!swap_load_item<MODE>(a, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
+      if (!swap_load_item<MODE>(a, ring, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
     }
   } else if (warp == 1) {
     if (rank == 0) {
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       bool ok = true;
       for (int t = pair; t < total && ok; t += npairs, cur = next) {
         if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-        ok = swap_issue_item<MODE>(a, smem, bars, tmem_base, is, cur, t, wc, dep);
+        ok = swap_issue_item<MODE>(a, ring, smem, bars, tmem_base, is, cur, t, wc, dep);
       }
       if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
@@ -82,14 +83,6 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, TMEM_COLS);
   }
-}
-
-void plan_ring(GemmMode mode, int T, GemmArgs& a) {
-  const bool merges = mode == GEMM_DOWN || mode == GEMM_GATE_GRAD || mode == GEMM_GATE_UP;   // gate+up: laid out like down
-  const int n32 = (T + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN;
-  a.tok_bytes = T <= 256 ? n32 / 2 * BK * 2 : (merges ? 3 : 2) * 64 * BK * 2;
-  a.stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + a.tok_bytes));
-  if (a.stages > MAX_STAGES) a.stages = MAX_STAGES;
 }
 
 template <int MODE>

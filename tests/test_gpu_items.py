@@ -94,3 +94,24 @@ def test_host_buffers_that_are_not_pinned():
         res.append((ids, w, out, dx, dw, dW1, dW2))
         layer.close()
     assert all(torch.equal(a, b) for a, b in zip(*res))
+
+
+@pytest.mark.parametrize("case", ["one_expert", "padded_batch", "merged"])
+@pytest.mark.parametrize("serial", [False, True])
+def test_ids_repeated_inside_a_token(case, serial):
+    """An expert may have more rows than the call has tokens: every slot of a token is a row of its own."""
+    d, E, F = 1032, 8, 392   # 17 and 7 k-blocks: more than the deepest ring has stages, and fewer
+    if case == "one_expert":       # 32 tokens x 8 slots, all of them expert 0's
+        T, k = 32, 8
+        ids = torch.zeros(T, k, dtype=torch.int32)
+    elif case == "padded_batch":   # half of a generation batch is padding with id 0 in every slot
+        T, k = 64, 6
+        ids = torch.stack([torch.randperm(E, generator=torch.Generator().manual_seed(t))[:k] for t in range(T)]).to(torch.int32)
+        ids[T // 2:] = 0
+    else:                          # 256 tokens: experts of 290 and 222 rows, the larger one's last two tiles merge
+        T, k = 256, 2
+        ids = torch.zeros(T, k, dtype=torch.int32)
+        ids[145:, :] = 3
+    w = torch.rand(T, k, generator=torch.Generator().manual_seed(T)) + 0.25
+    x, W1, W2, _, dout = small_problem(T, d, E, k, 0, F, T)
+    _against_oracle(ids.cuda(), w.cuda(), x, W1, W2, dout, serial)
