@@ -209,7 +209,8 @@ struct moe_ctx {
   const void *saved_x = nullptr, *saved_ids = nullptr, *saved_w = nullptr;  // that forward's inputs
   uint64_t budget_ns = 2000ull * 1000 * 1000;
   int* last_ctr = nullptr;      // event counters of the last persistent launch
-  bool bwd_ctr_clear = false;   // the backward's event counters are zero (the forward's layout clears both sets)
+  bool bwd_ctr_clear = false;   // the backward's event counters are zero (the forward's layout clears both sets) ..
+  unsigned long long clear_capture = 0;   // .. for work in this stream capture (0: none)
   int dep_extra = 0;  // test hook: makes the activation dependencies of the persistent launch unreachable
   cudaStream_t last_stream = nullptr;
   void* debug_copy = nullptr;   // moe_debug_buffer: the last row-space tensor asked for, compact
@@ -568,6 +569,15 @@ int combine_and_maybe_copy_out(moe_ctx* c, const Dims& dm, const LayoutView& lv,
   return MOE_OK;
 }
 
+// The stream capture that `st` is part of; 0: none.
+cudaError_t capture_of(cudaStream_t st, unsigned long long* id) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  unsigned long long seq = 0;
+  const cudaError_t e = cudaStreamGetCaptureInfo(st, &status, &seq);
+  *id = e == cudaSuccess && status != cudaStreamCaptureStatusNone ? seq : 0;
+  return e;
+}
+
 int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, const uint16_t* W1,
             const uint16_t* W2, uint16_t* out, int T, cudaStream_t st, uint16_t* out_host = nullptr, cudaEvent_t x_free = nullptr) {
   const WsPlan& p = c->plan;
@@ -583,6 +593,7 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     MOE_CUDA(launch_layout(ids, dm, lv, persistent && T >= COMBINE_ORDER_TOKENS, p.cap_rows / BLOCK_M, persistent ? c->at<int>(p.ctr) : nullptr,
                            persistent ? p.ctr_count * (c->train() ? 2 : 1) : 0, c->status(), st, &c->launches));
     c->bwd_ctr_clear = persistent && c->train();
+    if (c->bwd_ctr_clear) MOE_CUDA(capture_of(st, &c->clear_capture));
   }
   if (out_host) MOE_CUDA(cudaEventRecord(c->ev_fwd_start, st));
   c->host_fwd = out_host != nullptr;
@@ -700,8 +711,11 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     fa.dw_nparts = p.ntn_act * DW_PARTS_PER_TILE;
     fa.d_topk_w = d_w;
     Phase ph(c, MOE_PHASE_FUSED_BWD, st);
-    // the forward's layout cleared the counters; a second backward of one forward clears them itself
-    if (!c->bwd_ctr_clear) MOE_CUDA(cudaMemsetAsync(fa.ctr, 0, sizeof(int) * (size_t)p.ctr_count, st));
+    // The forward's layout cleared the counters; a second backward of one forward clears them itself, and so does a captured
+    // one whose forward is not in the same capture: its graph may run several times behind one forward.
+    unsigned long long capture = 0;
+    MOE_CUDA(capture_of(st, &capture));
+    if (!c->bwd_ctr_clear || capture != c->clear_capture) MOE_CUDA(cudaMemsetAsync(fa.ctr, 0, sizeof(int) * (size_t)p.ctr_count, st));
     c->bwd_ctr_clear = false;
     // Host buffers: dx is complete when the last backward-combine task is, well before the last weight-gradient
     // strips; the kernel then sets a word the copy-out stream waits for, so the copy overlaps the rest of the launch.
