@@ -51,6 +51,10 @@ int moe_debug_set_unreachable_dependency(moe_ctx* ctx, int32_t on);
  * the attribute (they do not need co-residency): with a ctx the call changes nothing. */
 int moe_debug_set_plain_launch(moe_ctx* ctx, int32_t on);
 
+/* 1 if the kernels of the host-buffer calls read or write this host buffer in place (pinned or registered memory, in one
+ * piece), 0 if it is copied. */
+int moe_debug_host_direct(const void* p, size_t bytes);
+
 /* Host-only check of the static tile schedule of the single persistent launch (Section 4.3: tasks
  * in statically ordered queues, dependent/trigger event counters with static thresholds).  For the
  * given per-expert row counts[Ep] and layer shape it builds the layout tables, the matrix queue of

@@ -505,18 +505,38 @@ int ensure_copy_streams(moe_ctx* c) {
   return MOE_OK;
 }
 
-// Device address of `n` elements of pinned (mapped) host memory; NULL for any other memory.  Both ends are looked up: a
-// buffer may reach beyond the range that was registered.
+// Device address of `n` elements of pinned (mapped) host memory; NULL for any other memory.  The whole buffer has to lie in
+// the allocation or registration that holds its first byte: it may reach beyond the range that was registered, or from one
+// registration over a gap into the next.
+typedef CUresult (*PointerAttributeFn)(void*, CUpointer_attribute, CUdeviceptr);
+PointerAttributeFn get_pointer_attribute_fn() {
+  static const PointerAttributeFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<PointerAttributeFn>(p);
+    cudaGetLastError();
+    return static_cast<PointerAttributeFn>(nullptr);
+  }();
+  return fn;
+}
 template <class T>
 T* mapped_host(T* p, size_t n) {
-  cudaPointerAttributes a, b;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, p + n - 1) != cudaSuccess) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
-  T* const first = static_cast<T*>(a.devicePointer);
-  return static_cast<T*>(b.devicePointer) == first + (n - 1) ? first : nullptr;
+  if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
+  const PointerAttributeFn attribute = get_pointer_attribute_fn();
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  CUdeviceptr first = 0;
+  size_t size = 0;
+  if (!attribute || attribute(&first, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) != CUDA_SUCCESS ||
+      attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) != CUDA_SUCCESS)
+    return nullptr;
+  const size_t before = at - first;   // (an address outside the range wraps around)
+  return before <= size && n * sizeof(T) <= size - before ? static_cast<T*>(a.devicePointer) : nullptr;
 }
 
 // The forward result leaves for the host: on `st`, or -- MOE_FLAG_DEFER_OUT_COPY -- on the copy-out stream behind an
@@ -1097,6 +1117,10 @@ int moe_debug_set_plain_launch(moe_ctx* c, int32_t on) {
     return MOE_OK;
   }
   return MOE_OK;   // a context's launches are made without the attribute anyway
+}
+
+int moe_debug_host_direct(const void* p, size_t bytes) {
+  return p && bytes && mapped_host(static_cast<const uint8_t*>(p), bytes) ? 1 : 0;
 }
 
 int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {

@@ -115,3 +115,22 @@ def test_ids_repeated_inside_a_token(case, serial):
     w = torch.rand(T, k, generator=torch.Generator().manual_seed(T)) + 0.25
     x, W1, W2, _, dout = small_problem(T, d, E, k, 0, F, T)
     _against_oracle(ids.cuda(), w.cuda(), x, W1, W2, dout, serial)
+
+
+def test_host_memory_is_used_in_place_only_within_one_registration():
+    """Looked up only: no kernel touches the memory."""
+    mb, rt = 1 << 20, torch.cuda.cudart()
+    torch.zeros(1, device="cuda")
+    pinned, pageable = torch.empty(mb, dtype=torch.uint8, pin_memory=True), torch.empty(9 * mb, dtype=torch.uint8)
+    assert B.moe_debug_host_direct(pinned.data_ptr(), mb) and B.moe_debug_host_direct(pinned.data_ptr() + mb - 4, 4)
+    assert not B.moe_debug_host_direct(pageable.data_ptr(), mb)
+    first = (pageable.data_ptr() + mb - 1) // mb * mb
+    second = first + 4 * mb
+    assert not int(rt.cudaHostRegister(first, mb, 0)) and not int(rt.cudaHostRegister(second, mb, 0))
+    try:
+        assert B.moe_debug_host_direct(first, mb) and B.moe_debug_host_direct(second + 4, mb - 4)
+        assert not B.moe_debug_host_direct(first, mb + 4)       # beyond the end
+        assert not B.moe_debug_host_direct(first, 5 * mb)       # both ends registered, a gap between them
+    finally:
+        rt.cudaHostUnregister(first)
+        rt.cudaHostUnregister(second)
