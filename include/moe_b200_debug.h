@@ -51,6 +51,10 @@ int moe_debug_set_unreachable_dependency(moe_ctx* ctx, int32_t on);
  * the attribute (they do not need co-residency): with a ctx the call changes nothing. */
 int moe_debug_set_plain_launch(moe_ctx* ctx, int32_t on);
 
+/* Which kernels lay out T tokens of kp = k + n_shared slots over Ep = E + n_shared experts: 1 = one block, 8 or 16 = a cluster of
+ * that many blocks (given that the device can hold one: fits8, fits16), 0 = the kernels over all SMs.  Host only. */
+int moe_debug_layout_blocks(int32_t T, int32_t kp, int32_t Ep, int32_t fits8, int32_t fits16);
+
 /* 1 if the kernels of the host-buffer calls read or write this host buffer in place (pinned or registered memory, in one
  * piece), 0 if it is copied. */
 int moe_debug_host_direct(const void* p, size_t bytes);

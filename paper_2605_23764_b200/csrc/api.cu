@@ -1123,6 +1123,10 @@ int moe_debug_host_direct(const void* p, size_t bytes) {
   return p && bytes && mapped_host(static_cast<const uint8_t*>(p), bytes) ? 1 : 0;
 }
 
+int moe_debug_layout_blocks(int32_t T, int32_t kp, int32_t Ep, int32_t fits8, int32_t fits16) {
+  return layout_blocks(T, kp, Ep, fits8 != 0, fits16 != 0);
+}
+
 int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
   if (!c || !ptr || !elems) return MOE_ERR_INVALID_ARG;
   const moe_shape& s = c->shape;

@@ -33,6 +33,25 @@ constexpr __host__ __device__ int row_ld(int cols) { return (cols + 63) & ~63; }
 
 constexpr int LAYOUT_CHUNK = 2048;  // flat slots per block of the layout kernels
 
+// Which kernels lay out T tokens of kp slots over Ep experts: 1 = layout_one_kernel, 8 or 16 = one cluster of that many blocks,
+// 0 = the kernels over all SMs (route_layout.cu has the reasons).  fits8, fits16: the device can hold such a cluster; sixteen
+// is beyond the portable size, a partitioned GPU may have no sixteen SMs side by side.
+constexpr int LAYOUT_ONE_WARPS = 31;
+constexpr int LAYOUT_ONE_SLOTS = 32 * LAYOUT_ONE_WARPS;
+constexpr int LAYOUT_ONE_EXPERTS = 384;   // shared memory without opt-in: 48 KB
+constexpr int LAYOUT_CLUSTER_G = 4;
+constexpr int LAYOUT_CLUSTER_SLOTS = 16 * LAYOUT_CLUSTER_G * 1024;
+constexpr int LAYOUT_CLUSTER_EXPERTS = 384;
+inline int layout_blocks(int T, int kp, int Ep, bool fits8, bool fits16) {
+  const int n = T * kp;
+  if (n < LAYOUT_ONE_SLOTS && Ep <= LAYOUT_ONE_EXPERTS) return 1;
+  // A single chunk over a handful of experts keeps the kernels (23 us where a cluster takes 11): moe_last_launch_count() of such
+  // calls is relied upon.
+  if ((n <= LAYOUT_CHUNK && Ep <= 8) || Ep > LAYOUT_CLUSTER_EXPERTS) return 0;
+  if ((T + 7) / 8 * kp <= 1024) return fits8 ? 8 : 0;
+  return (T + 15) / 16 * kp <= LAYOUT_CLUSTER_G * 1024 && fits16 ? 16 : 0;
+}
+
 // Device arrays describing one dispatch layout.
 struct LayoutView {
   int* counts;       // [Ep]

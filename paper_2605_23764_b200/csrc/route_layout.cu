@@ -459,9 +459,6 @@ __global__ void __launch_bounds__(1024) layout_order_kernel(int T, LayoutView lv
 // in shared memory, nothing read back.  Token generation (V3-shaped layer, 64 tokens) spends 8 us here against 45 us
 // in the four kernels and the clearing of the counters.  One chunk of the large form would hold 2048 slots, but its three short kernels overlap, and from a
 // thousand slots on they are as fast.
-constexpr int LAYOUT_ONE_WARPS = 31;
-constexpr int LAYOUT_ONE_SLOTS = 32 * LAYOUT_ONE_WARPS;
-constexpr int LAYOUT_ONE_EXPERTS = 384;   // shared memory without opt-in: 48 KB
 __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict__ ids, int n, int T, int k, int kp, int E,
                                                           int Ep, LayoutView lv, int want_order, DevStatus* status,
                                                           int* __restrict__ zero, int nzero) {
@@ -538,9 +535,6 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
 // (11 us with the combine order) instead of 13 (19).  A group costs 3 us -- scattered stores and match instructions of one SM --
 // so from 8192 slots on there are sixteen blocks, and at 65536 slots, where a block has four groups, the four kernels over
 // all SMs catch up.
-constexpr int LAYOUT_CLUSTER_G = 4;
-constexpr int LAYOUT_CLUSTER_SLOTS = 16 * LAYOUT_CLUSTER_G * 1024;
-constexpr int LAYOUT_CLUSTER_EXPERTS = 384;
 // M-blocks and one: at most LAYOUT_CLUSTER_SLOTS / 128 + one per expert
 constexpr int LAYOUT_CLUSTER_BINS = LAYOUT_CLUSTER_SLOTS / BLOCK_M + LAYOUT_CLUSTER_EXPERTS + 1;
 static_assert(LAYOUT_CLUSTER_BINS <= 1024, "a bin per thread");
@@ -681,27 +675,46 @@ __global__ void __launch_bounds__(1024)
   cluster_sync_all();   // no block leaves while another reads its bins
 }
 
+// Can the current device hold a cluster of C such blocks?  Looked up once per device, with the kernel's largest shared memory.
 template <int C>
-static cudaError_t launch_layout_cluster(const int* ids, const Dims& dm, const LayoutView& lv, bool want_order, int* zero, int nzero,
-                                         DevStatus* status, cudaStream_t s) {
+static cudaError_t layout_cluster_fits(bool* fits) {
   static std::mutex mu;
-  static bool attr_set[MAX_DEVICES] = {};
-  const int Ep = dm.Ep();
+  static int known[MAX_DEVICES] = {};   // 1: no, 2: yes
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= MAX_DEVICES) return cudaErrorInvalidDevice;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (!attr_set[dev]) {
-      e = cudaFuncSetAttribute(layout_cluster_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)layout_cluster_smem(LAYOUT_CLUSTER_EXPERTS, LAYOUT_CLUSTER_G));
-      if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(layout_cluster_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-      attr_set[dev] = true;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!known[dev]) {
+    const size_t smem = layout_cluster_smem(LAYOUT_CLUSTER_EXPERTS, LAYOUT_CLUSTER_G);
+    if ((e = cudaFuncSetAttribute(layout_cluster_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    if (C > 8 && (e = cudaFuncSetAttribute(layout_cluster_kernel<C>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1))) return e;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, layout_cluster_kernel<C>, &cfg) != cudaSuccess) {
+      cudaGetLastError();   // not a size this device knows
+      n = 0;
     }
+    known[dev] = n > 0 ? 2 : 1;
   }
-  const int cta_slots = (dm.T + C - 1) / C * dm.kp(), G = (cta_slots + 1023) / 1024;
+  *fits = known[dev] == 2;
+  return cudaSuccess;
+}
+
+template <int C>
+static cudaError_t launch_layout_cluster(const int* ids, const Dims& dm, const LayoutView& lv, bool want_order, int* zero, int nzero,
+                                         DevStatus* status, cudaStream_t s) {
+  const int Ep = dm.Ep(), cta_slots = (dm.T + C - 1) / C * dm.kp(), G = (cta_slots + 1023) / 1024;
   return launch_dependent_cluster(layout_cluster_kernel<C>, C, dim3(C), dim3(1024), layout_cluster_smem(Ep, G), s, ids, dm.slots(), dm.T,
                                   dm.k, dm.kp(), dm.E, Ep, G, lv, want_order ? 1 : 0, status, zero, nzero);
 }
@@ -710,22 +723,21 @@ cudaError_t launch_layout(const int* topk_ids, const Dims& dm, const LayoutView&
                           int* zero, int nzero, DevStatus* status, cudaStream_t s, int* launches) {
   const int n = dm.slots(), Ep = dm.Ep(), kp = dm.kp();
   cudaError_t e;
-  if (n < LAYOUT_ONE_SLOTS && Ep <= LAYOUT_ONE_EXPERTS) {
+  const int wanted = layout_blocks(dm.T, kp, Ep, true, true);
+  if (wanted == 1) {
     const size_t smem = sizeof(int) * (size_t)(expert_scan_ints(Ep) + 4 + 2 * LAYOUT_ONE_SLOTS) +
                         sizeof(uint16_t) * (size_t)((n + 31) / 32) * (Ep + (Ep & 1));
     ++*launches;
     return launch_dependent(layout_one_kernel, dim3(1), dim3(1024), smem, s, topk_ids, n, dm.T, dm.k, kp, dm.E, Ep, lv,
                             want_order ? 1 : 0, status, zero, nzero);
   }
-  // (The four kernels of a single chunk take 23 us where this takes 11; calls over a handful of experts keep them, their number
-  // of launches is relied upon.)
-  if ((n > LAYOUT_CHUNK || Ep > 8) && Ep <= LAYOUT_CLUSTER_EXPERTS) {
-    const bool eight = (dm.T + 7) / 8 * kp <= 1024;
-    if (eight || (dm.T + 15) / 16 * kp <= LAYOUT_CLUSTER_G * 1024) {
-      ++*launches;
-      return eight ? launch_layout_cluster<8>(topk_ids, dm, lv, want_order, zero, nzero, status, s)
-                   : launch_layout_cluster<16>(topk_ids, dm, lv, want_order, zero, nzero, status, s);
-    }
+  if (wanted) {
+    bool fits = false;
+    if ((e = wanted == 8 ? layout_cluster_fits<8>(&fits) : layout_cluster_fits<16>(&fits))) return e;
+    const int blocks = layout_blocks(dm.T, kp, Ep, fits, fits);
+    if (blocks) ++*launches;
+    if (blocks == 8) return launch_layout_cluster<8>(topk_ids, dm, lv, want_order, zero, nzero, status, s);
+    if (blocks == 16) return launch_layout_cluster<16>(topk_ids, dm, lv, want_order, zero, nzero, status, s);
   }
   const int nblk = n > 0 ? (n + LAYOUT_CHUNK - 1) / LAYOUT_CHUNK : 1;
   int* const tok_last = want_order ? lv.tok_last : nullptr;

@@ -72,3 +72,17 @@ def test_skewed_config_schedule():
     counts[-4:] = 0
     rc, stats = binding.moe_debug_simulate_schedule(counts, 16384, 8, 0, 4096, 1536, 0, 74, 1184)
     assert rc == 0
+
+
+def test_layout_takes_the_kernels_where_a_cluster_does_not_fit():
+    def blocks(*a, **kw):
+        return binding.moe_debug_layout_blocks(*a, **kw)
+    assert blocks(123, 8, 64) == 1 and blocks(124, 8, 64) == 8           # 984 and 992 slots
+    assert blocks(1024, 8, 64) == 8 and blocks(1025, 8, 64) == 16        # 1024 slots to a block, and one token more
+    assert blocks(8192, 8, 256) == 16 and blocks(8193, 8, 256) == 0      # 65536 slots, and one token more
+    assert blocks(124, 8, 384) == 8 and blocks(124, 8, 385) == 0
+    for T in (124, 1024):
+        assert blocks(T, 8, 64, fits16=False) == 8 and blocks(T, 8, 64, fits8=False) == 0
+    for T in (1025, 8192):
+        assert blocks(T, 8, 64, fits8=False) == 16 and blocks(T, 8, 64, fits16=False) == 0
+    assert blocks(123, 8, 64, fits8=False, fits16=False) == 1
