@@ -3,9 +3,11 @@ from __future__ import annotations
 
 import concurrent.futures
 import os
+import shutil
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
@@ -19,15 +21,20 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
 
 def _nvcc() -> str:
     for cand in (os.environ.get("NVCC"), "/usr/local/cuda/bin/nvcc", "nvcc"):
-        if cand and (os.path.sep not in cand or os.path.exists(cand)):
-            return cand
+        path = cand and shutil.which(cand)
+        if path:
+            return path
     raise RuntimeError("nvcc not found")
 
 
-def _stale() -> bool:
-    if not (os.path.exists(OUT) and os.path.exists(FAST)):
+def _cuda_include() -> str:
+    return os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+
+
+def _stale(out: str) -> bool:
+    if not os.path.exists(out):
         return True
-    t = min(os.path.getmtime(OUT), os.path.getmtime(FAST))
+    t = os.path.getmtime(out)
     inc = os.path.join(PKG, "..", "include")
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(inc, f) for f in os.listdir(inc)]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -50,7 +57,7 @@ def _build_fastcall() -> None:
     tmp = FAST + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
-           "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"),
+           "-I" + sysconfig.get_paths()["include"], "-I" + _cuda_include(),
            os.path.join(CSRC, "fastcall.cpp"), "-o", tmp, "-L" + os.path.join(root, "lib"),
            "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     r = subprocess.run(cmd, capture_output=True, text=True)
@@ -59,19 +66,33 @@ def _build_fastcall() -> None:
     os.replace(tmp, FAST)
 
 
+def _try_fastcall() -> None:
+    """The library does not need it (the binding then checks its arguments in Python), so a box without a C++ compiler, Python's
+    or torch's headers goes without; what an older source left there is not kept."""
+    try:
+        _build_fastcall()
+    except (OSError, RuntimeError, ImportError) as e:
+        if os.path.exists(FAST):
+            os.unlink(FAST)
+        warnings.warn(f"calls from Python go the slower way, the accelerator could not be built: {e}")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source for sm_100a and link the C-ABI shared library.  Returns its path."""
-    if not force and not _stale():
+    lib, fast = force or _stale(OUT), force or _stale(FAST)
+    if not (lib or fast):
         return OUT
     os.makedirs(OBJ, exist_ok=True)
     with concurrent.futures.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
-        fast = ex.submit(_build_fastcall)
-        objs = list(ex.map(_compile, SOURCES))
-        fast.result()
-    tmp = OUT + f".tmp{os.getpid()}"
-    cmd = [_nvcc(), "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
-    subprocess.check_call(cmd)
-    os.replace(tmp, OUT)
+        side = ex.submit(_try_fastcall) if fast else None
+        objs = list(ex.map(_compile, SOURCES)) if lib else []
+        if side:
+            side.result()
+    if lib:
+        tmp = OUT + f".tmp{os.getpid()}"
+        cmd = [_nvcc(), "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
+        subprocess.check_call(cmd)
+        os.replace(tmp, OUT)
     if verbose:
         for o in objs:
             sys.stdout.write(open(o + ".log").read())

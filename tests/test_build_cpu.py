@@ -1,0 +1,38 @@
+"""The build: the library comes out without the accelerator of the Python calls."""
+import ctypes
+import os
+import shutil
+
+import pytest
+
+from paper_2605_23764_b200 import build
+
+
+def test_library_is_built_without_the_accelerator(monkeypatch, tmp_path):
+    build.build()
+    compiled = build.OBJ
+
+    def no_compiler():
+        raise FileNotFoundError("g++")
+
+    def compile_(src):   # the objects are there
+        obj = src.replace(".cu", ".o")
+        return shutil.copy(os.path.join(compiled, obj), tmp_path / obj)
+    monkeypatch.setattr(build, "OBJ", str(tmp_path))
+    monkeypatch.setattr(build, "OUT", str(tmp_path / "lib.so"))
+    monkeypatch.setattr(build, "FAST", str(tmp_path / "fast.so"))
+    monkeypatch.setattr(build, "_compile", compile_)
+    monkeypatch.setattr(build, "_build_fastcall", no_compiler)
+    (tmp_path / "fast.so").write_bytes(b"of an older source")
+    with pytest.warns(UserWarning, match="g\\+\\+"):
+        out = build.build(force=True)
+    assert hasattr(ctypes.CDLL(out), "moe_create")
+    assert not (tmp_path / "fast.so").exists()
+
+
+def test_cuda_headers_are_found_from_a_bare_nvcc(monkeypatch):
+    nvcc = build._nvcc()
+    monkeypatch.setenv("NVCC", "nvcc")
+    monkeypatch.setenv("PATH", os.path.dirname(nvcc) + os.pathsep + os.environ.get("PATH", ""))
+    assert os.path.isabs(build._nvcc())
+    assert os.path.exists(os.path.join(build._cuda_include(), "cuda_runtime.h"))
