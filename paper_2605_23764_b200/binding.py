@@ -8,8 +8,10 @@ from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.util
 import os
 import struct
+import sysconfig
 import threading
 
 import torch
@@ -96,13 +98,31 @@ class MoeTfTd(ctypes.Structure):
 
 _lib = None
 
+
+def fastcall_path() -> str:
+    """The file of the accelerator.  It holds tensor objects' layouts of the torch and Python it was built with: their versions
+    are in its name, so that another torch or Python neither loads it nor takes it for built."""
+    abi = f"torch{torch.__version__}-abi{int(torch._C._GLIBCXX_USE_CXX11_ABI)}"
+    return os.path.join(os.path.dirname(os.path.abspath(__file__)), f"_fastcall-{abi}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
 # The calls of a step go through csrc/fastcall.cpp; it answers None for arguments it does not take as they are, and the
-# functions below then look at them one by one and say what is wrong.  Without it (torch's C++ interface has changed since it
-# was built) everything goes that way.
-try:
-    from . import _fastcall as _fast
-except ImportError:
-    _fast = None
+# functions below then look at them one by one and say what is wrong.  Without it (not built, or for another torch or Python)
+# everything goes that way.
+def _load_fastcall():
+    path = fastcall_path()
+    if not os.path.exists(path):
+        return None
+    spec = importlib.util.spec_from_file_location(__package__ + "._fastcall", path)
+    try:
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+    except ImportError:
+        return None
+    return module
+
+
+_fast = _load_fastcall()
 
 
 def lib_path() -> str:

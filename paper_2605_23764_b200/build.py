@@ -1,4 +1,4 @@
-"""Builds libmoe_b200.so in-tree with nvcc for sm_100a (no JIT cache), and _fastcall.so, the step calls' way in from Python."""
+"""Builds libmoe_b200.so in-tree with nvcc for sm_100a (no JIT cache), and _fastcall, the step calls' way in from Python."""
 from __future__ import annotations
 
 import concurrent.futures
@@ -9,10 +9,11 @@ import sys
 import sysconfig
 import warnings
 
+from .binding import fastcall_path
+
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 OUT = os.path.join(PKG, "libmoe_b200.so")
-FAST = os.path.join(PKG, "_fastcall.so")
 OBJ = os.path.join(PKG, "_build")
 SOURCES = ["api.cu", "route_layout.cu", "permute.cu", "gemm_tc3.cu", "gemm_wgrad.cu", "fused.cu", "study.cu", "router.cu", "taskflow.cu", "ep.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -53,8 +54,8 @@ def _compile(src: str) -> str:
 
 def _build_fastcall() -> None:
     import torch
-    root = os.path.dirname(torch.__file__)
-    tmp = FAST + f".tmp{os.getpid()}"
+    root, path = os.path.dirname(torch.__file__), fastcall_path()
+    tmp = path + f".tmp{os.getpid()}"
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
            "-I" + sysconfig.get_paths()["include"], "-I" + _cuda_include(),
@@ -63,7 +64,7 @@ def _build_fastcall() -> None:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed on fastcall.cpp:\n{r.stdout}{r.stderr}")
-    os.replace(tmp, FAST)
+    os.replace(tmp, path)
 
 
 def _try_fastcall() -> None:
@@ -72,14 +73,14 @@ def _try_fastcall() -> None:
     try:
         _build_fastcall()
     except (OSError, RuntimeError, ImportError) as e:
-        if os.path.exists(FAST):
-            os.unlink(FAST)
+        if os.path.exists(fastcall_path()):
+            os.unlink(fastcall_path())
         warnings.warn(f"calls from Python go the slower way, the accelerator could not be built: {e}")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every CUDA source for sm_100a and link the C-ABI shared library.  Returns its path."""
-    lib, fast = force or _stale(OUT), force or _stale(FAST)
+    lib, fast = force or _stale(OUT), force or _stale(fastcall_path())
     if not (lib or fast):
         return OUT
     os.makedirs(OBJ, exist_ok=True)

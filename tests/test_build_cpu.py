@@ -4,8 +4,9 @@ import os
 import shutil
 
 import pytest
+import torch
 
-from paper_2605_23764_b200 import build
+from paper_2605_23764_b200 import binding, build
 
 
 def test_library_is_built_without_the_accelerator(monkeypatch, tmp_path):
@@ -20,7 +21,7 @@ def test_library_is_built_without_the_accelerator(monkeypatch, tmp_path):
         return shutil.copy(os.path.join(compiled, obj), tmp_path / obj)
     monkeypatch.setattr(build, "OBJ", str(tmp_path))
     monkeypatch.setattr(build, "OUT", str(tmp_path / "lib.so"))
-    monkeypatch.setattr(build, "FAST", str(tmp_path / "fast.so"))
+    monkeypatch.setattr(build, "fastcall_path", lambda: str(tmp_path / "fast.so"))
     monkeypatch.setattr(build, "_compile", compile_)
     monkeypatch.setattr(build, "_build_fastcall", no_compiler)
     (tmp_path / "fast.so").write_bytes(b"of an older source")
@@ -36,3 +37,16 @@ def test_cuda_headers_are_found_from_a_bare_nvcc(monkeypatch):
     monkeypatch.setenv("PATH", os.path.dirname(nvcc) + os.pathsep + os.environ.get("PATH", ""))
     assert os.path.isabs(build._nvcc())
     assert os.path.exists(os.path.join(build._cuda_include(), "cuda_runtime.h"))
+
+
+def test_accelerator_of_another_torch_or_python_is_not_taken(monkeypatch):
+    build.build()
+    path = build.fastcall_path()
+    assert os.path.exists(path) and not build._stale(path)
+    assert binding._load_fastcall() is not None
+    with monkeypatch.context() as m:
+        m.setattr(torch, "__version__", "0.0.1")
+        assert build._stale(build.fastcall_path()) and binding._load_fastcall() is None
+    with monkeypatch.context() as m:
+        m.setattr(binding.sysconfig, "get_config_var", lambda name: ".cpython-399-other.so")
+        assert build._stale(build.fastcall_path()) and binding._load_fastcall() is None
