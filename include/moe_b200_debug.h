@@ -13,9 +13,13 @@ extern "C" {
 #endif
 
 /* Test/diagnostic access to workspace tensors of the last forward/backward.  `which` is a
- * MOE_BUF_* id; *ptr receives a device pointer into the workspace (valid until the next call on
- * the context), *elems its element count.  Rows of expert-ordered tensors live in a padded row
- * space: expert e starts at row pad_off[e] (a multiple of 128) and holds counts[e] rows. */
+ * MOE_BUF_* id; *ptr receives a device pointer (valid until the next call of the layer on the
+ * context), *elems its element count.  Rows of expert-ordered tensors live in a padded row
+ * space: expert e starts at row pad_off[e] (a multiple of 128) and holds counts[e] rows.
+ * The pointer is into the workspace -- except for an expert-ordered tensor whose row is not a multiple of
+ * 64 elements: its rows lie farther apart there, and *ptr is a compact copy made by this call on the context's last stream
+ * (it waits for that stream).  Each tensor has a copy of its own, allocated outside the workspace when it is
+ * first asked for and freed with the context. */
 enum {
   MOE_BUF_COUNTS = 0,    /* int32 [E+S] */
   MOE_BUF_OFFSETS = 1,   /* int32 [E+S+1] */

@@ -213,8 +213,7 @@ struct moe_ctx {
   unsigned long long clear_capture = 0;   // .. for work in this stream capture (0: none)
   int dep_extra = 0;  // test hook: makes the activation dependencies of the persistent launch unreachable
   cudaStream_t last_stream = nullptr;
-  void* debug_copy = nullptr;   // moe_debug_buffer: the last row-space tensor asked for, compact
-  size_t debug_bytes = 0;
+  void* debug_copy[MOE_BUF_EVENT_COUNTERS + 1] = {};   // moe_debug_buffer: the row-space tensors asked for, compact
   // host-buffer entry points: a copy-in stream (the next call's large input arrives while the previous
   // call still computes) and a copy-out stream (the result leaves in token chunks behind the combine)
   bool copy_ready = false;
@@ -852,7 +851,8 @@ int moe_destroy(moe_ctx* c) {
     cudaEventDestroy(c->ev_d2h_done);
     for (int i = 0; i < HOST_CHUNKS; ++i) cudaEventDestroy(c->ev_chunk[i]);
   }
-  if (c->debug_copy) cudaFree(c->debug_copy);
+  for (void* p : c->debug_copy)
+    if (p) cudaFree(p);
   if (c->owns_ws) cudaFree(c->ws);
   delete c;
   return MOE_OK;
@@ -1156,18 +1156,12 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
   *ptr = c->ws + off;
   *elems = cols ? cap * cols : n;
   if (cols && cols != (size_t)row_ld((int)cols)) {   // rows are farther apart in the workspace: a compact copy
-    const size_t ld = row_ld((int)cols), bytes = 2 * cap * cols;
-    if (bytes > c->debug_bytes) {
-      MOE_CUDA(cudaStreamSynchronize(c->last_stream));
-      if (c->debug_copy) MOE_CUDA(cudaFree(c->debug_copy));
-      c->debug_copy = nullptr;
-      c->debug_bytes = 0;
-      MOE_CUDA(cudaMalloc(&c->debug_copy, bytes));
-      c->debug_bytes = bytes;
-    }
-    MOE_CUDA(cudaMemcpy2DAsync(c->debug_copy, 2 * cols, c->ws + off, 2 * ld, 2 * cols, cap, cudaMemcpyDeviceToDevice, c->last_stream));
+    const size_t ld = row_ld((int)cols);
+    void*& copy = c->debug_copy[which];
+    if (!copy) MOE_CUDA(cudaMalloc(&copy, 2 * cap * cols));
+    MOE_CUDA(cudaMemcpy2DAsync(copy, 2 * cols, c->ws + off, 2 * ld, 2 * cols, cap, cudaMemcpyDeviceToDevice, c->last_stream));
     MOE_CUDA(cudaStreamSynchronize(c->last_stream));
-    *ptr = c->debug_copy;
+    *ptr = copy;
   }
   return MOE_OK;
 }

@@ -1,5 +1,7 @@
 """The matrix queue's items where its rules change: column tiles of long experts, strips cut into pieces, items taken in
 batches, the combine order's token limit; and host buffers that are not pinned."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -134,3 +136,23 @@ def test_host_memory_is_used_in_place_only_within_one_registration():
     finally:
         rt.cudaHostUnregister(first)
         rt.cudaHostUnregister(second)
+
+
+def test_workspace_views_of_one_context_stay_apart():
+    """Rows of 136 and 72 columns are padded in the workspace: each tensor's compact copy stays while others are asked for."""
+    T, d, E, k, S, F = 70, 136, 5, 2, 1, 72
+    x, W1, W2, logits, _ = small_problem(T, d, E, k, S, F, 12)
+    layer = MoeLayer(T, d, E, k, S, F, save_for_bwd=True)
+    ids, w = layer.route(logits)
+    layer.ffn_fwd(x, ids, w, W1, W2)
+    names = ("Xp", "Y", "A", "H")
+    want = [layer.debug(n) for n in names]
+    views = []
+    for n in names:
+        ptr, elems = ctypes.c_void_p(), ctypes.c_size_t()
+        assert B.load_library().moe_debug_buffer(layer.ctx, B.MOE_BUF[n], ctypes.byref(ptr), ctypes.byref(elems)) == 0
+        views.append(torch.as_tensor(B._DevView(ptr.value, elems.value, "<i2"), device="cuda"))
+    rows = (layer.debug("prow_of")[:T * (k + S)].long(), )
+    for n, v, t, cols in zip(names, views, want, (d, d, F, 2 * F)):
+        assert torch.equal(v.view(-1, cols)[rows], t.view(torch.int16).view(-1, cols)[rows]), n
+    layer.close()
