@@ -65,11 +65,11 @@ int moe_debug_host_direct(const void* p, size_t bytes);
 
 /* Host-only check of the static tile schedule of the single persistent launch (Section 4.3: tasks
  * in statically ordered queues, dependent/trigger event counters with static thresholds).  For the
- * given per-expert row counts[Ep] and layer shape it builds the layout tables, the matrix queue of
- * each of `pairs` CTA pairs (the operators of the pass as consecutive phases, items dealt round-robin)
- * and the vector queue, verifies that every M-block is covered exactly once by every column tile of
- * every row-space phase, lets the pairs and `vec_workers` vector workers run -- each blocking on the
- * dependent counters of its current item -- and verifies that every counter ends at its threshold.
+ * given per-expert row counts[Ep] and layer shape it builds the layout tables, the matrix queue (the operators of
+ * the pass as consecutive phases) and the vector queue, verifies that every M-block is covered exactly once by every
+ * column tile of every row-space phase, lets `pairs` CTA pairs and `vec_workers` vector workers run -- a pair takes
+ * tickets in the launch's batches, ahead of its work and before their events are met, and works them off in order; each blocks on
+ * the dependent counters of its current item -- and verifies that every counter ends at its threshold.
  * Returns 0, or a positive code naming the violated property (10 = malformed item, 13 = coverage,
  * 20 = deadlock, 30 = counter off its threshold).  stats[4] (may be NULL) = {matrix items, vector
  * tasks, scheduler rounds, stalled polls}.  Needs no GPU. */

@@ -434,43 +434,48 @@ int gate_mode(const moe_ctx* c) {
 }
 bool serial_mode(const moe_ctx* c) { return (c->shape.flags & MOE_FLAG_SERIAL_LAUNCH) != 0; }
 
-ChainParams chain_params(const moe_ctx* c, bool bwd, int T, bool want_dw) {
-  const moe_shape& s = c->shape;
+// What a pass over T tokens consists of in a launch on `pairs` CTA pairs.
+ChainParams make_chain(bool bwd, int T, int Ep, int k, int n_shared, int d, int F, int pairs) {
   ChainParams cp;
   memset(&cp, 0, sizeof cp);
   cp.is_bwd = bwd ? 1 : 0;
-  cp.Ep = s.E + s.n_shared;
+  cp.Ep = Ep;
   cp.T = T;
-  cp.k = s.k;
-  cp.kp = s.k + s.n_shared;
-  cp.dep_extra = c->dep_extra;
-  cp.want_dw = want_dw ? 1 : 0;
-  cp.combine_split = combine_split_of(T, s.d);
+  cp.k = k;
+  cp.kp = k + n_shared;
+  cp.combine_split = combine_split_of(T, d);
   if (!bwd) {
     cp.n_phases = 2;
-    cp.ntn[0] = (s.F + 127) / 128;                 // gate+up: 128 features (gate and up) per pair tile
-    cp.ntn[1] = (s.d + 255) / 256;                 // down
+    cp.ntn[0] = (F + 127) / 128;                 // gate+up: 128 features (gate and up) per pair tile
+    cp.ntn[1] = (d + 255) / 256;                 // down
     cp.merges[1] = 1;
   } else {
     cp.n_phases = 4;
-    cp.ntn[0] = c->plan.ntn_act;                   // act_grad
-    cp.ntn[1] = (s.F + 255) / 256;                 // w2_grad: column tiles per strip
-    cp.strips[1] = (s.d + 255) / 256;
-    cp.ntn[2] = (s.d + 255) / 256;                 // gate_grad
+    cp.ntn[0] = (F + 255) / 256;                 // act_grad
+    cp.ntn[1] = (F + 255) / 256;                 // w2_grad: column tiles per strip
+    cp.strips[1] = (d + 255) / 256;
+    cp.ntn[2] = (d + 255) / 256;                 // gate_grad
     cp.merges[2] = 1;
-    cp.ntn[3] = (s.d + 255) / 256;                 // w1_grad
-    cp.strips[3] = (2 * s.F + 255) / 256;
+    cp.ntn[3] = (d + 255) / 256;                 // w1_grad
+    cp.strips[3] = (2 * F + 255) / 256;
   }
   // k-blocks of an item: the reduction, or a strip's column tiles times those of an average expert
-  const int kb_d = (s.d + 63) / 64, kb_F = (s.F + 63) / 64, kb_rows = (int)(((long)T * cp.kp / cp.Ep + 63) / 64);
+  const int kb_d = (d + 63) / 64, kb_F = (F + 63) / 64, kb_rows = (int)(((long)T * cp.kp / cp.Ep + 63) / 64);
   for (int ph = 0; ph < cp.n_phases; ++ph) {
     int kb = ph == 0 ? kb_d : bwd ? 2 * kb_F : kb_F;
     if (cp.strips[ph]) {
-      cp.split[ph] = strip_split(cp.Ep, cp.strips[ph], cp.ntn[ph], c->num_sms / 2);
+      cp.split[ph] = strip_split(cp.Ep, cp.strips[ph], cp.ntn[ph], pairs);
       kb = (cp.ntn[ph] + cp.split[ph] - 1) / cp.split[ph] * (kb_rows > 4 ? kb_rows : 4);   // a tile's stores are worth four
     }
     cp.batch[ph] = sched_batch(kb);
   }
+  return cp;
+}
+ChainParams chain_params(const moe_ctx* c, bool bwd, int T, bool want_dw) {
+  const moe_shape& s = c->shape;
+  ChainParams cp = make_chain(bwd, T, s.E + s.n_shared, s.k, s.n_shared, s.d, s.F, c->num_sms / 2);
+  cp.dep_extra = c->dep_extra;
+  cp.want_dw = want_dw ? 1 : 0;
   return cp;
 }
 
@@ -1172,7 +1177,7 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
 // item's dependent counters.
 int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, int32_t k, int32_t n_shared, int32_t d,
                                 int32_t F, int32_t is_bwd, int32_t pairs, int32_t vec_workers, int64_t* stats) {
-  if (!counts || Ep < 1 || pairs < 1 || vec_workers < 1 || d < 8 || F < 16) return MOE_ERR_INVALID_ARG;
+  if (!counts || Ep < 1 || pairs < 1 || vec_workers < 1 || d < 8 || F < 8) return MOE_ERR_INVALID_ARG;
   // the tables of the layout kernels
   std::vector<int> mb_start(Ep + 1, 0), pair_start(Ep + 1, 0), work_start(Ep + 1, 0);
   for (int e = 0; e < Ep; ++e) {
@@ -1191,32 +1196,24 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
     for (int i = pair_start[e]; i < pair_start[e + 1]; ++i) pblk[i] = e;
     for (int i = work_start[e]; i < work_start[e + 1]; ++i) wblk[i] = e;
   }
-  ChainParams cp;
-  memset(&cp, 0, sizeof cp);
-  cp.is_bwd = is_bwd; cp.Ep = Ep; cp.T = T; cp.k = k; cp.kp = k + n_shared; cp.want_dw = 1;
-  cp.combine_split = combine_split_of(T, d);
-  if (!is_bwd) {
-    cp.n_phases = 2; cp.ntn[0] = (F + 127) / 128; cp.ntn[1] = (d + 255) / 256; cp.merges[1] = 1;
-  } else {
-    cp.n_phases = 4; cp.ntn[0] = (F + 255) / 256; cp.ntn[1] = (F + 255) / 256; cp.strips[1] = (d + 255) / 256;
-    cp.ntn[2] = (d + 255) / 256; cp.merges[2] = 1; cp.ntn[3] = (d + 255) / 256; cp.strips[3] = (2 * F + 255) / 256;
-  }
+  ChainParams cp = make_chain(is_bwd != 0, T, Ep, k, n_shared, d, F, pairs);
+  cp.want_dw = 1;
   // items of every phase: {first M-block, M-blocks of unit a, M-blocks of unit b} (strips: the expert's M-blocks)
   struct Item { int phase, mb_first, mb_a, mb_b, e; };
-  std::vector<std::vector<Item>> queue(pairs);
-  long n_items = 0, n_queued = 0;
+  std::vector<Item> queue;   // in ticket order
+  std::vector<int> batch_log2(cp.n_phases, 0);
+  long n_items = 0;
   std::vector<std::vector<int>> cover(cp.n_phases, std::vector<int>(M + 1, 0));
   for (int ph = 0; ph < cp.n_phases; ++ph) {
+    const size_t phase_first = queue.size();
     if (cp.strips[ph]) {
-      const int split = strip_split(Ep, cp.strips[ph], cp.ntn[ph], pairs);
-      const int total = strip_items(Ep, cp.strips[ph], cp.ntn[ph], split, n_long);
+      const int split = cp.split[ph], total = strip_items(Ep, cp.strips[ph], cp.ntn[ph], split, n_long);
       std::vector<int> tiles((size_t)Ep * cp.strips[ph], 0);
       for (int t = 0; t < total; ++t) {
         const StripItem it = decode_strip_item(t, cp.strips[ph], cp.ntn[ph], split, n_long, order.data());
         if (it.e < 0 || it.e >= Ep || it.strip < 0 || it.strip >= cp.strips[ph] || it.nb0 < 0 || it.nb1 > cp.ntn[ph]) return 11;
         tiles[(size_t)it.e * cp.strips[ph] + it.strip] += it.nb1 - it.nb0;
-        queue[t % pairs].push_back(Item{ph, mb_start[it.e], mb_start[it.e + 1] - mb_start[it.e], 0, it.e});
-        ++n_queued;
+        queue.push_back(Item{ph, mb_start[it.e], mb_start[it.e + 1] - mb_start[it.e], 0, it.e});
         n_items += it.nb0 == 0;   // the pieces of a strip count once
       }
       for (int n : tiles)
@@ -1234,10 +1231,11 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
             it.mb_count > 3 || it.mb_count_a < 1)
           return 10;
         for (int q = 0; q < it.mb_count; ++q) cover[ph][it.mb_first + q]++;
-        queue[tq % pairs].push_back(Item{ph, it.mb_first, it.mb_count_a, it.mb_count - it.mb_count_a, it.e});
-        ++n_items, ++n_queued;
+        queue.push_back(Item{ph, it.mb_first, it.mb_count_a, it.mb_count - it.mb_count_a, it.e});
+        ++n_items;
       }
     }
+    batch_log2[ph] = phase_batch_log2((int)(queue.size() - phase_first), cp.batch[ph], 2 * pairs);
   }
   // 1. coverage: every M-block is covered by every column tile of every row-space phase exactly once
   for (int ph = 0; ph < cp.n_phases; ++ph)
@@ -1246,7 +1244,11 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
         if (cover[ph][mb] != cp.ntn[ph]) return 13;
   // 2. execution with a bounded number of workers
   std::vector<long> ctr(ctr_ints(M + 1), 0);
-  std::vector<size_t> cursor(pairs, 0);
+  // a pair's scheduler takes the next tickets when the pair then holds at most sched_hold() items not begun, whether or not
+  // their dependent events are met; the pair works its items off in order
+  struct Pair { std::vector<size_t> held; size_t at = 0; int batch = 1, phase = 0; };
+  std::vector<Pair> pair(pairs);
+  size_t next_ticket = 0;
   // 32-row groups: first of each expert, M-block of each
   std::vector<int> group_start(Ep + 1, 0), group_mb;
   for (int e = 0; e < Ep; ++e) {
@@ -1268,11 +1270,20 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   long done_mat = 0, done_vec = 0, rounds = 0, stalls = 0;
   int next_gather = 0, next_post = 0;
   const int vtotal = ngather + npost;
-  while (done_mat < n_queued || done_vec < vtotal) {
+  while (done_mat < (long)queue.size() || done_vec < vtotal) {
     bool progress = false;
-    for (int q = 0; q < pairs; ++q) {
-      if (cursor[q] >= queue[q].size()) continue;
-      const Item& it = queue[q][cursor[q]];
+    for (Pair& p : pair) {
+      const size_t room = sched_hold(p.batch, cp.strips[p.phase] != 0);
+      if (next_ticket < queue.size() && p.held.size() - p.at + p.batch <= room) {
+        for (int b = 0; b < p.batch && next_ticket < queue.size(); ++b) {
+          p.phase = queue[next_ticket].phase;
+          p.held.push_back(next_ticket++);
+        }
+        p.batch = 1 << batch_log2[p.phase];
+        progress = true;
+      }
+      if (p.at == p.held.size()) continue;
+      const Item& it = queue[p.held[p.at]];
       const int wk = phase_wait_kind(cp, it.phase);
       bool ready = true;
       for (int m = 0; m < it.mb_a + it.mb_b; ++m)
@@ -1282,7 +1293,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
       const int tk = phase_trigger_kind(cp, it.phase);
       if (tk >= 0)
         for (int m = 0; m < it.mb_a + it.mb_b; ++m) ctr[ctr_index(it.mb_first + m, tk)] += SIG;
-      ++cursor[q]; ++done_mat; progress = true;
+      ++p.at; ++done_mat; progress = true;
     }
     for (size_t wi = 0; wi < vw.size(); ++wi) {
       auto& w = vw[wi];

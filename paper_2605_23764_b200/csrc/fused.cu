@@ -521,13 +521,10 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
     const PhaseTable pt = make_phase_table<BWD>(fa);
     const PhaseTable rot = make_rotation_table<BWD>(fa);   // first item of the first shared expert in each row-space phase
     const int total = pt.start[SCHED_MAX_SEG];
-    // batches pay with many items to a pair; with few, the last ones would lie with some of the pairs
     int batches = 0;   // two bits a phase: log2
 #pragma unroll
-    for (int p = 0; p < SCHED_MAX_SEG; ++p) {
-      const int items = pt.start[p + 1] - pt.start[p], most = fa.cp.batch[p];   // 16 and 8 for each pair
-      batches |= (items >= 8 * (int)gridDim.x && most == 4 ? 2 : items >= 4 * (int)gridDim.x && most >= 2 ? 1 : 0) << (2 * p);
-    }
+    for (int p = 0; p < SCHED_MAX_SEG; ++p)
+      batches |= phase_batch_log2(pt.start[p + 1] - pt.start[p], fa.cp.batch[p], (int)gridDim.x) << (2 * p);
     int batch = 1, phase = 0;   // of the last ticket
     bool more = true;
     for (uint32_t n = 0; more;) {

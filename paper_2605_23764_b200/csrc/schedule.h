@@ -183,6 +183,11 @@ struct ChainParams {
 // the pace of a pair whose items are shorter (down with F = 192: 0.7 us of MMAs, 4 us an item).  Items of a few k-blocks are
 // therefore taken two or four at a time.  Not longer ones: the last items of a launch would lie with few pairs.
 MOE_HD int sched_batch(int kblocks) { return kblocks <= 8 ? 4 : kblocks <= 16 ? 2 : 1; }
+// Batches pay with many items to a pair; with few, the last ones would lie with some of the pairs.  log2 of the batch of a phase
+// of `items` items, of at most `most`: 16 and 8 items for each pair of the launch's `ctas`.
+MOE_HD int phase_batch_log2(int items, int most, int ctas) {
+  return items >= 8 * ctas && most == 4 ? 2 : items >= 4 * ctas && most >= 2 ? 1 : 0;
+}
 // Items a pair holds at most that its epilogue has not begun: enough to hide the 3 us (with one fewer than four row-space
 // items the passes over few tokens were 2-6 % slower).  Strips of a weight gradient are tens of microseconds long and of
 // unequal length, four and a half to a pair in a step of 3400 tokens: what a pair holds beyond the next two nobody else can take.

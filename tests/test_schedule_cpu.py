@@ -86,3 +86,14 @@ def test_layout_takes_the_kernels_where_a_cluster_does_not_fit():
     for T in (1025, 8192):
         assert blocks(T, 8, 64, fits8=False) == 16 and blocks(T, 8, 64, fits16=False) == 0
     assert blocks(123, 8, 64, fits8=False, fits16=False) == 1
+
+
+@pytest.mark.parametrize("is_bwd", [0, 1])
+@pytest.mark.parametrize("pairs", [1, 2, 5, 74])
+@pytest.mark.parametrize("d,F", [(4096, 8), (2048, 64), (256, 520)])   # items of one, one and nine k-blocks of F
+def test_schedule_with_batches_of_tickets(is_bwd, pairs, d, F):
+    """Many short items: pairs hold up to eight of them whose events are not met yet; long experts and shared ones among them."""
+    rng = np.random.default_rng(pairs)
+    counts = np.concatenate([rng.integers(0, 90, 96), [1000, 640, 640]])   # the last two: shared experts
+    rc, stats = binding.moe_debug_simulate_schedule(counts, 640, 8, 2, d, F, is_bwd, pairs, 3)
+    assert rc == 0
