@@ -283,16 +283,11 @@ class Workload:
         # weights that fit L2 would stay there from step to step: flush between timed steps
         self.flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda") if cfg.weight_bytes() <= 4e8 else None
 
-    plain_launch = False   # --plain-launch: persistent launches without the cooperative attribute (profiler captures)
-
     def make_layer(self, mode, defer_out_copy=False):
-        from paper_2605_23764_b200 import MoeLayer, binding as B
+        from paper_2605_23764_b200 import MoeLayer
         c = self.cfg
-        lay = MoeLayer(c.T, c.d, c.E, c.k, c.S, c.F, renorm=c.renorm, save_for_bwd=self.train, serial=(mode == "serial"),
-                       defer_out_copy=defer_out_copy)
-        if Workload.plain_launch:
-            B.moe_debug_set_plain_launch(lay.ctx, True)
-        return lay
+        return MoeLayer(c.T, c.d, c.E, c.k, c.S, c.F, renorm=c.renorm, save_for_bwd=self.train, serial=(mode == "serial"),
+                        defer_out_copy=defer_out_copy)
 
     def step(self, lay, phases=None):
         """One pass of the hot path through the C ABI (device buffers).  -> kernels launched"""
@@ -658,7 +653,8 @@ def main():
     ap.add_argument("--only-ep", action="store_true", help="run the emulated expert-parallel dispatch / combine alone")
     ap.add_argument("--study-iters", type=int, default=30)
     ap.add_argument("--plain-launch", action="store_true",
-                    help="diagnostic: persistent launches without the cooperative launch attribute (for profiler captures)")
+                    help="diagnostic: the scheduling study's and the expert-parallel exchange's persistent launches without the "
+                         "cooperative launch attribute (for profiler captures; the layer's launches never have it)")
     ap.add_argument("--small", type=str, default="", help="T,d,F[,E]: reduced sizes of the chosen config (profiling captures)")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3) if args.impl == "ours" else args.warmup
@@ -681,7 +677,6 @@ def main():
 
     if args.plain_launch:
         from paper_2605_23764_b200 import binding as B
-        Workload.plain_launch = True
         B.moe_debug_set_plain_launch(None, True)
     if args.only_ep:
         torch.cuda.set_device(0)

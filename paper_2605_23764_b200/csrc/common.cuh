@@ -55,9 +55,6 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -237,19 +234,6 @@ __device__ __forceinline__ void ldmatrix4_trans(uint32_t addr, uint32_t* r) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Shared-memory matrix descriptor (sm_100 format): start address, leading/stride byte offsets
-// (all >> 4), descriptor version 1, 128-byte swizzle.  Tile bases are 1024-byte aligned, so the
-// base-offset field stays 0.
-__device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= static_cast<uint64_t>((smem_addr >> 4) & 0x3FFF);
-  d |= static_cast<uint64_t>((lbo_bytes >> 4) & 0x3FFF) << 16;
-  d |= static_cast<uint64_t>((sbo_bytes >> 4) & 0x3FFF) << 32;
-  d |= 1ull << 46;  // descriptor version (Blackwell)
-  d |= 2ull << 61;  // SWIZZLE_128B
-  return d;
-}
-
 // Instruction descriptor of tcgen05.mma kind::f16: bf16 x bf16 -> fp32, M x N tile, operand
 // major-ness (0 = K-major, 1 = MN-major).
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N, int a_mn_major, int b_mn_major) {
@@ -397,7 +381,8 @@ __device__ __forceinline__ void tc_mma1_bf16_pair(uint32_t d_tmem, uint32_t a_lo
       ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Halves of make_smem_desc(addr, lbo, sbo)
+// Shared-memory matrix descriptor (sm_100 format), its two words: start address and leading / stride byte offsets (all >> 4),
+// descriptor version 1, 128-byte swizzle.  Tile bases are 1024-byte aligned, so the base-offset field stays 0.
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t smem_addr, uint32_t lbo_bytes) {
   return ((smem_addr >> 4) & 0x3FFFu) | (((lbo_bytes >> 4) & 0x3FFFu) << 16);
 }

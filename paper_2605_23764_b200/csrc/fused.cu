@@ -5,8 +5,8 @@
 //   warp 1      tcgen05.mma issuer (even CTA) and TMEM owner
 //   warps 2-5, 8-11  epilogue: TMEM -> fused element-wise math -> global memory, then the tile's trigger event
 //   warp 6      TMA producer of the tokens (weight gradients: of the B operand)
-//   warp 7      even CTA: scheduler of the pair -- takes the next ticket of the matrix queue, waits for
-//               the item's dependent events, publishes it to the other roles; odd CTA: vector worker
+//   warp 7      even CTA: scheduler of the pair -- takes the next tickets of the matrix queue, looks at the
+//               items' dependent events and publishes the items to the other roles, met or not; odd CTA: vector worker
 //   warps 12-15 vector workers: tickets of the vector queue (permute-gather, routing-weight
 //               gradient, combine); the matrix-role warps join them once the matrix queue is empty.
 // The matrix roles are the ones of the one-launch-per-operator kernels (gemm_roles.cuh); here they

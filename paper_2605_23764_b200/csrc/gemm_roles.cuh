@@ -498,13 +498,13 @@ __device__ __forceinline__ bool wgrad_epilogue_strip(const GemmArgs& a, uint8_t*
                                                      const Strip& st, int sp, const WaitCtl& wc, const DEP& dep) {
   uint8_t* box = smem + WGRAD_STAGING_AT + ew * OUT_BOX_BYTES;
   Tile tl;
-  tl.e = st.e; tl.row0 = st.row0; tl.m0 = st.m0(rank); tl.nkb = st.nkb;
+  tl.e = st.e; tl.m0 = st.m0(rank); tl.nkb = st.nkb;
   const bool idle = tl.m0 >= a.M;   // the strip's second half lies outside dW: nothing to store
   bool ok = true;
   uint64_t t0 = 0;
   if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
   for (int nb = st.nb0; nb < st.nb1; ++nb) {
-    tl.nb = nb; tl.n0 = nb * BN;
+    tl.n0 = nb * BN;
     if (st.nkb == 0) {
       if (!idle) epilogue_wgrad_tile(a, tl, 0, ew, lane, box);  // an expert without rows: zeros
       continue;

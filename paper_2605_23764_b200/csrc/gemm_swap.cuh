@@ -4,13 +4,13 @@
 // steps of 32, half of them in each CTA's shared memory).  The MMA time of a tile then follows the
 // number of tokens it really holds instead of the padded 256 rows of a token-row tile.
 //
-// The accumulator arrives transposed (TMEM lane = output feature, column = token); the epilogues
-// write it back token-major through small un-swizzled staging boxes and TMA stores.
+// The accumulator arrives transposed (TMEM lane = output feature, column = token); the epilogues write it back token-major:
+// transposing stmatrix into a small staging box of the warp's own, read back by rows, plain 16-byte stores.
 #pragma once
 
 #include <cuda_bf16.h>
 
-#include "gemm_pair.cuh"
+#include "gemm_tile.cuh"
 
 namespace moe {
 

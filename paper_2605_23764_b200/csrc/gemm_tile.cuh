@@ -9,23 +9,27 @@
 
 namespace moe {
 
-
 constexpr int BN = 256;                       // accumulator columns per tile
 constexpr int BK = 64;                        // reduction elements per stage (one 128-byte swizzle row)
 constexpr int A_STAGE_BYTES = BLOCK_M * BK * 2;  // 16 KB
 constexpr int B_STAGE_BYTES = BN * BK * 2;       // 32 KB
 constexpr int MN_BOX_BYTES = 64 * BK * 2;        // one [64 k][64 mn] box of an MN-major operand
+constexpr int HALF_B_BYTES = B_STAGE_BYTES / 2;  // 16 KB: a CTA's half of a pair's B tile
 constexpr int TMEM_COLS = 512;
 constexpr int OUT_BOX_BYTES = 32 * 64 * 2;       // epilogue staging box: 32 rows x 64 bf16 columns
 
-struct Tile {
+struct Tile {   // of a weight gradient
   int e;      // expert
-  int row0;   // row-space modes: first padded row of the M-block; WGRAD: first padded row of the expert
   int n0;     // first output column of the tile
-  int m0;     // WGRAD: first output row (within the expert's slab)
-  int nkb;    // k-blocks of the main loop (may be 0 for an expert without rows in WGRAD)
-  int nb;     // column-tile index (ACT_GRAD partials)
+  int m0;     // first output row (within the expert's slab)
+  int nkb;    // k-blocks of the main loop (0 for an expert without rows)
 };
+
+// 16-row MMA steps needed in k-block kb of a reduction over `rows` rows
+__device__ __forceinline__ int k16_steps_of(int rows, int kb) {
+  const int left = rows - kb * BK;
+  return left >= BK ? BK / 16 : (left + 15) / 16;
+}
 
 // ---------------------------------------------------------------- epilogues
 // Weight gradients: an epilogue warp owns 32 rows of the tile (its TMEM lane quadrant) and private staging boxes of

@@ -6,7 +6,7 @@
 // tile of up to 256 tokens the B operand, and a cluster of 1, 2, 4 or 8 CTAs shares a tile by splitting the reduction
 // over d.  Each CTA streams its k-blocks through a TMA ring into TMEM; then the CTAs exchange partial sums through
 // distributed shared memory -- every CTA ends up with all experts' partials for its share of the tile's tokens, adds them in
-// CTA order, so the result does not depend on timing -- and its sixteen warps select, one token per warp
+// CTA order, so the result does not depend on timing -- and its sixteen warps select, four tokens per warp
 // (warp_topk: raw logits compared, ties to the lower id, slots in descending order).
 //
 // What bounds it: few tokens, latency -- W_r is 3.7 MB at 256 x 7168 and one CTA pair needed 65 us to stream it; many tokens,
@@ -14,7 +14,7 @@
 // tokens, with the selection exposed behind them: 70 us.  See plan_router_fwd for the choice of tile and split.
 #include <limits.h>
 
-#include "gemm_pair.cuh"
+#include "gemm_tile.cuh"
 #include "launch_pairs.cuh"
 #include "moe_internal.h"
 #include "topk.cuh"
