@@ -256,13 +256,12 @@ constexpr int TK_RING = 8;
 // scheduler does it once, ahead of time, for every role of both CTAs).
 struct __align__(16) WorkDesc {
   int ticket;                                  // -1: the queue is empty
-  int phase, item, flags;                      // WD_MERGED, WD_READY, the ring
+  int phase, item, flags;                      // WD_MERGED, WD_READY
   int e, n0, nb, nkb;                          // strips: nb = 256-row block of dW, n0 = first column tile
   int a_row0, a_ntok, a_mb_first, a_mb_count;  // strips: a_row0 = first padded row, a_ntok = rows of the expert
   int b_row0, b_ntok, b_mb_first, b_mb_count;  // strips: b_row0 = end of the column tiles
 };
 constexpr int WD_MERGED = 1, WD_READY = 2;   // READY: the dependent events were met when the item was published
-constexpr int WD_STAGES_AT = 8, WD_TOKENS_AT = 16;   // row-space items: their operand ring, token bytes of a stage in units of 2 KB
 static_assert(sizeof(WorkDesc) == 64, "published as four 16-byte stores");
 struct __align__(16) TicketRing {
   WorkDesc work[TK_RING];
@@ -323,18 +322,14 @@ __device__ __forceinline__ SwapWork desc_swap_work(const WorkDesc& wd) {
   w.b.row0 = wd.b_row0; w.b.ntok = wd.b_ntok; w.b.mb_first = wd.b_mb_first; w.b.mb_count = wd.b_mb_count;
   return w;
 }
-__device__ __forceinline__ Ring desc_ring(const WorkDesc& wd) {
-  return Ring{(wd.flags >> WD_STAGES_AT) & 0xFF, (wd.flags >> WD_TOKENS_AT) << 11};
-}
 __device__ __forceinline__ Strip desc_strip(const WorkDesc& wd) {
   Strip st;
   st.e = wd.e; st.mp = wd.nb; st.row0 = wd.a_row0; st.rows = wd.a_ntok; st.nkb = wd.nkb;
   st.nb0 = wd.n0; st.nb1 = wd.b_row0;
   return st;
 }
-__device__ __forceinline__ void pack_swap_work(WorkDesc& wd, const SwapWork& w, const Ring& r) {
-  static_assert(TOK_GRAIN / 2 * BK * 2 == 2048, "token bytes are multiples of 2 KB");
-  wd.flags = (w.merged ? WD_MERGED : 0) | r.stages << WD_STAGES_AT | (r.tok_bytes >> 11) << WD_TOKENS_AT;
+__device__ __forceinline__ void pack_swap_work(WorkDesc& wd, const SwapWork& w) {
+  wd.flags = w.merged ? WD_MERGED : 0;
   wd.e = w.a.e; wd.n0 = w.a.n0; wd.nb = w.a.nb; wd.nkb = w.a.nkb;
   wd.a_row0 = w.a.row0; wd.a_ntok = w.a.ntok; wd.a_mb_first = w.a.mb_first; wd.a_mb_count = w.a.mb_count;
   wd.b_row0 = w.b.row0; wd.b_ntok = w.b.ntok; wd.b_mb_first = w.b.mb_first; wd.b_mb_count = w.b.mb_count;
@@ -357,8 +352,7 @@ __device__ __forceinline__ void decode_item(const FusedArgs& fa, int phase, int 
   SwapWork w;
   if (!BWD) w = phase == 0 ? decode_swap_work<GEMM_GATE_UP>(fa.op[0], item) : decode_swap_work<GEMM_DOWN>(fa.op[1], item);
   else w = phase == 0 ? decode_swap_work<GEMM_ACT_GRAD>(fa.op[0], item) : decode_swap_work<GEMM_GATE_GRAD>(fa.op[2], item);
-  const GemmMode ring_mode = !BWD ? GEMM_GATE_UP : phase == 0 ? GEMM_ACT_GRAD : GEMM_GATE_GRAD;   // the forward's two share one
-  pack_swap_work(wd, w, ring_of(ring_mode, fa.lv.meta[7]));
+  pack_swap_work(wd, w);
   *first = w.a.mb_first; *count = w.a.mb_count + w.b.mb_count;
 }
 
@@ -423,7 +417,7 @@ __device__ __forceinline__ ChainDeps phase_deps(const FusedArgs& fa, int phase, 
 
 // ---------------------------------------------------------------- one item, by role
 template <bool BWD>
-__device__ __forceinline__ bool load_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool load_item(const FusedArgs& fa, bool full, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                           LoaderState& ls, bool second_warp, int rank, int lane, const WaitCtl& wc,
                                           const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
@@ -435,29 +429,27 @@ __device__ __forceinline__ bool load_item(const FusedArgs& fa, const WorkDesc& w
   if (strip)
     return wgrad_load_strip(fa.op[phase], smem, bars, ls, second_warp, rank, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
-  const Ring ring = desc_ring(wd);
   if (!BWD) {
-    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-    return swap_load_item<GEMM_DOWN>(fa.op[1], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+    return swap_load_item<GEMM_DOWN>(fa.op[1], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
 }
 template <bool BWD>
-__device__ __forceinline__ bool issue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool issue_item(const FusedArgs& fa, bool full, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                            uint32_t tmem_base, IssuerState& is, const WaitCtl& wc,
                                            const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
   if (BWD && (phase == 1 || phase == 3))
     return wgrad_issue_strip(fa.op[phase], smem, bars, tmem_base, is, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
-  const Ring ring = desc_ring(wd);
   if (!BWD) {
-    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], ring, smem, bars, tmem_base, is, wk, t, wc, dep);
-    return swap_issue_item<GEMM_DOWN>(fa.op[1], ring, smem, bars, tmem_base, is, wk, t, wc, dep);
+    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], full, smem, bars, tmem_base, is, wk, t, wc, dep);
+    return swap_issue_item<GEMM_DOWN>(fa.op[1], full, smem, bars, tmem_base, is, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], ring, smem, bars, tmem_base, is, wk, t, wc, dep);
-  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], ring, smem, bars, tmem_base, is, wk, t, wc, dep);
+  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], full, smem, bars, tmem_base, is, wk, t, wc, dep);
+  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], full, smem, bars, tmem_base, is, wk, t, wc, dep);
 }
 template <bool BWD>
 __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
@@ -569,6 +561,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
     }
   } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
+    const bool full = wants_full_ring(fa.op[0]);
     LoaderState ls;
     IssuerState is;
     EpiState es;
@@ -599,9 +592,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         }
       }
       if (warp == 0 || warp == 6)
-        ok = load_item<BWD>(fa, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
+        ok = load_item<BWD>(fa, full, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
       else if (warp == 1)
-        ok = issue_item<BWD>(fa, wd, smem, bars, tmem_base, is, wc, dep);
+        ok = issue_item<BWD>(fa, full, wd, smem, bars, tmem_base, is, wc, dep);
       else
         ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, wc, dep);
     }

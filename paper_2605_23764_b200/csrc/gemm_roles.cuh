@@ -17,7 +17,7 @@ namespace moe {
 
 constexpr int WG_A_SLOTS = 5;    // weight gradients: 16 KB slots of the strip's A operand
 constexpr int WG_B_STAGES = 7;   // weight gradients: 16 KB stages of the streamed B operand
-constexpr int MAX_STAGES = 12;   // row-space operators: see ring_of
+constexpr int MAX_STAGES = 12;   // row-space operators: see plan_ring
 constexpr size_t WGRAD_STAGING_AT = (size_t)WG_A_SLOTS * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES;   // behind both
 
 // Warps of a GEMM CTA: 0 weight loader, 1 MMA issuer, 2-5 and 8-11 epilogue, 6 token loader, 7 left to the kernel (scheduler).
@@ -186,38 +186,32 @@ struct ChainDeps {
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
 // Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes], and at
-// the end of LAYOUT_BYTES the staging.  The token part follows from the rows of the call's largest expert, which the layout
-// leaves in meta[7] -- not from the number of tokens: ids repeated in a token (a batch padded with id 0) give an expert more
-// rows than there are tokens.  Up to 256 rows a tile has at most all of them, n32(rows) / 2 per CTA, and nothing merges; beyond, a
-// merged item (128 + 256) / 2.  What the token stages do not need goes into more stages: with 32 rows eleven, 198 KB of weights
-// in flight instead of 80 -- a pass over few tokens is a stream of weights from HBM.
+// the end of LAYOUT_BYTES the staging.  A call of T <= 256 tokens whose ids are distinct in each token has experts of at most T
+// rows: a tile needs n32(T) / 2 rows per CTA and nothing merges; beyond, a merged item (128 + 256) / 2.  What the token stages do
+// not need goes into more stages: with 32 tokens eleven, 198 KB of weights in flight instead of 80 -- a pass over few tokens is a
+// stream of weights from HBM.  Ids repeated in a token (a batch padded with id 0) give an expert more rows than there are tokens:
+// the layout leaves the rows of the largest expert in meta[7], and a launch that finds more there takes the full stages.  (Both
+// rings come from the host and a bit chooses: worked out in the kernel for every item, passes of short items took 1-3 % longer.)
 constexpr size_t PIPE_BARRIER_BYTES = 384;
 constexpr size_t TICKET_RING_BYTES = 640;   // of the persistent launch
 constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_RING_BYTES;
 __host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return EPI_WARPS * (size_t)sw_staging_bytes(mode); }
 __host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
-struct Ring { int stages, tok_bytes; };   // operand stages, token bytes of a stage per CTA
-// Of an operator whose largest expert has `rows` rows; gate+up's is laid out like down's, behind which it runs on.
-__host__ __device__ inline Ring ring_of(GemmMode mode, int rows) {
-  const bool merges = mode != GEMM_ACT_GRAD;
-  Ring r;
-  r.tok_bytes = rows <= 2 * BLOCK_M ? (rows + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN / 2 * (BK * 2) : (merges ? 3 : 2) * 64 * (BK * 2);
-  r.stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + r.tok_bytes));
-  if (r.stages > MAX_STAGES) r.stages = MAX_STAGES;
-  return r;
-}
+// The same for every role and item of a launch: the layout is complete before them.
+__device__ __forceinline__ bool wants_full_ring(const GemmArgs& a) { return uniform(a.meta[7] > a.ring_rows ? 1 : 0) != 0; }
 // does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
-__device__ __forceinline__ bool above_guard(const Ring& r, uint32_t s) {
+__device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s) {
   return (size_t)r.stages * W_STAGE_BYTES + (size_t)(s + 1) * r.tok_bytes > WGRAD_STAGING_AT ||
          (size_t)(s + 1) * W_STAGE_BYTES > WGRAD_STAGING_AT;
 }
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
 // tokens.
 template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, const Ring& ring, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
+__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, bool full, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
                                                bool tok_warp, int rank, int lane, const SwapWork& wk, int t,
                                                const WaitCtl& wc, const DEP& dep) {
-  const int stages = uniform(ring.stages), tokb = uniform(ring.tok_bytes);
+  const GemmArgs::Ring ring = full ? a.full : a.ring;
+  const int stages = ring.stages, tokb = ring.tok_bytes;
   uint8_t* sW = smem;                              // [stages][16 KB] weights
   uint8_t* sT = smem + stages * W_STAGE_BYTES;     // [stages][tokb] tokens (this CTA's half)
   // with events: the tokens are there (acquired by the scheduler and handed on through the ticket ring, or by the caller);
@@ -248,10 +242,11 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, const Ring& ri
 // MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop with uniform control flow and operands; one elected
 // lane issues (common.cuh).
 template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, const Ring& ring, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
+__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, bool full, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
                                                 IssuerState& is, const SwapWork& wk, int t, const WaitCtl& wc,
                                                 const DEP& dep) {
-  const uint32_t stages = uniform(ring.stages), t_step = uniform(ring.tok_bytes) >> 4;
+  const GemmArgs::Ring ring = full ? a.full : a.ring;
+  const uint32_t stages = ring.stages, t_step = ring.tok_bytes >> 4;
   const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
   const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + stages * W_STAGE_BYTES), 16);
   uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * t_step;
