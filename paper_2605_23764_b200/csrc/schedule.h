@@ -192,9 +192,13 @@ MOE_HD int phase_batch_log2(int items, int most, int ctas) {
 // items the passes over few tokens were 2-6 % slower).  Strips of a weight gradient are tens of microseconds long and of
 // unequal length, four and a half to a pair in a step of 3400 tokens: what a pair holds beyond the next two nobody else can take.
 MOE_HD int sched_hold(int batch, bool strips) { return batch == 4 ? 8 : batch == 1 && strips ? 2 : 4; }
-// Vector warps per CTA that keep gathering after the first tasks.  Two gather 1.4 TB/s in and out, the pace of gate+up at
-// F = 800 and of act_grad at twice that; below, the matrix items waited for the rows (9678 tokens x 10 rows, F = 536: 250 us of
-// MMAs in 420).  Where the products are longer than the gather, more only take from the bandwidth of their loads.
+// Vector warps per CTA that keep gathering after the first tasks.  Two gather 1.4 TB/s in and out; below the F where gate+up (or
+// act_grad, half as long) takes that pace the matrix items wait for the rows, above it more gatherers only take from the
+// bandwidth of their loads.  Two against all four, us forward / backward: 16384 tokens x 8 rows, d = 1024, 32 experts, F = 512
+// 833 -> 530 / 1113 -> 837, F = 1024 913 -> 802 / 1552 -> 1500, F = 1280 even, F = 1536 1047 -> 1175 / 2112 -> 2370; 8192 tokens,
+// d = 2048, 64 experts, F = 512 503 -> 447 / 821 -> 771, F = 1280 925 -> 858 / 1924 -> 1753, even from 1536 on; 4096 tokens,
+// d = 4096, 590 -> 578 / 995 -> 917 at F = 512, even from 1024 on.  Where they part depends on d and the experts' rows, and the
+// runs differ by 5-10 % under the power cap: the lines lie within the band, not at a sharp point.
 MOE_HD int background_gatherers(int is_bwd, int F, int all) { return F <= (is_bwd ? 1536 : 1024) ? all : 2; }
 
 // Gather tasks of M-block `rel` (relative to its expert's first) of an expert with `rows` rows.
