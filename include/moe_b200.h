@@ -119,7 +119,7 @@ int moe_layout(moe_ctx* ctx, const int32_t* topk_ids, int32_t T, int32_t* counts
  *   out[t] = sum_j w(t,j) * ( silu(x_t Wg_e^T) * (x_t Wu_e^T) ) Wd_e^T ,  e = expert of slot j,
  * j over the k routed slots (weight topk_w) and the S shared experts (weight 1).
  * x, out: bf16 [T][d]; topk_ids int32 [T][k]; topk_w fp32 [T][k].  bf16 inputs, fp32
- * accumulation, bf16 output. */
+ * accumulation, bf16 output.  The ids of a token need not differ: each slot is a row of its expert. */
 int moe_ffn_fwd(moe_ctx* ctx, const uint16_t* x, const int32_t* topk_ids, const float* topk_w,
                 const uint16_t* W_gate_up, const uint16_t* W_down, uint16_t* out, int32_t T,
                 void* stream);
