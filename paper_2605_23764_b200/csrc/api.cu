@@ -337,9 +337,10 @@ GemmArgs base_args(const moe_ctx* c) {
 }
 
 // GMM1 + SwiGLU (+ routing weight): A = w * silu(Xp.Wg^T) * (Xp.Wu^T)
-GemmArgs args_gate_up(const moe_ctx* c) {
+GemmArgs args_gate_up(const moe_ctx* c, int T) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
+  plan_ring(GEMM_GATE_UP, T, g);
   memcpy(g.tmTok, c->tk_Xp, sizeof g.tmTok);
   g.tmB = c->tm_W1_gu;
   g.n_tiles_n = (s.F + 127) / 128;
@@ -352,9 +353,10 @@ GemmArgs args_gate_up(const moe_ctx* c) {
   return g;
 }
 // GMM2: Y = A . W_down^T
-GemmArgs args_down(const moe_ctx* c) {
+GemmArgs args_down(const moe_ctx* c, int T) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
+  plan_ring(GEMM_DOWN, T, g);
   memcpy(g.tmTok, c->tk_A, sizeof g.tmTok);
   g.tmB = c->tm_W2_k128;  // each CTA of a pair loads 128 of the tile's 256 rows
   g.n_tiles_n = (s.d + 255) / 256;
@@ -365,10 +367,11 @@ GemmArgs args_down(const moe_ctx* c) {
   return g;
 }
 // act_grad + SwiGLU_grad (+ routing-weight gradient partials)
-GemmArgs args_act_grad(const moe_ctx* c, bool want_dw) {
+GemmArgs args_act_grad(const moe_ctx* c, int T, bool want_dw) {
   const moe_shape& s = c->shape;
   const WsPlan& p = c->plan;
   GemmArgs g = base_args(c);
+  plan_ring(GEMM_ACT_GRAD, T, g);
   memcpy(g.tmTok, c->tk_dOutp, sizeof g.tmTok);
   g.tmB = c->tm_W2_mn;
   g.n_tiles_n = p.ntn_act;
@@ -396,9 +399,10 @@ GemmArgs args_wgrad_down(const moe_ctx* c) {
   return g;
 }
 // gate_grad: dXp = dH . W_gate_up[e]   (the forward's Y is dead by now: its buffer receives dXp)
-GemmArgs args_gate_grad(const moe_ctx* c) {
+GemmArgs args_gate_grad(const moe_ctx* c, int T) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
+  plan_ring(GEMM_GATE_GRAD, T, g);
   memcpy(g.tmTok, c->tk_dH, sizeof g.tmTok);
   g.tmB = c->tm_W1_mn;
   g.n_tiles_n = (s.d + 255) / 256;
@@ -630,11 +634,11 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     }
     {
       Phase ph(c, MOE_PHASE_GEMM_GATE_UP, st);
-      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_GATE_UP, args_gate_up(c), c->num_sms, st, &c->launches));
+      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_GATE_UP, args_gate_up(c, T), c->num_sms, st, &c->launches));
     }
     {
       Phase ph(c, MOE_PHASE_GEMM_DOWN, st);
-      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_DOWN, args_down(c), c->num_sms, st, &c->launches));
+      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_DOWN, args_down(c, T), c->num_sms, st, &c->launches));
     }
     {
       Phase ph(c, MOE_PHASE_COMBINE, st);
@@ -644,8 +648,8 @@ int run_fwd(moe_ctx* c, const uint16_t* x, const int32_t* ids, const float* w, c
     // one persistent launch: gather, GMM1+SwiGLU, GMM2 and combine tiles ordered by event counters
     FusedArgs fa = fused_base(c, false, T);
     fa.cp = chain_params(c, false, T, false);
-    fa.op[0] = args_gate_up(c);
-    fa.op[1] = args_down(c);
+    fa.op[0] = args_gate_up(c, T);
+    fa.op[1] = args_down(c, T);
     fa.gather_src = x;
     fa.gather_dst = c->at<uint16_t>(p.Xp);
     fa.topk_w = w;
@@ -690,7 +694,7 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     }
     {
       Phase ph(c, MOE_PHASE_ACT_GRAD, st);
-      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_ACT_GRAD, args_act_grad(c, d_w != nullptr), c->num_sms, st, &c->launches));
+      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_ACT_GRAD, args_act_grad(c, T, d_w != nullptr), c->num_sms, st, &c->launches));
     }
     if (d_w) {
       Phase ph(c, MOE_PHASE_DW_REDUCE, st);
@@ -703,7 +707,7 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
     }
     {
       Phase ph(c, MOE_PHASE_GATE_GRAD, st);
-      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_GATE_GRAD, args_gate_grad(c), c->num_sms, st, &c->launches));
+      MOE_CUDA(LAUNCH_GEMM_SERIAL(GEMM_GATE_GRAD, args_gate_grad(c, T), c->num_sms, st, &c->launches));
     }
     {  // backward Combine: before the last weight gradient, which does not need dXp, so that with
        // host buffers the copy of dx leaves on the copy-out stream while that GEMM runs
@@ -723,9 +727,9 @@ int run_bwd(moe_ctx* c, const uint16_t* dout, const uint16_t* W1, const uint16_t
   } else {
     FusedArgs fa = fused_base(c, true, T);
     fa.cp = chain_params(c, true, T, d_w != nullptr);
-    fa.op[0] = args_act_grad(c, d_w != nullptr);
+    fa.op[0] = args_act_grad(c, T, d_w != nullptr);
     fa.op[1] = args_wgrad_down(c);
-    fa.op[2] = args_gate_grad(c);
+    fa.op[2] = args_gate_grad(c, T);
     fa.op[3] = args_wgrad_gate_up(c);
     fa.gather_src = dout;
     fa.gather_dst = c->at<uint16_t>(p.dOutp);

@@ -417,7 +417,7 @@ __device__ __forceinline__ ChainDeps phase_deps(const FusedArgs& fa, int phase, 
 
 // ---------------------------------------------------------------- one item, by role
 template <bool BWD>
-__device__ __forceinline__ bool load_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool load_item(const FusedArgs& fa, bool full, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                           LoaderState& ls, bool second_warp, int rank, int lane, const WaitCtl& wc,
                                           const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
@@ -430,14 +430,14 @@ __device__ __forceinline__ bool load_item(const FusedArgs& fa, const WorkDesc& w
     return wgrad_load_strip(fa.op[phase], smem, bars, ls, second_warp, rank, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
-    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-    return swap_load_item<GEMM_DOWN>(fa.op[1], smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+    return swap_load_item<GEMM_DOWN>(fa.op[1], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
 }
 template <bool BWD>
-__device__ __forceinline__ bool issue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool issue_item(const FusedArgs& fa, bool full, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                            uint32_t tmem_base, IssuerState& is, const WaitCtl& wc,
                                            const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
@@ -445,11 +445,11 @@ __device__ __forceinline__ bool issue_item(const FusedArgs& fa, const WorkDesc& 
     return wgrad_issue_strip(fa.op[phase], smem, bars, tmem_base, is, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
-    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], smem, bars, tmem_base, is, wk, t, wc, dep);
-    return swap_issue_item<GEMM_DOWN>(fa.op[1], smem, bars, tmem_base, is, wk, t, wc, dep);
+    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], full, smem, bars, tmem_base, is, wk, t, wc, dep);
+    return swap_issue_item<GEMM_DOWN>(fa.op[1], full, smem, bars, tmem_base, is, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, tmem_base, is, wk, t, wc, dep);
-  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, tmem_base, is, wk, t, wc, dep);
+  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], full, smem, bars, tmem_base, is, wk, t, wc, dep);
+  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], full, smem, bars, tmem_base, is, wk, t, wc, dep);
 }
 template <bool BWD>
 __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
@@ -561,6 +561,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
     }
   } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
+    const bool full = wants_full_ring(fa.op[0]);
     LoaderState ls;
     IssuerState is;
     EpiState es;
@@ -579,7 +580,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         if (warp == 0 || warp == 6) {
           if (!loader_enter_phase(bars, ls, phase, wc)) break;
         } else if (warp == 1) {
-          is.head = is.a_s = 0;
+          is.s = is.a_s = 0;
         } else {
           int go = 1;
           if (lane == 0) {
@@ -591,9 +592,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         }
       }
       if (warp == 0 || warp == 6)
-        ok = load_item<BWD>(fa, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
+        ok = load_item<BWD>(fa, full, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
       else if (warp == 1)
-        ok = issue_item<BWD>(fa, wd, smem, bars, tmem_base, is, wc, dep);
+        ok = issue_item<BWD>(fa, full, wd, smem, bars, tmem_base, is, wc, dep);
       else
         ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, wc, dep);
     }

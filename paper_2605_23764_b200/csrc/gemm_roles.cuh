@@ -17,7 +17,7 @@ namespace moe {
 
 constexpr int WG_A_SLOTS = 5;    // weight gradients: 16 KB slots of the strip's A operand
 constexpr int WG_B_STAGES = 7;   // weight gradients: 16 KB stages of the streamed B operand
-constexpr int MAX_STAGES = 12;   // stages in flight at most, a pair of barriers each
+constexpr int MAX_STAGES = 12;   // row-space operators: see plan_ring
 constexpr size_t WGRAD_STAGING_AT = (size_t)WG_A_SLOTS * A_STAGE_BYTES + (size_t)WG_B_STAGES * HALF_B_BYTES;   // behind both
 
 // Warps of a GEMM CTA: 0 weight loader, 1 MMA issuer, 2-5 and 8-11 epilogue, 6 token loader, 7 left to the kernel (scheduler).
@@ -39,20 +39,14 @@ struct __align__(8) PipeBarriers {
   int pad;
 };
 
-// Pipeline state of a role, carried from item to item (the barriers persist).  A stage is a pair of barriers, taken in
-// rotation, and as many bytes of the operand ring as its item needs, behind the stage before or, if the ring's end is too near,
-// at its bottom (ring_place): loaders and issuer find the same place without a word between them.
+// Pipeline state of a role, carried from item to item (the barriers persist).  The parity to wait for is kept per
+// stage, so operators with rings of different depth can follow one another in one launch (the ring position
+// restarts at 0 at such a boundary, where every stage has been consumed).
 struct LoaderState {
-  uint32_t s = 0, tail = 0;      // barriers of the next stage and of the oldest one that has not been seen empty
-  uint32_t head = 0, start = 0;  // first byte behind the newest stage; lane i: where the stage with barriers i starts
-  uint32_t empty_par = 0;        // parity of the next completion, by barrier
-  int held = 0;                  // stages from tail on
-  uint32_t a_s = 0, a_ph = (1u << WG_A_SLOTS) - 1;
+  uint32_t s = 0, empty_par = (1u << MAX_STAGES) - 1, a_s = 0, a_ph = (1u << WG_A_SLOTS) - 1;
   int guard = 0;   // != 0: the phase whose epilogue warps must all have arrived before a stage above WGRAD_STAGING_AT is loaded
 };
-struct IssuerState { uint32_t s = 0, head = 0, full_par = 0, a_s = 0, acc_it = 0; };
-__device__ __forceinline__ uint32_t next_stage(uint32_t s) { return s + 1 == (uint32_t)MAX_STAGES ? 0 : s + 1; }
-__device__ __forceinline__ uint32_t ring_place(uint32_t head, uint32_t bytes, uint32_t end) { return head + bytes <= end ? head : 0; }
+struct IssuerState { uint32_t s = 0, full_par = 0, a_s = 0, acc_it = 0; };
 struct EpiState { uint32_t acc_it = 0; };
 
 __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
@@ -104,38 +98,13 @@ __device__ __forceinline__ bool phase_wait(PipeBarriers* bars, int phase, const 
   return true;
 }
 
-// The oldest stage of a loader warp has been multiplied.  Every loader warp waits for every stage, in order: one that waited
-// only where it needs the room could fall two completions behind, where a parity no longer tells "done" from "not yet".
-__device__ __forceinline__ bool ring_release(PipeBarriers* bars, LoaderState& ls, const WaitCtl& wc, int t) {
-  if (!mbar_wait_warp(&bars->empty[ls.tail], (ls.empty_par >> ls.tail) & 1, wc, SITE_EMPTY, t, 50)) return false;
-  ls.empty_par ^= 1u << ls.tail;
-  ls.tail = next_stage(ls.tail);
-  --ls.held;
-  return true;
-}
-// Room for a stage of `bytes` in the ring [0, end): its barriers are ls.s (the caller moves on), its first byte *at.  Stages are
-// freed oldest first until none starts between the newest stage and the end of the new one.
-__device__ __forceinline__ bool ring_claim(PipeBarriers* bars, LoaderState& ls, uint32_t bytes, uint32_t end, int lane,
-                                           const WaitCtl& wc, int t, uint32_t* at) {
-  const uint32_t o = ring_place(ls.head, bytes, end);
-  while (ls.held) {
-    const uint32_t first = __shfl_sync(0xffffffffu, ls.start, ls.tail);
-    const bool over = o == ls.head ? first >= o && first < o + bytes : first >= ls.head || first < bytes;
-    if (!over && ls.held < MAX_STAGES) break;
-    if (!ring_release(bars, ls, wc, t)) return false;
-  }
-  if (lane == (int)ls.s) ls.start = o;
-  ls.head = o + bytes;
-  ++ls.held;
-  *at = o;
-  return true;
-}
 // A loader warp enters a phase with another ring: every stage of the old one has been multiplied (the commit that frees a
-// stage also covers the A slots of a weight gradient).
+// stage also covers the A slots of a weight gradient).  Stages the old ring did not use pass at once.
 __device__ __forceinline__ bool loader_enter_phase(PipeBarriers* bars, LoaderState& ls, int phase, const WaitCtl& wc) {
-  while (ls.held)
-    if (!ring_release(bars, ls, wc, phase)) return false;
-  ls.head = ls.a_s = 0;
+#pragma unroll 1
+  for (int s = 0; s < MAX_STAGES; ++s)
+    if (!mbar_wait_warp(&bars->empty[s], (ls.empty_par >> s) & 1, wc, SITE_EMPTY, phase, 50)) return false;
+  ls.s = ls.a_s = 0;
   ls.guard = phase;
   return true;
 }
@@ -216,47 +185,56 @@ struct ChainDeps {
 // =====================================================================================================
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
-// Shared memory of an operator, from the 1024-byte aligned base: the operand ring, and at the end of LAYOUT_BYTES the staging.
-// A stage is one k-block of an item: 16 KB of weights, then this CTA's half of its tokens, 18 KB for 32 tokens to 40 KB for a
-// merged item of 384.  Loads take 1.5-2 us under load, so what a CTA has in flight bounds its rate: with stages of one size,
-// that of the largest item, a tile of 128 tokens had 120 KB in flight and took as long as one of 256 (10 against 12 us for 32
-// k-blocks); now eight stages, 192 KB.
+// Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes], and at
+// the end of LAYOUT_BYTES the staging.  A call of T <= 256 tokens whose ids are distinct in each token has experts of at most T
+// rows: a tile needs n32(T) / 2 rows per CTA and nothing merges; beyond, a merged item (128 + 256) / 2.  What the token stages do
+// not need goes into more stages: with 32 tokens eleven, 198 KB of weights in flight instead of 80 -- a pass over few tokens is a
+// stream of weights from HBM.  Ids repeated in a token (a batch padded with id 0) give an expert more rows than there are tokens:
+// the layout leaves the rows of the largest expert in meta[7], and a launch that finds more there takes the full stages.  (Both
+// rings come from the host and a bit chooses: worked out in the kernel for every item, passes of short items took 1-3 % longer.)
 constexpr size_t PIPE_BARRIER_BYTES = 384;
 constexpr size_t TICKET_RING_BYTES = 640;   // of the persistent launch
 constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_RING_BYTES;
 __host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return EPI_WARPS * (size_t)sw_staging_bytes(mode); }
 __host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
-__host__ __device__ constexpr uint32_t ring_end(int mode) { return (uint32_t)staging_at((GemmMode)mode); }
-static_assert(ring_end(GEMM_GATE_UP) == ring_end(GEMM_DOWN), "the ring of the forward launch runs on from operator to operator");
+// The same for every role and item of a launch: the layout is complete before them.
+__device__ __forceinline__ bool wants_full_ring(const GemmArgs& a) { return uniform(a.meta[7] > a.ring_rows ? 1 : 0) != 0; }
+// does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
+__device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s) {
+  return (size_t)r.stages * W_STAGE_BYTES + (size_t)(s + 1) * r.tok_bytes > WGRAD_STAGING_AT ||
+         (size_t)(s + 1) * W_STAGE_BYTES > WGRAD_STAGING_AT;
+}
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
 // tokens.
 template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
+__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, bool full, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
                                                bool tok_warp, int rank, int lane, const SwapWork& wk, int t,
                                                const WaitCtl& wc, const DEP& dep) {
+  const GemmArgs::Ring ring = full ? a.full : a.ring;
+  const int stages = ring.stages, tokb = ring.tok_bytes;
+  uint8_t* sW = smem;                              // [stages][16 KB] weights
+  uint8_t* sT = smem + stages * W_STAGE_BYTES;     // [stages][tokb] tokens (this CTA's half)
   // with events: the tokens are there (acquired by the scheduler and handed on through the ticket ring, or by the caller);
   // what the producers wrote must be seen by the TMA loads
   if (DEP::kOn && tok_warp) fence_proxy_async_global();
   const int nkb = uniform(wk.a.nkb), e = uniform(wk.a.e), n0 = uniform(wk.a.n0);
   const int row_a = uniform(wk.a.row0), half_a = uniform(wk.a.ntok) >> 1;
   const int row_b = uniform(wk.b.row0), half_b = wk.merged ? uniform(wk.b.ntok) >> 1 : 0;
-  const uint32_t bytes = W_STAGE_BYTES + (half_a + half_b) * (BK * 2);
   for (int kb = 0; kb < nkb; ++kb) {
-    uint32_t at;
-    if (!ring_claim(bars, ls, bytes, ring_end(MODE), lane, wc, t, &at)) return false;
-    if (DEP::kOn && ls.guard && at + bytes > WGRAD_STAGING_AT) {   // a weight gradient's staging may still be in use there
+    if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, t, 50)) return false;
+    ls.empty_par ^= 1u << ls.s;
+    if (DEP::kOn && ls.guard && above_guard(ring, ls.s)) {   // a weight gradient's staging may still be in use there
       if (!uniform(lane == 0 ? (int)phase_wait(bars, ls.guard, wc) : 1)) return false;
       ls.guard = 0;
     }
-    uint8_t* const stage = smem + at;   // [16 KB of weights][tokens, this CTA's half]
     if (!tok_warp) {
-      load_weights_swap<MODE>(a, e, n0, kb, rank, stage, &bars->full[ls.s], 2 * (half_a + half_b));
+      load_weights_swap<MODE>(a, e, n0, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], 2 * (half_a + half_b));
     } else {
-      load_tokens_swap(a, row_a, half_a, kb, rank, stage + W_STAGE_BYTES, &bars->full[ls.s]);
+      load_tokens_swap(a, row_a, half_a, kb, rank, sT + ls.s * tokb, &bars->full[ls.s]);
       if (half_b)   // the second token tile, behind the first in the stage
-        load_tokens_swap(a, row_b, half_b, kb, rank, stage + W_STAGE_BYTES + half_a * (BK * 2), &bars->full[ls.s]);
+        load_tokens_swap(a, row_b, half_b, kb, rank, sT + ls.s * tokb + half_a * (BK * 2), &bars->full[ls.s]);
     }
-    ls.s = next_stage(ls.s);
+    if (++ls.s == (uint32_t)stages) ls.s = 0;
   }
   return true;
 }
@@ -264,11 +242,14 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, uint8_t* smem,
 // MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop with uniform control flow and operands; one elected
 // lane issues (common.cuh).
 template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
+__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, bool full, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
                                                 IssuerState& is, const SwapWork& wk, int t, const WaitCtl& wc,
                                                 const DEP& dep) {
+  const GemmArgs::Ring ring = full ? a.full : a.ring;
+  const uint32_t stages = ring.stages, t_step = ring.tok_bytes >> 4;
   const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
-  const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + W_STAGE_BYTES), 16);
+  const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + stages * W_STAGE_BYTES), 16);
+  uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * t_step;
   const int as = is.acc_it & 1;
   const int nkb = uniform(wk.a.nkb), ntok = uniform(wk.a.ntok), ntok_b = uniform(wk.merged ? wk.b.ntok : 0);
   if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
@@ -278,20 +259,20 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, uint8_t* smem
   const uint32_t d_tmem = tmem_base + as * BN, d_tmem_b = tmem_base + (as ^ 1) * BN;
   const uint32_t idesc = swap_idesc<MODE>(ntok), idesc_b = swap_idesc<MODE>(ntok_b ? ntok_b : TOK_GRAIN);
   const uint32_t t_off_b = (uint32_t)((ntok >> 1) * (BK * 2)) >> 4;
-  const uint32_t bytes = W_STAGE_BYTES + ((ntok + ntok_b) >> 1) * (BK * 2);
   uint64_t t0 = 0;
   for (int kb = 0; kb < nkb; ++kb) {
     if (!mbar_wait_warp(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, t)) return false;
     is.full_par ^= 1u << is.s;
     if (DEP::kOn && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
     tc_fence_after_sync();
-    const uint32_t at = ring_place(is.head, bytes, ring_end(MODE));
-    is.head = at + bytes;
-    const uint32_t w_lo = w_lo0 + (at >> 4), t_lo = t_lo0 + (at >> 4);
     mma_kblock_swap<MODE>(d_tmem, w_lo, t_lo, idesc, kb == 0);
     if (ntok_b) mma_kblock_swap<MODE>(d_tmem_b, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
     tc_commit_pair(&bars->empty[is.s]);   // frees the stage in both CTAs
-    is.s = next_stage(is.s);
+    if (++is.s == stages) {
+      is.s = 0; w_lo = w_lo0; t_lo = t_lo0;
+    } else {
+      w_lo += W_STAGE_BYTES >> 4; t_lo += t_step;
+    }
   }
   tc_commit_pair(&bars->tmem_full[as]);  // accumulator slices ready in both CTAs
   ++is.acc_it;
@@ -428,7 +409,7 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
                                                  bool b_warp, int rank, int lane, const Strip& st, int sp,
                                                  const WaitCtl& wc, const DEP& dep) {
   uint8_t* sA = smem;                                   // [WG_A_SLOTS][16 KB] A slots
-  uint8_t* sB = smem + WG_A_SLOTS * A_STAGE_BYTES;     // the operand ring: [WG_B_STAGES][16 KB] B stages
+  uint8_t* sB = smem + WG_A_SLOTS * A_STAGE_BYTES;     // [WG_B_STAGES][16 KB] B stages
   const int m0 = uniform(st.m0(rank)), row0 = uniform(st.row0), nkb = uniform(st.nkb);
   const bool resident = nkb <= A_RES_KB;
   if (DEP::kOn) fence_proxy_async_global();   // as in swap_load_item
@@ -437,8 +418,7 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
     const bool load_a = !resident || nb == nb0;
     for (int kb = 0; kb < nkb; ++kb) {
       const int slot = resident ? kb : (int)ls.a_s;
-      uint32_t at;
-      if (!ring_claim(bars, ls, HALF_B_BYTES, WG_B_STAGES * HALF_B_BYTES, lane, wc, sp, &at)) return false;
+      if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, sp, 50)) return false;
       if (!b_warp && load_a && !mbar_wait_warp(&bars->a_empty[slot], (ls.a_ph >> slot) & 1, wc, SITE_EMPTY, sp, 50)) return false;
       const int k0 = row0 + kb * BK;
       if (!b_warp) {
@@ -448,12 +428,13 @@ __device__ __forceinline__ bool wgrad_load_strip(const GemmArgs& a, uint8_t* sme
           tma_load_2d_pair(sA + slot * A_STAGE_BYTES + MN_BOX_BYTES, &a.tmA, m0 + 64, k0, &bars->full[ls.s]);
         }
       } else {
-        tma_load_2d_pair(sB + at, &a.tmB, nb * BN + 2 * rank * 64, k0, &bars->full[ls.s]);
-        tma_load_2d_pair(sB + at + MN_BOX_BYTES, &a.tmB, nb * BN + (2 * rank + 1) * 64, k0, &bars->full[ls.s]);
+        tma_load_2d_pair(sB + ls.s * HALF_B_BYTES, &a.tmB, nb * BN + 2 * rank * 64, k0, &bars->full[ls.s]);
+        tma_load_2d_pair(sB + ls.s * HALF_B_BYTES + MN_BOX_BYTES, &a.tmB, nb * BN + (2 * rank + 1) * 64, k0, &bars->full[ls.s]);
       }
+      ls.empty_par ^= 1u << ls.s;
       if (load_a) ls.a_ph ^= 1u << slot;
       if (!resident && ++ls.a_s == WG_A_SLOTS) ls.a_s = 0;
-      ls.s = next_stage(ls.s);
+      if (++ls.s == WG_B_STAGES) ls.s = 0;
     }
   }
   return true;
@@ -484,9 +465,7 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
       if (DEP::kOn && nb == nb0 && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
       tc_fence_after_sync();
       const int slot = resident ? kb : (int)is.a_s;
-      const uint32_t at = ring_place(is.head, HALF_B_BYTES, WG_B_STAGES * HALF_B_BYTES);
-      is.head = at + HALF_B_BYTES;
-      const uint32_t a_lo = a_lo0 + slot * (A_STAGE_BYTES >> 4), b_lo = b_lo0 + (at >> 4);
+      const uint32_t a_lo = a_lo0 + slot * (A_STAGE_BYTES >> 4), b_lo = b_lo0 + is.s * (HALF_B_BYTES >> 4);
       // the last k-block may hold fewer than 64 rows of the expert: the 16-row steps that would only multiply
       // zero padding are not issued
       const int steps = k16_steps_of(rows, kb);
@@ -499,7 +478,7 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
       tc_commit_pair(&bars->empty[is.s]);
       if (last_use) tc_commit_pair(&bars->a_empty[slot]);
       if (!resident && ++is.a_s == WG_A_SLOTS) is.a_s = 0;
-      is.s = next_stage(is.s);
+      if (++is.s == WG_B_STAGES) is.s = 0;
     }
     tc_commit_pair(&bars->tmem_full[as]);
     ++is.acc_it;

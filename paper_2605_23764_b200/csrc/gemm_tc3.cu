@@ -5,6 +5,8 @@
 //
 // Roles per CTA: warp 0 TMA producer of the weights, warp 1 MMA issuer (even CTA) and TMEM owner,
 // warps 2-5 and 8-11 epilogue, warp 6 TMA producer of the tokens.
+#include <limits.h>
+
 #include "gemm_roles.cuh"
 #include "launch_pairs.cuh"
 
@@ -47,13 +49,14 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   // Items pair, pair + npairs, ..; each role decodes item i + 1 before it works on item i (the decode's chain of
   // global loads then completes behind the item's work).
   const int total = total_swap_work<MODE>(a);
+  const bool full = wants_full_ring(a);
   SwapWork cur, next;
   if (pair < total) cur = decode_swap_work<MODE>(a, pair);
   if (warp == 0 || warp == 6) {
     LoaderState ls;
     for (int t = pair; t < total; t += npairs, cur = next) {
       if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-      if (!swap_load_item<MODE>(a, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
+      if (!swap_load_item<MODE>(a, full, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
     }
   } else if (warp == 1) {
     if (rank == 0) {
@@ -61,7 +64,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       bool ok = true;
       for (int t = pair; t < total && ok; t += npairs, cur = next) {
         if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-        ok = swap_issue_item<MODE>(a, smem, bars, tmem_base, is, cur, t, wc, dep);
+        ok = swap_issue_item<MODE>(a, full, smem, bars, tmem_base, is, cur, t, wc, dep);
       }
       if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
@@ -81,6 +84,20 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc_pair(tmem_base, TMEM_COLS);
+  }
+}
+
+void plan_ring(GemmMode mode, int T, GemmArgs& a) {
+  const bool merges = mode == GEMM_DOWN || mode == GEMM_GATE_GRAD || mode == GEMM_GATE_UP;   // gate+up: laid out like down
+  auto of = [&](int tok_bytes) {
+    const int stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + tok_bytes));
+    return GemmArgs::Ring{stages < MAX_STAGES ? stages : MAX_STAGES, tok_bytes};
+  };
+  a.full = a.ring = of((merges ? 3 : 2) * 64 * BK * 2);
+  a.ring_rows = INT_MAX;
+  if (T <= 2 * BLOCK_M) {
+    a.ring_rows = (T + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN;
+    a.ring = of(a.ring_rows / 2 * BK * 2);
   }
 }
 

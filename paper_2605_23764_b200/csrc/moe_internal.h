@@ -71,7 +71,7 @@ struct LayoutView {
   int* group_start;  // [Ep+1]  first 32-row group of each expert (an expert's rows up to a multiple of 32); NULL: not wanted
   int* group_row;    // [groups] first padded row of each group
   int* group_slot;   // [groups * 32] slot of each of the groups' rows, -1 for padding
-  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, num_groups, long experts, unused}
+  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, num_groups, long experts, rows of the largest expert}
   int* blk_hist;     // [nblk][Ep] per-block histograms, then per-block exclusive prefixes
   int* combine_order; // [T] persistent launch: tokens in the order in which their last row is produced (NULL: token order)
   int* tok_last;      // [T] 1 + largest padded row of each token (0: none); NULL when the combine order is not wanted
@@ -141,6 +141,11 @@ struct GemmArgs {
   int M;               // WGRAD: rows of dW per expert
   int b_rows_per_expert;  // rows of the B tensor map per expert slab
   int F;               // intermediate size (GATE_UP / ACT_GRAD epilogues)
+  // row-space modes: operand stages and the token bytes of a stage per CTA (gemm_roles.cuh, plan_ring) ..
+  struct Ring { int stages, tok_bytes; };
+  Ring ring;           // .. where no expert has more than ring_rows rows
+  Ring full;           // .. and where one has
+  int ring_rows;
   // epilogue tensors
   uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]; rows row_ld(..) apart
   uint16_t* out1;      // GATE_UP: H [rows][2F], NULL: the pre-activations are not kept
@@ -151,6 +156,8 @@ struct GemmArgs {
   uint64_t budget_ns;
 };
 
+// Shared-memory plan of a row-space operator for calls of T tokens: fills ring, full and ring_rows.
+void plan_ring(GemmMode mode, int T, GemmArgs& a);
 // ---- gemm_tc3.cu: the row-space operators with the tokens as accumulator COLUMNS (weights take the
 // 256 accumulator rows of a CTA pair), so a tile's MMA time follows the expert's real token count
 cudaError_t launch_gemm3(GemmMode mode, const GemmArgs& a, int num_sms, cudaStream_t s, int* launches);

@@ -137,8 +137,10 @@ __global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __
 }
 
 // Exclusive scans over the experts of a block of 1024 threads: s_counts[Ep] -> offsets of rows, M-blocks, pairs of
-// M-blocks, work items, 32-row groups and long experts, in shared memory (each Ep + 1 long) and in the layout's tables.
-constexpr int SCAN_Q = 6;   // rows of `totals`: by warp and behind them the block's
+// M-blocks, work items, 32-row groups and long experts, in shared memory (each Ep + 1 long) and in the layout's tables; and the
+// rows of the largest expert.
+constexpr int SCAN_Q = 6;
+constexpr int SCAN_ROWS = SCAN_Q + 1;   // of `totals`: by warp and behind them the block's; the last row holds maxima
 struct ExpertScan { int *counts, *off, *mb, *pr, *wi, *gr, *lg; };   // shared memory
 __host__ __device__ constexpr int expert_scan_ints(int Ep) { return 7 * Ep + 6; }
 __device__ __forceinline__ ExpertScan expert_scan_at(int* sm, int Ep) {
@@ -148,7 +150,7 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
                                              bool write = true) {
   constexpr int NQ = SCAN_Q;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int carry[NQ] = {0, 0, 0, 0, 0, 0};
+  int carry[NQ] = {0, 0, 0, 0, 0, 0}, largest = 0;
   for (int e0 = 0; e0 < Ep; e0 += 1024) {
     const int e = e0 + threadIdx.x;
     const int c = e < Ep ? sc.counts[e] : 0;
@@ -171,6 +173,8 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
 #pragma unroll
       for (int q = 0; q < NQ; ++q) totals[q][warp] = inc[q];
     }
+    const int most = __reduce_max_sync(0xffffffffu, c);
+    if (lane == 0) totals[NQ][warp] = most;
     __syncthreads();
     if (warp < NQ) {   // warp q: exclusive scan of quantity q's warp totals, the block's total behind them
       const int w = totals[warp][lane];
@@ -182,6 +186,9 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
       }
       totals[warp][lane] = wi - w;
       if (lane == 31) totals[warp][32] = wi;
+    } else if (warp == NQ) {
+      const int m = __reduce_max_sync(0xffffffffu, totals[NQ][lane]);
+      if (lane == 0) totals[NQ][32] = m;
     }
     __syncthreads();
     int ex[NQ];
@@ -204,6 +211,7 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
     }
 #pragma unroll
     for (int q = 0; q < NQ; ++q) carry[q] += totals[q][32];
+    largest = max(largest, totals[NQ][32]);
     __syncthreads();
   }
   if (threadIdx.x == 0) {
@@ -222,6 +230,7 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
     lv.meta[4] = carry[3];
     lv.meta[5] = carry[4];
     lv.meta[6] = carry[5];
+    lv.meta[7] = largest;
     if (lv.group_start) lv.group_start[Ep] = carry[4];
   }
   __syncthreads();
@@ -256,7 +265,7 @@ __device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, cons
 // (2) scans over experts; (3) M-block, pair and work-item -> expert tables.
 __global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int E, int Ep, LayoutView lv) {
   extern __shared__ int sm[];
-  __shared__ int totals[SCAN_Q][33];
+  __shared__ int totals[SCAN_ROWS][33];
   const ExpertScan sc = expert_scan_at(sm, Ep);
   int* part = sm + expert_scan_ints(Ep);   // [ranges][Ep]
   pdl_trigger();
@@ -454,7 +463,7 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
                                                           int Ep, LayoutView lv, int want_order, DevStatus* status,
                                                           int* __restrict__ zero, int nzero) {
   extern __shared__ int sm[];
-  __shared__ int totals[SCAN_Q][33];
+  __shared__ int totals[SCAN_ROWS][33];
   __shared__ int carry_s;
   const ExpertScan sc = expert_scan_at(sm, Ep);
   int* s_last = sm + expert_scan_ints(Ep);                       // [LAYOUT_ONE_SLOTS] 1 + padded row of the slot
@@ -543,7 +552,7 @@ __global__ void __launch_bounds__(1024)
     layout_cluster_kernel(const int* __restrict__ ids, int n, int T, int k, int kp, int E, int Ep, int G, LayoutView lv,
                           int want_order, DevStatus* status, int* __restrict__ zero, int nzero) {
   extern __shared__ int sm[];
-  __shared__ int totals[SCAN_Q][33];
+  __shared__ int totals[SCAN_ROWS][33];
   __shared__ int carry_s;
   const ExpertScan sc = expert_scan_at(sm, Ep);
   int* hist = sm + expert_scan_ints(Ep);        // [Ep] rows of this block's tokens, read by the other blocks

@@ -61,19 +61,6 @@ def test_counts_on_tile_edges(d, F, serial):
     layer.close()
 
 
-@pytest.mark.parametrize("serial", [False, True])
-def test_operand_ring_over_tiles_of_all_sizes(serial):
-    """Reductions of ten and eighteen k-blocks: the operand ring, whose stages are as large as their tile, goes round several
-    times within an item and changes from tile to tile -- 18 KB (one token) to 40 KB (merged tiles)."""
-    counts = [1, 300, 64, 257, 0, 33, 320, 160, 31, 256, 96, 640, 5]
-    E, T, d, F = len(counts), sum(counts), 1096, 584
-    g = torch.Generator().manual_seed(31)
-    ids = torch.from_numpy(np.repeat(np.arange(E), counts).astype(np.int32))
-    ids = ids[torch.randperm(T, generator=g)].reshape(T, 1).contiguous().cuda()
-    w = (torch.rand(T, 1, generator=g) + 0.25).float().cuda()
-    _check_against_oracle(T, d, E, 1, F, ids, w, 32, serial)
-
-
 def _check_against_oracle(T, d, E, k, F, ids, w, seed, serial):
     g = torch.Generator().manual_seed(seed)
     x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
