@@ -340,30 +340,32 @@ GemmArgs base_args(const moe_ctx* c) {
 GemmArgs args_gate_up(const moe_ctx* c, int T) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
-  plan_ring(GEMM_GATE_UP, T, g);
   memcpy(g.tmTok, c->tk_Xp, sizeof g.tmTok);
   g.tmB = c->tm_W1_gu;
   g.n_tiles_n = (s.F + 127) / 128;
   g.K = s.d;
+  g.merges = phase_merges(g.K);
   g.N = s.F;
   g.b_rows_per_expert = 2 * s.F;
   g.out0 = c->at<uint16_t>(c->plan.A);
   g.out1 = c->train() ? c->at<uint16_t>(c->plan.H) : nullptr;
   g.prow_w = c->at<float>(c->plan.prow_w);
+  plan_ring(GEMM_GATE_UP, T, g);
   return g;
 }
 // GMM2: Y = A . W_down^T
 GemmArgs args_down(const moe_ctx* c, int T) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
-  plan_ring(GEMM_DOWN, T, g);
   memcpy(g.tmTok, c->tk_A, sizeof g.tmTok);
   g.tmB = c->tm_W2_k128;  // each CTA of a pair loads 128 of the tile's 256 rows
   g.n_tiles_n = (s.d + 255) / 256;
   g.K = s.F;
+  g.merges = 1;
   g.N = s.d;
   g.b_rows_per_expert = s.d;
   g.out0 = c->at<uint16_t>(c->plan.Y);
+  plan_ring(GEMM_DOWN, T, g);
   return g;
 }
 // act_grad + SwiGLU_grad (+ routing-weight gradient partials)
@@ -371,17 +373,18 @@ GemmArgs args_act_grad(const moe_ctx* c, int T, bool want_dw) {
   const moe_shape& s = c->shape;
   const WsPlan& p = c->plan;
   GemmArgs g = base_args(c);
-  plan_ring(GEMM_ACT_GRAD, T, g);
   memcpy(g.tmTok, c->tk_dOutp, sizeof g.tmTok);
   g.tmB = c->tm_W2_mn;
   g.n_tiles_n = p.ntn_act;
   g.K = s.d;
+  g.merges = phase_merges(g.K);
   g.N = s.F;
   g.b_rows_per_expert = s.d;
   g.out0 = c->at<uint16_t>(p.dH);
   g.in0 = c->at<uint16_t>(p.H);
   g.prow_w = c->at<float>(p.prow_w);
   g.dw_partial = want_dw ? c->at<float>(p.dw_partial) : nullptr;
+  plan_ring(GEMM_ACT_GRAD, T, g);
   return g;
 }
 // w2_grad: dW_down[e][c][f] = sum_rows dOutp[r][c] * A[r][f]   (shares dOutp with act_grad)
@@ -402,14 +405,15 @@ GemmArgs args_wgrad_down(const moe_ctx* c) {
 GemmArgs args_gate_grad(const moe_ctx* c, int T) {
   const moe_shape& s = c->shape;
   GemmArgs g = base_args(c);
-  plan_ring(GEMM_GATE_GRAD, T, g);
   memcpy(g.tmTok, c->tk_dH, sizeof g.tmTok);
   g.tmB = c->tm_W1_mn;
   g.n_tiles_n = (s.d + 255) / 256;
   g.K = 2 * s.F;
+  g.merges = 1;
   g.N = s.d;
   g.b_rows_per_expert = 2 * s.F;
   g.out0 = c->at<uint16_t>(c->plan.Y);
+  plan_ring(GEMM_GATE_GRAD, T, g);
   return g;
 }
 // w1_grad: dW_gate_up[e][n][c] = sum_rows dH[r][n] * Xp[r][c]   (shares dH with gate_grad)
@@ -452,6 +456,7 @@ ChainParams make_chain(bool bwd, int T, int Ep, int k, int n_shared, int d, int 
     cp.n_phases = 2;
     cp.ntn[0] = (F + 127) / 128;                 // gate+up: 128 features (gate and up) per pair tile
     cp.ntn[1] = (d + 255) / 256;                 // down
+    cp.merges[0] = phase_merges(d);
     cp.merges[1] = 1;
   } else {
     cp.n_phases = 4;
@@ -459,6 +464,7 @@ ChainParams make_chain(bool bwd, int T, int Ep, int k, int n_shared, int d, int 
     cp.ntn[1] = (F + 255) / 256;                 // w2_grad: column tiles per strip
     cp.strips[1] = (d + 255) / 256;
     cp.ntn[2] = (d + 255) / 256;                 // gate_grad
+    cp.merges[0] = phase_merges(d);
     cp.merges[2] = 1;
     cp.ntn[3] = (d + 255) / 256;                 // w1_grad
     cp.strips[3] = (2 * F + 255) / 256;

@@ -365,22 +365,21 @@ __device__ __forceinline__ PhaseTable make_phase_table(const FusedArgs& fa) {
   PhaseTable pt;
   pt.start[0] = 0;
   if (!BWD) {
-    pt.start[1] = total_swap_work<GEMM_GATE_UP>(fa.op[0]);
-    pt.start[2] = pt.start[1] + total_swap_work<GEMM_DOWN>(fa.op[1]);
+    pt.start[1] = total_swap_work(fa.op[0]);
+    pt.start[2] = pt.start[1] + total_swap_work(fa.op[1]);
     pt.start[3] = pt.start[4] = pt.start[2];
   } else {
-    pt.start[1] = total_swap_work<GEMM_ACT_GRAD>(fa.op[0]);
+    pt.start[1] = total_swap_work(fa.op[0]);
     pt.start[2] = pt.start[1] + wgrad_strips(fa.op[1]);
-    pt.start[3] = pt.start[2] + total_swap_work<GEMM_GATE_GRAD>(fa.op[2]);
+    pt.start[3] = pt.start[2] + total_swap_work(fa.op[2]);
     pt.start[4] = pt.start[3] + wgrad_strips(fa.op[3]);
   }
   return pt;
 }
 // Where each row-space phase's item list starts when there are shared experts (schedule.h, rotate_index): at the
 // first item of the first shared expert.  `first[p]` = 0: no rotation (no shared experts, or a weight-gradient phase).
-template <int MODE>
 __device__ __forceinline__ int swap_first_item(const GemmArgs& a, int first_shared) {
-  return (swap_merges<MODE>() ? a.work_start : a.pair_start)[first_shared] * a.n_tiles_n;
+  return (a.merges ? a.work_start : a.pair_start)[first_shared] * a.n_tiles_n;
 }
 template <bool BWD>
 __device__ __forceinline__ PhaseTable make_rotation_table(const FusedArgs& fa) {
@@ -389,11 +388,11 @@ __device__ __forceinline__ PhaseTable make_rotation_table(const FusedArgs& fa) {
   const int S = fa.cp.kp - fa.cp.k, E = fa.cp.Ep - S;
   if (S == 0) return r;
   if (!BWD) {
-    r.start[0] = swap_first_item<GEMM_GATE_UP>(fa.op[0], E);
-    r.start[1] = swap_first_item<GEMM_DOWN>(fa.op[1], E);
+    r.start[0] = swap_first_item(fa.op[0], E);
+    r.start[1] = swap_first_item(fa.op[1], E);
   } else {
-    r.start[0] = swap_first_item<GEMM_ACT_GRAD>(fa.op[0], E);
-    r.start[2] = swap_first_item<GEMM_GATE_GRAD>(fa.op[2], E);
+    r.start[0] = swap_first_item(fa.op[0], E);
+    r.start[2] = swap_first_item(fa.op[2], E);
   }
   return r;
 }

@@ -26,16 +26,25 @@ constexpr int GEMM_ROLE_WARPS = 12;
 __device__ __forceinline__ bool is_epilogue_warp(int warp) { return (warp >= 2 && warp < 6) || (warp >= 8 && warp < 12); }
 __device__ __forceinline__ int epilogue_index(int warp) { return (warp & 3) + (warp >= 8 ? 4 : 0); }
 
+// Accumulators.  An item of up to two tiles has 64 to 384 TMEM columns; items take the two ends of the 512 columns in turn, so
+// that an item's products run beside the epilogue of the one before.  Where the two overlap -- merged items -- the item begins
+// when the tile in the middle is drained: that tile is the larger one, and its epilogue comes first.  Four slots: end, tile.
+constexpr int ACC_SLOTS = 4;
+// first column of tile `part` (0: the one towards the middle) of an item of n0 + n1 columns
+__device__ __forceinline__ int acc_column(int end, int part, int n0, int n1) {
+  return part == 0 ? (end ? TMEM_COLS - n0 - n1 : n1) : (end ? TMEM_COLS - n1 : 0);
+}
+
 struct __align__(8) PipeBarriers {
   uint64_t full[MAX_STAGES];      // used in the even CTA: bytes of both CTAs' loads of the stage
   uint64_t empty[MAX_STAGES];     // in each CTA: the stage's MMAs are complete
   uint64_t a_empty[WG_A_SLOTS];  // weight gradients, in each CTA: every MMA that reads the A slot's content is complete
-  uint64_t tmem_full[2];          // in each CTA: accumulator ready
-  uint64_t tmem_empty[2];         // used in the even CTA: the epilogue warps of the pair have drained it
+  uint64_t tmem_full[ACC_SLOTS];  // in each CTA: accumulator ready
+  uint64_t tmem_empty[ACC_SLOTS]; // used in the even CTA: the epilogue warps of the pair have drained it
   uint64_t drain;
   uint32_t tmem_base;
   int epi_phase[EPI_WARPS];       // in each CTA: the phase each epilogue warp is in (its stores of earlier phases have read shared memory)
-  int epi_done[2];                // in each CTA, per accumulator: epilogue warps whose stores of the tile are under way
+  int epi_done[ACC_SLOTS];        // in each CTA, per accumulator: epilogue warps whose stores of the tile are under way
   int pad;
 };
 
@@ -46,8 +55,13 @@ struct LoaderState {
   uint32_t s = 0, empty_par = (1u << MAX_STAGES) - 1, a_s = 0, a_ph = (1u << WG_A_SLOTS) - 1;
   int guard = 0;   // != 0: the phase whose epilogue warps must all have arrived before a stage above WGRAD_STAGING_AT is loaded
 };
-struct IssuerState { uint32_t s = 0, full_par = 0, a_s = 0, acc_it = 0; };
-struct EpiState { uint32_t acc_it = 0; };
+struct IssuerState {
+  uint32_t s = 0, full_par = 0, a_s = 0;
+  int end = 0;                    // of the TMEM columns, for the next item
+  uint32_t busy = 0, acc_par = 0; // by slot: not seen drained; parity of the next drain
+  int before_n0 = 0, before_n = 0;   // columns of the item before: of its first tile, of both
+};
+struct EpiState { int end = 0; uint32_t full_par = 0; };
 
 __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
   for (int s = 0; s < MAX_STAGES; ++s) {
@@ -55,13 +69,13 @@ __device__ __forceinline__ void pipe_init(PipeBarriers* bars) {   // one thread
     mbar_init(&bars->empty[s], 1);
   }
   for (int s = 0; s < WG_A_SLOTS; ++s) mbar_init(&bars->a_empty[s], 1);
-  for (int s = 0; s < 2; ++s) {
+  for (int s = 0; s < ACC_SLOTS; ++s) {
     mbar_init(&bars->tmem_full[s], 1);
     mbar_init(&bars->tmem_empty[s], 2 * EPI_WARPS);
+    bars->epi_done[s] = 0;
   }
   mbar_init(&bars->drain, 1);
   for (int w = 0; w < EPI_WARPS; ++w) bars->epi_phase[w] = 0;
-  bars->epi_done[0] = bars->epi_done[1] = 0;
 }
 // Phase boundaries of the persistent launch.  The shared memory of a phase (operand ring, staging) is carved per operator.
 // Operand rings start at the bottom, staging lies at the top (staging_at), so the loads of a phase start as soon as the
@@ -239,6 +253,27 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, bool full, uin
   return true;
 }
 
+// The issuer takes columns for an item of n0 (+ n1) columns: what they overlap has been drained when this returns.  Its slots are
+// 2 * is.end and, for the second tile, the one behind; the caller flips is.end.
+__device__ __forceinline__ bool acc_claim(PipeBarriers* bars, IssuerState& is, int n0, int n1, const WaitCtl& wc, int t) {
+  const int over = is.before_n + n0 + n1 - TMEM_COLS, other = 2 * (is.end ^ 1);
+  uint32_t need = 3u << (2 * is.end);   // the item before the last, at the same end
+  if (over > 0) need |= (over > is.before_n0 ? 3u : 1u) << other;
+  need &= is.busy;
+#pragma unroll 1
+  while (need) {
+    const int slot = __ffs(need) - 1;
+    if (!mbar_wait_warp(&bars->tmem_empty[slot], (is.acc_par >> slot) & 1, wc, SITE_TMEM_EMPTY, t)) return false;
+    is.acc_par ^= 1u << slot;
+    is.busy &= ~(1u << slot);
+    need &= need - 1;
+  }
+  is.busy |= (n1 ? 3u : 1u) << (2 * is.end);
+  is.before_n0 = n0;
+  is.before_n = n0 + n1;
+  return true;
+}
+
 // MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop with uniform control flow and operands; one elected
 // lane issues (common.cuh).
 template <int MODE, class DEP>
@@ -250,13 +285,13 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, bool full, ui
   const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
   const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + stages * W_STAGE_BYTES), 16);
   uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * t_step;
-  const int as = is.acc_it & 1;
   const int nkb = uniform(wk.a.nkb), ntok = uniform(wk.a.ntok), ntok_b = uniform(wk.merged ? wk.b.ntok : 0);
-  if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
-  if (ntok_b &&   // the second token tile accumulates in the other buffer
-      !mbar_wait_warp(&bars->tmem_empty[as ^ 1], (((is.acc_it + 1) >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, t)) return false;
+  // a merged item's second tile is the larger one: the first in the accumulators
+  const int n0 = ntok_b ? ntok_b : ntok, n1 = ntok_b ? ntok : 0;
+  if (!acc_claim(bars, is, n0, n1, wc, t)) return false;
   tc_fence_after_sync();
-  const uint32_t d_tmem = tmem_base + as * BN, d_tmem_b = tmem_base + (as ^ 1) * BN;
+  const uint32_t d_first = uniform(tmem_base + acc_column(is.end, 0, n0, n1));
+  const uint32_t d_tmem = uniform(ntok_b ? tmem_base + acc_column(is.end, 1, n0, n1) : d_first);
   const uint32_t idesc = swap_idesc<MODE>(ntok), idesc_b = swap_idesc<MODE>(ntok_b ? ntok_b : TOK_GRAIN);
   const uint32_t t_off_b = (uint32_t)((ntok >> 1) * (BK * 2)) >> 4;
   uint64_t t0 = 0;
@@ -266,7 +301,7 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, bool full, ui
     if (DEP::kOn && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
     tc_fence_after_sync();
     mma_kblock_swap<MODE>(d_tmem, w_lo, t_lo, idesc, kb == 0);
-    if (ntok_b) mma_kblock_swap<MODE>(d_tmem_b, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
+    if (ntok_b) mma_kblock_swap<MODE>(d_first, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
     tc_commit_pair(&bars->empty[is.s]);   // frees the stage in both CTAs
     if (++is.s == stages) {
       is.s = 0; w_lo = w_lo0; t_lo = t_lo0;
@@ -274,12 +309,9 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, bool full, ui
       w_lo += W_STAGE_BYTES >> 4; t_lo += t_step;
     }
   }
-  tc_commit_pair(&bars->tmem_full[as]);  // accumulator slices ready in both CTAs
-  ++is.acc_it;
-  if (ntok_b) {
-    tc_commit_pair(&bars->tmem_full[as ^ 1]);
-    ++is.acc_it;
-  }
+  tc_commit_pair(&bars->tmem_full[2 * is.end]);  // accumulator slices ready in both CTAs
+  if (ntok_b) tc_commit_pair(&bars->tmem_full[2 * is.end + 1]);
+  is.end ^= 1;
   if (DEP::kOn && dep.tracing() && (threadIdx.x & 31) == 0) dep.trace(TR_MMA, t, t0, t0, globaltimer_ns());
   return true;
 }
@@ -293,24 +325,25 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
                                                    uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                    const SwapWork& wk, int t, const WaitCtl& wc, const DEP& dep) {
   uint8_t* staging = smem + staging_at((GemmMode)MODE) + ew * sw_staging_bytes((GemmMode)MODE);
-  for (int part = 0; part < (wk.merged ? 2 : 1); ++part) {   // a merged item is two consecutive tiles here
-    const SwapTile& st = part ? wk.b : wk.a;
-    const int as = es.acc_it & 1;
+  const int n0 = wk.merged ? wk.b.ntok : wk.a.ntok, n1 = wk.merged ? wk.a.ntok : 0;
+  for (int part = 0; part < (wk.merged ? 2 : 1); ++part) {   // a merged item is two tiles here, the larger one first
+    const SwapTile& st = part == 0 && wk.merged ? wk.b : wk.a;
+    const int as = 2 * es.end + part;
     uint64_t t0 = 0;
     auto ready = [&]() {
-      if (!mbar_wait_warp(&bars->tmem_full[as], (es.acc_it >> 1) & 1, wc, SITE_TMEM_FULL, t, 200)) return false;
+      if (!mbar_wait_warp(&bars->tmem_full[as], (es.full_par >> as) & 1, wc, SITE_TMEM_FULL, t, 200)) return false;
       if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) t0 = globaltimer_ns();
       __syncwarp();
       tc_fence_after_sync();
       return true;
     };
-    if (!epilogue_swap<MODE>(a, st, tmem_base + as * BN, rank, ew, lane, staging, ready)) return false;
+    if (!epilogue_swap<MODE>(a, st, tmem_base + acc_column(es.end, part, n0, n1), rank, ew, lane, staging, ready)) return false;
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) {
       bool last = false;
       if (DEP::kOn) {
-        // counted before the accumulator is given back: the tile after the next, which uses this counter again, follows
+        // counted before the accumulator is given back: the next tile of the slot, which uses this counter again, follows
         int before;
         asm volatile("atom.acq_rel.cta.shared::cta.add.s32 %0, [%1], 1;" : "=r"(before) : "r"(smem_u32(&bars->epi_done[as])) : "memory");
         last = before == EPI_WARPS - 1;
@@ -322,9 +355,10 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
         if (ew == 0 && dep.tracing()) dep.trace(TR_EPI, t, t0, t0, globaltimer_ns());
       }
     }
-    ++es.acc_it;
+    es.full_par ^= 1u << as;
     __syncwarp();
   }
+  es.end ^= 1;
   return true;
 }
 
@@ -454,10 +488,9 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
   uint64_t t0 = 0;
   const int nb0 = uniform(st.nb0), nb1 = uniform(st.nb1);
   for (int nb = nb0; nb < nb1; ++nb) {
-    const int as = is.acc_it & 1;
-    if (!mbar_wait_warp(&bars->tmem_empty[as], ((is.acc_it >> 1) & 1) ^ 1, wc, SITE_TMEM_EMPTY, sp)) return false;
+    if (!acc_claim(bars, is, BN, 0, wc, sp)) return false;
     tc_fence_after_sync();
-    const uint32_t d_tmem = tmem_base + as * BN;
+    const uint32_t d_tmem = uniform(tmem_base + acc_column(is.end, 0, BN, 0));
     const bool last_use = !resident || nb == nb1 - 1;
     for (int kb = 0; kb < nkb; ++kb) {
       if (!mbar_wait_warp(&bars->full[is.s], (is.full_par >> is.s) & 1, wc, SITE_FULL, sp)) return false;
@@ -480,8 +513,8 @@ __device__ __forceinline__ bool wgrad_issue_strip(const GemmArgs& a, uint8_t* sm
       if (!resident && ++is.a_s == WG_A_SLOTS) is.a_s = 0;
       if (++is.s == WG_B_STAGES) is.s = 0;
     }
-    tc_commit_pair(&bars->tmem_full[as]);
-    ++is.acc_it;
+    tc_commit_pair(&bars->tmem_full[2 * is.end]);
+    is.end ^= 1;
   }
   if (DEP::kOn && dep.tracing() && (threadIdx.x & 31) == 0) dep.trace(TR_MMA, sp, t0, t0, globaltimer_ns());
   return true;
@@ -504,14 +537,15 @@ __device__ __forceinline__ bool wgrad_epilogue_strip(const GemmArgs& a, uint8_t*
       if (!idle) epilogue_wgrad_tile(a, tl, 0, ew, lane, box);  // an expert without rows: zeros
       continue;
     }
-    const int as = es.acc_it & 1;
-    if (!mbar_wait(&bars->tmem_full[as], (es.acc_it >> 1) & 1, wc, SITE_TMEM_FULL, sp, 200)) { ok = false; break; }
+    const int as = 2 * es.end;
+    if (!mbar_wait(&bars->tmem_full[as], (es.full_par >> as) & 1, wc, SITE_TMEM_FULL, sp, 200)) { ok = false; break; }
     tc_fence_after_sync();
-    if (!idle) epilogue_wgrad_tile(a, tl, tmem_base + as * BN, ew, lane, box);
+    if (!idle) epilogue_wgrad_tile(a, tl, tmem_base + acc_column(es.end, 0, BN, 0), ew, lane, box);
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) mbar_arrive_leader(&bars->tmem_empty[as]);
-    ++es.acc_it;
+    es.full_par ^= 1u << as;
+    es.end ^= 1;
   }
   if (DEP::kOn && ew == 0 && lane == 0 && dep.tracing()) dep.trace(TR_EPI, sp, t0, t0, globaltimer_ns());
   return ok;

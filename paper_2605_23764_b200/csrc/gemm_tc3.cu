@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
 
   // Items pair, pair + npairs, ..; each role decodes item i + 1 before it works on item i (the decode's chain of
   // global loads then completes behind the item's work).
-  const int total = total_swap_work<MODE>(a);
+  const int total = total_swap_work(a);
   const bool full = wants_full_ring(a);
   SwapWork cur, next;
   if (pair < total) cur = decode_swap_work<MODE>(a, pair);
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
 }
 
 void plan_ring(GemmMode mode, int T, GemmArgs& a) {
-  const bool merges = mode == GEMM_DOWN || mode == GEMM_GATE_GRAD || mode == GEMM_GATE_UP;   // gate+up: laid out like down
+  const bool merges = a.merges || mode == GEMM_GATE_UP;   // gate+up: laid out like down
   auto of = [&](int tok_bytes) {
     const int stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + tok_bytes));
     return GemmArgs::Ring{stages < MAX_STAGES ? stages : MAX_STAGES, tok_bytes};

@@ -137,6 +137,7 @@ struct GemmArgs {
   int n_tiles_m;       // WGRAD only: tiles along M per expert
   int split;           // WGRAD only: ranges of column tiles per strip (schedule.h)
   int K;               // reduction length (row-space modes)
+  int merges;          // row-space modes: 1 if experts that can (expert_merges) have their last two token tiles under one k-loop
   int N;               // output columns (for masking); WGRAD: columns of dW
   int M;               // WGRAD: rows of dW per expert
   int b_rows_per_expert;  // rows of the B tensor map per expert slab

@@ -70,16 +70,23 @@ MOE_HD void balanced_unit(int mc, int u, int* first, int* count) {
 
 // Which experts merge their last two units in the phases that merge: an odd count of three or more M-blocks whose
 // last block is mostly padding (at most MERGE_TAIL_MAX rows).  Then the last unit (block + tail) is small, staging the
-// weights once for both units saves the larger half of the shared-memory traffic, and the epilogue that merging
-// exposes (both accumulators are in use) is short.  With a full last block (e.g. 384 rows) the exposed epilogue
-// costs more than the second weight pass: down was 5 % faster unmerged there and 6 % slower on 257..320-row experts.
+// weights once for both units saves the larger half of the shared-memory traffic, and what the next item waits for, the epilogue
+// of the larger of the two tiles (gemm_roles.cuh, acc_claim), is short.  With a full last block (e.g. 384 rows) that costs
+// as much as the second weight pass or more: down was 5 % faster unmerged there, 257..320-row experts 6 % slower.
 constexpr int MERGE_TAIL_MAX = 64;
+// Do gate+up and act_grad, whose reduction is K long, merge too?  128 + 160 tokens take 880 clocks a k-block as two tiles
+// (the loads of a small tile take longer than its products) and 595 as one item, so an item of 112 k-blocks is 18 us shorter; what
+// it exposes of gate+up's epilogue is 3 us, of act_grad's 10.  K = 7168, 128 experts of 256 rows: a training step 10260 -> 10015
+// us; K = 4096, skewed experts: forward 4920 -> 4780; K = 2048 (32 k-blocks), experts of up to 384 rows: a step 1830 -> 1870.
+constexpr int MERGE_MIN_K = 4096;
+MOE_HD int phase_merges(int K) { return K >= MERGE_MIN_K; }
 MOE_HD bool expert_merges(int rows, int mblocks) {
   return (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
 }
 
 // One work item of a row-space phase: a token tile (unit) of an expert and a column tile, or -- in the
-// phases that merge, for an expert that merges (expert_merges) -- its last two units under one k-loop.  `start[e]` = first unit (or first merged item) of expert e, `blk_expert[i]` =
+// phases that merge (down and gate_grad always, gate+up and act_grad by phase_merges), for an expert that merges
+// (expert_merges) -- its last two units under one k-loop.  `start[e]` = first unit (or first merged item) of expert e, `blk_expert[i]` =
 // expert of unit / item i (both from the layout kernels).
 struct SwapItem {
   int e, nb;            // expert, column tile

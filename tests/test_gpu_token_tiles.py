@@ -61,6 +61,20 @@ def test_counts_on_tile_edges(d, F, serial):
     layer.close()
 
 
+@pytest.mark.parametrize("d", [4088, 4096])   # both sides of the line from which gate+up and act_grad merge
+@pytest.mark.parametrize("serial", [False, True])
+def test_merged_tiles_in_every_operator(d, serial):
+    """Experts whose last two token tiles share a k-loop, of 257 to 320 rows and in a row of items: their accumulators take
+    turns at the two ends of the 512 columns and overlap; unmerged tiles of all sizes between them."""
+    counts = [257, 320, 300, 256, 290, 64, 320, 577, 320, 1, 384, 257]
+    E, T, F = len(counts), sum(counts), 264
+    g = torch.Generator().manual_seed(41)
+    ids = torch.from_numpy(np.repeat(np.arange(E), counts).astype(np.int32))
+    ids = ids[torch.randperm(T, generator=g)].reshape(T, 1).contiguous().cuda()
+    w = (torch.rand(T, 1, generator=g) + 0.25).float().cuda()
+    _check_against_oracle(T, d, E, 1, F, ids, w, 42, serial)
+
+
 def _check_against_oracle(T, d, E, k, F, ids, w, seed, serial):
     g = torch.Generator().manual_seed(seed)
     x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()

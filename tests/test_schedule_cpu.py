@@ -18,9 +18,10 @@ def _expected_items(counts, d, F, is_bwd):
     # an expert merges its last two units when its M-block count is odd, at least 3, and the last block holds <= 64 rows
     merged = units - ((mblocks % 2 == 1) & (mblocks >= 3) & (counts - (mblocks - 1) * 128 <= 64))
     Ep = len(counts)
+    first = merged if d >= 4096 else units   # gate+up and act_grad merge where their reduction is long
     if not is_bwd:
-        return int(units.sum()) * ((F + 127) // 128) + int(merged.sum()) * ((d + 255) // 256)
-    return (int(units.sum()) * ((F + 255) // 256) + Ep * ((d + 255) // 256) +
+        return int(first.sum()) * ((F + 127) // 128) + int(merged.sum()) * ((d + 255) // 256)
+    return (int(first.sum()) * ((F + 255) // 256) + Ep * ((d + 255) // 256) +
             int(merged.sum()) * ((d + 255) // 256) + Ep * ((2 * F + 255) // 256))
 
 
@@ -43,6 +44,14 @@ def test_schedule_is_sound(is_bwd, workers):
         rc, stats = binding.moe_debug_simulate_schedule(counts, T, 2, 0, d, F, is_bwd, *workers)
         assert rc == 0, (counts.tolist(), rc)
         assert stats[0] == _expected_items(counts, d, F, is_bwd)
+
+
+@pytest.mark.parametrize("is_bwd", [0, 1])
+@pytest.mark.parametrize("d", [4088, 4096, 7168])
+def test_first_operator_merges_where_its_reduction_is_long(is_bwd, d):
+    counts = np.array([300, 257, 320, 577, 321, 384, 0, 64])
+    rc, stats = binding.moe_debug_simulate_schedule(counts, 1111, 2, 0, d, 272, is_bwd, 74, 592)
+    assert rc == 0 and stats[0] == _expected_items(counts, d, 272, is_bwd)
 
 
 def test_balanced_units_cover_every_mblock_once():
