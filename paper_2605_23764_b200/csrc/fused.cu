@@ -416,7 +416,7 @@ __device__ __forceinline__ ChainDeps phase_deps(const FusedArgs& fa, int phase, 
 
 // ---------------------------------------------------------------- one item, by role
 template <bool BWD>
-__device__ __forceinline__ bool load_item(const FusedArgs& fa, bool full, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool load_item(const FusedArgs& fa, int ring_of, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                           LoaderState& ls, bool second_warp, int rank, int lane, const WaitCtl& wc,
                                           const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
@@ -429,14 +429,14 @@ __device__ __forceinline__ bool load_item(const FusedArgs& fa, bool full, const 
     return wgrad_load_strip(fa.op[phase], smem, bars, ls, second_warp, rank, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
-    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-    return swap_load_item<GEMM_DOWN>(fa.op[1], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+    return swap_load_item<GEMM_DOWN>(fa.op[1], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], full, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
 }
 template <bool BWD>
-__device__ __forceinline__ bool issue_item(const FusedArgs& fa, bool full, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool issue_item(const FusedArgs& fa, int ring_of, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                            uint32_t tmem_base, IssuerState& is, const WaitCtl& wc,
                                            const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
@@ -444,11 +444,11 @@ __device__ __forceinline__ bool issue_item(const FusedArgs& fa, bool full, const
     return wgrad_issue_strip(fa.op[phase], smem, bars, tmem_base, is, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
   if (!BWD) {
-    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], full, smem, bars, tmem_base, is, wk, t, wc, dep);
-    return swap_issue_item<GEMM_DOWN>(fa.op[1], full, smem, bars, tmem_base, is, wk, t, wc, dep);
+    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
+    return swap_issue_item<GEMM_DOWN>(fa.op[1], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
   }
-  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], full, smem, bars, tmem_base, is, wk, t, wc, dep);
-  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], full, smem, bars, tmem_base, is, wk, t, wc, dep);
+  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
+  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
 }
 template <bool BWD>
 __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
     }
   } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
-    const bool full = wants_full_ring(fa.op[0]);
+    const int ring_of = which_ring(fa.op[0]);
     LoaderState ls;
     IssuerState is;
     EpiState es;
@@ -591,9 +591,9 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         }
       }
       if (warp == 0 || warp == 6)
-        ok = load_item<BWD>(fa, full, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
+        ok = load_item<BWD>(fa, ring_of, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
       else if (warp == 1)
-        ok = issue_item<BWD>(fa, full, wd, smem, bars, tmem_base, is, wc, dep);
+        ok = issue_item<BWD>(fa, ring_of, wd, smem, bars, tmem_base, is, wc, dep);
       else
         ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, wc, dep);
     }

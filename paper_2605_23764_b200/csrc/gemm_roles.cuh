@@ -200,19 +200,24 @@ struct ChainDeps {
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
 // Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes], and at
-// the end of LAYOUT_BYTES the staging.  A call of T <= 256 tokens whose ids are distinct in each token has experts of at most T
-// rows: a tile needs n32(T) / 2 rows per CTA and nothing merges; beyond, a merged item (128 + 256) / 2.  What the token stages do
-// not need goes into more stages: with 32 tokens eleven, 198 KB of weights in flight instead of 80 -- a pass over few tokens is a
-// stream of weights from HBM.  Ids repeated in a token (a batch padded with id 0) give an expert more rows than there are tokens:
-// the layout leaves the rows of the largest expert in meta[7], and a launch that finds more there takes the full stages.  (Both
-// rings come from the host and a bit chooses: worked out in the kernel for every item, passes of short items took 1-3 % longer.)
+// the end of LAYOUT_BYTES the staging.  What the token stages do not need goes into more stages: the loads of a k-block take
+// about 2400 clocks, so that five stages bound a tile of 128 tokens at 480 clocks a k-block, whose products take 256; and a
+// pass over few tokens is a stream of weights from HBM (32 tokens: eleven stages, 198 KB in flight instead of 80).  Three rings
+// come from the host, for tiles of up to 128 tokens (or the call's tokens, if fewer), of 256, and for merged items of 320; the
+// layout leaves the rows of the largest expert in meta[7] and what merges in meta[3], meta[4], and every role finds the same
+// one.  (Worked out in the kernel for every item, passes of short items took 1-3 % longer; stages as large as their own tile,
+// in a ring of bytes, cost the loaders more than the depth gave.)
+// Against two rings, one for calls of up to 256 tokens: 4096 tokens x 8, 256 experts, 7168 x 2048: 4968 -> 4877 us (six stages for
+// five); 2048 x 4, 128 experts, 4096 x 1536: 894 -> 864 (eight); 512 x 6 + 2, 64 experts, 2048 x 1408: 236 -> 233.
 constexpr size_t PIPE_BARRIER_BYTES = 384;
 constexpr size_t TICKET_RING_BYTES = 640;   // of the persistent launch
 constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_RING_BYTES;
 __host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return EPI_WARPS * (size_t)sw_staging_bytes(mode); }
 __host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
 // The same for every role and item of a launch: the layout is complete before them.
-__device__ __forceinline__ bool wants_full_ring(const GemmArgs& a) { return uniform(a.meta[7] > a.ring_rows ? 1 : 0) != 0; }
+__device__ __forceinline__ int which_ring(const GemmArgs& a) {
+  return uniform(a.meta[7] <= a.ring_rows ? 0 : a.meta[3] == a.meta[4] ? 1 : 2);
+}
 // does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
 __device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s) {
   return (size_t)r.stages * W_STAGE_BYTES + (size_t)(s + 1) * r.tok_bytes > WGRAD_STAGING_AT ||
@@ -221,10 +226,10 @@ __device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s)
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
 // tokens.
 template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, bool full, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
+__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, int ring_of, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
                                                bool tok_warp, int rank, int lane, const SwapWork& wk, int t,
                                                const WaitCtl& wc, const DEP& dep) {
-  const GemmArgs::Ring ring = full ? a.full : a.ring;
+  const GemmArgs::Ring ring = a.ring[ring_of];
   const int stages = ring.stages, tokb = ring.tok_bytes;
   uint8_t* sW = smem;                              // [stages][16 KB] weights
   uint8_t* sT = smem + stages * W_STAGE_BYTES;     // [stages][tokb] tokens (this CTA's half)
@@ -277,10 +282,10 @@ __device__ __forceinline__ bool acc_claim(PipeBarriers* bars, IssuerState& is, i
 // MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop with uniform control flow and operands; one elected
 // lane issues (common.cuh).
 template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, bool full, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
+__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, int ring_of, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
                                                 IssuerState& is, const SwapWork& wk, int t, const WaitCtl& wc,
                                                 const DEP& dep) {
-  const GemmArgs::Ring ring = full ? a.full : a.ring;
+  const GemmArgs::Ring ring = a.ring[ring_of];
   const uint32_t stages = ring.stages, t_step = ring.tok_bytes >> 4;
   const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
   const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + stages * W_STAGE_BYTES), 16);

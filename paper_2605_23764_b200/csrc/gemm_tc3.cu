@@ -5,8 +5,6 @@
 //
 // Roles per CTA: warp 0 TMA producer of the weights, warp 1 MMA issuer (even CTA) and TMEM owner,
 // warps 2-5 and 8-11 epilogue, warp 6 TMA producer of the tokens.
-#include <limits.h>
-
 #include "gemm_roles.cuh"
 #include "launch_pairs.cuh"
 
@@ -49,14 +47,14 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   // Items pair, pair + npairs, ..; each role decodes item i + 1 before it works on item i (the decode's chain of
   // global loads then completes behind the item's work).
   const int total = total_swap_work(a);
-  const bool full = wants_full_ring(a);
+  const int ring = which_ring(a);
   SwapWork cur, next;
   if (pair < total) cur = decode_swap_work<MODE>(a, pair);
   if (warp == 0 || warp == 6) {
     LoaderState ls;
     for (int t = pair; t < total; t += npairs, cur = next) {
       if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-      if (!swap_load_item<MODE>(a, full, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
+      if (!swap_load_item<MODE>(a, ring, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
     }
   } else if (warp == 1) {
     if (rank == 0) {
@@ -64,7 +62,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       bool ok = true;
       for (int t = pair; t < total && ok; t += npairs, cur = next) {
         if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-        ok = swap_issue_item<MODE>(a, full, smem, bars, tmem_base, is, cur, t, wc, dep);
+        ok = swap_issue_item<MODE>(a, ring, smem, bars, tmem_base, is, cur, t, wc, dep);
       }
       if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }
@@ -93,12 +91,11 @@ void plan_ring(GemmMode mode, int T, GemmArgs& a) {
     const int stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + tok_bytes));
     return GemmArgs::Ring{stages < MAX_STAGES ? stages : MAX_STAGES, tok_bytes};
   };
-  a.full = a.ring = of((merges ? 3 : 2) * 64 * BK * 2);
-  a.ring_rows = INT_MAX;
-  if (T <= 2 * BLOCK_M) {
-    a.ring_rows = (T + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN;
-    a.ring = of(a.ring_rows / 2 * BK * 2);
-  }
+  const int rows = (T + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN;
+  a.ring_rows = rows < BLOCK_M ? rows : BLOCK_M;
+  a.ring[0] = of(a.ring_rows / 2 * BK * 2);
+  a.ring[1] = of(BLOCK_M * BK * 2);
+  a.ring[2] = merges ? of(3 * BLOCK_M / 2 * BK * 2) : a.ring[1];
 }
 
 template <int MODE>

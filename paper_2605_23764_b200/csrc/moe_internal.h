@@ -144,8 +144,7 @@ struct GemmArgs {
   int F;               // intermediate size (GATE_UP / ACT_GRAD epilogues)
   // row-space modes: operand stages and the token bytes of a stage per CTA (gemm_roles.cuh, plan_ring) ..
   struct Ring { int stages, tok_bytes; };
-  Ring ring;           // .. where no expert has more than ring_rows rows
-  Ring full;           // .. and where one has
+  Ring ring[3];        // .. where no expert has more than ring_rows rows; where none merges; and for merged items
   int ring_rows;
   // epilogue tensors
   uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]; rows row_ld(..) apart
@@ -157,7 +156,7 @@ struct GemmArgs {
   uint64_t budget_ns;
 };
 
-// Shared-memory plan of a row-space operator for calls of T tokens: fills ring, full and ring_rows.
+// Shared-memory plan of a row-space operator for calls of T tokens: fills ring and ring_rows.
 void plan_ring(GemmMode mode, int T, GemmArgs& a);
 // ---- gemm_tc3.cu: the row-space operators with the tokens as accumulator COLUMNS (weights take the
 // 256 accumulator rows of a CTA pair), so a tile's MMA time follows the expert's real token count

@@ -75,6 +75,18 @@ def test_merged_tiles_in_every_operator(d, serial):
     _check_against_oracle(T, d, E, 1, F, ids, w, 42, serial)
 
 
+@pytest.mark.parametrize("counts", [[128, 33, 96, 0, 128, 127], [129, 128, 256, 31, 511], [129, 257, 100, 320, 64]])
+@pytest.mark.parametrize("serial", [False, True])
+def test_operand_ring_by_largest_expert(counts, serial):
+    """Largest expert of 128 rows, of more without a merged item, and with one: the three rings; more k-blocks than stages."""
+    E, T, d, F = len(counts), sum(counts), 840, 392
+    g = torch.Generator().manual_seed(51)
+    ids = torch.from_numpy(np.repeat(np.arange(E), counts).astype(np.int32))
+    ids = ids[torch.randperm(T, generator=g)].reshape(T, 1).contiguous().cuda()
+    w = (torch.rand(T, 1, generator=g) + 0.25).float().cuda()
+    _check_against_oracle(T, d, E, 1, F, ids, w, 52, serial)
+
+
 def _check_against_oracle(T, d, E, k, F, ids, w, seed, serial):
     g = torch.Generator().manual_seed(seed)
     x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
