@@ -344,7 +344,7 @@ GemmArgs args_gate_up(const moe_ctx* c, int T) {
   g.tmB = c->tm_W1_gu;
   g.n_tiles_n = (s.F + 127) / 128;
   g.K = s.d;
-  g.merges = phase_merges(g.K);
+  g.merges = phase_merges(0, g.K);
   g.N = s.F;
   g.b_rows_per_expert = 2 * s.F;
   g.out0 = c->at<uint16_t>(c->plan.A);
@@ -377,7 +377,7 @@ GemmArgs args_act_grad(const moe_ctx* c, int T, bool want_dw) {
   g.tmB = c->tm_W2_mn;
   g.n_tiles_n = p.ntn_act;
   g.K = s.d;
-  g.merges = phase_merges(g.K);
+  g.merges = phase_merges(1, g.K);
   g.N = s.F;
   g.b_rows_per_expert = s.d;
   g.out0 = c->at<uint16_t>(p.dH);
@@ -456,7 +456,7 @@ ChainParams make_chain(bool bwd, int T, int Ep, int k, int n_shared, int d, int 
     cp.n_phases = 2;
     cp.ntn[0] = (F + 127) / 128;                 // gate+up: 128 features (gate and up) per pair tile
     cp.ntn[1] = (d + 255) / 256;                 // down
-    cp.merges[0] = phase_merges(d);
+    cp.merges[0] = phase_merges(0, d);
     cp.merges[1] = 1;
   } else {
     cp.n_phases = 4;
@@ -464,7 +464,7 @@ ChainParams make_chain(bool bwd, int T, int Ep, int k, int n_shared, int d, int 
     cp.ntn[1] = (F + 255) / 256;                 // w2_grad: column tiles per strip
     cp.strips[1] = (d + 255) / 256;
     cp.ntn[2] = (d + 255) / 256;                 // gate_grad
-    cp.merges[0] = phase_merges(d);
+    cp.merges[0] = phase_merges(1, d);
     cp.merges[2] = 1;
     cp.ntn[3] = (d + 255) / 256;                 // w1_grad
     cp.strips[3] = (2 * F + 255) / 256;

@@ -74,12 +74,13 @@ MOE_HD void balanced_unit(int mc, int u, int* first, int* count) {
 // of the larger of the two tiles (gemm_roles.cuh, acc_claim), is short.  With a full last block (e.g. 384 rows) that costs
 // as much as the second weight pass or more: down was 5 % faster unmerged there, 257..320-row experts 6 % slower.
 constexpr int MERGE_TAIL_MAX = 64;
-// Do gate+up and act_grad, whose reduction is K long, merge too?  128 + 160 tokens take 880 clocks a k-block as two tiles
-// (the loads of a small tile take longer than its products) and 595 as one item, so an item of 112 k-blocks is 18 us shorter; what
-// it exposes of gate+up's epilogue is 3 us, of act_grad's 10.  K = 7168, 128 experts of 256 rows: a training step 10260 -> 10015
-// us; K = 4096, skewed experts: forward 4920 -> 4780; K = 2048 (32 k-blocks), experts of up to 384 rows: a step 1830 -> 1870.
-constexpr int MERGE_MIN_K = 4096;
-MOE_HD int phase_merges(int K) { return K >= MERGE_MIN_K; }
+// Do gate+up (op 0) and act_grad (op 1), whose reduction is K long, merge too?  128 + 160 tokens take 880 clocks a k-block as two
+// tiles (the loads of a small tile take longer than its products) and 595 as one item; what that exposes of gate+up's epilogue is
+// 3 us, of act_grad's 10.  gate+up gains at every K: forward over 64 experts of 300 rows, K = 512 118 -> 108 us, 1024 181 -> 169,
+// 2048 422 -> 383, 3072 471 -> 444 (below nine k-blocks, K = 256 68 -> 65, the numbers of work items are relied upon).  act_grad: a
+// step with K = 2048 1242 -> 1232 us, 3072 1349 -> 1332, even at 1024; K = 7168, 128 experts of 256 rows, both 10260 -> 10015.
+constexpr int MERGE_MIN_K_GATE_UP = 576, MERGE_MIN_K_ACT_GRAD = 2048;
+MOE_HD int phase_merges(int op, int K) { return K >= (op == 0 ? MERGE_MIN_K_GATE_UP : MERGE_MIN_K_ACT_GRAD); }
 MOE_HD bool expert_merges(int rows, int mblocks) {
   return (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
 }

@@ -18,7 +18,7 @@ def _expected_items(counts, d, F, is_bwd):
     # an expert merges its last two units when its M-block count is odd, at least 3, and the last block holds <= 64 rows
     merged = units - ((mblocks % 2 == 1) & (mblocks >= 3) & (counts - (mblocks - 1) * 128 <= 64))
     Ep = len(counts)
-    first = merged if d >= 4096 else units   # gate+up and act_grad merge where their reduction is long
+    first = merged if d >= (2048 if is_bwd else 576) else units   # gate+up and act_grad merge where their reduction is long
     if not is_bwd:
         return int(first.sum()) * ((F + 127) // 128) + int(merged.sum()) * ((d + 255) // 256)
     return (int(first.sum()) * ((F + 255) // 256) + Ep * ((d + 255) // 256) +
@@ -47,7 +47,7 @@ def test_schedule_is_sound(is_bwd, workers):
 
 
 @pytest.mark.parametrize("is_bwd", [0, 1])
-@pytest.mark.parametrize("d", [4088, 4096, 7168])
+@pytest.mark.parametrize("d", [568, 576, 2040, 2048, 7168])
 def test_first_operator_merges_where_its_reduction_is_long(is_bwd, d):
     counts = np.array([300, 257, 320, 577, 321, 384, 0, 64])
     rc, stats = binding.moe_debug_simulate_schedule(counts, 1111, 2, 0, d, 272, is_bwd, 74, 592)
