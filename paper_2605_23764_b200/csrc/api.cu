@@ -1165,11 +1165,25 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
     case MOE_BUF_DXP: off = p.Y; cols = s.d; break;
     case MOE_BUF_META: off = p.meta; n = 8; break;
     case MOE_BUF_TRACE: if (!p.trace_cap) return MOE_ERR_STATE; off = p.trace; n = (size_t)p.trace_cap * 8; break;
-    case MOE_BUF_EVENT_COUNTERS: off = c->last_ctr ? (size_t)(reinterpret_cast<uint8_t*>(c->last_ctr) - c->ws) : p.ctr; n = p.ctr_count; break;
+    case MOE_BUF_EVENT_COUNTERS: off = c->last_ctr ? (size_t)(reinterpret_cast<uint8_t*>(c->last_ctr) - c->ws) : p.ctr; n = 8 + 4 * (size_t)((p.ctr_count - CTR_PER_MB) / CTR_STRIDE); break;
     default: return MOE_ERR_INVALID_ARG;
   }
   *ptr = c->ws + off;
   *elems = cols ? cap * cols : n;
+  if (which == MOE_BUF_EVENT_COUNTERS) {   // the words lie apart (schedule.h): a compact copy
+    const int* src = reinterpret_cast<const int*>(c->ws + off);
+    void*& copy = c->debug_copy[which];
+    if (!copy) MOE_CUDA(cudaMalloc(&copy, sizeof(int) * n));
+    int* dst = static_cast<int*>(copy);
+    auto bring = [&](int* to, const int* from, int ints) { return cudaMemcpyAsync(to, from, sizeof(int) * ints, cudaMemcpyDeviceToDevice, c->last_stream); };
+    MOE_CUDA(bring(dst, src, 8));
+    MOE_CUDA(bring(dst + 2, src + CTR_MAT_TICKET, 1));
+    MOE_CUDA(bring(dst + 3, src + CTR_POST_TICKET, 1));
+    MOE_CUDA(cudaMemcpy2DAsync(dst + 8, 4 * sizeof(int), src + CTR_PER_MB, CTR_STRIDE * sizeof(int), 4 * sizeof(int), (n - 8) / 4,
+                               cudaMemcpyDeviceToDevice, c->last_stream));
+    MOE_CUDA(cudaStreamSynchronize(c->last_stream));
+    *ptr = copy;
+  }
   if (cols && cols != (size_t)row_ld((int)cols)) {   // rows are farther apart in the workspace: a compact copy
     const size_t ld = row_ld((int)cols);
     void*& copy = c->debug_copy[which];

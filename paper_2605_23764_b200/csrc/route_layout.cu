@@ -107,6 +107,11 @@ __device__ __forceinline__ int slot_expert(const int* __restrict__ ids, int i, i
   return (e >= 0 && e < E) ? e : -1;
 }
 
+// zero[0, n), n a multiple of 4, 16-byte aligned: the share of thread `first` of `threads`
+__device__ __forceinline__ void clear_ints(int* zero, int n, int first, int threads) {
+  for (int i = first; i < n / 4; i += threads) reinterpret_cast<int4*>(zero)[i] = make_int4(0, 0, 0, 0);
+}
+
 constexpr int HIST_THREADS = 1024;
 __global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __restrict__ ids, int n, int k, int kp, int E,
                                                                    int Ep, int* __restrict__ blk_hist, int* __restrict__ tok_last,
@@ -126,7 +131,7 @@ __global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __
   if (tok_last)   // the tokens whose first slot lies in this block's chunk
     for (int i = base; i < min(n, (int)(blockIdx.x + 1) * LAYOUT_CHUNK); i += HIST_THREADS)
       if (i % kp == 0) tok_last[i / kp] = 0;
-  for (int i = blockIdx.x * HIST_THREADS + threadIdx.x; i < nzero; i += gridDim.x * HIST_THREADS) zero[i] = 0;
+  clear_ints(zero, nzero, blockIdx.x * HIST_THREADS + threadIdx.x, gridDim.x * HIST_THREADS);
 #pragma unroll
   for (int g = 0; g < LAYOUT_CHUNK / HIST_THREADS; ++g) {
     const uint32_t peers = __match_any_sync(0xffffffffu, e[g]);
@@ -478,7 +483,7 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
   pdl_trigger();
   pdl_wait();
   const int e = i < n ? slot_expert(ids, i, k, kp, E) : -1;
-  for (int q = threadIdx.x; q < nzero; q += 1024) zero[q] = 0;
+  clear_ints(zero, nzero, threadIdx.x, 1024);
   __syncthreads();
   int r = 0;
   if (warp < warps) {
@@ -575,7 +580,7 @@ __global__ void __launch_bounds__(1024)
   int e[LAYOUT_CLUSTER_G], r[LAYOUT_CLUSTER_G];
 #pragma unroll
   for (int g = 0; g < LAYOUT_CLUSTER_G; ++g) e[g] = g < G && i0 + 32 * g < s1 ? slot_expert(ids, i0 + 32 * g, k, kp, E) : -1;
-  for (int q = rank * 1024 + threadIdx.x; q < nzero; q += C * 1024) zero[q] = 0;
+  clear_ints(zero, nzero, rank * 1024 + threadIdx.x, C * 1024);
   __syncthreads();
   uint16_t* mine = whist + warp * ld;
 #pragma unroll

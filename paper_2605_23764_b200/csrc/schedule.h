@@ -229,12 +229,18 @@ MOE_HD int rotate_index(int i, int first, int n) {
 }
 
 // ---------------------------------------------------------------- counters (ints in device memory)
-constexpr int CTR_VEC_TICKET = 0, CTR_TRACE_CURSOR = 1, CTR_MAT_TICKET = 2, CTR_POST_TICKET = 3, CTR_PER_MB = 8, CTR_STRIDE = 4;
+// 700 warps and more poll these words.  By the times, about 1 KB of consecutive addresses is served by one part of L2: where all of
+// a small pass's counters lay in one such block -- a matter of where the workspace began -- signals and tickets queued behind
+// the polls.  The three tickets therefore have a block each and the counters of an M-block 64 bytes.  1024 tokens x 4, 32 experts,
+// 1024 x 512, forward: 57.6 us in one block, 51.7 in two, 49.2 so; 1777 x 3 + 1, 24 experts, 1160 x 712, a step: 217 -> 205; 256 x 2, 8
+// experts, 256 x 128, a step: 49.3 -> 46.2.  32 or 128 bytes an M-block: even to 2 % slower.
+constexpr int CTR_VEC_TICKET = 0, CTR_TRACE_CURSOR = 1, CTR_MAT_TICKET = 256, CTR_POST_TICKET = 512, CTR_PER_MB = 768, CTR_STRIDE = 16;
 // combine tasks finished, and the word that turns 1 when all of them are (a copy-out stream may wait on it)
 constexpr int CTR_COMBINE_DONE = 4, CTR_OUT_READY = 5;
 enum CtrKind : int { CTR_GATHERED = 0, CTR_ACTIVATED = 1, CTR_DONE = 2, CTR_NONE = -1 };
 MOE_HD int ctr_index(int mb, int kind) { return CTR_PER_MB + CTR_STRIDE * mb + kind; }
 MOE_HD int ctr_ints(int cap_mblocks) { return CTR_PER_MB + CTR_STRIDE * cap_mblocks; }
+static_assert(CTR_PER_MB % 4 == 0 && CTR_STRIDE % 4 == 0, "cleared 16 bytes at a time");
 
 // dependent / trigger counter kind of each phase
 MOE_HD int phase_wait_kind(const ChainParams& cp, int phase) {

@@ -156,3 +156,32 @@ def test_workspace_views_of_one_context_stay_apart():
     for n, v, t, cols in zip(names, views, want, (d, d, F, 2 * F)):
         assert torch.equal(v.view(-1, cols)[rows], t.view(torch.int16).view(-1, cols)[rows]), n
     layer.close()
+
+
+@pytest.mark.parametrize("T", [1, 70, 300])
+def test_event_counters_as_documented(T):
+    """moe_debug_buffer's view of the event counters, which lie apart in the workspace: eight words, then {gathered, activated,
+    done, 0} of each M-block -- after a forward, and again after a backward, at their thresholds."""
+    d, E, k, S, F = 264, 5, 2, 1, 136
+    x, W1, W2, logits, dout = small_problem(T, d, E, k, S, F, 12)
+    layer = MoeLayer(T, d, E, k, S, F, save_for_bwd=True)
+    ids, w = layer.route(logits)
+
+    def expect(col_tiles_first, col_tiles_last):
+        counts = layer.debug("counts").cpu().numpy()
+        want = []
+        for n in counts:
+            n32 = (int(n) + 31) // 32 * 32
+            want += [[min(128, n32 - r) // 4, 2 * col_tiles_first, 2 * col_tiles_last, 0] for r in range(0, int(n), 128)]
+        got = layer.debug("event_counters").cpu()
+        assert got[1] == 0   # no trace
+        assert got[8:8 + 4 * len(want)].reshape(-1, 4).tolist() == want
+        assert torch.count_nonzero(got[8 + 4 * len(want):]).item() == 0
+
+    layer.ffn_fwd(x, ids, w, W1, W2)
+    torch.cuda.synchronize()
+    expect((F + 127) // 128, (d + 255) // 256)
+    layer.ffn_bwd(dout, x, ids, w, W1, W2)
+    torch.cuda.synchronize()
+    expect((F + 255) // 256, (d + 255) // 256)
+    layer.close()
