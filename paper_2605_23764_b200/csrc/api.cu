@@ -132,7 +132,7 @@ struct Carve {
 
 // Byte offsets of every workspace tensor.
 struct WsPlan {
-  size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, pair_start, pblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, wg_order, group_start, group_row, group_slot, prow_w,
+  size_t status, meta, counts, offsets, pad_off, mb_start, mblk_expert, work_start, wblk_expert, blk_hist, row_of, src_of, prow_of, combine_order, tok_last, wg_order, group_start, group_row, group_slot, prow_w,
       dw_partial, Xp, H, A, Y, dOutp, dH, st_x[2], st_dout, st_ids, st_w, st_out, st_dx, st_dw, st_logits, ctr, trace, total;
   int cap_rows, nblk_max, ntn_act, ctr_count, trace_cap;
 };
@@ -155,8 +155,6 @@ WsPlan plan_workspace(const moe_shape& s) {
   p.pad_off = c.take(sizeof(int) * (Ep + 1));
   p.mb_start = c.take(sizeof(int) * (Ep + 1));
   p.mblk_expert = c.take(sizeof(int) * (cap / BLOCK_M + 1));
-  p.pair_start = c.take(sizeof(int) * (Ep + 1));
-  p.pblk_expert = c.take(sizeof(int) * (cap / BLOCK_M + 1));
   p.work_start = c.take(sizeof(int) * (Ep + 1));
   p.wblk_expert = c.take(sizeof(int) * (cap / BLOCK_M + 1));
   p.blk_hist = c.take(sizeof(int) * (size_t)p.nblk_max * Ep);
@@ -260,8 +258,6 @@ struct moe_ctx {
     lv.pad_off = at<int>(plan.pad_off);
     lv.mb_start = at<int>(plan.mb_start);
     lv.mblk_expert = at<int>(plan.mblk_expert);
-    lv.pair_start = at<int>(plan.pair_start);
-    lv.pblk_expert = at<int>(plan.pblk_expert);
     lv.work_start = at<int>(plan.work_start);
     lv.wblk_expert = at<int>(plan.wblk_expert);
     lv.meta = at<int>(plan.meta);
@@ -323,8 +319,6 @@ GemmArgs base_args(const moe_ctx* c) {
   g.mb_start = lv.mb_start;
   g.counts = lv.counts;
   g.meta = lv.meta;
-  g.pair_start = lv.pair_start;
-  g.pblk_expert = lv.pblk_expert;
   g.work_start = lv.work_start;
   g.wblk_expert = lv.wblk_expert;
   g.wg_order = lv.wg_order;
@@ -344,7 +338,6 @@ GemmArgs args_gate_up(const moe_ctx* c, int T) {
   g.tmB = c->tm_W1_gu;
   g.n_tiles_n = (s.F + 127) / 128;
   g.K = s.d;
-  g.merges = phase_merges(0, g.K);
   g.N = s.F;
   g.b_rows_per_expert = 2 * s.F;
   g.out0 = c->at<uint16_t>(c->plan.A);
@@ -361,7 +354,6 @@ GemmArgs args_down(const moe_ctx* c, int T) {
   g.tmB = c->tm_W2_k128;  // each CTA of a pair loads 128 of the tile's 256 rows
   g.n_tiles_n = (s.d + 255) / 256;
   g.K = s.F;
-  g.merges = 1;
   g.N = s.d;
   g.b_rows_per_expert = s.d;
   g.out0 = c->at<uint16_t>(c->plan.Y);
@@ -377,7 +369,6 @@ GemmArgs args_act_grad(const moe_ctx* c, int T, bool want_dw) {
   g.tmB = c->tm_W2_mn;
   g.n_tiles_n = p.ntn_act;
   g.K = s.d;
-  g.merges = phase_merges(1, g.K);
   g.N = s.F;
   g.b_rows_per_expert = s.d;
   g.out0 = c->at<uint16_t>(p.dH);
@@ -409,7 +400,6 @@ GemmArgs args_gate_grad(const moe_ctx* c, int T) {
   g.tmB = c->tm_W1_mn;
   g.n_tiles_n = (s.d + 255) / 256;
   g.K = 2 * s.F;
-  g.merges = 1;
   g.N = s.d;
   g.b_rows_per_expert = 2 * s.F;
   g.out0 = c->at<uint16_t>(c->plan.Y);
@@ -456,16 +446,12 @@ ChainParams make_chain(bool bwd, int T, int Ep, int k, int n_shared, int d, int 
     cp.n_phases = 2;
     cp.ntn[0] = (F + 127) / 128;                 // gate+up: 128 features (gate and up) per pair tile
     cp.ntn[1] = (d + 255) / 256;                 // down
-    cp.merges[0] = phase_merges(0, d);
-    cp.merges[1] = 1;
   } else {
     cp.n_phases = 4;
     cp.ntn[0] = (F + 255) / 256;                 // act_grad
     cp.ntn[1] = (F + 255) / 256;                 // w2_grad: column tiles per strip
     cp.strips[1] = (d + 255) / 256;
     cp.ntn[2] = (d + 255) / 256;                 // gate_grad
-    cp.merges[0] = phase_merges(1, d);
-    cp.merges[2] = 1;
     cp.ntn[3] = (d + 255) / 256;                 // w1_grad
     cp.strips[3] = (2 * F + 255) / 256;
   }
@@ -1203,11 +1189,10 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
                                 int32_t F, int32_t is_bwd, int32_t pairs, int32_t vec_workers, int64_t* stats) {
   if (!counts || Ep < 1 || pairs < 1 || vec_workers < 1 || d < 8 || F < 8) return MOE_ERR_INVALID_ARG;
   // the tables of the layout kernels
-  std::vector<int> mb_start(Ep + 1, 0), pair_start(Ep + 1, 0), work_start(Ep + 1, 0);
+  std::vector<int> mb_start(Ep + 1, 0), work_start(Ep + 1, 0);
   for (int e = 0; e < Ep; ++e) {
     const int m = (counts[e] + BLOCK_M - 1) / BLOCK_M, pr = (m + 1) >> 1;
     mb_start[e + 1] = mb_start[e] + m;
-    pair_start[e + 1] = pair_start[e] + pr;
     work_start[e + 1] = work_start[e] + pr - (expert_merges(counts[e], m) ? 1 : 0);
   }
   std::vector<int> long_before(Ep + 1, 0), order(Ep, -1);
@@ -1215,11 +1200,9 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   const int n_long = long_before[Ep], E = Ep - n_shared;
   for (int e = 0; e < Ep; ++e) order[strip_order(e, counts[e], E, Ep, long_before[e], long_before[E], n_long)] = e;
   const int M = mb_start[Ep];
-  std::vector<int> pblk(pair_start[Ep] + 1, 0), wblk(work_start[Ep] + 1, 0);
-  for (int e = 0; e < Ep; ++e) {
-    for (int i = pair_start[e]; i < pair_start[e + 1]; ++i) pblk[i] = e;
+  std::vector<int> wblk(work_start[Ep] + 1, 0);
+  for (int e = 0; e < Ep; ++e)
     for (int i = work_start[e]; i < work_start[e + 1]; ++i) wblk[i] = e;
-  }
   ChainParams cp = make_chain(is_bwd != 0, T, Ep, k, n_shared, d, F, pairs);
   cp.want_dw = 1;
   // items of every phase: {first M-block, M-blocks of unit a, M-blocks of unit b} (strips: the expert's M-blocks)
@@ -1243,13 +1226,11 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
       for (int n : tiles)
         if (n != cp.ntn[ph]) return 14;
     } else {
-      const bool mg = cp.merges[ph] != 0;
-      const int total = (mg ? work_start[Ep] : pair_start[Ep]) * cp.ntn[ph];
-      const int first = n_shared > 0 ? (mg ? work_start[Ep - n_shared] : pair_start[Ep - n_shared]) * cp.ntn[ph] : 0;
+      const int total = work_start[Ep] * cp.ntn[ph];
+      const int first = n_shared > 0 ? work_start[Ep - n_shared] * cp.ntn[ph] : 0;
       for (int tq = 0; tq < total; ++tq) {
         const int t = rotate_index(tq, first, total);   // shared experts first (schedule.h)
-        const SwapItem it = decode_swap_item(t, cp.ntn[ph], mg, mg ? work_start.data() : pair_start.data(),
-                                             mg ? wblk.data() : pblk.data(), mb_start.data());
+        const SwapItem it = decode_swap_item(t, cp.ntn[ph], work_start.data(), wblk.data(), mb_start.data());
         if (it.e < 0 || it.e >= Ep || it.nb < 0 || it.nb >= cp.ntn[ph]) return 10;
         if (it.mb_first < mb_start[it.e] || it.mb_first + it.mb_count > mb_start[it.e + 1] || it.mb_count < 1 ||
             it.mb_count > 3 || it.mb_count_a < 1)

@@ -379,7 +379,7 @@ __device__ __forceinline__ PhaseTable make_phase_table(const FusedArgs& fa) {
 // Where each row-space phase's item list starts when there are shared experts (schedule.h, rotate_index): at the
 // first item of the first shared expert.  `first[p]` = 0: no rotation (no shared experts, or a weight-gradient phase).
 __device__ __forceinline__ int swap_first_item(const GemmArgs& a, int first_shared) {
-  return (a.merges ? a.work_start : a.pair_start)[first_shared] * a.n_tiles_n;
+  return a.work_start[first_shared] * a.n_tiles_n;
 }
 template <bool BWD>
 __device__ __forceinline__ PhaseTable make_rotation_table(const FusedArgs& fa) {

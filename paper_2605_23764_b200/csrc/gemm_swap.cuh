@@ -41,24 +41,21 @@ __device__ __forceinline__ void unit_tokens(const GemmArgs& a, int e, int first,
   *ntok = end - first * BLOCK_M;
 }
 
-// One work item of a row-space operator: a token tile, or -- in the operators that merge (schedule.h),
-// for an expert with an odd count of three or more M-blocks -- its last two token tiles (one block;
-// block + tail) under ONE k-loop: the weight stage is written to shared memory once and multiplied with
+// One work item of a row-space operator: a token tile, or -- for an expert that merges (schedule.h) -- its last two token
+// tiles (one block; block + tail) under ONE k-loop: the weight stage is written to shared memory once and multiplied with
 // both token tiles into two accumulators (shared-memory traffic bounds these kernels, and the
 // weights are the larger half of it).  For the epilogue warps the item is two tiles.
 struct SwapWork {
   SwapTile a, b;
   bool merged;
 };
-__device__ __forceinline__ int total_swap_work(const GemmArgs& a) { return (a.merges ? a.meta[4] : a.meta[3]) * a.n_tiles_n; }
+__device__ __forceinline__ int total_swap_work(const GemmArgs& a) { return a.meta[4] * a.n_tiles_n; }
 
 // Item order: expert-major; inside an expert the feature tile is the slow index and the item the
 // fast one (items running at the same time share one slab of weights in L2).
 template <int MODE>
 __device__ __forceinline__ SwapWork decode_swap_work(const GemmArgs& a, int t) {
-  const bool mg = a.merges != 0;
-  const SwapItem it = decode_swap_item(t, a.n_tiles_n, mg, mg ? a.work_start : a.pair_start,
-                                       mg ? a.wblk_expert : a.pblk_expert, a.mb_start);
+  const SwapItem it = decode_swap_item(t, a.n_tiles_n, a.work_start, a.wblk_expert, a.mb_start);
   SwapWork w;
   w.merged = it.merged != 0;
   w.a.e = w.b.e = it.e;

@@ -86,7 +86,6 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
 }
 
 void plan_ring(GemmMode mode, int T, GemmArgs& a) {
-  const bool merges = a.merges || mode == GEMM_GATE_UP;   // gate+up: laid out like down
   auto of = [&](int tok_bytes) {
     const int stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + tok_bytes));
     return GemmArgs::Ring{stages < MAX_STAGES ? stages : MAX_STAGES, tok_bytes};
@@ -95,7 +94,7 @@ void plan_ring(GemmMode mode, int T, GemmArgs& a) {
   a.ring_rows = rows < BLOCK_M ? rows : BLOCK_M;
   a.ring[0] = of(a.ring_rows / 2 * BK * 2);
   a.ring[1] = of(BLOCK_M * BK * 2);
-  a.ring[2] = merges ? of(3 * BLOCK_M / 2 * BK * 2) : a.ring[1];
+  a.ring[2] = of(3 * BLOCK_M / 2 * BK * 2);
 }
 
 template <int MODE>

@@ -62,16 +62,14 @@ struct LayoutView {
   int* pad_off;      // [Ep+1]  first padded row of each expert (multiple of BLOCK_M)
   int* mb_start;     // [Ep+1]  first M-block of each expert
   int* mblk_expert;  // [R_pad_max / BLOCK_M] expert of each M-block
-  int* pair_start;   // [Ep+1]  first M-block pair of each expert (pairs = ceil(M-blocks / 2))
-  int* pblk_expert;  // [pairs] expert of each M-block pair
-  int* work_start;   // [Ep+1]  first work item of each expert (token-column GEMMs that merge: its units, the last
-                     //         two of an odd M-block count >= 3 merged into one item)
+  int* work_start;   // [Ep+1]  first work item of each expert (its token tiles, the last two merged into one item where
+                     //         expert_merges, schedule.h)
   int* wblk_expert;  // [items] expert of each work item
   int* wg_order;     // [Ep]    experts in the order of the weight-gradient phases (schedule.h); NULL: not wanted
   int* group_start;  // [Ep+1]  first 32-row group of each expert (an expert's rows up to a multiple of 32); NULL: not wanted
   int* group_row;    // [groups] first padded row of each group
   int* group_slot;   // [groups * 32] slot of each of the groups' rows, -1 for padding
-  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_pairs, num_work_items, num_groups, long experts, rows of the largest expert}
+  int* meta;         // [8]     {num_mblocks, R_pad, rows, num_token_tiles, num_work_items, num_groups, long experts, rows of the largest expert}
   int* blk_hist;     // [nblk][Ep] per-block histograms, then per-block exclusive prefixes
   int* combine_order; // [T] persistent launch: tokens in the order in which their last row is produced (NULL: token order)
   int* tok_last;      // [T] 1 + largest padded row of each token (0: none); NULL when the combine order is not wanted
@@ -126,8 +124,6 @@ struct GemmArgs {
   const int* mb_start;
   const int* counts;
   const int* meta;
-  const int* pair_start;   // CTA-pair kernels: first M-block pair of each expert
-  const int* pblk_expert;  // CTA-pair kernels: expert of each M-block pair
   const int* work_start;   // token-column kernel: first work item of each expert
   const int* wblk_expert;  // token-column kernel: expert of each work item
   const int* wg_order;     // WGRAD: order of the experts
@@ -137,14 +133,13 @@ struct GemmArgs {
   int n_tiles_m;       // WGRAD only: tiles along M per expert
   int split;           // WGRAD only: ranges of column tiles per strip (schedule.h)
   int K;               // reduction length (row-space modes)
-  int merges;          // row-space modes: 1 if experts that can (expert_merges) have their last two token tiles under one k-loop
   int N;               // output columns (for masking); WGRAD: columns of dW
   int M;               // WGRAD: rows of dW per expert
   int b_rows_per_expert;  // rows of the B tensor map per expert slab
   int F;               // intermediate size (GATE_UP / ACT_GRAD epilogues)
   // row-space modes: operand stages and the token bytes of a stage per CTA (gemm_roles.cuh, plan_ring) ..
   struct Ring { int stages, tok_bytes; };
-  Ring ring[3];        // .. where no expert has more than ring_rows rows; where none merges; and for merged items
+  Ring ring[3];        // .. where no expert has more than ring_rows rows; where none merges (expert_merges); and for merged items
   int ring_rows;
   // epilogue tensors
   uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]; rows row_ld(..) apart

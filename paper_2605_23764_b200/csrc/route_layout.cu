@@ -141,31 +141,30 @@ __global__ void __launch_bounds__(HIST_THREADS) layout_hist_kernel(const int* __
   for (int q = threadIdx.x; q < Ep; q += HIST_THREADS) blk_hist[(size_t)blockIdx.x * Ep + q] = hist[q];
 }
 
-// Exclusive scans over the experts of a block of 1024 threads: s_counts[Ep] -> offsets of rows, M-blocks, pairs of
-// M-blocks, work items, 32-row groups and long experts, in shared memory (each Ep + 1 long) and in the layout's tables; and the
-// rows of the largest expert.
-constexpr int SCAN_Q = 6;
-constexpr int SCAN_ROWS = SCAN_Q + 1;   // of `totals`: by warp and behind them the block's; the last row holds maxima
-struct ExpertScan { int *counts, *off, *mb, *pr, *wi, *gr, *lg; };   // shared memory
-__host__ __device__ constexpr int expert_scan_ints(int Ep) { return 7 * Ep + 6; }
+// Exclusive scans over the experts of a block of 1024 threads: s_counts[Ep] -> offsets of rows, M-blocks, work items,
+// 32-row groups and long experts, in shared memory (each Ep + 1 long) and in the layout's tables; the rows of the largest
+// expert and the number of token tiles.
+constexpr int SCAN_Q = 5;
+constexpr int SCAN_ROWS = SCAN_Q + 2;   // of `totals`: by warp and behind them the block's; the last rows hold maxima and sums
+struct ExpertScan { int *counts, *off, *mb, *wi, *gr, *lg; };   // shared memory
+__host__ __device__ constexpr int expert_scan_ints(int Ep) { return 6 * Ep + 5; }
 __device__ __forceinline__ ExpertScan expert_scan_at(int* sm, int Ep) {
-  return ExpertScan{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3, sm + 5 * Ep + 4, sm + 6 * Ep + 5};
+  return ExpertScan{sm, sm + Ep, sm + 2 * Ep + 1, sm + 3 * Ep + 2, sm + 4 * Ep + 3, sm + 5 * Ep + 4};
 }
 __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv, const ExpertScan& sc, int (*totals)[33],
                                              bool write = true) {
   constexpr int NQ = SCAN_Q;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int carry[NQ] = {0, 0, 0, 0, 0, 0}, largest = 0;
+  int carry[NQ] = {0, 0, 0, 0, 0}, largest = 0, tiles = 0;
   for (int e0 = 0; e0 < Ep; e0 += 1024) {
     const int e = e0 + threadIdx.x;
     const int c = e < Ep ? sc.counts[e] : 0;
     const int m = (c + BLOCK_M - 1) / BLOCK_M;
-    const int pr = (m + 1) >> 1;  // pairs of M-blocks (the tensor-core tile of a CTA pair)
-    // work items of the token-column GEMM kernels that merge: the units of the expert, except that an expert
+    const int pr = (m + 1) >> 1;  // token tiles (units, schedule.h)
+    // work items of the token-column GEMM kernels: the units of the expert, except that an expert
     // that merges (schedule.h) has its last two units (one block; block + tail) share one k-loop
-    const int val[NQ] = {c, m, pr, pr - (expert_merges(c, m) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS,
-                         strip_long(c)};
-    int inc[NQ] = {val[0], val[1], val[2], val[3], val[4], val[5]};
+    const int val[NQ] = {c, m, pr - (expert_merges(c, m) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS, strip_long(c)};
+    int inc[NQ] = {val[0], val[1], val[2], val[3], val[4]};
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
 #pragma unroll
@@ -178,8 +177,8 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
 #pragma unroll
       for (int q = 0; q < NQ; ++q) totals[q][warp] = inc[q];
     }
-    const int most = __reduce_max_sync(0xffffffffu, c);
-    if (lane == 0) totals[NQ][warp] = most;
+    const int most = __reduce_max_sync(0xffffffffu, c), prs = __reduce_add_sync(0xffffffffu, pr);
+    if (lane == 0) { totals[NQ][warp] = most; totals[NQ + 1][warp] = prs; }
     __syncthreads();
     if (warp < NQ) {   // warp q: exclusive scan of quantity q's warp totals, the block's total behind them
       const int w = totals[warp][lane];
@@ -194,49 +193,51 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
     } else if (warp == NQ) {
       const int m = __reduce_max_sync(0xffffffffu, totals[NQ][lane]);
       if (lane == 0) totals[NQ][32] = m;
+    } else if (warp == NQ + 1) {
+      const int n = __reduce_add_sync(0xffffffffu, totals[NQ + 1][lane]);
+      if (lane == 0) totals[NQ + 1][32] = n;
     }
     __syncthreads();
     int ex[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) ex[q] = carry[q] + totals[q][warp] + inc[q] - val[q];
     if (e < Ep) {
-      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.pr[e] = ex[2]; sc.wi[e] = ex[3]; sc.gr[e] = ex[4]; sc.lg[e] = ex[5];
+      sc.off[e] = ex[0]; sc.mb[e] = ex[1]; sc.wi[e] = ex[2]; sc.gr[e] = ex[3]; sc.lg[e] = ex[4];
     }
     if (write && e < Ep) {
       lv.counts[e] = c;
       lv.offsets[e] = ex[0];
       lv.mb_start[e] = ex[1];
       lv.pad_off[e] = ex[1] * BLOCK_M;
-      lv.pair_start[e] = ex[2];
-      lv.work_start[e] = ex[3];
+      lv.work_start[e] = ex[2];
       if (lv.group_start) {
-        lv.group_start[e] = ex[4];
-        for (int r = c; r < val[4] * GROUP_ROWS; ++r) lv.group_slot[ex[4] * GROUP_ROWS + r] = -1;   // padding rows of the last group
+        lv.group_start[e] = ex[3];
+        for (int r = c; r < val[3] * GROUP_ROWS; ++r) lv.group_slot[ex[3] * GROUP_ROWS + r] = -1;   // padding rows of the last group
       }
     }
 #pragma unroll
     for (int q = 0; q < NQ; ++q) carry[q] += totals[q][32];
     largest = max(largest, totals[NQ][32]);
+    tiles += totals[NQ + 1][32];
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.pr[Ep] = carry[2]; sc.wi[Ep] = carry[3]; sc.gr[Ep] = carry[4]; sc.lg[Ep] = carry[5];
+    sc.off[Ep] = carry[0]; sc.mb[Ep] = carry[1]; sc.wi[Ep] = carry[2]; sc.gr[Ep] = carry[3]; sc.lg[Ep] = carry[4];
   }
   if (write && threadIdx.x == 0) {
     lv.offsets[Ep] = carry[0];
     lv.mb_start[Ep] = carry[1];
     lv.pad_off[Ep] = carry[1] * BLOCK_M;
-    lv.pair_start[Ep] = carry[2];
-    lv.work_start[Ep] = carry[3];
+    lv.work_start[Ep] = carry[2];
     lv.meta[0] = carry[1];
     lv.meta[1] = carry[1] * BLOCK_M;
     lv.meta[2] = carry[0];
-    lv.meta[3] = carry[2];
-    lv.meta[4] = carry[3];
-    lv.meta[5] = carry[4];
-    lv.meta[6] = carry[5];
+    lv.meta[3] = tiles;
+    lv.meta[4] = carry[2];
+    lv.meta[5] = carry[3];
+    lv.meta[6] = carry[4];
     lv.meta[7] = largest;
-    if (lv.group_start) lv.group_start[Ep] = carry[4];
+    if (lv.group_start) lv.group_start[Ep] = carry[3];
   }
   __syncthreads();
   if (write && lv.wg_order)
@@ -256,7 +257,6 @@ __device__ __forceinline__ int expert_at(int Ep, const int* start, int i) {
 __device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, const ExpertScan& sc, int part = 0, int parts = 1) {
   const int first = part * blockDim.x + threadIdx.x, step = parts * blockDim.x;
   for (int i = first; i < sc.mb[Ep]; i += step) lv.mblk_expert[i] = expert_at(Ep, sc.mb, i);
-  for (int i = first; i < sc.pr[Ep]; i += step) lv.pblk_expert[i] = expert_at(Ep, sc.pr, i);
   for (int i = first; i < sc.wi[Ep]; i += step) lv.wblk_expert[i] = expert_at(Ep, sc.wi, i);
   if (lv.group_start)
     for (int i = first; i < sc.gr[Ep]; i += step) {
@@ -267,7 +267,7 @@ __device__ __forceinline__ void expert_tables(int Ep, const LayoutView& lv, cons
 
 // One block.  (1) per expert, exclusive scan of the block histograms over blocks: a thread per expert and range of
 // blocks (as many ranges as the block has threads for), so that the reads of a row are coalesced and independent;
-// (2) scans over experts; (3) M-block, pair and work-item -> expert tables.
+// (2) scans over experts; (3) M-block and work-item -> expert tables.
 __global__ void __launch_bounds__(1024) layout_scan_kernel(int nblk, int E, int Ep, LayoutView lv) {
   extern __shared__ int sm[];
   __shared__ int totals[SCAN_ROWS][33];
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(1024) layout_one_kernel(const int* __restrict_
   const ExpertScan sc = expert_scan_at(sm, Ep);
   int* s_last = sm + expert_scan_ints(Ep);                       // [LAYOUT_ONE_SLOTS] 1 + padded row of the slot
   int* bins = s_last + LAYOUT_ONE_SLOTS;               // [LAYOUT_ONE_SLOTS + 1]
-  uint16_t* whist = reinterpret_cast<uint16_t*>(bins + LAYOUT_ONE_SLOTS + 2 + (Ep & 1));   // [warps in use][ld]
+  uint16_t* whist = reinterpret_cast<uint16_t*>(bins + LAYOUT_ONE_SLOTS + 2 + (expert_scan_ints(Ep) & 1));   // [warps in use][ld]
   const int ld = Ep + (Ep & 1);
   const int warps = (n + 31) >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = threadIdx.x;
@@ -808,8 +808,6 @@ struct NoAllocScratch {
   int pad_off[NA_MAX_EP + 1];
   int mb_start[NA_MAX_EP + 1];
   int mblk_expert[NA_MAX_MBLK];
-  int pair_start[NA_MAX_EP + 1];
-  int pblk_expert[NA_MAX_MBLK];
   int work_start[NA_MAX_EP + 1];
   int wblk_expert[NA_MAX_MBLK];
   int blk_hist[NA_MAX_HIST];
@@ -862,8 +860,6 @@ extern "C" int moe_layout_noalloc(const int32_t* topk_ids, int32_t T, int32_t E,
   lv.pad_off = sc->pad_off;
   lv.mb_start = sc->mb_start;
   lv.mblk_expert = sc->mblk_expert;
-  lv.pair_start = sc->pair_start;
-  lv.pblk_expert = sc->pblk_expert;
   lv.work_start = sc->work_start;
   lv.wblk_expert = sc->wblk_expert;
   lv.meta = sc->meta;

@@ -68,27 +68,23 @@ MOE_HD void balanced_unit(int mc, int u, int* first, int* count) {
   }
 }
 
-// Which experts merge their last two units in the phases that merge: an odd count of three or more M-blocks whose
+// Which experts merge their last two units, in every row-space phase: an odd count of three or more M-blocks whose
 // last block is mostly padding (at most MERGE_TAIL_MAX rows).  Then the last unit (block + tail) is small, staging the
 // weights once for both units saves the larger half of the shared-memory traffic, and what the next item waits for, the epilogue
 // of the larger of the two tiles (gemm_roles.cuh, acc_claim), is short.  With a full last block (e.g. 384 rows) that costs
 // as much as the second weight pass or more: down was 5 % faster unmerged there, 257..320-row experts 6 % slower.
 constexpr int MERGE_TAIL_MAX = 64;
-// Do gate+up (op 0) and act_grad (op 1), whose reduction is K long, merge too?  128 + 160 tokens take 880 clocks a k-block as two
-// tiles (the loads of a small tile take longer than its products) and 595 as one item; what that exposes of gate+up's epilogue is
-// 3 us, of act_grad's 10.  gate+up gains at every K: forward over 64 experts of 300 rows, K = 512 118 -> 108 us, 1024 181 -> 169,
-// 2048 422 -> 383, 3072 471 -> 444 (below nine k-blocks, K = 256 68 -> 65, the numbers of work items are relied upon).  act_grad: a
-// step with K = 2048 1242 -> 1232 us, 3072 1349 -> 1332, even at 1024; K = 7168, 128 experts of 256 rows, both 10260 -> 10015.
-constexpr int MERGE_MIN_K_GATE_UP = 576, MERGE_MIN_K_ACT_GRAD = 2048;
-MOE_HD int phase_merges(int op, int K) { return K >= (op == 0 ? MERGE_MIN_K_GATE_UP : MERGE_MIN_K_ACT_GRAD); }
+// Merged against two items in gate+up (forward) and act_grad (backward), 64 experts of 300 rows, F = 1408, medians of 14 runs in
+// turn, us: d = 64 125 -> 107 forward; 256 132 -> 111 and 227 -> 207; 512 159 -> 136 and 313 -> 293; 1024 235 -> 217 and 473 -> 470;
+// 1536 even backward; 2048 428 -> 382 and 809 -> 801; 4096 1558 -> 1509 backward (quartiles of one side 1-2 % of these).  With
+// experts of 288 +- 17 rows, half of them merged, the same within 1 %.
 MOE_HD bool expert_merges(int rows, int mblocks) {
   return (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
 }
 
-// One work item of a row-space phase: a token tile (unit) of an expert and a column tile, or -- in the
-// phases that merge (down and gate_grad always, gate+up and act_grad by phase_merges), for an expert that merges
-// (expert_merges) -- its last two units under one k-loop.  `start[e]` = first unit (or first merged item) of expert e, `blk_expert[i]` =
-// expert of unit / item i (both from the layout kernels).
+// One work item of a row-space phase: a token tile (unit) of an expert and a column tile, or -- for an expert that merges
+// (expert_merges) -- its last two units under one k-loop.  `start[e]` = first item of a column tile of expert e, `blk_expert[i]` =
+// expert of item i (both from the layout kernels).
 struct SwapItem {
   int e, nb;            // expert, column tile
   int unit;             // first unit of the item
@@ -97,8 +93,7 @@ struct SwapItem {
   int mb_count;         // M-blocks of the item (both units): 1..3, contiguous
   int mb_count_a;       // M-blocks of the first unit
 };
-MOE_HD SwapItem decode_swap_item(int t, int n_tiles_n, bool merges, const int* start, const int* blk_expert,
-                                 const int* mb_start) {
+MOE_HD SwapItem decode_swap_item(int t, int n_tiles_n, const int* start, const int* blk_expert, const int* mb_start) {
   SwapItem it;
   const int e = blk_expert[t / n_tiles_n];
   const int ws = start[e];
@@ -110,7 +105,7 @@ MOE_HD SwapItem decode_swap_item(int t, int n_tiles_n, bool merges, const int* s
   it.e = e;
   it.unit = wi;
   // the item table has one entry fewer than the expert has units exactly when the expert merges
-  it.merged = (merges && wcount == ((mc + 1) >> 1) - 1 && wi == wcount - 1) ? 1 : 0;
+  it.merged = (wcount == ((mc + 1) >> 1) - 1 && wi == wcount - 1) ? 1 : 0;
   int f, c;
   balanced_unit(mc, wi, &f, &c);
   it.mb_first = mb_start[e] + f;
@@ -180,7 +175,6 @@ struct ChainParams {
   int n_phases;                 // 2 (forward) or 4 (backward)
   int ntn[SCHED_MAX_SEG];       // column tiles per item (row-space phases) / per strip (weight gradients)
   int strips[SCHED_MAX_SEG];    // weight-gradient phases: strips (256 rows of dW) per expert; else 0
-  int merges[SCHED_MAX_SEG];    // row-space phases: 1 if the phase merges the last two units of odd experts
   int dep_extra;                // test hook: added to the `activated` threshold (> 0 = never reached)
   int want_dw;                  // backward: routing-weight-gradient tasks are part of the vector queue
   int combine_split;            // combine tasks per token (column chunks)

@@ -61,7 +61,7 @@ def test_counts_on_tile_edges(d, F, serial):
     layer.close()
 
 
-@pytest.mark.parametrize("d", [568, 576, 2048])   # both sides of the lines from which gate+up and act_grad merge
+@pytest.mark.parametrize("d", [568, 576, 2048])
 @pytest.mark.parametrize("serial", [False, True])
 def test_merged_tiles_in_every_operator(d, serial):
     """Experts whose last two token tiles share a k-loop, of 257 to 320 rows and in a row of items: their accumulators take

@@ -15,13 +15,13 @@ def _lib():
 def _expected_items(counts, d, F, is_bwd):
     mblocks = (counts + 127) // 128
     units = (mblocks + 1) // 2
-    # an expert merges its last two units when its M-block count is odd, at least 3, and the last block holds <= 64 rows
+    # an expert merges its last two units, in every row-space phase, when its M-block count is odd, at least 3, and the last
+    # block holds <= 64 rows
     merged = units - ((mblocks % 2 == 1) & (mblocks >= 3) & (counts - (mblocks - 1) * 128 <= 64))
     Ep = len(counts)
-    first = merged if d >= (2048 if is_bwd else 576) else units   # gate+up and act_grad merge where their reduction is long
     if not is_bwd:
-        return int(first.sum()) * ((F + 127) // 128) + int(merged.sum()) * ((d + 255) // 256)
-    return (int(first.sum()) * ((F + 255) // 256) + Ep * ((d + 255) // 256) +
+        return int(merged.sum()) * ((F + 127) // 128 + (d + 255) // 256)
+    return (int(merged.sum()) * ((F + 255) // 256) + Ep * ((d + 255) // 256) +
             int(merged.sum()) * ((d + 255) // 256) + Ep * ((2 * F + 255) // 256))
 
 
@@ -35,7 +35,8 @@ def test_schedule_is_sound(is_bwd, workers):
         np.array([3000]),                              # a single expert
         np.zeros(6, int),                              # nothing routed at all
         np.full(64, 128),                              # exactly one M-block each
-        np.array([300, 257, 320, 577]),                # every expert ends in a merged item
+        np.array([300, 257, 320, 576]),                # every expert ends in a merged item
+        np.array([300, 257, 320, 577]),                # and its neighbour, whose last block holds 65 rows
         np.array([384, 321, 640, 385]),                # full last blocks / even counts: nothing merges
     ]
     d, F = 520, 272
@@ -47,8 +48,8 @@ def test_schedule_is_sound(is_bwd, workers):
 
 
 @pytest.mark.parametrize("is_bwd", [0, 1])
-@pytest.mark.parametrize("d", [568, 576, 2040, 2048, 7168])
-def test_first_operator_merges_where_its_reduction_is_long(is_bwd, d):
+@pytest.mark.parametrize("d", [8, 256, 568, 576, 2040, 2048, 7168])
+def test_every_operator_merges_at_every_reduction_length(is_bwd, d):
     counts = np.array([300, 257, 320, 577, 321, 384, 0, 64])
     rc, stats = binding.moe_debug_simulate_schedule(counts, 1111, 2, 0, d, 272, is_bwd, 74, 592)
     assert rc == 0 and stats[0] == _expected_items(counts, d, 272, is_bwd)
