@@ -256,13 +256,15 @@ constexpr int TK_RING = 8;
 // scheduler does it once, ahead of time, for every role of both CTAs).
 struct __align__(16) WorkDesc {
   int ticket;                                  // -1: the queue is empty
-  int phase, item, flags;                      // WD_MERGED, WD_READY
+  int phase, item, flags;                      // WD_READY
   int e, n0, nb, nkb;                          // strips: nb = 256-row block of dW, n0 = first column tile
-  int a_row0, a_ntok, a_mb_first, a_mb_count;  // strips: a_row0 = first padded row, a_ntok = rows of the expert
-  int b_row0, b_ntok, b_mb_first, b_mb_count;  // strips: b_row0 = end of the column tiles
+  int row0, ntok, ntok_b, nb1;                 // strips: ntok = rows of the expert, ntok_b = 0, nb1 = end of the column tiles
+  __device__ __forceinline__ int mb_first() const { return row0 / BLOCK_M; }              // M-blocks of the item's rows
+  __device__ __forceinline__ int mb_count() const { return mblocks_of(ntok + ntok_b); }
 };
-constexpr int WD_MERGED = 1, WD_READY = 2;   // READY: the dependent events were met when the item was published
-static_assert(sizeof(WorkDesc) == 64, "published as four 16-byte stores");
+constexpr int WD_READY = 1;   // the dependent events were met when the item was published
+constexpr int WD_PIECES = 3;
+static_assert(sizeof(WorkDesc) == 16 * WD_PIECES, "published as 16-byte stores");
 struct __align__(16) TicketRing {
   WorkDesc work[TK_RING];
   uint64_t full[TK_RING];    // in each CTA: the slot holds an item
@@ -272,17 +274,17 @@ struct __align__(16) TicketRing {
 constexpr int TK_CONSUMERS = 2 * (2 + EPI_WARPS) + 1;
 
 // The scheduler's `batch` groups of lanes (32 / batch lanes each) publish an item each, item n + group, as their slots come
-// free; `mine`: this group has an item.  Eight lanes store to both CTAs, one releases.
+// free; `mine`: this group has an item.  Three lanes store to each of the two CTAs, one releases.
 __device__ __forceinline__ bool ring_publish(TicketRing* r, uint32_t n, const WorkDesc& wd, bool mine, int group, int sub,
                                              uint32_t own /* the group's lanes */, const WaitCtl& wc) {
   const uint32_t it = n + group, slot = it % TK_RING;
   const uint4* src = reinterpret_cast<const uint4*>(&wd);
-  const uint4 piece = (sub & 3) == 0 ? src[0] : (sub & 3) == 1 ? src[1] : (sub & 3) == 2 ? src[2] : src[3];
+  const uint4 piece = (sub & 3) == 0 ? src[0] : (sub & 3) == 1 ? src[1] : src[2];
   uint64_t t0 = 0;
   for (uint32_t spin = 1;; ++spin) {
     const uint32_t free = __ballot_sync(0xffffffffu, mine && mbar_try_wait_cluster(&r->empty[slot], ((it / TK_RING) & 1) ^ 1));
     const bool go = (free & own) == own;   // every lane of the group has seen it
-    if (go && sub < 8) st_cluster_v4(map_to_rank(smem_u32(&r->work[slot]), sub >> 2) + 16 * (sub & 3), piece);
+    if (go && sub < 8 && (sub & 3) < WD_PIECES) st_cluster_v4(map_to_rank(smem_u32(&r->work[slot]), sub >> 2) + 16 * (sub & 3), piece);
     __syncwarp();
     if (go && sub == 0) {
       mbar_arrive_cluster_addr(map_to_rank(smem_u32(&r->full[slot]), 0));
@@ -315,45 +317,30 @@ __device__ __forceinline__ bool ring_take(TicketRing* r, uint32_t n, WorkDesc* w
   return true;
 }
 __device__ __forceinline__ SwapWork desc_swap_work(const WorkDesc& wd) {
-  SwapWork w;
-  w.merged = (wd.flags & WD_MERGED) != 0;
-  w.a.e = w.b.e = wd.e; w.a.n0 = w.b.n0 = wd.n0; w.a.nb = w.b.nb = wd.nb; w.a.nkb = w.b.nkb = wd.nkb;
-  w.a.row0 = wd.a_row0; w.a.ntok = wd.a_ntok; w.a.mb_first = wd.a_mb_first; w.a.mb_count = wd.a_mb_count;
-  w.b.row0 = wd.b_row0; w.b.ntok = wd.b_ntok; w.b.mb_first = wd.b_mb_first; w.b.mb_count = wd.b_mb_count;
-  return w;
+  return SwapWork{wd.e, wd.n0, wd.nb, wd.nkb, wd.row0, wd.ntok, wd.ntok_b};
 }
 __device__ __forceinline__ Strip desc_strip(const WorkDesc& wd) {
   Strip st;
-  st.e = wd.e; st.mp = wd.nb; st.row0 = wd.a_row0; st.rows = wd.a_ntok; st.nkb = wd.nkb;
-  st.nb0 = wd.n0; st.nb1 = wd.b_row0;
+  st.e = wd.e; st.mp = wd.nb; st.row0 = wd.row0; st.rows = wd.ntok; st.nkb = wd.nkb;
+  st.nb0 = wd.n0; st.nb1 = wd.nb1;
   return st;
 }
-__device__ __forceinline__ void pack_swap_work(WorkDesc& wd, const SwapWork& w) {
-  wd.flags = w.merged ? WD_MERGED : 0;
-  wd.e = w.a.e; wd.n0 = w.a.n0; wd.nb = w.a.nb; wd.nkb = w.a.nkb;
-  wd.a_row0 = w.a.row0; wd.a_ntok = w.a.ntok; wd.a_mb_first = w.a.mb_first; wd.a_mb_count = w.a.mb_count;
-  wd.b_row0 = w.b.row0; wd.b_ntok = w.b.ntok; wd.b_mb_first = w.b.mb_first; wd.b_mb_count = w.b.mb_count;
-}
-// Decode item `item` of phase `phase` (scheduler); *first / *count: the M-blocks whose dependent event it waits for.
+// Decode item `item` of phase `phase` (scheduler).
 template <bool BWD>
-__device__ __forceinline__ void decode_item(const FusedArgs& fa, int phase, int item, WorkDesc& wd, int* first, int* count) {
+__device__ __forceinline__ void decode_item(const FusedArgs& fa, int phase, int item, WorkDesc& wd) {
   const bool strip = BWD && (phase == 1 || phase == 3);
   if (strip) {
     const GemmArgs& a = fa.op[phase];
     const Strip st = decode_strip(a, item);
-    wd.flags = 0; wd.e = st.e; wd.n0 = st.nb0; wd.nb = st.mp; wd.nkb = st.nkb;
-    wd.a_row0 = st.row0; wd.a_ntok = st.rows; wd.a_mb_first = a.mb_start[st.e];
-    wd.a_mb_count = a.mb_start[st.e + 1] - a.mb_start[st.e];
-    wd.b_row0 = st.nb1;
-    wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
-    *first = wd.a_mb_first; *count = st.nkb > 0 ? wd.a_mb_count : 0;   // all rows of the expert
+    wd.e = st.e; wd.n0 = st.nb0; wd.nb = st.mp; wd.nkb = st.nkb;
+    wd.row0 = st.row0; wd.ntok = st.rows; wd.ntok_b = 0; wd.nb1 = st.nb1;   // all rows of the expert
     return;
   }
   SwapWork w;
   if (!BWD) w = phase == 0 ? decode_swap_work<GEMM_GATE_UP>(fa.op[0], item) : decode_swap_work<GEMM_DOWN>(fa.op[1], item);
   else w = phase == 0 ? decode_swap_work<GEMM_ACT_GRAD>(fa.op[0], item) : decode_swap_work<GEMM_GATE_GRAD>(fa.op[2], item);
-  pack_swap_work(wd, w);
-  *first = w.a.mb_first; *count = w.a.mb_count + w.b.mb_count;
+  wd.e = w.e; wd.n0 = w.n0; wd.nb = w.nb; wd.nkb = w.nkb;
+  wd.row0 = w.row0; wd.ntok = w.ntok; wd.ntok_b = w.ntok_b; wd.nb1 = 0;
 }
 
 // Items of each phase and their prefix sums: ticket t belongs to phase p iff start[p] <= t < start[p + 1].
@@ -416,39 +403,31 @@ __device__ __forceinline__ ChainDeps phase_deps(const FusedArgs& fa, int phase, 
 
 // ---------------------------------------------------------------- one item, by role
 template <bool BWD>
-__device__ __forceinline__ bool load_item(const FusedArgs& fa, int ring_of, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool load_item(const FusedArgs& fa, const GemmArgs::Ring ring, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                           LoaderState& ls, bool second_warp, int rank, int lane, const WaitCtl& wc,
                                           const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
   const bool strip = BWD && (phase == 1 || phase == 3);
   if (!(wd.flags & WD_READY) && (second_warp || strip)) {   // the item's dependent events (Section 4.3)
-    const int first = wd.a_mb_first, count = strip && wd.nkb == 0 ? 0 : wd.a_mb_count + wd.b_mb_count;
-    if (!dep.wait(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane, t)) return false;
+    const int first = wd.mb_first();
+    if (!dep.wait(first, wd.mb_count(), fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], lane, t)) return false;
   }
   if (strip)
     return wgrad_load_strip(fa.op[phase], smem, bars, ls, second_warp, rank, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
-  if (!BWD) {
-    if (phase == 0) return swap_load_item<GEMM_GATE_UP>(fa.op[0], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-    return swap_load_item<GEMM_DOWN>(fa.op[1], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-  }
-  if (phase == 0) return swap_load_item<GEMM_ACT_GRAD>(fa.op[0], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
-  return swap_load_item<GEMM_GATE_GRAD>(fa.op[2], ring_of, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  // one copy of the code for both operators of the pass: a launch over few tokens runs it once, from a cold instruction cache
+  const GemmMode mode = BWD ? GEMM_ACT_GRAD : phase == 0 ? GEMM_GATE_UP : GEMM_DOWN;   // gate_grad's weights lie like act_grad's
+  return swap_load_item(mode, fa.op[phase], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
 }
 template <bool BWD>
-__device__ __forceinline__ bool issue_item(const FusedArgs& fa, int ring_of, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
+__device__ __forceinline__ bool issue_item(const FusedArgs& fa, const GemmArgs::Ring ring, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
                                            uint32_t tmem_base, IssuerState& is, const WaitCtl& wc,
                                            const ChainDeps& dep) {
   const int phase = wd.phase, t = wd.item;
   if (BWD && (phase == 1 || phase == 3))
     return wgrad_issue_strip(fa.op[phase], smem, bars, tmem_base, is, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
-  if (!BWD) {
-    if (phase == 0) return swap_issue_item<GEMM_GATE_UP>(fa.op[0], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
-    return swap_issue_item<GEMM_DOWN>(fa.op[1], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
-  }
-  if (phase == 0) return swap_issue_item<GEMM_ACT_GRAD>(fa.op[0], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
-  return swap_issue_item<GEMM_GATE_GRAD>(fa.op[2], ring_of, smem, bars, tmem_base, is, wk, t, wc, dep);
+  return swap_issue_item<BWD>(ring, smem, bars, tmem_base, is, wk, t, wc, dep);
 }
 template <bool BWD>
 __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
@@ -466,6 +445,26 @@ __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDes
   if (phase == 0)
     return swap_epilogue_item<GEMM_ACT_GRAD>(fa.op[0], smem, bars, tmem_base, es, rank, ew, lane, wk, t, wc, dep);
   return swap_epilogue_item<GEMM_GATE_GRAD>(fa.op[2], smem, bars, tmem_base, es, rank, ew, lane, wk, t, wc, dep);
+}
+
+// A matrix role's walk over the pair's items in ticket order; `enter` at each phase boundary of the backward (gemm_roles.cuh): the
+// new phase's ring, of its own depth, starts at stage 0.  (The forward's two operators have one layout: the ring and the staging run
+// on.)  A loop for each role: in one for all of them every warp carried all roles' state, 14 registers of which act_grad's epilogue
+// has none to spare.
+template <bool BWD, class ENTER, class WORK>
+__device__ __forceinline__ bool walk_items(const FusedArgs& fa, TicketRing* ring, int lane, const WaitCtl& wc, const TraceCtl& tr,
+                                           ENTER enter, WORK work) {
+  int cur_phase = 0;
+  for (uint32_t n = 0;; ++n) {
+    WorkDesc wd;
+    if (!ring_take(ring, n, &wd, lane, wc)) return false;
+    if (wd.ticket < 0) return true;
+    if (BWD && wd.phase != cur_phase) {
+      cur_phase = wd.phase;
+      if (!enter(cur_phase)) return false;
+    }
+    if (!work(wd, phase_deps(fa, wd.phase, wc, tr))) return false;
+  }
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -540,12 +539,13 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
         wd.phase = phase_of(pt, t);
         wd.item = t - pt.start[wd.phase];
         if (rot.start[wd.phase]) wd.item = rotate_index(wd.item, rot.start[wd.phase], pt.start[wd.phase + 1] - pt.start[wd.phase]);
-        int first, count;
-        decode_item<BWD>(fa, wd.phase, wd.item, wd, &first, &count);
-        met = phase_deps(fa, wd.phase, wc, tr).met(first, count, fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], sub, lanes);
+        wd.flags = 0;
+        decode_item<BWD>(fa, wd.phase, wd.item, wd);
+        const int first = wd.mb_first();
+        met = phase_deps(fa, wd.phase, wc, tr).met(first, wd.mb_count(), fa.lv.counts[wd.e], first - fa.lv.mb_start[wd.e], sub, lanes);
       } else {
         wd.phase = wd.item = wd.flags = wd.e = wd.n0 = wd.nb = wd.nkb = 0;
-        wd.a_row0 = wd.a_ntok = wd.a_mb_first = wd.a_mb_count = wd.b_row0 = wd.b_ntok = wd.b_mb_first = wd.b_mb_count = 0;
+        wd.row0 = wd.ntok = wd.ntok_b = wd.nb1 = 0;
       }
       const uint32_t unmet = __ballot_sync(0xffffffffu, !met), own = (lanes == 32 ? ~0u : (1u << lanes) - 1u) << (group * lanes);
       if (wd.ticket >= 0 && (unmet & own) == 0) wd.flags |= WD_READY;
@@ -558,50 +558,42 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       phase = __shfl_sync(0xffffffffu, wd.phase, 31);
       batch = 1 << ((batches >> (2 * phase)) & 3);
     }
-  } else if (warp < GEMM_ROLE_WARPS && warp != SCHED_WARP && !(warp == 1 && rank != 0)) {
+  } else if (warp == 0 || warp == 6) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
-    const int ring_of = which_ring(fa.op[0]);
+    const GemmArgs::Ring op_ring = which_ring(fa.op[0]);   // the operators of a pass have the same staging, and the same rings
     LoaderState ls;
+    walk_items<BWD>(fa, ring, lane, wc, tr, [&](int phase) { return loader_enter_phase(bars, ls, phase, wc); },
+                    [&](const WorkDesc& wd, const ChainDeps& dep) {
+                      return load_item<BWD>(fa, op_ring, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
+                    });
+  } else if (warp == 1 && rank == 0) {
+    const GemmArgs::Ring op_ring = which_ring(fa.op[0]);
     IssuerState is;
+    const bool ok = walk_items<BWD>(fa, ring, lane, wc, tr, [&](int) { is.s = is.a_s = 0; return true; },
+                                    [&](const WorkDesc& wd, const ChainDeps& dep) {
+                                      return issue_item<BWD>(fa, op_ring, wd, smem, bars, tmem_base, is, wc, dep);
+                                    });
+    if (uniform(!ok || *reinterpret_cast<volatile int*>(&fa.status->abort) ? 1 : 0)) issuer_drain(bars, fa.status);
+  } else if (is_epilogue_warp(warp)) {
+    const int ew = epilogue_index(warp);
     EpiState es;
-    int cur_phase = 0;
-    bool ok = true;
-    for (uint32_t n = 0; ok; ++n) {
-      WorkDesc wd;
-      ok = ring_take(ring, n, &wd, lane, wc);
-      if (!ok || wd.ticket < 0) break;
-      const int phase = wd.phase;
-      const ChainDeps dep = phase_deps(fa, phase, wc, tr);
-      // the forward's two operators have one layout: the ring and the staging run on
-      // ---- phase boundary of the backward (gemm_roles.cuh): the new phase's ring, of its own depth, starts at stage 0
-      if (BWD && phase != cur_phase) {
-        cur_phase = phase;
-        if (warp == 0 || warp == 6) {
-          if (!loader_enter_phase(bars, ls, phase, wc)) break;
-        } else if (warp == 1) {
-          is.s = is.a_s = 0;
-        } else {
-          int go = 1;
-          if (lane == 0) {
-            tma_store_wait_read();
-            epi_enter_phase(bars, epilogue_index(warp), phase);
-            go = phase_wait(bars, phase, wc) ? 1 : 0;
-          }
-          if (!__shfl_sync(0xffffffffu, go, 0)) break;
-        }
-      }
-      if (warp == 0 || warp == 6)
-        ok = load_item<BWD>(fa, ring_of, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
-      else if (warp == 1)
-        ok = issue_item<BWD>(fa, ring_of, wd, smem, bars, tmem_base, is, wc, dep);
-      else
-        ok = epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, epilogue_index(warp), lane, wc, dep);
-    }
-    if (is_epilogue_warp(warp) && lane == 0) {
+    walk_items<BWD>(fa, ring, lane, wc, tr,
+                    [&](int phase) {
+                      int go = 1;
+                      if (lane == 0) {
+                        tma_store_wait_read();
+                        epi_enter_phase(bars, ew, phase);
+                        go = phase_wait(bars, phase, wc) ? 1 : 0;
+                      }
+                      return __shfl_sync(0xffffffffu, go, 0) != 0;
+                    },
+                    [&](const WorkDesc& wd, const ChainDeps& dep) {
+                      return epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, ew, lane, wc, dep);
+                    });
+    if (lane == 0) {
       tma_store_wait_all();
-      epi_enter_phase(bars, epilogue_index(warp), SCHED_MAX_SEG);   // nothing of this warp is left in shared memory
+      epi_enter_phase(bars, ew, SCHED_MAX_SEG);   // nothing of this warp is left in shared memory
     }
-    if (warp == 1 && uniform(!ok || *reinterpret_cast<volatile int*>(&fa.status->abort) ? 1 : 0)) issuer_drain(bars, fa.status);
   }
 
   // ------------------------------------------------ vector workers: the dedicated warps from the start, the

@@ -215,8 +215,8 @@ constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_
 __host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return EPI_WARPS * (size_t)sw_staging_bytes(mode); }
 __host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
 // The same for every role and item of a launch: the layout is complete before them.
-__device__ __forceinline__ int which_ring(const GemmArgs& a) {
-  return uniform(a.meta[7] <= a.ring_rows ? 0 : a.meta[3] == a.meta[4] ? 1 : 2);
+__device__ __forceinline__ GemmArgs::Ring which_ring(const GemmArgs& a) {
+  return a.ring[uniform(a.meta[7] <= a.ring_rows ? 0 : a.meta[3] == a.meta[4] ? 1 : 2)];
 }
 // does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
 __device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s) {
@@ -225,20 +225,19 @@ __device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s)
 }
 // TMA producers (both CTAs) of item t.  tok_warp = false: the weights and the stage's byte count; true: the
 // tokens.
-template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_load_item(const GemmArgs& a, int ring_of, uint8_t* smem, PipeBarriers* bars, LoaderState& ls,
-                                               bool tok_warp, int rank, int lane, const SwapWork& wk, int t,
+template <class DEP>
+__device__ __forceinline__ bool swap_load_item(GemmMode mode, const GemmArgs& a, const GemmArgs::Ring ring, uint8_t* smem,
+                                               PipeBarriers* bars, LoaderState& ls, bool tok_warp, int rank, int lane, const SwapWork& wk, int t,
                                                const WaitCtl& wc, const DEP& dep) {
-  const GemmArgs::Ring ring = a.ring[ring_of];
   const int stages = ring.stages, tokb = ring.tok_bytes;
   uint8_t* sW = smem;                              // [stages][16 KB] weights
   uint8_t* sT = smem + stages * W_STAGE_BYTES;     // [stages][tokb] tokens (this CTA's half)
   // with events: the tokens are there (acquired by the scheduler and handed on through the ticket ring, or by the caller);
   // what the producers wrote must be seen by the TMA loads
   if (DEP::kOn && tok_warp) fence_proxy_async_global();
-  const int nkb = uniform(wk.a.nkb), e = uniform(wk.a.e), n0 = uniform(wk.a.n0);
-  const int row_a = uniform(wk.a.row0), half_a = uniform(wk.a.ntok) >> 1;
-  const int row_b = uniform(wk.b.row0), half_b = wk.merged ? uniform(wk.b.ntok) >> 1 : 0;
+  const int nkb = uniform(wk.nkb), e = uniform(wk.e), n0 = uniform(wk.n0);
+  const int row_a = uniform(wk.row0), half_a = uniform(wk.ntok) >> 1;
+  const int row_b = row_a + 2 * half_a, half_b = uniform(wk.ntok_b) >> 1;
   for (int kb = 0; kb < nkb; ++kb) {
     if (!mbar_wait_warp(&bars->empty[ls.s], (ls.empty_par >> ls.s) & 1, wc, SITE_EMPTY, t, 50)) return false;
     ls.empty_par ^= 1u << ls.s;
@@ -247,7 +246,7 @@ __device__ __forceinline__ bool swap_load_item(const GemmArgs& a, int ring_of, u
       ls.guard = 0;
     }
     if (!tok_warp) {
-      load_weights_swap<MODE>(a, e, n0, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], 2 * (half_a + half_b));
+      load_weights_swap(mode, a, e, n0, kb, rank, sW + ls.s * W_STAGE_BYTES, &bars->full[ls.s], 2 * (half_a + half_b));
     } else {
       load_tokens_swap(a, row_a, half_a, kb, rank, sT + ls.s * tokb, &bars->full[ls.s]);
       if (half_b)   // the second token tile, behind the first in the stage
@@ -281,23 +280,22 @@ __device__ __forceinline__ bool acc_claim(PipeBarriers* bars, IssuerState& is, i
 
 // MMA issuer: warp 1 of the even CTA.  The whole warp walks the loop with uniform control flow and operands; one elected
 // lane issues (common.cuh).
-template <int MODE, class DEP>
-__device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, int ring_of, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
+template <bool W_MN, class DEP>
+__device__ __forceinline__ bool swap_issue_item(const GemmArgs::Ring ring, uint8_t* smem, PipeBarriers* bars, uint32_t tmem_base,
                                                 IssuerState& is, const SwapWork& wk, int t, const WaitCtl& wc,
                                                 const DEP& dep) {
-  const GemmArgs::Ring ring = a.ring[ring_of];
   const uint32_t stages = ring.stages, t_step = ring.tok_bytes >> 4;
-  const uint32_t w_lo0 = swap_w_desc_lo<MODE>(smem_u32(smem));
+  const uint32_t w_lo0 = swap_w_desc_lo<W_MN>(smem_u32(smem));
   const uint32_t t_lo0 = smem_desc_lo(smem_u32(smem + stages * W_STAGE_BYTES), 16);
   uint32_t w_lo = w_lo0 + is.s * (W_STAGE_BYTES >> 4), t_lo = t_lo0 + is.s * t_step;
-  const int nkb = uniform(wk.a.nkb), ntok = uniform(wk.a.ntok), ntok_b = uniform(wk.merged ? wk.b.ntok : 0);
+  const int nkb = uniform(wk.nkb), ntok = uniform(wk.ntok), ntok_b = uniform(wk.ntok_b);
   // a merged item's second tile is the larger one: the first in the accumulators
   const int n0 = ntok_b ? ntok_b : ntok, n1 = ntok_b ? ntok : 0;
   if (!acc_claim(bars, is, n0, n1, wc, t)) return false;
   tc_fence_after_sync();
   const uint32_t d_first = uniform(tmem_base + acc_column(is.end, 0, n0, n1));
   const uint32_t d_tmem = uniform(ntok_b ? tmem_base + acc_column(is.end, 1, n0, n1) : d_first);
-  const uint32_t idesc = swap_idesc<MODE>(ntok), idesc_b = swap_idesc<MODE>(ntok_b ? ntok_b : TOK_GRAIN);
+  const uint32_t idesc = swap_idesc<W_MN>(ntok), idesc_b = swap_idesc<W_MN>(ntok_b ? ntok_b : TOK_GRAIN);
   const uint32_t t_off_b = (uint32_t)((ntok >> 1) * (BK * 2)) >> 4;
   uint64_t t0 = 0;
   for (int kb = 0; kb < nkb; ++kb) {
@@ -305,8 +303,8 @@ __device__ __forceinline__ bool swap_issue_item(const GemmArgs& a, int ring_of, 
     is.full_par ^= 1u << is.s;
     if (DEP::kOn && kb == 0 && dep.tracing()) t0 = globaltimer_ns();
     tc_fence_after_sync();
-    mma_kblock_swap<MODE>(d_tmem, w_lo, t_lo, idesc, kb == 0);
-    if (ntok_b) mma_kblock_swap<MODE>(d_first, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
+    mma_kblock_swap<W_MN>(d_tmem, w_lo, t_lo, idesc, kb == 0);
+    if (ntok_b) mma_kblock_swap<W_MN>(d_first, w_lo, t_lo + t_off_b, idesc_b, kb == 0);
     tc_commit_pair(&bars->empty[is.s]);   // frees the stage in both CTAs
     if (++is.s == stages) {
       is.s = 0; w_lo = w_lo0; t_lo = t_lo0;
@@ -330,9 +328,14 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
                                                    uint32_t tmem_base, EpiState& es, int rank, int ew, int lane,
                                                    const SwapWork& wk, int t, const WaitCtl& wc, const DEP& dep) {
   uint8_t* staging = smem + staging_at((GemmMode)MODE) + ew * sw_staging_bytes((GemmMode)MODE);
-  const int n0 = wk.merged ? wk.b.ntok : wk.a.ntok, n1 = wk.merged ? wk.a.ntok : 0;
-  for (int part = 0; part < (wk.merged ? 2 : 1); ++part) {   // a merged item is two tiles here, the larger one first
-    const SwapTile& st = part == 0 && wk.merged ? wk.b : wk.a;
+  const bool merged = wk.ntok_b != 0;
+  for (int part = 0; part < (merged ? 2 : 1); ++part) {   // a merged item is two tiles here, the larger one -- the second -- first
+    SwapTile st{wk.row0, wk.ntok, wk.n0, wk.nb};
+    int acc = acc_column(es.end, 0, st.ntok, 0);
+    if (merged) {
+      acc = acc_column(es.end, part, wk.ntok_b, wk.ntok);
+      if (part == 0) { st.row0 += wk.ntok; st.ntok = wk.ntok_b; }
+    }
     const int as = 2 * es.end + part;
     uint64_t t0 = 0;
     auto ready = [&]() {
@@ -342,7 +345,7 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
       tc_fence_after_sync();
       return true;
     };
-    if (!epilogue_swap<MODE>(a, st, tmem_base + acc_column(es.end, part, n0, n1), rank, ew, lane, staging, ready)) return false;
+    if (!epilogue_swap<MODE>(a, st, tmem_base + acc, rank, ew, lane, staging, ready)) return false;
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) {
@@ -356,7 +359,7 @@ __device__ __forceinline__ bool swap_epilogue_item(const GemmArgs& a, uint8_t* s
       }
       mbar_arrive_leader(&bars->tmem_empty[as]);
       if (DEP::kOn) {
-        if (last) dep.signal(st.mb_first, st.mb_count);
+        if (last) dep.signal(st.row0 / BLOCK_M, mblocks_of(st.ntok));
         if (ew == 0 && dep.tracing()) dep.trace(TR_EPI, t, t0, t0, globaltimer_ns());
       }
     }

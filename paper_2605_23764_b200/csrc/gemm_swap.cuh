@@ -18,27 +18,22 @@ constexpr int TOK_GRAIN = 32;                    // tokens per tile: a multiple 
 constexpr int W_STAGE_BYTES = A_STAGE_BYTES;     // 128 weight rows (or 2 MN-major boxes) x 64 k: 16 KB
 
 struct SwapTile {
-  int e;      // expert
-  int row0;   // first padded row of the tile's tokens
+  int row0;   // first padded row of the tile's tokens, a multiple of BLOCK_M
   int ntok;   // tokens (accumulator columns) of the tile, multiple of TOK_GRAIN
   int n0;     // first output feature of the pair (GATE_UP: of the 128 gate/up feature pairs)
   int nb;     // feature-tile index
-  int nkb;    // k-blocks
-  int mb_first, mb_count;   // the tile's M-blocks (its event counters)
 };
+// M-blocks of `rows` consecutive rows from the first row of an M-block on (their event counters)
+__device__ __forceinline__ int mblocks_of(int rows) { return (rows + BLOCK_M - 1) / BLOCK_M; }
 
 // Features per pair tile: GATE_UP holds 64 gate + 64 up rows per CTA = 128 features per pair.
 template <int MODE>
 __device__ __forceinline__ int swap_tile_features() { return MODE == GEMM_GATE_UP ? 128 : 256; }
 
-// Tokens of the unit of M-blocks [first, first + count) (relative to the expert's first M-block) of expert e,
+// Tokens of the unit of M-blocks [first, first + count) (relative to the expert's first M-block) of an expert of `rows` rows,
 // cut at the expert's last 32-row group.
-__device__ __forceinline__ void unit_tokens(const GemmArgs& a, int e, int first, int count, int* row0, int* ntok) {
-  const int n32 = (a.counts[e] + TOK_GRAIN - 1) & ~(TOK_GRAIN - 1);
-  int end = (first + count) * BLOCK_M;
-  if (end > n32) end = n32;
-  *row0 = (a.mb_start[e] + first) * BLOCK_M;
-  *ntok = end - first * BLOCK_M;
+__device__ __forceinline__ int unit_tokens(int rows, int first, int count) {
+  return min((first + count) * BLOCK_M, (rows + TOK_GRAIN - 1) & ~(TOK_GRAIN - 1)) - first * BLOCK_M;
 }
 
 // One work item of a row-space operator: a token tile, or -- for an expert that merges (schedule.h) -- its last two token
@@ -46,8 +41,9 @@ __device__ __forceinline__ void unit_tokens(const GemmArgs& a, int e, int first,
 // both token tiles into two accumulators (shared-memory traffic bounds these kernels, and the
 // weights are the larger half of it).  For the epilogue warps the item is two tiles.
 struct SwapWork {
-  SwapTile a, b;
-  bool merged;
+  int e, n0, nb, nkb;   // expert, tile of features as in SwapTile, k-blocks
+  int row0;             // first padded row
+  int ntok, ntok_b;     // tokens of the tile; of the second one, whose rows follow (then ntok is BLOCK_M), 0 if the item is one tile
 };
 __device__ __forceinline__ int total_swap_work(const GemmArgs& a) { return a.meta[4] * a.n_tiles_n; }
 
@@ -57,17 +53,14 @@ template <int MODE>
 __device__ __forceinline__ SwapWork decode_swap_work(const GemmArgs& a, int t) {
   const SwapItem it = decode_swap_item(t, a.n_tiles_n, a.work_start, a.wblk_expert, a.mb_start);
   SwapWork w;
-  w.merged = it.merged != 0;
-  w.a.e = w.b.e = it.e;
-  w.a.nb = w.b.nb = it.nb;
-  w.a.n0 = w.b.n0 = it.nb * swap_tile_features<MODE>();
-  w.a.nkb = w.b.nkb = (a.K + BK - 1) / BK;
-  const int rel = it.mb_first - a.mb_start[it.e];
-  unit_tokens(a, it.e, rel, it.mb_count_a, &w.a.row0, &w.a.ntok);
-  w.a.mb_first = it.mb_first; w.a.mb_count = it.mb_count_a;
-  w.b.row0 = 0; w.b.ntok = 0;
-  w.b.mb_first = it.mb_first + it.mb_count_a; w.b.mb_count = it.mb_count - it.mb_count_a;
-  if (w.merged) unit_tokens(a, it.e, rel + it.mb_count_a, w.b.mb_count, &w.b.row0, &w.b.ntok);
+  w.e = it.e;
+  w.nb = it.nb;
+  w.n0 = it.nb * swap_tile_features<MODE>();
+  w.nkb = (a.K + BK - 1) / BK;
+  w.row0 = it.mb_first * BLOCK_M;
+  const int rel = it.mb_first - a.mb_start[it.e], rows = a.counts[it.e];
+  w.ntok = unit_tokens(rows, rel, it.mb_count_a);
+  w.ntok_b = it.merged ? unit_tokens(rows, rel + it.mb_count_a, it.mb_count - it.mb_count_a) : 0;
   return w;
 }
 
@@ -82,17 +75,16 @@ __device__ __forceinline__ void load_tokens_swap(const GemmArgs& a, int row0, in
   // half: a multiple of 16, at most 128: one box of exactly that many rows
   tma_load_2d_pair(sT, &a.tmTok[(half >> 4) - 1], kb * BK, row0 + rank * half, bar);
 }
-template <int MODE>
-__device__ __forceinline__ void load_weights_swap(const GemmArgs& a, int e, int n0, int kb, int rank, uint8_t* sW,
+__device__ __forceinline__ void load_weights_swap(GemmMode mode, const GemmArgs& a, int e, int n0, int kb, int rank, uint8_t* sW,
                                                   uint64_t* bar, int ntok_total) {
   const int k0 = kb * BK;
   if (rank == 0) mbar_expect_tx_elect(bar, swap_stage_tx_bytes(ntok_total));
   const int brow = e * a.b_rows_per_expert;
-  if (MODE == GEMM_GATE_UP) {
+  if (mode == GEMM_GATE_UP) {
     // one box [8 groups][gate | up][8 rows][64 k]: per group of 8 features the 8 gate rows, then the 8 up rows
     // (W_gate_up viewed as [Ep][F/8][2][8][d]); groups beyond F read as zeros
     tma_load_5d_pair(sW, &a.tmB, k0, 0, 0, (n0 + rank * 64) >> 3, e, bar);
-  } else if (MODE == GEMM_DOWN) {
+  } else if (mode == GEMM_DOWN) {
     tma_load_2d_pair(sW, &a.tmB, k0, brow + n0 + rank * 128, bar);
   } else {
     // ACT_GRAD / GATE_GRAD: the forward weight read along its rows -> two MN-major [64 k][64 features] boxes
@@ -103,21 +95,18 @@ __device__ __forceinline__ void load_weights_swap(const GemmArgs& a, int e, int 
 
 // One 64-deep k-block: D[256 features x ntok tokens] (+)= W . X^T.  w_lo / t_lo: low descriptor words of
 // the stage's weight and token tiles (smem_desc_lo).
-template <int MODE>
+template <bool W_MN>   // act_grad, gate_grad: the forward weights read along their rows
 __device__ __forceinline__ void mma_kblock_swap(uint32_t d_tmem, uint32_t w_lo, uint32_t t_lo, uint32_t idesc,
                                                 bool first_kblock) {
-  constexpr bool W_MN = (MODE == GEMM_ACT_GRAD || MODE == GEMM_GATE_GRAD);
   // 16 k-rows of an MN-major box / 32 bytes of a K-major row
   tc_mma4_bf16_pair<W_MN ? (2048 >> 4) : (32 >> 4), (32 >> 4)>(d_tmem, w_lo, t_lo, smem_desc_hi(1024), idesc, !first_kblock);
 }
-template <int MODE>
+template <bool W_MN>
 __device__ __forceinline__ uint32_t swap_w_desc_lo(uint32_t w_addr) {
-  constexpr bool W_MN = (MODE == GEMM_ACT_GRAD || MODE == GEMM_GATE_GRAD);
   return smem_desc_lo(w_addr, W_MN ? MN_BOX_BYTES : 16);
 }
-template <int MODE>
+template <bool W_MN>
 __device__ __forceinline__ uint32_t swap_idesc(int ntok) {
-  constexpr bool W_MN = (MODE == GEMM_ACT_GRAD || MODE == GEMM_GATE_GRAD);
   return make_idesc_bf16(2 * BLOCK_M, ntok, W_MN ? 1 : 0, 0);
 }
 

@@ -47,14 +47,15 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
   // Items pair, pair + npairs, ..; each role decodes item i + 1 before it works on item i (the decode's chain of
   // global loads then completes behind the item's work).
   const int total = total_swap_work(a);
-  const int ring = which_ring(a);
+  const GemmArgs::Ring ring = which_ring(a);
+  constexpr bool W_MN = MODE == GEMM_ACT_GRAD || MODE == GEMM_GATE_GRAD;
   SwapWork cur, next;
   if (pair < total) cur = decode_swap_work<MODE>(a, pair);
   if (warp == 0 || warp == 6) {
     LoaderState ls;
     for (int t = pair; t < total; t += npairs, cur = next) {
       if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-      if (!swap_load_item<MODE>(a, ring, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
+      if (!swap_load_item((GemmMode)MODE, a, ring, smem, bars, ls, warp == 6, rank, lane, cur, t, wc, dep)) break;
     }
   } else if (warp == 1) {
     if (rank == 0) {
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
       bool ok = true;
       for (int t = pair; t < total && ok; t += npairs, cur = next) {
         if (t + npairs < total) next = decode_swap_work<MODE>(a, t + npairs);
-        ok = swap_issue_item<MODE>(a, ring, smem, bars, tmem_base, is, cur, t, wc, dep);
+        ok = swap_issue_item<W_MN>(ring, smem, bars, tmem_base, is, cur, t, wc, dep);
       }
       if (uniform(!ok || *reinterpret_cast<volatile int*>(&a.status->abort) ? 1 : 0)) issuer_drain(bars, a.status);
     }

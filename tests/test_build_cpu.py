@@ -1,6 +1,7 @@
 """The build: the library comes out without the accelerator of the Python calls."""
 import ctypes
 import os
+import re
 import shutil
 
 import pytest
@@ -50,3 +51,13 @@ def test_accelerator_of_another_torch_or_python_is_not_taken(monkeypatch):
     with monkeypatch.context() as m:
         m.setattr(binding.sysconfig, "get_config_var", lambda name: ".cpython-399-other.so")
         assert build._stale(build.fastcall_path()) and binding._load_fastcall() is None
+
+
+def test_persistent_kernels_hardly_spill():
+    """The backward's epilogue takes every register of the 128 a thread has: what a role carries besides it spills, and 32 bytes of
+    that made a backward over a thousand tokens 4 % slower.  At most 16 bytes; the forward none."""
+    build.build()
+    with open(os.path.join(build.OBJ, "fused.o.log")) as f:
+        log = f.read()
+    spills = {m[0]: int(m[1]) for m in re.findall(r"fused_chain_kernelILb(\d)E.*?\n.*?(\d+) bytes spill stores", log)}
+    assert spills["0"] == 0 and spills["1"] <= 16, spills
