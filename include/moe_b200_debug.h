@@ -59,6 +59,10 @@ int moe_debug_set_plain_launch(moe_ctx* ctx, int32_t on);
  * that many blocks (given that the device can hold one: fits8, fits16), 0 = the kernels over all SMs.  Host only. */
 int moe_debug_layout_blocks(int32_t T, int32_t kp, int32_t Ep, int32_t fits8, int32_t fits16);
 
+/* The operand ring of the row-space operators of a pass over T tokens whose largest expert has `largest` rows; merged: one of its
+ * experts has two token tiles in one item.  Its stages, and the tokens each holds for a CTA pair.  Host only. */
+int moe_debug_ring(int32_t is_bwd, int32_t T, int32_t largest, int32_t merged, int32_t* stages, int32_t* tokens);
+
 /* 1 if the kernels of the host-buffer calls read or write this host buffer in place (pinned or registered memory, in one
  * piece), 0 if it is copied. */
 int moe_debug_host_direct(const void* p, size_t bytes);

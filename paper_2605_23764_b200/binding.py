@@ -28,7 +28,7 @@ EXPORTS = ["moe_workspace_bytes", "moe_create", "moe_destroy", "moe_route", "moe
            "moe_set_wait_budget_ms", "moe_debug_buffer", "moe_strerror", "moe_last_cuda_error",
            "moe_set_profiling", "moe_get_phase_ms", "moe_route_host", "moe_layout_noalloc",
            "moe_debug_simulate_schedule", "moe_debug_set_unreachable_dependency", "moe_debug_trace", "moe_debug_set_plain_launch",
-           "moe_debug_host_direct", "moe_debug_layout_blocks",
+           "moe_debug_host_direct", "moe_debug_layout_blocks", "moe_debug_ring",
            "moe_sched_study_workspace_bytes", "moe_sched_study", "moe_sched_study_stats", "moe_router_fwd",
            "moe_router_bwd", "moe_taskflow_compile", "moe_taskflow_workspace_bytes", "moe_taskflow_run",
            "moe_taskflow_status", "moe_ep_plan", "moe_ep_dispatch", "moe_ep_combine"]
@@ -163,6 +163,7 @@ def load_library() -> ctypes.CDLL:
     lib.moe_debug_set_plain_launch.argtypes = [vp, i32]
     lib.moe_debug_host_direct.argtypes = [vp, sz]
     lib.moe_debug_layout_blocks.argtypes = [i32] * 5
+    lib.moe_debug_ring.argtypes = [i32] * 4 + [ctypes.POINTER(i32)] * 2
     lib.moe_router_fwd.argtypes = [vp, vp, vp, i32, vp, vp, vp, vp, vp]
     lib.moe_router_bwd.argtypes = [vp, vp, vp, vp, i32, vp, vp]
     lib.moe_taskflow_compile.argtypes = [ctypes.POINTER(MoeTfTensor), i32, ctypes.POINTER(MoeTfOperator), i32, i32,
@@ -676,6 +677,14 @@ def moe_debug_set_plain_launch(ctx, on: bool):
 
 def moe_debug_layout_blocks(T, kp, Ep, fits8=True, fits16=True) -> int:
     return int(load_library().moe_debug_layout_blocks(T, kp, Ep, int(fits8), int(fits16)))
+
+
+def moe_debug_ring(is_bwd, T, largest, merged=False):
+    """(stages, tokens of a stage) of the row-space operators' operand ring"""
+    stages, tokens = ctypes.c_int32(), ctypes.c_int32()
+    _check(load_library().moe_debug_ring(int(is_bwd), T, largest, int(merged), ctypes.byref(stages), ctypes.byref(tokens)),
+           "moe_debug_ring")
+    return stages.value, tokens.value
 
 
 def moe_debug_host_direct(ptr: int, nbytes: int) -> bool:

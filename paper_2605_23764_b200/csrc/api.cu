@@ -1181,6 +1181,17 @@ int moe_debug_buffer(moe_ctx* c, int which, void** ptr, size_t* elems) {
   return MOE_OK;
 }
 
+// The operand ring of the row-space operators of a pass: stages, and tokens of a stage.
+int moe_debug_ring(int32_t is_bwd, int32_t T, int32_t largest, int32_t merged, int32_t* stages, int32_t* tokens) {
+  if (!stages || !tokens || T < 0) return MOE_ERR_INVALID_ARG;
+  GemmArgs g{};
+  plan_ring(is_bwd ? GEMM_ACT_GRAD : GEMM_GATE_UP, T, g);
+  const GemmArgs::Ring r = g.ring[ring_choice(largest, g.ring_rows[0], g.ring_rows[1], merged != 0)];
+  *stages = r.stages;
+  *tokens = r.tok_bytes / 64;   // 64 two-byte elements of half the tokens in each CTA
+  return MOE_OK;
+}
+
 // Host-only check of the static schedule (no GPU needed): builds the layout tables and the per-pair
 // matrix queues for the given per-expert row counts and lets `pairs` matrix workers (each walking its
 // own statically ordered queue) and `vec_workers` vector workers (tickets) run, each blocking on its

@@ -202,10 +202,9 @@ struct ChainDeps {
 // Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes], and at
 // the end of LAYOUT_BYTES the staging.  What the token stages do not need goes into more stages: the loads of a k-block take
 // about 2400 clocks, so that five stages bound a tile of 128 tokens at 480 clocks a k-block, whose products take 256; and a
-// pass over few tokens is a stream of weights from HBM (32 tokens: eleven stages, 198 KB in flight instead of 80).  Three rings
-// come from the host, for tiles of up to 128 tokens (or the call's tokens, if fewer), of 256, and for merged items of 320; the
-// layout leaves the rows of the largest expert in meta[7] and what merges in meta[3], meta[4], and every role finds the same
-// one.  (Worked out in the kernel for every item, passes of short items took 1-3 % longer; stages as large as their own tile,
+// pass over few tokens is a stream of weights from HBM (32 tokens: eleven stages, 198 KB in flight instead of 80).  The rings
+// come from the host (schedule.h, ring_rows); the layout leaves the rows of the largest expert in meta[7] and what merges in
+// meta[3], meta[4], and every role finds the same one.  (Worked out in the kernel for every item, passes of short items took 1-3 % longer; stages as large as their own tile,
 // in a ring of bytes, cost the loaders more than the depth gave.)
 // Against two rings, one for calls of up to 256 tokens: 4096 tokens x 8, 256 experts, 7168 x 2048: 4968 -> 4877 us (six stages for
 // five); 2048 x 4, 128 experts, 4096 x 1536: 894 -> 864 (eight); 512 x 6 + 2, 64 experts, 2048 x 1408: 236 -> 233.
@@ -216,7 +215,8 @@ __host__ __device__ constexpr size_t swap_staging_bytes(GemmMode mode) { return 
 __host__ __device__ constexpr size_t staging_at(GemmMode mode) { return (LAYOUT_BYTES - swap_staging_bytes(mode)) & ~size_t(127); }
 // The same for every role and item of a launch: the layout is complete before them.
 __device__ __forceinline__ GemmArgs::Ring which_ring(const GemmArgs& a) {
-  return a.ring[uniform(a.meta[7] <= a.ring_rows ? 0 : a.meta[3] == a.meta[4] ? 1 : 2)];
+  const int tiles = a.meta[3], items = a.meta[4], largest = a.meta[7];
+  return a.ring[uniform(ring_choice(largest, a.ring_rows[0], a.ring_rows[1], tiles != items))];
 }
 // does stage s (its weights or its tokens) reach above WGRAD_STAGING_AT?
 __device__ __forceinline__ bool above_guard(const GemmArgs::Ring& r, uint32_t s) {

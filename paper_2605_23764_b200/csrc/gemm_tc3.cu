@@ -87,15 +87,14 @@ __global__ void __launch_bounds__(GEMM3_THREADS, 1) grouped_gemm_swap_kernel(con
 }
 
 void plan_ring(GemmMode mode, int T, GemmArgs& a) {
-  auto of = [&](int tok_bytes) {
+  auto of = [&](int tokens) {   // half of them in each CTA
+    const int tok_bytes = tokens / 2 * BK * 2;
     const int stages = (int)((LAYOUT_BYTES - swap_staging_bytes(mode)) / (W_STAGE_BYTES + tok_bytes));
     return GemmArgs::Ring{stages < MAX_STAGES ? stages : MAX_STAGES, tok_bytes};
   };
-  const int rows = (T + TOK_GRAIN - 1) / TOK_GRAIN * TOK_GRAIN;
-  a.ring_rows = rows < BLOCK_M ? rows : BLOCK_M;
-  a.ring[0] = of(a.ring_rows / 2 * BK * 2);
-  a.ring[1] = of(BLOCK_M * BK * 2);
-  a.ring[2] = of(3 * BLOCK_M / 2 * BK * 2);
+  for (int i = 0; i < 2; ++i) a.ring[i] = of(a.ring_rows[i] = ring_rows(T, i));
+  a.ring[2] = of(2 * BLOCK_M);
+  a.ring[3] = of(MERGED_TOKENS_MAX);
 }
 
 template <int MODE>

@@ -139,8 +139,8 @@ struct GemmArgs {
   int F;               // intermediate size (GATE_UP / ACT_GRAD epilogues)
   // row-space modes: operand stages and the token bytes of a stage per CTA (gemm_roles.cuh, plan_ring) ..
   struct Ring { int stages, tok_bytes; };
-  Ring ring[3];        // .. where no expert has more than ring_rows rows; where none merges (expert_merges); and for merged items
-  int ring_rows;
+  Ring ring[4];        // .. one of them for the launch (schedule.h, ring_choice)
+  int ring_rows[2];    // rows of the largest expert up to which the first two serve
   // epilogue tensors
   uint16_t* out0;      // GATE_UP: A [rows][F]; ACT_GRAD: dH [rows][2F]; DOWN, GATE_GRAD: [rows][N]; rows row_ld(..) apart
   uint16_t* out1;      // GATE_UP: H [rows][2F], NULL: the pre-activations are not kept

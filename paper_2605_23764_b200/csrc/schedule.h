@@ -82,6 +82,20 @@ MOE_HD bool expert_merges(int rows, int mblocks) {
   return (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
 }
 
+constexpr int MERGED_TOKENS_MAX = 256 + MERGE_TAIL_MAX;   // of one item
+
+// The operand rings of a call of T tokens (gemm_tc3.cu, plan_ring), by the rows of the largest expert: a ring for tiles of at most
+// rows[0] tokens, of at most rows[1], of 256, and for merged items.  Distinct ids give an expert T rows at most, so that the
+// second ring holds what a call of 129 to 224 tokens needs (a shared expert has T rows always): seven stages for six up to 192.
+// Forward over 130 tokens x 8 + 1, 256 experts, 7168 x 2048: 3350 -> 3253 us; a step over 160 x 2 + 1, 8 experts, 4096 x 1536: 243 -> 234.
+MOE_HD int ring_rows(int T, int ring) {
+  const int rows = (T + GROUP_ROWS - 1) / GROUP_ROWS * GROUP_ROWS, most = ring == 0 ? 128 : 256;
+  return rows < most ? rows : most;
+}
+MOE_HD int ring_choice(int largest, int rows0, int rows1, bool merged) {
+  return largest <= rows0 ? 0 : largest <= rows1 ? 1 : merged ? 3 : 2;
+}
+
 // One work item of a row-space phase: a token tile (unit) of an expert and a column tile, or -- for an expert that merges
 // (expert_merges) -- its last two units under one k-loop.  `start[e]` = first item of a column tile of expert e, `blk_expert[i]` =
 // expert of item i (both from the layout kernels).

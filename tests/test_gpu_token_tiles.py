@@ -6,7 +6,7 @@ import torch
 
 import oracle
 from paper_2605_23764_b200 import MoeLayer
-from tests.gpu_util import assert_close_bf16
+from tests.gpu_util import assert_close_bf16, small_problem
 
 pytestmark = pytest.mark.gpu
 
@@ -64,8 +64,7 @@ def test_counts_on_tile_edges(d, F, serial):
 @pytest.mark.parametrize("d", [568, 576, 2048])
 @pytest.mark.parametrize("serial", [False, True])
 def test_merged_tiles_in_every_operator(d, serial):
-    """Experts whose last two token tiles share a k-loop, of 257 to 320 rows and in a row of items: their accumulators take
-    turns at the two ends of the 512 columns and overlap; unmerged tiles of all sizes between them."""
+    """Experts whose last two token tiles share a k-loop, of 257 to 320 rows, and unmerged tiles of all sizes between them."""
     counts = [257, 320, 300, 256, 290, 64, 320, 577, 320, 1, 384, 257]
     E, T, F = len(counts), sum(counts), 264
     g = torch.Generator().manual_seed(41)
@@ -75,10 +74,38 @@ def test_merged_tiles_in_every_operator(d, serial):
     _check_against_oracle(T, d, E, 1, F, ids, w, 42, serial)
 
 
+@pytest.mark.parametrize("T", [129, 160, 192, 200, 224, 256])
+@pytest.mark.parametrize("serial", [False, True])
+def test_few_tokens_with_a_shared_expert(T, serial):
+    """129 to 256 tokens, every one of them in the shared expert: the ring between those of 128- and of 256-token tiles; and more
+    rows in an expert than there are tokens (every token names one expert three times).  More k-blocks than stages."""
+    d, E, k, S, F = 840, 6, 3, 1, 392
+    x, W1, W2, logits, dout = small_problem(T, d, E, k, S, F, 60 + T)
+    for repeated in (False, True):
+        layer = MoeLayer(T, d, E, k, S, F, save_for_bwd=True, serial=serial)
+        ids, w = layer.route(logits)
+        if repeated:
+            ids = torch.full_like(ids, 2)
+        out = layer.ffn_fwd(x, ids, w, W1, W2)
+        dx, dW1, dW2, dw = layer.ffn_bwd(dout, x, ids, w, W1, W2)
+        torch.cuda.synchronize()
+        assert layer.status() == (0, 0)
+        rdx, rdW1, rdW2, rdw = oracle.bwd(dout, x, ids.cpu(), w.cpu(), W1, W2, S=S)
+        for got, ref, name in ((out, oracle.fwd(x, ids.cpu(), w.cpu(), W1, W2, S=S), "out"), (dx, rdx, "dx"), (dw, rdw, "d_topk_w")):
+            assert_close_bf16(got, ref, name)
+        for e in range(E + S):
+            if repeated and e not in (2, E):
+                assert torch.count_nonzero(dW1[e]).item() == 0 and torch.count_nonzero(dW2[e]).item() == 0
+            else:
+                assert_close_bf16(dW1[e], rdW1[e], f"dW_gate_up[{e}]")
+                assert_close_bf16(dW2[e], rdW2[e], f"dW_down[{e}]")
+        layer.close()
+
+
 @pytest.mark.parametrize("counts", [[128, 33, 96, 0, 128, 127], [129, 128, 256, 31, 511], [129, 257, 100, 320, 64]])
 @pytest.mark.parametrize("serial", [False, True])
 def test_operand_ring_by_largest_expert(counts, serial):
-    """Largest expert of 128 rows, of more without a merged item, and with one: the three rings; more k-blocks than stages."""
+    """Largest expert of 128 rows, of more without a merged item, and with one: a ring for each; more k-blocks than stages."""
     E, T, d, F = len(counts), sum(counts), 840, 392
     g = torch.Generator().manual_seed(51)
     ids = torch.from_numpy(np.repeat(np.arange(E), counts).astype(np.int32))

@@ -98,6 +98,22 @@ def test_layout_takes_the_kernels_where_a_cluster_does_not_fit():
     assert blocks(123, 8, 64, fits8=False, fits16=False) == 1
 
 
+def test_operand_ring_by_tokens_and_largest_expert():
+    ring = binding.moe_debug_ring
+    assert [ring(0, T, T)[0] for T in (32, 128, 129, 160, 161, 192, 193, 224, 225, 256)] == [11, 8, 7, 7, 7, 7, 6, 6, 6, 6]
+    assert [ring(1, T, T)[0] for T in (32, 128, 129, 160, 161, 192, 193, 224, 225, 256)] == [11, 8, 8, 8, 7, 7, 6, 6, 6, 6]
+    for is_bwd in (0, 1):
+        for T in (1, 31, 33, 127, 129, 160, 192, 255, 257, 4096, 16384):
+            # ids repeated in a token give an expert more rows than there are tokens
+            for largest in {1, 32, 33, T, T + 1, 128, 129, 160, 161, 256, 257, 300, 8 * T}:
+                for merged in (False, True) if largest > 256 else (False,):
+                    stages, tokens = ring(is_bwd, T, largest, merged)
+                    # the widest tile there can be: the largest expert's rows up to 256, or a merged item's 128 + 128 + 64
+                    need = 320 if merged else min(256, (largest + 31) // 32 * 32)
+                    assert tokens >= need and stages >= 5, (is_bwd, T, largest, merged, stages, tokens)
+            assert ring(is_bwd, T, min(T, 128))[0] >= 8   # as deep as the largest expert allows, whatever the call's size
+
+
 @pytest.mark.parametrize("is_bwd", [0, 1])
 @pytest.mark.parametrize("pairs", [1, 2, 5, 74])
 @pytest.mark.parametrize("d,F", [(4096, 8), (2048, 64), (256, 520)])   # items of one, one and nine k-blocks of F
