@@ -6,7 +6,7 @@
 // global loads (two or three microseconds), so callers decode the NEXT item while the current one runs.  The one-launch-per-operator kernels (gemm_tc3.cu,
 // gemm_wgrad.cu) walk an operator's items in a static order with no event counters; the persistent
 // launch (fused.cu) takes items of all operators of a pass from one ticket queue, carries the pipeline
-// state (stage ring position, barrier parities, accumulator parity) from item to item and orders
+// state (stage ring position, barrier parities, end of TMEM in turn) from item to item and orders
 // tiles by event counters (the dependent and trigger events of Section 4.3).  Both use exactly this
 // code, so they produce the same bits.
 #pragma once
@@ -26,10 +26,13 @@ constexpr int GEMM_ROLE_WARPS = 12;
 __device__ __forceinline__ bool is_epilogue_warp(int warp) { return (warp >= 2 && warp < 6) || (warp >= 8 && warp < 12); }
 __device__ __forceinline__ int epilogue_index(int warp) { return (warp & 3) + (warp >= 8 ? 4 : 0); }
 
-// Accumulators.  An item of up to two tiles has 64 to 384 TMEM columns; items take the two ends of the 512 columns in turn, so
-// that an item's products run beside the epilogue of the one before.  Where the two overlap -- merged items -- the item begins
-// when the tile in the middle is drained: that tile is the larger one, and its epilogue comes first.  Four slots: end, tile.
+// Accumulators.  An item has 32 to 256 TMEM columns, a merged one 128 + 160 or 128 + 192; items take the two ends of the 512
+// columns in turn, so that an item's products run beside the epilogue of the one before.  Where the two overlap -- behind or before
+// merged items -- the item begins when the tile in the middle is drained: that tile is the larger one, and its epilogue comes
+// first.  The overlap never reaches the tile behind it: two items have 320 columns at most.  Four slots: end, tile.
 constexpr int ACC_SLOTS = 4;
+static_assert(2 * MERGED_TOKENS_MAX - TMEM_COLS <= BLOCK_M + TOK_GRAIN, "a merged item's first tile is at least as wide as any overlap");
+static_assert(MERGED_TOKENS_MAX + 2 * BLOCK_M - TMEM_COLS <= 2 * BLOCK_M, "an item of one tile as well");
 // first column of tile `part` (0: the one towards the middle) of an item of n0 + n1 columns
 __device__ __forceinline__ int acc_column(int end, int part, int n0, int n1) {
   return part == 0 ? (end ? TMEM_COLS - n0 - n1 : n1) : (end ? TMEM_COLS - n1 : 0);
@@ -59,7 +62,7 @@ struct IssuerState {
   uint32_t s = 0, full_par = 0, a_s = 0;
   int end = 0;                    // of the TMEM columns, for the next item
   uint32_t busy = 0, acc_par = 0; // by slot: not seen drained; parity of the next drain
-  int before_n0 = 0, before_n = 0;   // columns of the item before: of its first tile, of both
+  int before_n = 0;               // columns of the item before
 };
 struct EpiState { int end = 0; uint32_t full_par = 0; };
 
@@ -260,9 +263,8 @@ __device__ __forceinline__ bool swap_load_item(GemmMode mode, const GemmArgs& a,
 // The issuer takes columns for an item of n0 (+ n1) columns: what they overlap has been drained when this returns.  Its slots are
 // 2 * is.end and, for the second tile, the one behind; the caller flips is.end.
 __device__ __forceinline__ bool acc_claim(PipeBarriers* bars, IssuerState& is, int n0, int n1, const WaitCtl& wc, int t) {
-  const int over = is.before_n + n0 + n1 - TMEM_COLS, other = 2 * (is.end ^ 1);
   uint32_t need = 3u << (2 * is.end);   // the item before the last, at the same end
-  if (over > 0) need |= (over > is.before_n0 ? 3u : 1u) << other;
+  if (is.before_n + n0 + n1 > TMEM_COLS) need |= 1u << (2 * (is.end ^ 1));   // and the tile in the middle of the last
   need &= is.busy;
 #pragma unroll 1
   while (need) {
@@ -273,7 +275,6 @@ __device__ __forceinline__ bool acc_claim(PipeBarriers* bars, IssuerState& is, i
     need &= need - 1;
   }
   is.busy |= (n1 ? 3u : 1u) << (2 * is.end);
-  is.before_n0 = n0;
   is.before_n = n0 + n1;
   return true;
 }

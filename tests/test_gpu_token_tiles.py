@@ -74,6 +74,42 @@ def test_merged_tiles_in_every_operator(d, serial):
     _check_against_oracle(T, d, E, 1, F, ids, w, 42, serial)
 
 
+@pytest.mark.parametrize("d", [136, 328])   # three and six k-blocks of gate+up and act_grad: fewer and more than stages
+def test_merged_items_follow_one_another(d):
+    """Items enough that every CTA pair works off several merged ones in a row: their accumulators take turns at the two ends of the
+    512 columns and overlap -- after one another, after one of 256 columns and before one; three and five M-blocks.  Expert by
+    expert: a wrong column would hide in whole tensors."""
+    counts = [257, 320, 300, 288, 256, 290, 319, 320, 513, 576, 577, 300] * 5
+    E, T, F = len(counts), sum(counts), 1288
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    assert E * ((F + 255) // 256) >= 4 * pairs   # act_grad; gate+up has more
+    g = torch.Generator().manual_seed(43 + d)
+    ids = torch.from_numpy(np.repeat(np.arange(E), counts).astype(np.int32))
+    ids = ids[torch.randperm(T, generator=g)].reshape(T, 1).contiguous().cuda()
+    w = (torch.rand(T, 1, generator=g) + 0.25).float().cuda()
+    x = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
+    W1 = (torch.randn(E, 2 * F, d, generator=g) / d ** 0.5).to(torch.bfloat16).cuda()
+    W2 = (torch.randn(E, d, F, generator=g) / d ** 0.5).to(torch.bfloat16).cuda()
+    dout = torch.randn(T, d, generator=g).to(torch.bfloat16).cuda()
+    ref_out = np.asarray(oracle.fwd(x, ids.cpu(), w.cpu(), W1, W2))
+    rdx, rdW1, rdW2, rdw = [np.asarray(r) for r in oracle.bwd(dout, x, ids.cpu(), w.cpu(), W1, W2)]
+    for serial in (False, True):
+        layer = MoeLayer(T, d, E, 1, 0, F, renorm=False, save_for_bwd=True, serial=serial)
+        out = layer.ffn_fwd(x, ids, w, W1, W2)
+        dx, dW1, dW2, dw = layer.ffn_bwd(dout, x, ids, w, W1, W2)
+        torch.cuda.synchronize()
+        assert layer.status() == (0, 0)
+        for e, n in enumerate(counts):
+            tok = (ids[:, 0] == e).nonzero()[:, 0].cpu()
+            what = f"of expert {e} ({n} rows, serial {serial})"
+            assert_close_bf16(out[tok], ref_out[tok.numpy()], "out " + what)
+            assert_close_bf16(dx[tok], rdx[tok.numpy()], "dx " + what)
+            assert_close_bf16(dw[tok], rdw[tok.numpy()], "d_topk_w " + what)
+            assert_close_bf16(dW1[e], rdW1[e], "dW_gate_up " + what)
+            assert_close_bf16(dW2[e], rdW2[e], "dW_down " + what)
+        layer.close()
+
+
 @pytest.mark.parametrize("T", [129, 160, 192, 200, 224, 256])
 @pytest.mark.parametrize("serial", [False, True])
 def test_few_tokens_with_a_shared_expert(T, serial):
