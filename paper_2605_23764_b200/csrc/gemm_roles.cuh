@@ -203,14 +203,15 @@ struct ChainDeps {
 // Token-column row-space operators (gemm_swap.cuh)
 // =====================================================================================================
 // Shared memory of an operator, from the 1024-byte aligned base: weights [stages][16 KB] | tokens [stages][tok_bytes], and at
-// the end of LAYOUT_BYTES the staging.  What the token stages do not need goes into more stages: the loads of a k-block take
-// about 2400 clocks, so that five stages bound a tile of 128 tokens at 480 clocks a k-block, whose products take 256; and a
+// the end of LAYOUT_BYTES the staging.  What the token stages do not need goes into more stages: the products of a k-block of a
+// small tile are over long before the loads of one are, so that the stages in flight bound the tile; and a
 // pass over few tokens is a stream of weights from HBM (32 tokens: eleven stages, 198 KB in flight instead of 80).  The rings
 // come from the host (schedule.h, ring_rows); the layout leaves the rows of the largest expert in meta[7] and what merges in
 // meta[3], meta[4], and every role finds the same one.  (Worked out in the kernel for every item, passes of short items took 1-3 % longer; stages as large as their own tile,
 // in a ring of bytes, cost the loaders more than the depth gave.)
-// Against two rings, one for calls of up to 256 tokens: 4096 tokens x 8, 256 experts, 7168 x 2048: 4968 -> 4877 us (six stages for
-// five); 2048 x 4, 128 experts, 4096 x 1536: 894 -> 864 (eight); 512 x 6 + 2, 64 experts, 2048 x 1408: 236 -> 233.
+// Against five stages in all of these, forward, medians of 12 runs in turn in three processes each, within 1 % of one another: 2048
+// tokens x 8, 128 experts, 7168 x 2048: 2373 -> 2323 us (six); 2048 x 4, 128 experts, 4096 x 1536: 904 -> 864 (eight, no expert above
+// 128 rows); 512 x 6 + 2, 64 experts, 2048 x 1408: 241 -> 233 (six).  One merged item takes a launch back to five.
 constexpr size_t PIPE_BARRIER_BYTES = 384;
 constexpr size_t TICKET_RING_BYTES = 640;   // of the persistent launch
 constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_RING_BYTES;

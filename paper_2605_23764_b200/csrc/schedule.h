@@ -76,8 +76,8 @@ MOE_HD void balanced_unit(int mc, int u, int* first, int* count) {
 constexpr int MERGE_TAIL_MAX = 64;
 // Merged against two items in gate+up (forward) and act_grad (backward), 64 experts of 300 rows, F = 1408, medians of 14 runs in
 // turn, us: d = 64 125 -> 107 forward; 256 132 -> 111 and 227 -> 207; 512 159 -> 136 and 313 -> 293; 1024 235 -> 217 and 473 -> 470;
-// 1536 even backward; 2048 428 -> 382 and 809 -> 801; 4096 1558 -> 1509 backward (quartiles of one side 1-2 % of these).  With
-// experts of 288 +- 17 rows, half of them merged, the same within 1 %.
+// 1536 even backward; 2048 428 -> 382 and 809 -> 801; 4096 1558 -> 1509 backward (quartiles of one side 1-2 % of these).  Experts
+// of 288 +- 17 rows, almost all of which merge, gain alike.
 MOE_HD bool expert_merges(int rows, int mblocks) {
   return (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
 }
