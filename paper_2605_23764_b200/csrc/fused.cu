@@ -415,9 +415,12 @@ __device__ __forceinline__ bool load_item(const FusedArgs& fa, const GemmArgs::R
   if (strip)
     return wgrad_load_strip(fa.op[phase], smem, bars, ls, second_warp, rank, lane, desc_strip(wd), t, wc, dep);
   const SwapWork wk = desc_swap_work(wd);
-  // one copy of the code for both operators of the pass: a launch over few tokens runs it once, from a cold instruction cache
-  const GemmMode mode = BWD ? GEMM_ACT_GRAD : phase == 0 ? GEMM_GATE_UP : GEMM_DOWN;   // gate_grad's weights lie like act_grad's
-  return swap_load_item(mode, fa.op[phase], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  // act_grad's and gate_grad's weights lie alike: one copy of the code serves both.  The forward's loaders know their operator when
+  // compiled: chosen per k-block, passes that stream weights take 1-2.5 % longer (4096 tokens x 4, 128 experts, 7168 x 2048: 2334 us
+  // against 2397).
+  if (BWD) return swap_load_item(GEMM_ACT_GRAD, fa.op[phase], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  if (phase == 0) return swap_load_item(GEMM_GATE_UP, fa.op[0], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
+  return swap_load_item(GEMM_DOWN, fa.op[1], ring, smem, bars, ls, second_warp, rank, lane, wk, t, wc, dep);
 }
 template <bool BWD>
 __device__ __forceinline__ bool issue_item(const FusedArgs& fa, const GemmArgs::Ring ring, const WorkDesc& wd, uint8_t* smem, PipeBarriers* bars,
