@@ -1204,7 +1204,7 @@ int moe_debug_simulate_schedule(const int32_t* counts, int32_t Ep, int32_t T, in
   for (int e = 0; e < Ep; ++e) {
     const int m = (counts[e] + BLOCK_M - 1) / BLOCK_M, pr = (m + 1) >> 1;
     mb_start[e + 1] = mb_start[e] + m;
-    work_start[e + 1] = work_start[e] + pr - (expert_merges(counts[e], m) ? 1 : 0);
+    work_start[e + 1] = work_start[e] + pr - (expert_merges(counts[e], m, e >= Ep - n_shared) ? 1 : 0);
   }
   std::vector<int> long_before(Ep + 1, 0), order(Ep, -1);
   for (int e = 0; e < Ep; ++e) long_before[e + 1] = long_before[e] + strip_long(counts[e]);

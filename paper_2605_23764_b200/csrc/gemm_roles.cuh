@@ -211,7 +211,8 @@ struct ChainDeps {
 // in a ring of bytes, cost the loaders more than the depth gave.)
 // Against five stages in all of these, forward, medians of 12 runs in turn in three processes each, within 1 % of one another: 2048
 // tokens x 8, 128 experts, 7168 x 2048: 2373 -> 2323 us (six); 2048 x 4, 128 experts, 4096 x 1536: 904 -> 864 (eight, no expert above
-// 128 rows); 512 x 6 + 2, 64 experts, 2048 x 1408: 241 -> 233 (six).  One merged item takes a launch back to five.
+// 128 rows); 512 x 6 + 2, 64 experts, 2048 x 1408: 241 -> 233 (six).  One merged item takes a launch back to
+// five.
 constexpr size_t PIPE_BARRIER_BYTES = 384;
 constexpr size_t TICKET_RING_BYTES = 640;   // of the persistent launch
 constexpr size_t LAYOUT_BYTES = 227 * 1024 - 1024 - PIPE_BARRIER_BYTES - TICKET_RING_BYTES;

@@ -163,7 +163,7 @@ __device__ __forceinline__ void scan_experts(int E, int Ep, const LayoutView& lv
     const int pr = (m + 1) >> 1;  // token tiles (units, schedule.h)
     // work items of the token-column GEMM kernels: the units of the expert, except that an expert
     // that merges (schedule.h) has its last two units (one block; block + tail) share one k-loop
-    const int val[NQ] = {c, m, pr - (expert_merges(c, m) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS, strip_long(c)};
+    const int val[NQ] = {c, m, pr - (expert_merges(c, m, e >= E) ? 1 : 0), (c + GROUP_ROWS - 1) / GROUP_ROWS, strip_long(c)};
     int inc[NQ] = {val[0], val[1], val[2], val[3], val[4]};
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {

@@ -78,8 +78,13 @@ constexpr int MERGE_TAIL_MAX = 64;
 // turn, us: d = 64 125 -> 107 forward; 256 132 -> 111 and 227 -> 207; 512 159 -> 136 and 313 -> 293; 1024 235 -> 217 and 473 -> 470;
 // 1536 even backward; 2048 428 -> 382 and 809 -> 801; 4096 1558 -> 1509 backward (quartiles of one side 1-2 % of these).  Experts
 // of 288 +- 17 rows, almost all of which merge, gain alike.
-MOE_HD bool expert_merges(int rows, int mblocks) {
-  return (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
+// A shared expert does not merge: one merged item takes a stage from every other (ring_choice), and a shared expert with a short
+// last block is there at a quarter of all token counts; where items are few to a pair, a merged one is also the longest.  Merged
+// against two items, us: 300 tokens, 8 x 2 + 1 experts, 2048 x 1408, forward 62.2 against 56.4, a step 174 against 161; 2060 x 4 + 1,
+// 128 experts, 4096 x 1536, forward 975 against 945; 4100 x 4 + 1, 128 experts, 7168 x 2048 2640 against 2551.  Of 14 shapes with more
+// shared experts than usual (2 to 16) two lose, 300 tokens, 2048 x 1408, forward: 16 x 2 + 4 87.7 against 91.6, 8 x 1 + 8 87.7 against 89.8.
+MOE_HD bool expert_merges(int rows, int mblocks, bool shared) {
+  return !shared && (mblocks & 1) && mblocks >= 3 && rows - (mblocks - 1) * 128 <= MERGE_TAIL_MAX;
 }
 
 constexpr int MERGED_TOKENS_MAX = 256 + MERGE_TAIL_MAX;   // of one item

@@ -110,11 +110,12 @@ def test_merged_items_follow_one_another(d):
         layer.close()
 
 
-@pytest.mark.parametrize("T", [129, 160, 192, 200, 224, 256])
+@pytest.mark.parametrize("T", [129, 160, 192, 200, 224, 256, 300, 577])
 @pytest.mark.parametrize("serial", [False, True])
 def test_few_tokens_with_a_shared_expert(T, serial):
-    """129 to 256 tokens, every one of them in the shared expert: the ring between those of 128- and of 256-token tiles; and more
-    rows in an expert than there are tokens (every token names one expert three times).  More k-blocks than stages."""
+    """129 to 256 tokens, every one of them in the shared expert: the ring between those of 128- and of 256-token tiles; three and
+    five M-blocks of the shared expert, which do not merge; and more rows in an expert than there are tokens (every token names one
+    expert three times).  More k-blocks than stages."""
     d, E, k, S, F = 840, 6, 3, 1, 392
     x, W1, W2, logits, dout = small_problem(T, d, E, k, S, F, 60 + T)
     for repeated in (False, True):

@@ -12,13 +12,13 @@ def _lib():
     build.build()
 
 
-def _expected_items(counts, d, F, is_bwd):
+def _expected_items(counts, d, F, is_bwd, n_shared=0):
     mblocks = (counts + 127) // 128
     units = (mblocks + 1) // 2
     # an expert merges its last two units, in every row-space phase, when its M-block count is odd, at least 3, and the last
-    # block holds <= 64 rows
-    merged = units - ((mblocks % 2 == 1) & (mblocks >= 3) & (counts - (mblocks - 1) * 128 <= 64))
+    # block holds <= 64 rows -- unless it is a shared one
     Ep = len(counts)
+    merged = units - ((mblocks % 2 == 1) & (mblocks >= 3) & (counts - (mblocks - 1) * 128 <= 64) & (np.arange(Ep) < Ep - n_shared))
     if not is_bwd:
         return int(merged.sum()) * ((F + 127) // 128 + (d + 255) // 256)
     return (int(merged.sum()) * ((F + 255) // 256) + Ep * ((d + 255) // 256) +
@@ -96,6 +96,16 @@ def test_layout_takes_the_kernels_where_a_cluster_does_not_fit():
     for T in (1025, 8192):
         assert blocks(T, 8, 64, fits8=False) == 16 and blocks(T, 8, 64, fits16=False) == 0
     assert blocks(123, 8, 64, fits8=False, fits16=False) == 1
+
+
+@pytest.mark.parametrize("is_bwd", [0, 1])
+@pytest.mark.parametrize("T", [257, 300, 320, 321, 576, 1060, 4096, 4100])
+def test_shared_experts_do_not_merge(is_bwd, T):
+    """A call's operand ring is the same for 4096 and for 4100 tokens: a shared expert's short last block merges with nothing."""
+    for n_shared in (1, 2):
+        counts = np.array([128, 300, 0, 250] + [T] * n_shared)
+        rc, stats = binding.moe_debug_simulate_schedule(counts, T, 2, n_shared, 264, 272, is_bwd, 74, 592)
+        assert rc == 0 and stats[0] == _expected_items(counts, 264, 272, is_bwd, n_shared)
 
 
 def test_operand_ring_by_tokens_and_largest_expert():
