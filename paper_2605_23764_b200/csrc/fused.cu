@@ -452,8 +452,9 @@ __device__ __forceinline__ bool epilogue_item(const FusedArgs& fa, const WorkDes
 
 // A matrix role's walk over the pair's items in ticket order; `enter` at each phase boundary of the backward (gemm_roles.cuh): the
 // new phase's ring, of its own depth, starts at stage 0.  (The forward's two operators have one layout: the ring and the staging run
-// on.)  A loop for each role: in one for all of them every warp carried all roles' state, 14 registers of which act_grad's epilogue
-// has none to spare.
+// on.)  The backward has a loop for each role: in one for all of them every warp carries all roles' state, 14 registers of which
+// act_grad's epilogue has none to spare (1056 tokens, 32 + 1 experts, 1024 x 512: 90 us, in three loops 84).  The forward has
+// registers left, and one loop: in three, 4096 tokens x 8, 256 experts, 7168 x 2048 take 4569 us for 4520.
 template <bool BWD, class ENTER, class WORK>
 __device__ __forceinline__ bool walk_items(const FusedArgs& fa, TicketRing* ring, int lane, const WaitCtl& wc, const TraceCtl& tr,
                                            ENTER enter, WORK work) {
@@ -505,6 +506,7 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
   // (No trigger for the next launch: a router that takes the SMs as this launch's CTAs leave them is 2-3 % slower.)
   pdl_wait();   // the layout's tables, and everything else in front of this launch
   const int M = fa.lv.meta[0];
+  const bool loader = warp == 0 || warp == 6, issuer = warp == 1 && rank == 0, epilogue = is_epilogue_warp(warp);
 
   if (warp == SCHED_WARP && rank == 0) {
     // ------------------------------------------------ scheduler of the pair (even CTA)
@@ -561,42 +563,49 @@ __global__ void __launch_bounds__(FUSED_THREADS, 1) fused_chain_kernel(const __g
       phase = __shfl_sync(0xffffffffu, wd.phase, 31);
       batch = 1 << ((batches >> (2 * phase)) & 3);
     }
-  } else if (warp == 0 || warp == 6) {
+  } else if (loader || issuer || epilogue) {
     // ------------------------------------------------ matrix roles: the pair's items in ticket order
-    const GemmArgs::Ring op_ring = which_ring(fa.op[0]);   // the operators of a pass have the same staging, and the same rings
-    LoaderState ls;
-    walk_items<BWD>(fa, ring, lane, wc, tr, [&](int phase) { return loader_enter_phase(bars, ls, phase, wc); },
-                    [&](const WorkDesc& wd, const ChainDeps& dep) {
-                      return load_item<BWD>(fa, op_ring, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
-                    });
-  } else if (warp == 1 && rank == 0) {
-    const GemmArgs::Ring op_ring = which_ring(fa.op[0]);
-    IssuerState is;
-    const bool ok = walk_items<BWD>(fa, ring, lane, wc, tr, [&](int) { is.s = is.a_s = 0; return true; },
-                                    [&](const WorkDesc& wd, const ChainDeps& dep) {
-                                      return issue_item<BWD>(fa, op_ring, wd, smem, bars, tmem_base, is, wc, dep);
-                                    });
-    if (uniform(!ok || *reinterpret_cast<volatile int*>(&fa.status->abort) ? 1 : 0)) issuer_drain(bars, fa.status);
-  } else if (is_epilogue_warp(warp)) {
     const int ew = epilogue_index(warp);
+    GemmArgs::Ring op_ring{};
+    if (!epilogue) op_ring = which_ring(fa.op[0]);   // the operators of a pass have the same staging, and the same rings
+    LoaderState ls;
+    IssuerState is;
     EpiState es;
-    walk_items<BWD>(fa, ring, lane, wc, tr,
-                    [&](int phase) {
-                      int go = 1;
-                      if (lane == 0) {
-                        tma_store_wait_read();
-                        epi_enter_phase(bars, ew, phase);
-                        go = phase_wait(bars, phase, wc) ? 1 : 0;
-                      }
-                      return __shfl_sync(0xffffffffu, go, 0) != 0;
-                    },
-                    [&](const WorkDesc& wd, const ChainDeps& dep) {
-                      return epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, ew, lane, wc, dep);
-                    });
-    if (lane == 0) {
+    auto load = [&](const WorkDesc& wd, const ChainDeps& dep) {
+      return load_item<BWD>(fa, op_ring, wd, smem, bars, ls, warp == 6, rank, lane, wc, dep);
+    };
+    auto issue = [&](const WorkDesc& wd, const ChainDeps& dep) {
+      return issue_item<BWD>(fa, op_ring, wd, smem, bars, tmem_base, is, wc, dep);
+    };
+    auto finish = [&](const WorkDesc& wd, const ChainDeps& dep) {
+      return epilogue_item<BWD>(fa, wd, smem, bars, tmem_base, es, rank, ew, lane, wc, dep);
+    };
+    bool ok;
+    if (!BWD) {
+      ok = walk_items<BWD>(fa, ring, lane, wc, tr, [](int) { return true; }, [&](const WorkDesc& wd, const ChainDeps& dep) {
+        return loader ? load(wd, dep) : issuer ? issue(wd, dep) : finish(wd, dep);
+      });
+    } else if (loader) {
+      ok = walk_items<BWD>(fa, ring, lane, wc, tr, [&](int phase) { return loader_enter_phase(bars, ls, phase, wc); }, load);
+    } else if (issuer) {
+      ok = walk_items<BWD>(fa, ring, lane, wc, tr, [&](int) { is.s = is.a_s = 0; return true; }, issue);
+    } else {
+      auto enter = [&](int phase) {
+        int go = 1;
+        if (lane == 0) {
+          tma_store_wait_read();
+          epi_enter_phase(bars, ew, phase);
+          go = phase_wait(bars, phase, wc) ? 1 : 0;
+        }
+        return __shfl_sync(0xffffffffu, go, 0) != 0;
+      };
+      ok = walk_items<BWD>(fa, ring, lane, wc, tr, enter, finish);
+    }
+    if (epilogue && lane == 0) {
       tma_store_wait_all();
       epi_enter_phase(bars, ew, SCHED_MAX_SEG);   // nothing of this warp is left in shared memory
     }
+    if (issuer && uniform(!ok || *reinterpret_cast<volatile int*>(&fa.status->abort) ? 1 : 0)) issuer_drain(bars, fa.status);
   }
 
   // ------------------------------------------------ vector workers: the dedicated warps from the start, the
